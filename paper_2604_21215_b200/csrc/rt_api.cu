@@ -18,7 +18,7 @@ constexpr int kSmallBatchMax = 64;      // above this the per-token chain runs a
 constexpr int kAutoLeaf = 64;
 
 struct WsLayout {
-  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, dec_part, ll, ll_bytes, hid0, hid1,
+  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, dec_words, ll, ll_bytes, hid0, hid1,
       blk_h, blk_u, blk_c, blk_g, total;
 };
 
@@ -45,7 +45,10 @@ rt_status config_supported(const rt_config* c, int B, bool wide_ok = false) {
   return RT_OK;
 }
 
-WsLayout ws_layout(const rt_config* c, int B, int N) {
+// Sequences per launch of the decode kernel: a batch above 16 runs as slices of equal size (the sequences are independent).
+int decode_slice(int B) { return ceil_div(B, ceil_div(B, 16)); }
+
+WsLayout ws_layout(const rt_config* c, int B, int N, int n_layers) {
   WsLayout L;
   const size_t e = esize_of(c->dtype), d = c->d_model, H = c->n_heads, f = c->d_ff;
   const size_t tok = (size_t)B * N;
@@ -64,7 +67,8 @@ WsLayout ws_layout(const rt_config* c, int B, int N) {
   L.ex_z = take((size_t)B * d * 4);
   L.ex_k = take((size_t)B * d * 4);
   L.ex_part = take((size_t)B * H * kMaxChunks * 68 * 4);
-  L.dec_part = take((size_t)B * H * kDecodeMaxRowChunks * 66 * 4);   // chunk partials of the decode-step attention
+  // exchange area of the decode kernel (a decode step is a call with N = 1, of any workspace at least that large)
+  L.dec_words = take(c->dtype == RT_BF16 && B <= kSmallBatchMax ? decode_words_bytes(n_layers, decode_slice(B), (int)d, (int)H, (int)f) : 0);
   // exchange buffers of the tensor-core leaf kernel: c, h, z as flag-carrying words (16 sequence slots each),
   // g as packed bf16 in fragment order (16 sequence slots), raw k|v as flag-carrying fp32 words
   L.ll_bytes = ((size_t)16 * 3 * (d / 2) + (size_t)16 * (f / 4) + (size_t)B * 2 * d) * 8;
@@ -180,22 +184,8 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   pp.n = ws + L.n; pp.q = ws + L.q; pp.kt = ws + L.kt; pp.vt = ws + L.vt;
   pp.st_o = (float*)(ws + L.st_o); pp.st_m = (float*)(ws + L.st_m); pp.st_l = (float*)(ws + L.st_l);
   pp.sync = (SyncArea*)(ws + L.sync);
-  // decode step on the fast path (bf16 shapes the tensor-core leaf kernel takes): its attention warps seed the state
   LeafMmaLaunch ml;
-  const bool dec_fast = n_rows == 1 && pos0 > 0 && c->dtype == RT_BF16 && c->recur_block <= 1 &&
-                        leaf_mma_plan(B, c->d_model, c->n_heads, c->d_ff, c->leaf, &ml);
-  if (dec_fast && (size_t)16 * (c->d_model + 16) * 2 <= 190 * 1024) {
-    // the decode step's pre-pass in one launch (the leaf kernel's attention warps seed the state)
-    DecodePrepassParams dp;
-    memset(&dp, 0, sizeof(dp));
-    dp.B = B; dp.d = c->d_model; dp.H = c->n_heads; dp.norm_flags = c->norm_flags; dp.eps = c->rms_eps;
-    dp.x = x; dp.x_bs = x_bs;
-    dp.w_q = w->w_q; dp.w_k = w->w_k; dp.w_v = w->w_v; dp.g_attn = w->g_attn; dp.g_q = w->g_q; dp.g_k = w->g_k;
-    dp.q = pp.q; dp.kt = pp.kt; dp.vt = pp.vt;
-    ProfScope ps(s, kProfPrepass);
-    if (decode_prepass_launch(dp, s) != cudaSuccess) return RT_ERR_CUDA;
-  } else {
-    if (dec_fast) pp.no_seed = 1;
+  {
     ProfScope ps(s, kProfPrepass);
     if (prepass_launch(c->dtype, pp, s) != cudaSuccess) return RT_ERR_CUDA;
   }
@@ -426,27 +416,6 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
     return true;
   };
 
-  if (dec_fast) {
-    // decode step on the fast path: the new position's query attends to the whole cache in chunks (Algorithm 2 per
-    // chunk), then the tensor-core leaf kernel merges the partial states and runs the one token step
-    DecodeAttnParams da;
-    memset(&da, 0, sizeof(da));
-    da.B = B; da.d = c->d_model; da.H = c->n_heads; da.scale_log2 = scale_log2; da.alibi = w->alibi_slopes;
-    da.q = ws + L.q; da.k_cache = k_cache; da.v_cache = v_cache; da.pos = pos0;
-    da.part = (float*)(ws + L.dec_part);
-    int n_chunks = 0, chunk_stride = 0;
-    {
-      ProfScope ps(s, kProfTile);
-      if (decode_attn_launch(da, &n_chunks, &chunk_stride, s) != cudaSuccess) return RT_ERR_CUDA;
-    }
-    lp.kt = ws + L.kt; lp.vt = ws + L.vt; lp.dec_part = da.part; lp.dec_chunks = n_chunks; lp.dec_stride = chunk_stride;
-    lp.t0 = pos0; lp.t1 = pos0 + 1; lp.attn_begin = pos0; lp.seq_base = ctx.seq_base; lp.bar_base = ctx.bar_base;
-    ProfScope ps(s, kProfLeaf);
-    if (leaf_mma_launch(lp, ml, mb, s) != cudaSuccess) return RT_ERR_CUDA;
-    ctx.seq_base += 1u;
-    ctx.bar_base += (unsigned)ml.grid;
-    return RT_OK;
-  }
   if (c->sched == RT_SCHED_NAIVE || pos0 > 0) {
     // token-sequential: every position reads its whole prefix from the cache
     return leaf(pos0, pos0 + n_rows, 0) ? RT_OK : RT_ERR_CUDA;
@@ -471,13 +440,54 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   return RT_OK;
 }
 
+// One decode step through all layers on the decode kernel (bf16): slices of at most 16 sequences, launches of at most
+// kDecMaxLayers layers.  Input rows x (row stride x_bs) or embedding rows emb[ids]; output rows z.  `hid` holds [B, d] rows between launches.
+rt_status run_decode(const rt_config* c, int n_layers, const rt_layer_weights* layers, const void* x, long long x_bs, const void* emb,
+                     const int32_t* ids, int vocab, int B, int pos, void* z, long long z_bs, void* const* k_caches, void* const* v_caches,
+                     unsigned char* ws, const WsLayout& L, void* const* hid, const void* next_bytes, size_t next_size, cudaStream_t s) {
+  const int sub = decode_slice(B), d = c->d_model;
+  ProfScope ps(s, kProfLeaf);
+  for (int b0 = 0; b0 < B; b0 += sub) {
+    DecodeParams p;
+    memset(&p, 0, sizeof(p));
+    p.B = B - b0 < sub ? B - b0 : sub; p.Bs = B; p.b0 = b0;
+    p.d = d; p.H = c->n_heads; p.dff = c->d_ff; p.pos = pos;
+    p.norm_flags = c->norm_flags; p.eps = c->rms_eps; p.scale_log2 = c->softmax_scale * kLog2e; p.alpha = c->residual_scale;
+    p.words = ws + L.dec_words; p.sync = (SyncArea*)(ws + L.sync);
+    for (int l0 = 0; l0 < n_layers; l0 += kDecMaxLayers) {
+      const bool to_z = l0 + kDecMaxLayers >= n_layers;
+      const size_t off = (size_t)b0 * 2;
+      p.n_layers = to_z ? n_layers - l0 : kDecMaxLayers;
+      p.x = nullptr; p.ids = nullptr;
+      if (l0 > 0) { p.x = (const unsigned char*)hid[(l0 / kDecMaxLayers - 1) & 1] + off * d; p.x_bs = d; }
+      else if (x) { p.x = (const unsigned char*)x + off * x_bs; p.x_bs = x_bs; }
+      else { p.emb = emb; p.ids = ids + b0; p.vocab = vocab; }
+      p.z_out = (unsigned char*)(to_z ? z : hid[(l0 / kDecMaxLayers) & 1]) + off * (to_z ? z_bs : d);
+      p.z_bs = to_z ? z_bs : d;
+      if (to_z && b0 + sub >= B) { p.next_bytes = next_bytes; p.next_size = next_size; }
+      for (int l = 0; l < p.n_layers; ++l) {
+        const rt_layer_weights& w = layers[l0 + l];
+        DecLayer& o = p.layer[l];
+        o.w_q = w.w_q; o.w_k = w.w_k; o.w_v = w.w_v; o.w_o = w.w_o; o.w_up = w.w_up; o.w_down = w.w_down;
+        o.g_attn = w.g_attn; o.g_mlp = w.g_mlp; o.g_kv = w.g_kv ? w.g_kv : w.g_attn; o.g_q = w.g_q; o.g_k = w.g_k;
+        o.alibi = w.alibi_slopes; o.k_cache = k_caches[l0 + l]; o.v_cache = v_caches[l0 + l];
+      }
+      if (decode_launch(p, s) != cudaSuccess) return RT_ERR_CUDA;
+    }
+  }
+  return RT_OK;
+}
+
+// bf16 shapes whose widths fit the decode kernel's 64-byte blocks; everything else takes the generic leaf kernel.
+bool decode_fast(const rt_config* c) { return c->dtype == RT_BF16 && c->d_model % 64 == 0 && c->d_ff % 32 == 0; }
+
 rt_status common_checks(const rt_config* c, int B, int N, int n_layers, void* ws, size_t ws_bytes, bool wide_ok = false) {
   if (!config_ok(c) || B <= 0 || N <= 0 || n_layers <= 0 || !ws || !aligned16(ws)) return RT_ERR_INVALID_ARG;
   const rt_status st = config_supported(c, B, wide_ok);
   if (st != RT_OK) return st;
   // the recurrence over blocks exists for tiled prefill only (wide_ok marks the prefill entry points)
   if (c->recur_block > 1 && !(wide_ok && c->sched == RT_SCHED_TILED)) return RT_ERR_UNSUPPORTED;
-  if (ws_bytes < ws_layout(c, B, N).total) return RT_ERR_WORKSPACE;
+  if (ws_bytes < ws_layout(c, B, N, n_layers).total) return RT_ERR_WORKSPACE;
   return RT_OK;
 }
 
@@ -492,7 +502,7 @@ extern "C" {
 
 size_t rt_workspace_bytes(const rt_config* cfg, int32_t B, int32_t N, int32_t n_layers) {
   if (!config_ok(cfg) || B <= 0 || N <= 0 || n_layers <= 0) return 0;
-  return ws_layout(cfg, B, N).total;
+  return ws_layout(cfg, B, N, n_layers).total;
 }
 
 rt_status rt_layer_prefill(const rt_config* cfg, const rt_layer_weights* w, const void* x, int32_t B, int32_t N,
@@ -506,7 +516,7 @@ rt_status rt_layer_prefill(const rt_config* cfg, const rt_layer_weights* w, cons
   if (overlaps(x, xz_bytes, z, xz_bytes)) return RT_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   unsigned char* ws = (unsigned char*)workspace;
-  const WsLayout L = ws_layout(cfg, B, N);
+  const WsLayout L = ws_layout(cfg, B, N, 1);
   if (cudaMemsetAsync(ws + L.sync, 0, sizeof(SyncArea), s) != cudaSuccess) return RT_ERR_CUDA;
   if (cudaMemsetAsync(ws + L.ll, 0, L.ll_bytes, s) != cudaSuccess) return RT_ERR_CUDA;
   const long long d = cfg->d_model;
@@ -516,7 +526,7 @@ rt_status rt_layer_prefill(const rt_config* cfg, const rt_layer_weights* w, cons
 
 size_t rt_recompute_workspace_bytes(const rt_config* cfg, int32_t B, int32_t N) {
   if (!config_ok(cfg) || B <= 0 || N <= 0) return 0;
-  return ws_layout(cfg, B, N).total + align_up((size_t)B * N * cfg->d_ff * esize_of(cfg->dtype), 256);
+  return ws_layout(cfg, B, N, 1).total + align_up((size_t)B * N * cfg->d_ff * esize_of(cfg->dtype), 256);
 }
 
 rt_status rt_layer_recompute(const rt_config* cfg, const rt_layer_weights* w, const void* x, const void* z_claim,
@@ -533,7 +543,7 @@ rt_status rt_layer_recompute(const rt_config* cfg, const rt_layer_weights* w, co
     return RT_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   unsigned char* ws = (unsigned char*)workspace;
-  const WsLayout L = ws_layout(cfg, B, N);
+  const WsLayout L = ws_layout(cfg, B, N, 1);
   if (cudaMemsetAsync(ws + L.sync, 0, sizeof(SyncArea), s) != cudaSuccess) return RT_ERR_CUDA;
   const long long d = cfg->d_model, f = cfg->d_ff;
   const long long tok = (long long)B * N;
@@ -643,10 +653,14 @@ rt_status rt_layer_decode_step(const rt_config* cfg, const rt_layer_weights* w, 
   }
   cudaStream_t s = (cudaStream_t)cuda_stream;
   unsigned char* ws = (unsigned char*)workspace;
-  const WsLayout L = ws_layout(cfg, B, 1);
+  const WsLayout L = ws_layout(cfg, B, 1, 1);
   if (cudaMemsetAsync(ws + L.sync, 0, sizeof(SyncArea), s) != cudaSuccess) return RT_ERR_CUDA;
-  if (cudaMemsetAsync(ws + L.ll, 0, L.ll_bytes, s) != cudaSuccess) return RT_ERR_CUDA;
   const long long d = cfg->d_model;
+  if (decode_fast(cfg)) {
+    void* hid[2] = {ws + L.hid0, ws + L.hid1};
+    return run_decode(cfg, 1, w, x, d, nullptr, nullptr, 0, B, pos, z, d, &k_cache, &v_cache, ws, L, hid, nullptr, 0, s);
+  }
+  if (cudaMemsetAsync(ws + L.ll, 0, L.ll_bytes, s) != cudaSuccess) return RT_ERR_CUDA;
   rt_config c = *cfg;
   c.sched = RT_SCHED_NAIVE;
   CallCtx ctx{s};
@@ -668,7 +682,7 @@ rt_status rt_stack_prefill(const rt_config* cfg, int32_t n_layers, const rt_laye
   if ((size_t)B * cfg->d_model * 4 > 200 * 1024) return RT_ERR_UNSUPPORTED;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   unsigned char* ws = (unsigned char*)workspace;
-  const WsLayout L = ws_layout(cfg, B, N);
+  const WsLayout L = ws_layout(cfg, B, N, n_layers);
   if (cudaMemsetAsync(ws + L.sync, 0, sizeof(SyncArea), s) != cudaSuccess) return RT_ERR_CUDA;
   if (cudaMemsetAsync(ws + L.ll, 0, L.ll_bytes, s) != cudaSuccess) return RT_ERR_CUDA;
   const long long d = cfg->d_model;
@@ -712,13 +726,21 @@ rt_status rt_decode_step(const rt_config* cfg, int32_t n_layers, const rt_layer_
   if ((size_t)B * cfg->d_model * 4 > 200 * 1024) return RT_ERR_UNSUPPORTED;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   unsigned char* ws = (unsigned char*)workspace;
-  const WsLayout L = ws_layout(cfg, B, 1);
+  const WsLayout L = ws_layout(cfg, B, 1, n_layers);
   if (cudaMemsetAsync(ws + L.sync, 0, sizeof(SyncArea), s) != cudaSuccess) return RT_ERR_CUDA;
-  if (cudaMemsetAsync(ws + L.ll, 0, L.ll_bytes, s) != cudaSuccess) return RT_ERR_CUDA;
   const long long d = cfg->d_model;
   rt_config c = *cfg;
   c.sched = RT_SCHED_NAIVE;
   void* bufs[2] = {ws + L.hid0, ws + L.hid1};
+  if (decode_fast(cfg)) {
+    // the last launch's output goes to the buffer that the last but one does not use
+    void* z = bufs[(ceil_div(n_layers, kDecMaxLayers) - 1) & 1];
+    st = run_decode(cfg, n_layers, layers, nullptr, 0, emb, ids, vocab, B, pos, z, d, k_caches, v_caches, ws, L, bufs, emb,
+                    (size_t)vocab * d * 2, s);
+    if (st != RT_OK) return st;
+    return head_launch(c.dtype, emb, g_final, z, d, B, (int)d, vocab, c.norm_flags, c.rms_eps, logits, s) == cudaSuccess ? RT_OK : RT_ERR_CUDA;
+  }
+  if (cudaMemsetAsync(ws + L.ll, 0, L.ll_bytes, s) != cudaSuccess) return RT_ERR_CUDA;
   CallCtx ctx{s};
   if (embed_launch(c.dtype, emb, ids, B, 1, (int)d, vocab, bufs[0], s) != cudaSuccess) return RT_ERR_CUDA;
   const void* cur = bufs[0];

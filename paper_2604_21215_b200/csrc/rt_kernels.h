@@ -35,12 +35,6 @@ struct LeafParams {
   unsigned bar_base;                             // arrivals counted by earlier launches of the same call (bar_count is
                                                  // zeroed once per API call and only ever grows)
   unsigned seq_base;                             // token steps enqueued before this launch in the same call (flag values)
-  // decode step through the tensor-core leaf kernel (one position): the attention warps build the position's state
-  // themselves -- seeded with the temporary pair (kt, vt rows [B, d]), then the cache's chunk partials
-  // ([B*H][dec_chunks][66] floats: o, m, l) folded in chunk order; dec_chunks = 0 otherwise
-  const void *kt, *vt;
-  const float* dec_part;
-  int dec_chunks, dec_stride;
   int timers;                                    // 1: CTA 0 accumulates per-phase times in the sync area (costs a few per cent)
   SyncArea* sync;
 };
@@ -113,36 +107,32 @@ cudaError_t tile_simt_launch(int dtype, const TileParams& p, cudaStream_t s);
 // one query row (position q0) per (sequence, head) against the pairs [k0, k1): the in-leaf step of wide batches
 cudaError_t row_attn_launch(int dtype, const TileParams& p, cudaStream_t s);
 
-// Attention of one decode step over the whole cache (bf16): query row q [B, d] of the new position against the pairs
-// [0, pos), chunk partials (o, m, l) in `part` ([B*H][n_chunks][66] floats, n_chunks <= kDecodeMaxChunks); the leaf
-// kernel's attention warps fold them, in chunk order, into the state seeded with the temporary pair.
-constexpr int kDecodeMaxChunks = 64;
-constexpr int kDecodeMaxRowChunks = 320;         // chunks of the long-cache kernel (its partials are merged to one per pair)
-struct DecodeAttnParams {
-  int B, d, H;
-  float scale_log2;
-  const float* alibi;                            // [H] slopes or NULL
-  const void* q;                                 // [B, d] bf16
-  const void *k_cache, *v_cache;                 // [N_max, B, d] bf16
-  int pos;                                       // positions in the cache
-  int chunk, n_chunks;                           // set by the launcher
-  float* part;
+// Decode step of up to kDecMaxLayers layers in one cooperative launch (bf16, at most 16 sequences; rt_decode.cu).
+constexpr int kDecMaxLayers = 16;
+struct DecLayer {
+  const void *w_q, *w_k, *w_v, *w_o, *w_up, *w_down;
+  const void *g_attn, *g_mlp, *g_kv, *g_q, *g_k;   // storage type or NULL (g_kv: g_attn where the layer has none)
+  const float* alibi;
+  void *k_cache, *v_cache;
 };
-// Launches the partial kernel(s); *n_chunks = partial states per (sequence, head) left for the leaf kernel to fold in,
-// *chunk_stride = slots per pair in `part` (the leaf kernel reads slots 0 .. n_chunks-1 of pair u at u * chunk_stride).
-cudaError_t decode_attn_launch(const DecodeAttnParams& p, int* n_chunks, int* chunk_stride, cudaStream_t s);
-
-// Pre-pass of a decode step (bf16, B <= 16, d a multiple of 16 with 16 (d + 16) 2 bytes of shared memory available):
-// n = RMS(x), q, k~, v~ of the one new row per sequence in one launch; x [B, d] with row stride x_bs, outputs [B, d].
-struct DecodePrepassParams {
-  int B, d, H;
+struct DecodeParams {
+  int n_layers, B, d, H, dff;                      // B: sequences of this launch
+  int pos;                                         // positions in the caches
+  int Bs, b0;                                      // sequences per cache row, first of this launch
   int norm_flags;
-  float eps;
-  const void* x; long long x_bs;
-  const void *w_q, *w_k, *w_v, *g_attn, *g_q, *g_k;
-  void *q, *kt, *vt;
+  float eps, scale_log2, alpha;
+  const void* x; long long x_bs;                   // input rows [B, d] (row stride x_bs), or NULL:
+  const void* emb; const int32_t* ids; int vocab;  // rows of the embedding
+  void* z_out; long long z_bs;                     // the last layer's output rows
+  const void* next_bytes; size_t next_size;        // what the following kernel reads (L2 prefetch); may be NULL
+  unsigned char* words;                            // exchange area, decode_words_bytes(...)
+  SyncArea* sync;
+  DecLayer layer[kDecMaxLayers];
+  int quads, chunks, chunk_len, warps_per_cta, pf_keys;   // attention split, set by the launcher
 };
-cudaError_t decode_prepass_launch(const DecodePrepassParams& p, cudaStream_t s);
+// Bytes of exchange area for a launch (0: the kernel does not take the shape).
+size_t decode_words_bytes(int n_layers, int B, int d, int H, int dff);
+cudaError_t decode_launch(const DecodeParams& p, cudaStream_t s);
 
 // Stack helpers.
 cudaError_t embed_launch(int dtype, const void* emb, const int32_t* ids, int B, int N, int d, int vocab,

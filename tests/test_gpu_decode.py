@@ -1,0 +1,62 @@
+"""The one-launch decode kernel at the edges of its splits: chunks of eight positions, four (sequence, head) pairs per warp,
+slices of at most 16 sequences, weight slices that do not fit shared memory, more layers than one launch takes."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+# bf16 storage, fp32 accumulation: each stored value carries 2^-9 relative; the outputs pass about five of them
+TOL = 2e-2
+
+
+def _case(d, H, dff, B, N, seed, gains):
+    from paper_2604_21215_b200 import inputs
+    wl = inputs.Workload("dec", 1, B, N, d, H, dff, "bf16")
+    data = inputs.make_inputs(wl, seed=seed)
+    lw = data["layers"][0]
+    if gains:
+        rng = np.random.default_rng(seed)
+        for g in ("g_attn", "g_mlp", "g_kv", "g_q", "g_k"):
+            lw[g] = inputs.round_to(1.0 + 0.2 * rng.standard_normal(d), "bf16")
+    return data["x"], lw
+
+
+@pytest.mark.parametrize("d,H,dff,B,pos,gains", [
+    (128, 2, 256, 1, 0, False), (128, 2, 512, 3, 1, True), (192, 3, 224, 1, 7, False), (192, 3, 768, 5, 8, True),
+    (256, 4, 1024, 8, 9, False), (320, 5, 1280, 9, 33, True), (768, 12, 3072, 16, 70, False), (1024, 16, 4096, 16, 40, True),
+    (256, 4, 1024, 17, 100, False), (128, 2, 512, 48, 19, True), (1408, 22, 5632, 2, 12, False), (64, 1, 128, 1, 300, False)])
+def test_decode_step_matches_oracle(d, H, dff, B, pos, gains):
+    import torch
+    from oracle import RTConfig, RTWeights, layer_seq
+    from paper_2604_21215_b200 import rt
+    x, lw = _case(d, H, dff, B, pos + 1, 40 + pos + B, gains)
+    ref = layer_seq(RTConfig(d, H, 64, dff, residual_scale=0.7), RTWeights(**lw), x)
+    layer = rt.Layer(d, H, dff, dtype="bf16", residual_scale=0.7)
+    layer.set_weights(lw)
+    layer.reserve(B, 1, pos + 3)
+    for cache, r in ((layer.k_cache, ref[1]), (layer.v_cache, ref[2])):
+        cache.fill_(7.0)                                        # rows at and beyond pos must not be read
+        cache[:pos] = torch.from_numpy(np.ascontiguousarray(r[:, :pos].transpose(1, 0, 2))).to(cache)
+    z = layer.decode(x[:, pos], pos)
+    got = {"z": (z, ref[0][:, pos])}
+    for n, cache, r in (("k", layer.k_cache, ref[1]), ("v", layer.v_cache, ref[2])):
+        rows = cache.to(torch.float64).cpu().numpy()
+        got[n] = (rows[pos], r[:, pos])
+        assert (rows[pos + 1:] == 7.0).all()
+    for n, (a, b) in got.items():
+        assert np.abs(a - b).max() <= TOL * np.abs(b).max(), n
+
+
+def test_decode_of_more_layers_than_one_launch_takes():
+    from oracle import RTConfig, RTWeights, stack_prefill
+    from paper_2604_21215_b200 import inputs, rt
+    L, d, H, dff, V, B, N = 18, 64, 1, 128, 77, 2, 5
+    wl = inputs.Workload("deep", L, B, N + 1, d, H, dff, "bf16", vocab=V, residual_scale=1 / np.sqrt(L))
+    data = inputs.make_inputs(wl, seed=11)
+    ocfg = RTConfig(d, H, 64, dff, residual_scale=wl.residual_scale)
+    _, ref, _ = stack_prefill(ocfg, [RTWeights(**w) for w in data["layers"]], data["emb"], None, data["ids"])
+    st = rt.Stack(L, d, H, dff, V, dtype="bf16", residual_scale=wl.residual_scale)
+    st.set_weights(data["layers"], data["emb"])
+    st.prefill(data["ids"][:, :N], N_max=N + 1)
+    got = st.decode(data["ids"][:, N], N)
+    # roundings of 18 layers, each scaled by 1/sqrt(18), add up like one layer's
+    assert np.abs(got - ref).max() <= 2 * TOL * np.abs(ref).max()
