@@ -381,6 +381,10 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   lp.timers = g_prof_timers ? 1 : 0;
   lp.sync = (SyncArea*)(ws + L.sync);
 
+  // small layers: the whole chain inside one cluster, same leaves and tiles
+  LeafSmallLaunch sl;
+  const bool small = c->sched == RT_SCHED_TILED && pos0 == 0 &&
+                     leaf_small_shape(c->dtype, B, c->d_model, c->n_heads, c->d_ff, plan.leaf, kB200SmemPerCta, &sl);
   auto leaf = [&](int t0, int t1, int attn_begin) -> bool {
     lp.t0 = t0; lp.t1 = t1; lp.attn_begin = attn_begin; lp.bar_base = ctx.bar_base;
     ProfScope ps(s, kProfLeaf);
@@ -392,7 +396,7 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   // bf16 tiled prefill takes the tensor-core leaf kernel when the shape fits it
   // (batches of 17 .. 48 sequences: in slices of at most 16, see effective_schedule)
   const int b_sub = (plan.path == kPathMmaSplit && pos0 == 0) ? plan.sub : B;
-  const bool use_mma = c->dtype == RT_BF16 && c->sched == RT_SCHED_TILED && pos0 == 0 &&
+  const bool use_mma = !small && c->dtype == RT_BF16 && c->sched == RT_SCHED_TILED && pos0 == 0 &&
                        leaf_mma_plan(b_sub, c->d_model, c->n_heads, c->d_ff, c->leaf, &ml);
   LeafMmaBuffers mb;
   {
@@ -426,10 +430,15 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   tp.q = ws + L.q; tp.k_cache = k_cache; tp.v_cache = v_cache;
   tp.st_o = pp.st_o; tp.st_m = pp.st_m; tp.st_l = pp.st_l;
   tp.rows_q = n_rows; tp.rows_kv = n_max; tp.sync = lp.sync;
-  const int Lf = use_mma ? ml.leaf : leaf_size(c), N = n_rows;
+  auto leaf_small = [&](int t0, int t1) -> bool {
+    lp.t0 = t0; lp.t1 = t1; lp.attn_begin = t0;
+    ProfScope ps(s, kProfLeaf);
+    return leaf_small_launch(c->dtype, lp, sl, s) == cudaSuccess;
+  };
+  const int Lf = small ? sl.leaf : (use_mma ? ml.leaf : leaf_size(c)), N = n_rows;
   for (int s0 = 0; s0 < N; s0 += Lf) {
     const int e0 = s0 + Lf < N ? s0 + Lf : N;
-    if (!(use_mma ? leaf_mma(s0, e0) : leaf(s0, e0, s0))) return RT_ERR_CUDA;
+    if (!(small ? leaf_small(s0, e0) : (use_mma ? leaf_mma(s0, e0) : leaf(s0, e0, s0)))) return RT_ERR_CUDA;
     if (e0 < N) {
       const int P = e0 & -e0;                              // largest power of two dividing the block end
       tp.q0 = e0; tp.q1 = e0 + P < N ? e0 + P : N; tp.k0 = e0 - P; tp.k1 = e0;

@@ -60,6 +60,11 @@ constexpr int kB200Sms = 148;                    // the part this library is wri
 constexpr size_t kB200SmemPerCta = 232448;
 cudaError_t leaf_mma_launch(const LeafParams& p, const LeafMmaLaunch& l, const LeafMmaBuffers& buf, cudaStream_t s);
 
+// Leaf kernel for layers that fit one cluster's shared memory (rt_leaf_small.cu).
+struct LeafSmallLaunch { int nb, leaf; size_t smem; };
+bool leaf_small_shape(int dtype, int B, int d, int H, int dff, int leaf, size_t max_smem, LeafSmallLaunch* out);
+cudaError_t leaf_small_launch(int dtype, const LeafParams& p, const LeafSmallLaunch& l, cudaStream_t s);
+
 // Pre-pass (Algorithm 1, line 1 and the temporary pair of line 7, hoisted out of the loop).
 struct PrepassParams {
   int B, N, d, H;
