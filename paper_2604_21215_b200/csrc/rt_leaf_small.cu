@@ -72,13 +72,14 @@ __device__ __forceinline__ void send(uint32_t dst, uint32_t bar, const float (&v
                ::"r"(dst), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])), "r"(bar) : "memory");
 }
 
-// Bounded wait that also leaves when another CTA has given up.
+// Bounded wait of a whole warp that also leaves when another CTA has given up; the answer is the same in every lane.
 __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile int* s_abort, SyncArea* sync) {
   unsigned spins = 0;
   unsigned long long t_start = 0;
-  while (!mbar_try_wait(bar, parity)) {
+  bool ok = true;
+  while (ok && !mbar_try_wait_cluster(bar, parity)) {
     if ((++spins & 255u) != 0u) continue;
-    if (*s_abort || *reinterpret_cast<volatile unsigned*>(&sync->abort_flag)) { *s_abort = 1; return false; }
+    if (*s_abort || *reinterpret_cast<volatile unsigned*>(&sync->abort_flag)) { *s_abort = 1; ok = false; break; }
     const unsigned long long now = globaltimer_ns();
     if (t_start == 0) t_start = now;
     else if (now - t_start > kWaitLimitNs) {
@@ -86,10 +87,10 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile
       sync->status = RT_ERR_TIMEOUT;
       __threadfence();
       atomicExch(&sync->abort_flag, 1u);
-      return false;
+      ok = false;
     }
   }
-  return true;
+  return __all_sync(0xffffffffu, ok);
 }
 
 // U consecutive rows of W (row stride K) times the NB vectors at `vec` ([NB][K] fp32): y[u][b], summed over the warp; with

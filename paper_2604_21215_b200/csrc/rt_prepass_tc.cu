@@ -46,7 +46,7 @@ qkv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_n, const __grid_const
   using GemmSmem = GemmSmemT<BN>;
   constexpr int kGemmBN = BN, kGemmStages = GemmSmem::stages;
   constexpr uint32_t kGemmBBytes = GemmSmem::b_bytes;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int M = p.N * p.B, d = p.d;
   const int tiles_per_mat = d / kGemmBN;
   const int which = blockIdx.y / tiles_per_mat;             // 0: q, 1: k~, 2: v~
@@ -77,15 +77,15 @@ qkv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_n, const __grid_const
 
   if (warp == 4) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
+    {
       const CUtensorMap* mw = which == 0 ? &map_wq : (which == 1 ? &map_wk : &map_wv);
       int issued = 0;
       bool ok = true;
       for (int kb = 0; kb < n_kb && ok; ++kb) {
         const int s = kb % kGemmStages;
-        if (kb >= kGemmStages) ok = mbar_wait(empty(s), ((kb / kGemmStages) - 1) & 1, s_abort, sync);
+        if (kb >= kGemmStages) ok = warp_mbar_wait(empty(s), ((kb / kGemmStages) - 1) & 1, s_abort, sync);
         if (!ok) break;
-        mbar_expect_tx(full(s), kGemmABytes + kGemmBBytes);
+        expect_tx_elect(full(s), kGemmABytes + kGemmBBytes);
         tma_load_2d(sbase + GemmSmem::a + s * kGemmABytes, &map_n, full(s), kb * kGemmBK, m0);
         tma_load_2d(sbase + GemmSmem::b + s * kGemmBBytes, mw, full(s), kb * kGemmBK, col0);
         ++issued;
@@ -101,12 +101,12 @@ qkv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_n, const __grid_const
     __syncwarp();
   } else if (warp == 5) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    {
       constexpr uint32_t idesc = make_idesc(kGemmBN, false);
       bool ok = true;
       for (int kb = 0; kb < n_kb && ok; ++kb) {
         const int s = kb % kGemmStages;
-        ok = mbar_wait(full(s), (kb / kGemmStages) & 1, s_abort, sync);
+        ok = warp_mbar_wait(full(s), (kb / kGemmStages) & 1, s_abort, sync);
         if (!ok) break;
         tc_fence_after();
         const uint64_t a0 = make_desc(sbase + GemmSmem::a + s * kGemmABytes, 16, 1024);

@@ -220,7 +220,7 @@ dense_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(smem);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   using DS = DenseSmem<BN>;
   constexpr int kTStages = DS::stages;
   constexpr int kTBN = BN;
@@ -254,14 +254,14 @@ dense_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 
   if (warp == 4) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
+    {
       int issued = 0;
       bool ok = true;
       for (int kb = 0; kb < n_kb && ok; ++kb) {
         const int s = kb % kTStages;
-        if (kb >= kTStages) ok = mbar_wait(empty(s), ((kb / kTStages) - 1) & 1, s_abort, sync);
+        if (kb >= kTStages) ok = warp_mbar_wait(empty(s), ((kb / kTStages) - 1) & 1, s_abort, sync);
         if (!ok) break;
-        mbar_expect_tx(full(s), kTABytes + kTBBytes);
+        expect_tx_elect(full(s), kTABytes + kTBBytes);
         tma_load_2d(sbase + DS::a + s * kTABytes, &map_a, full(s), (kb0 + kb) * kTBK, m0);
         tma_load_2d(sbase + DS::b + s * kTBBytes, &map_w, full(s), (kb0 + kb) * kTBK, n0);
         ++issued;
@@ -277,12 +277,12 @@ dense_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     __syncwarp();
   } else if (warp == 5) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    {
       constexpr uint32_t idesc = make_idesc(kTBN, false);
       bool ok = true;
       for (int kb = 0; kb < n_kb && ok; ++kb) {
         const int s = kb % kTStages;
-        ok = mbar_wait(full(s), (kb / kTStages) & 1, s_abort, sync);
+        ok = warp_mbar_wait(full(s), (kb / kTStages) & 1, s_abort, sync);
         if (!ok) break;
         tc_fence_after();
         const uint64_t a0 = make_desc(sbase + DS::a + s * kTABytes, 16, 1024);
@@ -336,11 +336,11 @@ __device__ __forceinline__ void cluster_sync_all() {
 // TMA load of this CTA's tile whose bytes are reported to the LEADER's barrier at the same offset (bit 24 of a
 // shared::cluster address selects the CTA of the pair)
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
-  asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+  asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n @e cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n}"
                ::"r"(dst), "l"(map), "r"(bar & 0xFEFFFFFFu), "r"(c0), "r"(c1) : "memory");
 }
 __device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
+  asm volatile("{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n elect.sync _|e, 0xffffffff;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
                ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 // Issued by the leader: arrives on the barrier at this offset in BOTH CTAs once the pair's products so far are done
@@ -348,8 +348,8 @@ __device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t a_desc, ui
 __device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
   uint32_t peer;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(bar), "r"(1u));
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(peer) : "memory");
+  asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n @e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(bar) : "memory");
+  asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n @e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(peer) : "memory");
 }
 
 template <int BN>
@@ -360,7 +360,7 @@ dense_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(smem);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   using PS = PairSmem<BN>;
   constexpr int kSt = PS::stages;
   const int rank = (int)cluster_rank();                         // 0: leader (issues the products)
@@ -394,14 +394,14 @@ dense_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   // No role returns early: every thread of both CTAs reaches the cluster barrier at the end.
   if (warp == 4) {
     // ---------------- TMA producer (each CTA: its 128 rows of A, its half of the weight rows) ----------------
-    if (lane == 0) {
+    {
       int issued = 0;
       bool ok = true;
       for (int kb = 0; kb < n_kb && ok; ++kb) {
         const int s = kb % kSt;
-        if (kb >= kSt) ok = mbar_wait(empty(s), ((kb / kSt) - 1) & 1, s_abort, sync);
+        if (kb >= kSt) ok = warp_mbar_wait(empty(s), ((kb / kSt) - 1) & 1, s_abort, sync);
         if (!ok) break;
-        if (rank == 0) mbar_expect_tx(full(s), 2u * (kTABytes + PS::b_bytes));      // the bytes of both CTAs
+        if (rank == 0) expect_tx_elect(full(s), 2u * (kTABytes + PS::b_bytes));      // the bytes of both CTAs
         tma_load_2d_pair(sbase + PS::a + s * kTABytes, &map_a, full(s), (kb0 + kb) * kTBK, m0);
         tma_load_2d_pair(sbase + PS::b + s * PS::b_bytes, &map_w, full(s), (kb0 + kb) * kTBK, n0 + rank * (BN / 2));
         ++issued;
@@ -411,12 +411,12 @@ dense_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     __syncwarp();
   } else if (warp == 5) {
     // ---------------- MMA issuer (leader only) ----------------
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)((2 * kBM) >> 4) << 24);
       bool ok = true;
       for (int kb = 0; kb < n_kb && ok; ++kb) {
         const int s = kb % kSt;
-        ok = mbar_wait(full(s), (kb / kSt) & 1, s_abort, sync);
+        ok = warp_mbar_wait(full(s), (kb / kSt) & 1, s_abort, sync);
         if (!ok) break;
         tc_fence_after();
         const uint64_t a0 = make_desc(sbase + PS::a + s * kTABytes, 16, 1024);
@@ -520,7 +520,7 @@ dense_pair_persist_kernel(const __grid_constant__ CUtensorMap map_a, const __gri
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(smem);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   using PS = PersistSmem;
   constexpr int kSt = PS::stages, BN = 256;
   const int rank = (int)cluster_rank();
@@ -554,7 +554,7 @@ dense_pair_persist_kernel(const __grid_constant__ CUtensorMap map_a, const __gri
   // No role returns early: every thread of both CTAs reaches the cluster barrier at the end.
   if (warp == 4) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
+    {
       int it = 0;
       bool ok = true;
       for (int t = pair_id; t < T && ok; t += pairs) {
@@ -563,9 +563,9 @@ dense_pair_persist_kernel(const __grid_constant__ CUtensorMap map_a, const __gri
         const CUtensorMap* mw = which == 0 ? &map_w : (which == 1 ? &map_w2 : &map_w3);
         for (int kb = 0; kb < n_kb && ok; ++kb, ++it) {
           const int s = it % kSt;
-          if (it >= kSt) ok = mbar_wait(empty(s), ((it / kSt) - 1) & 1, s_abort, sync);
+          if (it >= kSt) ok = warp_mbar_wait(empty(s), ((it / kSt) - 1) & 1, s_abort, sync);
           if (!ok) break;
-          if (rank == 0) mbar_expect_tx(full(s), 2u * (kTABytes + PS::b_bytes));
+          if (rank == 0) expect_tx_elect(full(s), 2u * (kTABytes + PS::b_bytes));
           tma_load_2d_pair(sbase + PS::a + s * kTABytes, &map_a, full(s), kb * kTBK, m0);
           tma_load_2d_pair(sbase + PS::b + s * PS::b_bytes, mw, full(s), kb * kTBK, n0 + rank * (BN / 2));
         }
@@ -574,18 +574,18 @@ dense_pair_persist_kernel(const __grid_constant__ CUtensorMap map_a, const __gri
     __syncwarp();
   } else if (warp == 5) {
     // ---------------- MMA issuer (leader only) ----------------
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)((2 * kBM) >> 4) << 24);
       int it = 0, i = 0;
       bool ok = true;
       for (int t = pair_id; t < T && ok; t += pairs, ++i) {
         const int b = i & 1;
-        if (i >= 2) ok = mbar_wait(acc_empty(b), ((i >> 1) - 1) & 1, s_abort, sync);     // both CTAs have drained this buffer
+        if (i >= 2) ok = warp_mbar_wait(acc_empty(b), ((i >> 1) - 1) & 1, s_abort, sync);     // both CTAs have drained this buffer
         if (!ok) break;
         tc_fence_after();
         for (int kb = 0; kb < n_kb && ok; ++kb, ++it) {
           const int s = it % kSt;
-          ok = mbar_wait(full(s), (it / kSt) & 1, s_abort, sync);
+          ok = warp_mbar_wait(full(s), (it / kSt) & 1, s_abort, sync);
           if (!ok) break;
           tc_fence_after();
           const uint64_t a0 = make_desc(sbase + PS::a + s * kTABytes, 16, 1024);

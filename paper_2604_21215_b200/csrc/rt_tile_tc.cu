@@ -113,7 +113,7 @@ tile_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(smem);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int b = blockIdx.y / p.H, h = blockIdx.y % p.H;
   // copy blockIdx.z of the tile (one level of Algorithm 1 in one launch); the few values derived from it are
   // recomputed where they are used rather than kept in registers across the roles
@@ -159,17 +159,17 @@ tile_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   } else if (warp == kTmaWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
     // ------------------------------ TMA producer ------------------------------
-    if (lane == 0) {
+    {
       const int k0 = p.k0 + shift();
-      mbar_expect_tx(bar(BAR_Q_FULL), kQBytes);
+      expect_tx_elect(bar(BAR_Q_FULL), kQBytes);
       tma_load_4d(sbase + C::q, &map_q, bar(BAR_Q_FULL), 0, h, b, qb);
       int issued = 0;
       bool ok = true;
       for (int kb = 0; kb < n_blocks && ok; ++kb) {
         const int st = kb % kStages;
-        if (kb >= kStages) ok = mbar_wait(bar(BAR_KV_EMPTY + st), ((kb / kStages) - 1) & 1, s_abort, sync);
+        if (kb >= kStages) ok = warp_mbar_wait(bar(BAR_KV_EMPTY + st), ((kb / kStages) - 1) & 1, s_abort, sync);
         if (!ok) break;
-        mbar_expect_tx(bar(BAR_KV_FULL + st), 2 * kKVBytes);
+        expect_tx_elect(bar(BAR_KV_FULL + st), 2 * kKVBytes);
         tma_load_4d(sbase + C::k + st * kKVBytes, &map_k, bar(BAR_KV_FULL + st), 0, h, b, k0 + kb * kBK);
         tma_load_4d(sbase + C::v + st * kKVBytes, &map_v, bar(BAR_KV_FULL + st), 0, h, b, k0 + kb * kBK);
         ++issued;
@@ -188,7 +188,7 @@ tile_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   } else if (warp == kMmaWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
     // ------------------------------ MMA issuer ------------------------------
-    if (lane == 0) {
+    {
       constexpr uint32_t idesc_s = make_idesc(kBK, false);
       constexpr uint32_t idesc_pv = make_idesc(kHeadDim, true);
       // S(kb) = Q . K(kb)^T over the S columns (both operands K-major: 32 bytes along K per step)
@@ -200,8 +200,8 @@ tile_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         for (int ks = 0; ks < kHeadDim / 16; ++ks)
           tc_mma(tmem, q_desc + 2u * ks, k_desc + 2u * ks, idesc_s, ks > 0 ? 1u : 0u);
       };
-      bool ok = mbar_wait(bar(BAR_Q_FULL), 0, s_abort, sync);
-      if (ok) ok = mbar_wait(bar(BAR_KV_FULL), 0, s_abort, sync);
+      bool ok = warp_mbar_wait(bar(BAR_Q_FULL), 0, s_abort, sync);
+      if (ok) ok = warp_mbar_wait(bar(BAR_KV_FULL), 0, s_abort, sync);
       if (ok) {
         tc_fence_after();
         issue_s(0);
@@ -210,8 +210,8 @@ tile_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
       for (int kb = 0; kb < n_blocks && ok; ++kb) {
         const int st = kb % kStages;
         const bool more = kb + 1 < n_blocks;
-        if (more) ok = mbar_wait(bar(BAR_KV_FULL + (kb + 1) % kStages), ((kb + 1) / kStages) & 1, s_abort, sync);
-        if (ok) ok = mbar_wait(bar(BAR_P_READY), kb & 1, s_abort, sync);
+        if (more) ok = warp_mbar_wait(bar(BAR_KV_FULL + (kb + 1) % kStages), ((kb + 1) / kStages) & 1, s_abort, sync);
+        if (ok) ok = warp_mbar_wait(bar(BAR_P_READY), kb & 1, s_abort, sync);
         if (!ok) break;
         tc_fence_after();
         const uint64_t v_desc = make_desc(sbase + C::v + st * kKVBytes, 16, 1024);
