@@ -18,7 +18,7 @@ constexpr int kSmallBatchMax = 64;      // above this the per-token chain runs a
 constexpr int kAutoLeaf = 64;
 
 struct WsLayout {
-  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, dec_words, ll, ll_bytes, hid0, hid1,
+  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, dec_words, ll, ll_bytes, grp, packed, wave, wave_stride, hid0, hid1,
       blk_h, blk_u, blk_c, blk_g, total;
 };
 
@@ -43,6 +43,75 @@ rt_status config_supported(const rt_config* c, int B, bool wide_ok = false) {
   if (c->d_ff % 4) return RT_ERR_UNSUPPORTED;
   if (B > kSmallBatchMax && !(wide_ok && c->sched == RT_SCHED_TILED)) return RT_ERR_UNSUPPORTED;
   return RT_OK;
+}
+
+int leaf_size(const rt_config* c) { return c->leaf ? c->leaf : kAutoLeaf; }
+
+// Which form of the per-token chain a prefill with this configuration and batch runs, and the granularity of
+// Algorithm 1's tiles that goes with it.  Used by run_layer and by rt_plan_counters, so that the modelled schedule is
+// the one that runs (the tensor-core leaf kernel's leaf depends on the shared memory of the part; the planner assumes
+// a B200).
+enum ChainPath { kPathGeneric = 0, kPathMma = 1, kPathWide = 2, kPathBlocks = 3, kPathMmaSplit = 4, kPathGroups = 5 };
+struct Schedule { ChainPath path; int leaf; int sub; };      // sub: sequences per slice (kPathMmaSplit, kPathGroups)
+constexpr int kWideLeafDefault = 16;    // leaf of the dense-product token steps: the in-leaf attention re-reads the leaf's pairs for every position,
+                                        // so short leaves win (p512: 16 -> 41.6 ms, 32 -> 42.3, 64 -> 45.9 per layer)
+constexpr int kMmaSplitMax = 48;         // largest batch that runs as slices of at most 16 sequences through the tensor-core leaf kernel
+constexpr int kGroupsMax = 64;           // largest batch that runs as slices of at most 16 sequences side by side on groups of SMs
+Schedule effective_schedule(const rt_config* c, int B) {
+  if (c->recur_block > 1) return {kPathBlocks, c->recur_block, 0};
+  if (c->sched == RT_SCHED_TILED) {
+    LeafMmaLaunch ml;
+    if (c->dtype == RT_BF16 && B > 16 && B <= kGroupsMax) {
+      // slices side by side, a group of SMs each (rt_leaf_group.cu)
+      const int n_sub = ceil_div(B, 16), sub = ceil_div(B, n_sub);
+      if (leaf_group_shape(sub, c->d_model, c->n_heads, c->d_ff, n_sub, kB200SmemPerCta))
+        return {kPathGroups, c->leaf ? c->leaf : kAutoLeaf, sub};
+    }
+    if (c->dtype == RT_BF16 && B > 16 && B <= kMmaSplitMax) {
+      // Sequences are independent (Sec. 2.2 states the layer per sequence) and a token step of the tensor-core leaf
+      // kernel costs 10 - 14 us whatever its batch, against 53 us for the dense-product step at B = 32: up to 48
+      // sequences run as 2 or 3 slices of at most 16 through that kernel, leaf by leaf, and share the cross tiles.
+      const int n_sub = (B + 15) / 16, sub = (B + n_sub - 1) / n_sub;
+      if (leaf_mma_shape(sub, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml))
+        return {kPathMmaSplit, ml.leaf, sub};
+    }
+    // bf16 batches beyond that (or whose slices the tensor-core leaf kernel does not take) run as dense products from
+    // 24 sequences on, where they overtake the generic kernel (measured at d = 1024: 53 us per token step at B = 32
+    // against 99 us); fp32 keeps the generic kernel up to its limit
+    if (B > kSmallBatchMax || (c->dtype == RT_BF16 && B >= 24)) return {kPathWide, c->leaf ? c->leaf : kWideLeafDefault, 0};
+    if (c->dtype == RT_BF16 && leaf_mma_shape(B, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml))
+      return {kPathMma, ml.leaf, B};
+  }
+  return {kPathGeneric, leaf_size(c), 0};
+}
+
+// The layers of a stack side by side (rt_leaf_group.cu): layer l works on a leaf that layer l-1 finished one launch
+// earlier, up to `places` layers in a launch, a group of SMs each.  places = 0: one layer after the other.
+struct Wave { int places, leaf; };
+constexpr size_t kWaveCacheMax = (size_t)512 << 20;
+constexpr int kWaveFoldMax = 192;        // leaves that begin earlier absorb all earlier pairs inside the leaf kernel
+Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
+  const Wave none = {0, 0};
+  if (n_layers < 2 || N < 2 || c->dtype != RT_BF16 || c->sched != RT_SCHED_TILED || c->recur_block > 1) return none;
+  const int places = n_layers < kGroupJobs ? n_layers : kGroupJobs;
+  if (!leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, places, kB200SmemPerCta)) return none;
+  // A leaf meets all earlier pairs at once when its queries exist (they depend on the layer below, so Algorithm 1's tiles
+  // cannot run ahead): each leaf reads the layer's whole cache so far.  While that cache is small the launch hides it; a large one goes layer by layer.
+  if ((size_t)N * B * c->d_model * 4 > kWaveCacheMax) return none;
+  // Short leaves fill the pipeline of layers sooner, long ones have fewer launches.
+  const int leaf = c->leaf ? c->leaf : N <= 128 ? 16 : N <= 1024 ? 32 : 64;
+  return {places, leaf};
+}
+struct WaveRows { size_t n, q, kt, vt, st_o, st_m, st_l, total; };
+WaveRows wave_rows_layout(const rt_config* c, int B, int leaf) {
+  WaveRows W;
+  const size_t e = esize_of(c->dtype), d = c->d_model, H = c->n_heads, rows = (size_t)B * leaf;
+  size_t o = 0;
+  auto take = [&](size_t bytes) { size_t at = o; o += align_up(bytes, 256); return at; };
+  W.n = take(rows * d * e); W.q = take(rows * d * e); W.kt = take(rows * d * e); W.vt = take(rows * d * e);
+  W.st_o = take(rows * d * 4); W.st_m = take(rows * H * 4); W.st_l = take(rows * H * 4);
+  W.total = o;
+  return W;
 }
 
 // Sequences per launch of the decode kernel: a batch above 16 runs as slices of equal size (the sequences are independent).
@@ -73,6 +142,15 @@ WsLayout ws_layout(const rt_config* c, int B, int N, int n_layers) {
   // g as packed bf16 in fragment order (16 sequence slots), raw k|v as flag-carrying fp32 words
   L.ll_bytes = ((size_t)16 * 3 * (d / 2) + (size_t)16 * (f / 4) + (size_t)B * 2 * d) * 8;
   L.ll = take(L.ll_bytes);
+  // group kernel: one exchange area per group of SMs, the packed weights of a layer (of every layer, when the layers of a
+  // stack run side by side) and, for a stack, a leaf's rows of n, q, k~, v~ and the state per group
+  const Wave wv = stack_wave(c, B, N, n_layers);
+  const Schedule sch = effective_schedule(c, B);
+  const bool grp = N > 1 && (wv.places || sch.path == kPathGroups);
+  L.grp = take(grp ? (size_t)kGroupJobs * leaf_group_words_bytes((int)d, (int)f) : 0);
+  L.packed = take(grp ? (wv.places ? (size_t)n_layers : 1) * leaf_group_packed_bytes((int)d, (int)f, wv.places ? wv.places : ceil_div(B, sch.sub)) : 0);
+  L.wave_stride = wv.places ? wave_rows_layout(c, B, wv.leaf).total : 0;
+  L.wave = take(L.wave_stride * wv.places);
   L.hid0 = take(tok * d * e);
   L.hid1 = take(tok * d * e);
   // recurrence over blocks: the position-wise chain of one block (rows = block length x B)
@@ -101,39 +179,6 @@ bool weights_ok(const rt_layer_weights* w) {
   const void* opt[] = {w->g_attn, w->g_mlp, w->g_kv, w->g_q, w->g_k};
   for (const void* p : opt) if (p && !aligned16(p)) return false;
   return true;
-}
-
-int leaf_size(const rt_config* c) { return c->leaf ? c->leaf : kAutoLeaf; }
-
-// Which form of the per-token chain a prefill with this configuration and batch runs, and the granularity of
-// Algorithm 1's tiles that goes with it.  Used by run_layer and by rt_plan_counters, so that the modelled schedule is
-// the one that runs (the tensor-core leaf kernel's leaf depends on the shared memory of the part; the planner assumes
-// a B200).
-enum ChainPath { kPathGeneric = 0, kPathMma = 1, kPathWide = 2, kPathBlocks = 3, kPathMmaSplit = 4 };
-struct Schedule { ChainPath path; int leaf; int sub; };      // sub: sequences per launch of the tensor-core leaf kernel (kPathMmaSplit)
-constexpr int kWideLeafDefault = 16;    // leaf of the dense-product token steps: the in-leaf attention re-reads the leaf's pairs for every position,
-                                        // so short leaves win (p512: 16 -> 41.6 ms, 32 -> 42.3, 64 -> 45.9 per layer)
-constexpr int kMmaSplitMax = 48;         // largest batch that runs as slices of at most 16 sequences through the tensor-core leaf kernel
-Schedule effective_schedule(const rt_config* c, int B) {
-  if (c->recur_block > 1) return {kPathBlocks, c->recur_block, 0};
-  if (c->sched == RT_SCHED_TILED) {
-    LeafMmaLaunch ml;
-    if (c->dtype == RT_BF16 && B > 16 && B <= kMmaSplitMax) {
-      // Sequences are independent (Sec. 2.2 states the layer per sequence) and a token step of the tensor-core leaf
-      // kernel costs 10 - 14 us whatever its batch, against 53 us for the dense-product step at B = 32: up to 48
-      // sequences run as 2 or 3 slices of at most 16 through that kernel, leaf by leaf, and share the cross tiles.
-      const int n_sub = (B + 15) / 16, sub = (B + n_sub - 1) / n_sub;
-      if (leaf_mma_shape(sub, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml))
-        return {kPathMmaSplit, ml.leaf, sub};
-    }
-    // bf16 batches beyond that (or whose slices the tensor-core leaf kernel does not take) run as dense products from
-    // 24 sequences on, where they overtake the generic kernel (measured at d = 1024: 53 us per token step at B = 32
-    // against 99 us); fp32 keeps the generic kernel up to its limit
-    if (B > kSmallBatchMax || (c->dtype == RT_BF16 && B >= 24)) return {kPathWide, c->leaf ? c->leaf : kWideLeafDefault, 0};
-    if (c->dtype == RT_BF16 && leaf_mma_shape(B, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml))
-      return {kPathMma, ml.leaf, B};
-  }
-  return {kPathGeneric, leaf_size(c), 0};
 }
 
 // ---- optional per-kernel-class timing (rt_profile_enable / rt_profile_read) -----------------
@@ -165,7 +210,21 @@ struct ProfScope {
 };
 
 // State of one API call: the stream and the barrier arrivals enqueued so far.
-struct CallCtx { cudaStream_t s; unsigned bar_base = 0; unsigned seq_base = 0; };
+struct CallCtx { cudaStream_t s; unsigned bar_base = 0; unsigned seq_base = 0; unsigned group_steps[kGroupJobs] = {0, 0, 0, 0}; bool groups_zeroed = false; };
+
+// The exchange areas of the group kernel start from zero, once per API call.
+bool zero_groups(const rt_config* c, unsigned char* ws, const WsLayout& L, CallCtx& ctx) {
+  if (ctx.groups_zeroed) return true;
+  ctx.groups_zeroed = true;
+  return cudaMemsetAsync(ws + L.grp, 0, (size_t)kGroupJobs * leaf_group_words_bytes(c->d_model, c->d_ff), ctx.s) == cudaSuccess;
+}
+GroupCommon group_common(const rt_config* c, int B, unsigned char* ws, const WsLayout& L) {
+  GroupCommon g;
+  memset(&g, 0, sizeof(g));
+  g.d = c->d_model; g.H = c->n_heads; g.dff = c->d_ff; g.Bs = B; g.norm_flags = c->norm_flags; g.eps = c->rms_eps;
+  g.scale_log2 = c->softmax_scale * kLog2e; g.alpha = c->residual_scale; g.sync = (SyncArea*)(ws + L.sync);
+  return g;
+}
 
 // One layer on position-major scratch; x / z given with explicit strides.
 rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x, long long x_bs, long long x_ts,
@@ -283,7 +342,7 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   }
 
   const Schedule plan = effective_schedule(c, B);
-  const bool wide = B > kSmallBatchMax || (plan.path == kPathWide && pos0 == 0);
+  const bool wide = plan.path == kPathWide && pos0 == 0;
   if (wide) {
     // Wide batches (the regime of the paper's own experiments, Sec. 6: B in the hundreds): a token step is a chain
     // of dense products with M = B rows, so it runs on the tensor cores through the same kernels as the parallel
@@ -318,7 +377,7 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
     dp.partial = (float*)(ws + L.ex_part); dp.partial_bytes = (size_t)B * c->n_heads * kMaxChunks * 68 * 4;
     // in-leaf attention re-reads the leaf's pairs for every position (leaf^2 * B * d bytes per leaf), so wide
     // batches default to a shorter leaf
-    const int Lf = plan.path == kPathWide ? plan.leaf : (c->leaf ? c->leaf : kWideLeafDefault), N = n_rows;
+    const int Lf = plan.leaf, N = n_rows;
     for (int s0 = 0; s0 < N; s0 += Lf) {
       const int e0 = s0 + Lf < N ? s0 + Lf : N;
       {
@@ -435,16 +494,116 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
     ProfScope ps(s, kProfLeaf);
     return leaf_small_launch(c->dtype, lp, sl, s) == cudaSuccess;
   };
-  const int Lf = small ? sl.leaf : (use_mma ? ml.leaf : leaf_size(c)), N = n_rows;
+  const bool groups = !small && plan.path == kPathGroups && pos0 == 0 && n_rows > 1;      // (one position: no workspace for it, see ws_layout)
+  const int places = groups ? ceil_div(B, plan.sub) : 0;
+  if (groups) {
+    if (!zero_groups(c, ws, L, ctx)) return RT_ERR_CUDA;
+    const GroupPackLayer pl = {w->w_o, w->w_up, w->w_down, w->w_k, w->w_v, ws + L.packed};
+    ProfScope ps(s, kProfPrepass);
+    if (leaf_group_pack(&pl, 1, c->d_model, c->d_ff, places, s) != cudaSuccess) return RT_ERR_CUDA;
+  }
+  auto leaf_groups = [&](int t0, int t1) -> bool {
+    ProfScope ps(s, kProfLeaf);
+    const size_t e = esize_of(c->dtype);
+    GroupJob jobs[kGroupJobs];
+    memset(jobs, 0, sizeof(jobs));
+    for (int i = 0; i < places; ++i) {
+      GroupJob& j = jobs[i];
+      const int b0 = i * plan.sub;
+      j.packed = ws + L.packed; j.g_mlp = lp.g_mlp; j.g_kv = lp.g_kv; j.g_k = lp.g_k; j.alibi = w->alibi_slopes;
+      j.q = lp.q; j.st_o = lp.st_o; j.st_m = lp.st_m; j.st_l = lp.st_l; j.row_off = 0;
+      j.x = (const unsigned char*)x + (size_t)b0 * x_bs * e; j.x_bs = x_bs; j.x_ts = x_ts;
+      j.z = (unsigned char*)z + (size_t)b0 * z_bs * e; j.z_bs = z_bs; j.z_ts = z_ts;
+      j.k_cache = k_cache; j.v_cache = v_cache; j.t0 = t0; j.t1 = t1; j.key0 = t0;
+      j.B = B - b0 < plan.sub ? B - b0 : plan.sub; j.b0 = b0;
+      j.words = ws + L.grp + (size_t)i * leaf_group_words_bytes(c->d_model, c->d_ff); j.steps = ctx.group_steps[i];
+      ctx.group_steps[i] += (unsigned)(t1 - t0);
+    }
+    return leaf_group_launch(group_common(c, B, ws, L), jobs, places, places, s) == cudaSuccess;
+  };
+  const int Lf = groups ? plan.leaf : small ? sl.leaf : (use_mma ? ml.leaf : leaf_size(c)), N = n_rows;
   for (int s0 = 0; s0 < N; s0 += Lf) {
     const int e0 = s0 + Lf < N ? s0 + Lf : N;
-    if (!(small ? leaf_small(s0, e0) : (use_mma ? leaf_mma(s0, e0) : leaf(s0, e0, s0)))) return RT_ERR_CUDA;
+    if (!(groups ? leaf_groups(s0, e0) : small ? leaf_small(s0, e0) : (use_mma ? leaf_mma(s0, e0) : leaf(s0, e0, s0)))) return RT_ERR_CUDA;
     if (e0 < N) {
       const int P = e0 & -e0;                              // largest power of two dividing the block end
       tp.q0 = e0; tp.q1 = e0 + P < N ? e0 + P : N; tp.k0 = e0 - P; tp.k1 = e0;
       ProfScope ps(s, kProfTile);
       if (tile_launch(c->dtype, tp, s) != cudaSuccess) return RT_ERR_CUDA;
     }
+  }
+  return RT_OK;
+}
+
+// All layers of a stack, several at a time (stack_wave): x^0 in hid[0], layer l reads hid[l & 1] and writes hid[(l + 1) & 1] (the
+// last one `out`, if given); a row is overwritten only after the layer that reads it has finished it.
+rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weights* layers, void* const* hid, void* out, int B, int N, void* const* k_caches,
+                         void* const* v_caches, int N_max, unsigned char* ws, const WsLayout& L, const Wave& wv, CallCtx& ctx) {
+  cudaStream_t s = ctx.s;
+  const int places = wv.places, n_leaves = ceil_div(N, wv.leaf);
+  const size_t e = esize_of(c->dtype), d = c->d_model, packed = leaf_group_packed_bytes(c->d_model, c->d_ff, places);
+  const WaveRows W = wave_rows_layout(c, B, wv.leaf);
+  if (!zero_groups(c, ws, L, ctx)) return RT_ERR_CUDA;
+  std::vector<GroupPackLayer> pl(n_layers);
+  std::vector<int> start(n_layers);                            // wave in which a layer begins
+  for (int l = 0; l < n_layers; ++l) {
+    const rt_layer_weights& w = layers[l];
+    pl[l] = {w.w_o, w.w_up, w.w_down, w.w_k, w.w_v, ws + L.packed + (size_t)l * packed};
+    start[l] = l == 0 ? 0 : start[l - 1] + 1;
+    if (l >= places && start[l] < start[l - places] + n_leaves) start[l] = start[l - places] + n_leaves;
+  }
+  {
+    ProfScope ps(s, kProfPrepass);
+    if (leaf_group_pack(pl.data(), n_layers, c->d_model, c->d_ff, places, s) != cudaSuccess) return RT_ERR_CUDA;
+  }
+  const GroupCommon gc = group_common(c, B, ws, L);
+  const long long bs = (long long)N * d;
+  for (int wave = 0, waves = start[n_layers - 1] + n_leaves; wave < waves; ++wave) {
+    GroupJob jobs[kGroupJobs];
+    memset(jobs, 0, sizeof(jobs));
+    int nj = 0;
+    for (int l = 0; l < n_layers; ++l) {
+      const int k = wave - start[l];
+      if (k < 0 || k >= n_leaves) continue;
+      const rt_layer_weights& w = layers[l];
+      const int place = l % places, t0 = k * wv.leaf, t1 = t0 + wv.leaf < N ? t0 + wv.leaf : N;
+      unsigned char* rows = ws + L.wave + L.wave_stride * place;
+      const void* x = hid[l & 1];
+      PrepassParams pp;
+      memset(&pp, 0, sizeof(pp));
+      pp.B = B; pp.N = t1 - t0; pp.d = c->d_model; pp.H = c->n_heads; pp.norm_flags = c->norm_flags; pp.eps = c->rms_eps; pp.scale_log2 = gc.scale_log2;
+      pp.x = (const unsigned char*)x + (size_t)t0 * d * e; pp.x_bs = bs; pp.x_ts = (long long)d;
+      pp.w_q = w.w_q; pp.w_k = w.w_k; pp.w_v = w.w_v; pp.g_attn = w.g_attn; pp.g_q = w.g_q; pp.g_k = w.g_k;
+      pp.n = rows + W.n; pp.q = rows + W.q; pp.kt = rows + W.kt; pp.vt = rows + W.vt;
+      pp.st_o = (float*)(rows + W.st_o); pp.st_m = (float*)(rows + W.st_m); pp.st_l = (float*)(rows + W.st_l); pp.sync = gc.sync;
+      {
+        ProfScope ps(s, kProfPrepass);
+        if (prepass_launch(c->dtype, pp, s) != cudaSuccess) return RT_ERR_CUDA;
+      }
+      GroupJob& j = jobs[nj++];
+      j.key0 = 0;
+      if (t0 >= kWaveFoldMax) {
+        // the leaf's queries against the whole blocks of 64 earlier pairs; the kernel's attention warps absorb the rest
+        TileParams tp;
+        memset(&tp, 0, sizeof(tp));
+        tp.B = B; tp.d = c->d_model; tp.H = c->n_heads; tp.scale_log2 = gc.scale_log2; tp.alibi = w.alibi_slopes;
+        tp.q = pp.q; tp.k_cache = k_caches[l]; tp.v_cache = v_caches[l]; tp.st_o = pp.st_o; tp.st_m = pp.st_m; tp.st_l = pp.st_l;
+        tp.rows_q = t1 - t0; tp.rows_kv = N_max; tp.sync = gc.sync; tp.q_pos0 = t0;
+        tp.q0 = 0; tp.q1 = t1 - t0; tp.k0 = 0; tp.k1 = t0 & ~63;
+        j.key0 = tp.k1;
+        ProfScope ps(s, kProfTile);
+        if (tile_tc_launch(tp, tp.rows_q, tp.rows_kv, tp.sync, s) != cudaSuccess) return RT_ERR_CUDA;
+      }
+      j.packed = pl[l].out; j.g_mlp = w.g_mlp; j.g_kv = w.g_kv ? w.g_kv : w.g_attn; j.g_k = w.g_k; j.alibi = w.alibi_slopes;
+      j.q = pp.q; j.st_o = pp.st_o; j.st_m = pp.st_m; j.st_l = pp.st_l; j.row_off = t0;
+      j.x = x; j.x_bs = bs; j.x_ts = (long long)d;
+      j.z = l == n_layers - 1 && out ? out : hid[(l + 1) & 1]; j.z_bs = bs; j.z_ts = (long long)d;
+      j.k_cache = k_caches[l]; j.v_cache = v_caches[l]; j.t0 = t0; j.t1 = t1; j.B = B; j.b0 = 0;
+      j.words = ws + L.grp + (size_t)place * leaf_group_words_bytes(c->d_model, c->d_ff); j.steps = ctx.group_steps[place];
+      ctx.group_steps[place] += (unsigned)(t1 - t0);
+    }
+    ProfScope ps(s, kProfLeaf);
+    if (leaf_group_launch(gc, jobs, nj, places, s) != cudaSuccess) return RT_ERR_CUDA;
   }
   return RT_OK;
 }
@@ -702,7 +861,13 @@ rt_status rt_stack_prefill(const rt_config* cfg, int32_t n_layers, const rt_laye
     if (embed_launch(cfg->dtype, emb, ids, B, N, (int)d, vocab, bufs[0], s) != cudaSuccess) return RT_ERR_CUDA;
   }
   const void* cur = bufs[0];
-  for (int l = 0; l < n_layers; ++l) {
+  const Wave wv = stack_wave(cfg, B, N, n_layers);
+  if (wv.places) {
+    st = run_stack_wave(cfg, n_layers, layers, bufs, hidden, B, N, k_caches, v_caches, N_max, ws, L, wv, ctx);
+    if (st != RT_OK) return st;
+    cur = hidden ? hidden : bufs[n_layers & 1];
+  }
+  for (int l = 0; l < n_layers && !wv.places; ++l) {
     void* out = (l == n_layers - 1 && hidden) ? hidden : bufs[(l + 1) & 1];
     st = run_layer(cfg, &layers[l], cur, (long long)N * d, d, out, (long long)N * d, d, B, N, 0, k_caches[l],
                    v_caches[l], N_max, ws, L, ctx);
@@ -879,19 +1044,20 @@ rt_status rt_plan_counters(const rt_config* cfg, int32_t B, int32_t N, int32_t n
   } else {
     // the schedule that runs: leaf (or block) granularity of the chain form this shape takes
     const Schedule plan = effective_schedule(cfg, B);
-    const uint64_t Lf = plan.leaf;
+    const Wave wv = stack_wave(cfg, B, N, n_layers);             // layers side by side: every leaf meets all earlier pairs at once
+    const uint64_t Lf = wv.places ? wv.leaf : plan.leaf;
     for (uint64_t s0 = 0; s0 < n; s0 += Lf) {
       const uint64_t e0 = s0 + Lf < n ? s0 + Lf : n, len = e0 - s0;
       ++leaves;
       // persistent kernels stage their weight rows once per leaf launch; dense products (wide batches, block sweeps)
-      // stream them once per position resp. once per block
-      rd += chain_w * (plan.path == kPathWide ? len : (plan.path == kPathMmaSplit ? (b + plan.sub - 1) / plan.sub : 1));
+      // stream them once per position resp. once per block (the group kernel re-reads them from L2)
+      rd += chain_w * (plan.path == kPathWide ? len : (plan.path == kPathMmaSplit || plan.path == kPathGroups ? (b + plan.sub - 1) / plan.sub : 1));
       kv_leaf += 2 * b * d * e * (len * (len - 1) / 2);  // in-leaf pairs: written a few steps earlier, L2-resident
       fl_leaf += 4 * d * b * (len * (len - 1) / 2);
       if (e0 < n) {
         const uint64_t blocks = e0 / Lf;
-        const uint64_t P = Lf * (blocks & (~blocks + 1));
-        const uint64_t nq = (e0 + P < n ? e0 + P : n) - e0;
+        const uint64_t P = wv.places ? e0 : Lf * (blocks & (~blocks + 1));
+        const uint64_t nq = (wv.places ? (e0 + Lf < n ? e0 + Lf : n) : (e0 + P < n ? e0 + P : n)) - e0;
         ++tiles;
         kv += 2 * P * b * d * e;
         rd += nq * b * d * e + nq * b * (d + 2 * H) * 4;

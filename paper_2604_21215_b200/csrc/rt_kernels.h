@@ -65,6 +65,39 @@ struct LeafSmallLaunch { int nb, leaf; size_t smem; };
 bool leaf_small_shape(int dtype, int B, int d, int H, int dff, int leaf, size_t max_smem, LeafSmallLaunch* out);
 cudaError_t leaf_small_launch(int dtype, const LeafParams& p, const LeafSmallLaunch& l, cudaStream_t s);
 
+// Leaf kernel for several independent (layer, slice) jobs side by side, a group of SMs each (bf16; rt_leaf_group.cu).
+constexpr int kGroupJobs = 4;
+struct GroupJob {
+  const void* packed;                            // W_o, W_up, W_down, W_k, W_v in the order of use (leaf_group_pack)
+  const void *g_mlp, *g_kv, *g_k;                // storage type or NULL
+  const float* alibi;
+  const void* q;                                 // [row, Bs, d]
+  const float *st_o, *st_m, *st_l;
+  const void* x; long long x_bs, x_ts;           // x[b, t, :] of this job's first sequence
+  void* z; long long z_bs, z_ts;
+  void *k_cache, *v_cache;                       // [N_max, Bs, d]
+  int row_off;                                   // position of row 0 of q and of the state
+  int t0, t1;                                    // positions
+  int key0;                                      // first position whose pair is not in the states yet (key0 <= t0)
+  int B, b0;                                     // sequences of the slice, first column in q / state / caches
+  unsigned char* words;                          // exchange area of the job's place, zeroed once per API call
+  unsigned steps;                                // token steps enqueued on that place before this launch in the same call
+};
+struct GroupCommon {
+  int d, H, dff, Bs;                             // Bs: sequences per row of q, state and caches
+  int norm_flags;
+  float eps, scale_log2, alpha;
+  SyncArea* sync;
+};
+constexpr int kGroupPackLayers = 8;
+struct GroupPackLayer { const void *w_o, *w_up, *w_down, *w_k, *w_v; void* out; };
+struct GroupPackArgs { int d, dff, g; GroupPackLayer layer[kGroupPackLayers]; };
+bool leaf_group_shape(int B, int d, int H, int dff, int places, size_t max_smem);   // B: sequences of one job; groups of 148 / places SMs
+size_t leaf_group_words_bytes(int d, int dff);   // exchange area of one place
+size_t leaf_group_packed_bytes(int d, int dff, int places);
+cudaError_t leaf_group_pack(const GroupPackLayer* layers, int n, int d, int dff, int places, cudaStream_t s);
+cudaError_t leaf_group_launch(const GroupCommon& c, const GroupJob* jobs, int n_jobs, int places, cudaStream_t s);   // n_jobs <= places
+
 // Pre-pass (Algorithm 1, line 1 and the temporary pair of line 7, hoisted out of the loop).
 struct PrepassParams {
   int B, N, d, H;
@@ -102,6 +135,7 @@ struct TileParams {
                                                  // launch over [q0,q1) x [k0,k1) covers every query's whole causal prefix; heavy tiles first
   int chained;                                   // row_attn only: launch as a programmatic dependent launch
   void* c_out;                                   // row_attn only: also write the attention value o/l of the row, [B, d] storage type
+  int q_pos0;                                    // position of query row 0 (ALiBi distances; tensor-core kernel without a mask only)
   int rows_q, rows_kv;                           // rows held by the query buffer / the caches (tensor-map bounds)
   SyncArea* sync;
 };

@@ -261,7 +261,7 @@ tile_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
       // applied below), the row constant into the maximum and the exponent offset.  Causal launches turn the
       // pairs at or beyond the row's position into -inf (p = 0).
       float base_l2 = 0.f;
-      if (ALIBI) base_l2 = -slope_l2 * (float)(qi - (p.k0 + shift() + kb * kBK));
+      if (ALIBI) base_l2 = -slope_l2 * (float)(p.q_pos0 + qi - (p.k0 + shift() + kb * kBK));
       auto adjust = [&](uint32_t (&v)[32], int col0) {
         if (ALIBI) {
 #pragma unroll

@@ -1,0 +1,62 @@
+"""The group leaf kernel (several jobs side by side, a group of SMs each) against the oracle: widths whose row slices are ragged
+tiles, MLPs that are no multiple of the width, slices of at most eight and of sixteen sequences, one to several windows and leaves; and
+the layers of a stack side by side: fewer and more layers than places, leaves that absorb earlier pairs with and without a tile launch."""
+import numpy as np
+import pytest
+
+from parity_metrics import check_tensor
+
+pytestmark = pytest.mark.gpu
+
+
+def _gains(lw, d, seed):
+    from paper_2604_21215_b200 import inputs
+    rng = np.random.default_rng(seed)
+    for g in ("g_attn", "g_mlp", "g_kv", "g_q", "g_k"):
+        lw[g] = inputs.round_to(1.0 + 0.2 * rng.standard_normal(d), "bf16")
+
+
+@pytest.mark.parametrize("d,H,dff,B,N,leaf,gains,alibi", [
+    (512, 8, 2048, 17, 18, 0, False, False), (768, 12, 3072, 33, 70, 0, True, False), (640, 10, 2560, 19, 130, 0, True, True),
+    (896, 14, 3584, 20, 33, 32, False, False), (1024, 16, 4096, 64, 20, 16, True, False), (1024, 16, 3872, 32, 67, 0, False, True),
+    (512, 8, 96, 50, 1, 0, False, False), (512, 8, 256, 50, 1, 0, False, False), (512, 8, 96, 20, 20, 0, False, False)])
+def test_slices_match_oracle(d, H, dff, B, N, leaf, gains, alibi):
+    from oracle import RTConfig, RTWeights, layer_seq
+    from paper_2604_21215_b200 import inputs, rt
+    wl = inputs.Workload("groups", 1, B, N, d, H, dff, "bf16")
+    data = inputs.make_inputs(wl, seed=300 + N)
+    lw = data["layers"][0]
+    if gains:
+        _gains(lw, d, N)
+    slopes = [2.0 ** (-8.0 * (h + 1) / H) for h in range(H)] if alibi else None
+    ref = layer_seq(RTConfig(d, H, 64, dff, residual_scale=0.8, alibi_slopes=slopes), RTWeights(**lw), data["x"])
+    layer = rt.Layer(d, H, dff, dtype="bf16", leaf=leaf, residual_scale=0.8)
+    layer.set_weights(dict(lw, alibi_slopes=slopes))
+    got = layer.prefill(data["x"])
+    for name, a, b in zip(("z", "k", "v"), got, ref):
+        check_tensor(f"groups d={d} B={B} N={N}", name, a, b, 2e-2)
+
+
+@pytest.mark.parametrize("L,d,H,dff,B,N,leaf,gains,alibi", [
+    (2, 512, 8, 2048, 1, 2, 0, False, False), (5, 512, 8, 1024, 3, 77, 0, True, True), (9, 448, 7, 896, 1, 17, 0, False, False),
+    (3, 768, 12, 3072, 9, 300, 0, True, True), (6, 512, 8, 512, 2, 230, 16, False, True), (4, 640, 10, 1280, 16, 130, 64, True, False)])
+def test_layers_side_by_side_match_oracle(L, d, H, dff, B, N, leaf, gains, alibi):
+    from oracle import RTConfig, RTWeights, stack_prefill
+    from paper_2604_21215_b200 import inputs, rt
+    V = 91
+    wl = inputs.Workload("wave", L, B, N, d, H, dff, "bf16", vocab=V, residual_scale=1 / np.sqrt(L))
+    data = inputs.make_inputs(wl, seed=500 + N)
+    if gains:
+        for i, lw in enumerate(data["layers"]):
+            _gains(lw, d, N + i)
+    slopes = [2.0 ** (-8.0 * (h + 1) / H) for h in range(H)] if alibi else None
+    ocfg = RTConfig(d, H, 64, dff, residual_scale=wl.residual_scale, alibi_slopes=slopes)
+    hid_ref, logits_ref, caches_ref = stack_prefill(ocfg, [RTWeights(**lw) for lw in data["layers"]], data["emb"], None, data["ids"])
+    st = rt.Stack(L, d, H, dff, V, dtype="bf16", leaf=leaf, residual_scale=wl.residual_scale)
+    st.set_weights([dict(lw, alibi_slopes=slopes) for lw in data["layers"]], data["emb"])
+    hid, logits = st.prefill(data["ids"])
+    check_tensor(f"wave L={L} B={B} N={N}", "hidden", hid, hid_ref, 2e-2)
+    assert np.abs(logits - logits_ref).max() <= 2e-2 * np.abs(logits_ref).max()
+    for l, (k, v) in enumerate(st.caches_numpy(N)):
+        check_tensor(f"wave L={L} layer {l}", "k", k, caches_ref[l][0], 2e-2)
+        check_tensor(f"wave L={L} layer {l}", "v", v, caches_ref[l][1], 2e-2)
