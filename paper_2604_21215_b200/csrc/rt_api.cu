@@ -89,15 +89,17 @@ Schedule effective_schedule(const rt_config* c, int B) {
 // earlier, up to `places` layers in a launch, a group of SMs each.  places = 0: one layer after the other.
 struct Wave { int places, leaf; };
 constexpr size_t kWaveCacheMax = (size_t)512 << 20;
+constexpr int kWaveMaxN = 1024;
 constexpr int kWaveFoldMax = 192;        // leaves that begin earlier absorb all earlier pairs inside the leaf kernel
 Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
   const Wave none = {0, 0};
   if (n_layers < 2 || N < 2 || c->dtype != RT_BF16 || c->sched != RT_SCHED_TILED || c->recur_block > 1) return none;
   const int places = n_layers < kGroupJobs ? n_layers : kGroupJobs;
   if (!leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, places, kB200SmemPerCta)) return none;
-  // A leaf meets all earlier pairs at once when its queries exist (they depend on the layer below, so Algorithm 1's tiles
-  // cannot run ahead): each leaf reads the layer's whole cache so far.  While that cache is small the launch hides it; a large one goes layer by layer.
-  if ((size_t)N * B * c->d_model * 4 > kWaveCacheMax) return none;
+  // A leaf meets all earlier pairs at once when its queries exist (they depend on the layer below, so Algorithm 1's tiles cannot
+  // run ahead): each leaf reads the layer's whole cache so far, which a launch hides only while that is short.  Longer
+  // sequences go layer by layer, as the same layers called one by one do (and give the same bits).
+  if (N > kWaveMaxN || (size_t)N * B * c->d_model * 4 > kWaveCacheMax) return none;
   // Short leaves fill the pipeline of layers sooner, long ones have fewer launches.
   const int leaf = c->leaf ? c->leaf : N <= 128 ? 16 : N <= 1024 ? 32 : 64;
   return {places, leaf};

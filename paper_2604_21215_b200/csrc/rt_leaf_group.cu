@@ -164,7 +164,8 @@ __global__ void __launch_bounds__(256) group_pack_kernel(GroupPackArgs a) {
   }
 }
 
-template <int MB>
+// kQuad: tiles of weight rows a warp works on at a time (one or two pieces).
+template <int MB, int kQuad>
 __global__ void __launch_bounds__(kGThreads, 1) leaf_group_kernel(const __grid_constant__ GroupArgs a, const GroupLayout L) {
   extern __shared__ __align__(128) unsigned char smem[];
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem);
@@ -432,6 +433,12 @@ __global__ void __launch_bounds__(kGThreads, 1) leaf_group_kernel(const __grid_c
           for (int r = 0; r < MB; ++r) av[i][r] = make_uint4(0u, 0u, 0u, 0u);
         unsigned spins = 0;
         unsigned long long t0 = 0;
+        // more than eight sequences: one pair of words first; rounds over all of them would crowd out the attention warps' own loads (33 -> 28 us a step)
+        while (MB == 2 && n_kp > 0) {
+          const uint4 w = ld_two_words_if(base, has0 ? 1u : 0u);
+          if (__all_sync(0xffffffffu, !has0 || (w.y == seq && w.w == seq))) break;
+          if ((++spins & 63u) == 0u && __any_sync(0xffffffffu, group_give_up(sync, s_abort, &t0))) break;
+        }
         while (true) {
           uint4 wa[kKP][MB], wb[kKP][MB];                      // all outstanding words are on their way before any is looked at
 #pragma unroll
@@ -477,44 +484,54 @@ __global__ void __launch_bounds__(kGThreads, 1) leaf_group_kernel(const __grid_c
           if (c == 0) { ssq_red[warp * 16 + g] = sq0; ssq_red[warp * 16 + 8 + g] = sq1; }
         }
       }
-      // ---- products: pieces of two tiles x d columns from the ring ----
+      // ---- products: one or two pieces of the ring at a time ----
       const int n_q = ph == 2 ? nq : 1;
+      const bool keep = tiles <= kQuad;                        // the sums of all stretches stay in registers
+      float acc[kQuad][2][4];
 #pragma unroll 1
       for (int q = 0; q < n_q; ++q) {
         if (q + 1 < n_q) load_g(an, q + 1);
 #pragma unroll 1
-        for (int ti = 0; ti < tiles; ti += kPieceTiles) {
+        for (int ti = 0; ti < tiles; ti += kQuad) {
+          const int slot2 = slot + 1 == L.slots ? 0 : slot + 1;
+          const bool two = kQuad > kPieceTiles && ti + kPieceTiles < tiles;
           ring_wait(full + 8 * slot, par, sync, s_abort);
-          const unsigned char* w = ring + (size_t)slot * kPieceTiles * L.tile_bytes;
-          float acc[kPieceTiles][2][4];
+          if (two) ring_wait(full + 8 * slot2, slot2 ? par : par ^ 1, sync, s_abort);
+          const unsigned char* w0 = ring + (size_t)slot * kPieceTiles * L.tile_bytes;
+          const unsigned char* w1 = ring + (size_t)(two ? slot2 : slot) * kPieceTiles * L.tile_bytes;      // (products of tiles that do not exist are not used)
+          if (q == 0 || !keep) {
 #pragma unroll
-          for (int u = 0; u < kPieceTiles; ++u)
+            for (int u = 0; u < kQuad; ++u)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) { acc[u][0][e] = 0.f; acc[u][1][e] = 0.f; }
+              for (int e = 0; e < 4; ++e) { acc[u][0][e] = 0.f; acc[u][1][e] = 0.f; }
+          }
 #pragma unroll
           for (int i = 0; i < kKP; ++i) {
             if (i < n_kp) {
-              uint4 bw[kPieceTiles];
+              uint4 bw[kQuad];
 #pragma unroll
-              for (int u = 0; u < kPieceTiles; ++u) bw[u] = *reinterpret_cast<const uint4*>(w + (size_t)u * L.tile_bytes + i * 512);   // (a piece of one tile: the second is not used)
+              for (int u = 0; u < kQuad; ++u) bw[u] = *reinterpret_cast<const uint4*>((u < kPieceTiles ? w0 : w1) + (size_t)(u & 1) * L.tile_bytes + i * 512);
 #pragma unroll
-              for (int u = 0; u < kPieceTiles; ++u) {
+              for (int u = 0; u < kQuad; ++u)
                 gmma(acc[u][0], av[i][0].x, MB == 2 ? av[i][MB - 1].x : 0u, av[i][0].y, MB == 2 ? av[i][MB - 1].y : 0u, bw[u].x, bw[u].y);
+#pragma unroll
+              for (int u = 0; u < kQuad; ++u)
                 gmma(acc[u][1], av[i][0].z, MB == 2 ? av[i][MB - 1].z : 0u, av[i][0].w, MB == 2 ? av[i][MB - 1].w : 0u, bw[u].z, bw[u].w);
-              }
             }
           }
           __syncwarp();
-          if (lane == 0) mbar_arrive(empty + 8 * slot);
-          if (++slot == L.slots) { slot = 0; par ^= 1; }
+          if (lane == 0) { mbar_arrive(empty + 8 * slot); if (two) mbar_arrive(empty + 8 * slot2); }
+          for (int k = 0; k < (two ? 2 : 1); ++k)
+            if (++slot == L.slots) { slot = 0; par ^= 1; }
+          if (keep && q + 1 < n_q) continue;
 #pragma unroll
-          for (int u = 0; u < kPieceTiles; ++u) {
+          for (int u = 0; u < kQuad; ++u) {
             if (ti + u < tiles) {
               Part* dst = red + ((ti + u) * kGMma + warp) * 32 + lane;
               Part v;
               v.x = acc[u][0][0] + acc[u][1][0]; v.y = acc[u][0][1] + acc[u][1][1];
               if constexpr (MB == 2) { v.z = acc[u][0][2] + acc[u][1][2]; v.w = acc[u][0][3] + acc[u][1][3]; }
-              if (q > 0) {
+              if (q > 0 && !keep) {
                 const Part old = *dst;
                 v.x += old.x; v.y += old.y;
                 if constexpr (MB == 2) { v.z += old.z; v.w += old.w; }
@@ -624,7 +641,11 @@ cudaError_t leaf_group_launch(const GroupCommon& c, const GroupJob* jobs, int n_
   for (int i = 0; i < n_jobs; ++i) { a.job[i] = jobs[i]; most = jobs[i].B > most ? jobs[i].B : most; }
   const int mb = most > 8 ? 2 : 1;
   GroupLayout L = group_layout(c.d, c.dff, mb, a.gsize, kB200SmemPerCta);
-  const void* fn = mb == 2 ? (const void*)&leaf_group_kernel<2> : (const void*)&leaf_group_kernel<1>;
+  // Two pieces at a time overlap more loads and products, but the longer code costs every phase (the step runs each instruction once or a few
+  // times): at 37 SMs per group, d = 1024, B = 16 a step takes 29.5 us so against 31.3; at d = 768, B = 14 21.4 against 20.3, at d = 256 17.5 against 15.9.
+  const bool wide = mb == 2 && L.s.nt_f > 12;
+  const void* fn = wide ? (const void*)&leaf_group_kernel<2, 2 * kPieceTiles>
+                        : mb == 2 ? (const void*)&leaf_group_kernel<2, kPieceTiles> : (const void*)&leaf_group_kernel<1, kPieceTiles>;
   cudaError_t e = ensure_dynamic_smem(fn, (int)L.total);
   if (e != cudaSuccess) return e;
   void* args[] = {(void*)&a, (void*)&L};
