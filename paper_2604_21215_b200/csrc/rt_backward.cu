@@ -1140,12 +1140,19 @@ __global__ void __launch_bounds__(kRmThreads, 1) bwd_loop_kernel(RowmatParams p,
 // ------------------------------------------------------------------------------------------------ workspace
 struct BwdLayout {
   size_t sync, n, qraw, ktraw, vt, q, kt, r, kraw, k, v, c, h, u, act, gl, lse, D;
-  size_t dK, dV, dkraw, dr, Gz, dpre, du, dh, dc, dq, dkt, dvt, dn, gprod, part, part2, sa, sb, wt, wt5, dzp, qkv16;
+  size_t dK, dV, dkraw, dr, Gz, dpre, du, dh, dc, dq, dkt, dvt, dn, gprod, part, part2, sa, sb, wt, wt5, dzp, qkv16, dvf;
   size_t zero_begin, zero_end, total;
 };
 constexpr int kColParts = 128;
 constexpr int kWideLeaf = 16;
 constexpr int kWideBatchFrom = 32;      // above this many sequences a step of the reverse loop runs as dense products over the batch
+
+// Sequences per launch of the tensor-core leaf kernel of the reverse loop (rt_backward_loop.cu), 0: not taken.
+constexpr int kFastLoopMax = 48;
+int bwd_fast_slice(const rt_config* c, int B) {
+  if (c->dtype != RT_BF16 || (c->flags & RT_FLAG_BACKWARD_STEP_LAUNCHES)) return 0;
+  return bwd_leaf_slice(B, c->d_model, c->n_heads, c->d_ff, kFastLoopMax);
+}
 
 BwdLayout bwd_layout(const rt_config* c, int B, int N) {
   BwdLayout L;
@@ -1166,8 +1173,9 @@ BwdLayout bwd_layout(const rt_config* c, int B, int N) {
   L.part = take((size_t)kColParts * (d > f ? d : f));
   L.part2 = take((size_t)4 * B * d);
   // wide batches: bf16 transposes of the five matrices of the reverse loop, dL/dz in position-major order
+  L.dvf = bwd_fast_slice(c, B) ? take(rows * d) : L.dV;        // final dv of every position (the exchange words of the leaf kernel)
   L.qkv16 = take(3 * rows * d / 2 + 64);                       // bf16 copies of q, k, v for the tile kernels
-  L.wt5 = take((3 * d * d + 2 * d * f) / 2 + 64); L.dzp = B > kWideBatchFrom ? take(rows * d) : o;
+  L.wt5 = take((3 * d * d + 2 * d * f) / 2 + 64); L.dzp = B > kWideBatchFrom && !bwd_fast_slice(c, B) ? take(rows * d) : o;
   // bf16 operands of the tensor-core products (bf16 storage): two [rows, max(d, d_ff)] arrays and one [d, d]
   L.sa = take(rows * (d > f ? d : f) / 2 + 64); L.sb = take(rows * (d > f ? d : f) / 2 + 64); L.wt = take(d * d / 2 + 64);
   L.total = o;
@@ -1375,21 +1383,39 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   unsigned bar_base = 0;
   // leaf of the reverse schedule; wide batches take short leaves (the in-leaf step re-reads and rewrites the fp32
   // pairs of its leaf at every position, the tiles do not)
-  const int Lf = B > kWideBatchFrom ? kWideLeaf : 64;
+  const int Lf = B > kWideBatchFrom && !(kBf16 && bwd_fast_slice(c, B)) ? kWideLeaf : 64;
   // Wide batches (the paper's own regime, Sec. 6): a step of the reverse loop is a dense product over the B rows of the
   // position -- tensor cores for bf16 storage -- between small row-wise kernels, instead of tasks of four sequences.
-  const bool wide = B > kWideBatchFrom;
+  const int fast = kBf16 ? bwd_fast_slice(c, B) : 0;             // sequences per launch of the tensor-core leaf kernel
+  const bool wide = B > kWideBatchFrom && !fast;
   const size_t pos_d = (size_t)B * d, pos_f = (size_t)B * f;
   __nv_bfloat16* WkT = reinterpret_cast<__nv_bfloat16*>(ws + L.wt5);
   __nv_bfloat16 *WvT = WkT + (size_t)d * d, *WoT = WvT + (size_t)d * d, *WdnT = WoT + (size_t)d * d, *WupT = WdnT + (size_t)d * f;
+  if (fast || (wide && tc)) {
+    auto tr = [&](const T* W, int n_out, int n_in, __nv_bfloat16* out) {
+      transpose_bf16_kernel<T><<<dim3(ceil_div(n_in, 32), ceil_div(n_out, 32)), dim3(32, 8), 0, s>>>(W, n_out, n_in, out);
+    };
+    tr(Wk, d, d, WkT); tr(Wv, d, d, WvT); tr(Wo, d, d, WoT); tr(Wdn, d, f, WdnT); tr(Wup, f, d, WupT);
+    RT_TRY(cudaGetLastError());
+  }
+  BwdLeafParams bl;
+  memset(&bl, 0, sizeof(bl));
+  if (fast) {
+    // the exchanged arrays double as their own flags
+    for (size_t at : {L.dkraw, L.dvf, L.dr, L.du, L.dc}) RT_TRY(cudaMemsetAsync(ws + at, 0xff, rows * d * sizeof(float), s));
+    RT_TRY(cudaMemsetAsync(ws + L.dpre, 0xff, rows * f * sizeof(float), s));
+    bl.Bs = B; bl.d = d; bl.H = H; bl.dff = f; bl.z_norm = z_norm ? 1 : 0; bl.pre = pre ? 1 : 0; bl.qk = qk ? 1 : 0;
+    bl.eps = eps; bl.alpha = alpha; bl.scale = c->softmax_scale; bl.scale_log2 = ab.scale_log2;
+    bl.wkT = WkT; bl.wvT = WvT; bl.wdnT = WdnT; bl.wupT = WupT; bl.woT = WoT;
+    bl.g_k = g_k; bl.g_kv = g_kv; bl.g_mlp = g_mlp; bl.alibi = w->alibi_slopes;
+    bl.z = z; bl.z_bs = xbs; bl.z_ts = xts; bl.dz = dz; bl.dz_bs = xbs; bl.dz_ts = xts;
+    bl.q = ab.q; bl.k = ab.k; bl.v = ab.v; bl.kt = ab.kt; bl.vt = ab.vt; bl.c = ab.c; bl.lse = ab.lse; bl.kraw = F(L.kraw); bl.h = F(L.h); bl.act = F(L.act);
+    bl.dK = F(L.dK); bl.dV = F(L.dV); bl.dvf = F(L.dvf); bl.dkraw = F(L.dkraw); bl.dr = F(L.dr); bl.Gz = F(L.Gz); bl.dpre = F(L.dpre);
+    bl.du = F(L.du); bl.dh = F(L.dh); bl.dc = F(L.dc); bl.dkt = F(L.dkt); bl.dvt = F(L.dvt); bl.D = F(L.D);
+    bl.sync = reinterpret_cast<SyncArea*>(ws + L.sync);
+  }
   if (wide) {
     norm_fwd_kernel<float, T><<<warps_grid(rows), tpb, 0, s>>>(dz, xbs, xts, B, (const T*)nullptr, F(L.dzp), rows, d, d, eps, 0);
-    if (tc) {
-      auto tr = [&](const T* W, int n_out, int n_in, __nv_bfloat16* out) {
-        transpose_bf16_kernel<T><<<dim3(ceil_div(n_in, 32), ceil_div(n_out, 32)), dim3(32, 8), 0, s>>>(W, n_out, n_in, out);
-      };
-      tr(Wk, d, d, WkT); tr(Wv, d, d, WvT); tr(Wo, d, d, WoT); tr(Wdn, d, f, WdnT); tr(Wup, f, d, WupT);
-    }
     RT_TRY(cudaGetLastError());
   }
   // out[B, n_in] (+)= al * dY[B, n_out] W[n_out, n_in] for the rows of one position; A_bf = bf16 copy of dY (scale folded in)
@@ -1436,14 +1462,21 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
       const int q1 = e0 + P < N ? e0 + P : N;
       ProfSpanScope span(s, 2);
       if (P % kPB == 0 && (long long)B * H <= 65535) {
-        RT_TRY(launch_chained(attn_bwd_kv_block_kernel, dim3(P / kPB, B * H), dim3(256), kPairBlockSmem, s, !use_coop && !wide, ab, e0, q1,
+        RT_TRY(launch_chained(attn_bwd_kv_block_kernel, dim3(P / kPB, B * H), dim3(256), kPairBlockSmem, s, !use_coop && !wide && !fast, ab, e0, q1,
                               e0 - P, e0));
       } else {
-        RT_TRY(launch_chained(attn_bwd_kv_tile_kernel, dim3(warps_grid((long long)P * B * H)), dim3(tpb), 0, s, !use_coop && !wide, ab,
+        RT_TRY(launch_chained(attn_bwd_kv_tile_kernel, dim3(warps_grid((long long)P * B * H)), dim3(tpb), 0, s, !use_coop && !wide && !fast, ab,
                               e0, q1, e0 - P, e0));
       }
     }
     ProfSpanScope span(s, 1);
+    if (fast) {
+      for (int b0 = 0; b0 < B; b0 += fast) {
+        bl.s0 = s0; bl.e0 = e0; bl.b0 = b0; bl.B = B - b0 < fast ? B - b0 : fast;
+        RT_TRY(bwd_leaf_launch(bl, s));
+      }
+      continue;
+    }
     if (wide) {
       for (int i = e0 - 1; i >= s0; --i) {
         const rt_status st = wide_position(i, s0);
@@ -1532,7 +1565,7 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
     return tc_product(n_out, n_in, (int)rows, SA, SB, out, al, acc);
   };
   if (gr->w_k) RT_TRY(wgrad(gr->w_k, F(L.dkraw), d, F(L.r), d, 1.f, false));
-  if (gr->w_v) RT_TRY(wgrad(gr->w_v, F(L.dV), d, F(L.r), d, 1.f, false));
+  if (gr->w_v) RT_TRY(wgrad(gr->w_v, F(L.dvf), d, F(L.r), d, 1.f, false));
   if (gr->w_k) RT_TRY(wgrad(gr->w_k, F(L.dkt), d, F(L.n), d, 1.f, true));
   if (gr->w_v) RT_TRY(wgrad(gr->w_v, F(L.dvt), d, F(L.n), d, 1.f, true));
   if (gr->w_q) RT_TRY(wgrad(gr->w_q, F(L.dq), d, F(L.n), d, 1.f, false));

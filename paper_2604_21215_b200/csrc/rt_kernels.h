@@ -98,6 +98,25 @@ size_t leaf_group_packed_bytes(int d, int dff, int places);
 cudaError_t leaf_group_pack(const GroupPackLayer* layers, int n, int d, int dff, int places, cudaStream_t s);
 cudaError_t leaf_group_launch(const GroupCommon& c, const GroupJob* jobs, int n_jobs, int places, cudaStream_t s);   // n_jobs <= places
 
+// Reverse loop of the backward pass over one leaf of at most 64 positions (bf16 weights, at most eight sequences; rt_backward_loop.cu).
+// Arrays are position-major fp32 [position, Bs, d | dff] unless said otherwise; dkraw, dvf, dr, dpre, du, dc are filled with 0xFF bytes before.
+struct BwdLeafParams {
+  int B, b0, Bs, d, H, dff;
+  int s0, e0;
+  int z_norm, pre, qk;
+  float eps, alpha, scale, scale_log2;
+  const void *wkT, *wvT, *wdnT, *wupT, *woT;     // transposed weights, bf16
+  const void *g_k, *g_kv, *g_mlp;                // bf16 or NULL
+  const float* alibi;
+  const void* z; long long z_bs, z_ts;           // layer output [B, N, d] bf16
+  const float* dz; long long dz_bs, dz_ts;
+  const float *q, *k, *v, *kt, *vt, *c, *lse, *kraw, *h, *act;
+  float *dK, *dV, *dvf, *dkraw, *dr, *Gz, *dpre, *du, *dh, *dc, *dkt, *dvt, *D;
+  SyncArea* sync;
+};
+int bwd_leaf_slice(int B, int d, int H, int dff, int max_b);
+cudaError_t bwd_leaf_launch(const BwdLeafParams& p, cudaStream_t s);
+
 // Pre-pass (Algorithm 1, line 1 and the temporary pair of line 7, hoisted out of the loop).
 struct PrepassParams {
   int B, N, d, H;
