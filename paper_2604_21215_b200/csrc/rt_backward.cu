@@ -90,9 +90,10 @@ __global__ void to_bf16_kernel(const float* __restrict__ in, __nv_bfloat16* __re
     for (long long j = idx; j < n; ++j) out[j] = __float2bfloat16_rn(in[j]);
   }
 }
-// out[c * R + r] = in[r * C + c]
+// out[c * ld + r] = in[r * C + c]
+// (row stride ld >= R of the output; the entries [R, ld) of each row become zero)
 template <typename TI>
-__global__ void transpose_bf16_kernel(const TI* __restrict__ in, long long R, int C, __nv_bfloat16* __restrict__ out) {
+__global__ void transpose_bf16_kernel(const TI* __restrict__ in, long long R, int C, __nv_bfloat16* __restrict__ out, long long ld) {
   __shared__ float tile[32][33];
   const long long r0 = (long long)blockIdx.y * 32;
   const int c0 = blockIdx.x * 32;
@@ -105,7 +106,7 @@ __global__ void transpose_bf16_kernel(const TI* __restrict__ in, long long R, in
   for (int j = threadIdx.y; j < 32; j += 8) {
     const int c = c0 + j;
     const long long r = r0 + threadIdx.x;
-    if (r < R && c < C) out[(long long)c * R + r] = __float2bfloat16_rn(tile[threadIdx.x][j]);
+    if (r < ld && c < C) out[(long long)c * ld + r] = __float2bfloat16_rn(tile[threadIdx.x][j]);
   }
 }
 
@@ -1177,7 +1178,8 @@ BwdLayout bwd_layout(const rt_config* c, int B, int N) {
   L.qkv16 = take(3 * rows * d / 2 + 64);                       // bf16 copies of q, k, v for the tile kernels
   L.wt5 = take((3 * d * d + 2 * d * f) / 2 + 64); L.dzp = B > kWideBatchFrom && !bwd_fast_slice(c, B) ? take(rows * d) : o;
   // bf16 operands of the tensor-core products (bf16 storage): two [rows, max(d, d_ff)] arrays and one [d, d]
-  L.sa = take(rows * (d > f ? d : f) / 2 + 64); L.sb = take(rows * (d > f ? d : f) / 2 + 64); L.wt = take(d * d / 2 + 64);
+  const size_t rows_k = align_up(rows, 64);
+  L.sa = take(rows_k * (d > f ? d : f) / 2 + 64); L.sb = take(rows_k * (d > f ? d : f) / 2 + 64); L.wt = take(d * d / 2 + 64);
   L.total = o;
   return L;
 }
@@ -1218,7 +1220,7 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   // the operands, fp32 accumulation and fp32 results; otherwise the fp32 product above.
   constexpr bool kBf16 = sizeof(T) == 2;
   const bool tc = kBf16 && d % 128 == 0 && f % 128 == 0;
-  const bool tc_w = tc && rows % 64 == 0;                       // dW = dY^T X contracts over the rows
+  const long long rows_k = align_up(rows, 64);                  // dW = dY^T X contracts over the rows, padded with zeros to whole blocks of 64
   SyncArea* sync = reinterpret_cast<SyncArea*>(ws + L.sync);
   __nv_bfloat16* SA = reinterpret_cast<__nv_bfloat16*>(ws + L.sa);
   __nv_bfloat16* SB = reinterpret_cast<__nv_bfloat16*>(ws + L.sb);
@@ -1235,7 +1237,7 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
     to_bf16_kernel<<<elems_grid((n + 3) / 4), tpb, 0, s>>>(in, out, n);
   };
   auto transpose_f = [&](const float* in, long long R, int C, __nv_bfloat16* out) {
-    transpose_bf16_kernel<float><<<dim3(ceil_div(C, 32), (unsigned)((R + 31) / 32)), dim3(32, 8), 0, s>>>(in, R, C, out);
+    transpose_bf16_kernel<float><<<dim3(ceil_div(C, 32), (unsigned)(rows_k / 32)), dim3(32, 8), 0, s>>>(in, R, C, out, rows_k);
   };
   const float* sa_holds = nullptr;                               // which array SA currently holds as a plain bf16 copy
   // out[rows, n_out] = A[rows, k] W[n_out, k]^T  (a product of the forward pass)
@@ -1248,7 +1250,7 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   auto dgrad_product = [&](const float* dY, int n_out, const T* W, int n_in, float* out, bool acc) -> cudaError_t {
     if (!tc) return gemm<float, T>((int)rows, n_in, n_out, dY, n_out, 1, W, n_in, 1, out, n_in, 1.f, acc, s);
     to_bf16(dY, SA, rows * n_out); sa_holds = nullptr;
-    transpose_bf16_kernel<T><<<dim3(ceil_div(n_in, 32), ceil_div(n_out, 32)), dim3(32, 8), 0, s>>>(W, n_out, n_in, WT);
+    transpose_bf16_kernel<T><<<dim3(ceil_div(n_in, 32), ceil_div(n_out, 32)), dim3(32, 8), 0, s>>>(W, n_out, n_in, WT, n_out);
     return tc_product((int)rows, n_in, n_out, SA, WT, out, 1.f, acc);
   };
   RT_TRY(cudaMemsetAsync(ws + L.sync, 0, sizeof(SyncArea), s));
@@ -1393,7 +1395,7 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   __nv_bfloat16 *WvT = WkT + (size_t)d * d, *WoT = WvT + (size_t)d * d, *WdnT = WoT + (size_t)d * d, *WupT = WdnT + (size_t)d * f;
   if (fast || (wide && tc)) {
     auto tr = [&](const T* W, int n_out, int n_in, __nv_bfloat16* out) {
-      transpose_bf16_kernel<T><<<dim3(ceil_div(n_in, 32), ceil_div(n_out, 32)), dim3(32, 8), 0, s>>>(W, n_out, n_in, out);
+      transpose_bf16_kernel<T><<<dim3(ceil_div(n_in, 32), ceil_div(n_out, 32)), dim3(32, 8), 0, s>>>(W, n_out, n_in, out, n_out);
     };
     tr(Wk, d, d, WkT); tr(Wv, d, d, WvT); tr(Wo, d, d, WoT); tr(Wdn, d, f, WdnT); tr(Wup, f, d, WupT);
     RT_TRY(cudaGetLastError());
@@ -1559,10 +1561,10 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   // parameter matrices: dW[o, i] = sum_rows dY[row, o] X[row, i]
   const float* sb_holds = nullptr;                               // which array SB currently holds transposed
   auto wgrad = [&](float* out, const float* dY, int n_out, const float* X, int n_in, float al, bool acc) -> cudaError_t {
-    if (!tc_w) return gemm<float, float>(n_out, n_in, (int)rows, dY, 1, n_out, X, n_in, 1, out, n_in, al, acc, s);
+    if (!tc) return gemm<float, float>(n_out, n_in, (int)rows, dY, 1, n_out, X, n_in, 1, out, n_in, al, acc, s);
     transpose_f(dY, rows, n_out, SA); sa_holds = nullptr;
     if (sb_holds != X) { transpose_f(X, rows, n_in, SB); sb_holds = X; }
-    return tc_product(n_out, n_in, (int)rows, SA, SB, out, al, acc);
+    return tc_product(n_out, n_in, (int)rows_k, SA, SB, out, al, acc);
   };
   if (gr->w_k) RT_TRY(wgrad(gr->w_k, F(L.dkraw), d, F(L.r), d, 1.f, false));
   if (gr->w_v) RT_TRY(wgrad(gr->w_v, F(L.dvf), d, F(L.r), d, 1.f, false));

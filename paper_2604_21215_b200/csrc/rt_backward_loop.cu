@@ -7,10 +7,11 @@
 //   * every exchanged value is an entry of an array that stage 3 needs anyway ([position, sequence, ...] fp32), written once.  The
 //     arrays are filled with 0xFFFFFFFF (a NaN that no arithmetic produces) before the loop, so the entries are their own flags and a
 //     consumer polls them directly: no barrier across CTAs, no second round trip.  (Five grid barriers per position took 30 us.)
-//   * products run as tf32 m16n8k8 MMAs: rows g carry the leading 11 bits of sequence g's fp32 value, rows g + 8 the next
-//     11, so the sum of the two accumulators is the product of a 22-bit value with the exact bf16 weight, summed in fp32 (what
-//     the fp32 fused multiply-adds did to within their own rounding).  K split over eight warps, weights (transposed once per call)
-//     resident in shared memory for the leaf.
+//   * products run as bf16 m16n8k16 MMAs on the exact split x = hi + mid + lo of every fp32 value into three bf16 terms (24 bits), which
+//     take the MMA's 16 rows: up to four sequences all three terms of each (one MMA per 16 x 8 block of weights), up to eight hi and mid, lo in a
+//     second one.  So nothing is lost against fp32 fused multiply-adds with the bf16 weights.  (tf32 MMAs with two 11-bit terms took 65
+//     cycles each, eight times a bf16 one: 20 us per position.)  K split over eight warps, weights (transposed once per call) resident in
+//     shared memory for the leaf.
 //   * five attention warps per (sequence, head): one on the chain (finishes the pair of position i-1 with the query of position i and
 //     publishes it), four that hold d(k, v) of the leaf's 64 positions in registers (two lanes per position) and absorb the query
 //     while the products run.
@@ -76,10 +77,17 @@ __device__ __forceinline__ void bl_st2(void* p, float a, float b) {
   const unsigned long long w = ((unsigned long long)__float_as_uint(b) << 32) | __float_as_uint(a);
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
 }
-// 16 rows x 8 columns += 16 x 8 (two halves of fp32 values) times 8 x 8
-__device__ __forceinline__ void mma_tf32(float (&c)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0, unsigned b1) {
-  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+__device__ __forceinline__ void bl_mma(float (&c)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0, unsigned b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// A pair of fp32 values as three pairs of bf16 whose sums are the values.
+__device__ __forceinline__ void split3(float x0, float x1, unsigned& hi, unsigned& mid, unsigned& lo) {
+  auto pk = [](float a, float b) { const __nv_bfloat162 v = __floats2bfloat162_rn(a, b); return *reinterpret_cast<const unsigned*>(&v); };
+  hi = pk(x0, x1);
+  x0 -= blo(hi); x1 -= bhi(hi);
+  mid = pk(x0, x1);
+  lo = pk(x0 - blo(mid), x1 - bhi(mid));
 }
 __device__ __forceinline__ float gelu_grad(float a) {          // d/da [a Phi(a)] = Phi(a) + a phi(a)
   return 0.5f * (1.f + erff(a * 0.70710678118654752f)) + a * 0.3989422804014327f * __expf(-0.5f * a * a);
@@ -117,6 +125,8 @@ __device__ __forceinline__ uint2 bl_poll2(const void* p, SyncArea* s, volatile i
   return w;
 }
 
+// SMALL: at most four sequences (all three terms of each in one MMA).
+template <bool SMALL>
 __global__ void __launch_bounds__(kBThreads, 1) bwd_leaf_kernel(const __grid_constant__ BwdLeafParams p, const BLoopLayout L) {
   extern __shared__ __align__(128) unsigned char smem[];
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem);
@@ -142,6 +152,30 @@ __global__ void __launch_bounds__(kBThreads, 1) bwd_leaf_kernel(const __grid_con
   if (warp >= kBMma) {
     // ------------------------------ attention: one (sequence, head) pair ------------------------------
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kBRegsAtt));
+    if (warp == kBChain + 1 && cta >= G - 4) {
+      // Rows that nobody has touched since the sweep (W_up u, h, dz, z) would each cost a trip to HBM in the middle of a step: an idle
+      // warp of four CTAs asks L2 for them, one array each, two positions ahead of the chain (whose first output it watches).
+      const int which = G - 1 - cta, width = which == 0 ? dff : d, esz = which == 3 ? 2 : 4;
+      for (int i = p.e0 + 1; i >= p.s0; --i) {
+        if (i < p.e0 - 2) {
+          unsigned spins = 0;
+          unsigned long long t0 = 0;
+          while (bl_ld2(p.dr + ((size_t)(i + 2) * p.Bs + p.b0) * d).x == kBEmpty) {
+            __nanosleep(200);
+            if ((++spins & 63u) == 0u && bl_give_up(sync, s_abort, &t0)) return;
+          }
+        }
+        if (i >= p.e0) continue;
+        for (int bb = 0; bb < B; ++bb) {
+          const size_t seq = (size_t)(p.b0 + bb), row = (size_t)i * p.Bs + seq;
+          const unsigned char* a = which == 0 ? reinterpret_cast<const unsigned char*>(p.act + row * dff) : which == 1 ? reinterpret_cast<const unsigned char*>(p.h + row * d)
+                                 : which == 2 ? reinterpret_cast<const unsigned char*>(p.dz + seq * p.dz_bs + (size_t)i * p.dz_ts)
+                                              : reinterpret_cast<const unsigned char*>(reinterpret_cast<const __nv_bfloat16*>(p.z) + seq * p.z_bs + (size_t)i * p.z_ts);
+          for (int e = lane * 128; e < width * esz; e += 32 * 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(a + e));
+        }
+      }
+      return;
+    }
     if (!owner || warp > kBChain) return;
     const int b = cta / H, h = cta % H;
     const size_t rstride = (size_t)p.Bs * d, col = (size_t)(p.b0 + b) * d + h * kHeadDim;      // a position's row; this pair's columns
@@ -298,9 +332,9 @@ __global__ void __launch_bounds__(kBThreads, 1) bwd_leaf_kernel(const __grid_con
     stage(L.off_o, L.stride_d, p.woT, d_lo, nd, d, 0);
   }
   constexpr int KC = 8;                                        // k-steps of 16 per round
-  const int g = lane >> 2, c = lane & 3;
-  const bool has = g < B;
-  const size_t brow = (size_t)(p.b0 + (has ? g : 0));          // sequence of this lane's rows
+  const int g = lane >> 2, c = lane & 3, sq = SMALL ? g & 3 : g;  // sq: sequence of this lane's rows
+  const bool has = sq < B;
+  const size_t brow = (size_t)(p.b0 + (has ? sq : 0));
   const float inv_d = 1.0f / (float)d;
   const __nv_bfloat16 *z = reinterpret_cast<const __nv_bfloat16*>(p.z), *g_kv = reinterpret_cast<const __nv_bfloat16*>(p.g_kv), *g_mlp = reinterpret_cast<const __nv_bfloat16*>(p.g_mlp);
   float gz[KC][4];                                             // Gz of this warp's stretch of d
@@ -309,20 +343,6 @@ __global__ void __launch_bounds__(kBThreads, 1) bwd_leaf_kernel(const __grid_con
 
   for (int i = p.e0 - 1; i >= p.s0; --i) {
     const size_t row = (size_t)i * p.Bs + brow;
-    // rows that nobody has touched since the sweep come from HBM: ask L2 for the next position's, one CTA per array
-    if (i > p.s0) {
-      const size_t nrow = (size_t)(i - 1) * p.Bs + p.b0;
-      for (int l = tid; l < B * dff / 32; l += kBMmaThreads) {
-        const int which = cta % 4;
-        if (cta >= 4) break;
-        const int bb = (l * 32) / dff, e = l * 32 - bb * dff;
-        const float* a = which == 0 ? p.act + (nrow + bb) * dff + e : nullptr;
-        if (which == 1 && e < d) a = p.h + (nrow + bb) * d + e;
-        if (which == 2 && e < d) a = p.dz + (size_t)(p.b0 + bb) * p.dz_bs + (size_t)(i - 1) * p.dz_ts + e;
-        if (which == 3 && e < d) a = reinterpret_cast<const float*>(z + (size_t)(p.b0 + bb) * p.z_bs + (size_t)(i - 1) * p.z_ts + e);
-        if (a) asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
-      }
-    }
 #pragma unroll 1
     for (int ph = 0; ph < 4; ++ph) {                           // 0: W_k | W_v   1: W_down   2: W_up   3: W_o
       const int K = ph == 0 ? 2 * d : ph == 2 ? dff : d, stride = ph == 0 ? L.stride_2d : ph == 2 ? L.stride_f : L.stride_d;
@@ -383,43 +403,58 @@ __global__ void __launch_bounds__(kBThreads, 1) bwd_leaf_kernel(const __grid_con
             const __nv_bfloat16* gain = ph == 1 ? g_kv : g_mlp;
             float ss = 0.f, tu = 0.f;
 #pragma unroll
-            for (int s = 0; s < KC; ++s) {
-              if (ks0 + s < ks1) {
-                if (gain) {
-                  const uint2 w = *reinterpret_cast<const uint2*>(gain + kb + 16 * s);
-                  x[s][0] *= blo(w.x); x[s][1] *= bhi(w.x); x[s][2] *= blo(w.y); x[s][3] *= bhi(w.y);
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) { ss = fmaf(uu[s][e], uu[s][e], ss); tu = fmaf(x[s][e], uu[s][e], tu); }
+            for (int s = 0; s < KC; ++s) {                     // (steps beyond the stretch: x = 0, u masked)
+              const int k = ks0 + s < ks1 ? kb + 16 * s : 4 * c;
+              const float on = ks0 + s < ks1 ? 1.f : 0.f;
+              if (gain) {
+                const uint2 w = *reinterpret_cast<const uint2*>(gain + k);
+                x[s][0] *= blo(w.x); x[s][1] *= bhi(w.x); x[s][2] *= blo(w.y); x[s][3] *= bhi(w.y);
               }
+#pragma unroll
+              for (int e = 0; e < 4; ++e) { ss = fmaf(on * uu[s][e], uu[s][e], ss); tu = fmaf(x[s][e], uu[s][e], tu); }
             }
             ss += __shfl_xor_sync(0xffffffffu, ss, 1); ss += __shfl_xor_sync(0xffffffffu, ss, 2);
             tu += __shfl_xor_sync(0xffffffffu, tu, 1); tu += __shfl_xor_sync(0xffffffffu, tu, 2);
-            float2* sq = reinterpret_cast<float2*>(smem + L.off_ssq) + (ph >> 1) * kBMma * 8;
-            if (c == 0) sq[warp * 8 + g] = make_float2(ss, tu);
+            float2* sums = reinterpret_cast<float2*>(smem + L.off_ssq) + (ph >> 1) * kBMma * 8;
+            if (c == 0) sums[warp * 8 + g] = make_float2(ss, tu);
             b_sync();
             ss = 0.f; tu = 0.f;
 #pragma unroll
-            for (int w = 0; w < kBMma; ++w) { const float2 v = sq[w * 8 + g]; ss += v.x; tu += v.y; }
+            for (int w = 0; w < kBMma; ++w) { const float2 v = sums[w * 8 + g]; ss += v.x; tu += v.y; }
             inv = rsqrtf(ss * inv_d + p.eps);
             coef = tu * inv * inv_d * inv;                     // mean(t uh) inv:  du = inv t - u inv (inv mean)
           } else inv = 1.f;
 #pragma unroll
           for (int s = 0; s < KC; ++s) {
-            if (ks0 + s < ks1) {
 #pragma unroll
-              for (int e = 0; e < 4; ++e) x[s][e] = gz[s][e] + inv * (x[s][e] - (norm ? uu[s][e] * coef : 0.f));
-              if (ph == 1) {
+            for (int e = 0; e < 4; ++e) x[s][e] = gz[s][e] + inv * (x[s][e] - (norm ? uu[s][e] * coef : 0.f));
+            if (ph == 1) {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) gz[s][e] = x[s][e];
-              }
-              // kept for the products over all rows: each column by the CTA that owns it (pairs of columns)
-              float* keep = (ph == 1 ? p.Gz : p.dh) + row * d;
-              const int k = kb + 16 * s;
-              if (has && k >= d_lo && k < d_lo + nd) *reinterpret_cast<float2*>(keep + k) = make_float2(x[s][0], x[s][1]);
-              if (has && k + 2 >= d_lo && k + 2 < d_lo + nd) *reinterpret_cast<float2*>(keep + k + 2) = make_float2(x[s][2], x[s][3]);
+              for (int e = 0; e < 4; ++e) gz[s][e] = x[s][e];
             }
           }
+          // kept for the products over all rows: each column by the CTA that owns it (pairs of columns)
+          float* keep = (ph == 1 ? p.Gz : p.dh) + row * d;
+          if (has && (!SMALL || g < 4) && kb - 4 * c < d_lo + nd && ks1 * 16 > d_lo) {
+#pragma unroll
+            for (int s = 0; s < KC; ++s) {
+              const int k = kb + 16 * s;
+              if (ks0 + s < ks1 && k >= d_lo && k < d_lo + nd) *reinterpret_cast<float2*>(keep + k) = make_float2(x[s][0], x[s][1]);
+              if (ks0 + s < ks1 && k + 2 >= d_lo && k + 2 < d_lo + nd) *reinterpret_cast<float2*>(keep + k + 2) = make_float2(x[s][2], x[s][3]);
+            }
+          }
+        }
+        const int n_here = ks1 - ks0 - s0;
+        // the three terms of every value: rows g (hi | mid) and g + 8 (lo), or hi, mid and lo
+        unsigned fa[KC][SMALL ? 4 : 6];
+#pragma unroll
+        for (int s = 0; s < KC; ++s) {
+          unsigned h0, m0, l0, h1, m1, l1;
+          if (s >= n_here) { x[s][0] = 0.f; x[s][1] = 0.f; x[s][2] = 0.f; x[s][3] = 0.f; }
+          split3(x[s][0], x[s][1], h0, m0, l0);
+          split3(x[s][2], x[s][3], h1, m1, l1);
+          if constexpr (SMALL) { fa[s][0] = g < 4 ? h0 : m0; fa[s][1] = g < 4 ? l0 : 0u; fa[s][2] = g < 4 ? h1 : m1; fa[s][3] = g < 4 ? l1 : 0u; }
+          else { fa[s][0] = h0; fa[s][1] = m0; fa[s][2] = h1; fa[s][3] = m1; fa[s][4] = l0; fa[s][5] = l1; }
         }
         // (several tiles only where one round covers the contraction)
 #pragma unroll 1
@@ -428,18 +463,10 @@ __global__ void __launch_bounds__(kBThreads, 1) bwd_leaf_kernel(const __grid_con
           const int r = t * 8 + g < rows ? t * 8 + g : rows - 1;
           const unsigned char* wrow = wbase + ((size_t)r * stride + kb + 16 * s0) * 2;
 #pragma unroll
-          for (int s = 0; s < KC; ++s) {
-            if (ks0 + s0 + s < ks1) {
-              unsigned hi[4], lo[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                hi[e] = __float_as_uint(x[s][e]) & 0xffffe000u;
-                lo[e] = __float_as_uint(x[s][e] - __uint_as_float(hi[e]));
-              }
-              const uint2 w = *reinterpret_cast<const uint2*>(wrow + s * 32);
-              mma_tf32(acc0, hi[0], lo[0], hi[1], lo[1], w.x << 16, w.x & 0xffff0000u);
-              mma_tf32(acc1, hi[2], lo[2], hi[3], lo[3], w.y << 16, w.y & 0xffff0000u);
-            }
+          for (int s = 0; s < KC; ++s) {                       // (no branch around a product: steps beyond the stretch multiply zeros)
+            const uint2 w = *reinterpret_cast<const uint2*>(wrow + (s < n_here ? s * 32 : 0));
+            if constexpr (SMALL) bl_mma((s & 1) ? acc1 : acc0, fa[s][0], fa[s][1], fa[s][2], fa[s][3], w.x, w.y);
+            else { bl_mma(acc0, fa[s][0], fa[s][1], fa[s][2], fa[s][3], w.x, w.y); bl_mma(acc1, fa[s][4], 0u, fa[s][5], 0u, w.x, w.y); }
           }
           red[(t * kBMma + warp) * 32 + lane] = make_float2((acc0[0] + acc0[2]) + (acc1[0] + acc1[2]), (acc0[1] + acc0[3]) + (acc1[1] + acc1[3]));
         }
@@ -456,7 +483,8 @@ __global__ void __launch_bounds__(kBThreads, 1) bwd_leaf_kernel(const __grid_con
         float y0 = 0.f, y1 = 0.f;
 #pragma unroll
         for (int w = 0; w < kBMma; ++w) { const float2 v = red[(warp * kBMma + w) * 32 + lane]; y0 += v.x; y1 += v.y; }
-        if (has && rl < rows) {
+        if (SMALL) { y0 += __shfl_xor_sync(0xffffffffu, y0, 16); y1 += __shfl_xor_sync(0xffffffffu, y1, 16); }
+        if (has && rl < rows && (!SMALL || g < 4)) {
           if (ph == 0) bl_st2(p.dr + row * d + d_lo + rl, y0, y1);
           else if (ph == 1) {
             const float2 a = *reinterpret_cast<const float2*>(p.act + row * dff + f_lo + rl);
@@ -482,11 +510,12 @@ int bwd_leaf_slice(int B, int d, int H, int dff, int max_b) {
 
 cudaError_t bwd_leaf_launch(const BwdLeafParams& p, cudaStream_t s) {
   BLoopLayout L = bloop_layout(p.d, p.dff, kB200Sms);
-  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(&bwd_leaf_kernel), (int)L.total);
+  const void* fn = p.B <= 4 ? reinterpret_cast<const void*>(&bwd_leaf_kernel<true>) : reinterpret_cast<const void*>(&bwd_leaf_kernel<false>);
+  cudaError_t e = ensure_dynamic_smem(fn, (int)L.total);
   if (e != cudaSuccess) return e;
   BwdLeafParams pp = p;
   void* args[] = {(void*)&pp, (void*)&L};
-  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&bwd_leaf_kernel), dim3(kB200Sms), dim3(kBThreads), args, L.total, s);
+  return cudaLaunchCooperativeKernel(fn, dim3(kB200Sms), dim3(kBThreads), args, L.total, s);
 }
 
 }  // namespace rt

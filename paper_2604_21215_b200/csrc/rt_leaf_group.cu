@@ -187,6 +187,7 @@ __global__ void __launch_bounds__(kGThreads, 1) leaf_group_kernel(const __grid_c
 
   if (tid == 0) {
     *s_abort = *reinterpret_cast<volatile unsigned*>(&sync->abort_flag) ? 1 : 0;
+#pragma unroll 1
     for (int i = 0; i < L.slots; ++i) { mbar_init(full + 8 * i, 1); mbar_init(empty + 8 * i, kGMma); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -200,28 +201,32 @@ __global__ void __launch_bounds__(kGThreads, 1) leaf_group_kernel(const __grid_c
       uint32_t par = 0;
       bool ok = true, fresh = true;                            // fresh: first round of the ring, nothing to wait for
       const unsigned char* src = reinterpret_cast<const unsigned char*>(J.packed) + (size_t)cta * L.s.tiles * L.tile_bytes;
-      auto next = [&](int tiles) {
-        if (!ok) return;
-        if (!fresh) ok = ring_wait(empty + 8 * slot, par, sync, s_abort);
-        if (!ok) return;
-        const uint32_t bar = full + 8 * slot, dst = smem_u32(smem + L.off_ring) + (uint32_t)slot * kPieceTiles * L.tile_bytes, bytes = (uint32_t)tiles * L.tile_bytes;
-        expect_tx_elect(bar, bytes);
-        asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n @e cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n}"
-                     ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-        src += bytes;
-        if (++slot == L.slots) { slot = 0; if (!fresh) par ^= 1; fresh = false; }
-      };
-      auto run = [&](int tiles) { for (int t = 0; t < tiles; t += kPieceTiles) next(tiles - t < kPieceTiles ? tiles - t : kPieceTiles); };
+      // (one copy of the code, rolled: what this warp runs shares the instruction cache with the chain)
+#pragma unroll 1
       for (int j = 0; j < n && ok; ++j) {
-        const unsigned char* const first = src;
-        run(nt_d);
-        run(nt_f);
-        for (int q = 0; q < nq; ++q) run(nt_d);
-        run(2 * nt_d);
-        src = first;
+        const unsigned char* at = src;
+#pragma unroll 1
+        for (int r = 0; r < nq + 3 && ok; ++r) {               // W_o, W_up, the stretches of W_down, W_k | W_v
+          int left = r == 1 ? nt_f : r == nq + 2 ? 2 * nt_d : nt_d;
+#pragma unroll 1
+          while (left > 0) {
+            if (!fresh) ok = ring_wait(empty + 8 * slot, par, sync, s_abort);
+            if (!ok) break;
+            const uint32_t bar = full + 8 * slot, dst = smem_u32(smem + L.off_ring) + (uint32_t)slot * kPieceTiles * L.tile_bytes;
+            const uint32_t bytes = (uint32_t)(left < kPieceTiles ? left : kPieceTiles) * L.tile_bytes;
+            expect_tx_elect(bar, bytes);
+            asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n @e cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n}"
+                         ::"r"(dst), "l"(at), "r"(bytes), "r"(bar) : "memory");
+            at += bytes;
+            left -= kPieceTiles;
+            if (++slot == L.slots) { slot = 0; if (!fresh) par ^= 1; fresh = false; }
+          }
+        }
       }
       if (!ok)                                                 // gave up: let the copies in flight land (bounded)
+#pragma unroll 1
         for (int i = 0; i < L.slots; ++i)
+#pragma unroll 1
           for (int spins = 0; spins < (1 << 13); ++spins) mbar_try_wait(full + 8 * i, 0);
       return;
     }
@@ -271,23 +276,52 @@ __global__ void __launch_bounds__(kGThreads, 1) leaf_group_kernel(const __grid_c
         for (int e = 0; e < 32; e += 4) *reinterpret_cast<float4*>(st + e0 + e) = make_float4(o[e], o[e + 1], o[e + 2], o[e + 3]);
         if (e0 == 0) { st[kHeadDim] = m; st[kHeadDim + 1] = l; }
       };
-      auto open_window = [&](int first, int known) {           // queries first ..., positions key0 .. t0 + known - 1 are in the cache
-        w0 = first;
-        const int i = min(first + qi, n - 1);
-        const size_t row = (size_t)(J.t0 - J.row_off + i), at = row * qrow + qcol + e0;
-#pragma unroll
-        for (int e = 0; e < 32; e += 8) {
-          const uint4 w = *reinterpret_cast<const uint4*>(q + at + e);
-          qr[e / 2] = w.x; qr[e / 2 + 1] = w.y; qr[e / 2 + 2] = w.z; qr[e / 2 + 3] = w.w;
-        }
-#pragma unroll
-        for (int e = 0; e < 32; e += 4) {
-          const float4 w = *reinterpret_cast<const float4*>(J.st_o + at + e);
-          o[e] = w.x; o[e + 1] = w.y; o[e + 2] = w.z; o[e + 3] = w.w;
-        }
-        m = J.st_m[(row * C.Bs + bc) * H + h]; l = J.st_l[(row * C.Bs + bc) * H + h];
-        const int key1 = J.t0 + known;
+      // One copy of everything long (what these warps run shares the instruction cache with the chain): iteration j = -1 opens the
+      // first window, iteration j >= 0 finishes query j + 1 and absorbs pair j -- or opens the next window and absorbs every earlier pair.
+#pragma unroll 1
+      for (int j = -1; j < n; ++j) {
+        const unsigned seq = J.steps + (unsigned)(j + 1);      // step that reveals position t0 + j
         unsigned kw[4], vw[4];
+        kw[0] = vw[0] = 0u;
+        if (j >= 0) {
+          float q0 = 0.f, q1 = 0.f;
+          if (j + 1 < n) {
+            const unsigned qw = *reinterpret_cast<const unsigned*>(q + (size_t)(J.t0 - J.row_off + j + 1) * qrow + qcol + 2 * lane);
+            q0 = glo(qw); q1 = ghi(qw);
+          }
+          uint4 ka, va;
+          {
+            unsigned spins = 0;
+            unsigned long long t0 = 0;
+            while (true) {
+              ka = ld_two_words(kv_at);
+              va = ld_two_words(kv_at + (size_t)d * 8);
+              if (__all_sync(0xffffffffu, ka.y == seq && ka.w == seq && va.y == seq && va.w == seq)) break;
+              if ((++spins & 63u) == 0u && __any_sync(0xffffffffu, group_give_up(sync, s_abort, &t0))) break;
+            }
+          }
+          const float2 kr = make_float2(__uint_as_float(ka.x), __uint_as_float(ka.z)), vr = make_float2(__uint_as_float(va.x), __uint_as_float(va.z));
+          // Eq. (1): qkRMS over the head, then the storage rounding the cache applies
+          const float rk = qkn ? rsqrtf(warp_sum(kr.x * kr.x + kr.y * kr.y) * (1.0f / kHeadDim) + C.eps) : 1.0f;
+          const unsigned kq = gpack(kr.x * rk * gk0, kr.y * rk * gk1), vq = gpack(vr.x, vr.y);
+          const float k0 = glo(kq), k1 = ghi(kq), v0 = glo(vq), v1 = ghi(vq);
+          if (j + 1 < n) {
+            const float s = warp_sum(q0 * k0 + q1 * k1) * C.scale_log2 - slope;
+            const float mo = st[kHeadDim], mn = fmaxf(mo, s), corr = exp2f(mo - mn), pj = exp2f(s - mn);
+            const float il = 1.0f / (st[kHeadDim + 1] * corr + pj);
+            const float2 oo = *reinterpret_cast<const float2*>(st + 2 * lane);
+            st_flag(c_at, gpack((oo.x * corr + pj * v0) * il, (oo.y * corr + pj * v1) * il), seq + 1u);
+          }
+          const size_t crow = (size_t)(J.t0 + j) * qrow + qcol + 2 * lane;
+          *reinterpret_cast<unsigned*>(kc + crow) = kq;
+          *reinterpret_cast<unsigned*>(vc + crow) = vq;
+          if (j + 2 >= n) continue;
+          kw[0] = kq; vw[0] = vq;
+          __syncwarp();
+        }
+        const bool open = j < 0 || j + 2 == w0 + kWin;
+        const int key1 = J.t0 + j + 1;
+        int key = J.t0 + j;                                    // pairs [key, key1) to absorb
         auto fetch = [&](int j0) {                             // four pairs in flight
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
@@ -295,73 +329,47 @@ __global__ void __launch_bounds__(kGThreads, 1) leaf_group_kernel(const __grid_c
             kw[u] = __ldcg(reinterpret_cast<const unsigned*>(kc + kr)); vw[u] = __ldcg(reinterpret_cast<const unsigned*>(vc + kr));
           }
         };
-        if (J.key0 < key1) fetch(J.key0);
-        for (int j = J.key0; j < key1; j += 4) {
+        if (open) {
+          w0 = j < 0 ? 0 : j + 2;
+          const int i = min(w0 + qi, n - 1);
+          const size_t row = (size_t)(J.t0 - J.row_off + i), at = row * qrow + qcol + e0;
+#pragma unroll
+          for (int e = 0; e < 32; e += 8) {
+            const uint4 w = *reinterpret_cast<const uint4*>(q + at + e);
+            qr[e / 2] = w.x; qr[e / 2 + 1] = w.y; qr[e / 2 + 2] = w.z; qr[e / 2 + 3] = w.w;
+          }
+#pragma unroll
+          for (int e = 0; e < 32; e += 4) {
+            const float4 w = *reinterpret_cast<const float4*>(J.st_o + at + e);
+            o[e] = w.x; o[e + 1] = w.y; o[e + 2] = w.z; o[e + 3] = w.w;
+          }
+          m = J.st_m[(row * C.Bs + bc) * H + h]; l = J.st_l[(row * C.Bs + bc) * H + h];
+          key = J.key0;
+          if (key < key1) fetch(key);
+        }
+#pragma unroll 1
+        for (; key < key1; key += 4) {
           __syncwarp();
+          const int here = min(4, key1 - key);
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            *reinterpret_cast<float2*>(fin + u * 128 + 2 * lane) = make_float2(glo(kw[u]), ghi(kw[u]));
-            *reinterpret_cast<float2*>(fin + u * 128 + kHeadDim + 2 * lane) = make_float2(glo(vw[u]), ghi(vw[u]));
+            if (u < here) {
+              *reinterpret_cast<float2*>(fin + u * 128 + 2 * lane) = make_float2(glo(kw[u]), ghi(kw[u]));
+              *reinterpret_cast<float2*>(fin + u * 128 + kHeadDim + 2 * lane) = make_float2(glo(vw[u]), ghi(vw[u]));
+            }
           }
           __syncwarp();
-          if (j + 4 < key1) fetch(j + 4);
+          if (key + 4 < key1) fetch(key + 4);
 #pragma unroll 1
-          for (int u = 0; u < 4 && j + u < key1; ++u) fold(fin + u * 128, J.t0 + first + qi - j - u);
+          for (int u = 0; u < here; ++u) fold(fin + u * 128, J.t0 + w0 + qi - key - u);
         }
-        __syncwarp();
-      };
-      open_window(0, 0);
-      if (qi == 0) leave_state();
-      __syncwarp();
-      {
-        const float il = 1.f / st[kHeadDim + 1];
-        const float2 oo = *reinterpret_cast<const float2*>(st + 2 * lane);
-        st_flag(c_at, gpack(oo.x * il, oo.y * il), J.steps + 1u);
-      }
-      __syncwarp();
-      if (qi == 1) leave_state();
-      __syncwarp();
-      for (int j = 0; j < n; ++j) {
-        const unsigned seq = J.steps + (unsigned)j + 1u;       // step that reveals position t0 + j
-        float q0 = 0.f, q1 = 0.f;
-        if (j + 1 < n) {
-          const unsigned qw = *reinterpret_cast<const unsigned*>(q + (size_t)(J.t0 - J.row_off + j + 1) * qrow + qcol + 2 * lane);
-          q0 = glo(qw); q1 = ghi(qw);
-        }
-        uint4 kw, vw;
-        {
-          unsigned spins = 0;
-          unsigned long long t0 = 0;
-          while (true) {
-            kw = ld_two_words(kv_at);
-            vw = ld_two_words(kv_at + (size_t)d * 8);
-            if (__all_sync(0xffffffffu, kw.y == seq && kw.w == seq && vw.y == seq && vw.w == seq)) break;
-            if ((++spins & 63u) == 0u && __any_sync(0xffffffffu, group_give_up(sync, s_abort, &t0))) break;
-          }
-        }
-        const float2 kr = make_float2(__uint_as_float(kw.x), __uint_as_float(kw.z)), vr = make_float2(__uint_as_float(vw.x), __uint_as_float(vw.z));
-        // Eq. (1): qkRMS over the head, then the storage rounding the cache applies
-        const float rk = qkn ? rsqrtf(warp_sum(kr.x * kr.x + kr.y * kr.y) * (1.0f / kHeadDim) + C.eps) : 1.0f;
-        const unsigned kq = gpack(kr.x * rk * gk0, kr.y * rk * gk1), vq = gpack(vr.x, vr.y);
-        const float k0 = glo(kq), k1 = ghi(kq), v0 = glo(vq), v1 = ghi(vq);
-        if (j + 1 < n) {
-          const float s = warp_sum(q0 * k0 + q1 * k1) * C.scale_log2 - slope;
-          const float mo = st[kHeadDim], mn = fmaxf(mo, s), corr = exp2f(mo - mn), pj = exp2f(s - mn);
-          const float il = 1.0f / (st[kHeadDim + 1] * corr + pj);
-          const float2 oo = *reinterpret_cast<const float2*>(st + 2 * lane);
-          st_flag(c_at, gpack((oo.x * corr + pj * v0) * il, (oo.y * corr + pj * v1) * il), seq + 1u);
-        }
-        const size_t crow = (size_t)(J.t0 + j) * qrow + qcol + 2 * lane;
-        *reinterpret_cast<unsigned*>(kc + crow) = kq;
-        *reinterpret_cast<unsigned*>(vc + crow) = vq;
-        if (j + 2 >= n) continue;
-        __syncwarp();
-        if (j + 2 == w0 + kWin) open_window(j + 2, j + 1);
-        else {
-          *reinterpret_cast<float2*>(fin + 2 * lane) = make_float2(k0, k1);
-          *reinterpret_cast<float2*>(fin + kHeadDim + 2 * lane) = make_float2(v0, v1);
+        if (j < 0) {
+          if (qi == 0) leave_state();
           __syncwarp();
-          fold(fin, w0 + qi - j);
+          const float il = 1.f / st[kHeadDim + 1];
+          const float2 oo = *reinterpret_cast<const float2*>(st + 2 * lane);
+          st_flag(c_at, gpack(oo.x * il, oo.y * il), J.steps + 1u);
+          __syncwarp();
         }
         if (w0 + qi == j + 2) leave_state();
         __syncwarp();
@@ -380,8 +388,9 @@ __global__ void __launch_bounds__(kGThreads, 1) leaf_group_kernel(const __grid_c
   const bool pre = (C.norm_flags & RT_NORM_PRE) != 0, kv_norm = pre && !(C.norm_flags & RT_NORM_SKIP_Z);
   const float inv_d = 1.0f / (float)d;
   const bool has0 = g < B, has1 = MB == 2 && g + 8 < B;
-  const int nkp = d >> 5, per = (nkp + kGMma - 1) / kGMma, kp0 = warp * per;
-  const int n_kp = max(0, min(per, nkp - kp0));                // this warp's blocks of 32 k in a stretch of d
+  const int nkp = d >> 5, per = (nkp + kGMma - 1) / kGMma;
+  const int n_kp = max(0, min(per, nkp - warp * per));         // this warp's blocks of 32 k in a stretch of d
+  const int kp0 = n_kp > 0 ? warp * per : 0;                   // (a warp without any multiplies the first one by zeros)
   const __nv_bfloat16* x = reinterpret_cast<const __nv_bfloat16*>(J.x);
   __nv_bfloat16* z = reinterpret_cast<__nv_bfloat16*>(J.z);
   unsigned target = J.steps * (unsigned)G;
@@ -389,6 +398,7 @@ __global__ void __launch_bounds__(kGThreads, 1) leaf_group_kernel(const __grid_c
   uint32_t par = 0;
   const unsigned char* const ring = smem + L.off_ring + g * 64 + c * 16 + kp0 * 512;
 
+#pragma unroll 1
   for (int j = 0; j < n; ++j) {
     const unsigned seq = J.steps + (unsigned)j + 1u;
     const size_t t = (size_t)(J.t0 + j);
@@ -506,18 +516,17 @@ __global__ void __launch_bounds__(kGThreads, 1) leaf_group_kernel(const __grid_c
               for (int e = 0; e < 4; ++e) { acc[u][0][e] = 0.f; acc[u][1][e] = 0.f; }
           }
 #pragma unroll
-          for (int i = 0; i < kKP; ++i) {
-            if (i < n_kp) {
-              uint4 bw[kQuad];
+          for (int i = 0; i < kKP; ++i) {                      // (no branch around a product: blocks beyond the stretch multiply zeros)
+            const int at = i < n_kp ? i * 512 : 0;
+            uint4 bw[kQuad];
 #pragma unroll
-              for (int u = 0; u < kQuad; ++u) bw[u] = *reinterpret_cast<const uint4*>((u < kPieceTiles ? w0 : w1) + (size_t)(u & 1) * L.tile_bytes + i * 512);
+            for (int u = 0; u < kQuad; ++u) bw[u] = *reinterpret_cast<const uint4*>((u < kPieceTiles ? w0 : w1) + (size_t)(u & 1) * L.tile_bytes + at);
 #pragma unroll
-              for (int u = 0; u < kQuad; ++u)
-                gmma(acc[u][0], av[i][0].x, MB == 2 ? av[i][MB - 1].x : 0u, av[i][0].y, MB == 2 ? av[i][MB - 1].y : 0u, bw[u].x, bw[u].y);
+            for (int u = 0; u < kQuad; ++u)
+              gmma(acc[u][0], av[i][0].x, MB == 2 ? av[i][MB - 1].x : 0u, av[i][0].y, MB == 2 ? av[i][MB - 1].y : 0u, bw[u].x, bw[u].y);
 #pragma unroll
-              for (int u = 0; u < kQuad; ++u)
-                gmma(acc[u][1], av[i][0].z, MB == 2 ? av[i][MB - 1].z : 0u, av[i][0].w, MB == 2 ? av[i][MB - 1].w : 0u, bw[u].z, bw[u].w);
-            }
+            for (int u = 0; u < kQuad; ++u)
+              gmma(acc[u][1], av[i][0].z, MB == 2 ? av[i][MB - 1].z : 0u, av[i][0].w, MB == 2 ? av[i][MB - 1].w : 0u, bw[u].z, bw[u].w);
           }
           __syncwarp();
           if (lane == 0) { mbar_arrive(empty + 8 * slot); if (two) mbar_arrive(empty + 8 * slot2); }
