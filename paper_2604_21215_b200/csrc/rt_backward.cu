@@ -138,8 +138,7 @@ __global__ void norm_fwd_kernel(const TI* __restrict__ in, long long bs, long lo
 template <typename TU, typename TG>
 __global__ void norm_bwd_kernel(const float* dy, const TU* __restrict__ u, long long u_bs, long long u_ts, int B,
                                 const TG* __restrict__ g, const float* add, float* out, long long o_bs, long long o_ts,
-                                float* gprod, int gprod_acc, long long rows, int d, int G, float eps, int enable,
-                                __nv_bfloat16* out_bf = nullptr, float bf_scale = 1.f) {
+                                float* gprod, int gprod_acc, long long rows, int d, int G, float eps, int enable) {
   grid_dep_sync();
   const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31, groups = d / G;
@@ -168,7 +167,6 @@ __global__ void norm_bwd_kernel(const float* dy, const TU* __restrict__ u, long 
     }
     const float res = (add ? add[r * d + c0 + e] : 0.f) + du;
     if (out) out[row_at(r, B, o_bs, o_ts) + c0 + e] = res;
-    if (out_bf) out_bf[r * d + c0 + e] = __float2bfloat16_rn(res * bf_scale);   // operand copy for the next product
     if (gprod) gprod[r * d + c0 + e] = (gprod_acc ? gprod[r * d + c0 + e] : 0.f) + gp;
   }
 }
@@ -178,7 +176,7 @@ __global__ void norm_bwd_kernel(const float* dy, const TU* __restrict__ u, long 
 template <typename TU, typename TG>
 __global__ void __launch_bounds__(256) norm_bwd_row_kernel(const float* dy, const TU* __restrict__ u, long long u_bs, long long u_ts, int B,
                                                            const TG* __restrict__ g, const float* add, float* out, int d, float eps,
-                                                           int enable, __nv_bfloat16* out_bf, float bf_scale) {
+                                                           int enable) {
   grid_dep_sync();
   __shared__ float red[2][8];
   const long long r = blockIdx.x;
@@ -203,9 +201,7 @@ __global__ void __launch_bounds__(256) norm_bwd_row_kernel(const float* dy, cons
   for (int e = tid; e < d; e += 256) {
     float du = dyr[e];
     if (enable) du = inv * (dyr[e] * gain_at(g, e) - to_f(ur[e]) * inv * mean);
-    const float res = add[r * d + e] + du;
-    out[r * d + e] = res;
-    if (out_bf) out_bf[r * d + e] = __float2bfloat16_rn(res * bf_scale);
+    out[r * d + e] = add[r * d + e] + du;
   }
 }
 
@@ -243,17 +239,13 @@ __device__ __forceinline__ float gelu_grad_f(float a) {
   return 0.5f * (1.f + erff(a * 0.70710678118654752f)) + a * 0.3989422804014327f * __expf(-0.5f * a * a);
 }
 // four consecutive entries per thread (n a multiple of 4: d_ff is)
-__global__ void gelu_bwd_kernel(float* __restrict__ dg, const float* __restrict__ a, long long n, __nv_bfloat16* out_bf) {
+__global__ void gelu_bwd_kernel(float* __restrict__ dg, const float* __restrict__ a, long long n) {
   grid_dep_sync();
   const long long idx = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
   if (idx < n) {
     const float4 g = *reinterpret_cast<const float4*>(dg + idx), x = *reinterpret_cast<const float4*>(a + idx);
     const float4 v = make_float4(g.x * gelu_grad_f(x.x), g.y * gelu_grad_f(x.y), g.z * gelu_grad_f(x.z), g.w * gelu_grad_f(x.w));
     *reinterpret_cast<float4*>(dg + idx) = v;
-    if (out_bf) {
-      const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
-      *reinterpret_cast<uint2*>(out_bf + idx) = make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
-    }
   }
 }
 __global__ void gelu_kernel(const float* __restrict__ a, float* __restrict__ out, long long n) {
@@ -474,6 +466,162 @@ __global__ void attn_self_wide_kernel(AttnBufs a, int i, int k0) {
 #pragma unroll
       for (int e = 0; e < 8; ++e) { gk.v[e] = fmaf(ds, q.v[e], gk.v[e]); gv.v[e] = fmaf(p, dc.v[e], gv.v[e]); }
       st8(a.dK + rj, gk); st8(a.dV + rj, gv);
+    }
+  }
+  const F8 kt = ld8(a.kt + ri), vt = ld8(a.vt + ri);
+  const float p = exp2f(group_sum(dot8(q, kt)) * a.scale_log2 - lse);
+  const float ds = p * (group_sum(dot8(dc, vt)) - D) * a.scale;
+  if (g == 0) {
+    F8 o1, o2;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) { o1.v[e] = ds * q.v[e]; o2.v[e] = p * dc.v[e]; }
+    st8(a.dkt + ri, o1); st8(a.dvt + ri, o2);
+    if (t == 0) a.D[si] = D;
+  }
+}
+
+// ---- wide batches on the tensor cores: a position is seven launches ------------------------------------------------
+// (product, row kernel, product, product, row kernel, product, attention).  Every launch of the chain costs about 5 us whatever it
+// does at these sizes, so the sums of split products, the norm backwards and the operand copies live in the kernels that need them
+// anyway: 15 launches and 73 us per position at B = 96, d = 1024 before.
+
+// qkRMS backward of dk of one (position, sequence, head) and the bf16 operand row [dk_raw | dv] of the next product; a group of eight
+// lanes, eight entries each.
+__device__ __forceinline__ void pair_operand(const F8& dk, const F8& dv, const F8& u, const __nv_bfloat16* g_k, int h, int t, float eps, int qk, float* dkraw,
+                                             __nv_bfloat16* op_k, __nv_bfloat16* op_v) {
+  F8 r = dk;
+  if (qk) {
+    F8 ty;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) ty.v[e] = dk.v[e] * gain_at(g_k, h * kHeadDim + 8 * t + e);
+    const float ss = group_sum(dot8(u, u)), tu = group_sum(dot8(ty, u));
+    const float inv = rsqrtf(ss / kHeadDim + eps), mean = tu * inv / kHeadDim;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) r.v[e] = inv * (ty.v[e] - u.v[e] * inv * mean);
+  }
+  st8(dkraw, r);
+  unsigned a[4], b[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const __nv_bfloat162 x = __floats2bfloat162_rn(r.v[2 * e], r.v[2 * e + 1]), y = __floats2bfloat162_rn(dv.v[2 * e], dv.v[2 * e + 1]);
+    a[e] = *reinterpret_cast<const unsigned*>(&x); b[e] = *reinterpret_cast<const unsigned*>(&y);
+  }
+  *reinterpret_cast<uint4*>(op_k) = make_uint4(a[0], a[1], a[2], a[3]);
+  *reinterpret_cast<uint4*>(op_v) = make_uint4(b[0], b[1], b[2], b[3]);
+}
+struct WidePair { const float* kraw; float* dkraw; const __nv_bfloat16* g_k; __nv_bfloat16* op; float eps; int qk; };      // op [B][2 d]
+
+// The operand of position i when nothing of its leaf has to be added first (the last position of a leaf): one warp per four (sequence, head).
+__global__ void wide_pair_kernel(AttnBufs a, WidePair w, int i) {
+  grid_dep_sync();
+  const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+  const int t = threadIdx.x & 7;
+  const bool live = gid < (long long)a.B * a.H;
+  const long long u = live ? gid : 0;
+  const int h = (int)(u % a.H), b = (int)(u / a.H);
+  const long long at = ((long long)i * a.B + b) * a.d + (long long)h * kHeadDim + 8 * t;
+  const F8 dk = ld8(a.dK + at), dv = ld8(a.dV + at), kr = ld8(w.kraw + at);
+  __nv_bfloat16* op = w.op + (long long)b * 2 * a.d + h * kHeadDim + 8 * t;
+  if (live) pair_operand(dk, dv, kr, w.g_k, h, t, w.eps, w.qk, w.dkraw + at, op, op + a.d);
+}
+
+// out = add + RMS backward of the row sum of `splits` partial products through RMS(u); keeps the sum, leaves scale * out in bf16 as the
+// next operand.  One CTA per sequence, up to CH groups of four columns per thread (d <= 1024 CH, a multiple of 4).
+template <typename TU, int CH>
+__global__ void __launch_bounds__(256) wide_norm_bwd_kernel(const float* __restrict__ partial, int splits, const TU* __restrict__ u, long long u_bs, const __nv_bfloat16* __restrict__ g,
+                                                            const float* __restrict__ add, long long add_bs, float* __restrict__ sum, float* __restrict__ out, __nv_bfloat16* __restrict__ out_bf,
+                                                            float scale, int B, int d, float eps, int enable) {
+  grid_dep_sync();
+  __shared__ float red[2][8];
+  const int b = blockIdx.x, tid = threadIdx.x;
+  float dy[CH][4], uv[CH][4];
+  float ss = 0.f, tu = 0.f;
+#pragma unroll
+  for (int c = 0; c < CH; ++c) {
+    const int n = 4 * (tid + 256 * c);
+    if (n >= d) break;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int z = 0; z < splits; ++z) {
+      const float4 v = *reinterpret_cast<const float4*>(partial + ((size_t)z * B + b) * d + n);
+      acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+    }
+    *reinterpret_cast<float4*>(sum + (size_t)b * d + n) = acc;
+    dy[c][0] = acc.x; dy[c][1] = acc.y; dy[c][2] = acc.z; dy[c][3] = acc.w;
+    if (enable) {
+      reinterpret_cast<const Vec4<TU>*>(u + (size_t)b * u_bs + n)->to_float(uv[c]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        dy[c][e] *= gain_at(g, n + e);
+        ss = fmaf(uv[c][e], uv[c][e], ss);
+        tu = fmaf(dy[c][e], uv[c][e], tu);
+      }
+    }
+  }
+  if (enable) {
+    ss = warp_sum(ss); tu = warp_sum(tu);
+    if ((tid & 31) == 0) { red[0][tid >> 5] = ss; red[1][tid >> 5] = tu; }
+    __syncthreads();
+    ss = 0.f; tu = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) { ss += red[0][w]; tu += red[1][w]; }
+  }
+  const float inv = rsqrtf(ss / d + eps), mean = tu * inv / d;
+#pragma unroll
+  for (int c = 0; c < CH; ++c) {
+    const int n = 4 * (tid + 256 * c);
+    if (n >= d) break;
+    const float4 av = *reinterpret_cast<const float4*>(add + (size_t)b * add_bs + n);
+    float r[4] = {av.x, av.y, av.z, av.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) r[e] += enable ? inv * (dy[c][e] - uv[c][e] * inv * mean) : dy[c][e];
+    *reinterpret_cast<float4*>(out + (size_t)b * d + n) = make_float4(r[0], r[1], r[2], r[3]);
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(r[0] * scale, r[1] * scale), hi = __floats2bfloat162_rn(r[2] * scale, r[3] * scale);
+    *reinterpret_cast<uint2*>(out_bf + (size_t)b * d + n) = make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
+  }
+}
+
+// attn_self_wide_kernel on the partial sums of dc, and the operand of position i - 1, whose pair is complete then.
+__global__ void wide_attn_kernel(AttnBufs a, WidePair w, const float* __restrict__ partial, int splits, int i, int k0) {
+  grid_dep_sync();
+  const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31, g = lane >> 3, t = lane & 7;
+  if (wid >= (long long)a.B * a.H) return;
+  const int h = (int)(wid % a.H), b = (int)(wid / a.H);
+  const long long col = (long long)h * kHeadDim + 8 * t;
+  const long long rstride = (long long)a.B * a.d;
+  const long long ri = (long long)i * rstride + (long long)b * a.d + col;
+  const long long si = ((long long)i * a.B + b) * a.H + h;
+  const float slope = a.alibi ? a.alibi[h] * kLog2e : 0.f;
+  F8 dc = {};
+  for (int z = 0; z < splits; ++z) {
+    const F8 v = ld8(partial + ((size_t)z * a.B + b) * a.d + col);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) dc.v[e] += v.v[e];
+  }
+  if (g == 0) st8(const_cast<float*>(a.dc) + ri, dc);
+  const F8 q = ld8(a.q + ri), cc = ld8(a.c + ri);
+  const float D = group_sum(dot8(dc, cc)), lse = a.lse[si];
+  // the pairs k0 .. i - 2 by the four groups in turn, then pair i - 1 by all of them (the first one stores it)
+  for (int j0 = k0; j0 < i; j0 += 4) {
+    const bool last = j0 + 4 >= i;
+    for (int pass = 0; pass < (last ? 2 : 1); ++pass) {
+      const int j = pass ? i - 1 : j0 + g;
+      const bool valid = pass ? true : j < i - 1;
+      const long long rj = (long long)(valid ? j : k0) * rstride + (long long)b * a.d + col;
+      const F8 kk = ld8(a.k + rj), vv = ld8(a.v + rj);
+      F8 gk = ld8(a.dK + rj), gv = ld8(a.dV + rj);
+      const float sd = group_sum(dot8(q, kk)), dp = group_sum(dot8(dc, vv));
+      const float p = exp2f(sd * a.scale_log2 - slope * (float)(i - j) - lse);
+      const float ds = p * (dp - D) * a.scale;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) { gk.v[e] = fmaf(ds, q.v[e], gk.v[e]); gv.v[e] = fmaf(p, dc.v[e], gv.v[e]); }
+      if (pass ? g == 0 : valid) { st8(a.dK + rj, gk); st8(a.dV + rj, gv); }
+      if (pass) {
+        const F8 kr = ld8(w.kraw + rj);
+        __nv_bfloat16* op = w.op + (long long)b * 2 * a.d + col;
+        // (all groups hold the same values; each writes them)
+        pair_operand(gk, gv, kr, w.g_k, h, t, w.eps, w.qk, w.dkraw + rj, op, op + a.d);
+      }
     }
   }
   const F8 kt = ld8(a.kt + ri), vt = ld8(a.vt + ri);
@@ -1149,7 +1297,7 @@ constexpr int kWideLeaf = 16;
 constexpr int kWideBatchFrom = 32;      // above this many sequences a step of the reverse loop runs as dense products over the batch
 
 // Sequences per launch of the tensor-core leaf kernel of the reverse loop (rt_backward_loop.cu), 0: not taken.
-constexpr int kFastLoopMax = 48;
+constexpr int kFastLoopMax = 32;          // beyond, dense products over the batch win (slices of 8: 21 us per position each)
 int bwd_fast_slice(const rt_config* c, int B) {
   if (c->dtype != RT_BF16 || (c->flags & RT_FLAG_BACKWARD_STEP_LAUNCHES)) return 0;
   return bwd_leaf_slice(B, c->d_model, c->n_heads, c->d_ff, kFastLoopMax);
@@ -1173,13 +1321,16 @@ BwdLayout bwd_layout(const rt_config* c, int B, int N) {
   L.dkt = take(rows * d); L.dvt = take(rows * d); L.dn = take(rows * d); L.gprod = take(rows * d);
   L.part = take((size_t)kColParts * (d > f ? d : f));
   L.part2 = take((size_t)4 * B * d);
-  // wide batches: bf16 transposes of the five matrices of the reverse loop, dL/dz in position-major order
+  const bool tc = c->dtype == RT_BF16 && d % 128 == 0 && f % 128 == 0, wide = B > kWideBatchFrom && !bwd_fast_slice(c, B);
+  // wide batches: bf16 transposes of the five matrices of the reverse loop, dL/dz in position-major order (fp32 products)
   L.dvf = bwd_fast_slice(c, B) ? take(rows * d) : L.dV;        // final dv of every position (the exchange words of the leaf kernel)
   L.qkv16 = take(3 * rows * d / 2 + 64);                       // bf16 copies of q, k, v for the tile kernels
-  L.wt5 = take((3 * d * d + 2 * d * f) / 2 + 64); L.dzp = B > kWideBatchFrom && !bwd_fast_slice(c, B) ? take(rows * d) : o;
+  L.wt5 = take((3 * d * d + 2 * d * f) / 2 + 64); L.dzp = wide && !tc ? take(rows * d) : o;
   // bf16 operands of the tensor-core products (bf16 storage): two [rows, max(d, d_ff)] arrays and one [d, d]
   const size_t rows_k = align_up(rows, 64);
-  L.sa = take(rows_k * (d > f ? d : f) / 2 + 64); L.sb = take(rows_k * (d > f ? d : f) / 2 + 64); L.wt = take(d * d / 2 + 64);
+  size_t sb_elems = rows_k * (d > f ? d : f);
+  if (wide && sb_elems < (2 * d + f) * B + 64) sb_elems = (2 * d + f) * B + 64;     // the operands of one position side by side
+  L.sa = take(rows_k * (d > f ? d : f) / 2 + 64); L.sb = take(sb_elems / 2 + 64); L.wt = take(d * d / 2 + 64);
   L.total = o;
   return L;
 }
@@ -1225,12 +1376,12 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   __nv_bfloat16* SA = reinterpret_cast<__nv_bfloat16*>(ws + L.sa);
   __nv_bfloat16* SB = reinterpret_cast<__nv_bfloat16*>(ws + L.sb);
   __nv_bfloat16* WT = reinterpret_cast<__nv_bfloat16*>(ws + L.wt);
-  auto tc_product = [&](int M, int Nn, int K, const void* A, const void* W, float* out, float al, bool acc, bool chained = false) {
+  __nv_bfloat16* SC = SB + align_up((size_t)2 * B * d, 64);      // wide batches: operand rows of one position beside SB's [B, 2 d]
+  auto tc_product = [&](int M, int Nn, int K, const void* A, const void* W, float* out, float al, bool acc) {
     DenseParams dp;
     memset(&dp, 0, sizeof(dp));
     dp.M = M; dp.N = Nn; dp.K = K; dp.B = 1; dp.A = A; dp.W = W; dp.epi = DENSE_F32; dp.alpha = al; dp.accumulate = acc ? 1 : 0;
-    dp.h = out; dp.chained = chained ? 1 : 0;
-    if (chained) { dp.partial = F(L.gprod); dp.partial_bytes = (size_t)rows * d * sizeof(float); }   // few rows: split contraction
+    dp.h = out;
     return dense_launch(RT_BF16, dp, sync, s);
   };
   auto to_bf16 = [&](const float* in, __nv_bfloat16* out, long long n) {
@@ -1383,21 +1534,23 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   lp.resident = resident ? 1 : 0; lp.stage_bytes = (unsigned)smem_max;
   lp.sync = reinterpret_cast<SyncArea*>(ws + L.sync);
   unsigned bar_base = 0;
-  // leaf of the reverse schedule; wide batches take short leaves (the in-leaf step re-reads and rewrites the fp32
-  // pairs of its leaf at every position, the tiles do not)
-  const int Lf = B > kWideBatchFrom && !(kBf16 && bwd_fast_slice(c, B)) ? kWideLeaf : 64;
   // Wide batches (the paper's own regime, Sec. 6): a step of the reverse loop is a dense product over the B rows of the
   // position -- tensor cores for bf16 storage -- between small row-wise kernels, instead of tasks of four sequences.
   const int fast = kBf16 ? bwd_fast_slice(c, B) : 0;             // sequences per launch of the tensor-core leaf kernel
   const bool wide = B > kWideBatchFrom && !fast;
+  // leaf of the reverse schedule; wide batches take short leaves (the in-leaf step re-reads and rewrites the fp32
+  // pairs of its leaf at every position, the tiles do not)
+  const int Lf = wide ? kWideLeaf : 64;
   const size_t pos_d = (size_t)B * d, pos_f = (size_t)B * f;
   __nv_bfloat16* WkT = reinterpret_cast<__nv_bfloat16*>(ws + L.wt5);
   __nv_bfloat16 *WvT = WkT + (size_t)d * d, *WoT = WvT + (size_t)d * d, *WdnT = WoT + (size_t)d * d, *WupT = WdnT + (size_t)d * f;
   if (fast || (wide && tc)) {
-    auto tr = [&](const T* W, int n_out, int n_in, __nv_bfloat16* out) {
-      transpose_bf16_kernel<T><<<dim3(ceil_div(n_in, 32), ceil_div(n_out, 32)), dim3(32, 8), 0, s>>>(W, n_out, n_in, out, n_out);
+    auto tr = [&](const T* W, int n_out, int n_in, __nv_bfloat16* out, int ld = 0) {
+      transpose_bf16_kernel<T><<<dim3(ceil_div(n_in, 32), ceil_div(n_out, 32)), dim3(32, 8), 0, s>>>(W, n_out, n_in, out, ld ? ld : n_out);
     };
-    tr(Wk, d, d, WkT); tr(Wv, d, d, WvT); tr(Wo, d, d, WoT); tr(Wdn, d, f, WdnT); tr(Wup, f, d, WupT);
+    if (fast) { tr(Wk, d, d, WkT); tr(Wv, d, d, WvT); }
+    else { tr(Wk, d, d, WkT, 2 * d); tr(Wv, d, d, WkT + d, 2 * d); }       // wide: rows [W_k^T | W_v^T], one product for dk_raw and dv
+    tr(Wo, d, d, WoT); tr(Wdn, d, f, WdnT); tr(Wup, f, d, WupT);
     RT_TRY(cudaGetLastError());
   }
   BwdLeafParams bl;
@@ -1416,44 +1569,74 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
     bl.du = F(L.du); bl.dh = F(L.dh); bl.dc = F(L.dc); bl.dkt = F(L.dkt); bl.dvt = F(L.dvt); bl.D = F(L.D);
     bl.sync = reinterpret_cast<SyncArea*>(ws + L.sync);
   }
-  if (wide) {
+  if (wide && !tc) {
     norm_fwd_kernel<float, T><<<warps_grid(rows), tpb, 0, s>>>(dz, xbs, xts, B, (const T*)nullptr, F(L.dzp), rows, d, d, eps, 0);
     RT_TRY(cudaGetLastError());
   }
-  // out[B, n_in] (+)= al * dY[B, n_out] W[n_out, n_in] for the rows of one position; A_bf = bf16 copy of dY (scale folded in)
-  auto step_product = [&](const float* dY, const __nv_bfloat16* A_bf, int n_out, const T* W, const __nv_bfloat16* Wt, int n_in, float* out,
-                          float al, bool acc) -> cudaError_t {
-    if (!tc) return gemm<float, T>(B, n_in, n_out, dY, n_out, 1, W, n_in, 1, out, n_in, al, acc, s);
-    return tc_product(B, n_in, n_out, A_bf, Wt, out, 1.f, acc, true);
+  // out[B, n_in] (+)= al * dY[B, n_out] W[n_out, n_in] for the rows of one position, fp32
+  auto step_product = [&](const float* dY, int n_out, const T* W, int n_in, float* out, float al, bool acc) -> cudaError_t {
+    return gemm<float, T>(B, n_in, n_out, dY, n_out, 1, W, n_in, 1, out, n_in, al, acc, s);
   };
-  // The launches of a position are chained (programmatic dependent launches); each producer also leaves the bf16 operand
-  // of the product that follows (SA, SB), so a position is eleven launches.
+  // fp32 storage, or widths off the tensor-core products
   auto wide_position = [&](int i, int s0) -> rt_status {
     const size_t od = (size_t)i * pos_d, of = (size_t)i * pos_f;
-    sa_holds = nullptr;
     const dim3 blk(tpb);
     // dk_raw = qkRMS backward of dk_i;  dr = dk_raw W_k + dv_i W_v
     RT_TRY(launch_chained(norm_bwd_kernel<float, T>, dim3(warps_grid((long long)B * H)), blk, 0, s, true, (const float*)(F(L.dK) + od),
                           (const float*)(F(L.kraw) + od), pbs, pts, B, g_k, (const float*)nullptr, F(L.dkraw) + od, pbs, pts, (float*)nullptr, 0,
-                          (long long)B, d, (int)kHeadDim, eps, qk ? 1 : 0, tc ? SA : (__nv_bfloat16*)nullptr, 1.f));
-    if (tc) RT_TRY(launch_chained(to_bf16_kernel, dim3(elems_grid((long long)(pos_d + 3) / 4)), blk, 0, s, true, (const float*)(F(L.dV) + od), SB,
-                                  (long long)pos_d));
-    RT_TRY(step_product(F(L.dkraw) + od, SA, d, Wk, WkT, d, F(L.dr) + od, 1.f, false));
-    RT_TRY(step_product(F(L.dV) + od, SB, d, Wv, WvT, d, F(L.dr) + od, 1.f, true));
+                          (long long)B, d, (int)kHeadDim, eps, qk ? 1 : 0));
+    RT_TRY(step_product(F(L.dkraw) + od, d, Wk, d, F(L.dr) + od, 1.f, false));
+    RT_TRY(step_product(F(L.dV) + od, d, Wv, d, F(L.dr) + od, 1.f, true));
     // Gz = dz_i + RMS backward of dr;  dpre = (alpha Gz W_down) * GELU'
     RT_TRY(launch_chained(norm_bwd_row_kernel<T, T>, dim3(B), dim3(256), 0, s, true, (const float*)(F(L.dr) + od), z + (size_t)i * xts, xbs, xts, B,
-                          g_kv, (const float*)(F(L.dzp) + od), F(L.Gz) + od, d, eps, z_norm ? 1 : 0, tc ? SA : (__nv_bfloat16*)nullptr, alpha));
-    RT_TRY(step_product(F(L.Gz) + od, SA, d, Wdn, WdnT, f, F(L.dpre) + of, alpha, false));
+                          g_kv, (const float*)(F(L.dzp) + od), F(L.Gz) + od, d, eps, z_norm ? 1 : 0));
+    RT_TRY(step_product(F(L.Gz) + od, d, Wdn, f, F(L.dpre) + of, alpha, false));
     RT_TRY(launch_chained(gelu_bwd_kernel, dim3(elems_grid(((long long)pos_f + 3) / 4)), blk, 0, s, true, F(L.dpre) + of, (const float*)(F(L.act) + of),
-                          (long long)pos_f, tc ? SA : (__nv_bfloat16*)nullptr));
+                          (long long)pos_f));
     // du = dpre W_up;  dh = Gz + RMS backward of du;  dc = alpha dh W_o
-    RT_TRY(step_product(F(L.dpre) + of, SA, f, Wup, WupT, d, F(L.du) + od, 1.f, false));
+    RT_TRY(step_product(F(L.dpre) + of, f, Wup, d, F(L.du) + od, 1.f, false));
     RT_TRY(launch_chained(norm_bwd_row_kernel<float, T>, dim3(B), dim3(256), 0, s, true, (const float*)(F(L.du) + od), (const float*)(F(L.h) + od),
-                          pbs, pts, B, g_mlp, (const float*)(F(L.Gz) + od), F(L.dh) + od, d, eps, pre ? 1 : 0,
-                          tc ? SA : (__nv_bfloat16*)nullptr, alpha));
-    RT_TRY(step_product(F(L.dh) + od, SA, d, Wo, WoT, d, F(L.dc) + od, alpha, false));
+                          pbs, pts, B, g_mlp, (const float*)(F(L.Gz) + od), F(L.dh) + od, d, eps, pre ? 1 : 0));
+    RT_TRY(step_product(F(L.dh) + od, d, Wo, d, F(L.dc) + od, alpha, false));
     // the query's share of the pairs of its own leaf, its temporary pair and D_i
     RT_TRY(launch_chained(attn_self_wide_kernel, dim3(warps_grid((long long)B * H)), blk, 0, s, true, ab, i, s0));
+    return RT_OK;
+  };
+  const bool wide_tc = wide && tc;
+  WidePair wp;
+  memset(&wp, 0, sizeof(wp));
+  wp.kraw = F(L.kraw); wp.dkraw = F(L.dkraw); wp.g_k = reinterpret_cast<const __nv_bfloat16*>(g_k); wp.op = SB; wp.eps = eps; wp.qk = qk ? 1 : 0;
+  // partial sums of out[B, n_out] = A[B, k] W[n_out, k]^T; *splits of them
+  auto wide_partial = [&](const __nv_bfloat16* A, const __nv_bfloat16* W, int n_out, int k, int* splits) -> cudaError_t {
+    DenseParams dp;
+    memset(&dp, 0, sizeof(dp));
+    dp.M = B; dp.N = n_out; dp.K = k; dp.B = 1; dp.A = A; dp.W = W; dp.epi = DENSE_F32; dp.alpha = 1.f; dp.h = F(L.gprod); dp.chained = 1;
+    dp.partial = F(L.gprod); dp.partial_bytes = (size_t)rows * d * sizeof(float); dp.keep_partial = 1;
+    return dense_launch(RT_BF16, dp, sync, s, nullptr, splits);
+  };
+  auto wide_position_tc = [&](int i, int s0, bool first) -> rt_status {
+    const size_t od = (size_t)i * pos_d, of = (size_t)i * pos_f;
+    const float* part = F(L.gprod);
+    const __nv_bfloat16 *gkv = reinterpret_cast<const __nv_bfloat16*>(g_kv), *gmlp = reinterpret_cast<const __nv_bfloat16*>(g_mlp);
+    int sp = 1;
+    sa_holds = nullptr;
+    if (first) RT_TRY(launch_chained(wide_pair_kernel, dim3((unsigned)(((long long)B * H * 8 + tpb - 1) / tpb)), dim3(tpb), 0, s, true, ab, wp, i));
+    // dr = dk_raw W_k + dv W_v;  Gz = dz_i + RMS backward of dr
+    RT_TRY(wide_partial(SB, WkT, d, 2 * d, &sp));
+    RT_TRY(launch_chained(d <= 4096 ? wide_norm_bwd_kernel<T, 4> : wide_norm_bwd_kernel<T, 16>, dim3(B), dim3(256), 0, s, true, part, sp, z + (size_t)i * xts, xbs, gkv, dz + (size_t)i * xts, xbs,
+                          F(L.dr) + od, F(L.Gz) + od, SA, alpha, B, d, eps, z_norm ? 1 : 0));
+    // dpre = (alpha Gz W_down) * GELU'
+    DenseParams dp;
+    memset(&dp, 0, sizeof(dp));
+    dp.M = B; dp.N = f; dp.K = d; dp.B = 1; dp.A = SA; dp.W = WdnT; dp.epi = DENSE_GELU_BWD; dp.alpha = 1.f; dp.x = F(L.act) + of; dp.h = F(L.dpre) + of; dp.out = SC; dp.chained = 1;
+    RT_TRY(dense_launch(RT_BF16, dp, sync, s));
+    // du = dpre W_up;  dh = Gz + RMS backward of du;  dc = alpha dh W_o
+    RT_TRY(wide_partial(SC, WupT, d, f, &sp));
+    RT_TRY(launch_chained(d <= 4096 ? wide_norm_bwd_kernel<float, 4> : wide_norm_bwd_kernel<float, 16>, dim3(B), dim3(256), 0, s, true, part, sp, (const float*)(F(L.h) + od), pbs, gmlp, (const float*)(F(L.Gz) + od), pbs,
+                          F(L.du) + od, F(L.dh) + od, SA, alpha, B, d, eps, pre ? 1 : 0));
+    RT_TRY(wide_partial(SA, WoT, d, d, &sp));
+    // the query's share of the pairs of its own leaf, its temporary pair and D_i; the operand of position i - 1
+    RT_TRY(launch_chained(wide_attn_kernel, dim3(warps_grid((long long)B * H)), dim3(tpb), 0, s, true, ab, wp, part, sp, i, s0));
     return RT_OK;
   };
   RT_TRY(cudaFuncSetAttribute(attn_bwd_kv_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairBlockSmem));
@@ -1481,7 +1664,9 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
     }
     if (wide) {
       for (int i = e0 - 1; i >= s0; --i) {
-        const rt_status st = wide_position(i, s0);
+        rt_status st = RT_OK;
+        if constexpr (kBf16) { if (wide_tc) st = wide_position_tc(i, s0, i == e0 - 1); }
+        if (!wide_tc) st = wide_position(i, s0);
         if (st != RT_OK) return st;
       }
       continue;

@@ -199,13 +199,14 @@ cudaError_t head_launch(int dtype, const void* emb, const void* g_final, const v
                         int B, int d, int vocab, int norm_flags, float eps, float* logits, cudaStream_t s);
 
 // Position-wise part of the parallel sweep (Sec. 6, activation checkpointing): dense products over all rows.
-enum { DENSE_RES_X = 0, DENSE_GELU = 1, DENSE_RES_H = 2, DENSE_F32 = 3 };
+enum { DENSE_RES_X = 0, DENSE_GELU = 1, DENSE_RES_H = 2, DENSE_F32 = 3, DENSE_GELU_BWD = 4 };
 struct DenseParams {
   int M, N, K, B;                                // C[M,N] = A[M,K] W[N,K]^T; rows m = position * B + sequence
   const void *A, *W;                             // storage type, K contiguous
   int epi;                                       // DENSE_RES_X: h = x + alpha C (fp32);  DENSE_GELU: out = GELU(C);
                                                  // DENSE_RES_H: out = h + alpha C (storage type, caller's strides)
                                                  // DENSE_F32: h = alpha C, or h += alpha C with `accumulate` (fp32 [M, N])
+                                                 // DENSE_GELU_BWD: h = C GELU'(x) (x, h fp32 [M, N]), out = h in the storage type (tensor cores, not split)
   float alpha;
   int accumulate;                                // DENSE_F32 only
   const void* x; long long x_bs, x_ts;           // x[b, r, :] (DENSE_RES_X)
@@ -213,6 +214,8 @@ struct DenseParams {
   void* out; long long o_bs, o_ts;               // DENSE_GELU: [M, N];  DENSE_RES_H: out[b, r, :]
   float* partial; size_t partial_bytes;          // optional scratch for a split contraction (few rows): [splits, M, N] fp32
   int splits;                                    // set by the launcher
+  int keep_partial;                              // 1: leave the partial sums in `partial` ([splits, M, N], one split included) and reduce nothing;
+                                                 // the number of splits comes back through dense_launch's last argument
   int chained;                                   // 1: launch the product (and its reduction) as programmatic dependent launches
   // optional: also write RMS_g(row) of the epilogue's result (h or z) for the next product.  Only a split
   // contraction does this (its reduction kernel owns whole rows); `normed` tells the caller whether it happened.
@@ -229,7 +232,7 @@ constexpr int DENSE_QKV = 100;
 // wave of tiles); false when the shape does not qualify (the caller then takes qkv_gemm_tc_launch's own kernel).
 bool dense_qkv_pair_supported(int M, int d);
 cudaError_t dense_qkv_pair_launch(const DenseParams& p, SyncArea* sync, cudaStream_t s);
-cudaError_t dense_launch(int dtype, const DenseParams& p, SyncArea* sync, cudaStream_t s, bool* normed = nullptr);
+cudaError_t dense_launch(int dtype, const DenseParams& p, SyncArea* sync, cudaStream_t s, bool* normed = nullptr, int* splits = nullptr);
 cudaError_t attn_value_launch(int dtype, const float* st_o, const float* st_l, void* c, long long rows, int d, int H, cudaStream_t s,
                               bool chained = false);
 cudaError_t rms_rows_f32_launch(int dtype, const float* h, const void* g, void* u, int rows, int d, float eps, int pre, cudaStream_t s,

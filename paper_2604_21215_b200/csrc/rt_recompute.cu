@@ -17,6 +17,10 @@
 namespace rt {
 
 __device__ __forceinline__ float gelu_exact(float v) { return 0.5f * v * (1.0f + erff(v * 0.70710678118654752f)); }
+// d/da [a Phi(a)] = Phi(a) + a phi(a)
+__device__ __forceinline__ float gelu_grad_exact(float a) {
+  return 0.5f * (1.f + erff(a * 0.70710678118654752f)) + a * 0.3989422804014327f * __expf(-0.5f * a * a);
+}
 
 // ---- c = o / l ------------------------------------------------------------------------------
 template <typename T>
@@ -160,6 +164,21 @@ __device__ __forceinline__ void dense_epilogue_row(const DenseParams& p, uint32_
                                p.alpha * __uint_as_float(v[4 * q + 2]), p.alpha * __uint_as_float(v[4 * q + 3]));
         if (p.accumulate) { const float4 old = dst[q]; o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w; }
         dst[q] = o;
+      }
+      continue;
+    }
+    if (p.epi == DENSE_GELU_BWD) {
+      const float4* xs = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p.x) + (size_t)m * p.N + n);
+      float4* dst = reinterpret_cast<float4*>(p.h + (size_t)m * p.N + n);
+      uint2* ob = reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + (size_t)m * p.N + n);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float4 a = xs[q];
+        const float4 o = make_float4(__uint_as_float(v[4 * q]) * gelu_grad_exact(a.x), __uint_as_float(v[4 * q + 1]) * gelu_grad_exact(a.y),
+                                     __uint_as_float(v[4 * q + 2]) * gelu_grad_exact(a.z), __uint_as_float(v[4 * q + 3]) * gelu_grad_exact(a.w));
+        dst[q] = o;
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(o.x, o.y), hi = __floats2bfloat162_rn(o.z, o.w);
+        ob[q] = make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
       }
       continue;
     }
@@ -738,10 +757,10 @@ __global__ void __launch_bounds__(256) dense_reduce_kernel(const DenseParams p) 
 
 static_assert(kTBK == 64, "tensor_map_rows_bf16 encodes 64-column boxes");
 
-cudaError_t dense_launch(int dtype, const DenseParams& p, SyncArea* sync, cudaStream_t s, bool* normed) {
+cudaError_t dense_launch(int dtype, const DenseParams& p, SyncArea* sync, cudaStream_t s, bool* normed, int* splits) {
   if (normed) *normed = false;
   if (p.M <= 0) return cudaSuccess;
-  const bool strides_ok = p.epi == DENSE_GELU || p.epi == DENSE_F32 || (((p.epi == DENSE_RES_X ? p.x_bs : p.o_bs) % 8 == 0) &&
+  const bool strides_ok = p.epi == DENSE_GELU || p.epi == DENSE_F32 || p.epi == DENSE_GELU_BWD || (((p.epi == DENSE_RES_X ? p.x_bs : p.o_bs) % 8 == 0) &&
                                                   ((p.epi == DENSE_RES_X ? p.x_ts : p.o_ts) % 8 == 0));
   if (dtype == RT_BF16 && p.N % 128 == 0 && p.K % kTBK == 0 && strides_ok) {
     // Few rows (the wide-batch token step: M = B): narrow tiles and a split contraction so that the launch still
@@ -753,11 +772,15 @@ cudaError_t dense_launch(int dtype, const DenseParams& p, SyncArea* sync, cudaSt
     DenseParams q = p;
     q.splits = 1;
     const int ctas = m_tiles * (p.N / bn), kb_all = p.K / kTBK;
-    if (p.partial && ctas < sms / 2 && kb_all >= 8) {
+    if (p.partial && p.epi != DENSE_GELU_BWD && ctas < sms / 2 && kb_all >= 8) {
       int want = (sms + ctas - 1) / ctas;                         // about one wave
       if (want > 8) want = 8;
       while (want > 1 && kb_all / want < 4) --want;               // at least 4 k blocks per split
       if ((size_t)want * p.M * p.N * sizeof(float) <= p.partial_bytes) q.splits = want;
+    }
+    if (p.keep_partial) {
+      if (q.splits == 1) { q.epi = DENSE_F32; q.h = q.partial; q.accumulate = 0; q.alpha = 1.f; }
+      if (splits) *splits = q.splits;
     }
     // CTA pairs on 256-row tiles (each CTA fetches half of the weight tile) for products of at least a wave of CTAs:
     // c3's chain products 0.892 -> 0.850 ms; the few-row products of a wide-batch token step are 3 % slower as pairs
@@ -784,7 +807,7 @@ cudaError_t dense_launch(int dtype, const DenseParams& p, SyncArea* sync, cudaSt
     } else if (pair) e = bn == 256 ? run(dense_pair_kernel<256>, PairSmem<256>::total + 1024) : run(dense_pair_kernel<128>, PairSmem<128>::total + 1024);
     else e = bn == 256 ? run(dense_tc_kernel<256>, DenseSmem<256>::total + 1024) : run(dense_tc_kernel<128>, DenseSmem<128>::total + 1024);
     if (e != cudaSuccess) return e;
-    if (q.splits > 1) {
+    if (q.splits > 1 && !p.keep_partial) {
       cudaError_t er = launch_chained(dense_reduce_kernel<__nv_bfloat16>, dim3(p.M), dim3(256), 0, s, p.chained != 0, q);
       if (er != cudaSuccess) return er;
       if (normed && p.norm_out) *normed = true;
