@@ -380,9 +380,29 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
     // in-leaf attention re-reads the leaf's pairs for every position (leaf^2 * B * d bytes per leaf), so wide
     // batches default to a shorter leaf
     const int Lf = plan.leaf, N = n_rows;
+    // one launch per leaf where the shape allows (rt_wide_loop.cu), else the launches of every position
+    const bool loop = c->dtype == RT_BF16 && wide_loop_groups(B, c->d_model, c->d_ff) > 0 && x_bs % 8 == 0 && x_ts % 8 == 0 && z_bs % 8 == 0 && z_ts % 8 == 0;
+    WideFwdParams wf;
+    memset(&wf, 0, sizeof(wf));
+    if (loop) {
+      // counters and the bf16 operand rows live in the unused halves of the exchange buffers
+      wf.B = B; wf.d = (int)d; wf.H = c->n_heads; wf.dff = (int)f; wf.norm_flags = c->norm_flags; wf.eps = c->rms_eps; wf.scale_log2 = scale_log2; wf.alpha = c->residual_scale;
+      wf.w_o = w->w_o; wf.w_up = w->w_up; wf.w_down = w->w_down; wf.w_k = w->w_k; wf.w_v = w->w_v;
+      wf.g_mlp = w->g_mlp; wf.g_kv = w->g_kv ? w->g_kv : w->g_attn; wf.g_k = w->g_k; wf.alibi = w->alibi_slopes;
+      wf.x = x; wf.x_bs = x_bs; wf.x_ts = x_ts; wf.z = z; wf.z_bs = z_bs; wf.z_ts = z_ts;
+      wf.q = ws + L.q; wf.st_o = pp.st_o; wf.st_m = pp.st_m; wf.st_l = pp.st_l; wf.k_cache = k_cache; wf.v_cache = v_cache;
+      wf.h = hbuf; wf.partial = dp.partial; wf.c16 = cbuf; wf.u16 = ubuf; wf.g16 = gbuf; wf.r16 = ws + L.ex_z + (size_t)B * d * 2;
+      wf.ssq_h = (float*)(ws + L.ex_k + (size_t)B * d * 2);
+      wf.counters = (unsigned*)(ws + L.ex_g + align_up((size_t)B * f * 2, 256)); wf.sync = sync;
+      if (cudaMemsetAsync(wf.counters, 0, wide_counter_bytes(B), s) != cudaSuccess) return RT_ERR_CUDA;
+    }
     for (int s0 = 0; s0 < N; s0 += Lf) {
       const int e0 = s0 + Lf < N ? s0 + Lf : N;
-      {
+      if (loop) {
+        ProfScope ps(s, kProfLeaf);
+        wf.t0 = s0; wf.t1 = e0; wf.steps = (unsigned)s0;
+        if (wide_forward_launch(wf, s) != cudaSuccess) return RT_ERR_CUDA;
+      } else {
         ProfScope ps(s, kProfLeaf);
         for (int t = s0; t < e0; ++t) {
           // pairs of this leaf revealed so far (none for its first position), then c = o / l of the finished row

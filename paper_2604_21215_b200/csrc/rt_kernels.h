@@ -198,6 +198,33 @@ cudaError_t embed_launch(int dtype, const void* emb, const int32_t* ids, int B, 
 cudaError_t head_launch(int dtype, const void* emb, const void* g_final, const void* hidden, long long h_bs,
                         int B, int d, int vocab, int norm_flags, float eps, float* logits, cudaStream_t s);
 
+// Token loop of wide batches in one cooperative launch per leaf (bf16; rt_wide_loop.cu).
+constexpr int kWideGroupsMax = 8;                // groups of at most 128 sequences
+struct WideStage { int pairs, bn, tiles, splits, slots; };     // pairs of 64-wide blocks of the contraction, tile width, tiles, parts of the contraction, ring slots
+struct WideFwdParams {
+  int B, d, H, dff, norm_flags;
+  float eps, scale_log2, alpha;
+  const void *w_o, *w_up, *w_down, *w_k, *w_v, *g_mlp, *g_kv, *g_k;
+  const float* alibi;
+  const void* x; long long x_bs, x_ts;
+  void* z; long long z_bs, z_ts;
+  const void* q;                                 // [N, B, d]
+  const float *st_o, *st_m, *st_l;               // state of every row before its leaf
+  void *k_cache, *v_cache;                       // [N_max, B, d]
+  int t0, t1;                                    // positions of the leaf
+  unsigned steps;                                // positions since the counters were zeroed
+  unsigned* counters;                            // wide_counter_bytes(B)
+  float *h, *partial, *ssq_h, *ssq_z;            // [B, d], [8, B, d], [wide_ssq_floats, B] (ssq_z is set by the launcher)
+  void *c16, *u16, *g16, *r16;                   // bf16 operand rows [B, d], [B, d_ff] (g16)
+  SyncArea* sync;
+  int R, G, a_bytes;                             // set by the launcher: sequences and SMs per group, bytes of an operand block
+  WideStage st_out, st_up, st_dn, st_kv;
+};
+int wide_loop_groups(int B, int d, int dff);     // 0: not taken
+size_t wide_counter_bytes(int B);
+int wide_ssq_floats(int d);
+cudaError_t wide_forward_launch(WideFwdParams p, cudaStream_t s);
+
 // Position-wise part of the parallel sweep (Sec. 6, activation checkpointing): dense products over all rows.
 enum { DENSE_RES_X = 0, DENSE_GELU = 1, DENSE_RES_H = 2, DENSE_F32 = 3, DENSE_GELU_BWD = 4 };
 struct DenseParams {

@@ -1,0 +1,743 @@
+// Token loop of wide batches (up to 128 sequences per group of SMs), one cooperative launch per leaf, bf16.
+//
+// A token step of B sequences is a chain of dense products over B rows.  As separate launches (rt_recompute.cu, rt_prepass_tc.cu,
+// rt_tile.cu) a position of a layer of width 1024 is seven or eight launches of 5 to 8 us each, of which two thirds are launch, fill and
+// drain: every launch begins with an empty pipeline and fetches its weights only then.  Here the chain runs inside one kernel:
+//   - the batch is cut into groups of at most 128 sequences (one row tile of the tensor cores); a group of 148 / groups SMs runs its
+//     positions on its own (sequences are independent), so steps meet at a barrier of that group only;
+//   - one CTA per SM, three roles: warp 0 fetches operands by TMA, warp 1 issues tcgen05.mma, eight warps read the accumulators and do the
+//     row-wise work (attention, sums of split products);
+//   - the weights of the next product do not depend on the step before it: warp 0 fetches them while it waits, and only the operand rows
+//     (at most 128 KB to 256 KB per CTA, at 145 GB/s per SM) and the barrier stay on the chain.
+// RMS norms need whole rows, which no CTA owns: the product's epilogue leaves h * gain in bf16 and the sums of squares of its columns, and
+// the next product scales its accumulator rows by 1 / rms.  The down projection contracts over d_ff: it runs in up to eight parts whose sums
+// meet in a row step.
+//
+// Exchange: data through global memory (L2), a counter per step and group; a CTA's writes are fenced for the async proxy before it counts
+// itself in, the waiting CTA fences after it saw the count.  Every wait is bounded (2 s).
+#include <type_traits>
+
+#include "rt_kernels.h"
+#include "rt_tc.cuh"
+
+namespace rt {
+
+namespace {
+constexpr int kWThreads = 320, kWEpi = 256;
+constexpr uint32_t kWRing = 192512;                        // operand ring: a slot holds two 64-wide blocks of A and of W
+constexpr int kWSlotsMax = 11;
+constexpr int kWStagePitch = 36;                           // floats per row of a warp's 32 x 32 staging area
+constexpr uint32_t kWStage = kWRing, kWStageWarp = 32 * kWStagePitch * 4;
+constexpr uint32_t kWBars = kWStage + 8 * kWStageWarp, kWTmem = kWBars + 256, kWAbort = kWTmem + 8, kWTotal = kWAbort + 8;
+constexpr int kWBuf = 128;                                 // TMEM columns per accumulator, two of them
+constexpr int kWCounterStride = 32;                        // unsigned words between counters
+constexpr int kWMaxSteps = 8;
+
+__device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async;" ::: "memory"); }
+__device__ __forceinline__ bool epi_all(bool ok) {         // barrier of the eight row warps; true when all of them are fine
+  int r;
+  asm volatile("{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n barrier.cta.red.and.pred q, 1, 256, p;\n selp.b32 %0, 1, 0, q;\n}" : "=r"(r) : "r"((int)ok) : "memory");
+  return r != 0;
+}
+// 16 consecutive columns of this thread's TMEM lane
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                 "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+               : "r"(taddr) : "memory");
+  tc_wait_ld();
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void unpack8(const uint4& w, float (&f)[8]) {
+  const unsigned a[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { f[2 * i] = __uint_as_float(a[i] << 16); f[2 * i + 1] = __uint_as_float(a[i] & 0xffff0000u); }
+}
+__device__ __forceinline__ unsigned pack2(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const unsigned*>(&v);
+}
+__device__ __forceinline__ uint4 ldcg16(const __nv_bfloat16* p) { return __ldcg(reinterpret_cast<const uint4*>(p)); }
+__device__ __forceinline__ float sum8(float v) {           // over the eight lanes of a (sequence, head)
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  v += __shfl_xor_sync(0xffffffffu, v, 4);
+  return v;
+}
+__device__ __forceinline__ float gelu_wide(float v) { return 0.5f * v * (1.0f + erff(v * 0.70710678118654752f)); }
+
+// Where a CTA stands and how its group meets.
+struct WideCta {
+  unsigned char* smem;
+  uint32_t sbase;
+  volatile int* s_abort;
+  SyncArea* sync;
+  unsigned* counters;                                      // of this group
+  int rank, G, arank;                                      // arank: rank in the attention step, which begins with the CTAs that have no tile of the step before
+  __device__ uint32_t full(int s) const { return sbase + kWBars + 8u * (uint32_t)s; }
+  __device__ uint32_t empty(int s) const { return sbase + kWBars + 8u * (uint32_t)(kWSlotsMax + s); }
+  __device__ uint32_t tfull(int b) const { return sbase + kWBars + 8u * (uint32_t)(2 * kWSlotsMax + b); }
+  __device__ uint32_t tempty(int b) const { return sbase + kWBars + 8u * (uint32_t)(2 * kWSlotsMax + 2 + b); }
+  __device__ uint32_t flag() const { return sbase + kWBars + 8u * (uint32_t)(2 * kWSlotsMax + 4); }
+  // warp 0: until `target` CTAs have counted themselves in at a step
+  __device__ bool poll(int step, unsigned target) const {
+    const unsigned* c = counters + step * kWCounterStride;
+    unsigned spins = 0;
+    unsigned long long t_start = 0;
+    bool ok = true;
+    while (ld_acquire_u32(c) < target) {
+      if ((++spins & 1023u) == 0u) {
+        if (*s_abort || *reinterpret_cast<volatile unsigned*>(&sync->abort_flag)) { ok = false; break; }
+        const unsigned long long now = globaltimer_ns();
+        if (t_start == 0) t_start = now;
+        else if (now - t_start > kWaitLimitNs) {
+          sync->status = RT_ERR_TIMEOUT;
+          __threadfence();
+          atomicExch(&sync->abort_flag, 1u);
+          ok = false;
+          break;
+        }
+      }
+    }
+    ok = __all_sync(0xffffffffu, ok);
+    if (!ok) *s_abort = 1;
+    fence_async_proxy();
+    return ok;
+  }
+};
+
+// Operand fetches of one product step: the weights of the first blocks, then (after the wait) their operand rows, then the rest block by block.
+// emask / fmask: parity of the next wait on a slot's empty barrier / of the latest fill of a slot.
+// A fetch of one block of 16 KB or less costs an SM about 90 ns whatever its size, so a copy covers two blocks (a three-dimensional map:
+// 64 columns, rows, blocks).
+struct WideFetch { uint32_t emask, fmask; };
+template <typename Wait>
+__device__ __forceinline__ bool wide_fetch(const WideCta& c, WideFetch& f, const WideStage& st, const CUtensorMap* ma, const CUtensorMap* mw, const CUtensorMap* mw2, int m0,
+                                           uint32_t a_bytes, Wait wait) {
+  const uint32_t w_bytes = (uint32_t)st.bn * 128u, slot_bytes = 2u * (a_bytes + w_bytes);
+  bool ok = true, waited = false;
+  for (int job = c.rank; job < st.tiles * st.splits && ok; job += c.G) {
+    const int tile = job % st.tiles, split = job / st.tiles;
+    const int k0 = st.pairs * split / st.splits, n = st.pairs * (split + 1) / st.splits - k0;
+    const bool second = mw2 && tile >= st.tiles / 2;
+    const CUtensorMap* w = second ? mw2 : mw;
+    const int n0 = (second ? tile - st.tiles / 2 : tile) * st.bn;
+    const int pre = n < st.slots ? n : st.slots;
+    for (int k = 0; k < pre; ++k) {
+      expect_tx_elect(c.full(k), slot_bytes);
+      tma_load_3d(c.sbase + k * slot_bytes + 2u * a_bytes, w, c.full(k), 0, n0, 2 * (k0 + k));
+      f.fmask ^= 1u << k;
+    }
+    if (!waited) { ok = wait(); waited = true; }
+    for (int k = 0; k < pre; ++k) tma_load_3d(c.sbase + k * slot_bytes, ma, c.full(k), 0, m0, 2 * (k0 + k));      // (given up or not: the fill has to land)
+    int s = 0;
+    for (int k = pre; k < n && ok; ++k) {
+      ok = warp_mbar_wait(c.empty(s), (f.emask >> s) & 1u, c.s_abort, c.sync);
+      if (!ok) break;
+      f.emask ^= 1u << s;
+      f.fmask ^= 1u << s;
+      expect_tx_elect(c.full(s), slot_bytes);
+      tma_load_3d(c.sbase + s * slot_bytes, ma, c.full(s), 0, m0, 2 * (k0 + k));
+      tma_load_3d(c.sbase + s * slot_bytes + 2u * a_bytes, w, c.full(s), 0, n0, 2 * (k0 + k));
+      if (++s == st.slots) s = 0;
+    }
+    for (int j = 0; j < pre && ok; ++j) {                  // every slot read: the next product lays the ring out anew
+      ok = warp_mbar_wait(c.empty(j), (f.emask >> j) & 1u, c.s_abort, c.sync);
+      if (ok) f.emask ^= 1u << j;
+    }
+    if (!ok) {
+      // gave up: the fills under way have to land before the shared memory goes away (bounded).  fmask holds the parity AFTER the fill.
+      for (int j = 0; j < pre; ++j) {
+        unsigned spins = 0;
+        while (!mbar_try_wait(c.full(j), ((f.fmask >> j) & 1u) ^ 1u) && ++spins < (1u << 20)) {}
+      }
+    }
+  }
+  return ok;
+}
+
+// The products of one step.
+struct WideIssue { uint32_t fmask; int jobs; };
+__device__ __forceinline__ bool wide_issue(const WideCta& c, WideIssue& w, const WideStage& st, uint32_t a_bytes, uint32_t tmem) {
+  const uint32_t w_bytes = (uint32_t)st.bn * 128u, slot_bytes = 2u * (a_bytes + w_bytes), idesc = make_idesc(st.bn, false);
+  bool ok = true;
+  for (int job = c.rank; job < st.tiles * st.splits && ok; job += c.G) {
+    const int split = job / st.tiles;
+    const int n = st.pairs * (split + 1) / st.splits - st.pairs * split / st.splits;
+    const int buf = w.jobs & 1;
+    if (w.jobs >= 2) ok = warp_mbar_wait(c.tempty(buf), ((w.jobs >> 1) - 1) & 1, c.s_abort, c.sync);
+    int s = 0;
+    for (int k = 0; k < n && ok; ++k) {
+      ok = warp_mbar_wait(c.full(s), (w.fmask >> s) & 1u, c.s_abort, c.sync);
+      if (!ok) break;
+      w.fmask ^= 1u << s;
+      tc_fence_after();
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const uint64_t a0 = make_desc(c.sbase + s * slot_bytes + j * a_bytes, 16, 1024), b0 = make_desc(c.sbase + s * slot_bytes + 2u * a_bytes + j * w_bytes, 16, 1024);
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) tc_mma(tmem + (uint32_t)(buf * kWBuf), a0 + 2u * ks, b0 + 2u * ks, idesc, (k > 0 || j > 0 || ks > 0) ? 1u : 0u);
+      }
+      tc_commit(c.empty(s));
+      if (++s == st.slots) s = 0;
+    }
+    if (ok) tc_commit(c.tfull(buf));
+    ++w.jobs;
+  }
+  return ok;
+}
+
+// An accumulator block of 32 rows and W columns (16 or 32) through the warp's staging area: rows belong to lanes in TMEM, and storing them that
+// way touches 32 lines per instruction (the stores of a 128 x 128 fp32 tile took 2.6 us); afterwards W / 4 lanes hold a row, four columns each.
+// f(row of the block, column, values) is called by every lane.
+template <int W, typename F>
+__device__ __forceinline__ void wide_rows(float* st, uint32_t taddr, int lane, F f) {
+  uint32_t r[32];
+  if (W == 32) { tc_ld32(taddr, r); tc_wait_ld(); }
+  else {
+    float v[16];
+    tc_ld16(taddr, v);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(v[i]);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < W / 4; ++i) *reinterpret_cast<uint4*>(st + lane * kWStagePitch + 4 * i) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+  __syncwarp();
+  constexpr int L = W / 4;                                 // lanes per row
+#pragma unroll
+  for (int i = 0; i < L; ++i) {
+    const int row = i * (32 / L) + lane / L, col = 4 * (lane % L);
+    f(row, col, *reinterpret_cast<const float4*>(st + row * kWStagePitch + col));
+  }
+}
+
+// ---- attention of one (sequence, head) on eight lanes: the row's state (the pre-pass and the tiles before this leaf) and the leaf's keys
+struct WideAttn { float q[8], o[8], m, l; };
+__device__ __forceinline__ void wide_attn_keys(WideAttn& a, const __nv_bfloat16* K, const __nv_bfloat16* V, size_t rstride, int ka, int kb, int t, float scale_log2, float slope) {
+  for (int j0 = ka; j0 < kb; j0 += 8) {
+    uint4 kw[8], vw[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const size_t at = (size_t)(j0 + e < kb ? j0 + e : kb - 1) * rstride;
+      kw[e] = ldcg16(K + at); vw[e] = ldcg16(V + at);
+    }
+    float s[8], m_new = a.m;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      float kf[8], x = 0.f;
+      unpack8(kw[e], kf);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x = fmaf(a.q[i], kf[i], x);
+      x = sum8(x);
+      s[e] = j0 + e < kb ? x * scale_log2 - slope * (float)(t - (j0 + e)) : -INFINITY;
+      m_new = fmaxf(m_new, s[e]);
+    }
+    const float corr = exp2f(a.m - m_new);
+    a.l *= corr; a.m = m_new;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) a.o[i] *= corr;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const float pj = exp2f(s[e] - m_new);
+      float vf[8];
+      unpack8(vw[e], vf);
+      a.l += pj;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) a.o[i] = fmaf(pj, vf[i], a.o[i]);
+    }
+  }
+}
+
+// one key whose rows have been fetched
+__device__ __forceinline__ void wide_attn_one(WideAttn& a, const uint4& kw, const uint4& vw, float scale_log2, float bias) {
+  float kf[8], vf[8], x = 0.f;
+  unpack8(kw, kf); unpack8(vw, vf);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) x = fmaf(a.q[i], kf[i], x);
+  const float s = sum8(x) * scale_log2 - bias, m_new = fmaxf(a.m, s);
+  const float corr = exp2f(a.m - m_new), pj = exp2f(s - m_new);
+  a.m = m_new; a.l = a.l * corr + pj;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) a.o[i] = fmaf(pj, vf[i], a.o[i] * corr);
+}
+
+// ---- forward ------------------------------------------------------------------------------------------------
+enum { F_ATTN = 0, F_OUT = 1, F_UP = 2, F_DOWN = 3, F_Z = 4, F_KV = 5, F_STEPS = 6 };
+
+struct WideFwdMaps { CUtensorMap c, u, g, r, wo, wup, wdn, wk, wv; };
+
+__device__ __forceinline__ int wide_active_rows(int units, int per_cta, int G) {
+  const int n = (units + per_cta - 1) / per_cta;
+  return n < G ? n : G;
+}
+__device__ __forceinline__ int wide_active(const WideStage& st, int G) { return st.tiles * st.splits < G ? st.tiles * st.splits : G; }
+
+__global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid_constant__ WideFwdMaps maps, const __grid_constant__ WideFwdParams p) {
+  extern __shared__ unsigned char smem_raw[];
+  WideCta c;
+  c.smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  c.sbase = smem_u32(c.smem);
+  c.s_abort = reinterpret_cast<volatile int*>(c.smem + kWAbort);
+  c.sync = p.sync;
+  c.G = p.G;
+  const int group = blockIdx.x / p.G;
+  c.rank = blockIdx.x % p.G;
+  c.arank = p.G - 1 - c.rank;
+  c.counters = p.counters + group * kWMaxSteps * kWCounterStride;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int m0 = group * p.R, R = p.B - m0 < p.R ? p.B - m0 : p.R;
+  volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(c.smem + kWTmem);
+  if (tid == 0) {
+    *c.s_abort = 0;
+    for (int s = 0; s < kWSlotsMax; ++s) { mbar_init(c.full(s), 1); mbar_init(c.empty(s), 1); }
+    for (int b = 0; b < 2; ++b) { mbar_init(c.tfull(b), 1); mbar_init(c.tempty(b), 8); }
+    mbar_init(c.flag(), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(c.sbase + kWTmem), "n"(2 * kWBuf) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *s_tmem, a_bytes = (uint32_t)p.a_bytes;
+
+  const int d = p.d, H = p.H, chunks = d >> 7;
+  int active[F_STEPS];
+  active[F_ATTN] = wide_active_rows(R * H, 32, p.G);
+  active[F_OUT] = wide_active(p.st_out, p.G);
+  active[F_UP] = wide_active(p.st_up, p.G);
+  active[F_DOWN] = wide_active(p.st_dn, p.G);
+  active[F_Z] = wide_active_rows(R * chunks, 8, p.G);
+  active[F_KV] = wide_active(p.st_kv, p.G);
+
+  if (warp == 0) {
+    // ---------------- operand fetches and the group's barrier ----------------
+    WideFetch f = {0u, 0u};
+    bool ok = true;
+    for (int t = p.t0; t < p.t1 && ok; ++t) {
+      const unsigned n = p.steps + (unsigned)(t - p.t0);                     // positions done before this one
+      auto wait_for = [&](int step, unsigned rounds) {
+        const bool r = c.poll(step, rounds * (unsigned)active[step]);
+        if (lane == 0 && r) mbar_arrive(c.flag());
+        __syncwarp();
+        return r;
+      };
+      if (c.arank < active[F_ATTN]) {
+        if (t == p.t0) { if (lane == 0) mbar_arrive(c.flag()); __syncwarp(); }
+        else ok = wait_for(F_KV, n);
+      }
+      if (ok && c.rank < active[F_OUT]) ok = wide_fetch(c, f, p.st_out, &maps.c, &maps.wo, nullptr, m0, a_bytes, [&] { return wait_for(F_ATTN, n + 1); });
+      if (ok && c.rank < active[F_UP]) ok = wide_fetch(c, f, p.st_up, &maps.u, &maps.wup, nullptr, m0, a_bytes, [&] { return wait_for(F_OUT, n + 1); });
+      if (ok && c.rank < active[F_DOWN]) ok = wide_fetch(c, f, p.st_dn, &maps.g, &maps.wdn, nullptr, m0, a_bytes, [&] { return wait_for(F_UP, n + 1); });
+      if (ok && c.rank < active[F_Z]) ok = wait_for(F_DOWN, n + 1);
+      if (ok && c.rank < active[F_KV]) ok = wide_fetch(c, f, p.st_kv, &maps.r, &maps.wk, &maps.wv, m0, a_bytes, [&] { return wait_for(F_Z, n + 1); });
+    }
+  } else if (warp == 1) {
+    // ---------------- tensor cores ----------------
+    WideIssue w = {0u, 0};
+    bool ok = true;
+    for (int t = p.t0; t < p.t1 && ok; ++t) {
+      if (c.rank < active[F_OUT]) ok = wide_issue(c, w, p.st_out, a_bytes, tmem);
+      if (ok && c.rank < active[F_UP]) ok = wide_issue(c, w, p.st_up, a_bytes, tmem);
+      if (ok && c.rank < active[F_DOWN]) ok = wide_issue(c, w, p.st_dn, a_bytes, tmem);
+      if (ok && c.rank < active[F_KV]) ok = wide_issue(c, w, p.st_kv, a_bytes, tmem);
+    }
+  } else {
+    // ---------------- row work: eight warps, a warp reads the 32 TMEM lanes of its quadrant, two warps share a quadrant's columns ----------------
+    const int ew = warp - 2, quad = warp & 3, half = ew >> 2;
+    const int row = quad * 32 + lane, m = m0 + row;
+    const bool live = row < R;
+    const uint32_t t_row = tmem + ((uint32_t)(quad * 32) << 16);
+    const bool pre = (p.norm_flags & RT_NORM_PRE) != 0, znorm = pre && !(p.norm_flags & RT_NORM_SKIP_Z), qkn = (p.norm_flags & RT_NORM_QK) != 0;
+    const __nv_bfloat16 *g_mlp = reinterpret_cast<const __nv_bfloat16*>(p.g_mlp), *g_kv = reinterpret_cast<const __nv_bfloat16*>(p.g_kv), *g_k = reinterpret_cast<const __nv_bfloat16*>(p.g_k);
+    const __nv_bfloat16 *X = reinterpret_cast<const __nv_bfloat16*>(p.x), *Q = reinterpret_cast<const __nv_bfloat16*>(p.q);
+    __nv_bfloat16 *Z = reinterpret_cast<__nv_bfloat16*>(p.z), *Kc = reinterpret_cast<__nv_bfloat16*>(p.k_cache), *Vc = reinterpret_cast<__nv_bfloat16*>(p.v_cache);
+    const size_t rstride = (size_t)p.B * d;
+    uint32_t flags = 0;
+    int jobs = 0;
+    auto flag_wait = [&]() { const bool r = warp_mbar_wait(c.flag(), flags & 1u, c.s_abort, c.sync); ++flags; return r; };
+    auto acc_wait = [&]() {
+      const bool r = warp_mbar_wait(c.tfull(jobs & 1), (jobs >> 1) & 1, c.s_abort, c.sync);
+      tc_fence_after();
+      return r;
+    };
+    auto acc_done = [&]() {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(c.tempty(jobs & 1));
+      ++jobs;
+    };
+    auto finish = [&](bool ok, int step) {                     // this CTA's part of a step is written
+      ok = epi_all(ok);
+      if (tid == 64 && ok) { red_release_add_u32(c.counters + step * kWCounterStride, 1u); }
+      return ok;
+    };
+    // 1 / rms of this thread's row from the sums of squares that the step before left ([part][B])
+    auto row_scale = [&](const float* ssq, int parts, bool on) {
+      if (!on || !live) return 1.0f;
+      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+      const float* a = ssq + m;
+      int i = 0;
+      for (; i + 4 <= parts; i += 4) {
+        s0 += __ldcg(a + (size_t)i * p.B); s1 += __ldcg(a + (size_t)(i + 1) * p.B); s2 += __ldcg(a + (size_t)(i + 2) * p.B); s3 += __ldcg(a + (size_t)(i + 3) * p.B);
+      }
+      for (; i < parts; ++i) s0 += __ldcg(a + (size_t)i * p.B);
+      return rsqrtf(((s0 + s1) + (s2 + s3)) / (float)d + p.eps);
+    };
+    // columns [c_begin, c_end) of a tile of width bn that this warp handles, 16 at a time
+    auto col_range = [&](int bn, int& c_begin, int& c_end) {
+      if (bn == 16) { c_begin = 0; c_end = half ? 0 : 16; }
+      else { c_begin = half * (bn >> 1); c_end = c_begin + (bn >> 1); }
+    };
+    float* stage = reinterpret_cast<float*>(c.smem + kWStage + ew * kWStageWarp);
+    // the accumulator columns [ca, cb) of this warp, f(row of the quadrant, column, values)
+    auto blocks = [&](int ca, int cb, auto f) {
+      if (cb - ca >= 32) {
+        for (int cc = ca; cc < cb; cc += 32)
+          wide_rows<32>(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane, [&](int r, int col, const float4& a) { f(r, cc + col, a); });
+      } else if (ca < cb) {
+        wide_rows<16>(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + ca), lane, [&](int r, int col, const float4& a) { f(r, ca + col, a); });
+      }
+    };
+    bool ok = true;
+    for (int t = p.t0; t < p.t1 && ok; ++t) {
+      if (c.arank < active[F_ATTN]) {
+        constexpr int kAhead = 2;                              // units whose older keys are absorbed before the newest pair arrives
+        WideAttn a[kAhead];
+        const int units = R * H;
+        auto unit_of = [&](int i, bool& alive) { const int u = (i * c.G + c.arank) * 32 + ew * 4 + (lane >> 3); alive = u < units; return alive ? u : 0; };
+        auto load = [&](WideAttn& x, int u) {
+          const int b = m0 + u / H, h = u % H;
+          const size_t sidx = (size_t)t * p.B + b, at = sidx * d + h * kHeadDim + 8 * (lane & 7);
+          unpack8(*reinterpret_cast<const uint4*>(Q + at), x.q);
+          const float4 o0 = *reinterpret_cast<const float4*>(p.st_o + at), o1 = *reinterpret_cast<const float4*>(p.st_o + at + 4);
+          x.o[0] = o0.x; x.o[1] = o0.y; x.o[2] = o0.z; x.o[3] = o0.w; x.o[4] = o1.x; x.o[5] = o1.y; x.o[6] = o1.z; x.o[7] = o1.w;
+          x.m = p.st_m[sidx * H + h]; x.l = p.st_l[sidx * H + h];
+        };
+        auto keys = [&](WideAttn& x, int u, int ka, int kb) {
+          const int b = m0 + u / H, h = u % H;
+          const size_t col = (size_t)b * d + h * kHeadDim + 8 * (lane & 7);
+          wide_attn_keys(x, Kc + col, Vc + col, rstride, ka, kb, t, p.scale_log2, p.alibi ? p.alibi[h] * kLog2e : 0.f);
+        };
+        auto store = [&](const WideAttn& x, int u) {
+          const int b = m0 + u / H, h = u % H;
+          const float il = 1.0f / x.l;
+          *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.c16) + (size_t)b * d + h * kHeadDim + 8 * (lane & 7)) =
+              make_uint4(pack2(x.o[0] * il, x.o[1] * il), pack2(x.o[2] * il, x.o[3] * il), pack2(x.o[4] * il, x.o[5] * il), pack2(x.o[6] * il, x.o[7] * il));
+        };
+        const int rounds = (units + 32 * c.G - 1) / (32 * c.G);
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+          if (i < rounds) {
+            bool alive;
+            const int u = unit_of(i, alive);
+            load(a[i], u);
+            keys(a[i], u, p.t0, t - 1);
+          }
+        }
+        ok = flag_wait();
+        if (ok) {
+          uint4 kn[kAhead], vn[kAhead];
+#pragma unroll
+          for (int i = 0; i < kAhead; ++i) {
+            if (i < rounds && t > p.t0) {
+              bool alive;
+              const int u = unit_of(i, alive);
+              const size_t at = (size_t)(t - 1) * rstride + (size_t)(m0 + u / H) * d + (u % H) * kHeadDim + 8 * (lane & 7);
+              kn[i] = ldcg16(Kc + at); vn[i] = ldcg16(Vc + at);
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < kAhead; ++i) {
+            if (i < rounds) {
+              bool alive;
+              const int u = unit_of(i, alive);
+              if (t > p.t0) wide_attn_one(a[i], kn[i], vn[i], p.scale_log2, p.alibi ? p.alibi[u % H] * kLog2e : 0.f);
+              if (alive) store(a[i], u);
+            }
+          }
+        }
+        for (int i = kAhead; i < rounds && ok; ++i) {
+          bool alive;
+          const int u = unit_of(i, alive);
+          WideAttn x;
+          load(x, u);
+          keys(x, u, p.t0, t);
+          if (alive) store(x, u);
+        }
+        ok = finish(ok, F_ATTN);
+        if (!ok) break;
+      }
+      if (c.rank < active[F_OUT]) {
+        // h = x + alpha c W_o;  u = bf16(h g), sums of squares of h
+        bool good = flag_wait();
+        const int bn = p.st_out.bn, halves = bn == 16 ? 1 : 2;
+        int ca, cb;
+        col_range(bn, ca, cb);
+        for (int job = c.rank; job < p.st_out.tiles; job += c.G) {
+          const int n0 = job * bn;
+          if (!good || !(good = acc_wait())) break;
+          auto block = [&](auto width, int cc, float* sums) {
+            constexpr int W = decltype(width)::value, L = W / 4;
+            uint2 xw[L];                                       // fetched before the staging
+#pragma unroll
+            for (int i = 0; i < L; ++i) {
+              const int rr = quad * 32 + i * (32 / L) + lane / L;
+              xw[i] = *reinterpret_cast<const uint2*>(X + (size_t)(m0 + (rr < R ? rr : 0)) * p.x_bs + (size_t)t * p.x_ts + n0 + cc + 4 * (lane % L));
+            }
+            int i = 0;
+            wide_rows<W>(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane, [&](int r, int col, const float4& a) {
+              const int rr = quad * 32 + r;
+              const float h0 = __uint_as_float(xw[i].x << 16) + p.alpha * a.x, h1 = __uint_as_float(xw[i].x & 0xffff0000u) + p.alpha * a.y,
+                          h2 = __uint_as_float(xw[i].y << 16) + p.alpha * a.z, h3 = __uint_as_float(xw[i].y & 0xffff0000u) + p.alpha * a.w;
+              sums[i] = fmaf(h0, h0, fmaf(h1, h1, fmaf(h2, h2, fmaf(h3, h3, sums[i]))));
+              ++i;
+              if (rr >= R) return;
+              const int n = n0 + cc + col;
+              const size_t at = (size_t)(m0 + rr) * d + n;
+              *reinterpret_cast<float4*>(p.h + at) = make_float4(h0, h1, h2, h3);
+              float g0 = 1.f, g1 = 1.f, g2 = 1.f, g3 = 1.f;
+              if (pre && g_mlp) {
+                const uint2 gw = *reinterpret_cast<const uint2*>(g_mlp + n);
+                g0 = __uint_as_float(gw.x << 16); g1 = __uint_as_float(gw.x & 0xffff0000u); g2 = __uint_as_float(gw.y << 16); g3 = __uint_as_float(gw.y & 0xffff0000u);
+              }
+              *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.u16) + at) = make_uint2(pack2(h0 * g0, h1 * g1), pack2(h2 * g2, h3 * g3));
+            });
+          };
+          auto put = [&](float v, int L, int i) {              // the sum of squares of row i * 32 / L + lane / L over this warp's columns
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
+            v += __shfl_xor_sync(0xffffffffu, v, 2);
+            if (L == 8) v += __shfl_xor_sync(0xffffffffu, v, 4);
+            const int rr = quad * 32 + i * (32 / L) + lane / L;
+            if (lane % L == 0 && rr < R) p.ssq_h[(size_t)(job * halves + (halves == 2 ? half : 0)) * p.B + m0 + rr] = v;
+          };
+          float sums[8] = {};
+          if (cb - ca >= 32) {
+            for (int cc = ca; cc < cb; cc += 32) block(std::integral_constant<int, 32>(), cc, sums);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) put(sums[i], 8, i);
+          } else if (ca < cb) {
+            block(std::integral_constant<int, 16>(), ca, sums);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) put(sums[i], 4, i);
+          }
+          acc_done();
+        }
+        ok = finish(good, F_OUT);
+        if (!ok) break;
+      }
+      if (c.rank < active[F_UP]) {
+        // g = GELU(u W_up / rms(h))
+        bool good = flag_wait();
+        const float inv = good ? row_scale(p.ssq_h, p.st_out.tiles * (p.st_out.bn == 16 ? 1 : 2), pre) : 1.f;
+        const int bn = p.st_up.bn;
+        int ca, cb;
+        col_range(bn, ca, cb);
+        for (int job = c.rank; job < p.st_up.tiles; job += c.G) {
+          if (!good || !(good = acc_wait())) break;
+          auto put = [&](int r, int col, const float4& a) {
+            const float sc = __shfl_sync(0xffffffffu, inv, r);
+            const float g0 = gelu_wide(a.x * sc), g1 = gelu_wide(a.y * sc), g2 = gelu_wide(a.z * sc), g3 = gelu_wide(a.w * sc);
+            if (quad * 32 + r < R)
+              *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.g16) + (size_t)(m0 + quad * 32 + r) * p.dff + job * bn + col) = make_uint2(pack2(g0, g1), pack2(g2, g3));
+          };
+          blocks(ca, cb, put);
+          acc_done();
+        }
+        ok = finish(good, F_UP);
+        if (!ok) break;
+      }
+      if (c.rank < active[F_DOWN]) {
+        // a part of g W_down
+        bool good = flag_wait();
+        const int bn = p.st_dn.bn;
+        int ca, cb;
+        col_range(bn, ca, cb);
+        for (int job = c.rank; job < p.st_dn.tiles * p.st_dn.splits; job += c.G) {
+          const int n0 = (job % p.st_dn.tiles) * bn, split = job / p.st_dn.tiles;
+          if (!good || !(good = acc_wait())) break;
+          blocks(ca, cb, [&](int r, int col, const float4& a) {
+            if (quad * 32 + r < R) *reinterpret_cast<float4*>(p.partial + ((size_t)split * p.B + m0 + quad * 32 + r) * d + n0 + col) = a;
+          });
+          acc_done();
+        }
+        ok = finish(good, F_DOWN);
+        if (!ok) break;
+      }
+      if (c.rank < active[F_Z]) {
+        // z = h + alpha g W_down;  r = bf16(z g), sums of squares of z: a warp per row and 128 columns
+        constexpr int kRows = 2;                               // fetched together
+        const int total = R * chunks, step = c.G * 8;
+        auto at_of = [&](int u) { return (size_t)(m0 + u / chunks) * d + (u % chunks) * 128 + 4 * lane; };
+        float4 hv[kRows];
+        auto fetch_h = [&](int u0) {
+#pragma unroll
+          for (int k = 0; k < kRows; ++k) { const int u = u0 + k * step; hv[k] = __ldcg(reinterpret_cast<const float4*>(p.h + at_of(u < total ? u : 0))); }
+        };
+        fetch_h(c.rank * 8 + ew);                              // h is complete since the up projection began
+        const bool good = flag_wait();
+        if (good) {
+          for (int u0 = c.rank * 8 + ew; u0 < total; u0 += kRows * step) {
+            if (u0 != c.rank * 8 + ew) fetch_h(u0);
+            float4 pv[kRows][8];
+#pragma unroll
+            for (int k = 0; k < kRows; ++k) {
+              const int u = u0 + k * step;
+              const size_t at = at_of(u < total ? u : 0);
+#pragma unroll
+              for (int z = 0; z < 8; ++z)
+                if (z < p.st_dn.splits) pv[k][z] = __ldcg(reinterpret_cast<const float4*>(p.partial + (size_t)z * p.B * d + at));
+            }
+#pragma unroll
+            for (int k = 0; k < kRows; ++k) {
+              const int u = u0 + k * step;
+              if (u >= total) break;
+              const int b = m0 + u / chunks, ch = u % chunks, col = ch * 128 + 4 * lane;
+              float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+              for (int z = 0; z < 8; ++z)
+                if (z < p.st_dn.splits) { acc.x += pv[k][z].x; acc.y += pv[k][z].y; acc.z += pv[k][z].z; acc.w += pv[k][z].w; }
+              float v[4] = {hv[k].x + p.alpha * acc.x, hv[k].y + p.alpha * acc.y, hv[k].z + p.alpha * acc.z, hv[k].w + p.alpha * acc.w};
+              float ss = 0.f;
+#pragma unroll
+              for (int i = 0; i < 4; ++i) { v[i] = round_T<__nv_bfloat16>(v[i]); ss = fmaf(v[i], v[i], ss); }    // the pair comes from the stored (rounded) z
+              *reinterpret_cast<uint2*>(Z + (size_t)b * p.z_bs + (size_t)t * p.z_ts + col) = make_uint2(pack2(v[0], v[1]), pack2(v[2], v[3]));
+              ss = warp_sum(ss);
+              if (lane == 0) p.ssq_z[(size_t)ch * p.B + b] = ss;
+              if (znorm && g_kv) {
+                const uint2 gw = *reinterpret_cast<const uint2*>(g_kv + col);
+                v[0] *= __uint_as_float(gw.x << 16); v[1] *= __uint_as_float(gw.x & 0xffff0000u); v[2] *= __uint_as_float(gw.y << 16); v[3] *= __uint_as_float(gw.y & 0xffff0000u);
+              }
+              *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.r16) + (size_t)b * d + col) = make_uint2(pack2(v[0], v[1]), pack2(v[2], v[3]));
+            }
+          }
+        }
+        ok = finish(good, F_Z);
+        if (!ok) break;
+      }
+      if (c.rank < active[F_KV]) {
+        // k = qkRMS(r W_k / rms(z)), v = r W_v / rms(z): a tile is one head
+        bool good = flag_wait();
+        const float inv = good ? row_scale(p.ssq_z, chunks, znorm) : 1.f;
+        const int heads = d / kHeadDim;
+        for (int job = c.rank; job < p.st_kv.tiles; job += c.G) {
+          if (!good || !(good = acc_wait())) break;
+          const bool is_k = job < heads;
+          const int col = (is_k ? job : job - heads) * kHeadDim;
+          float v[32], ss = 0.f;
+          {
+            uint32_t w[32];
+            tc_ld32(t_row + (uint32_t)((jobs & 1) * kWBuf + half * 32), w);
+            tc_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 32; ++i) { v[i] = __uint_as_float(w[i]) * inv; ss = fmaf(v[i], v[i], ss); }
+          }
+          if (is_k && qkn) {
+            uint32_t w[32];
+            tc_ld32(t_row + (uint32_t)((jobs & 1) * kWBuf + (half ^ 1) * 32), w);
+            tc_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 32; ++i) { const float x = __uint_as_float(w[i]) * inv; ss = fmaf(x, x, ss); }
+          }
+          acc_done();
+          const float rs = is_k && qkn ? rsqrtf(ss * (1.0f / kHeadDim) + p.eps) : 1.0f;
+          const int cc = col + half * 32;
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < 8; ++i) *reinterpret_cast<float4*>(stage + lane * kWStagePitch + 4 * i) = make_float4(v[4 * i] * rs, v[4 * i + 1] * rs, v[4 * i + 2] * rs, v[4 * i + 3] * rs);
+          __syncwarp();
+          float g[4] = {1.f, 1.f, 1.f, 1.f};
+          if (is_k && qkn && g_k) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) g[i] = __bfloat162float(g_k[cc + 4 * (lane & 7) + i]);
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int r = 4 * i + (lane >> 3), rr = quad * 32 + r;
+            const float4 o = *reinterpret_cast<const float4*>(stage + r * kWStagePitch + 4 * (lane & 7));
+            if (rr < R)
+              *reinterpret_cast<uint2*>((is_k ? Kc : Vc) + (size_t)t * rstride + (size_t)(m0 + rr) * d + cc + 4 * (lane & 7)) = make_uint2(pack2(o.x * g[0], o.y * g[1]), pack2(o.z * g[2], o.w * g[3]));
+          }
+        }
+        ok = finish(good, F_KV);
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(2 * kWBuf) : "memory");
+  }
+}
+
+int ring_slots(int bn, int a_bytes) {
+  const int n = (int)(kWRing / (2u * ((unsigned)a_bytes + (unsigned)bn * 128u)));
+  return n < kWSlotsMax ? n : kWSlotsMax;
+}
+// A product of n columns over k on G CTAs, not split: the narrowest tile that gives every CTA at most one.
+WideStage stage_whole(int n, int k, int G, int a_bytes, int bn_min, int bn_max) {
+  int bn = bn_min;
+  while (bn < bn_max && (ceil_div(n, bn) > G || n % bn)) bn *= 2;
+  return {k / 128, bn, n / bn, 1, ring_slots(bn, a_bytes)};
+}
+// The same in parts of the contraction, summed by a row step: the operand rows of a part, not its weights, are what a CTA waits for, so as
+// many parts (of at least four blocks, at most eight) as the group has CTAs for; tiles of 64 columns where the group is large enough.
+WideStage stage_split(int n, int k, int G, int a_bytes) {
+  const int bn = (n / 64) * 8 <= G ? 64 : 128, pairs = k / 128;
+  int sp = G / (n / bn);
+  if (sp > 8) sp = 8;
+  if (sp > pairs / 2) sp = pairs / 2;
+  return {pairs, bn, n / bn, sp < 1 ? 1 : sp, ring_slots(bn, a_bytes)};
+}
+// [rows, cols] bf16 as blocks of 64 columns: a box is two blocks of box_rows rows
+bool map_blocks(CUtensorMap* out, const void* base, long long rows, int cols, int box_rows) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  const cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)(cols / 64)}, strides[2] = {(cuuint64_t)cols * 2, 128};
+  const cuuint32_t box[3] = {64u, (cuuint32_t)box_rows, 2u}, estr[3] = {1, 1, 1};
+  return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+}  // namespace
+
+// Groups of at most 128 sequences; beyond kWideGroupsMax of them (16 SMs each or fewer) the products are long enough for launches of their own.
+int wide_loop_groups(int B, int d, int dff) {
+  const int groups = ceil_div(B, kBM);
+  return d % 128 == 0 && dff % 128 == 0 && groups <= kWideGroupsMax ? groups : 0;
+}
+size_t wide_counter_bytes(int B) { return (size_t)ceil_div(B, kBM) * kWMaxSteps * kWCounterStride * sizeof(unsigned); }
+int wide_ssq_floats(int d) { return d / 16 + d / 128; }        // per sequence: parts of ssq_h (at most d / 16), of ssq_z
+
+cudaError_t wide_forward_launch(WideFwdParams p, cudaStream_t s) {
+  const int groups = wide_loop_groups(p.B, p.d, p.dff);
+  if (!groups) return cudaErrorInvalidValue;
+  p.R = ceil_div(p.B, groups); p.G = kB200Sms / groups;
+  const int box = (p.R + 7) / 8 * 8;
+  p.a_bytes = box * 128;
+  p.st_out = stage_whole(p.d, p.d, p.G, p.a_bytes, 16, 128);
+  p.st_up = stage_whole(p.dff, p.d, p.G, p.a_bytes, 16, 128);
+  p.st_dn = stage_split(p.d, p.dff, p.G, p.a_bytes);
+  p.st_kv = stage_whole(2 * p.d, p.d, p.G, p.a_bytes, 64, 64);             // a tile is one head
+  p.ssq_z = p.ssq_h + (size_t)(p.d / 16) * p.B;
+  WideFwdMaps m;
+  if (!map_blocks(&m.c, p.c16, p.B, p.d, box) || !map_blocks(&m.u, p.u16, p.B, p.d, box) ||
+      !map_blocks(&m.g, p.g16, p.B, p.dff, box) || !map_blocks(&m.r, p.r16, p.B, p.d, box) ||
+      !map_blocks(&m.wo, p.w_o, p.d, p.d, p.st_out.bn) || !map_blocks(&m.wup, p.w_up, p.dff, p.d, p.st_up.bn) ||
+      !map_blocks(&m.wdn, p.w_down, p.d, p.dff, p.st_dn.bn) || !map_blocks(&m.wk, p.w_k, p.d, p.d, 64) ||
+      !map_blocks(&m.wv, p.w_v, p.d, p.d, 64))
+    return cudaErrorInvalidValue;
+  const void* fn = reinterpret_cast<const void*>(&wide_forward_kernel);
+  const int smem = (int)kWTotal + 1024;
+  cudaError_t e = ensure_dynamic_smem(fn, smem);
+  if (e != cudaSuccess) return e;
+  void* args[] = {(void*)&m, (void*)&p};
+  return cudaLaunchCooperativeKernel(fn, dim3(groups * p.G), dim3(kWThreads), args, smem, s);
+}
+
+}  // namespace rt
