@@ -218,7 +218,7 @@ struct WideFwdParams {
   void *c16, *u16, *g16, *r16;                   // bf16 operand rows [B, d], [B, d_ff] (g16)
   SyncArea* sync;
   int R, G, a_bytes;                             // set by the launcher: sequences and SMs per group, bytes of an operand block
-  WideStage st_out, st_up, st_dn, st_kv;
+  WideStage st[4];                               // W_o, W_up, W_down, W_k | W_v
 };
 int wide_loop_groups(int B, int d, int dff);     // 0: not taken
 size_t wide_counter_bytes(int B);

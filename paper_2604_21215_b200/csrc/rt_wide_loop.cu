@@ -15,8 +15,6 @@
 //
 // Exchange: data through global memory (L2), a counter per step and group; a CTA's writes are fenced for the async proxy before it counts
 // itself in, the waiting CTA fences after it saw the count.  Every wait is bounded (2 s).
-#include <type_traits>
-
 #include "rt_kernels.h"
 #include "rt_tc.cuh"
 
@@ -39,17 +37,6 @@ __device__ __forceinline__ bool epi_all(bool ok) {         // barrier of the eig
   asm volatile("{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n barrier.cta.red.and.pred q, 1, 256, p;\n selp.b32 %0, 1, 0, q;\n}" : "=r"(r) : "r"((int)ok) : "memory");
   return r != 0;
 }
-// 16 consecutive columns of this thread's TMEM lane
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                 "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-               : "r"(taddr) : "memory");
-  tc_wait_ld();
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
 __device__ __forceinline__ void unpack8(const uint4& w, float (&f)[8]) {
   const unsigned a[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
@@ -66,7 +53,18 @@ __device__ __forceinline__ float sum8(float v) {           // over the eight lan
   v += __shfl_xor_sync(0xffffffffu, v, 4);
   return v;
 }
-__device__ __forceinline__ float gelu_wide(float v) { return 0.5f * v * (1.0f + erff(v * 0.70710678118654752f)); }
+// x Phi(x) with erfc by Abramowitz and Stegun 7.1.26.  Largest error 2.1e-7 (0.5 x (1 + erff) in fp32: 6.8e-7), and no cancellation for
+// negative x; a third of the instructions, which a step that applies it to 128 x 128 accumulators per CTA notices (4 us before).
+__device__ __forceinline__ float gelu_wide(float x) {
+  const float z = fabsf(x) * 0.70710678118654752f, t = __fdividef(1.0f, fmaf(0.3275911f, z, 1.0f));
+  const float poly = t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 1.061405429f, -1.453152027f), 1.421413741f), -0.284496736f), 0.254829592f);
+  const float q = 0.5f * poly * __expf(-z * z);            // Phi(-|x|)
+  return x * (x < 0.f ? q : 1.0f - q);
+}
+
+// Every step's code runs once per position, so what does not fit the instruction caches is fetched again each time: a first version of this
+// kernel with everything unrolled (295 KB) spent a third of its time on that.  Waits are out of line and loops stay loops.
+__device__ __noinline__ bool wide_wait(uint32_t bar, uint32_t parity, volatile int* s_abort, SyncArea* sync) { return warp_mbar_wait(bar, parity, s_abort, sync); }
 
 // Where a CTA stands and how its group meets.
 struct WideCta {
@@ -134,7 +132,7 @@ __device__ __forceinline__ bool wide_fetch(const WideCta& c, WideFetch& f, const
     for (int k = 0; k < pre; ++k) tma_load_3d(c.sbase + k * slot_bytes, ma, c.full(k), 0, m0, 2 * (k0 + k));      // (given up or not: the fill has to land)
     int s = 0;
     for (int k = pre; k < n && ok; ++k) {
-      ok = warp_mbar_wait(c.empty(s), (f.emask >> s) & 1u, c.s_abort, c.sync);
+      ok = wide_wait(c.empty(s), (f.emask >> s) & 1u, c.s_abort, c.sync);
       if (!ok) break;
       f.emask ^= 1u << s;
       f.fmask ^= 1u << s;
@@ -144,7 +142,7 @@ __device__ __forceinline__ bool wide_fetch(const WideCta& c, WideFetch& f, const
       if (++s == st.slots) s = 0;
     }
     for (int j = 0; j < pre && ok; ++j) {                  // every slot read: the next product lays the ring out anew
-      ok = warp_mbar_wait(c.empty(j), (f.emask >> j) & 1u, c.s_abort, c.sync);
+      ok = wide_wait(c.empty(j), (f.emask >> j) & 1u, c.s_abort, c.sync);
       if (ok) f.emask ^= 1u << j;
     }
     if (!ok) {
@@ -167,10 +165,10 @@ __device__ __forceinline__ bool wide_issue(const WideCta& c, WideIssue& w, const
     const int split = job / st.tiles;
     const int n = st.pairs * (split + 1) / st.splits - st.pairs * split / st.splits;
     const int buf = w.jobs & 1;
-    if (w.jobs >= 2) ok = warp_mbar_wait(c.tempty(buf), ((w.jobs >> 1) - 1) & 1, c.s_abort, c.sync);
+    if (w.jobs >= 2) ok = wide_wait(c.tempty(buf), ((w.jobs >> 1) - 1) & 1, c.s_abort, c.sync);
     int s = 0;
     for (int k = 0; k < n && ok; ++k) {
-      ok = warp_mbar_wait(c.full(s), (w.fmask >> s) & 1u, c.s_abort, c.sync);
+      ok = wide_wait(c.full(s), (w.fmask >> s) & 1u, c.s_abort, c.sync);
       if (!ok) break;
       w.fmask ^= 1u << s;
       tc_fence_after();
@@ -189,75 +187,67 @@ __device__ __forceinline__ bool wide_issue(const WideCta& c, WideIssue& w, const
   return ok;
 }
 
-// An accumulator block of 32 rows and W columns (16 or 32) through the warp's staging area: rows belong to lanes in TMEM, and storing them that
-// way touches 32 lines per instruction (the stores of a 128 x 128 fp32 tile took 2.6 us); afterwards W / 4 lanes hold a row, four columns each.
-// f(row of the block, column, values) is called by every lane.
-template <int W, typename F>
-__device__ __forceinline__ void wide_rows(float* st, uint32_t taddr, int lane, F f) {
+// An accumulator block of 32 rows and 32 columns through the warp's staging area: rows belong to lanes in TMEM, and storing them that way
+// touches 32 lines per instruction (the stores of a 128 x 128 fp32 tile took 2.6 us); afterwards eight lanes hold a row, four columns each.
+__device__ __forceinline__ void wide_stage(float* st, uint32_t taddr, int lane) {
   uint32_t r[32];
-  if (W == 32) { tc_ld32(taddr, r); tc_wait_ld(); }
-  else {
-    float v[16];
-    tc_ld16(taddr, v);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(v[i]);
-  }
+  tc_ld32(taddr, r);
+  tc_wait_ld();
   __syncwarp();
 #pragma unroll
-  for (int i = 0; i < W / 4; ++i) *reinterpret_cast<uint4*>(st + lane * kWStagePitch + 4 * i) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+  for (int i = 0; i < 8; ++i) *reinterpret_cast<uint4*>(st + lane * kWStagePitch + 4 * i) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
   __syncwarp();
-  constexpr int L = W / 4;                                 // lanes per row
-#pragma unroll
-  for (int i = 0; i < L; ++i) {
-    const int row = i * (32 / L) + lane / L, col = 4 * (lane % L);
-    f(row, col, *reinterpret_cast<const float4*>(st + row * kWStagePitch + col));
-  }
 }
 
 // ---- attention of one (sequence, head) on eight lanes: the row's state (the pre-pass and the tiles before this leaf) and the leaf's keys
-struct WideAttn { float q[8], o[8], m, l; };
-__device__ __forceinline__ void wide_attn_keys(WideAttn& a, const __nv_bfloat16* K, const __nv_bfloat16* V, size_t rstride, int ka, int kb, int t, float scale_log2, float slope) {
-  for (int j0 = ka; j0 < kb; j0 += 8) {
-    uint4 kw[8], vw[8];
+struct WideAttn { float q[8], o[8], m, l, slope; size_t col; };
+// the keys [ka, kb) of two units, four keys at a time
+__device__ __forceinline__ void wide_attn_keys(WideAttn (&a)[2], const __nv_bfloat16* K, const __nv_bfloat16* V, size_t rstride, int ka, int kb, int t, float scale_log2) {
+#pragma unroll 1
+  for (int j0 = ka; j0 < kb; j0 += 4) {
+    uint4 kw[2][4], vw[2][4];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
+    for (int e = 0; e < 4; ++e) {
       const size_t at = (size_t)(j0 + e < kb ? j0 + e : kb - 1) * rstride;
-      kw[e] = ldcg16(K + at); vw[e] = ldcg16(V + at);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) { kw[i][e] = ldcg16(K + at + a[i].col); vw[i][e] = ldcg16(V + at + a[i].col); }
     }
-    float s[8], m_new = a.m;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      float kf[8], x = 0.f;
-      unpack8(kw[e], kf);
+    for (int i = 0; i < 2; ++i) {
+      float s[4], m_new = a[i].m;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) x = fmaf(a.q[i], kf[i], x);
-      x = sum8(x);
-      s[e] = j0 + e < kb ? x * scale_log2 - slope * (float)(t - (j0 + e)) : -INFINITY;
-      m_new = fmaxf(m_new, s[e]);
-    }
-    const float corr = exp2f(a.m - m_new);
-    a.l *= corr; a.m = m_new;
+      for (int e = 0; e < 4; ++e) {
+        float kf[8], x = 0.f;
+        unpack8(kw[i][e], kf);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) a.o[i] *= corr;
+        for (int k = 0; k < 8; ++k) x = fmaf(a[i].q[k], kf[k], x);
+        x = sum8(x);
+        s[e] = j0 + e < kb ? x * scale_log2 - a[i].slope * (float)(t - (j0 + e)) : -INFINITY;
+        m_new = fmaxf(m_new, s[e]);
+      }
+      const float corr = exp2f(a[i].m - m_new);
+      a[i].l *= corr; a[i].m = m_new;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const float pj = exp2f(s[e] - m_new);
-      float vf[8];
-      unpack8(vw[e], vf);
-      a.l += pj;
+      for (int k = 0; k < 8; ++k) a[i].o[k] *= corr;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) a.o[i] = fmaf(pj, vf[i], a.o[i]);
+      for (int e = 0; e < 4; ++e) {
+        const float pj = exp2f(s[e] - m_new);
+        float vf[8];
+        unpack8(vw[i][e], vf);
+        a[i].l += pj;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) a[i].o[k] = fmaf(pj, vf[k], a[i].o[k]);
+      }
     }
   }
 }
-
 // one key whose rows have been fetched
-__device__ __forceinline__ void wide_attn_one(WideAttn& a, const uint4& kw, const uint4& vw, float scale_log2, float bias) {
+__device__ __forceinline__ void wide_attn_one(WideAttn& a, const uint4& kw, const uint4& vw, float scale_log2) {
   float kf[8], vf[8], x = 0.f;
   unpack8(kw, kf); unpack8(vw, vf);
 #pragma unroll
   for (int i = 0; i < 8; ++i) x = fmaf(a.q[i], kf[i], x);
-  const float s = sum8(x) * scale_log2 - bias, m_new = fmaxf(a.m, s);
+  const float s = sum8(x) * scale_log2 - a.slope, m_new = fmaxf(a.m, s);
   const float corr = exp2f(a.m - m_new), pj = exp2f(s - m_new);
   a.m = m_new; a.l = a.l * corr + pj;
 #pragma unroll
@@ -267,7 +257,8 @@ __device__ __forceinline__ void wide_attn_one(WideAttn& a, const uint4& kw, cons
 // ---- forward ------------------------------------------------------------------------------------------------
 enum { F_ATTN = 0, F_OUT = 1, F_UP = 2, F_DOWN = 3, F_Z = 4, F_KV = 5, F_STEPS = 6 };
 
-struct WideFwdMaps { CUtensorMap c, u, g, r, wo, wup, wdn, wk, wv; };
+// The products in the order of the chain (indices of WideFwdParams::st): W_o, W_up, W_down, W_k | W_v; the last map is W_v's.
+struct WideFwdMaps { CUtensorMap a[4], w[5]; };
 
 __device__ __forceinline__ int wide_active_rows(int units, int per_cta, int G) {
   const int n = (units + per_cta - 1) / per_cta;
@@ -307,46 +298,47 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
   const uint32_t tmem = *s_tmem, a_bytes = (uint32_t)p.a_bytes;
 
   const int d = p.d, H = p.H, chunks = d >> 7;
-  int active[F_STEPS];
-  active[F_ATTN] = wide_active_rows(R * H, 32, p.G);
-  active[F_OUT] = wide_active(p.st_out, p.G);
-  active[F_UP] = wide_active(p.st_up, p.G);
-  active[F_DOWN] = wide_active(p.st_dn, p.G);
-  active[F_Z] = wide_active_rows(R * chunks, 8, p.G);
-  active[F_KV] = wide_active(p.st_kv, p.G);
+  auto active_of = [&](int step) {                             // CTAs of the group that have work in a step
+    if (step == F_ATTN) return wide_active_rows(R * H, 64, p.G);
+    if (step == F_Z) return wide_active_rows(R * chunks, 8, p.G);
+    return wide_active(p.st[step < F_Z ? step - 1 : 3], p.G);
+  };
 
   if (warp == 0) {
     // ---------------- operand fetches and the group's barrier ----------------
     WideFetch f = {0u, 0u};
     bool ok = true;
+#pragma unroll 1
     for (int t = p.t0; t < p.t1 && ok; ++t) {
       const unsigned n = p.steps + (unsigned)(t - p.t0);                     // positions done before this one
-      auto wait_for = [&](int step, unsigned rounds) {
-        const bool r = c.poll(step, rounds * (unsigned)active[step]);
-        if (lane == 0 && r) mbar_arrive(c.flag());
-        __syncwarp();
-        return r;
-      };
-      if (c.arank < active[F_ATTN]) {
-        if (t == p.t0) { if (lane == 0) mbar_arrive(c.flag()); __syncwarp(); }
-        else ok = wait_for(F_KV, n);
+      int product = 0;
+#pragma unroll 1
+      for (int step = 0; step < F_STEPS && ok; ++step) {
+        const bool rows = step == F_ATTN || step == F_Z;
+        const int mine = step == F_ATTN ? c.arank : c.rank;
+        auto wait = [&]() {
+          bool r = true;
+          if (step == F_ATTN) { if (t > p.t0) r = c.poll(F_KV, n * (unsigned)active_of(F_KV)); }
+          else r = c.poll(step - 1, (n + 1) * (unsigned)active_of(step - 1));
+          if (lane == 0 && r) mbar_arrive(c.flag());
+          __syncwarp();
+          return r;
+        };
+        if (mine < active_of(step)) {
+          if (rows) ok = wait();
+          else ok = wide_fetch(c, f, p.st[product], &maps.a[product], &maps.w[product], step == F_KV ? &maps.w[4] : nullptr, m0, a_bytes, wait);
+        }
+        if (!rows) ++product;
       }
-      if (ok && c.rank < active[F_OUT]) ok = wide_fetch(c, f, p.st_out, &maps.c, &maps.wo, nullptr, m0, a_bytes, [&] { return wait_for(F_ATTN, n + 1); });
-      if (ok && c.rank < active[F_UP]) ok = wide_fetch(c, f, p.st_up, &maps.u, &maps.wup, nullptr, m0, a_bytes, [&] { return wait_for(F_OUT, n + 1); });
-      if (ok && c.rank < active[F_DOWN]) ok = wide_fetch(c, f, p.st_dn, &maps.g, &maps.wdn, nullptr, m0, a_bytes, [&] { return wait_for(F_UP, n + 1); });
-      if (ok && c.rank < active[F_Z]) ok = wait_for(F_DOWN, n + 1);
-      if (ok && c.rank < active[F_KV]) ok = wide_fetch(c, f, p.st_kv, &maps.r, &maps.wk, &maps.wv, m0, a_bytes, [&] { return wait_for(F_Z, n + 1); });
     }
   } else if (warp == 1) {
     // ---------------- tensor cores ----------------
     WideIssue w = {0u, 0};
     bool ok = true;
-    for (int t = p.t0; t < p.t1 && ok; ++t) {
-      if (c.rank < active[F_OUT]) ok = wide_issue(c, w, p.st_out, a_bytes, tmem);
-      if (ok && c.rank < active[F_UP]) ok = wide_issue(c, w, p.st_up, a_bytes, tmem);
-      if (ok && c.rank < active[F_DOWN]) ok = wide_issue(c, w, p.st_dn, a_bytes, tmem);
-      if (ok && c.rank < active[F_KV]) ok = wide_issue(c, w, p.st_kv, a_bytes, tmem);
-    }
+#pragma unroll 1
+    for (int t = p.t0; t < p.t1 && ok; ++t)
+#pragma unroll 1
+      for (int product = 0; product < 4 && ok; ++product) ok = wide_issue(c, w, p.st[product], a_bytes, tmem);
   } else {
     // ---------------- row work: eight warps, a warp reads the 32 TMEM lanes of its quadrant, two warps share a quadrant's columns ----------------
     const int ew = warp - 2, quad = warp & 3, half = ew >> 2;
@@ -360,9 +352,9 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
     const size_t rstride = (size_t)p.B * d;
     uint32_t flags = 0;
     int jobs = 0;
-    auto flag_wait = [&]() { const bool r = warp_mbar_wait(c.flag(), flags & 1u, c.s_abort, c.sync); ++flags; return r; };
+    auto flag_wait = [&]() { const bool r = wide_wait(c.flag(), flags & 1u, c.s_abort, c.sync); ++flags; return r; };
     auto acc_wait = [&]() {
-      const bool r = warp_mbar_wait(c.tfull(jobs & 1), (jobs >> 1) & 1, c.s_abort, c.sync);
+      const bool r = wide_wait(c.tfull(jobs & 1), (jobs >> 1) & 1, c.s_abort, c.sync);
       tc_fence_after();
       return r;
     };
@@ -389,179 +381,144 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
       for (; i < parts; ++i) s0 += __ldcg(a + (size_t)i * p.B);
       return rsqrtf(((s0 + s1) + (s2 + s3)) / (float)d + p.eps);
     };
-    // columns [c_begin, c_end) of a tile of width bn that this warp handles, 16 at a time
-    auto col_range = [&](int bn, int& c_begin, int& c_end) {
-      if (bn == 16) { c_begin = 0; c_end = half ? 0 : 16; }
-      else { c_begin = half * (bn >> 1); c_end = c_begin + (bn >> 1); }
-    };
     float* stage = reinterpret_cast<float*>(c.smem + kWStage + ew * kWStageWarp);
-    // the accumulator columns [ca, cb) of this warp, f(row of the quadrant, column, values)
-    auto blocks = [&](int ca, int cb, auto f) {
-      if (cb - ca >= 32) {
-        for (int cc = ca; cc < cb; cc += 32)
-          wide_rows<32>(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane, [&](int r, int col, const float4& a) { f(r, cc + col, a); });
-      } else if (ca < cb) {
-        wide_rows<16>(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + ca), lane, [&](int r, int col, const float4& a) { f(r, ca + col, a); });
+    // this warp's half of an accumulator of bn columns, f(row of the quadrant, column, values) called by every lane
+    auto blocks = [&](int bn, auto f) {
+#pragma unroll 1
+      for (int cc = half * (bn >> 1); cc < (half + 1) * (bn >> 1); cc += 32) {
+        wide_stage(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane);
+#pragma unroll 2
+        for (int i = 0; i < 8; ++i) {
+          const int r = 4 * i + (lane >> 3), col = 4 * (lane & 7);
+          f(r, cc + col, *reinterpret_cast<const float4*>(stage + r * kWStagePitch + col));
+        }
       }
     };
     bool ok = true;
+#pragma unroll 1
     for (int t = p.t0; t < p.t1 && ok; ++t) {
-      if (c.arank < active[F_ATTN]) {
-        constexpr int kAhead = 2;                              // units whose older keys are absorbed before the newest pair arrives
-        WideAttn a[kAhead];
-        const int units = R * H;
-        auto unit_of = [&](int i, bool& alive) { const int u = (i * c.G + c.arank) * 32 + ew * 4 + (lane >> 3); alive = u < units; return alive ? u : 0; };
-        auto load = [&](WideAttn& x, int u) {
-          const int b = m0 + u / H, h = u % H;
-          const size_t sidx = (size_t)t * p.B + b, at = sidx * d + h * kHeadDim + 8 * (lane & 7);
-          unpack8(*reinterpret_cast<const uint4*>(Q + at), x.q);
-          const float4 o0 = *reinterpret_cast<const float4*>(p.st_o + at), o1 = *reinterpret_cast<const float4*>(p.st_o + at + 4);
-          x.o[0] = o0.x; x.o[1] = o0.y; x.o[2] = o0.z; x.o[3] = o0.w; x.o[4] = o1.x; x.o[5] = o1.y; x.o[6] = o1.z; x.o[7] = o1.w;
-          x.m = p.st_m[sidx * H + h]; x.l = p.st_l[sidx * H + h];
-        };
-        auto keys = [&](WideAttn& x, int u, int ka, int kb) {
-          const int b = m0 + u / H, h = u % H;
-          const size_t col = (size_t)b * d + h * kHeadDim + 8 * (lane & 7);
-          wide_attn_keys(x, Kc + col, Vc + col, rstride, ka, kb, t, p.scale_log2, p.alibi ? p.alibi[h] * kLog2e : 0.f);
-        };
-        auto store = [&](const WideAttn& x, int u) {
-          const int b = m0 + u / H, h = u % H;
-          const float il = 1.0f / x.l;
-          *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.c16) + (size_t)b * d + h * kHeadDim + 8 * (lane & 7)) =
-              make_uint4(pack2(x.o[0] * il, x.o[1] * il), pack2(x.o[2] * il, x.o[3] * il), pack2(x.o[4] * il, x.o[5] * il), pack2(x.o[6] * il, x.o[7] * il));
-        };
-        const int rounds = (units + 32 * c.G - 1) / (32 * c.G);
+      if (c.arank < active_of(F_ATTN)) {
+        // eight lanes per (sequence, head), two of these at a time per group of lanes; the keys before the newest were complete a position ago
+        const int units = R * H, per_round = 64 * c.G;
+        bool waited = false;
+#pragma unroll 1
+        for (int u0 = c.arank * 64 + ew * 8 + (lane >> 3); u0 - (lane >> 3) < units && ok; u0 += per_round) {
+          WideAttn a[2];
 #pragma unroll
-        for (int i = 0; i < kAhead; ++i) {
-          if (i < rounds) {
-            bool alive;
-            const int u = unit_of(i, alive);
-            load(a[i], u);
-            keys(a[i], u, p.t0, t - 1);
+          for (int i = 0; i < 2; ++i) {
+            const int u = u0 + 4 * i < units ? u0 + 4 * i : 0, b = m0 + u / H, h = u % H;
+            const size_t sidx = (size_t)t * p.B + b;
+            a[i].col = (size_t)b * d + h * kHeadDim + 8 * (lane & 7);
+            const size_t at = (size_t)t * rstride + a[i].col;
+            unpack8(*reinterpret_cast<const uint4*>(Q + at), a[i].q);
+            const float4 o0 = *reinterpret_cast<const float4*>(p.st_o + at), o1 = *reinterpret_cast<const float4*>(p.st_o + at + 4);
+            a[i].o[0] = o0.x; a[i].o[1] = o0.y; a[i].o[2] = o0.z; a[i].o[3] = o0.w; a[i].o[4] = o1.x; a[i].o[5] = o1.y; a[i].o[6] = o1.z; a[i].o[7] = o1.w;
+            a[i].m = p.st_m[sidx * H + h]; a[i].l = p.st_l[sidx * H + h];
+            a[i].slope = p.alibi ? p.alibi[h] * kLog2e : 0.f;
           }
-        }
-        ok = flag_wait();
-        if (ok) {
-          uint4 kn[kAhead], vn[kAhead];
+          wide_attn_keys(a, Kc, Vc, rstride, p.t0, t - 1, t, p.scale_log2);
+          if (!waited) { ok = flag_wait(); waited = true; }
+          if (!ok) break;
+          if (t > p.t0) {
+            uint4 kn[2], vn[2];
 #pragma unroll
-          for (int i = 0; i < kAhead; ++i) {
-            if (i < rounds && t > p.t0) {
-              bool alive;
-              const int u = unit_of(i, alive);
-              const size_t at = (size_t)(t - 1) * rstride + (size_t)(m0 + u / H) * d + (u % H) * kHeadDim + 8 * (lane & 7);
-              kn[i] = ldcg16(Kc + at); vn[i] = ldcg16(Vc + at);
-            }
+            for (int i = 0; i < 2; ++i) { kn[i] = ldcg16(Kc + (size_t)(t - 1) * rstride + a[i].col); vn[i] = ldcg16(Vc + (size_t)(t - 1) * rstride + a[i].col); }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) wide_attn_one(a[i], kn[i], vn[i], p.scale_log2);
           }
 #pragma unroll
-          for (int i = 0; i < kAhead; ++i) {
-            if (i < rounds) {
-              bool alive;
-              const int u = unit_of(i, alive);
-              if (t > p.t0) wide_attn_one(a[i], kn[i], vn[i], p.scale_log2, p.alibi ? p.alibi[u % H] * kLog2e : 0.f);
-              if (alive) store(a[i], u);
-            }
+          for (int i = 0; i < 2; ++i) {
+            const float il = 1.0f / a[i].l;
+            if (u0 + 4 * i < units)
+              *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.c16) + a[i].col) =
+                  make_uint4(pack2(a[i].o[0] * il, a[i].o[1] * il), pack2(a[i].o[2] * il, a[i].o[3] * il), pack2(a[i].o[4] * il, a[i].o[5] * il), pack2(a[i].o[6] * il, a[i].o[7] * il));
           }
         }
-        for (int i = kAhead; i < rounds && ok; ++i) {
-          bool alive;
-          const int u = unit_of(i, alive);
-          WideAttn x;
-          load(x, u);
-          keys(x, u, p.t0, t);
-          if (alive) store(x, u);
-        }
+        if (!waited) ok = flag_wait();                         // (a warp without units)
         ok = finish(ok, F_ATTN);
         if (!ok) break;
       }
-      if (c.rank < active[F_OUT]) {
+      if (c.rank < active_of(F_OUT)) {
         // h = x + alpha c W_o;  u = bf16(h g), sums of squares of h
         bool good = flag_wait();
-        const int bn = p.st_out.bn, halves = bn == 16 ? 1 : 2;
-        int ca, cb;
-        col_range(bn, ca, cb);
-        for (int job = c.rank; job < p.st_out.tiles; job += c.G) {
+        const int bn = p.st[0].bn;
+#pragma unroll 1
+        for (int job = c.rank; job < p.st[0].tiles; job += c.G) {
           const int n0 = job * bn;
-          if (!good || !(good = acc_wait())) break;
-          auto block = [&](auto width, int cc, float* sums) {
-            constexpr int W = decltype(width)::value, L = W / 4;
-            uint2 xw[L];                                       // fetched before the staging
+          uint2 xw[8];                                         // x of the first 32 columns: fetched before the accumulators are there
+          auto fetch_x = [&](int cc) {
 #pragma unroll
-            for (int i = 0; i < L; ++i) {
-              const int rr = quad * 32 + i * (32 / L) + lane / L;
-              xw[i] = *reinterpret_cast<const uint2*>(X + (size_t)(m0 + (rr < R ? rr : 0)) * p.x_bs + (size_t)t * p.x_ts + n0 + cc + 4 * (lane % L));
+            for (int i = 0; i < 8; ++i) {
+              const int rr = quad * 32 + 4 * i + (lane >> 3);
+              xw[i] = *reinterpret_cast<const uint2*>(X + (size_t)(m0 + (rr < R ? rr : 0)) * p.x_bs + (size_t)t * p.x_ts + n0 + cc + 4 * (lane & 7));
             }
-            int i = 0;
-            wide_rows<W>(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane, [&](int r, int col, const float4& a) {
-              const int rr = quad * 32 + r;
+          };
+          fetch_x(half * (bn >> 1));
+          if (!good || !(good = acc_wait())) break;
+          float sums[8] = {};
+#pragma unroll 1
+          for (int cc = half * (bn >> 1); cc < (half + 1) * (bn >> 1); cc += 32) {
+            if (cc != half * (bn >> 1)) fetch_x(cc);
+            const int n = n0 + cc + 4 * (lane & 7);
+            float g0 = 1.f, g1 = 1.f, g2 = 1.f, g3 = 1.f;
+            if (pre && g_mlp) {
+              const uint2 gw = *reinterpret_cast<const uint2*>(g_mlp + n);
+              g0 = __uint_as_float(gw.x << 16); g1 = __uint_as_float(gw.x & 0xffff0000u); g2 = __uint_as_float(gw.y << 16); g3 = __uint_as_float(gw.y & 0xffff0000u);
+            }
+            wide_stage(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int r = 4 * i + (lane >> 3);
+              const float4 a = *reinterpret_cast<const float4*>(stage + r * kWStagePitch + 4 * (lane & 7));
               const float h0 = __uint_as_float(xw[i].x << 16) + p.alpha * a.x, h1 = __uint_as_float(xw[i].x & 0xffff0000u) + p.alpha * a.y,
                           h2 = __uint_as_float(xw[i].y << 16) + p.alpha * a.z, h3 = __uint_as_float(xw[i].y & 0xffff0000u) + p.alpha * a.w;
               sums[i] = fmaf(h0, h0, fmaf(h1, h1, fmaf(h2, h2, fmaf(h3, h3, sums[i]))));
-              ++i;
-              if (rr >= R) return;
-              const int n = n0 + cc + col;
-              const size_t at = (size_t)(m0 + rr) * d + n;
-              *reinterpret_cast<float4*>(p.h + at) = make_float4(h0, h1, h2, h3);
-              float g0 = 1.f, g1 = 1.f, g2 = 1.f, g3 = 1.f;
-              if (pre && g_mlp) {
-                const uint2 gw = *reinterpret_cast<const uint2*>(g_mlp + n);
-                g0 = __uint_as_float(gw.x << 16); g1 = __uint_as_float(gw.x & 0xffff0000u); g2 = __uint_as_float(gw.y << 16); g3 = __uint_as_float(gw.y & 0xffff0000u);
+              if (quad * 32 + r < R) {
+                const size_t at = (size_t)(m0 + quad * 32 + r) * d + n;
+                *reinterpret_cast<float4*>(p.h + at) = make_float4(h0, h1, h2, h3);
+                *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.u16) + at) = make_uint2(pack2(h0 * g0, h1 * g1), pack2(h2 * g2, h3 * g3));
               }
-              *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.u16) + at) = make_uint2(pack2(h0 * g0, h1 * g1), pack2(h2 * g2, h3 * g3));
-            });
-          };
-          auto put = [&](float v, int L, int i) {              // the sum of squares of row i * 32 / L + lane / L over this warp's columns
-            v += __shfl_xor_sync(0xffffffffu, v, 1);
-            v += __shfl_xor_sync(0xffffffffu, v, 2);
-            if (L == 8) v += __shfl_xor_sync(0xffffffffu, v, 4);
-            const int rr = quad * 32 + i * (32 / L) + lane / L;
-            if (lane % L == 0 && rr < R) p.ssq_h[(size_t)(job * halves + (halves == 2 ? half : 0)) * p.B + m0 + rr] = v;
-          };
-          float sums[8] = {};
-          if (cb - ca >= 32) {
-            for (int cc = ca; cc < cb; cc += 32) block(std::integral_constant<int, 32>(), cc, sums);
+            }
+          }
 #pragma unroll
-            for (int i = 0; i < 8; ++i) put(sums[i], 8, i);
-          } else if (ca < cb) {
-            block(std::integral_constant<int, 16>(), ca, sums);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) put(sums[i], 4, i);
+          for (int i = 0; i < 8; ++i) {                        // the sum of squares of a row over this warp's columns
+            const float v = sum8(sums[i]);
+            const int rr = quad * 32 + 4 * i + (lane >> 3);
+            if ((lane & 7) == 0 && rr < R) p.ssq_h[(size_t)(2 * job + half) * p.B + m0 + rr] = v;
           }
           acc_done();
         }
         ok = finish(good, F_OUT);
         if (!ok) break;
       }
-      if (c.rank < active[F_UP]) {
+      if (c.rank < active_of(F_UP)) {
         // g = GELU(u W_up / rms(h))
         bool good = flag_wait();
-        const float inv = good ? row_scale(p.ssq_h, p.st_out.tiles * (p.st_out.bn == 16 ? 1 : 2), pre) : 1.f;
-        const int bn = p.st_up.bn;
-        int ca, cb;
-        col_range(bn, ca, cb);
-        for (int job = c.rank; job < p.st_up.tiles; job += c.G) {
+        const float inv = good ? row_scale(p.ssq_h, p.st[0].tiles * 2, pre) : 1.f;
+        const int bn = p.st[1].bn;
+#pragma unroll 1
+        for (int job = c.rank; job < p.st[1].tiles; job += c.G) {
           if (!good || !(good = acc_wait())) break;
-          auto put = [&](int r, int col, const float4& a) {
+          blocks(bn, [&](int r, int col, const float4& a) {
             const float sc = __shfl_sync(0xffffffffu, inv, r);
             const float g0 = gelu_wide(a.x * sc), g1 = gelu_wide(a.y * sc), g2 = gelu_wide(a.z * sc), g3 = gelu_wide(a.w * sc);
             if (quad * 32 + r < R)
               *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.g16) + (size_t)(m0 + quad * 32 + r) * p.dff + job * bn + col) = make_uint2(pack2(g0, g1), pack2(g2, g3));
-          };
-          blocks(ca, cb, put);
+          });
           acc_done();
         }
         ok = finish(good, F_UP);
         if (!ok) break;
       }
-      if (c.rank < active[F_DOWN]) {
+      if (c.rank < active_of(F_DOWN)) {
         // a part of g W_down
         bool good = flag_wait();
-        const int bn = p.st_dn.bn;
-        int ca, cb;
-        col_range(bn, ca, cb);
-        for (int job = c.rank; job < p.st_dn.tiles * p.st_dn.splits; job += c.G) {
-          const int n0 = (job % p.st_dn.tiles) * bn, split = job / p.st_dn.tiles;
+        const int bn = p.st[2].bn;
+#pragma unroll 1
+        for (int job = c.rank; job < p.st[2].tiles * p.st[2].splits; job += c.G) {
+          const int n0 = (job % p.st[2].tiles) * bn, split = job / p.st[2].tiles;
           if (!good || !(good = acc_wait())) break;
-          blocks(ca, cb, [&](int r, int col, const float4& a) {
+          blocks(bn, [&](int r, int col, const float4& a) {
             if (quad * 32 + r < R) *reinterpret_cast<float4*>(p.partial + ((size_t)split * p.B + m0 + quad * 32 + r) * d + n0 + col) = a;
           });
           acc_done();
@@ -569,7 +526,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
         ok = finish(good, F_DOWN);
         if (!ok) break;
       }
-      if (c.rank < active[F_Z]) {
+      if (c.rank < active_of(F_Z)) {
         // z = h + alpha g W_down;  r = bf16(z g), sums of squares of z: a warp per row and 128 columns
         constexpr int kRows = 2;                               // fetched together
         const int total = R * chunks, step = c.G * 8;
@@ -579,11 +536,13 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
 #pragma unroll
           for (int k = 0; k < kRows; ++k) { const int u = u0 + k * step; hv[k] = __ldcg(reinterpret_cast<const float4*>(p.h + at_of(u < total ? u : 0))); }
         };
-        fetch_h(c.rank * 8 + ew);                              // h is complete since the up projection began
+        const bool ahead = c.rank < active_of(F_UP) || c.rank < active_of(F_DOWN);      // such a CTA has seen that h is complete
+        if (ahead) fetch_h(c.rank * 8 + ew);
         const bool good = flag_wait();
         if (good) {
+#pragma unroll 1
           for (int u0 = c.rank * 8 + ew; u0 < total; u0 += kRows * step) {
-            if (u0 != c.rank * 8 + ew) fetch_h(u0);
+            if (!ahead || u0 != c.rank * 8 + ew) fetch_h(u0);
             float4 pv[kRows][8];
 #pragma unroll
             for (int k = 0; k < kRows; ++k) {
@@ -591,7 +550,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
               const size_t at = at_of(u < total ? u : 0);
 #pragma unroll
               for (int z = 0; z < 8; ++z)
-                if (z < p.st_dn.splits) pv[k][z] = __ldcg(reinterpret_cast<const float4*>(p.partial + (size_t)z * p.B * d + at));
+                if (z < p.st[2].splits) pv[k][z] = __ldcg(reinterpret_cast<const float4*>(p.partial + (size_t)z * p.B * d + at));
             }
 #pragma unroll
             for (int k = 0; k < kRows; ++k) {
@@ -601,7 +560,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
               float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
               for (int z = 0; z < 8; ++z)
-                if (z < p.st_dn.splits) { acc.x += pv[k][z].x; acc.y += pv[k][z].y; acc.z += pv[k][z].z; acc.w += pv[k][z].w; }
+                if (z < p.st[2].splits) { acc.x += pv[k][z].x; acc.y += pv[k][z].y; acc.z += pv[k][z].z; acc.w += pv[k][z].w; }
               float v[4] = {hv[k].x + p.alpha * acc.x, hv[k].y + p.alpha * acc.y, hv[k].z + p.alpha * acc.z, hv[k].w + p.alpha * acc.w};
               float ss = 0.f;
 #pragma unroll
@@ -620,12 +579,13 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
         ok = finish(good, F_Z);
         if (!ok) break;
       }
-      if (c.rank < active[F_KV]) {
+      if (c.rank < active_of(F_KV)) {
         // k = qkRMS(r W_k / rms(z)), v = r W_v / rms(z): a tile is one head
         bool good = flag_wait();
         const float inv = good ? row_scale(p.ssq_z, chunks, znorm) : 1.f;
         const int heads = d / kHeadDim;
-        for (int job = c.rank; job < p.st_kv.tiles; job += c.G) {
+#pragma unroll 1
+        for (int job = c.rank; job < p.st[3].tiles; job += c.G) {
           if (!good || !(good = acc_wait())) break;
           const bool is_k = job < heads;
           const int col = (is_k ? job : job - heads) * kHeadDim;
@@ -682,7 +642,7 @@ int ring_slots(int bn, int a_bytes) {
 }
 // A product of n columns over k on G CTAs, not split: the narrowest tile that gives every CTA at most one.
 WideStage stage_whole(int n, int k, int G, int a_bytes, int bn_min, int bn_max) {
-  int bn = bn_min;
+  int bn = bn_min;                                         // (d and d_ff are multiples of 128)
   while (bn < bn_max && (ceil_div(n, bn) > G || n % bn)) bn *= 2;
   return {k / 128, bn, n / bn, 1, ring_slots(bn, a_bytes)};
 }
@@ -712,7 +672,7 @@ int wide_loop_groups(int B, int d, int dff) {
   return d % 128 == 0 && dff % 128 == 0 && groups <= kWideGroupsMax ? groups : 0;
 }
 size_t wide_counter_bytes(int B) { return (size_t)ceil_div(B, kBM) * kWMaxSteps * kWCounterStride * sizeof(unsigned); }
-int wide_ssq_floats(int d) { return d / 16 + d / 128; }        // per sequence: parts of ssq_h (at most d / 16), of ssq_z
+int wide_ssq_floats(int d) { return d / 32 + d / 128; }        // per sequence: parts of ssq_h (at most d / 32), of ssq_z
 
 cudaError_t wide_forward_launch(WideFwdParams p, cudaStream_t s) {
   const int groups = wide_loop_groups(p.B, p.d, p.dff);
@@ -720,17 +680,17 @@ cudaError_t wide_forward_launch(WideFwdParams p, cudaStream_t s) {
   p.R = ceil_div(p.B, groups); p.G = kB200Sms / groups;
   const int box = (p.R + 7) / 8 * 8;
   p.a_bytes = box * 128;
-  p.st_out = stage_whole(p.d, p.d, p.G, p.a_bytes, 16, 128);
-  p.st_up = stage_whole(p.dff, p.d, p.G, p.a_bytes, 16, 128);
-  p.st_dn = stage_split(p.d, p.dff, p.G, p.a_bytes);
-  p.st_kv = stage_whole(2 * p.d, p.d, p.G, p.a_bytes, 64, 64);             // a tile is one head
-  p.ssq_z = p.ssq_h + (size_t)(p.d / 16) * p.B;
+  p.st[0] = stage_whole(p.d, p.d, p.G, p.a_bytes, 64, 128);
+  p.st[1] = stage_whole(p.dff, p.d, p.G, p.a_bytes, 64, 128);
+  p.st[2] = stage_split(p.d, p.dff, p.G, p.a_bytes);
+  p.st[3] = stage_whole(2 * p.d, p.d, p.G, p.a_bytes, 64, 64);             // a tile is one head
+  p.ssq_z = p.ssq_h + (size_t)(p.d / 32) * p.B;
   WideFwdMaps m;
-  if (!map_blocks(&m.c, p.c16, p.B, p.d, box) || !map_blocks(&m.u, p.u16, p.B, p.d, box) ||
-      !map_blocks(&m.g, p.g16, p.B, p.dff, box) || !map_blocks(&m.r, p.r16, p.B, p.d, box) ||
-      !map_blocks(&m.wo, p.w_o, p.d, p.d, p.st_out.bn) || !map_blocks(&m.wup, p.w_up, p.dff, p.d, p.st_up.bn) ||
-      !map_blocks(&m.wdn, p.w_down, p.d, p.dff, p.st_dn.bn) || !map_blocks(&m.wk, p.w_k, p.d, p.d, 64) ||
-      !map_blocks(&m.wv, p.w_v, p.d, p.d, 64))
+  if (!map_blocks(&m.a[0], p.c16, p.B, p.d, box) || !map_blocks(&m.a[1], p.u16, p.B, p.d, box) ||
+      !map_blocks(&m.a[2], p.g16, p.B, p.dff, box) || !map_blocks(&m.a[3], p.r16, p.B, p.d, box) ||
+      !map_blocks(&m.w[0], p.w_o, p.d, p.d, p.st[0].bn) || !map_blocks(&m.w[1], p.w_up, p.dff, p.d, p.st[1].bn) ||
+      !map_blocks(&m.w[2], p.w_down, p.d, p.dff, p.st[2].bn) || !map_blocks(&m.w[3], p.w_k, p.d, p.d, 64) ||
+      !map_blocks(&m.w[4], p.w_v, p.d, p.d, 64))
     return cudaErrorInvalidValue;
   const void* fn = reinterpret_cast<const void*>(&wide_forward_kernel);
   const int smem = (int)kWTotal + 1024;
