@@ -15,6 +15,8 @@
 //
 // Exchange: data through global memory (L2), a counter per step and group; a CTA's writes are fenced for the async proxy before it counts
 // itself in, the waiting CTA fences after it saw the count.  Every wait is bounded (2 s).
+#include <type_traits>
+
 #include "rt_kernels.h"
 #include "rt_tc.cuh"
 
@@ -62,8 +64,6 @@ __device__ __forceinline__ float gelu_wide(float x) {
   return x * (x < 0.f ? q : 1.0f - q);
 }
 
-// Every step's code runs once per position, so what does not fit the instruction caches is fetched again each time: a first version of this
-// kernel with everything unrolled (295 KB) spent a third of its time on that.  Waits are out of line and loops stay loops.
 __device__ __noinline__ bool wide_wait(uint32_t bar, uint32_t parity, volatile int* s_abort, SyncArea* sync) { return warp_mbar_wait(bar, parity, s_abort, sync); }
 
 // Where a CTA stands and how its group meets.
@@ -116,6 +116,7 @@ __device__ __forceinline__ bool wide_fetch(const WideCta& c, WideFetch& f, const
                                            uint32_t a_bytes, Wait wait) {
   const uint32_t w_bytes = (uint32_t)st.bn * 128u, slot_bytes = 2u * (a_bytes + w_bytes);
   bool ok = true, waited = false;
+#pragma unroll 1
   for (int job = c.rank; job < st.tiles * st.splits && ok; job += c.G) {
     const int tile = job % st.tiles, split = job / st.tiles;
     const int k0 = st.pairs * split / st.splits, n = st.pairs * (split + 1) / st.splits - k0;
@@ -123,14 +124,17 @@ __device__ __forceinline__ bool wide_fetch(const WideCta& c, WideFetch& f, const
     const CUtensorMap* w = second ? mw2 : mw;
     const int n0 = (second ? tile - st.tiles / 2 : tile) * st.bn;
     const int pre = n < st.slots ? n : st.slots;
+#pragma unroll 1
     for (int k = 0; k < pre; ++k) {
       expect_tx_elect(c.full(k), slot_bytes);
       tma_load_3d(c.sbase + k * slot_bytes + 2u * a_bytes, w, c.full(k), 0, n0, 2 * (k0 + k));
       f.fmask ^= 1u << k;
     }
     if (!waited) { ok = wait(); waited = true; }
+#pragma unroll 1
     for (int k = 0; k < pre; ++k) tma_load_3d(c.sbase + k * slot_bytes, ma, c.full(k), 0, m0, 2 * (k0 + k));      // (given up or not: the fill has to land)
     int s = 0;
+#pragma unroll 1
     for (int k = pre; k < n && ok; ++k) {
       ok = wide_wait(c.empty(s), (f.emask >> s) & 1u, c.s_abort, c.sync);
       if (!ok) break;
@@ -141,12 +145,14 @@ __device__ __forceinline__ bool wide_fetch(const WideCta& c, WideFetch& f, const
       tma_load_3d(c.sbase + s * slot_bytes + 2u * a_bytes, w, c.full(s), 0, n0, 2 * (k0 + k));
       if (++s == st.slots) s = 0;
     }
+#pragma unroll 1
     for (int j = 0; j < pre && ok; ++j) {                  // every slot read: the next product lays the ring out anew
       ok = wide_wait(c.empty(j), (f.emask >> j) & 1u, c.s_abort, c.sync);
       if (ok) f.emask ^= 1u << j;
     }
     if (!ok) {
       // gave up: the fills under way have to land before the shared memory goes away (bounded).  fmask holds the parity AFTER the fill.
+#pragma unroll 1
       for (int j = 0; j < pre; ++j) {
         unsigned spins = 0;
         while (!mbar_try_wait(c.full(j), ((f.fmask >> j) & 1u) ^ 1u) && ++spins < (1u << 20)) {}
@@ -161,12 +167,14 @@ struct WideIssue { uint32_t fmask; int jobs; };
 __device__ __forceinline__ bool wide_issue(const WideCta& c, WideIssue& w, const WideStage& st, uint32_t a_bytes, uint32_t tmem) {
   const uint32_t w_bytes = (uint32_t)st.bn * 128u, slot_bytes = 2u * (a_bytes + w_bytes), idesc = make_idesc(st.bn, false);
   bool ok = true;
+#pragma unroll 1
   for (int job = c.rank; job < st.tiles * st.splits && ok; job += c.G) {
     const int split = job / st.tiles;
     const int n = st.pairs * (split + 1) / st.splits - st.pairs * split / st.splits;
     const int buf = w.jobs & 1;
     if (w.jobs >= 2) ok = wide_wait(c.tempty(buf), ((w.jobs >> 1) - 1) & 1, c.s_abort, c.sync);
     int s = 0;
+#pragma unroll 1
     for (int k = 0; k < n && ok; ++k) {
       ok = wide_wait(c.full(s), (w.fmask >> s) & 1u, c.s_abort, c.sync);
       if (!ok) break;
@@ -189,20 +197,26 @@ __device__ __forceinline__ bool wide_issue(const WideCta& c, WideIssue& w, const
 
 // An accumulator block of 32 rows and 32 columns through the warp's staging area: rows belong to lanes in TMEM, and storing them that way
 // touches 32 lines per instruction (the stores of a 128 x 128 fp32 tile took 2.6 us); afterwards eight lanes hold a row, four columns each.
-__device__ __forceinline__ void wide_stage(float* st, uint32_t taddr, int lane) {
+// f is applied to every entry on the way (by the lane of its row, 32 independent entries).
+template <typename F>
+__device__ __forceinline__ void wide_stage(float* st, uint32_t taddr, int lane, F f) {
   uint32_t r[32];
   tc_ld32(taddr, r);
   tc_wait_ld();
   __syncwarp();
 #pragma unroll
-  for (int i = 0; i < 8; ++i) *reinterpret_cast<uint4*>(st + lane * kWStagePitch + 4 * i) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+  for (int i = 0; i < 8; ++i)
+    *reinterpret_cast<float4*>(st + lane * kWStagePitch + 4 * i) =
+        make_float4(f(__uint_as_float(r[4 * i])), f(__uint_as_float(r[4 * i + 1])), f(__uint_as_float(r[4 * i + 2])), f(__uint_as_float(r[4 * i + 3])));
   __syncwarp();
 }
 
 // ---- attention of one (sequence, head) on eight lanes: the row's state (the pre-pass and the tiles before this leaf) and the leaf's keys
-struct WideAttn { float q[8], o[8], m, l, slope; size_t col; };
+struct WideAttn { uint4 q; float o[8], m, l; unsigned col; };      // q in bf16; col: offset of the eight entries within a position's rows [B, d]
 // the keys [ka, kb) of two units, four keys at a time
-__device__ __forceinline__ void wide_attn_keys(WideAttn (&a)[2], const __nv_bfloat16* K, const __nv_bfloat16* V, size_t rstride, int ka, int kb, int t, float scale_log2) {
+__device__ __forceinline__ void wide_attn_keys(WideAttn (&a)[2], const __nv_bfloat16* K, const __nv_bfloat16* V, size_t rstride, int ka, int kb, int t, float scale_log2, const float* alibi, int d) {
+  float slope[2] = {0.f, 0.f};
+  if (alibi) { slope[0] = alibi[a[0].col % d / kHeadDim] * kLog2e; slope[1] = alibi[a[1].col % d / kHeadDim] * kLog2e; }
 #pragma unroll 1
   for (int j0 = ka; j0 < kb; j0 += 4) {
     uint4 kw[2][4], vw[2][4];
@@ -214,15 +228,16 @@ __device__ __forceinline__ void wide_attn_keys(WideAttn (&a)[2], const __nv_bflo
     }
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      float s[4], m_new = a[i].m;
+      float s[4], qf[8], m_new = a[i].m;
+      unpack8(a[i].q, qf);
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         float kf[8], x = 0.f;
         unpack8(kw[i][e], kf);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) x = fmaf(a[i].q[k], kf[k], x);
+        for (int k = 0; k < 8; ++k) x = fmaf(qf[k], kf[k], x);
         x = sum8(x);
-        s[e] = j0 + e < kb ? x * scale_log2 - a[i].slope * (float)(t - (j0 + e)) : -INFINITY;
+        s[e] = j0 + e < kb ? x * scale_log2 - slope[i] * (float)(t - (j0 + e)) : -INFINITY;
         m_new = fmaxf(m_new, s[e]);
       }
       const float corr = exp2f(a[i].m - m_new);
@@ -242,12 +257,12 @@ __device__ __forceinline__ void wide_attn_keys(WideAttn (&a)[2], const __nv_bflo
   }
 }
 // one key whose rows have been fetched
-__device__ __forceinline__ void wide_attn_one(WideAttn& a, const uint4& kw, const uint4& vw, float scale_log2) {
-  float kf[8], vf[8], x = 0.f;
-  unpack8(kw, kf); unpack8(vw, vf);
+__device__ __forceinline__ void wide_attn_one(WideAttn& a, const uint4& kw, const uint4& vw, float scale_log2, float slope) {
+  float kf[8], vf[8], qf[8], x = 0.f;
+  unpack8(kw, kf); unpack8(vw, vf); unpack8(a.q, qf);
 #pragma unroll
-  for (int i = 0; i < 8; ++i) x = fmaf(a.q[i], kf[i], x);
-  const float s = sum8(x) * scale_log2 - a.slope, m_new = fmaxf(a.m, s);
+  for (int i = 0; i < 8; ++i) x = fmaf(qf[i], kf[i], x);
+  const float s = sum8(x) * scale_log2 - slope, m_new = fmaxf(a.m, s);
   const float corr = exp2f(a.m - m_new), pj = exp2f(s - m_new);
   a.m = m_new; a.l = a.l * corr + pj;
 #pragma unroll
@@ -372,73 +387,89 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
     // 1 / rms of this thread's row from the sums of squares that the step before left ([part][B])
     auto row_scale = [&](const float* ssq, int parts, bool on) {
       if (!on || !live) return 1.0f;
-      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+      float sum = 0.f;
       const float* a = ssq + m;
-      int i = 0;
-      for (; i + 4 <= parts; i += 4) {
-        s0 += __ldcg(a + (size_t)i * p.B); s1 += __ldcg(a + (size_t)(i + 1) * p.B); s2 += __ldcg(a + (size_t)(i + 2) * p.B); s3 += __ldcg(a + (size_t)(i + 3) * p.B);
+#pragma unroll 1
+      for (int i0 = 0; i0 < parts; i0 += 16) {
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = i0 + i < parts ? __ldcg(a + (size_t)(i0 + i) * p.B) : 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) sum += v[i];
       }
-      for (; i < parts; ++i) s0 += __ldcg(a + (size_t)i * p.B);
-      return rsqrtf(((s0 + s1) + (s2 + s3)) / (float)d + p.eps);
+      return rsqrtf(sum / (float)d + p.eps);
     };
     float* stage = reinterpret_cast<float*>(c.smem + kWStage + ew * kWStageWarp);
-    // this warp's half of an accumulator of bn columns, f(row of the quadrant, column, values) called by every lane
-    auto blocks = [&](int bn, auto f) {
+    // this warp's half of an accumulator of bn columns, entry(value) by the lane of the row, then f(row of the quadrant, column, values) by every lane
+    auto blocks = [&](int bn, auto entry, auto f) {
 #pragma unroll 1
       for (int cc = half * (bn >> 1); cc < (half + 1) * (bn >> 1); cc += 32) {
-        wide_stage(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane);
-#pragma unroll 2
+        wide_stage(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane, entry);
+#pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int r = 4 * i + (lane >> 3), col = 4 * (lane & 7);
           f(r, cc + col, *reinterpret_cast<const float4*>(stage + r * kWStagePitch + col));
         }
       }
     };
+    // Attention: eight lanes per (sequence, head), two of these at a time per group of lanes.  The state of the row and the leaf's keys but the
+    // newest are taken in while the four products of the position before are under way, a quarter of the keys in front of each.
+    const int units = R * H, unit0 = c.arank * 64 + ew * 8 + (lane >> 3);
+    WideAttn at[2];
+    auto attn_begin = [&](int u0, int t) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int u = u0 + 4 * i < units ? u0 + 4 * i : 0, b = m0 + u / H, h = u % H;
+        const size_t sidx = (size_t)t * p.B + b;
+        at[i].col = (unsigned)(b * d + h * kHeadDim + 8 * (lane & 7));
+        const size_t row = (size_t)t * rstride + at[i].col;
+        at[i].q = *reinterpret_cast<const uint4*>(Q + row);
+        const float4 o0 = *reinterpret_cast<const float4*>(p.st_o + row), o1 = *reinterpret_cast<const float4*>(p.st_o + row + 4);
+        at[i].o[0] = o0.x; at[i].o[1] = o0.y; at[i].o[2] = o0.z; at[i].o[3] = o0.w; at[i].o[4] = o1.x; at[i].o[5] = o1.y; at[i].o[6] = o1.z; at[i].o[7] = o1.w;
+        at[i].m = p.st_m[sidx * H + h]; at[i].l = p.st_l[sidx * H + h];
+      }
+    };
+    const bool attends = c.arank < active_of(F_ATTN);
+    if (attends) attn_begin(unit0, p.t0);
     bool ok = true;
 #pragma unroll 1
     for (int t = p.t0; t < p.t1 && ok; ++t) {
-      if (c.arank < active_of(F_ATTN)) {
-        // eight lanes per (sequence, head), two of these at a time per group of lanes; the keys before the newest were complete a position ago
-        const int units = R * H, per_round = 64 * c.G;
+#pragma unroll 1
+    for (int step = 0; step < F_STEPS; ++step) {
+      if (attends && t + 1 < p.t1 && step != F_ATTN && step != F_Z) {
+        const int product = step < F_Z ? step - 1 : 3, per = ((t - p.t0 + 3) / 4 + 3) / 4 * 4;     // whole batches of four keys
+        if (product == 0) attn_begin(unit0, t + 1);
+        const int ka = p.t0 + product * per, kb = ka + per < t ? ka + per : t;
+        wide_attn_keys(at, Kc, Vc, rstride, ka, kb, t + 1, p.scale_log2, p.alibi, d);
+      }
+      if (step == F_ATTN && attends) {
+        const int per_round = 64 * c.G;
         bool waited = false;
 #pragma unroll 1
-        for (int u0 = c.arank * 64 + ew * 8 + (lane >> 3); u0 - (lane >> 3) < units && ok; u0 += per_round) {
-          WideAttn a[2];
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const int u = u0 + 4 * i < units ? u0 + 4 * i : 0, b = m0 + u / H, h = u % H;
-            const size_t sidx = (size_t)t * p.B + b;
-            a[i].col = (size_t)b * d + h * kHeadDim + 8 * (lane & 7);
-            const size_t at = (size_t)t * rstride + a[i].col;
-            unpack8(*reinterpret_cast<const uint4*>(Q + at), a[i].q);
-            const float4 o0 = *reinterpret_cast<const float4*>(p.st_o + at), o1 = *reinterpret_cast<const float4*>(p.st_o + at + 4);
-            a[i].o[0] = o0.x; a[i].o[1] = o0.y; a[i].o[2] = o0.z; a[i].o[3] = o0.w; a[i].o[4] = o1.x; a[i].o[5] = o1.y; a[i].o[6] = o1.z; a[i].o[7] = o1.w;
-            a[i].m = p.st_m[sidx * H + h]; a[i].l = p.st_l[sidx * H + h];
-            a[i].slope = p.alibi ? p.alibi[h] * kLog2e : 0.f;
-          }
-          wide_attn_keys(a, Kc, Vc, rstride, p.t0, t - 1, t, p.scale_log2);
+        for (int u0 = unit0; u0 - (lane >> 3) < units && ok; u0 += per_round) {
+          if (u0 != unit0) { attn_begin(u0, t); wide_attn_keys(at, Kc, Vc, rstride, p.t0, t - 1, t, p.scale_log2, p.alibi, d); }
           if (!waited) { ok = flag_wait(); waited = true; }
           if (!ok) break;
           if (t > p.t0) {
             uint4 kn[2], vn[2];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) { kn[i] = ldcg16(Kc + (size_t)(t - 1) * rstride + a[i].col); vn[i] = ldcg16(Vc + (size_t)(t - 1) * rstride + a[i].col); }
+            for (int i = 0; i < 2; ++i) { kn[i] = ldcg16(Kc + (size_t)(t - 1) * rstride + at[i].col); vn[i] = ldcg16(Vc + (size_t)(t - 1) * rstride + at[i].col); }
 #pragma unroll
-            for (int i = 0; i < 2; ++i) wide_attn_one(a[i], kn[i], vn[i], p.scale_log2);
+            for (int i = 0; i < 2; ++i) wide_attn_one(at[i], kn[i], vn[i], p.scale_log2, p.alibi ? p.alibi[at[i].col % d / kHeadDim] * kLog2e : 0.f);
           }
 #pragma unroll
           for (int i = 0; i < 2; ++i) {
-            const float il = 1.0f / a[i].l;
+            const float il = 1.0f / at[i].l;
             if (u0 + 4 * i < units)
-              *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.c16) + a[i].col) =
-                  make_uint4(pack2(a[i].o[0] * il, a[i].o[1] * il), pack2(a[i].o[2] * il, a[i].o[3] * il), pack2(a[i].o[4] * il, a[i].o[5] * il), pack2(a[i].o[6] * il, a[i].o[7] * il));
+              *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.c16) + at[i].col) =
+                  make_uint4(pack2(at[i].o[0] * il, at[i].o[1] * il), pack2(at[i].o[2] * il, at[i].o[3] * il), pack2(at[i].o[4] * il, at[i].o[5] * il), pack2(at[i].o[6] * il, at[i].o[7] * il));
           }
         }
         if (!waited) ok = flag_wait();                         // (a warp without units)
         ok = finish(ok, F_ATTN);
         if (!ok) break;
       }
-      if (c.rank < active_of(F_OUT)) {
+      if (step == F_OUT && c.rank < active_of(F_OUT)) {
         // h = x + alpha c W_o;  u = bf16(h g), sums of squares of h
         bool good = flag_wait();
         const int bn = p.st[0].bn;
@@ -465,7 +496,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
               const uint2 gw = *reinterpret_cast<const uint2*>(g_mlp + n);
               g0 = __uint_as_float(gw.x << 16); g1 = __uint_as_float(gw.x & 0xffff0000u); g2 = __uint_as_float(gw.y << 16); g3 = __uint_as_float(gw.y & 0xffff0000u);
             }
-            wide_stage(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane);
+            wide_stage(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane, [](float v) { return v; });
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
               const int r = 4 * i + (lane >> 3);
@@ -491,7 +522,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
         ok = finish(good, F_OUT);
         if (!ok) break;
       }
-      if (c.rank < active_of(F_UP)) {
+      if (step == F_UP && c.rank < active_of(F_UP)) {
         // g = GELU(u W_up / rms(h))
         bool good = flag_wait();
         const float inv = good ? row_scale(p.ssq_h, p.st[0].tiles * 2, pre) : 1.f;
@@ -499,18 +530,16 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
 #pragma unroll 1
         for (int job = c.rank; job < p.st[1].tiles; job += c.G) {
           if (!good || !(good = acc_wait())) break;
-          blocks(bn, [&](int r, int col, const float4& a) {
-            const float sc = __shfl_sync(0xffffffffu, inv, r);
-            const float g0 = gelu_wide(a.x * sc), g1 = gelu_wide(a.y * sc), g2 = gelu_wide(a.z * sc), g3 = gelu_wide(a.w * sc);
+          blocks(bn, [&](float v) { return gelu_wide(v * inv); }, [&](int r, int col, const float4& a) {
             if (quad * 32 + r < R)
-              *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.g16) + (size_t)(m0 + quad * 32 + r) * p.dff + job * bn + col) = make_uint2(pack2(g0, g1), pack2(g2, g3));
+              *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.g16) + (size_t)(m0 + quad * 32 + r) * p.dff + job * bn + col) = make_uint2(pack2(a.x, a.y), pack2(a.z, a.w));
           });
           acc_done();
         }
         ok = finish(good, F_UP);
         if (!ok) break;
       }
-      if (c.rank < active_of(F_DOWN)) {
+      if (step == F_DOWN && c.rank < active_of(F_DOWN)) {
         // a part of g W_down
         bool good = flag_wait();
         const int bn = p.st[2].bn;
@@ -518,7 +547,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
         for (int job = c.rank; job < p.st[2].tiles * p.st[2].splits; job += c.G) {
           const int n0 = (job % p.st[2].tiles) * bn, split = job / p.st[2].tiles;
           if (!good || !(good = acc_wait())) break;
-          blocks(bn, [&](int r, int col, const float4& a) {
+          blocks(bn, [](float v) { return v; }, [&](int r, int col, const float4& a) {
             if (quad * 32 + r < R) *reinterpret_cast<float4*>(p.partial + ((size_t)split * p.B + m0 + quad * 32 + r) * d + n0 + col) = a;
           });
           acc_done();
@@ -526,60 +555,67 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
         ok = finish(good, F_DOWN);
         if (!ok) break;
       }
-      if (c.rank < active_of(F_Z)) {
+      if (step == F_Z && c.rank < active_of(F_Z)) {
         // z = h + alpha g W_down;  r = bf16(z g), sums of squares of z: a warp per row and 128 columns
-        constexpr int kRows = 2;                               // fetched together
-        const int total = R * chunks, step = c.G * 8;
-        auto at_of = [&](int u) { return (size_t)(m0 + u / chunks) * d + (u % chunks) * 128 + 4 * lane; };
-        float4 hv[kRows];
-        auto fetch_h = [&](int u0) {
-#pragma unroll
-          for (int k = 0; k < kRows; ++k) { const int u = u0 + k * step; hv[k] = __ldcg(reinterpret_cast<const float4*>(p.h + at_of(u < total ? u : 0))); }
-        };
+        const int total = R * chunks, stride = c.G * 8, splits = p.st[2].splits;
         const bool ahead = c.rank < active_of(F_UP) || c.rank < active_of(F_DOWN);      // such a CTA has seen that h is complete
-        if (ahead) fetch_h(c.rank * 8 + ew);
-        const bool good = flag_wait();
-        if (good) {
+        bool good = true, waited = false;
+        // ROWS units with PER parts each are fetched together
+        auto units_of = [&](auto rows, auto per) {
+          constexpr int kRows = decltype(rows)::value, kPer = decltype(per)::value;
 #pragma unroll 1
-          for (int u0 = c.rank * 8 + ew; u0 < total; u0 += kRows * step) {
-            if (!ahead || u0 != c.rank * 8 + ew) fetch_h(u0);
-            float4 pv[kRows][8];
+          for (int u0 = c.rank * 8 + ew; u0 < total; u0 += kRows * stride) {
+            int b[kRows], col[kRows];
+            float4 hv[kRows], pv[kRows][kPer];
 #pragma unroll
             for (int k = 0; k < kRows; ++k) {
-              const int u = u0 + k * step;
-              const size_t at = at_of(u < total ? u : 0);
+              const int u = u0 + k * stride < total ? u0 + k * stride : u0;
+              b[k] = m0 + u / chunks; col[k] = (u % chunks) * 128 + 4 * lane;
+            }
+            auto fetch_h = [&]() {
 #pragma unroll
-              for (int z = 0; z < 8; ++z)
-                if (z < p.st[2].splits) pv[k][z] = __ldcg(reinterpret_cast<const float4*>(p.partial + (size_t)z * p.B * d + at));
+              for (int k = 0; k < kRows; ++k) hv[k] = __ldcg(reinterpret_cast<const float4*>(p.h + (size_t)b[k] * d + col[k]));
+            };
+            if (ahead || waited) fetch_h();
+            if (!waited) {
+              good = flag_wait();
+              waited = true;
+              if (!good) break;
+              if (!ahead) fetch_h();
             }
 #pragma unroll
+            for (int k = 0; k < kRows; ++k)
+#pragma unroll
+              for (int z = 0; z < kPer; ++z) pv[k][z] = __ldcg(reinterpret_cast<const float4*>(p.partial + ((size_t)(z < splits ? z : 0) * p.B + b[k]) * d + col[k]));
+#pragma unroll
             for (int k = 0; k < kRows; ++k) {
-              const int u = u0 + k * step;
-              if (u >= total) break;
-              const int b = m0 + u / chunks, ch = u % chunks, col = ch * 128 + 4 * lane;
+              if (u0 + k * stride >= total) break;
               float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-              for (int z = 0; z < 8; ++z)
-                if (z < p.st[2].splits) { acc.x += pv[k][z].x; acc.y += pv[k][z].y; acc.z += pv[k][z].z; acc.w += pv[k][z].w; }
+              for (int z = 0; z < kPer; ++z)
+                if (z < splits) { acc.x += pv[k][z].x; acc.y += pv[k][z].y; acc.z += pv[k][z].z; acc.w += pv[k][z].w; }
               float v[4] = {hv[k].x + p.alpha * acc.x, hv[k].y + p.alpha * acc.y, hv[k].z + p.alpha * acc.z, hv[k].w + p.alpha * acc.w};
               float ss = 0.f;
 #pragma unroll
               for (int i = 0; i < 4; ++i) { v[i] = round_T<__nv_bfloat16>(v[i]); ss = fmaf(v[i], v[i], ss); }    // the pair comes from the stored (rounded) z
-              *reinterpret_cast<uint2*>(Z + (size_t)b * p.z_bs + (size_t)t * p.z_ts + col) = make_uint2(pack2(v[0], v[1]), pack2(v[2], v[3]));
+              *reinterpret_cast<uint2*>(Z + (size_t)b[k] * p.z_bs + (size_t)t * p.z_ts + col[k]) = make_uint2(pack2(v[0], v[1]), pack2(v[2], v[3]));
               ss = warp_sum(ss);
-              if (lane == 0) p.ssq_z[(size_t)ch * p.B + b] = ss;
+              if (lane == 0) p.ssq_z[(size_t)(col[k] >> 7) * p.B + b[k]] = ss;
               if (znorm && g_kv) {
-                const uint2 gw = *reinterpret_cast<const uint2*>(g_kv + col);
+                const uint2 gw = *reinterpret_cast<const uint2*>(g_kv + col[k]);
                 v[0] *= __uint_as_float(gw.x << 16); v[1] *= __uint_as_float(gw.x & 0xffff0000u); v[2] *= __uint_as_float(gw.y << 16); v[3] *= __uint_as_float(gw.y & 0xffff0000u);
               }
-              *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.r16) + (size_t)b * d + col) = make_uint2(pack2(v[0], v[1]), pack2(v[2], v[3]));
+              *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.r16) + (size_t)b[k] * d + col[k]) = make_uint2(pack2(v[0], v[1]), pack2(v[2], v[3]));
             }
           }
-        }
+        };
+        if (splits > 4) units_of(std::integral_constant<int, 1>(), std::integral_constant<int, 8>());
+        else units_of(std::integral_constant<int, 2>(), std::integral_constant<int, 4>());
+        if (!waited) good = flag_wait();                       // (a warp without units)
         ok = finish(good, F_Z);
         if (!ok) break;
       }
-      if (c.rank < active_of(F_KV)) {
+      if (step == F_KV && c.rank < active_of(F_KV)) {
         // k = qkRMS(r W_k / rms(z)), v = r W_v / rms(z): a tile is one head
         bool good = flag_wait();
         const float inv = good ? row_scale(p.ssq_z, chunks, znorm) : 1.f;
@@ -626,6 +662,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
         }
         ok = finish(good, F_KV);
       }
+    }
     }
   }
   tc_fence_before();
