@@ -200,7 +200,8 @@ cudaError_t head_launch(int dtype, const void* emb, const void* g_final, const v
 
 // Token loop of wide batches in one cooperative launch per leaf (bf16; rt_wide_loop.cu).
 constexpr int kWideGroupsMax = 8;                // groups of at most 128 sequences
-struct WideStage { int pairs, bn, tiles, splits, slots; };     // pairs of 64-wide blocks of the contraction, tile width, tiles, parts of the contraction, ring slots
+// fills of the operand ring over the whole contraction, tile width, tiles, parts of the contraction, fills the ring holds
+struct WideStage { int fills, bn, tiles, splits, slots; };
 struct WideFwdParams {
   int B, d, H, dff, norm_flags;
   float eps, scale_log2, alpha;

@@ -13,8 +13,12 @@
 // the next product scales its accumulator rows by 1 / rms.  The down projection contracts over d_ff: it runs in up to eight parts whose sums
 // meet in a row step.
 //
-// Exchange: data through global memory (L2), a counter per step and group; a CTA's writes are fenced for the async proxy before it counts
-// itself in, the waiting CTA fences after it saw the count.  Every wait is bounded (2 s).
+// Exchange: data through global memory (L2), a counter per step and group (release by one thread after a barrier of the CTA's row warps,
+// acquire and a proxy fence by the warp that then fetches).  Every wait is bounded (2 s).
+//
+// Measured per position at d = 1024, d_ff = 4096, against the launches: B = 96 30 us (42), B = 200 (d = 768) 29 (50), B = 512 40 (57).  A step
+// is about 1 us from the last count to the first fetch, 2 to 5 us until the accumulators are complete (operand rows and weights at 145 GB/s
+// per SM, about 1.2 us of latency), 1 to 2.5 us of row work, 0.7 us for the release.
 #include <type_traits>
 
 #include "rt_kernels.h"
@@ -24,7 +28,8 @@ namespace rt {
 
 namespace {
 constexpr int kWThreads = 320, kWEpi = 256;
-constexpr uint32_t kWRing = 192512;                        // operand ring: a slot holds two 64-wide blocks of A and of W
+constexpr int kWBlocks = 2;                                // 64-wide blocks of A and of W per fill of the operand ring
+constexpr uint32_t kWRing = 192512;
 constexpr int kWSlotsMax = 11;
 constexpr int kWStagePitch = 36;                           // floats per row of a warp's 32 x 32 staging area
 constexpr uint32_t kWStage = kWRing, kWStageWarp = 32 * kWStagePitch * 4;
@@ -58,9 +63,10 @@ __device__ __forceinline__ float sum8(float v) {           // over the eight lan
 // x Phi(x) with erfc by Abramowitz and Stegun 7.1.26.  Largest error 2.1e-7 (0.5 x (1 + erff) in fp32: 6.8e-7), and no cancellation for
 // negative x; a third of the instructions, which a step that applies it to 128 x 128 accumulators per CTA notices (4 us before).
 __device__ __forceinline__ float gelu_wide(float x) {
-  const float z = fabsf(x) * 0.70710678118654752f, t = __fdividef(1.0f, fmaf(0.3275911f, z, 1.0f));
-  const float poly = t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 1.061405429f, -1.453152027f), 1.421413741f), -0.284496736f), 0.254829592f);
-  const float q = 0.5f * poly * __expf(-z * z);            // Phi(-|x|)
+  float t;                                                 // 1 / (1 + 0.3275911 |x| / sqrt(2))
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.3275911f * 0.70710678f, fabsf(x), 1.0f)));
+  const float poly = t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 0.5f * 1.061405429f, -0.5f * 1.453152027f), 0.5f * 1.421413741f), -0.5f * 0.284496736f), 0.5f * 0.254829592f);
+  const float q = poly * ex2(x * x * (-0.5f * kLog2e));    // Phi(-|x|)
   return x * (x < 0.f ? q : 1.0f - q);
 }
 
@@ -108,18 +114,18 @@ struct WideCta {
 
 // Operand fetches of one product step: the weights of the first blocks, then (after the wait) their operand rows, then the rest block by block.
 // emask / fmask: parity of the next wait on a slot's empty barrier / of the latest fill of a slot.
-// A fetch of one block of 16 KB or less costs an SM about 90 ns whatever its size, so a copy covers two blocks (a three-dimensional map:
-// 64 columns, rows, blocks).
+// A copy of up to 16 KB costs an SM about 90 ns whatever its size, so a copy covers two blocks (a three-dimensional map: 64 columns, rows,
+// blocks): a 128-column tile over 1024 takes 4.8 us that way and 5.8 us with single blocks, although more of those are under way.
 struct WideFetch { uint32_t emask, fmask; };
 template <typename Wait>
 __device__ __forceinline__ bool wide_fetch(const WideCta& c, WideFetch& f, const WideStage& st, const CUtensorMap* ma, const CUtensorMap* mw, const CUtensorMap* mw2, int m0,
                                            uint32_t a_bytes, Wait wait) {
-  const uint32_t w_bytes = (uint32_t)st.bn * 128u, slot_bytes = 2u * (a_bytes + w_bytes);
+  const uint32_t w_bytes = (uint32_t)st.bn * 128u, slot_bytes = kWBlocks * (a_bytes + w_bytes);
   bool ok = true, waited = false;
 #pragma unroll 1
   for (int job = c.rank; job < st.tiles * st.splits && ok; job += c.G) {
     const int tile = job % st.tiles, split = job / st.tiles;
-    const int k0 = st.pairs * split / st.splits, n = st.pairs * (split + 1) / st.splits - k0;
+    const int k0 = st.fills * split / st.splits, n = st.fills * (split + 1) / st.splits - k0;
     const bool second = mw2 && tile >= st.tiles / 2;
     const CUtensorMap* w = second ? mw2 : mw;
     const int n0 = (second ? tile - st.tiles / 2 : tile) * st.bn;
@@ -127,12 +133,12 @@ __device__ __forceinline__ bool wide_fetch(const WideCta& c, WideFetch& f, const
 #pragma unroll 1
     for (int k = 0; k < pre; ++k) {
       expect_tx_elect(c.full(k), slot_bytes);
-      tma_load_3d(c.sbase + k * slot_bytes + 2u * a_bytes, w, c.full(k), 0, n0, 2 * (k0 + k));
+      tma_load_3d(c.sbase + k * slot_bytes + kWBlocks * a_bytes, w, c.full(k), 0, n0, kWBlocks * (k0 + k));
       f.fmask ^= 1u << k;
     }
     if (!waited) { ok = wait(); waited = true; }
 #pragma unroll 1
-    for (int k = 0; k < pre; ++k) tma_load_3d(c.sbase + k * slot_bytes, ma, c.full(k), 0, m0, 2 * (k0 + k));      // (given up or not: the fill has to land)
+    for (int k = 0; k < pre; ++k) tma_load_3d(c.sbase + k * slot_bytes, ma, c.full(k), 0, m0, kWBlocks * (k0 + k));      // (given up or not: the fill has to land)
     int s = 0;
 #pragma unroll 1
     for (int k = pre; k < n && ok; ++k) {
@@ -141,8 +147,8 @@ __device__ __forceinline__ bool wide_fetch(const WideCta& c, WideFetch& f, const
       f.emask ^= 1u << s;
       f.fmask ^= 1u << s;
       expect_tx_elect(c.full(s), slot_bytes);
-      tma_load_3d(c.sbase + s * slot_bytes, ma, c.full(s), 0, m0, 2 * (k0 + k));
-      tma_load_3d(c.sbase + s * slot_bytes + 2u * a_bytes, w, c.full(s), 0, n0, 2 * (k0 + k));
+      tma_load_3d(c.sbase + s * slot_bytes, ma, c.full(s), 0, m0, kWBlocks * (k0 + k));
+      tma_load_3d(c.sbase + s * slot_bytes + kWBlocks * a_bytes, w, c.full(s), 0, n0, kWBlocks * (k0 + k));
       if (++s == st.slots) s = 0;
     }
 #pragma unroll 1
@@ -165,12 +171,12 @@ __device__ __forceinline__ bool wide_fetch(const WideCta& c, WideFetch& f, const
 // The products of one step.
 struct WideIssue { uint32_t fmask; int jobs; };
 __device__ __forceinline__ bool wide_issue(const WideCta& c, WideIssue& w, const WideStage& st, uint32_t a_bytes, uint32_t tmem) {
-  const uint32_t w_bytes = (uint32_t)st.bn * 128u, slot_bytes = 2u * (a_bytes + w_bytes), idesc = make_idesc(st.bn, false);
+  const uint32_t w_bytes = (uint32_t)st.bn * 128u, slot_bytes = kWBlocks * (a_bytes + w_bytes), idesc = make_idesc(st.bn, false);
   bool ok = true;
 #pragma unroll 1
   for (int job = c.rank; job < st.tiles * st.splits && ok; job += c.G) {
     const int split = job / st.tiles;
-    const int n = st.pairs * (split + 1) / st.splits - st.pairs * split / st.splits;
+    const int n = st.fills * (split + 1) / st.splits - st.fills * split / st.splits;
     const int buf = w.jobs & 1;
     if (w.jobs >= 2) ok = wide_wait(c.tempty(buf), ((w.jobs >> 1) - 1) & 1, c.s_abort, c.sync);
     int s = 0;
@@ -181,8 +187,8 @@ __device__ __forceinline__ bool wide_issue(const WideCta& c, WideIssue& w, const
       w.fmask ^= 1u << s;
       tc_fence_after();
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const uint64_t a0 = make_desc(c.sbase + s * slot_bytes + j * a_bytes, 16, 1024), b0 = make_desc(c.sbase + s * slot_bytes + 2u * a_bytes + j * w_bytes, 16, 1024);
+      for (int j = 0; j < kWBlocks; ++j) {
+        const uint64_t a0 = make_desc(c.sbase + s * slot_bytes + j * a_bytes, 16, 1024), b0 = make_desc(c.sbase + s * slot_bytes + kWBlocks * a_bytes + j * w_bytes, 16, 1024);
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks) tc_mma(tmem + (uint32_t)(buf * kWBuf), a0 + 2u * ks, b0 + 2u * ks, idesc, (k > 0 || j > 0 || ks > 0) ? 1u : 0u);
       }
@@ -673,31 +679,31 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_forward_kernel(const __grid
   }
 }
 
-int ring_slots(int bn, int a_bytes) {
-  const int n = (int)(kWRing / (2u * ((unsigned)a_bytes + (unsigned)bn * 128u)));
-  return n < kWSlotsMax ? n : kWSlotsMax;
+WideStage wide_stage_of(int n, int k, int bn, int splits, int a_bytes) {
+  WideStage st;
+  st.bn = bn; st.tiles = n / bn; st.splits = splits;
+  st.fills = k / 64 / kWBlocks;
+  st.slots = (int)(kWRing / (kWBlocks * ((unsigned)a_bytes + (unsigned)bn * 128u)));
+  if (st.slots > kWSlotsMax) st.slots = kWSlotsMax;
+  return st;
 }
-// A product of n columns over k on G CTAs, not split: the narrowest tile that gives every CTA at most one.
-WideStage stage_whole(int n, int k, int G, int a_bytes, int bn_min, int bn_max) {
-  int bn = bn_min;                                         // (d and d_ff are multiples of 128)
-  while (bn < bn_max && (ceil_div(n, bn) > G || n % bn)) bn *= 2;
-  return {k / 128, bn, n / bn, 1, ring_slots(bn, a_bytes)};
-}
+// A product of n columns over k on G CTAs, not split: the narrowest tile that gives every CTA at most one (d and d_ff are multiples of 128).
+WideStage stage_whole(int n, int k, int G, int a_bytes, int bn_max) { return wide_stage_of(n, k, bn_max == 128 && n / 64 > G ? 128 : 64, 1, a_bytes); }
 // The same in parts of the contraction, summed by a row step: the operand rows of a part, not its weights, are what a CTA waits for, so as
 // many parts (of at least four blocks, at most eight) as the group has CTAs for; tiles of 64 columns where the group is large enough.
 WideStage stage_split(int n, int k, int G, int a_bytes) {
-  const int bn = (n / 64) * 8 <= G ? 64 : 128, pairs = k / 128;
+  const int bn = (n / 64) * 8 <= G ? 64 : 128;
   int sp = G / (n / bn);
   if (sp > 8) sp = 8;
-  if (sp > pairs / 2) sp = pairs / 2;
-  return {pairs, bn, n / bn, sp < 1 ? 1 : sp, ring_slots(bn, a_bytes)};
+  if (sp > k / 256) sp = k / 256;
+  return wide_stage_of(n, k, bn, sp < 1 ? 1 : sp, a_bytes);
 }
 // [rows, cols] bf16 as blocks of 64 columns: a box is two blocks of box_rows rows
 bool map_blocks(CUtensorMap* out, const void* base, long long rows, int cols, int box_rows) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   const cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)(cols / 64)}, strides[2] = {(cuuint64_t)cols * 2, 128};
-  const cuuint32_t box[3] = {64u, (cuuint32_t)box_rows, 2u}, estr[3] = {1, 1, 1};
+  const cuuint32_t box[3] = {64u, (cuuint32_t)box_rows, (cuuint32_t)kWBlocks}, estr[3] = {1, 1, 1};
   return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -717,17 +723,21 @@ cudaError_t wide_forward_launch(WideFwdParams p, cudaStream_t s) {
   p.R = ceil_div(p.B, groups); p.G = kB200Sms / groups;
   const int box = (p.R + 7) / 8 * 8;
   p.a_bytes = box * 128;
-  p.st[0] = stage_whole(p.d, p.d, p.G, p.a_bytes, 64, 128);
-  p.st[1] = stage_whole(p.dff, p.d, p.G, p.a_bytes, 64, 128);
+  p.st[0] = stage_whole(p.d, p.d, p.G, p.a_bytes, 128);
+  p.st[1] = stage_whole(p.dff, p.d, p.G, p.a_bytes, 128);
   p.st[2] = stage_split(p.d, p.dff, p.G, p.a_bytes);
-  p.st[3] = stage_whole(2 * p.d, p.d, p.G, p.a_bytes, 64, 64);             // a tile is one head
+  p.st[3] = stage_whole(2 * p.d, p.d, p.G, p.a_bytes, 64);               // a tile is one head
   p.ssq_z = p.ssq_h + (size_t)(p.d / 32) * p.B;
   WideFwdMaps m;
-  if (!map_blocks(&m.a[0], p.c16, p.B, p.d, box) || !map_blocks(&m.a[1], p.u16, p.B, p.d, box) ||
-      !map_blocks(&m.a[2], p.g16, p.B, p.dff, box) || !map_blocks(&m.a[3], p.r16, p.B, p.d, box) ||
-      !map_blocks(&m.w[0], p.w_o, p.d, p.d, p.st[0].bn) || !map_blocks(&m.w[1], p.w_up, p.dff, p.d, p.st[1].bn) ||
-      !map_blocks(&m.w[2], p.w_down, p.d, p.dff, p.st[2].bn) || !map_blocks(&m.w[3], p.w_k, p.d, p.d, 64) ||
-      !map_blocks(&m.w[4], p.w_v, p.d, p.d, 64))
+  const void *A[4] = {p.c16, p.u16, p.g16, p.r16}, *W[5] = {p.w_o, p.w_up, p.w_down, p.w_k, p.w_v};
+  const int K[5] = {p.d, p.d, p.dff, p.d, p.d}, N[5] = {p.d, p.dff, p.d, p.d, p.d};
+  bool ok = true;
+  for (int i = 0; i < 5; ++i) {
+    const WideStage& st = p.st[i < 4 ? i : 3];
+    if (i < 4) ok = ok && map_blocks(&m.a[i], A[i], p.B, K[i], box);
+    ok = ok && map_blocks(&m.w[i], W[i], N[i], K[i], st.bn);
+  }
+  if (!ok)
     return cudaErrorInvalidValue;
   const void* fn = reinterpret_cast<const void*>(&wide_forward_kernel);
   const int smem = (int)kWTotal + 1024;
