@@ -14,6 +14,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include "rt_bwd.cuh"
 #include "rt_common.cuh"
 #include "rt_kernels.h"
 
@@ -254,41 +255,9 @@ __global__ void gelu_kernel(const float* __restrict__ a, float* __restrict__ out
 }
 
 // ------------------------------------------------------------------------------------------------ attention
-struct AttnBufs {
-  const float *q, *k, *v, *kt, *vt;        // position-major [rows, d]
-  float *lse, *D;                          // [rows, H]: log2-sum-exp of the logits (log2 units), <dc, c> per head
-  float *c;                                // [rows, d] attention value
-  const float* dc;                         // [rows, d] gradient of the attention value
-  float *dK, *dV, *dkt, *dvt, *dq;
-  const float* alibi;                      // [H] or NULL
-  float scale, scale_log2;
-  int B, H, d, N;
-};
-
 // ---- eight lanes per (query, key) pair -------------------------------------------------------------------------------
 // The three all-pairs kernels below split a warp into four groups of eight lanes; a group works on one pair at a time,
 // each lane holding eight consecutive entries of the 64-wide head, so a dot product costs three shuffles for four pairs.
-struct F8 { float v[8]; };
-__device__ __forceinline__ F8 ld8(const float* p) {
-  const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
-  return F8{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
-}
-__device__ __forceinline__ void st8(float* p, const F8& x) {
-  *reinterpret_cast<float4*>(p) = make_float4(x.v[0], x.v[1], x.v[2], x.v[3]);
-  *reinterpret_cast<float4*>(p + 4) = make_float4(x.v[4], x.v[5], x.v[6], x.v[7]);
-}
-__device__ __forceinline__ float dot8(const F8& a, const F8& b) {
-  float s = 0.f;
-#pragma unroll
-  for (int e = 0; e < 8; ++e) s = fmaf(a.v[e], b.v[e], s);
-  return s;
-}
-__device__ __forceinline__ float group_sum(float v) {          // over the eight lanes of a group
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
-  v += __shfl_xor_sync(0xffffffffu, v, 2);
-  v += __shfl_xor_sync(0xffffffffu, v, 4);
-  return v;
-}
 __device__ __forceinline__ float across_groups_sum(float v) {   // over the four groups, lane by lane
   v += __shfl_xor_sync(0xffffffffu, v, 8);
   v += __shfl_xor_sync(0xffffffffu, v, 16);
@@ -485,32 +454,6 @@ __global__ void attn_self_wide_kernel(AttnBufs a, int i, int k0) {
 // does at these sizes, so the sums of split products, the norm backwards and the operand copies live in the kernels that need them
 // anyway: 15 launches and 73 us per position at B = 96, d = 1024 before.
 
-// qkRMS backward of dk of one (position, sequence, head) and the bf16 operand row [dk_raw | dv] of the next product; a group of eight
-// lanes, eight entries each.
-__device__ __forceinline__ void pair_operand(const F8& dk, const F8& dv, const F8& u, const __nv_bfloat16* g_k, int h, int t, float eps, int qk, float* dkraw,
-                                             __nv_bfloat16* op_k, __nv_bfloat16* op_v) {
-  F8 r = dk;
-  if (qk) {
-    F8 ty;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) ty.v[e] = dk.v[e] * gain_at(g_k, h * kHeadDim + 8 * t + e);
-    const float ss = group_sum(dot8(u, u)), tu = group_sum(dot8(ty, u));
-    const float inv = rsqrtf(ss / kHeadDim + eps), mean = tu * inv / kHeadDim;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) r.v[e] = inv * (ty.v[e] - u.v[e] * inv * mean);
-  }
-  st8(dkraw, r);
-  unsigned a[4], b[4];
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const __nv_bfloat162 x = __floats2bfloat162_rn(r.v[2 * e], r.v[2 * e + 1]), y = __floats2bfloat162_rn(dv.v[2 * e], dv.v[2 * e + 1]);
-    a[e] = *reinterpret_cast<const unsigned*>(&x); b[e] = *reinterpret_cast<const unsigned*>(&y);
-  }
-  *reinterpret_cast<uint4*>(op_k) = make_uint4(a[0], a[1], a[2], a[3]);
-  *reinterpret_cast<uint4*>(op_v) = make_uint4(b[0], b[1], b[2], b[3]);
-}
-struct WidePair { const float* kraw; float* dkraw; const __nv_bfloat16* g_k; __nv_bfloat16* op; float eps; int qk; };      // op [B][2 d]
-
 // The operand of position i when nothing of its leaf has to be added first (the last position of a leaf): one warp per four (sequence, head).
 __global__ void wide_pair_kernel(AttnBufs a, WidePair w, int i) {
   grid_dep_sync();
@@ -522,7 +465,7 @@ __global__ void wide_pair_kernel(AttnBufs a, WidePair w, int i) {
   const long long at = ((long long)i * a.B + b) * a.d + (long long)h * kHeadDim + 8 * t;
   const F8 dk = ld8(a.dK + at), dv = ld8(a.dV + at), kr = ld8(w.kraw + at);
   __nv_bfloat16* op = w.op + (long long)b * 2 * a.d + h * kHeadDim + 8 * t;
-  if (live) pair_operand(dk, dv, kr, w.g_k, h, t, w.eps, w.qk, w.dkraw + at, op, op + a.d);
+  pair_operand(dk, dv, kr, w.g_k, h, t, w.eps, w.qk, w.dkraw + at, op, op + a.d, live);
 }
 
 // out = add + RMS backward of the row sum of `splits` partial products through RMS(u); keeps the sum, leaves scale * out in bf16 as the
@@ -620,7 +563,7 @@ __global__ void wide_attn_kernel(AttnBufs a, WidePair w, const float* __restrict
         const F8 kr = ld8(w.kraw + rj);
         __nv_bfloat16* op = w.op + (long long)b * 2 * a.d + col;
         // (all groups hold the same values; each writes them)
-        pair_operand(gk, gv, kr, w.g_k, h, t, w.eps, w.qk, w.dkraw + rj, op, op + a.d);
+        pair_operand(gk, gv, kr, w.g_k, h, t, w.eps, w.qk, w.dkraw + rj, op, op + a.d, true);
       }
     }
   }
@@ -1289,6 +1232,7 @@ __global__ void __launch_bounds__(kRmThreads, 1) bwd_loop_kernel(RowmatParams p,
 // ------------------------------------------------------------------------------------------------ workspace
 struct BwdLayout {
   size_t sync, n, qraw, ktraw, vt, q, kt, r, kraw, k, v, c, h, u, act, gl, lse, D;
+  size_t wctr;
   size_t dK, dV, dkraw, dr, Gz, dpre, du, dh, dc, dq, dkt, dvt, dn, gprod, part, part2, sa, sb, wt, wt5, dzp, qkv16, dvf;
   size_t zero_begin, zero_end, total;
 };
@@ -1328,6 +1272,8 @@ BwdLayout bwd_layout(const rt_config* c, int B, int N) {
   L.wt5 = take((3 * d * d + 2 * d * f) / 2 + 64); L.dzp = wide && !tc ? take(rows * d) : o;
   // bf16 operands of the tensor-core products (bf16 storage): two [rows, max(d, d_ff)] arrays and one [d, d]
   const size_t rows_k = align_up(rows, 64);
+  L.wctr = wide && tc ? take(wide_counter_bytes(B) / 4) : o;
+  if (wide && tc && N < 8) L.gprod = take((size_t)8 * B * d);    // parts of split products
   size_t sb_elems = rows_k * (d > f ? d : f);
   if (wide && sb_elems < (2 * d + f) * B + 64) sb_elems = (2 * d + f) * B + 64;     // the operands of one position side by side
   L.sa = take(rows_k * (d > f ? d : f) / 2 + 64); L.sb = take(sb_elems / 2 + 64); L.wt = take(d * d / 2 + 64);
@@ -1639,6 +1585,19 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
     RT_TRY(launch_chained(wide_attn_kernel, dim3(warps_grid((long long)B * H)), dim3(tpb), 0, s, true, ab, wp, part, sp, i, s0));
     return RT_OK;
   };
+  // one launch per leaf where the shape allows (rt_wide_backward.cu)
+  const bool wide_loop = wide_tc && wide_backward_groups(B, d, f) > 0;
+  WideBwdParams wl;
+  memset(&wl, 0, sizeof(wl));
+  if (wide_loop) {
+    wl.B = B; wl.d = d; wl.H = H; wl.dff = f; wl.z_norm = z_norm ? 1 : 0; wl.pre = pre ? 1 : 0; wl.eps = eps; wl.alpha = alpha;
+    wl.wkvT = WkT; wl.wdnT = WdnT; wl.wupT = WupT; wl.woT = WoT; wl.g_kv = g_kv; wl.g_mlp = g_mlp;
+    wl.z = z; wl.z_bs = xbs; wl.z_ts = xts; wl.dz = dz; wl.dz_bs = xbs; wl.dz_ts = xts; wl.h = F(L.h); wl.act = F(L.act);
+    wl.dr = F(L.dr); wl.Gz = F(L.Gz); wl.dpre = F(L.dpre); wl.du = F(L.du); wl.dh = F(L.dh); wl.dc = F(L.dc);
+    wl.partial = F(L.gprod); wl.s16 = SA; wl.p16 = SC; wl.counters = reinterpret_cast<unsigned*>(ws + L.wctr); wl.sync = sync;
+    RT_TRY(cudaMemsetAsync(wl.counters, 0, wide_counter_bytes(B), s));
+  }
+  unsigned wide_steps = 0;
   RT_TRY(cudaFuncSetAttribute(attn_bwd_kv_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairBlockSmem));
   for (int s0 = ((N - 1) / Lf) * Lf; s0 >= 0; s0 -= Lf) {
     const int e0 = s0 + Lf < N ? s0 + Lf : N;
@@ -1660,6 +1619,13 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
         bl.s0 = s0; bl.e0 = e0; bl.b0 = b0; bl.B = B - b0 < fast ? B - b0 : fast;
         RT_TRY(bwd_leaf_launch(bl, s));
       }
+      continue;
+    }
+    if (wide_loop) {
+      RT_TRY(launch_chained(wide_pair_kernel, dim3((unsigned)(((long long)B * H * 8 + tpb - 1) / tpb)), dim3(tpb), 0, s, true, ab, wp, e0 - 1));
+      wl.s0 = s0; wl.e0 = e0; wl.steps = wide_steps;
+      RT_TRY(wide_backward_launch(wl, ab, wp, s));
+      wide_steps += (unsigned)(e0 - s0);
       continue;
     }
     if (wide) {

@@ -221,6 +221,28 @@ struct WideFwdParams {
   int R, G, a_bytes;                             // set by the launcher: sequences and SMs per group, bytes of an operand block
   WideStage st[4];                               // W_o, W_up, W_down, W_k | W_v
 };
+struct AttnBufs;
+struct WidePair;
+struct WideBwdParams {
+  int B, d, H, dff, z_norm, pre;
+  float eps, alpha;
+  const void *wkvT, *wdnT, *wupT, *woT;          // bf16 [d, 2 d], [d_ff, d], [d, d_ff], [d, d]
+  const void *g_kv, *g_mlp;
+  const void* z; long long z_bs, z_ts;
+  const float* dz; long long dz_bs, dz_ts;
+  const float *h, *act;                          // fp32 position-major [N, B, ...], as the arrays below
+  float *dr, *Gz, *dpre, *du, *dh, *dc;
+  float* partial;                                // [8, B, d]
+  void *s16, *p16;                               // bf16 operand rows [B, d], [B, d_ff]
+  int s0, e0;                                    // positions of the leaf, last one first
+  unsigned steps;                                // positions since the counters were zeroed
+  unsigned* counters;
+  SyncArea* sync;
+  int R, G, a_bytes;                             // set by the launcher
+  WideStage st[4];                               // W_k | W_v, W_down, W_up, W_o
+};
+int wide_backward_groups(int B, int d, int dff); // 0: not taken
+cudaError_t wide_backward_launch(WideBwdParams p, const AttnBufs& a, const WidePair& wp, cudaStream_t s);
 int wide_loop_groups(int B, int d, int dff);     // 0: not taken
 size_t wide_counter_bytes(int B);
 int wide_ssq_floats(int d);

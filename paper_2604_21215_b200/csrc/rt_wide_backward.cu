@@ -1,0 +1,373 @@
+// Reverse loop of wide batches (up to 128 sequences per group of SMs), one cooperative launch per leaf, bf16: the counterpart of
+// rt_wide_loop.cu, same roles, barriers and operand ring.  A position is seven steps (the launches of rt_backward.cu's wide_position_tc):
+//   P1 [dk_raw | dv] [W_k; W_v] in parts    R1 dr = sum, Gz = dz + RMS backward through z
+//   P2 (alpha Gz) W_down, times GELU'       P3 dpre W_up in parts    R3 du = sum, dh = Gz + RMS backward through h
+//   P4 dc = (alpha dh) W_o                  A  the pairs of the leaf, the temporary pair, the operand of the position before
+// R1 and R3 need sums over whole rows: four warps own a row.  In A only the newest pair, i - 1, is on the chain; the leaf's older pairs are
+// updated after the step has been counted in, by the same threads at every position.
+//
+// Measured per position at d = 1024, d_ff = 4096, B = 96: see the figures at wide_backward_launch.
+#include "rt_bwd.cuh"
+#include "rt_wide.cuh"
+
+namespace rt {
+namespace {
+
+enum { B_KV = 0, B_RZ = 1, B_DOWN = 2, B_UP = 3, B_RH = 4, B_OUT = 5, B_ATTN = 6, B_STEPS = 7 };
+// The products in order (indices of WideBwdParams::st): W_k | W_v, W_down, W_up, W_o (all transposed).
+struct WideBwdMaps { CUtensorMap a[4], w[4]; };
+
+// Phi(a) + a phi(a), Phi as in gelu_wide
+__device__ __forceinline__ float gelu_grad_wide(float x) {
+  float t;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.3275911f * 0.70710678f, fabsf(x), 1.0f)));
+  const float poly = t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 0.5f * 1.061405429f, -0.5f * 1.453152027f), 0.5f * 1.421413741f), -0.5f * 0.284496736f), 0.5f * 0.254829592f);
+  const float e = ex2(x * x * (-0.5f * kLog2e)), q = poly * e;
+  return (x < 0.f ? q : 1.0f - q) + x * 0.3989422804014327f * e;
+}
+__device__ __forceinline__ F8 ldcg8(const float* p) {
+  const float4 a = __ldcg(reinterpret_cast<const float4*>(p)), b = __ldcg(reinterpret_cast<const float4*>(p + 4));
+  return F8{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
+}
+
+// CH: groups of four columns per thread of a row's four warps (d <= 512 CH)
+template <int CH>
+__global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __grid_constant__ WideBwdMaps maps, const __grid_constant__ WideBwdParams p, const __grid_constant__ AttnBufs a,
+                                                                     const __grid_constant__ WidePair wp) {
+  extern __shared__ unsigned char smem_raw[];
+  WideCta c;
+  c.smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  c.sbase = smem_u32(c.smem);
+  c.s_abort = reinterpret_cast<volatile int*>(c.smem + kWAbort);
+  c.sync = p.sync;
+  c.G = p.G;
+  const int group = blockIdx.x / p.G;
+  c.rank = blockIdx.x % p.G;
+  c.arank = c.rank;
+  c.counters = p.counters + group * kWMaxSteps * kWCounterStride;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int m0 = group * p.R, R = p.B - m0 < p.R ? p.B - m0 : p.R;
+  wide_setup(c, tid, warp);
+  const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(c.smem + kWTmem), a_bytes = (uint32_t)p.a_bytes;
+  const int d = p.d, H = p.H, units = R * H;
+  auto active_of = [&](int step) {
+    if (step == B_RZ || step == B_RH) return R < p.G ? R : p.G;
+    if (step == B_ATTN) return wide_active_rows(units, 4, p.G);
+    return wide_active(p.st[step == B_KV ? 0 : step == B_OUT ? 3 : step - 1], p.G);
+  };
+  if (warp == 0) {
+    WideFetch f = {0u, 0u};
+    bool ok = true;
+#pragma unroll 1
+    for (int i = p.e0 - 1; i >= p.s0 && ok; --i) {
+      const unsigned n = p.steps + (unsigned)(p.e0 - 1 - i);                 // positions done before this one
+      int product = 0;
+#pragma unroll 1
+      for (int step = 0; step < B_STEPS && ok; ++step) {
+        const bool rows = step == B_RZ || step == B_RH || step == B_ATTN;
+        auto wait = [&]() {
+          bool r = true;
+          if (step == B_KV) { if (i < p.e0 - 1) r = c.poll(B_ATTN, n * (unsigned)active_of(B_ATTN)); }
+          else r = c.poll(step - 1, (n + 1) * (unsigned)active_of(step - 1));
+          if (lane == 0 && r) mbar_arrive(c.flag());
+          __syncwarp();
+          return r;
+        };
+        if (c.rank < active_of(step)) {
+          if (rows) ok = wait();
+          else ok = wide_fetch(c, f, p.st[product], &maps.a[product], &maps.w[product], nullptr, m0, a_bytes, wait);
+        }
+        if (!rows) ++product;
+      }
+    }
+  } else if (warp == 1) {
+    WideIssue w = {0u, 0};
+    bool ok = true;
+#pragma unroll 1
+    for (int i = p.e0 - 1; i >= p.s0 && ok; --i)
+#pragma unroll 1
+      for (int product = 0; product < 4 && ok; ++product) ok = wide_issue(c, w, p.st[product], a_bytes, tmem);
+  } else {
+    const int ew = warp - 2, quad = warp & 3, half = ew >> 2;
+    const uint32_t t_row = tmem + ((uint32_t)(quad * 32) << 16);
+    const size_t rstride = (size_t)p.B * d;
+    float* stage = reinterpret_cast<float*>(c.smem + kWStage + ew * kWStageWarp);
+    uint32_t flags = 0;
+    int jobs = 0;
+    auto flag_wait = [&]() { const bool r = wide_wait(c.flag(), flags & 1u, c.s_abort, c.sync); ++flags; return r; };
+    auto acc_wait = [&]() {
+      const bool r = wide_wait(c.tfull(jobs & 1), (jobs >> 1) & 1, c.s_abort, c.sync);
+      tc_fence_after();
+      return r;
+    };
+    auto acc_done = [&]() {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(c.tempty(jobs & 1));
+      ++jobs;
+    };
+    auto finish = [&](bool ok, int step) {
+      ok = epi_all(ok);
+      if (tid == 64 && ok) red_release_add_u32(c.counters + step * kWCounterStride, 1u);
+      return ok;
+    };
+    // a product whose sums (or parts of them) go to memory as they are: out[split][row][column]
+    auto plain_product = [&](const WideStage& st, float* out) {
+      bool good = flag_wait();
+#pragma unroll 1
+      for (int job = c.rank; job < st.tiles * st.splits; job += c.G) {
+        const int n0 = (job % st.tiles) * st.bn, split = job / st.tiles;
+        if (!good || !(good = acc_wait())) break;
+#pragma unroll 1
+        for (int cc = half * (st.bn >> 1); cc < (half + 1) * (st.bn >> 1); cc += 32) {
+          wide_stage(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane, [](float v) { return v; });
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const int r = 4 * k + (lane >> 3), col = 4 * (lane & 7);
+            const float4 v = *reinterpret_cast<const float4*>(stage + r * kWStagePitch + col);
+            if (quad * 32 + r < R) *reinterpret_cast<float4*>(out + ((size_t)split * p.B + m0 + quad * 32 + r) * d + n0 + cc + col) = v;
+          }
+        }
+        acc_done();
+      }
+      return good;
+    };
+    // out = add + RMS backward of the sum of the parts through RMS(u) g; keeps the sum, leaves bf16(alpha out) as the next operand.  Four warps
+    // per row; u and add do not depend on the step before and are fetched ahead of it for the first row.
+    const int team = ew >> 2, tt = (ew & 3) * 32 + lane;
+    float* red = reinterpret_cast<float*>(c.smem + kWStage + team * 4 * kWStageWarp);
+    auto norm_rows = [&](int splits, auto load_u, auto load_add, const __nv_bfloat16* g, bool enable, float* sum, float* out) {
+      float uv[CH][4], av[CH][4];
+      int parity = 0;
+      auto fetch = [&](int row) {
+#pragma unroll
+        for (int k = 0; k < CH; ++k) {
+          const int n = 4 * (tt + 128 * k);
+          if (n >= d) break;
+          load_u(row, n, uv[k]);
+          load_add(row, n, av[k]);
+        }
+      };
+      const int row0 = c.rank + team * c.G;
+      if (row0 < R) fetch(row0);
+      const bool good = epi_all(flag_wait());
+      if (!good) return false;
+#pragma unroll 1
+      for (int row = row0; row < R; row += 2 * c.G) {
+        if (row != row0) fetch(row);
+        const size_t at = (size_t)(m0 + row) * d;
+        float dy[CH][4], ss = 0.f, tu = 0.f;
+#pragma unroll
+        for (int k = 0; k < CH; ++k) {
+          const int n = 4 * (tt + 128 * k);
+          if (n >= d) break;
+          float4 pv[8];
+#pragma unroll
+          for (int z = 0; z < 8; ++z)
+            if (z < splits) pv[z] = __ldcg(reinterpret_cast<const float4*>(p.partial + (size_t)z * rstride + at + n));
+          float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int z = 0; z < 8; ++z)
+            if (z < splits) { acc.x += pv[z].x; acc.y += pv[z].y; acc.z += pv[z].z; acc.w += pv[z].w; }
+          *reinterpret_cast<float4*>(sum + at + n) = acc;
+          dy[k][0] = acc.x; dy[k][1] = acc.y; dy[k][2] = acc.z; dy[k][3] = acc.w;
+          if (enable) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              dy[k][e] *= gain_at(g, n + e);
+              ss = fmaf(uv[k][e], uv[k][e], ss);
+              tu = fmaf(dy[k][e], uv[k][e], tu);
+            }
+          }
+        }
+        float inv = 1.f, mean = 0.f;
+        if (enable) {
+          ss = warp_sum(ss); tu = warp_sum(tu);
+          if (lane == 0) { red[parity * 8 + (ew & 3)] = ss; red[parity * 8 + 4 + (ew & 3)] = tu; }
+          asm volatile("barrier.cta.sync %0, 128;" ::"r"(2 + team) : "memory");
+          ss = red[parity * 8] + red[parity * 8 + 1] + red[parity * 8 + 2] + red[parity * 8 + 3];
+          tu = red[parity * 8 + 4] + red[parity * 8 + 5] + red[parity * 8 + 6] + red[parity * 8 + 7];
+          inv = rsqrtf(ss / d + p.eps); mean = tu * inv / d;
+          parity ^= 1;
+        }
+#pragma unroll
+        for (int k = 0; k < CH; ++k) {
+          const int n = 4 * (tt + 128 * k);
+          if (n >= d) break;
+          float r[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) r[e] = av[k][e] + (enable ? inv * (dy[k][e] - uv[k][e] * inv * mean) : dy[k][e]);
+          *reinterpret_cast<float4*>(out + at + n) = make_float4(r[0], r[1], r[2], r[3]);
+          *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.s16) + at + n) = make_uint2(pack2(r[0] * p.alpha, r[1] * p.alpha), pack2(r[2] * p.alpha, r[3] * p.alpha));
+        }
+      }
+      return true;
+    };
+    const __nv_bfloat16* Z = reinterpret_cast<const __nv_bfloat16*>(p.z);
+    const int t8 = lane & 7;
+    bool ok = true;
+#pragma unroll 1
+    for (int i = p.e0 - 1; i >= p.s0 && ok; --i) {
+      const size_t od = (size_t)i * rstride, of = (size_t)i * p.B * p.dff;
+      if (c.rank < active_of(B_KV)) {
+        ok = finish(plain_product(p.st[0], p.partial), B_KV);
+        if (!ok) break;
+      }
+      if (c.rank < active_of(B_RZ)) {
+        ok = norm_rows(p.st[0].splits,
+                       [&](int row, int n, float (&v)[4]) { reinterpret_cast<const Vec4<__nv_bfloat16>*>(Z + (size_t)(m0 + row) * p.z_bs + (size_t)i * p.z_ts + n)->to_float(v); },
+                       [&](int row, int n, float (&v)[4]) { reinterpret_cast<const Vec4<float>*>(p.dz + (size_t)(m0 + row) * p.dz_bs + (size_t)i * p.dz_ts + n)->to_float(v); },
+                       reinterpret_cast<const __nv_bfloat16*>(p.g_kv), p.z_norm != 0, p.dr + od, p.Gz + od);
+        ok = finish(ok, B_RZ);
+        if (!ok) break;
+      }
+      if (c.rank < active_of(B_DOWN)) {
+        // dpre = (alpha Gz W_down) GELU'(act)
+        bool good = flag_wait();
+        const WideStage& st = p.st[1];
+#pragma unroll 1
+        for (int job = c.rank; job < st.tiles; job += c.G) {
+          const int n0 = job * st.bn;
+          float4 xv[8];
+          auto fetch = [&](int cc) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const int rr = quad * 32 + 4 * k + (lane >> 3);
+              xv[k] = *reinterpret_cast<const float4*>(p.act + of + (size_t)(m0 + (rr < R ? rr : 0)) * p.dff + n0 + cc + 4 * (lane & 7));
+            }
+          };
+          fetch(half * (st.bn >> 1));
+          if (!good || !(good = acc_wait())) break;
+#pragma unroll 1
+          for (int cc = half * (st.bn >> 1); cc < (half + 1) * (st.bn >> 1); cc += 32) {
+            if (cc != half * (st.bn >> 1)) fetch(cc);
+            wide_stage(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane, [](float v) { return v; });
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const int r = 4 * k + (lane >> 3);
+              const float4 v = *reinterpret_cast<const float4*>(stage + r * kWStagePitch + 4 * (lane & 7));
+              const float4 o = make_float4(v.x * gelu_grad_wide(xv[k].x), v.y * gelu_grad_wide(xv[k].y), v.z * gelu_grad_wide(xv[k].z), v.w * gelu_grad_wide(xv[k].w));
+              if (quad * 32 + r < R) {
+                const size_t at = (size_t)(m0 + quad * 32 + r) * p.dff + n0 + cc + 4 * (lane & 7);
+                *reinterpret_cast<float4*>(p.dpre + of + at) = o;
+                *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.p16) + at) = make_uint2(pack2(o.x, o.y), pack2(o.z, o.w));
+              }
+            }
+          }
+          acc_done();
+        }
+        ok = finish(good, B_DOWN);
+        if (!ok) break;
+      }
+      if (c.rank < active_of(B_UP)) {
+        ok = finish(plain_product(p.st[2], p.partial), B_UP);
+        if (!ok) break;
+      }
+      if (c.rank < active_of(B_RH)) {
+        ok = norm_rows(p.st[2].splits,
+                       [&](int row, int n, float (&v)[4]) { reinterpret_cast<const Vec4<float>*>(p.h + od + (size_t)(m0 + row) * d + n)->to_float(v); },
+                       [&](int row, int n, float (&v)[4]) { reinterpret_cast<const Vec4<float>*>(p.Gz + od + (size_t)(m0 + row) * d + n)->to_float(v); },     // this thread's own
+                       reinterpret_cast<const __nv_bfloat16*>(p.g_mlp), p.pre != 0, p.du + od, p.dh + od);
+        ok = finish(ok, B_RH);
+        if (!ok) break;
+      }
+      if (c.rank < active_of(B_OUT)) {
+        ok = finish(plain_product(p.st[3], p.dc + od), B_OUT);
+        if (!ok) break;
+      }
+      if (c.rank < active_of(B_ATTN)) {
+        // one (sequence, head) per eight lanes, spread over the group's CTAs warp by warp
+        const int u = (ew * c.G + c.rank) * 4 + (lane >> 3), stride = 32 * c.G;
+        auto col_of = [&](int v, int& b, int& h) { const int w = v < units ? v : 0; b = m0 + w / H; h = w % H; return (size_t)b * d + h * kHeadDim + 8 * t8; };
+        bool waited = false;
+#pragma unroll 1
+        for (int v = u; v - (lane >> 3) < units && ok; v += stride) {
+          int b, h;
+          const size_t col = col_of(v, b, h), ri = od + col, rj = ri - rstride;
+          const bool live = v < units, newest = i > p.s0;
+          const size_t si = ((size_t)i * p.B + b) * H + h;
+          const F8 q = ld8(a.q + ri), cc = ld8(a.c + ri);
+          const float lse = a.lse[si], slope = a.alibi ? a.alibi[h] * kLog2e : 0.f;
+          F8 kk, vv, gk, gv, kr;
+          if (newest) { kk = ld8(a.k + rj); vv = ld8(a.v + rj); gk = ld8(a.dK + rj); gv = ld8(a.dV + rj); kr = ld8(wp.kraw + rj); }
+          if (!waited) { ok = flag_wait(); waited = true; }
+          if (!ok) break;
+          const F8 dc = ldcg8(p.dc + ri);
+          const float D = group_sum(dot8(dc, cc));
+          if (newest) {
+            const float pr = exp2f(group_sum(dot8(q, kk)) * a.scale_log2 - slope - lse);
+            const float ds = pr * (group_sum(dot8(dc, vv)) - D) * a.scale;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) { gk.v[e] = fmaf(ds, q.v[e], gk.v[e]); gv.v[e] = fmaf(pr, dc.v[e], gv.v[e]); }
+            if (live) { st8(a.dK + rj, gk); st8(a.dV + rj, gv); }
+            __nv_bfloat16* op = wp.op + (size_t)b * 2 * d + h * kHeadDim + 8 * t8;
+            pair_operand(gk, gv, kr, wp.g_k, h, t8, wp.eps, wp.qk, wp.dkraw + rj, op, op + d, live);
+          }
+          if (live && t8 == 0) a.D[si] = D;
+        }
+        if (!waited) ok = flag_wait();
+        ok = finish(ok, B_ATTN);
+        if (!ok) break;
+        // off the chain: the older pairs of the leaf and the temporary pair
+#pragma unroll 1
+        for (int v = u; v - (lane >> 3) < units; v += stride) {
+          int b, h;
+          const size_t col = col_of(v, b, h), ri = od + col;
+          const bool live = v < units;
+          const size_t si = ((size_t)i * p.B + b) * H + h;
+          const F8 q = ld8(a.q + ri), dc = ldcg8(p.dc + ri), kt = ld8(a.kt + ri), vt = ld8(a.vt + ri), cc = ld8(a.c + ri);
+          const float lse = a.lse[si], slope = a.alibi ? a.alibi[h] * kLog2e : 0.f, D = group_sum(dot8(dc, cc));
+          {
+            const float pr = exp2f(group_sum(dot8(q, kt)) * a.scale_log2 - lse);
+            const float ds = pr * (group_sum(dot8(dc, vt)) - D) * a.scale;
+            F8 o1, o2;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) { o1.v[e] = ds * q.v[e]; o2.v[e] = pr * dc.v[e]; }
+            if (live) { st8(a.dkt + ri, o1); st8(a.dvt + ri, o2); }
+          }
+#pragma unroll 2
+          for (int j = p.s0; j < i - 1; ++j) {
+            const size_t rj = (size_t)j * rstride + col;
+            const F8 kk = ld8(a.k + rj), vv = ld8(a.v + rj);
+            F8 gk = ld8(a.dK + rj), gv = ld8(a.dV + rj);
+            const float pr = exp2f(group_sum(dot8(q, kk)) * a.scale_log2 - slope * (float)(i - j) - lse);
+            const float ds = pr * (group_sum(dot8(dc, vv)) - D) * a.scale;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) { gk.v[e] = fmaf(ds, q.v[e], gk.v[e]); gv.v[e] = fmaf(pr, dc.v[e], gv.v[e]); }
+            if (live) { st8(a.dK + rj, gk); st8(a.dV + rj, gv); }
+          }
+        }
+      }
+    }
+  }
+  wide_teardown(tmem, warp);
+}
+}  // namespace
+
+// Of the reverse loop: 0, or the number of groups.  A row of more than 4096 entries would not fit the registers of its four warps.
+int wide_backward_groups(int B, int d, int dff) { return d <= 4096 ? wide_loop_groups(B, d, dff) : 0; }
+
+cudaError_t wide_backward_launch(WideBwdParams p, const AttnBufs& a, const WidePair& wp, cudaStream_t s) {
+  const int groups = wide_backward_groups(p.B, p.d, p.dff);
+  if (!groups) return cudaErrorInvalidValue;
+  p.R = ceil_div(p.B, groups); p.G = kB200Sms / groups;
+  const int box = (p.R + 7) / 8 * 8;
+  p.a_bytes = box * 128;
+  p.st[0] = stage_split(p.d, 2 * p.d, p.G, p.a_bytes);
+  p.st[1] = stage_whole(p.dff, p.d, p.G, p.a_bytes, 128);
+  p.st[2] = stage_split(p.d, p.dff, p.G, p.a_bytes);
+  p.st[3] = stage_whole(p.d, p.d, p.G, p.a_bytes, 128);
+  WideBwdMaps m;
+  const void *A[4] = {wp.op, p.s16, p.p16, p.s16}, *W[4] = {p.wkvT, p.wdnT, p.wupT, p.woT};
+  const int K[4] = {2 * p.d, p.d, p.dff, p.d}, N[4] = {p.d, p.dff, p.d, p.d};
+  for (int i = 0; i < 4; ++i)
+    if (!map_blocks(&m.a[i], A[i], p.B, K[i], box) || !map_blocks(&m.w[i], W[i], N[i], K[i], p.st[i].bn)) return cudaErrorInvalidValue;
+  const void* fn = p.d <= 1024 ? reinterpret_cast<const void*>(&wide_backward_kernel<2>) : reinterpret_cast<const void*>(&wide_backward_kernel<8>);
+  const int smem = (int)kWTotal + 1024;
+  cudaError_t e = ensure_dynamic_smem(fn, smem);
+  if (e != cudaSuccess) return e;
+  void* args[] = {(void*)&m, (void*)&p, (void*)&a, (void*)&wp};
+  return cudaLaunchCooperativeKernel(fn, dim3(groups * p.G), dim3(kWThreads), args, smem, s);
+}
+
+}  // namespace rt
