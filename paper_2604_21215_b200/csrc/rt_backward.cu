@@ -111,6 +111,32 @@ __global__ void transpose_bf16_kernel(const TI* __restrict__ in, long long R, in
   }
 }
 
+// The same for fp32 arrays whose width and padded row count are multiples of 64: 16-byte loads and stores on both sides (12288 x 1024: 35 us
+// with the kernel above, whose stores are 64 bytes per warp).  grid (C / 64, ld / 64), 256 threads.
+__global__ void __launch_bounds__(256) transpose_f32_kernel(const float* __restrict__ in, long long R, int C, __nv_bfloat16* __restrict__ out, long long ld) {
+  __shared__ float tile[64][65];
+  const long long r0 = (long long)blockIdx.y * 64;
+  const int c0 = blockIdx.x * 64, tid = threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int r = (tid >> 4) + 16 * k, c = 4 * (tid & 15);
+    const float4 v = r0 + r < R ? *reinterpret_cast<const float4*>(in + (r0 + r) * C + c0 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    tile[r][c] = v.x; tile[r][c + 1] = v.y; tile[r][c + 2] = v.z; tile[r][c + 3] = v.w;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int c = (tid >> 3) + 32 * k, r = 8 * (tid & 7);
+    unsigned w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const __nv_bfloat162 v = __floats2bfloat162_rn(tile[r + 2 * e][c], tile[r + 2 * e + 1][c]);
+      w[e] = *reinterpret_cast<const unsigned*>(&v);
+    }
+    *reinterpret_cast<uint4*>(out + (long long)(c0 + c) * ld + r0 + r) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
 // ------------------------------------------------------------------------------------------------ RMS forward / backward
 // Row r = i*B + b of a [B, N, *] array sits at b*bs + i*ts; position-major fp32 buffers use bs = width, ts = B*width.
 __device__ __forceinline__ long long row_at(long long r, int B, long long bs, long long ts) { return (r % B) * bs + (r / B) * ts; }
@@ -131,6 +157,58 @@ __global__ void norm_fwd_kernel(const TI* __restrict__ in, long long bs, long lo
   ss = warp_sum(ss);
   const float inv = rsqrtf(ss / G + eps);
   for (int e = lane; e < G; e += 32) dst[e] = enable ? to_f(src[e]) * inv * gain_at(g, c0 + e) : to_f(src[e]);
+}
+
+// qkRMS of a position-major fp32 array [heads, 64]: eight lanes per head, 16-byte accesses (24576 heads of a warp each moved 1.6 TB/s).
+template <typename TG>
+__global__ void __launch_bounds__(256) head_norm_fwd_kernel(const float* __restrict__ in, const TG* __restrict__ g, float* __restrict__ out, long long heads, int H, float eps, int enable) {
+  const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+  const int t = threadIdx.x & 7;
+  const bool live = gid < heads;
+  const long long at = (live ? gid : 0) * kHeadDim + 8 * t;
+  F8 u = ld8(in + at);
+  const float inv = rsqrtf(group_sum(dot8(u, u)) / kHeadDim + eps);
+  if (enable) {
+    const int c = (int)((live ? gid : 0) % H) * kHeadDim + 8 * t;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) u.v[e] *= inv * gain_at(g, c + e);
+  }
+  if (live) st8(out + at, u);
+}
+// Its backward: out = du (dy itself when !enable), gprod (=|+=) dy uh; out and gprod may each be NULL.  dy and out may be the same array.
+template <typename TG>
+__global__ void __launch_bounds__(256) head_norm_bwd_kernel(const float* dy, const float* __restrict__ u_in, const TG* __restrict__ g, float* out, float* gprod, int gprod_acc, long long heads,
+                                                            int H, float eps, int enable) {
+  const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+  const int t = threadIdx.x & 7;
+  const bool live = gid < heads;
+  const long long at = (live ? gid : 0) * kHeadDim + 8 * t;
+  const F8 dyv = ld8(dy + at), u = ld8(u_in + at);
+  F8 du = dyv, gp = {};
+  if (enable) {
+    const int c = (int)((live ? gid : 0) % H) * kHeadDim + 8 * t;
+    F8 ty;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) ty.v[e] = dyv.v[e] * gain_at(g, c + e);
+    const float ss = group_sum(dot8(u, u)), tu = group_sum(dot8(ty, u));
+    const float inv = rsqrtf(ss / kHeadDim + eps), mean = tu * inv / kHeadDim;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const float uh = u.v[e] * inv;
+      du.v[e] = inv * (ty.v[e] - uh * mean);
+      gp.v[e] = dyv.v[e] * uh;
+    }
+  }
+  if (!live) return;
+  if (out) st8(out + at, du);
+  if (gprod) {
+    if (gprod_acc) {
+      const F8 old = ld8(gprod + at);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) gp.v[e] += old.v[e];
+    }
+    st8(gprod + at, gp);
+  }
 }
 
 // With y = g u inv, inv = (mean(u^2)+eps)^(-1/2), t = g dy and uh = u inv:  du = inv (t - uh mean(t uh)),  dg += dy uh.
@@ -223,15 +301,18 @@ __global__ void col_final_kernel(const float* __restrict__ part, int P, int d, f
   out[c] = (accumulate ? out[c] : 0.f) + s;
 }
 
-// h = x + alpha a  (x [B,N,d] storage type, a and h position-major fp32)
+// h = x + alpha a  (x [B,N,d] storage type, a and h position-major fp32), four consecutive entries per thread
 template <typename T>
 __global__ void residual_kernel(const T* __restrict__ x, long long bs, long long ts, int B, const float* __restrict__ a, float alpha,
                                 float* __restrict__ h, long long rows, int d) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long idx = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
   if (idx >= rows * d) return;
-  const long long r = idx / d;
-  const int c = (int)(idx % d);
-  h[idx] = to_f(x[row_at(r, B, bs, ts) + c]) + alpha * a[idx];
+  const unsigned r = (unsigned)(idx / d);
+  const int c = (int)(idx - (long long)r * d);
+  const float4 av = *reinterpret_cast<const float4*>(a + idx);
+  float xv[4];
+  reinterpret_cast<const Vec4<T>*>(x + row_at(r, B, bs, ts) + c)->to_float(xv);
+  *reinterpret_cast<float4*>(h + idx) = make_float4(xv[0] + alpha * av.x, xv[1] + alpha * av.y, xv[2] + alpha * av.z, xv[3] + alpha * av.w);
 }
 
 __device__ __forceinline__ float gelu_f(float a) { return 0.5f * a * (1.f + erff(a * 0.70710678118654752f)); }
@@ -250,8 +331,10 @@ __global__ void gelu_bwd_kernel(float* __restrict__ dg, const float* __restrict_
   }
 }
 __global__ void gelu_kernel(const float* __restrict__ a, float* __restrict__ out, long long n) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < n) out[idx] = gelu_f(a[idx]);
+  const long long idx = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
+  if (idx >= n) return;
+  const float4 v = *reinterpret_cast<const float4*>(a + idx);
+  *reinterpret_cast<float4*>(out + idx) = make_float4(gelu_f(v.x), gelu_f(v.y), gelu_f(v.z), gelu_f(v.w));
 }
 
 // ------------------------------------------------------------------------------------------------ attention
@@ -1311,6 +1394,7 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   const T* g_kv = (const T*)(w->g_kv ? w->g_kv : w->g_attn);
   const int tpb = 256;
   auto warps_grid = [&](long long warps) { return (unsigned)((warps * 32 + tpb - 1) / tpb); };
+  const unsigned heads_grid = (unsigned)((rows * H * 8 + tpb - 1) / tpb);
   auto elems_grid = [&](long long n) { return (unsigned)((n + tpb - 1) / tpb); };
 
   // Products over all rows.  bf16 storage with tile-friendly widths: tensor cores (dense_tc_kernel) on bf16 copies of
@@ -1323,18 +1407,19 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   __nv_bfloat16* SB = reinterpret_cast<__nv_bfloat16*>(ws + L.sb);
   __nv_bfloat16* WT = reinterpret_cast<__nv_bfloat16*>(ws + L.wt);
   __nv_bfloat16* SC = SB + align_up((size_t)2 * B * d, 64);      // wide batches: operand rows of one position beside SB's [B, 2 d]
-  auto tc_product = [&](int M, int Nn, int K, const void* A, const void* W, float* out, float al, bool acc) {
+  auto tc_product = [&](int M, int Nn, int K, const void* A, const void* W, float* out, float al, bool acc, bool split = false) {
     DenseParams dp;
     memset(&dp, 0, sizeof(dp));
     dp.M = M; dp.N = Nn; dp.K = K; dp.B = 1; dp.A = A; dp.W = W; dp.epi = DENSE_F32; dp.alpha = al; dp.accumulate = acc ? 1 : 0;
     dp.h = out;
+    if (split) { dp.partial = F(L.gprod); dp.partial_bytes = (size_t)rows * d * sizeof(float); }
     return dense_launch(RT_BF16, dp, sync, s);
   };
   auto to_bf16 = [&](const float* in, __nv_bfloat16* out, long long n) {
     to_bf16_kernel<<<elems_grid((n + 3) / 4), tpb, 0, s>>>(in, out, n);
   };
   auto transpose_f = [&](const float* in, long long R, int C, __nv_bfloat16* out) {
-    transpose_bf16_kernel<float><<<dim3(ceil_div(C, 32), (unsigned)(rows_k / 32)), dim3(32, 8), 0, s>>>(in, R, C, out, rows_k);
+    transpose_f32_kernel<<<dim3(C / 64, (unsigned)(rows_k / 64)), 256, 0, s>>>(in, R, C, out, rows_k);      // (tensor cores: widths of 128)
   };
   const float* sa_holds = nullptr;                               // which array SA currently holds as a plain bf16 copy
   // out[rows, n_out] = A[rows, k] W[n_out, k]^T  (a product of the forward pass)
@@ -1361,12 +1446,12 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   RT_TRY(fwd_product(F(L.n), d, Wq, d, F(L.qraw)));
   RT_TRY(fwd_product(F(L.n), d, Wk, d, F(L.ktraw)));
   RT_TRY(fwd_product(F(L.n), d, Wv, d, F(L.vt)));
-  norm_fwd_kernel<float, T><<<warps_grid(rows * H), tpb, 0, s>>>(F(L.qraw), pbs, pts, B, g_q, F(L.q), rows, d, kHeadDim, eps, qk);
-  norm_fwd_kernel<float, T><<<warps_grid(rows * H), tpb, 0, s>>>(F(L.ktraw), pbs, pts, B, g_k, F(L.kt), rows, d, kHeadDim, eps, qk);
+  head_norm_fwd_kernel<T><<<heads_grid, tpb, 0, s>>>(F(L.qraw), g_q, F(L.q), rows * H, H, eps, qk);
+  head_norm_fwd_kernel<T><<<heads_grid, tpb, 0, s>>>(F(L.ktraw), g_k, F(L.kt), rows * H, H, eps, qk);
   norm_fwd_kernel<T, T><<<warps_grid(rows), tpb, 0, s>>>(z, xbs, xts, B, g_kv, F(L.r), rows, d, d, eps, z_norm ? 1 : 0);
   RT_TRY(fwd_product(F(L.r), d, Wk, d, F(L.kraw)));
   RT_TRY(fwd_product(F(L.r), d, Wv, d, F(L.v)));
-  norm_fwd_kernel<float, T><<<warps_grid(rows * H), tpb, 0, s>>>(F(L.kraw), pbs, pts, B, g_k, F(L.k), rows, d, kHeadDim, eps, qk);
+  head_norm_fwd_kernel<T><<<heads_grid, tpb, 0, s>>>(F(L.kraw), g_k, F(L.k), rows * H, H, eps, qk);
   memset(&ab, 0, sizeof(ab));
   ab.q = F(L.q); ab.k = F(L.k); ab.v = F(L.v); ab.kt = F(L.kt); ab.vt = F(L.vt); ab.lse = F(L.lse); ab.D = F(L.D);
   ab.c = F(L.c); ab.dc = F(L.dc); ab.dK = F(L.dK); ab.dV = F(L.dV); ab.dkt = F(L.dkt); ab.dvt = F(L.dvt); ab.dq = F(L.dq);
@@ -1413,10 +1498,10 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
     attn_stats_kernel<<<warps_grid((long long)((N + 3) / 4) * B * H), tpb, 0, s>>>(ab);
   }
   RT_TRY(fwd_product(F(L.c), d, Wo, d, F(L.dn)));                     // a = W_o c (dn as scratch)
-  residual_kernel<T><<<elems_grid(rows * d), tpb, 0, s>>>(x, xbs, xts, B, F(L.dn), alpha, F(L.h), rows, d);
+  residual_kernel<T><<<elems_grid(rows * d / 4), tpb, 0, s>>>(x, xbs, xts, B, F(L.dn), alpha, F(L.h), rows, d);
   norm_fwd_kernel<float, T><<<warps_grid(rows), tpb, 0, s>>>(F(L.h), pbs, pts, B, g_mlp, F(L.u), rows, d, d, eps, pre ? 1 : 0);
   RT_TRY(fwd_product(F(L.u), d, Wup, f, F(L.act)));
-  gelu_kernel<<<elems_grid(rows * f), tpb, 0, s>>>(F(L.act), F(L.gl), rows * f);
+  gelu_kernel<<<elems_grid((rows * f + 3) / 4), tpb, 0, s>>>(F(L.act), F(L.gl), rows * f);
   RT_TRY(cudaGetLastError());
   }
 
@@ -1669,15 +1754,12 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   };
   // qkRMS backward of dq and of the temporary keys (in place), and their gain products
   const bool want_gq = gr->g_q && w->g_q && qk, want_gk = gr->g_k && w->g_k && qk;
-  norm_bwd_kernel<float, T><<<warps_grid(rows * H), tpb, 0, s>>>(F(L.dq), F(L.qraw), pbs, pts, B, g_q, nullptr, F(L.dq), pbs, pts,
-                                                                 want_gq ? gprod : nullptr, 0, rows, d, kHeadDim, eps, qk);
+  head_norm_bwd_kernel<T><<<heads_grid, tpb, 0, s>>>(F(L.dq), F(L.qraw), g_q, F(L.dq), want_gq ? gprod : nullptr, 0, rows * H, H, eps, qk);
   if (want_gq) col_sum(gprod, d, gr->g_q, false);
   else if (gr->g_q) RT_TRY(cudaMemsetAsync(gr->g_q, 0, (size_t)d * 4, s));
-  norm_bwd_kernel<float, T><<<warps_grid(rows * H), tpb, 0, s>>>(F(L.dkt), F(L.ktraw), pbs, pts, B, g_k, nullptr, F(L.dkt), pbs, pts,
-                                                                 want_gk ? gprod : nullptr, 0, rows, d, kHeadDim, eps, qk);
+  head_norm_bwd_kernel<T><<<heads_grid, tpb, 0, s>>>(F(L.dkt), F(L.ktraw), g_k, F(L.dkt), want_gk ? gprod : nullptr, 0, rows * H, H, eps, qk);
   if (want_gk) {
-    norm_bwd_kernel<float, T><<<warps_grid(rows * H), tpb, 0, s>>>(F(L.dK), F(L.kraw), pbs, pts, B, g_k, nullptr, nullptr, pbs, pts,
-                                                                   gprod, 1, rows, d, kHeadDim, eps, qk);
+    head_norm_bwd_kernel<T><<<heads_grid, tpb, 0, s>>>(F(L.dK), F(L.kraw), g_k, nullptr, gprod, 1, rows * H, H, eps, qk);
     col_sum(gprod, d, gr->g_k, false);
   } else if (gr->g_k) RT_TRY(cudaMemsetAsync(gr->g_k, 0, (size_t)d * 4, s));
   // dn = dqraw W_q + dktraw W_k + dvt W_v;  dx = dh + RMS backward of dn through RMS(x)
@@ -1715,7 +1797,7 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
     if (!tc) return gemm<float, float>(n_out, n_in, (int)rows, dY, 1, n_out, X, n_in, 1, out, n_in, al, acc, s);
     transpose_f(dY, rows, n_out, SA); sa_holds = nullptr;
     if (sb_holds != X) { transpose_f(X, rows, n_in, SB); sb_holds = X; }
-    return tc_product(n_out, n_in, (int)rows_k, SA, SB, out, al, acc);
+    return tc_product(n_out, n_in, (int)rows_k, SA, SB, out, al, acc, true);     // d x d results are 64 tiles at d = 1024: in parts over the rows
   };
   if (gr->w_k) RT_TRY(wgrad(gr->w_k, F(L.dkraw), d, F(L.r), d, 1.f, false));
   if (gr->w_v) RT_TRY(wgrad(gr->w_v, F(L.dvf), d, F(L.r), d, 1.f, false));
