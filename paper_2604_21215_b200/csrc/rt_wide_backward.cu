@@ -7,6 +7,8 @@
 // updated after the step has been counted in, by the same threads at every position.
 //
 // Measured per position at d = 1024, d_ff = 4096, B = 96: see the figures at wide_backward_launch.
+#include <type_traits>
+
 #include "rt_bwd.cuh"
 #include "rt_wide.cuh"
 
@@ -136,8 +138,15 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __gri
     // per row; u and add do not depend on the step before and are fetched ahead of it for the first row.
     const int team = ew >> 2, tt = (ew & 3) * 32 + lane;
     float* red = reinterpret_cast<float*>(c.smem + kWStage + team * 4 * kWStageWarp);
-    auto norm_rows = [&](int splits, auto load_u, auto load_add, const __nv_bfloat16* g, bool enable, float* sum, float* out) {
-      float uv[CH][4], av[CH][4];
+    auto norm_rows = [&](auto per, int splits, auto load_u, auto load_add, const __nv_bfloat16* g, bool enable, float* sum, float* out) {
+      constexpr int kPer = decltype(per)::value;
+      float uv[CH][4], av[CH][4], gv[CH][4];
+#pragma unroll
+      for (int k = 0; k < CH; ++k) {
+        const int n = 4 * (tt + 128 * k);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) gv[k][e] = n < d ? gain_at(g, n + e) : 1.f;
+      }
       int parity = 0;
       auto fetch = [&](int row) {
 #pragma unroll
@@ -157,24 +166,31 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __gri
         if (row != row0) fetch(row);
         const size_t at = (size_t)(m0 + row) * d;
         float dy[CH][4], ss = 0.f, tu = 0.f;
+        float4 pv[CH <= 2 ? CH : 1][kPer];                     // all parts of a row of up to 1024 entries are requested before the first sum
+        auto fetch_parts = [&](int k, float4 (&v)[kPer]) {
+          const int n = 4 * (tt + 128 * k) < d ? 4 * (tt + 128 * k) : 0;
+#pragma unroll
+          for (int z = 0; z < kPer; ++z) v[z] = __ldcg(reinterpret_cast<const float4*>(p.partial + (size_t)(z < splits ? z : 0) * rstride + at + n));
+        };
+        if (CH <= 2) {
+#pragma unroll
+          for (int k = 0; k < CH; ++k) fetch_parts(k, pv[k < 2 ? k : 0]);
+        }
 #pragma unroll
         for (int k = 0; k < CH; ++k) {
           const int n = 4 * (tt + 128 * k);
           if (n >= d) break;
-          float4 pv[8];
-#pragma unroll
-          for (int z = 0; z < 8; ++z)
-            if (z < splits) pv[z] = __ldcg(reinterpret_cast<const float4*>(p.partial + (size_t)z * rstride + at + n));
+          if (CH > 2) fetch_parts(k, pv[0]);
           float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-          for (int z = 0; z < 8; ++z)
-            if (z < splits) { acc.x += pv[z].x; acc.y += pv[z].y; acc.z += pv[z].z; acc.w += pv[z].w; }
+          for (int z = 0; z < kPer; ++z)
+            if (z < splits) { acc.x += pv[CH <= 2 ? k : 0][z].x; acc.y += pv[CH <= 2 ? k : 0][z].y; acc.z += pv[CH <= 2 ? k : 0][z].z; acc.w += pv[CH <= 2 ? k : 0][z].w; }
           *reinterpret_cast<float4*>(sum + at + n) = acc;
           dy[k][0] = acc.x; dy[k][1] = acc.y; dy[k][2] = acc.z; dy[k][3] = acc.w;
           if (enable) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              dy[k][e] *= gain_at(g, n + e);
+              dy[k][e] *= gv[k][e];
               ss = fmaf(uv[k][e], uv[k][e], ss);
               tu = fmaf(dy[k][e], uv[k][e], tu);
             }
@@ -205,6 +221,44 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __gri
     };
     const __nv_bfloat16* Z = reinterpret_cast<const __nv_bfloat16*>(p.z);
     const int t8 = lane & 7;
+    // one (sequence, head) per eight lanes, spread over the group's CTAs warp by warp
+    const int unit0 = (ew * c.G + c.rank) * 4 + (lane >> 3), unit_stride = 32 * c.G;
+    auto col_of = [&](int v, int& b, int& h) { const int w = v < units ? v : 0; b = m0 + w / H; h = w % H; return (size_t)b * d + h * kHeadDim + 8 * t8; };
+    // What of a position's attention is off the chain: the leaf's older pairs, by thirds, and the temporary pair (with the first third).  It
+    // waits for the products of the next position, whose accumulators the row warps would only wait for.
+    auto older_pairs = [&](int i, int third) {
+      const int n = i - 1 - p.s0, ja = p.s0 + n * third / 3, jb = p.s0 + n * (third + 1) / 3;
+      if (third && ja >= jb) return;
+#pragma unroll 1
+      for (int v = unit0; v - (lane >> 3) < units; v += unit_stride) {
+        int b, h;
+        const size_t col = col_of(v, b, h), ri = (size_t)i * rstride + col;
+        const bool live = v < units;
+        const size_t si = ((size_t)i * p.B + b) * H + h;
+        const F8 q = ld8(a.q + ri), dc = ldcg8(p.dc + ri), cc = ld8(a.c + ri);
+        const float lse = a.lse[si], slope = a.alibi ? a.alibi[h] * kLog2e : 0.f, D = group_sum(dot8(dc, cc));
+        if (third == 0) {
+          const F8 kt = ld8(a.kt + ri), vt = ld8(a.vt + ri);
+          const float pr = exp2f(group_sum(dot8(q, kt)) * a.scale_log2 - lse);
+          const float ds = pr * (group_sum(dot8(dc, vt)) - D) * a.scale;
+          F8 o1, o2;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) { o1.v[e] = ds * q.v[e]; o2.v[e] = pr * dc.v[e]; }
+          if (live) { st8(a.dkt + ri, o1); st8(a.dvt + ri, o2); }
+        }
+#pragma unroll 2
+        for (int j = ja; j < jb; ++j) {
+          const size_t rj = (size_t)j * rstride + col;
+          const F8 kk = ld8(a.k + rj), vv = ld8(a.v + rj);
+          F8 gk = ld8(a.dK + rj), gv = ld8(a.dV + rj);
+          const float pr = exp2f(group_sum(dot8(q, kk)) * a.scale_log2 - slope * (float)(i - j) - lse);
+          const float ds = pr * (group_sum(dot8(dc, vv)) - D) * a.scale;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) { gk.v[e] = fmaf(ds, q.v[e], gk.v[e]); gv.v[e] = fmaf(pr, dc.v[e], gv.v[e]); }
+          if (live) { st8(a.dK + rj, gk); st8(a.dV + rj, gv); }
+        }
+      }
+    };
     bool ok = true;
 #pragma unroll 1
     for (int i = p.e0 - 1; i >= p.s0 && ok; --i) {
@@ -214,13 +268,17 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __gri
         if (!ok) break;
       }
       if (c.rank < active_of(B_RZ)) {
-        ok = norm_rows(p.st[0].splits,
+        auto rows = [&](auto per) {
+          return norm_rows(per, p.st[0].splits,
                        [&](int row, int n, float (&v)[4]) { reinterpret_cast<const Vec4<__nv_bfloat16>*>(Z + (size_t)(m0 + row) * p.z_bs + (size_t)i * p.z_ts + n)->to_float(v); },
                        [&](int row, int n, float (&v)[4]) { reinterpret_cast<const Vec4<float>*>(p.dz + (size_t)(m0 + row) * p.dz_bs + (size_t)i * p.dz_ts + n)->to_float(v); },
                        reinterpret_cast<const __nv_bfloat16*>(p.g_kv), p.z_norm != 0, p.dr + od, p.Gz + od);
+        };
+        ok = p.st[0].splits > 4 ? rows(std::integral_constant<int, 8>()) : rows(std::integral_constant<int, 4>());
         ok = finish(ok, B_RZ);
         if (!ok) break;
       }
+      if (i + 1 < p.e0) older_pairs(i + 1, 0);
       if (c.rank < active_of(B_DOWN)) {
         // dpre = (alpha Gz W_down) GELU'(act)
         bool good = flag_wait();
@@ -228,25 +286,34 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __gri
 #pragma unroll 1
         for (int job = c.rank; job < st.tiles; job += c.G) {
           const int n0 = job * st.bn;
-          float4 xv[8];
-          auto fetch = [&](int cc) {
+          const int cols = st.bn >> 1;                          // 32 or 64 of this warp; GELU' is ready before the accumulators are
+          float4 xv[2][8];
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
               const int rr = quad * 32 + 4 * k + (lane >> 3);
-              xv[k] = *reinterpret_cast<const float4*>(p.act + of + (size_t)(m0 + (rr < R ? rr : 0)) * p.dff + n0 + cc + 4 * (lane & 7));
+              if (32 * q < cols) xv[q][k] = *reinterpret_cast<const float4*>(p.act + of + (size_t)(m0 + (rr < R ? rr : 0)) * p.dff + n0 + half * cols + 32 * q + 4 * (lane & 7));
             }
-          };
-          fetch(half * (st.bn >> 1));
+          }
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            if (32 * q >= cols) break;
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+              xv[q][k] = make_float4(gelu_grad_wide(xv[q][k].x), gelu_grad_wide(xv[q][k].y), gelu_grad_wide(xv[q][k].z), gelu_grad_wide(xv[q][k].w));
+          }
           if (!good || !(good = acc_wait())) break;
-#pragma unroll 1
-          for (int cc = half * (st.bn >> 1); cc < (half + 1) * (st.bn >> 1); cc += 32) {
-            if (cc != half * (st.bn >> 1)) fetch(cc);
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            if (32 * q >= cols) break;
+            const int cc = half * cols + 32 * q;
             wide_stage(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane, [](float v) { return v; });
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
               const int r = 4 * k + (lane >> 3);
-              const float4 v = *reinterpret_cast<const float4*>(stage + r * kWStagePitch + 4 * (lane & 7));
-              const float4 o = make_float4(v.x * gelu_grad_wide(xv[k].x), v.y * gelu_grad_wide(xv[k].y), v.z * gelu_grad_wide(xv[k].z), v.w * gelu_grad_wide(xv[k].w));
+              const float4 v = *reinterpret_cast<const float4*>(stage + r * kWStagePitch + 4 * (lane & 7)), x = xv[q][k];
+              const float4 o = make_float4(v.x * x.x, v.y * x.y, v.z * x.z, v.w * x.w);
               if (quad * 32 + r < R) {
                 const size_t at = (size_t)(m0 + quad * 32 + r) * p.dff + n0 + cc + 4 * (lane & 7);
                 *reinterpret_cast<float4*>(p.dpre + of + at) = o;
@@ -259,29 +326,31 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __gri
         ok = finish(good, B_DOWN);
         if (!ok) break;
       }
+      if (i + 1 < p.e0) older_pairs(i + 1, 1);
       if (c.rank < active_of(B_UP)) {
         ok = finish(plain_product(p.st[2], p.partial), B_UP);
         if (!ok) break;
       }
       if (c.rank < active_of(B_RH)) {
-        ok = norm_rows(p.st[2].splits,
+        auto rows = [&](auto per) {
+          return norm_rows(per, p.st[2].splits,
                        [&](int row, int n, float (&v)[4]) { reinterpret_cast<const Vec4<float>*>(p.h + od + (size_t)(m0 + row) * d + n)->to_float(v); },
                        [&](int row, int n, float (&v)[4]) { reinterpret_cast<const Vec4<float>*>(p.Gz + od + (size_t)(m0 + row) * d + n)->to_float(v); },     // this thread's own
                        reinterpret_cast<const __nv_bfloat16*>(p.g_mlp), p.pre != 0, p.du + od, p.dh + od);
+        };
+        ok = p.st[2].splits > 4 ? rows(std::integral_constant<int, 8>()) : rows(std::integral_constant<int, 4>());
         ok = finish(ok, B_RH);
         if (!ok) break;
       }
+      if (i + 1 < p.e0) older_pairs(i + 1, 2);
       if (c.rank < active_of(B_OUT)) {
         ok = finish(plain_product(p.st[3], p.dc + od), B_OUT);
         if (!ok) break;
       }
       if (c.rank < active_of(B_ATTN)) {
-        // one (sequence, head) per eight lanes, spread over the group's CTAs warp by warp
-        const int u = (ew * c.G + c.rank) * 4 + (lane >> 3), stride = 32 * c.G;
-        auto col_of = [&](int v, int& b, int& h) { const int w = v < units ? v : 0; b = m0 + w / H; h = w % H; return (size_t)b * d + h * kHeadDim + 8 * t8; };
         bool waited = false;
 #pragma unroll 1
-        for (int v = u; v - (lane >> 3) < units && ok; v += stride) {
+        for (int v = unit0; v - (lane >> 3) < units && ok; v += unit_stride) {
           int b, h;
           const size_t col = col_of(v, b, h), ri = od + col, rj = ri - rstride;
           const bool live = v < units, newest = i > p.s0;
@@ -308,37 +377,9 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __gri
         if (!waited) ok = flag_wait();
         ok = finish(ok, B_ATTN);
         if (!ok) break;
-        // off the chain: the older pairs of the leaf and the temporary pair
-#pragma unroll 1
-        for (int v = u; v - (lane >> 3) < units; v += stride) {
-          int b, h;
-          const size_t col = col_of(v, b, h), ri = od + col;
-          const bool live = v < units;
-          const size_t si = ((size_t)i * p.B + b) * H + h;
-          const F8 q = ld8(a.q + ri), dc = ldcg8(p.dc + ri), kt = ld8(a.kt + ri), vt = ld8(a.vt + ri), cc = ld8(a.c + ri);
-          const float lse = a.lse[si], slope = a.alibi ? a.alibi[h] * kLog2e : 0.f, D = group_sum(dot8(dc, cc));
-          {
-            const float pr = exp2f(group_sum(dot8(q, kt)) * a.scale_log2 - lse);
-            const float ds = pr * (group_sum(dot8(dc, vt)) - D) * a.scale;
-            F8 o1, o2;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) { o1.v[e] = ds * q.v[e]; o2.v[e] = pr * dc.v[e]; }
-            if (live) { st8(a.dkt + ri, o1); st8(a.dvt + ri, o2); }
-          }
-#pragma unroll 2
-          for (int j = p.s0; j < i - 1; ++j) {
-            const size_t rj = (size_t)j * rstride + col;
-            const F8 kk = ld8(a.k + rj), vv = ld8(a.v + rj);
-            F8 gk = ld8(a.dK + rj), gv = ld8(a.dV + rj);
-            const float pr = exp2f(group_sum(dot8(q, kk)) * a.scale_log2 - slope * (float)(i - j) - lse);
-            const float ds = pr * (group_sum(dot8(dc, vv)) - D) * a.scale;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) { gk.v[e] = fmaf(ds, q.v[e], gk.v[e]); gv.v[e] = fmaf(pr, dc.v[e], gv.v[e]); }
-            if (live) { st8(a.dK + rj, gk); st8(a.dV + rj, gv); }
-          }
-        }
       }
     }
+    if (ok) older_pairs(p.s0, 0);                              // (the first position's temporary pair)
   }
   wide_teardown(tmem, warp);
 }
