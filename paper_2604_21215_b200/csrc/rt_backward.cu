@@ -547,8 +547,7 @@ __global__ void wide_pair_kernel(AttnBufs a, WidePair w, int i) {
   const int h = (int)(u % a.H), b = (int)(u / a.H);
   const long long at = ((long long)i * a.B + b) * a.d + (long long)h * kHeadDim + 8 * t;
   const F8 dk = ld8(a.dK + at), dv = ld8(a.dV + at), kr = ld8(w.kraw + at);
-  __nv_bfloat16* op = w.op + (long long)b * 2 * a.d + h * kHeadDim + 8 * t;
-  pair_operand(dk, dv, kr, w.g_k, h, t, w.eps, w.qk, w.dkraw + at, op, op + a.d, live);
+  pair_operand(dk, dv, kr, w, b, a.d, h, t, w.dkraw + at, live);
 }
 
 // out = add + RMS backward of the row sum of `splits` partial products through RMS(u); keeps the sum, leaves scale * out in bf16 as the
@@ -644,9 +643,8 @@ __global__ void wide_attn_kernel(AttnBufs a, WidePair w, const float* __restrict
       if (pass ? g == 0 : valid) { st8(a.dK + rj, gk); st8(a.dV + rj, gv); }
       if (pass) {
         const F8 kr = ld8(w.kraw + rj);
-        __nv_bfloat16* op = w.op + (long long)b * 2 * a.d + col;
         // (all groups hold the same values; each writes them)
-        pair_operand(gk, gv, kr, w.g_k, h, t, w.eps, w.qk, w.dkraw + rj, op, op + a.d, true);
+        pair_operand(gk, gv, kr, w, b, a.d, h, t, w.dkraw + rj, true);
       }
     }
   }
@@ -1323,12 +1321,20 @@ constexpr int kColParts = 128;
 constexpr int kWideLeaf = 16;
 constexpr int kWideBatchFrom = 32;      // above this many sequences a step of the reverse loop runs as dense products over the batch
 
-// Sequences per launch of the tensor-core leaf kernel of the reverse loop (rt_backward_loop.cu), 0: not taken.
-constexpr int kFastLoopMax = 32;          // beyond, dense products over the batch win (slices of 8: 21 us per position each)
+// Up to 32 sequences the reverse loop keeps its operands to fp32 (three bf16 terms): up to 8 as mat-vecs of one launch per leaf
+// (rt_backward_loop.cu, 16 to 22 us per position), from 9 on as the dense products of wide batches with the terms as further rows of the
+// 128-row tile (rt_wide_backward.cu), or in slices of 8 where the widths are off the tensor-core products.
+constexpr int kFastLoopMax = 32, kFastLoopBest = 8;
+int bwd_wide_terms(const rt_config* c, int B) {
+  if (B > kFastLoopMax) return 1;
+  const bool ok = c->dtype == RT_BF16 && !(c->flags & RT_FLAG_BACKWARD_STEP_LAUNCHES) && B > kFastLoopBest && wide_backward_groups(B, c->d_model, c->d_ff) > 0;
+  return ok ? 3 : 0;
+}
 int bwd_fast_slice(const rt_config* c, int B) {
-  if (c->dtype != RT_BF16 || (c->flags & RT_FLAG_BACKWARD_STEP_LAUNCHES)) return 0;
+  if (c->dtype != RT_BF16 || (c->flags & RT_FLAG_BACKWARD_STEP_LAUNCHES) || bwd_wide_terms(c, B) == 3) return 0;
   return bwd_leaf_slice(B, c->d_model, c->n_heads, c->d_ff, kFastLoopMax);
 }
+bool bwd_is_wide(const rt_config* c, int B) { return (B > kWideBatchFrom || bwd_wide_terms(c, B) == 3) && !bwd_fast_slice(c, B); }
 
 BwdLayout bwd_layout(const rt_config* c, int B, int N) {
   BwdLayout L;
@@ -1348,7 +1354,7 @@ BwdLayout bwd_layout(const rt_config* c, int B, int N) {
   L.dkt = take(rows * d); L.dvt = take(rows * d); L.dn = take(rows * d); L.gprod = take(rows * d);
   L.part = take((size_t)kColParts * (d > f ? d : f));
   L.part2 = take((size_t)4 * B * d);
-  const bool tc = c->dtype == RT_BF16 && d % 128 == 0 && f % 128 == 0, wide = B > kWideBatchFrom && !bwd_fast_slice(c, B);
+  const bool tc = c->dtype == RT_BF16 && d % 128 == 0 && f % 128 == 0, wide = bwd_is_wide(c, B);
   // wide batches: bf16 transposes of the five matrices of the reverse loop, dL/dz in position-major order (fp32 products)
   L.dvf = bwd_fast_slice(c, B) ? take(rows * d) : L.dV;        // final dv of every position (the exchange words of the leaf kernel)
   L.qkv16 = take(3 * rows * d / 2 + 64);                       // bf16 copies of q, k, v for the tile kernels
@@ -1357,9 +1363,11 @@ BwdLayout bwd_layout(const rt_config* c, int B, int N) {
   const size_t rows_k = align_up(rows, 64);
   L.wctr = wide && tc ? take(wide_counter_bytes(B) / 4) : o;
   if (wide && tc && N < 8) L.gprod = take((size_t)8 * B * d);    // parts of split products
-  size_t sb_elems = rows_k * (d > f ? d : f);
-  if (wide && sb_elems < (2 * d + f) * B + 64) sb_elems = (2 * d + f) * B + 64;     // the operands of one position side by side
-  L.sa = take(rows_k * (d > f ? d : f) / 2 + 64); L.sb = take(sb_elems / 2 + 64); L.wt = take(d * d / 2 + 64);
+  size_t sa_elems = rows_k * (d > f ? d : f), sb_elems = sa_elems;
+  const size_t op_rows = bwd_wide_terms(c, B) == 3 ? kWideTermRows * 3 : B;
+  if (wide && sb_elems < (2 * d + f) * op_rows + 64) sb_elems = (2 * d + f) * op_rows + 64;     // the operands of one position side by side
+  if (wide && sa_elems < d * op_rows) sa_elems = d * op_rows;
+  L.sa = take(sa_elems / 2 + 64); L.sb = take(sb_elems / 2 + 64); L.wt = take(d * d / 2 + 64);
   L.total = o;
   return L;
 }
@@ -1406,7 +1414,8 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   __nv_bfloat16* SA = reinterpret_cast<__nv_bfloat16*>(ws + L.sa);
   __nv_bfloat16* SB = reinterpret_cast<__nv_bfloat16*>(ws + L.sb);
   __nv_bfloat16* WT = reinterpret_cast<__nv_bfloat16*>(ws + L.wt);
-  __nv_bfloat16* SC = SB + align_up((size_t)2 * B * d, 64);      // wide batches: operand rows of one position beside SB's [B, 2 d]
+  const int terms = kBf16 ? bwd_wide_terms(c, B) : 1;
+  __nv_bfloat16* SC = SB + align_up((size_t)2 * (terms == 3 ? kWideTermRows * 3 : B) * d, 64);      // wide batches: operand rows of one position beside SB's [B, 2 d]
   auto tc_product = [&](int M, int Nn, int K, const void* A, const void* W, float* out, float al, bool acc, bool split = false) {
     DenseParams dp;
     memset(&dp, 0, sizeof(dp));
@@ -1568,7 +1577,7 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   // Wide batches (the paper's own regime, Sec. 6): a step of the reverse loop is a dense product over the B rows of the
   // position -- tensor cores for bf16 storage -- between small row-wise kernels, instead of tasks of four sequences.
   const int fast = kBf16 ? bwd_fast_slice(c, B) : 0;             // sequences per launch of the tensor-core leaf kernel
-  const bool wide = B > kWideBatchFrom && !fast;
+  const bool wide = kBf16 ? bwd_is_wide(c, B) : B > kWideBatchFrom;
   // leaf of the reverse schedule; wide batches take short leaves (the in-leaf step re-reads and rewrites the fp32
   // pairs of its leaf at every position, the tiles do not)
   const int Lf = wide ? kWideLeaf : 64;
@@ -1636,7 +1645,7 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   const bool wide_tc = wide && tc;
   WidePair wp;
   memset(&wp, 0, sizeof(wp));
-  wp.kraw = F(L.kraw); wp.dkraw = F(L.dkraw); wp.g_k = reinterpret_cast<const __nv_bfloat16*>(g_k); wp.op = SB; wp.eps = eps; wp.qk = qk ? 1 : 0;
+  wp.kraw = F(L.kraw); wp.dkraw = F(L.dkraw); wp.g_k = reinterpret_cast<const __nv_bfloat16*>(g_k); wp.op = SB; wp.eps = eps; wp.qk = qk ? 1 : 0; wp.terms = terms; wp.term_stride = (long long)kWideTermRows * 2 * d;
   // partial sums of out[B, n_out] = A[B, k] W[n_out, k]^T; *splits of them
   auto wide_partial = [&](const __nv_bfloat16* A, const __nv_bfloat16* W, int n_out, int k, int* splits) -> cudaError_t {
     DenseParams dp;
@@ -1675,7 +1684,7 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   WideBwdParams wl;
   memset(&wl, 0, sizeof(wl));
   if (wide_loop) {
-    wl.B = B; wl.d = d; wl.H = H; wl.dff = f; wl.z_norm = z_norm ? 1 : 0; wl.pre = pre ? 1 : 0; wl.eps = eps; wl.alpha = alpha;
+    wl.B = B; wl.terms = terms; wl.d = d; wl.H = H; wl.dff = f; wl.z_norm = z_norm ? 1 : 0; wl.pre = pre ? 1 : 0; wl.eps = eps; wl.alpha = alpha;
     wl.wkvT = WkT; wl.wdnT = WdnT; wl.wupT = WupT; wl.woT = WoT; wl.g_kv = g_kv; wl.g_mlp = g_mlp;
     wl.z = z; wl.z_bs = xbs; wl.z_ts = xts; wl.dz = dz; wl.dz_bs = xbs; wl.dz_ts = xts; wl.h = F(L.h); wl.act = F(L.act);
     wl.dr = F(L.dr); wl.Gz = F(L.Gz); wl.dpre = F(L.dpre); wl.du = F(L.du); wl.dh = F(L.dh); wl.dc = F(L.dc);

@@ -39,31 +39,51 @@ __device__ __forceinline__ float group_sum(float v) {          // over the eight
   return v;
 }
 
-// qkRMS backward of dk of one (position, sequence, head) and the bf16 operand row [dk_raw | dv] of the next product; a group of eight
+// Operand rows of the tensor-core products: one bf16 value per entry, or (terms = 3) three whose sum is the fp32 value to 2^-24, at rows
+// term_stride apart.
+struct WidePair { const float* kraw; float* dkraw; const __nv_bfloat16* g_k; __nv_bfloat16* op; float eps; int qk, terms; long long term_stride; };      // op [B][2 d]
+__device__ __forceinline__ unsigned split_pair(float& a, float& b) {       // bf16 of both, which keep the rest
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  const unsigned w = *reinterpret_cast<const unsigned*>(&v);
+  a -= __uint_as_float(w << 16); b -= __uint_as_float(w & 0xffff0000u);
+  return w;
+}
+__device__ __forceinline__ void store_operand8(__nv_bfloat16* at, F8 x, int terms, long long term_stride) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (k >= terms) break;
+    unsigned w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) w[e] = split_pair(x.v[2 * e], x.v[2 * e + 1]);
+    *reinterpret_cast<uint4*>(at + k * term_stride) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+__device__ __forceinline__ void store_operand4(__nv_bfloat16* at, float a, float b, float c, float d, int terms, long long term_stride) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (k >= terms) break;
+    const unsigned lo = split_pair(a, b), hi = split_pair(c, d);
+    *reinterpret_cast<uint2*>(at + k * term_stride) = make_uint2(lo, hi);
+  }
+}
+// qkRMS backward of dk of one (position, sequence, head) and the operand row [dk_raw | dv] of the next product; a group of eight
 // lanes, eight entries each; all lanes of the warp take part, those that are not live store nothing.
-__device__ __forceinline__ void pair_operand(const F8& dk, const F8& dv, const F8& u, const __nv_bfloat16* g_k, int h, int t, float eps, int qk, float* dkraw,
-                                             __nv_bfloat16* op_k, __nv_bfloat16* op_v, bool live) {
+__device__ __forceinline__ void pair_operand(const F8& dk, const F8& dv, const F8& u, const WidePair& w, int b, int d, int h, int t, float* dkraw, bool live) {
   F8 r = dk;
-  if (qk) {
+  if (w.qk) {
     F8 ty;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) ty.v[e] = dk.v[e] * gain_at(g_k, h * kHeadDim + 8 * t + e);
+    for (int e = 0; e < 8; ++e) ty.v[e] = dk.v[e] * gain_at(w.g_k, h * kHeadDim + 8 * t + e);
     const float ss = group_sum(dot8(u, u)), tu = group_sum(dot8(ty, u));
-    const float inv = rsqrtf(ss / kHeadDim + eps), mean = tu * inv / kHeadDim;
+    const float inv = rsqrtf(ss / kHeadDim + w.eps), mean = tu * inv / kHeadDim;
 #pragma unroll
     for (int e = 0; e < 8; ++e) r.v[e] = inv * (ty.v[e] - u.v[e] * inv * mean);
   }
   if (!live) return;
   st8(dkraw, r);
-  unsigned a[4], b[4];
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const __nv_bfloat162 x = __floats2bfloat162_rn(r.v[2 * e], r.v[2 * e + 1]), y = __floats2bfloat162_rn(dv.v[2 * e], dv.v[2 * e + 1]);
-    a[e] = *reinterpret_cast<const unsigned*>(&x); b[e] = *reinterpret_cast<const unsigned*>(&y);
-  }
-  *reinterpret_cast<uint4*>(op_k) = make_uint4(a[0], a[1], a[2], a[3]);
-  *reinterpret_cast<uint4*>(op_v) = make_uint4(b[0], b[1], b[2], b[3]);
+  __nv_bfloat16* op = w.op + (long long)b * 2 * d + h * kHeadDim + 8 * t;
+  store_operand8(op, r, w.terms, w.term_stride);
+  store_operand8(op + d, dv, w.terms, w.term_stride);
 }
-struct WidePair { const float* kraw; float* dkraw; const __nv_bfloat16* g_k; __nv_bfloat16* op; float eps; int qk; };      // op [B][2 d]
 
 }  // namespace rt

@@ -223,8 +223,9 @@ struct WideFwdParams {
 };
 struct AttnBufs;
 struct WidePair;
+constexpr int kWideTermRows = 32;                // rows between the terms of a three-term operand (batches of at most 32)
 struct WideBwdParams {
-  int B, d, H, dff, z_norm, pre;
+  int B, terms, d, H, dff, z_norm, pre;
   float eps, alpha;
   const void *wkvT, *wdnT, *wupT, *woT;          // bf16 [d, 2 d], [d_ff, d], [d, d_ff], [d, d]
   const void *g_kv, *g_mlp;

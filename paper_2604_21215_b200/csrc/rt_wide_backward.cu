@@ -32,8 +32,10 @@ __device__ __forceinline__ F8 ldcg8(const float* p) {
   return F8{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
 }
 
-// CH: groups of four columns per thread of a row's four warps (d <= 512 CH)
-template <int CH>
+// CH: groups of four columns per thread of a row's four warps (d <= 512 CH).  TERMS = 3: at most 32 sequences whose operands are three bf16
+// terms each (2^-24 of the value): rows 0 .. 31, 32 .. 63 and 64 .. 95 of the row tile, so a product costs what it does anyway, and the row
+// warps add the three accumulator quadrants through their staging areas.
+template <int CH, int TERMS>
 __global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __grid_constant__ WideBwdMaps maps, const __grid_constant__ WideBwdParams p, const __grid_constant__ AttnBufs a,
                                                                      const __grid_constant__ WidePair wp) {
   extern __shared__ unsigned char smem_raw[];
@@ -113,23 +115,51 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __gri
       if (tid == 64 && ok) red_release_add_u32(c.counters + step * kWCounterStride, 1u);
       return ok;
     };
+    constexpr int kIter = TERMS == 3 ? 2 : 8;              // rows of a staged block per warp: all 32 of its own quadrant, or 8 of the 32 sequences
+    const int row_base = TERMS == 3 ? 8 * (ew & 3) : 0, row_of0 = TERMS == 3 ? 0 : quad * 32;
+    auto team_all = [&](bool ok) {                             // the four warps of a half agree (and have staged their blocks)
+      int r;
+      asm volatile("{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n barrier.cta.red.and.pred q, %2, 128, p;\n selp.b32 %0, 1, 0, q;\n}" : "=r"(r) : "r"((int)ok), "r"(2 + half) : "memory");
+      return r != 0;
+    };
+    // columns [cc, cc + 32) of the accumulator: f(sequence of the group, column of the block, values), called by every lane kIter times; false when
+    // the accumulator never came
+    auto staged = [&](bool good, int cc, auto f) {
+      if (good) wide_stage(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane, [](float v) { return v; });
+      if (TERMS == 3) good = team_all(good);
+      if (!good) return false;
+      const float* base = reinterpret_cast<const float*>(c.smem + kWStage);
+#pragma unroll
+      for (int k = 0; k < kIter; ++k) {
+        const int r = row_base + 4 * k + (lane >> 3), at = r * kWStagePitch + 4 * (lane & 7);
+        float4 v;
+        if (TERMS == 3) {                                      // quadrant q belongs to warp (q + 2) & 3 of the half
+          const float4 x = *reinterpret_cast<const float4*>(base + (2 + 4 * half) * (kWStageWarp / 4) + at), y = *reinterpret_cast<const float4*>(base + (3 + 4 * half) * (kWStageWarp / 4) + at),
+                       z = *reinterpret_cast<const float4*>(base + (0 + 4 * half) * (kWStageWarp / 4) + at);
+          v = make_float4(x.x + (y.x + z.x), x.y + (y.y + z.y), x.z + (y.z + z.z), x.w + (y.w + z.w));
+        } else {
+          v = *reinterpret_cast<const float4*>(stage + at);
+        }
+        f(k, row_of0 + r, 4 * (lane & 7), v);
+      }
+      if (TERMS == 3) team_all(true);                          // (read before the next block is staged)
+      return true;
+    };
     // a product whose sums (or parts of them) go to memory as they are: out[split][row][column]
     auto plain_product = [&](const WideStage& st, float* out) {
       bool good = flag_wait();
 #pragma unroll 1
       for (int job = c.rank; job < st.tiles * st.splits; job += c.G) {
         const int n0 = (job % st.tiles) * st.bn, split = job / st.tiles;
-        if (!good || !(good = acc_wait())) break;
+        if (good) good = acc_wait();
 #pragma unroll 1
         for (int cc = half * (st.bn >> 1); cc < (half + 1) * (st.bn >> 1); cc += 32) {
-          wide_stage(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane, [](float v) { return v; });
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const int r = 4 * k + (lane >> 3), col = 4 * (lane & 7);
-            const float4 v = *reinterpret_cast<const float4*>(stage + r * kWStagePitch + col);
-            if (quad * 32 + r < R) *reinterpret_cast<float4*>(out + ((size_t)split * p.B + m0 + quad * 32 + r) * d + n0 + cc + col) = v;
-          }
+          const bool done = staged(good, cc, [&](int, int rr, int col, const float4& v) {
+            if (rr < R) *reinterpret_cast<float4*>(out + ((size_t)split * p.B + m0 + rr) * d + n0 + cc + col) = v;
+          });
+          good = good && done;
         }
+        if (!good) break;
         acc_done();
       }
       return good;
@@ -214,7 +244,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __gri
 #pragma unroll
           for (int e = 0; e < 4; ++e) r[e] = av[k][e] + (enable ? inv * (dy[k][e] - uv[k][e] * inv * mean) : dy[k][e]);
           *reinterpret_cast<float4*>(out + at + n) = make_float4(r[0], r[1], r[2], r[3]);
-          *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.s16) + at + n) = make_uint2(pack2(r[0] * p.alpha, r[1] * p.alpha), pack2(r[2] * p.alpha, r[3] * p.alpha));
+          store_operand4(reinterpret_cast<__nv_bfloat16*>(p.s16) + at + n, r[0] * p.alpha, r[1] * p.alpha, r[2] * p.alpha, r[3] * p.alpha, TERMS, (long long)kWideTermRows * d);
         }
       }
       return true;
@@ -287,12 +317,12 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __gri
         for (int job = c.rank; job < st.tiles; job += c.G) {
           const int n0 = job * st.bn;
           const int cols = st.bn >> 1;                          // 32 or 64 of this warp; GELU' is ready before the accumulators are
-          float4 xv[2][8];
+          float4 xv[2][kIter];
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              const int rr = quad * 32 + 4 * k + (lane >> 3);
+            for (int k = 0; k < kIter; ++k) {
+              const int rr = row_of0 + row_base + 4 * k + (lane >> 3);
               if (32 * q < cols) xv[q][k] = *reinterpret_cast<const float4*>(p.act + of + (size_t)(m0 + (rr < R ? rr : 0)) * p.dff + n0 + half * cols + 32 * q + 4 * (lane & 7));
             }
           }
@@ -300,27 +330,26 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __gri
           for (int q = 0; q < 2; ++q) {
             if (32 * q >= cols) break;
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
+            for (int k = 0; k < kIter; ++k)
               xv[q][k] = make_float4(gelu_grad_wide(xv[q][k].x), gelu_grad_wide(xv[q][k].y), gelu_grad_wide(xv[q][k].z), gelu_grad_wide(xv[q][k].w));
           }
-          if (!good || !(good = acc_wait())) break;
+          if (good) good = acc_wait();
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
             if (32 * q >= cols) break;
             const int cc = half * cols + 32 * q;
-            wide_stage(stage, t_row + (uint32_t)((jobs & 1) * kWBuf + cc), lane, [](float v) { return v; });
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              const int r = 4 * k + (lane >> 3);
-              const float4 v = *reinterpret_cast<const float4*>(stage + r * kWStagePitch + 4 * (lane & 7)), x = xv[q][k];
+            const bool done = staged(good, cc, [&](int k, int rr, int col, const float4& v) {
+              const float4 x = xv[q][k];
               const float4 o = make_float4(v.x * x.x, v.y * x.y, v.z * x.z, v.w * x.w);
-              if (quad * 32 + r < R) {
-                const size_t at = (size_t)(m0 + quad * 32 + r) * p.dff + n0 + cc + 4 * (lane & 7);
+              if (rr < R) {
+                const size_t at = (size_t)(m0 + rr) * p.dff + n0 + cc + col;
                 *reinterpret_cast<float4*>(p.dpre + of + at) = o;
-                *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.p16) + at) = make_uint2(pack2(o.x, o.y), pack2(o.z, o.w));
+                store_operand4(reinterpret_cast<__nv_bfloat16*>(p.p16) + at, o.x, o.y, o.z, o.w, TERMS, (long long)kWideTermRows * p.dff);
               }
-            }
+            });
+            good = good && done;
           }
+          if (!good) break;
           acc_done();
         }
         ok = finish(good, B_DOWN);
@@ -369,8 +398,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_backward_kernel(const __gri
 #pragma unroll
             for (int e = 0; e < 8; ++e) { gk.v[e] = fmaf(ds, q.v[e], gk.v[e]); gv.v[e] = fmaf(pr, dc.v[e], gv.v[e]); }
             if (live) { st8(a.dK + rj, gk); st8(a.dV + rj, gv); }
-            __nv_bfloat16* op = wp.op + (size_t)b * 2 * d + h * kHeadDim + 8 * t8;
-            pair_operand(gk, gv, kr, wp.g_k, h, t8, wp.eps, wp.qk, wp.dkraw + rj, op, op + d, live);
+            pair_operand(gk, gv, kr, wp, b, d, h, t8, wp.dkraw + rj, live);
           }
           if (live && t8 == 0) a.D[si] = D;
         }
@@ -392,7 +420,7 @@ cudaError_t wide_backward_launch(WideBwdParams p, const AttnBufs& a, const WideP
   const int groups = wide_backward_groups(p.B, p.d, p.dff);
   if (!groups) return cudaErrorInvalidValue;
   p.R = ceil_div(p.B, groups); p.G = kB200Sms / groups;
-  const int box = (p.R + 7) / 8 * 8;
+  const int box = p.terms == 3 ? 3 * kWideTermRows : (p.R + 7) / 8 * 8, rows = p.terms == 3 ? box : p.B;
   p.a_bytes = box * 128;
   p.st[0] = stage_split(p.d, 2 * p.d, p.G, p.a_bytes);
   p.st[1] = stage_whole(p.dff, p.d, p.G, p.a_bytes, 128);
@@ -402,8 +430,9 @@ cudaError_t wide_backward_launch(WideBwdParams p, const AttnBufs& a, const WideP
   const void *A[4] = {wp.op, p.s16, p.p16, p.s16}, *W[4] = {p.wkvT, p.wdnT, p.wupT, p.woT};
   const int K[4] = {2 * p.d, p.d, p.dff, p.d}, N[4] = {p.d, p.dff, p.d, p.d};
   for (int i = 0; i < 4; ++i)
-    if (!map_blocks(&m.a[i], A[i], p.B, K[i], box) || !map_blocks(&m.w[i], W[i], N[i], K[i], p.st[i].bn)) return cudaErrorInvalidValue;
-  const void* fn = p.d <= 1024 ? reinterpret_cast<const void*>(&wide_backward_kernel<2>) : reinterpret_cast<const void*>(&wide_backward_kernel<8>);
+    if (!map_blocks(&m.a[i], A[i], rows, K[i], box) || !map_blocks(&m.w[i], W[i], N[i], K[i], p.st[i].bn)) return cudaErrorInvalidValue;
+  const void* fn = p.terms == 3 ? (p.d <= 1024 ? reinterpret_cast<const void*>(&wide_backward_kernel<2, 3>) : reinterpret_cast<const void*>(&wide_backward_kernel<8, 3>))
+                                : (p.d <= 1024 ? reinterpret_cast<const void*>(&wide_backward_kernel<2, 1>) : reinterpret_cast<const void*>(&wide_backward_kernel<8, 1>));
   const int smem = (int)kWTotal + 1024;
   cudaError_t e = ensure_dynamic_smem(fn, smem);
   if (e != cudaSuccess) return e;

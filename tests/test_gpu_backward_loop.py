@@ -1,6 +1,7 @@
-"""The reverse loop of the backward pass at the edges of its kernels, bf16, against the gradient oracle (fp64): one launch per leaf for
-up to 32 sequences (slices of one to eight sequences, narrow widths where CTAs own no columns, leaves of 1, 63, 64 and 65 positions)
-and, above, dense products over the batch (leaves of 16 positions; batches off the 128-row tiles; one to eight parts per contraction).
+"""The reverse loop of the backward pass at the edges of its kernels, bf16, against the gradient oracle (fp64): mat-vecs of up
+to eight sequences (narrow widths where CTAs own no columns, leaves of 1, 63, 64 and 65 positions; slices of a larger batch), three-term dense
+products of 9 to 32 sequences and, above, dense products over the batch (leaves of 16 positions; batches off the 128-row tiles; one to eight
+parts per contraction).
 
 Tolerance: every product takes bf16 operands or a three-term bf16 split and accumulates in fp32, so a gradient carries a few roundings of
 2^-9 relative to its largest entries; 2e-2 is that of the other backward tests."""
@@ -49,6 +50,9 @@ def _check(d, H, dff, B, N, flags, gains, alibi, alpha):
     (128, 2, 256, 9, 70, 1, ("g_kv",), False, 1.0),
     (320, 5, 960, 16, 33, 3, (), True, 0.7),
     (128, 2, 384, 32, 20, 0, (), False, 1.0),
+    (192, 3, 768, 12, 30, 3, (), False, 1.0),
+    (256, 4, 512, 24, 35, 3 | 8, G_NAMES, True, 1.0),
+    (1024, 16, 4096, 17, 6, 3, ("g_attn",), False, 1.0),
     (1024, 16, 4096, 3, 9, 3, ("g_attn",), False, 1.0)])
 def test_loop_of_up_to_32_sequences(d, H, dff, B, N, flags, gains, alibi, alpha):
     _check(d, H, dff, B, N, flags, gains, alibi, alpha)
