@@ -106,11 +106,11 @@ size_t rt_workspace_bytes(const rt_config *cfg, int32_t B, int32_t N, int32_t n_
 
 /* One RT layer over x[B,N,d] (Sec. 2.2; Algorithm 1).  Writes z[B,N,d] and rows [0,N) of
  * k_cache / v_cache [N_max,B,d] (Eqs. 1-2).  N_max >= N.
- * Batch sizes (tiled schedule): B <= 16 in bf16 takes the persistent tensor-core leaf kernel; 17 <= B <= 48 in bf16
- * runs as 2 or 3 slices of at most 16 sequences through that kernel, leaf by leaf (the sequences are independent),
- * sharing the pre-pass and the cross tiles; larger batches run each token step as dense products over the batch
- * (bf16 from B = 49, fp32 from B = 65: the regime of the paper's own experiments, Sec. 6).  fp32 up to B = 64, the
- * naive schedule and decode up to B = 64 take a generic kernel.
+ * Batch sizes (tiled schedule): B <= 16 in bf16 takes the persistent tensor-core leaf kernel (small layers of either
+ * type a kernel inside thread-block clusters); 17 <= B <= 64 in bf16 runs as slices of at most 16 sequences side by side
+ * on groups of SMs (the sequences are independent), sharing the pre-pass and the cross tiles; larger batches run each
+ * token step as dense products over the batch (the regime of the paper's own experiments, Sec. 6).  fp32 up to B = 64,
+ * the naive schedule and decode up to B = 64 take a generic kernel.
  * The naive schedule and the decode entry points return RT_ERR_UNSUPPORTED for B > 64. */
 rt_status rt_layer_prefill(const rt_config *cfg, const rt_layer_weights *w,
                            const void *x, int32_t B, int32_t N,
@@ -236,9 +236,10 @@ rt_status rt_layer_recompute(const rt_config *cfg, const rt_layer_weights *w, co
  * accumulating only d(k_j, v_j) -- position i needs dL/dz_i, which needs d(k_i, v_i) complete; pairs in other leaves
  * of 64 positions receive their share from Algorithm 1's tiles run backwards -- and finally forms dq, the temporary
  * pairs, dx and every parameter gradient as products over all B*N rows at once.
- * Batches above 32 sequences run each step of the reverse loop as dense products over the batch (Sec. 6's regime).
- * The reverse loop and the attention terms are fp32 on CUDA cores; with bf16 storage the products over all rows run
- * on the tensor cores (operands rounded to bf16, fp32 accumulation).  recur_block > 1 returns RT_ERR_UNSUPPORTED.
+ * With bf16 storage the reverse loop runs on the tensor cores: up to 32 sequences with operands kept to 2^-24 (three
+ * bf16 terms), above (Sec. 6's regime, dense products over the batch) with operands rounded to bf16; the products over
+ * all rows round their operands to bf16 too.  Accumulation is fp32 throughout; the attention terms and everything with
+ * fp32 storage are fp32 on CUDA cores.  recur_block > 1 returns RT_ERR_UNSUPPORTED.
  * The workspace needs rt_backward_workspace_bytes (about 40 fp32 arrays of B*N*d plus 4 of B*N*d_ff: 1.1 GB at B=4, N=2048, d=768; 48 GB at B=N=512, d=1024). */
 typedef struct {
   float *w_q, *w_k, *w_v, *w_o, *w_up, *w_down;   /* shapes of rt_layer_weights */
