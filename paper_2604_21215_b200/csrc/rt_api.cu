@@ -583,7 +583,9 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
   for (int wave = 0, waves = start[n_layers - 1] + n_leaves; wave < waves; ++wave) {
     GroupJob jobs[kGroupJobs];
     memset(jobs, 0, sizeof(jobs));
-    int nj = 0;
+    int nj = 0, np = 0;
+    PrepassParams pre[kGroupJobs];
+    int layer_of[kGroupJobs];
     for (int l = 0; l < n_layers; ++l) {
       const int k = wave - start[l];
       if (k < 0 || k >= n_leaves) continue;
@@ -591,17 +593,25 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
       const int place = l % places, t0 = k * wv.leaf, t1 = t0 + wv.leaf < N ? t0 + wv.leaf : N;
       unsigned char* rows = ws + L.wave + L.wave_stride * place;
       const void* x = hid[l & 1];
-      PrepassParams pp;
+      PrepassParams& pp = pre[np];
       memset(&pp, 0, sizeof(pp));
+      layer_of[np++] = l;
       pp.B = B; pp.N = t1 - t0; pp.d = c->d_model; pp.H = c->n_heads; pp.norm_flags = c->norm_flags; pp.eps = c->rms_eps; pp.scale_log2 = gc.scale_log2;
       pp.x = (const unsigned char*)x + (size_t)t0 * d * e; pp.x_bs = bs; pp.x_ts = (long long)d;
       pp.w_q = w.w_q; pp.w_k = w.w_k; pp.w_v = w.w_v; pp.g_attn = w.g_attn; pp.g_q = w.g_q; pp.g_k = w.g_k;
       pp.n = rows + W.n; pp.q = rows + W.q; pp.kt = rows + W.kt; pp.vt = rows + W.vt;
       pp.st_o = (float*)(rows + W.st_o); pp.st_m = (float*)(rows + W.st_m); pp.st_l = (float*)(rows + W.st_l); pp.sync = gc.sync;
-      {
-        ProfScope ps(s, kProfPrepass);
-        if (prepass_launch(c->dtype, pp, s) != cudaSuccess) return RT_ERR_CUDA;
-      }
+    }
+    {
+      ProfScope ps(s, kProfPrepass);
+      if (prepass_batch_launch(c->dtype, pre, np, s) != cudaSuccess) return RT_ERR_CUDA;
+    }
+    for (int i = 0; i < np; ++i) {
+      const int l = layer_of[i];
+      const PrepassParams& pp = pre[i];
+      const rt_layer_weights& w = layers[l];
+      const int k = wave - start[l], place = l % places, t0 = k * wv.leaf, t1 = t0 + wv.leaf < N ? t0 + wv.leaf : N;
+      const void* x = hid[l & 1];
       GroupJob& j = jobs[nj++];
       j.key0 = 0;
       if (t0 >= kWaveFoldMax) {

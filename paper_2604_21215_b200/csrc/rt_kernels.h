@@ -134,9 +134,14 @@ struct PrepassParams {
   SyncArea* sync;
 };
 cudaError_t prepass_launch(int dtype, const PrepassParams& p, cudaStream_t s);
+// The pre-passes of up to kPrepassBatch layers' rows together (same B, d and flags): three launches for all of them.
+constexpr int kPrepassBatch = 4;
+struct PrepassBatch { PrepassParams p[kPrepassBatch]; };
+cudaError_t prepass_batch_launch(int dtype, const PrepassParams* p, int n, cudaStream_t s);
 // tensor-core projection (bf16, d a multiple of 128)
 bool qkv_gemm_tc_supported(const PrepassParams& p);
 cudaError_t qkv_gemm_tc_launch(const PrepassParams& p, SyncArea* sync, cudaStream_t s);
+cudaError_t qkv_gemm_tc_batch_launch(const PrepassBatch& b, int n, int rows_max, SyncArea* sync, cudaStream_t s);
 
 // Cross-block tile (Algorithm 2 on a [q0,q1) x [k0,k1) block for every sequence and head).
 struct TileParams {

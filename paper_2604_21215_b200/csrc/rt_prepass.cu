@@ -14,8 +14,7 @@ namespace rt {
 
 // ---- n = RMS(x) (or a copy when pre-norm is off), position-major rows m = r*B + b ----------
 template <typename T>
-__global__ void rms_rows_kernel(const PrepassParams p) {
-  grid_dep_sync();
+__device__ __forceinline__ void rms_rows(const PrepassParams& p) {
   const int lane = threadIdx.x & 31;
   const int m = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (m >= p.N * p.B) return;
@@ -29,6 +28,16 @@ __global__ void rms_rows_kernel(const PrepassParams p) {
   const bool pre = (p.norm_flags & RT_NORM_PRE) != 0;
   const float rs = pre ? rsqrtf(ss / (float)p.d + p.eps) : 1.0f;
   for (int k = lane; k < p.d; k += 32) out[k] = from_f<T>(to_f(xr[k]) * rs * (pre ? gain_at(g, k) : 1.0f));
+}
+
+template <typename T>
+__global__ void rms_rows_kernel(const PrepassParams p) {
+  grid_dep_sync();
+  rms_rows<T>(p);
+}
+__global__ void rms_rows_batch_kernel(const __grid_constant__ PrepassBatch b) {
+  grid_dep_sync();
+  rms_rows<__nv_bfloat16>(b.p[blockIdx.z]);
 }
 
 // ---- SIMT projection: C[m, col] = sum_k n[m,k] W[col,k], one head (64 columns) per CTA -----
@@ -115,7 +124,7 @@ __global__ void __launch_bounds__(256) qkv_gemm_simt_kernel(const PrepassParams 
 
 // ---- running stats seeded with the temporary pair ------------------------------------------
 template <typename T>
-__global__ void state_init_kernel(const PrepassParams p) {
+__device__ __forceinline__ void state_init(const PrepassParams& p) {
   const int lane = threadIdx.x & 31;
   const long long u = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);   // (m, h)
   const long long total = (long long)p.N * p.B * p.H;
@@ -132,6 +141,13 @@ __global__ void state_init_kernel(const PrepassParams p) {
     p.st_m[u] = dot * p.scale_log2;
     p.st_l[u] = 1.0f;
   }
+}
+
+template <typename T>
+__global__ void state_init_kernel(const PrepassParams p) { state_init<T>(p); }
+__global__ void state_init_batch_kernel(const __grid_constant__ PrepassBatch b) {
+  grid_dep_sync();
+  state_init<__nv_bfloat16>(b.p[blockIdx.z]);
 }
 
 template <typename T>
@@ -153,6 +169,31 @@ static cudaError_t prepass_typed(const PrepassParams& p, cudaStream_t s) {
     state_init_kernel<T><<<(unsigned)((units + 7) / 8), 256, 0, s>>>(p);
   }
   return cudaGetLastError();
+}
+
+// The few rows of a leaf keep a launch busy for a few microseconds only: the layers of a wave share theirs, chained (8 layers, B = 1,
+// N = 77: 40 pre-passes of three launches took 1.29 of 5.4 ms).
+cudaError_t prepass_batch_launch(int dtype, const PrepassParams* p, int n, cudaStream_t s) {
+  int rows = 0;
+  bool together = dtype == RT_BF16 && n > 0 && n <= kPrepassBatch;
+  for (int i = 0; i < n; ++i) {
+    const int m = p[i].N * p[i].B;
+    if (m > rows) rows = m;
+    together = together && qkv_gemm_tc_supported(p[i]) && !dense_qkv_pair_supported(m, p[i].d) && !p[i].mats && !p[i].skip_rms && !p[i].no_seed;
+  }
+  if (!together) {
+    for (int i = 0; i < n; ++i) {
+      const cudaError_t e = prepass_launch(dtype, p[i], s);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
+  PrepassBatch b;
+  for (int i = 0; i < kPrepassBatch; ++i) b.p[i] = p[i < n ? i : 0];
+  cudaError_t e = launch_chained(rms_rows_batch_kernel, dim3(ceil_div(rows, 8), 1, n), dim3(256), 0, s, true, b);
+  if (e == cudaSuccess) e = qkv_gemm_tc_batch_launch(b, n, rows, p[0].sync, s);
+  if (e == cudaSuccess) e = launch_chained(state_init_batch_kernel, dim3((unsigned)(((long long)rows * p[0].H + 7) / 8), 1, n), dim3(256), 0, s, true, b);
+  return e;
 }
 
 cudaError_t prepass_launch(int dtype, const PrepassParams& p, cudaStream_t s) {

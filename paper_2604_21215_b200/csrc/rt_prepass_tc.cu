@@ -35,11 +35,8 @@ struct GemmSmemT {
 };
 
 template <int BN>
-__global__ void __launch_bounds__(kGemmThreads, 2)
-qkv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_n, const __grid_constant__ CUtensorMap map_wq,
-                   const __grid_constant__ CUtensorMap map_wk, const __grid_constant__ CUtensorMap map_wv,
-                   const PrepassParams p, SyncArea* sync) {
-  grid_dep_sync();
+__device__ __forceinline__ void qkv_gemm_tc(const CUtensorMap& map_n, const CUtensorMap& map_wq, const CUtensorMap& map_wk, const CUtensorMap& map_wv, const PrepassParams& p,
+                                            SyncArea* sync) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(smem);
@@ -174,6 +171,23 @@ qkv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_n, const __grid_const
   }
 }
 
+template <int BN>
+__global__ void __launch_bounds__(kGemmThreads, 2)
+qkv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_n, const __grid_constant__ CUtensorMap map_wq, const __grid_constant__ CUtensorMap map_wk,
+                   const __grid_constant__ CUtensorMap map_wv, const __grid_constant__ PrepassParams p, SyncArea* sync) {
+  grid_dep_sync();
+  qkv_gemm_tc<BN>(map_n, map_wq, map_wk, map_wv, p, sync);
+}
+struct QkvMaps { CUtensorMap n, wq, wk, wv; };
+struct QkvMapsBatch { QkvMaps m[kPrepassBatch]; };
+template <int BN>
+__global__ void __launch_bounds__(kGemmThreads, 2)
+qkv_gemm_tc_batch_kernel(const __grid_constant__ QkvMapsBatch maps, const __grid_constant__ PrepassBatch b, SyncArea* sync) {
+  grid_dep_sync();
+  const QkvMaps& m = maps.m[blockIdx.z];
+  qkv_gemm_tc<BN>(m.n, m.wq, m.wk, m.wv, b.p[blockIdx.z], sync);
+}
+
 static_assert(kGemmBK == 64, "tensor_map_rows_bf16 encodes 64-column boxes");
 
 bool qkv_gemm_tc_supported(const PrepassParams& p) { return p.d % 128 == 0 && p.d >= 128; }
@@ -206,6 +220,22 @@ cudaError_t qkv_gemm_tc_launch(const PrepassParams& p, SyncArea* sync, cudaStrea
   };
   if (bn == 64) return run(qkv_gemm_tc_kernel<64>, GemmSmemT<64>::total + 1024);
   return run(qkv_gemm_tc_kernel<128>, GemmSmemT<128>::total + 1024);
+}
+
+cudaError_t qkv_gemm_tc_batch_launch(const PrepassBatch& b, int n, int rows_max, SyncArea* sync, cudaStream_t s) {
+  const int d = b.p[0].d;
+  QkvMapsBatch maps;
+  for (int i = 0; i < kPrepassBatch; ++i) {
+    const PrepassParams& p = b.p[i];
+    QkvMaps& m = maps.m[i];
+    if (!tensor_map_rows_bf16(&m.n, p.n, p.N * p.B, d, kBM) || !tensor_map_rows_bf16(&m.wq, p.w_q, d, d, 64) || !tensor_map_rows_bf16(&m.wk, p.w_k, d, d, 64) ||
+        !tensor_map_rows_bf16(&m.wv, p.w_v, d, d, 64))
+      return cudaErrorInvalidValue;
+  }
+  const size_t smem = GemmSmemT<64>::total + 1024;
+  const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(&qkv_gemm_tc_batch_kernel<64>), (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_chained(qkv_gemm_tc_batch_kernel<64>, dim3(ceil_div(rows_max, kBM), 3 * (d / 64), n), dim3(kGemmThreads), smem, s, true, maps, b, sync);
 }
 
 }  // namespace rt
