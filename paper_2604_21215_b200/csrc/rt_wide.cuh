@@ -18,7 +18,7 @@ constexpr int kWBuf = 128;                                 // TMEM columns per a
 constexpr int kWCounterStride = 32;                        // unsigned words between counters
 constexpr int kWMaxSteps = 8;
 
-__device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ bool epi_all(bool ok) {         // barrier of the eight row warps; true when all of them are fine
   int r;
   asm volatile("{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n barrier.cta.red.and.pred q, 1, 256, p;\n selp.b32 %0, 1, 0, q;\n}" : "=r"(r) : "r"((int)ok) : "memory");
