@@ -18,7 +18,7 @@ constexpr int kSmallBatchMax = 64;      // above this the per-token chain runs a
 constexpr int kAutoLeaf = 64;
 
 struct WsLayout {
-  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, dec_words, ll, ll_bytes, grp, packed, wave, wave_stride, hid0, hid1,
+  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, dec_words, ll, ll_bytes, gx, grp, packed, wave, wave_stride, hid0, hid1,
       blk_h, blk_u, blk_c, blk_g, total;
 };
 
@@ -141,13 +141,14 @@ WsLayout ws_layout(const rt_config* c, int B, int N, int n_layers) {
   // exchange area of the decode kernel (a decode step is a call with N = 1, of any workspace at least that large)
   L.dec_words = take(c->dtype == RT_BF16 && B <= kSmallBatchMax ? decode_words_bytes(n_layers, decode_slice(B), (int)d, (int)H, (int)f) : 0);
   // exchange buffers of the tensor-core leaf kernel: c, h, z as flag-carrying words (16 sequence slots each),
-  // g as packed bf16 in fragment order (16 sequence slots), raw k|v as flag-carrying fp32 words
-  L.ll_bytes = ((size_t)16 * 3 * (d / 2) + (size_t)16 * (f / 4) + (size_t)B * 2 * d) * 8;
+  // raw k|v as flag-carrying fp32 words; g as packed bf16 in fragment order (16 sequence slots), an array per position of a leaf (gx)
+  L.ll_bytes = ((size_t)16 * 3 * (d / 2) + (size_t)B * 2 * d) * 8;
   L.ll = take(L.ll_bytes);
   // group kernel: one exchange area per group of SMs, the packed weights of a layer (of every layer, when the layers of a
   // stack run side by side) and, for a stack, a leaf's rows of n, q, k~, v~ and the state per group
   const Wave wv = stack_wave(c, B, N, n_layers);
   const Schedule sch = effective_schedule(c, B);
+  L.gx = take(sch.path == kPathMma || sch.path == kPathMmaSplit ? (size_t)(sch.leaf < N ? sch.leaf : N) * 16 * f * 2 : 0);     // g of the tensor-core leaf kernel
   const bool grp = N > 1 && (wv.places || sch.path == kPathGroups);
   L.grp = take(grp ? (size_t)kGroupJobs * leaf_group_words_bytes((int)d, (int)f) : 0);
   L.packed = take(grp ? (wv.places ? (size_t)n_layers : 1) * leaf_group_packed_bytes((int)d, (int)f, wv.places ? wv.places : ceil_div(B, sch.sub)) : 0);
@@ -483,8 +484,8 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   {
     unsigned long long* w = (unsigned long long*)(ws + L.ll);
     const size_t bd2 = (size_t)16 * (c->d_model / 2);
-    mb.ll_c = w; mb.ll_h = w + bd2; mb.ll_z = w + 2 * bd2; mb.ll_g = w + 3 * bd2;
-    mb.ll_kv = mb.ll_g + (size_t)16 * (c->d_ff / 4);
+    mb.ll_c = w; mb.ll_h = w + bd2; mb.ll_z = w + 2 * bd2; mb.ll_g = (unsigned long long*)(ws + L.gx);
+    mb.ll_kv = w + 3 * bd2;
   }
   auto leaf_mma = [&](int t0, int t1) -> bool {
     ProfScope ps(s, kProfLeaf);
@@ -493,10 +494,10 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
       lp.B = B - b0 < b_sub ? B - b0 : b_sub; lp.Bs = B; lp.b0 = b0;
       lp.x = (const unsigned char*)x + (size_t)b0 * x_bs * e;
       lp.z = (unsigned char*)z + (size_t)b0 * z_bs * e;
-      lp.t0 = t0; lp.t1 = t1; lp.attn_begin = t0; lp.seq_base = ctx.seq_base; lp.bar_base = ctx.bar_base;
+      lp.t0 = t0; lp.t1 = t1; lp.attn_begin = t0; lp.seq_base = ctx.seq_base;
+      if (cudaMemsetAsync(ws + L.gx, 0xff, (size_t)(t1 - t0) * 16 * c->d_ff * 2, s) != cudaSuccess) return false;
       if (leaf_mma_launch(lp, ml, mb, s) != cudaSuccess) return false;
       ctx.seq_base += (unsigned)(t1 - t0);
-      ctx.bar_base += (unsigned)(t1 - t0) * (unsigned)ml.grid;    // one grid barrier per token step
     }
     return true;
   };

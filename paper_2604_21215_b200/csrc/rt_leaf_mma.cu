@@ -101,12 +101,14 @@ __device__ __forceinline__ uint4 ld_relaxed_v4_if(const void* p, unsigned on) {
 // 8 bytes through L2 under a predicate (zeros when `on` is zero).  An asm statement, so that a run
 // of these stays a run of loads: written as plain loads the compiler placed each one's first use
 // right behind it and the round trips added up.
-__device__ __forceinline__ uint2 ld_cg_v2_if(const void* p, unsigned on) {
-  uint2 w = make_uint2(0u, 0u);
-  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %3, 0;\n @q ld.global.cg.v2.u32 {%0,%1}, [%2];\n}"
-               : "+r"(w.x), "+r"(w.y) : "l"(p), "r"(on) : "memory");
-  return w;
+// Words that are their own flags: all ones = not written yet (no pair of bf16 results is: NaN results are 0x7fff).
+constexpr unsigned kNotYet = 0xffffffffu;
+__device__ __forceinline__ bool missing(const uint2& w) { return (w.x == kNotYet) | (w.y == kNotYet); }
+__device__ __forceinline__ void ld_relaxed_v2_missing(const void* p, uint2& w) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %3, 0;\n @q ld.relaxed.gpu.global.v2.u32 {%0,%1}, [%2];\n}"
+               : "+r"(w.x), "+r"(w.y) : "l"(p), "r"(missing(w) ? 1u : 0u) : "memory");
 }
+__device__ __forceinline__ void st_relaxed_u32(void* p, unsigned v) { asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory"); }
 __device__ __forceinline__ void st_relaxed_u64(void* p, unsigned lo, unsigned hi) {
   const unsigned long long w = ((unsigned long long)hi << 32) | lo;
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
@@ -168,22 +170,6 @@ __device__ __forceinline__ void frag_ssq_gain(unsigned (&a)[4], const __nv_bfloa
     if (r == 0) sq0 += s; else sq1 += s;
     if (gp) { a[r] = pack_bf2(v0 * gn[0], v1 * gn[1]); a[2 + r] = pack_bf2(v2 * gn[2], v3 * gn[3]); }
   }
-}
-
-// Barrier over all CTAs, run by the MMA warps only (the attention warps never wait on it).
-__device__ __forceinline__ bool mma_grid_barrier(SyncArea* sync, volatile int* s_abort, unsigned target) {
-  mma_warps_sync();
-  if (threadIdx.x == 0) {
-    // the release is cumulative over what the CTA barrier above ordered before it: no separate fence
-    red_release_add_u32(&sync->bar_count, 1u);
-    unsigned spins = 0;
-    unsigned long long t_start = 0;
-    while (ld_acquire_u32(&sync->bar_count) < target) {
-      if ((++spins & 255u) == 0u && wait_expired(sync, t_start)) { *s_abort = 1; break; }
-    }
-  }
-  mma_warps_sync();
-  return *s_abort == 0;
 }
 
 // ---- attention warp: one (sequence, head) pair for the whole leaf ----------------------------
@@ -392,13 +378,13 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
   const __nv_bfloat16* x = reinterpret_cast<const __nv_bfloat16*>(p.x);
   __nv_bfloat16* z = reinterpret_cast<__nv_bfloat16*>(p.z);
   // g as packed bf16 in the order the fragments are read: [k-step of 16][16 sequence slots][16 k], so the
-  // 8 sequences x 32 bytes one warp-wide load touches are 256 contiguous bytes (2 lines instead of 8)
-  __nv_bfloat16* g_pk = reinterpret_cast<__nv_bfloat16*>(ll_g);
+  // 8 sequences x 32 bytes one warp-wide load touches are 256 contiguous bytes (2 lines instead of 8).  Every position of the leaf has its
+  // own array, filled with the pattern of kNotYet before the launch, so a word is its own flag and nobody waits for a barrier: the release,
+  // the count and the first load behind it were 1 to 1.5 us of a token step.
   auto g_index = [](int b, int k) -> size_t { return ((size_t)((k >> 4) * 16 + b) << 4) + (size_t)(k & 15); };
   const float inv_d = 1.0f / (float)d;
   const int nt_d = (nd + 7) / 8, nt_f = (nf + 7) / 8;
   const bool has0 = g < B, has1 = (MB == 2) && (g + 8 < B);
-  unsigned bar_target = p.bar_base;
   const bool timing = TIMERS && (cta == 0 && tid == 0);
   unsigned long long t_ph = timing ? globaltimer_ns() : 0ull;
 
@@ -410,6 +396,7 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
 
   for (int t = p.t0; t < p.t1; ++t) {
     const unsigned seq = p.seq_base + (unsigned)(t - p.t0) + 1u;
+    __nv_bfloat16* g_pk = reinterpret_cast<__nv_bfloat16*>(ll_g) + (size_t)(t - p.t0) * 16 * dff;
 #pragma unroll 1
     for (int ph = 0; ph < 4; ++ph) {                              // 0: W_o   1: W_up   2: W_down   3: W_k | W_v
       // ---- what this phase multiplies ----
@@ -425,13 +412,6 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
       if (ph == 3 && kv_norm) { if (GAINS) gain = reinterpret_cast<const __nv_bfloat16*>(p.g_kv); want_ssq = true; }
       const __nv_bfloat16* gp = (GAINS && gain) ? gain + 4 * c : nullptr;
       unsigned long long wait_ns = 0;
-      if (ph == 2) {
-        // every CTA's slice of g (packed bf16) must be complete before anyone multiplies by W_down
-        bar_target += (unsigned)G;
-        const unsigned long long tb = timing ? globaltimer_ns() : 0ull;
-        if (!mma_grid_barrier(p.sync, s_abort, bar_target)) return;
-        if (timing) wait_ns += globaltimer_ns() - tb;
-      }
       const int n_ks = K / 16;
       const int ks_per_warp = (n_ks + kMmaWarps - 1) / kMmaWarps;
       const int ks0 = warp * ks_per_warp;
@@ -459,7 +439,7 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
         const int g0 = has0 ? g : 0, g1 = has1 ? g + 8 : 0;        // rows read by lanes without a sequence (masked below)
         const unsigned keep0 = has0 ? 0xffffffffu : 0u, keep1 = has1 ? 0xffffffffu : 0u;
         if (ph == 2) {
-          // W_down reads g as packed bf16 after the barrier: plain loads, and ALL of this warp's
+          // W_down reads g as packed bf16 words that are their own flags, and ALL of this warp's
           // k-steps are in flight before the first product (at d_ff = 4096: 32 k-steps, 64 loads when B > 8).  One tile per
           // pass keeps this at 32 products; the two accumulators halve the dependent chain.
           constexpr int KD = 32;
@@ -476,11 +456,35 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
             const int n_here = ks1 - kc0;
             uint2 w0[KD], w1[MB == 2 ? KD : 1];
 #pragma unroll
-            for (int i = 0; i < KD; ++i) w0[i] = ld_cg_v2_if(b0p + (size_t)(kc0 + (i < n_here ? i : 0)) * 256, (i < n_here ? 1u : 0u) & keep0);
-            if (MB == 2) {
-#pragma unroll
-              for (int i = 0; i < KD; ++i) w1[i] = ld_cg_v2_if(b1p + (size_t)(kc0 + (i < n_here ? i : 0)) * 256, (i < n_here ? 1u : 0u) & keep1);
+            for (int i = 0; i < KD; ++i) {
+              w0[i].x = w0[i].y = i < n_here ? keep0 : 0u;             // all ones: to be fetched
+              if (MB == 2) w1[i].x = w1[i].y = i < n_here ? keep1 : 0u;
             }
+            unsigned spins = 0;
+            unsigned long long t_start = 0;
+            const unsigned long long t_poll = timing ? globaltimer_ns() : 0ull;
+            while (alive) {
+#pragma unroll
+              for (int i = 0; i < KD; ++i) ld_relaxed_v2_missing(b0p + (size_t)(kc0 + (i < n_here ? i : 0)) * 256, w0[i]);
+              if (MB == 2) {
+#pragma unroll
+                for (int i = 0; i < KD; ++i) ld_relaxed_v2_missing(b1p + (size_t)(kc0 + (i < n_here ? i : 0)) * 256, w1[i]);
+              }
+              bool more = false;
+#pragma unroll
+              for (int i = 0; i < KD; ++i) more |= missing(w0[i]);
+              if (MB == 2) {
+#pragma unroll
+                for (int i = 0; i < KD; ++i) more |= missing(w1[i]);
+              }
+              if (__all_sync(0xffffffffu, !more)) break;
+              if ((++spins & 63u) == 0u) {
+                int bad = 0;
+                if (lane == 0) bad = wait_expired(p.sync, t_start) ? 1 : 0;
+                if (__shfl_sync(0xffffffffu, bad, 0)) { *s_abort = 1; alive = false; }
+              }
+            }
+            if (timing) wait_ns += globaltimer_ns() - t_poll;
 #pragma unroll
             for (int i = 0; i < KD; ++i) {
               ad[i][0] = w0[i].x; ad[i][2] = w0[i].y;
@@ -616,11 +620,11 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
           } else if (ph == 1) {                                     // g = GELU(W_up RMS(h)), packed bf16
             if (has0) {
               const float rs = pre ? rsqrtf(ssq_lo * inv_d + p.eps) : 1.0f;
-              *reinterpret_cast<unsigned*>(g_pk + g_index(g, f_lo + rl)) = pack_bf2(gelu_erf_f(y0 * rs), gelu_erf_f(y1 * rs));
+              st_relaxed_u32(g_pk + g_index(g, f_lo + rl), pack_bf2(gelu_erf_f(y0 * rs), gelu_erf_f(y1 * rs)));
             }
             if (has1) {
               const float rs = pre ? rsqrtf(ssq_hi * inv_d + p.eps) : 1.0f;
-              *reinterpret_cast<unsigned*>(g_pk + g_index(g + 8, f_lo + rl)) = pack_bf2(gelu_erf_f(y2 * rs), gelu_erf_f(y3 * rs));
+              st_relaxed_u32(g_pk + g_index(g + 8, f_lo + rl), pack_bf2(gelu_erf_f(y2 * rs), gelu_erf_f(y3 * rs)));
             }
           } else if (ph == 2) {                                     // z_t = h + alpha W_down g   (layer output)
             if (has0) {
