@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
   // g as packed bf16 in the order the fragments are read: [k-step of 16][16 sequence slots][16 k], so the
   // 8 sequences x 32 bytes one warp-wide load touches are 256 contiguous bytes (2 lines instead of 8).  Every position of the leaf has its
   // own array, filled with the pattern of kNotYet before the launch, so a word is its own flag and nobody waits for a barrier: the release,
-  // the count and the first load behind it were 1 to 1.5 us of a token step.
+  // the count and the first load behind it were 0.7 us of a token step (9.8 -> 9.1 us at B = 4, d = 768, 13.9 -> 13.2 at B = 16, d = 1024).
   auto g_index = [](int b, int k) -> size_t { return ((size_t)((k >> 4) * 16 + b) << 4) + (size_t)(k & 15); };
   const float inv_d = 1.0f / (float)d;
   const int nt_d = (nd + 7) / 8, nt_f = (nf + 7) / 8;

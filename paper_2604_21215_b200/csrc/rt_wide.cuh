@@ -18,6 +18,7 @@ constexpr int kWBuf = 128;                                 // TMEM columns per a
 constexpr int kWCounterStride = 32;                        // unsigned words between counters
 constexpr int kWMaxSteps = 8;
 
+// (for global memory only: over all state spaces the fence took 0.5 us longer, a tenth of a step)
 __device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ bool epi_all(bool ok) {         // barrier of the eight row warps; true when all of them are fine
   int r;

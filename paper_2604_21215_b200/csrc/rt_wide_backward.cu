@@ -6,7 +6,8 @@
 // R1 and R3 need sums over whole rows: four warps own a row.  In A only the newest pair, i - 1, is on the chain; the leaf's older pairs are
 // updated after the step has been counted in, by the same threads at every position.
 //
-// Measured per position at d = 1024, d_ff = 4096, B = 96: see the figures at wide_backward_launch.
+// Measured per position at d = 1024, d_ff = 4096: B = 96 36 us (63 as seven launches, 74 as fifteen), B = 512 75 (106); three-term operands B = 16 32
+// (43 in two slices of the mat-vec kernel), B = 32 33 (84 in four).  A step is about 5 us, as in the forward loop.
 #include <type_traits>
 
 #include "rt_bwd.cuh"

@@ -16,7 +16,7 @@
 // Exchange: data through global memory (L2), a counter per step and group (release by one thread after a barrier of the CTA's row warps,
 // acquire and a proxy fence by the warp that then fetches).  Every wait is bounded (2 s).
 //
-// Measured per position at d = 1024, d_ff = 4096, against the launches: B = 96 30 us (42), B = 200 (d = 768) 29 (50), B = 512 40 (57).  A step
+// Measured per position at d = 1024, d_ff = 4096, against the launches: B = 96 27.6 us (42), B = 200 (d = 768) 27 (50), B = 512 38 (57).  A step
 // is about 1 us from the last count to the first fetch, 2 to 5 us until the accumulators are complete (operand rows and weights at 145 GB/s
 // per SM, about 1.2 us of latency), 1 to 2.5 us of row work, 0.7 us for the release.
 #include <type_traits>
