@@ -67,6 +67,8 @@ def test_loop_of_up_to_32_sequences(d, H, dff, B, N, flags, gains, alibi, alpha)
     # With no norms at all this case is ill conditioned (one of the 130 sequences has gradients of 916; the fp64 oracle itself moves by 187
     # there when the weights change by up to 2^-9 of themselves), so it keeps the pre-norms; without them only half the length is used.
     (128, 2, 512, 130, 35, 1, (), False, 1.0),
-    (128, 2, 512, 130, 18, 0, (), False, 0.5)])
+    (128, 2, 512, 130, 18, 0, (), False, 0.5),
+    (256, 4, 512, 300, 20, 3, G_NAMES, True, 1.0),                           # three groups
+    (128, 2, 256, 1030, 18, 3, ("g_k", "g_kv"), False, 1.0)])                # too many groups: the launches of every position
 def test_dense_products_over_wide_batches(d, H, dff, B, N, flags, gains, alibi, alpha):
     _check(d, H, dff, B, N, flags, gains, alibi, alpha)
