@@ -18,7 +18,7 @@ constexpr int kSmallBatchMax = 64;      // above this the per-token chain runs a
 constexpr int kAutoLeaf = 64;
 
 struct WsLayout {
-  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, dec_words, ll, ll_bytes, gx, grp, packed, wave, wave_stride, hid0, hid1,
+  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, dec_words, dec_words_bytes, ll, ll_bytes, gx, grp, packed, wave, wave_stride, hid0, hid1,
       blk_h, blk_u, blk_c, blk_g, total;
 };
 
@@ -116,9 +116,6 @@ WaveRows wave_rows_layout(const rt_config* c, int B, int leaf) {
   return W;
 }
 
-// Sequences per launch of the decode kernel: a batch above 16 runs as slices of equal size (the sequences are independent).
-int decode_slice(int B) { return ceil_div(B, ceil_div(B, 16)); }
-
 WsLayout ws_layout(const rt_config* c, int B, int N, int n_layers) {
   WsLayout L;
   const size_t e = esize_of(c->dtype), d = c->d_model, H = c->n_heads, f = c->d_ff;
@@ -139,7 +136,8 @@ WsLayout ws_layout(const rt_config* c, int B, int N, int n_layers) {
   L.ex_k = take((size_t)B * d * 4);
   L.ex_part = take((size_t)B * H * kMaxChunks * 68 * 4);
   // exchange area of the decode kernel (a decode step is a call with N = 1, of any workspace at least that large)
-  L.dec_words = take(c->dtype == RT_BF16 && B <= kSmallBatchMax ? decode_words_bytes(n_layers, decode_slice(B), (int)d, (int)H, (int)f) : 0);
+  L.dec_words_bytes = c->dtype == RT_BF16 && B <= kSmallBatchMax ? decode_words_bytes(n_layers, B, (int)d, (int)H, (int)f) : 0;
+  L.dec_words = take(L.dec_words_bytes);
   // exchange buffers of the tensor-core leaf kernel: c, h, z as flag-carrying words (16 sequence slots each),
   // raw k|v as flag-carrying fp32 words; g as packed bf16 in fragment order (16 sequence slots), an array per position of a leaf (gx)
   L.ll_bytes = ((size_t)16 * 3 * (d / 2) + (size_t)B * 2 * d) * 8;
@@ -654,7 +652,7 @@ rt_status run_decode(const rt_config* c, int n_layers, const rt_layer_weights* l
     p.B = B - b0 < sub ? B - b0 : sub; p.Bs = B; p.b0 = b0;
     p.d = d; p.H = c->n_heads; p.dff = c->d_ff; p.pos = pos;
     p.norm_flags = c->norm_flags; p.eps = c->rms_eps; p.scale_log2 = c->softmax_scale * kLog2e; p.alpha = c->residual_scale;
-    p.words = ws + L.dec_words; p.sync = (SyncArea*)(ws + L.sync);
+    p.words = ws + L.dec_words; p.words_size = L.dec_words_bytes; p.sync = (SyncArea*)(ws + L.sync);
     for (int l0 = 0; l0 < n_layers; l0 += kDecMaxLayers) {
       const bool to_z = l0 + kDecMaxLayers >= n_layers;
       const size_t off = (size_t)b0 * 2;

@@ -757,10 +757,15 @@ int seg_bound(int quads, int grid) { return ceil_div(grid, quads) + 2; }
 
 }  // namespace
 
+int decode_slice(int B) { return ceil_div(B, ceil_div(B, 16)); }
+
+// The largest area that one of the batch's slices asks for.  That need not be the fullest slice: a smaller one has fewer groups of four pairs,
+// hence more partial states for each pair (d = 128, H = 2: 17 sequences are slices of 9 and 8, and the 8 need 10 KB a layer more).
 size_t decode_words_bytes(int n_layers, int B, int d, int H, int dff) {
-  if (B < 1 || B > 16 || d % 64 || dff % 32) return 0;
-  const int n = n_layers < kDecMaxLayers ? n_layers : kDecMaxLayers;
-  return (size_t)(n + 1) * dec_words(B, d, H, dff, seg_bound(ceil_div(B * H, 4), kB200Sms)).bytes;
+  if (B < 1 || d % 64 || dff % 32) return 0;
+  const int n = n_layers < kDecMaxLayers ? n_layers : kDecMaxLayers, sub = decode_slice(B), last = B - (ceil_div(B, sub) - 1) * sub;
+  auto slice = [&](int b) { return (size_t)(n + 1) * dec_words(b, d, H, dff, seg_bound(ceil_div(b * H, 4), kB200Sms)).bytes; };
+  return slice(sub) > slice(last) ? slice(sub) : slice(last);
 }
 
 cudaError_t decode_launch(const DecodeParams& p0, cudaStream_t s) {
@@ -790,6 +795,7 @@ cudaError_t decode_launch(const DecodeParams& p0, cudaStream_t s) {
     p.pf_keys = (int)(keys < (size_t)p.chunk_len ? keys : (size_t)p.chunk_len);
   }
   const DecWords W = dec_words(p.B, p.d, p.H, p.dff, seg_max);
+  if ((size_t)(p.n_layers + 1) * W.bytes > p.words_size) return cudaErrorInvalidConfiguration;
   bool gains = false;
   for (int l = 0; l < p.n_layers; ++l)
     gains = gains || p.layer[l].g_attn || p.layer[l].g_mlp || p.layer[l].g_kv || p.layer[l].g_q || p.layer[l].g_k;

@@ -188,12 +188,14 @@ struct DecodeParams {
   const void* emb; const int32_t* ids; int vocab;  // rows of the embedding
   void* z_out; long long z_bs;                     // the last layer's output rows
   const void* next_bytes; size_t next_size;        // what the following kernel reads (L2 prefetch); may be NULL
-  unsigned char* words;                            // exchange area, decode_words_bytes(...)
+  unsigned char* words; size_t words_size;         // exchange area, decode_words_bytes(...)
   SyncArea* sync;
   DecLayer layer[kDecMaxLayers];
   int quads, chunks, chunk_len, warps_per_cta, pf_keys;   // attention split, set by the launcher
 };
-// Bytes of exchange area for a launch (0: the kernel does not take the shape).
+// Sequences per launch: a batch above 16 runs as slices of equal size (the sequences are independent), the last one with what is left.
+int decode_slice(int B);
+// Bytes of exchange area for the slices of a batch of B, one after the other (0: the kernel does not take the shape).
 size_t decode_words_bytes(int n_layers, int B, int d, int H, int dff);
 cudaError_t decode_launch(const DecodeParams& p, cudaStream_t s);
 

@@ -125,3 +125,18 @@ def test_unknown_flags_are_invalid_configurations():
     assert rt.rt_workspace_bytes(rt.make_config(128, 2, 512, dtype="f32", norm_flags=4 | 3), 1, 16) == 0
     assert rt.rt_workspace_bytes(rt.make_config(128, 2, 512, dtype="f32", flags=2), 1, 16) == 0
     assert rt.rt_workspace_bytes(rt.make_config(128, 2, 512, dtype="f32", flags=rt.RT_FLAG_BACKWARD_STEP_LAUNCHES), 1, 16) > 0
+
+
+def test_decode_workspace_covers_every_slice_of_the_batch():
+    # A bf16 decode step above 16 sequences runs as slices one after the other in one exchange area, whose size per layer the
+    # workspace shows (nothing else of a one-position workspace depends on the number of layers).  A smaller last slice can need
+    # more of it than the fuller ones: each pair's attention is then split over more CTAs.
+    def per_layer(B, d, dff):
+        ws = [rt.rt_workspace_bytes(rt.make_config(d, d // 64, dff, dtype="bf16"), B, 1, n) for n in (2, 3)]
+        return ws[1] - ws[0]
+    for H in range(1, 17):
+        for B in range(17, 65):
+            slices = -(-B // 16)
+            sub = -(-B // slices)
+            need = max(per_layer(b, 64 * H, 256 * H) for b in (sub, B - (-(-B // sub) - 1) * sub))
+            assert per_layer(B, 64 * H, 256 * H) >= need > 0, (B, H)

@@ -60,3 +60,31 @@ def test_decode_of_more_layers_than_one_launch_takes():
     got = st.decode(data["ids"][:, N], N)
     # roundings of 18 layers, each scaled by 1/sqrt(18), add up like one layer's
     assert np.abs(got - ref).max() <= 2 * TOL * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("d,H,B,L", [(128, 2, 17, 8), (128, 2, 21, 8), (64, 1, 40, 3)])
+def test_decode_slices_stay_inside_the_workspace(d, H, B, L):
+    # the last slice is smaller than the others and needs more of the exchange area per sequence
+    import torch
+    from oracle import RTConfig, RTWeights, stack_prefill
+    from paper_2604_21215_b200 import inputs, rt
+    dff, V, N = 2 * d, 77, 9
+    wl = inputs.Workload("slices", L, B, N + 1, d, H, dff, "bf16", vocab=V, residual_scale=1 / np.sqrt(L))
+    data = inputs.make_inputs(wl, seed=B)
+    ocfg = RTConfig(d, H, 64, dff, residual_scale=wl.residual_scale)
+    _, ref, _ = stack_prefill(ocfg, [RTWeights(**w) for w in data["layers"]], data["emb"], None, data["ids"])
+    st = rt.Stack(L, d, H, dff, V, dtype="bf16", residual_scale=wl.residual_scale)
+    st.set_weights(data["layers"], data["emb"])
+    st.prefill(data["ids"][:, :N], N_max=N + 1)
+    need = rt.rt_workspace_bytes(st.cfg, B, 1, L)
+    ws = torch.full((need + (1 << 20),), 0x5a, dtype=torch.uint8, device=st.device)
+    logits = torch.empty((B, V), dtype=torch.float32, device=st.device)
+    ids = torch.as_tensor(data["ids"][:, N], dtype=torch.int32, device=st.device).contiguous()
+    s = torch.cuda.current_stream(st.device).cuda_stream
+    assert rt.rt_decode_step(st.cfg, L, st.layers, st.emb.data_ptr(), None, V, ids.data_ptr(), B, N, logits.data_ptr(), st._kp, st._vp,
+                             st.N_max, ws.data_ptr(), need, s) == rt.RT_OK
+    torch.cuda.synchronize()
+    assert rt.rt_get_status(ws.data_ptr()) == rt.RT_OK
+    assert bool((ws[need:] == 0x5a).all())
+    got = logits.double().cpu().numpy()
+    assert np.abs(got - ref).max() <= 2 * TOL * np.abs(ref).max()
