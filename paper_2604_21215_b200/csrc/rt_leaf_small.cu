@@ -15,6 +15,7 @@
 
 #include <type_traits>
 
+#include "rt_handover.h"
 #include "rt_kernels.h"
 #include "rt_tc.cuh"
 
@@ -27,7 +28,7 @@ constexpr int kSmWarps = 16;                      // mat-vec warps per CTA; then
 constexpr int kFoldWarps = 4;                     // two lanes per query of the leaf: 64 queries
 constexpr int kSmThreads = (kSmWarps + 1 + kFoldWarps) * 32;
 constexpr int kSmLeafMax = kFoldWarps * 16;
-constexpr int kFin = 4;                           // final (k, v) of the last four positions
+constexpr int kFin = Handover::kSlots;            // final (k, v) of the last four positions
 constexpr int kStateStride = kHeadDim + 4;        // o[64], m, l of the query that is finished next
 
 struct SmallLayout {
@@ -36,7 +37,7 @@ struct SmallLayout {
 
 SmallLayout small_layout(size_t es, int nb, int d, int dff) {
   SmallLayout L;
-  size_t o = 128;
+  size_t o = 160;                                 // abort flag, mbarriers
   auto take = [&](size_t n) { const size_t at = o; o += align_up(n, 16); return (unsigned)at; };
   L.off_c = take((size_t)nb * d * 4); L.off_h = take((size_t)nb * d * 4); L.off_z = take((size_t)nb * d * 4);
   L.off_g = take((size_t)nb * dff * 4);
@@ -139,7 +140,8 @@ __global__ void __launch_bounds__(kSmThreads, 1) leaf_small_kernel(const LeafPar
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem);
   const uint32_t bars = smem_u32(smem + 16);
   const uint32_t bar_c = bars, bar_h = bars + 8, bar_g = bars + 16, bar_z = bars + 24, bar_kv = bars + 32, bar_w = bars + 40;
-  const uint32_t bar_key = bars + 48, bar_state = bars + 56, bar_done = bars + 72;   // attention: key ready; state of query (even, odd) ready; key (mod 4) folded
+  // attention: state of query (even, odd) ready; key (mod 4) ready, folded (rt_handover.h)
+  const uint32_t bar_state = bars + 48, bar_key = bars + 64, bar_done = bar_key + 8 * Handover::kReadyBars;
   float *vec_c = reinterpret_cast<float*>(smem + L.off_c), *vec_h = reinterpret_cast<float*>(smem + L.off_h);
   float *vec_g = reinterpret_cast<float*>(smem + L.off_g), *vec_z = reinterpret_cast<float*>(smem + L.off_z);
   float *kv = reinterpret_cast<float*>(smem + L.off_kv), *gain_mlp = reinterpret_cast<float*>(smem + L.off_gain), *gain_kv = gain_mlp + p.d;
@@ -158,8 +160,9 @@ __global__ void __launch_bounds__(kSmThreads, 1) leaf_small_kernel(const LeafPar
 
   if (tid == 0) {
     *s_abort = dead ? 1 : 0;
-    for (int i = 0; i < 7; ++i) mbar_init(bars + 8 * i, 1);
+    for (int i = 0; i < 6; ++i) mbar_init(bars + 8 * i, 1);
     mbar_init(bar_state, 2); mbar_init(bar_state + 8, 2);
+    for (int i = 0; i < Handover::kReadyBars; ++i) mbar_init(bar_key + 8 * i, 1);
     for (int i = 0; i < kFin; ++i) mbar_init(bar_done + 8 * i, kFoldWarps);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     mbar_expect_tx(bar_c, (uint32_t)(nb * d * 4)); mbar_expect_tx(bar_h, (uint32_t)(nb * d * 4));
@@ -216,7 +219,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) leaf_small_kernel(const LeafPar
           q0 = to_f(qp[0]); q1 = to_f(qp[1]);
           if (!wait_bar(bar_state + 8 * ((j + 1) & 1), ((j + 1) >> 1) & 1, s_abort, sync)) break;       // state of query j + 1
         }
-        if (j >= kFin && !wait_bar(bar_done + 8 * (j % kFin), (j / kFin - 1) & 1, s_abort, sync)) break;  // place of the pair j - 4
+        if (j >= kFin && !wait_bar(bar_done + 8 * Handover::slot(j), Handover::read_parity(j - kFin), s_abort, sync)) break;  // place of the pair j - 4
         if (!wait_bar(bar_kv, j & 1, s_abort, sync)) break;
         const float2 kr = *reinterpret_cast<const float2*>(kv + 2 * lane), vr = *reinterpret_cast<const float2*>(kv + kHeadDim + 2 * lane);
         const float rs = qkn ? rsqrtf(warp_sum(kr.x * kr.x + kr.y * kr.y) * (1.0f / kHeadDim) + p.eps) : 1.0f;
@@ -229,13 +232,13 @@ __global__ void __launch_bounds__(kSmThreads, 1) leaf_small_kernel(const LeafPar
           const float2 o = *reinterpret_cast<const float2*>(st + 2 * lane);
           publish((o.x * corr + pj * v0) * il, (o.y * corr + pj * v1) * il);
         }
-        float* f = fin + (j % kFin) * 2 * kHeadDim;
+        float* f = fin + Handover::slot(j) * 2 * kHeadDim;
         *reinterpret_cast<float2*>(f + 2 * lane) = make_float2(k0, k1);
         *reinterpret_cast<float2*>(f + kHeadDim + 2 * lane) = make_float2(v0, v1);
         __syncwarp();
         if (lane == 0) {
           if (j + 1 < n) mbar_expect_tx(bar_kv, 2 * kHeadDim * 4);
-          mbar_arrive(bar_key);
+          mbar_arrive(bar_key + 8 * Handover::ready_bar(j));
         }
         const size_t crow = ((size_t)(p.t0 + j) * B + b) * d + h * kHeadDim + 2 * lane;
         kc[crow] = from_f<T>(k0); kc[crow + 1] = from_f<T>(k1); vc[crow] = from_f<T>(v0); vc[crow + 1] = from_f<T>(v1);
@@ -268,8 +271,8 @@ __global__ void __launch_bounds__(kSmThreads, 1) leaf_small_kernel(const LeafPar
       if (i < 2 && i < n) leave_state();
       __syncwarp();
       for (int j = 0; j + 2 < n; ++j) {
-        if (!wait_bar(bar_key, j & 1, s_abort, sync)) break;
-        const float* f = fin + (j % kFin) * 2 * kHeadDim;
+        if (!wait_bar(bar_key + 8 * Handover::ready_bar(j), Handover::ready_parity(j), s_abort, sync)) break;
+        const float* f = fin + Handover::slot(j) * 2 * kHeadDim;
         if ((ft | 31) >> 1 >= j + 2) {                         // some query of this warp is still open
           float s0 = 0.f, s1 = 0.f;
 #pragma unroll
@@ -291,7 +294,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) leaf_small_kernel(const LeafPar
           if (i == j + 2) leave_state();
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_done + 8 * (j % kFin));
+        if (lane == 0) mbar_arrive(bar_done + 8 * Handover::slot(j));
       }
     }
   } else if (wait_bar(bar_w, 0, s_abort, sync)) {
