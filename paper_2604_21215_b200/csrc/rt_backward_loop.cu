@@ -18,6 +18,7 @@
 #include <cuda_bf16.h>
 #include <string.h>
 
+#include "rt_handover.h"
 #include "rt_kernels.h"
 #include "rt_tc.cuh"
 
@@ -31,7 +32,7 @@ constexpr int kBThreads = 512;
 constexpr int kBRegsMma = 160, kBRegsAtt = 96;               // (160 + 96) * 256 = 65536
 constexpr int kBMmaThreads = kBMma * 32;
 constexpr int kBLeaf = 64;
-constexpr int kBRing = 4;                         // queries handed to the fold warps
+constexpr int kBRing = Handover::kSlots;          // queries handed to the fold warps
 constexpr int kKvRow = 144;                       // floats of one position's k | v in shared memory: halves 36 apart (no bank conflicts)
 constexpr unsigned kBEmpty = 0xffffffffu;
 
@@ -131,8 +132,8 @@ __global__ void __launch_bounds__(kBThreads, 1) bwd_leaf_kernel(const __grid_con
   extern __shared__ __align__(128) unsigned char smem[];
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem);
   const uint32_t bars = smem_u32(smem + 16);
-  // weights; query handed over; state of the pair that is finished next (even, odd); query absorbed (ring)
-  const uint32_t w_bar = bars, bar_key = bars + 8, bar_state = bars + 16, bar_done = bars + 32;
+  // weights; state of the pair that is finished next (even, odd); query handed over, absorbed (ring, rt_handover.h)
+  const uint32_t w_bar = bars, bar_state = bars + 8, bar_key = bars + 24, bar_done = bar_key + 8 * Handover::kReadyBars;
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int G = gridDim.x, cta = blockIdx.x, B = p.B, d = p.d, H = p.H, dff = p.dff;
   const int d_lo = 2 * (int)((long long)(d / 2) * cta / G), nd = 2 * (int)((long long)(d / 2) * (cta + 1) / G) - d_lo;
@@ -142,7 +143,8 @@ __global__ void __launch_bounds__(kBThreads, 1) bwd_leaf_kernel(const __grid_con
 
   if (tid == 0) {
     *s_abort = *reinterpret_cast<volatile unsigned*>(&sync->abort_flag) ? 1 : 0;
-    mbar_init(w_bar, 1); mbar_init(bar_key, 1); mbar_init(bar_state, 2); mbar_init(bar_state + 8, 2);
+    mbar_init(w_bar, 1); mbar_init(bar_state, 2); mbar_init(bar_state + 8, 2);
+    for (int i = 0; i < Handover::kReadyBars; ++i) mbar_init(bar_key + 8 * i, 1);
     for (int i = 0; i < kBRing; ++i) mbar_init(bar_done + 8 * i, kBFold);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     mbar_expect_tx(w_bar, (uint32_t)(((size_t)3 * nd * d + (size_t)nf * d + (size_t)nd * dff) * 2));
@@ -220,8 +222,8 @@ __global__ void __launch_bounds__(kBThreads, 1) bwd_leaf_kernel(const __grid_con
       __syncwarp();
       int step = 0;
       for (int i = p.e0 - 1; i >= p.s0 + 2; --i, ++step) {
-        bl_wait(bar_key, step & 1, sync, s_abort);
-        const float* f = ring + (step % kBRing) * kRingRow;
+        bl_wait(bar_key + 8 * Handover::ready_bar(step), Handover::ready_parity(step), sync, s_abort);
+        const float* f = ring + Handover::slot(step) * kRingRow;
         if (p.s0 + (ft & ~31) / 2 <= i - 2) {                  // some position of this warp is still open
           float s0 = 0.f, s1 = 0.f, t0 = 0.f, t1 = 0.f;
 #pragma unroll 2
@@ -247,7 +249,7 @@ __global__ void __launch_bounds__(kBThreads, 1) bwd_leaf_kernel(const __grid_con
           }
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_done + 8 * (step % kBRing));
+        if (lane == 0) mbar_arrive(bar_done + 8 * Handover::slot(step));
       }
       return;
     }
@@ -298,13 +300,13 @@ __global__ void __launch_bounds__(kBThreads, 1) bwd_leaf_kernel(const __grid_con
       }
       // off the chain: hand the query to the fold warps, then the temporary pair
       if (i >= p.s0 + 2) {
-        if (step >= kBRing) bl_wait(bar_done + 8 * (step % kBRing), (step / kBRing - 1) & 1, sync, s_abort);
-        float* f = ring + (step % kBRing) * kRingRow;
+        if (step >= kBRing) bl_wait(bar_done + 8 * Handover::slot(step), Handover::read_parity(step - kBRing), sync, s_abort);
+        float* f = ring + Handover::slot(step) * kRingRow;
         *reinterpret_cast<float2*>(f + e2) = q;
         *reinterpret_cast<float2*>(f + kHeadDim + e2) = make_float2(c0, c1);
         if (lane == 0) { f[2 * kHeadDim] = lse; f[2 * kHeadDim + 1] = D; }
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_key);
+        if (lane == 0) mbar_arrive(bar_key + 8 * Handover::ready_bar(step));
       }
       const float dst = pt * (warp_sum(c0 * vt.x + c1 * vt.y) - D) * p.scale;
       const size_t at = (size_t)i * rstride + col + e2;

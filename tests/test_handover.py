@@ -84,7 +84,8 @@ def test_no_order_of_the_warps_stops_the_ring(tmp_path):
     assert one_barrier != "0"                                  # (the walk does find the dead end of a single ready barrier)
 
 
-def test_the_kernel_uses_the_ring():
-    text = open(os.path.join(ROOT, "paper_2604_21215_b200", "csrc", "rt_leaf_small.cu")).read()
-    for call in ("Handover::ready_bar(", "Handover::ready_parity(", "Handover::read_parity("):
-        assert call in text, call
+def test_both_kernels_use_the_ring():
+    for name in ("rt_leaf_small.cu", "rt_backward_loop.cu"):
+        text = open(os.path.join(ROOT, "paper_2604_21215_b200", "csrc", name)).read()
+        for call in ("Handover::ready_bar(", "Handover::ready_parity(", "Handover::read_parity("):
+            assert call in text, (name, call)
