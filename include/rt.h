@@ -101,7 +101,9 @@ typedef struct {            /* device pointers; read-only */
 } rt_layer_weights;
 
 /* Bytes of workspace a call with these shapes needs (N = positions per call: the prefill
- * length, or 1 for decode).  n_layers >= 1.  Returns 0 for an invalid configuration. */
+ * length, or 1 for decode).  n_layers >= 1.  Returns 0 for an invalid configuration.  Never
+ * smaller for a larger B, N or n_layers (the same holds for the two sizes below): a workspace for
+ * the fullest batch, the longest prompt and the deepest stack serves every smaller call. */
 size_t rt_workspace_bytes(const rt_config *cfg, int32_t B, int32_t N, int32_t n_layers);
 
 /* One RT layer over x[B,N,d] (Sec. 2.2; Algorithm 1).  Writes z[B,N,d] and rows [0,N) of

@@ -18,7 +18,7 @@ constexpr int kSmallBatchMax = 64;      // above this the per-token chain runs a
 constexpr int kAutoLeaf = 64;
 
 struct WsLayout {
-  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, dec_words, dec_words_bytes, ll, ll_bytes, gx, grp, packed, wave, wave_stride, hid0, hid1,
+  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, ll, ll_bytes, form, dec_words, dec_words_bytes, hid0, hid1,
       blk_h, blk_u, blk_c, blk_g, total;
 };
 
@@ -101,7 +101,7 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
   // sequences go layer by layer, as the same layers called one by one do (and give the same bits).
   if (N > kWaveMaxN || (size_t)N * B * c->d_model * 4 > kWaveCacheMax) return none;
   // Short leaves fill the pipeline of layers sooner, long ones have fewer launches.
-  const int leaf = c->leaf ? c->leaf : N <= 128 ? 16 : N <= 1024 ? 32 : 64;
+  const int leaf = c->leaf ? c->leaf : N <= 128 ? 16 : 32;
   return {places, leaf};
 }
 struct WaveRows { size_t n, q, kt, vt, st_o, st_m, st_l, total; };
@@ -114,6 +114,40 @@ WaveRows wave_rows_layout(const rt_config* c, int B, int leaf) {
   W.st_o = take(rows * d * 4); W.st_m = take(rows * H * 4); W.st_l = take(rows * H * 4);
   W.total = o;
   return W;
+}
+
+// Groups of SMs working side by side (slices of a batch, or layers of a stack): an exchange area and a packed layer per group, and for a
+// stack a leaf's rows of n, q, k~, v~ and the state per group.
+struct GroupArea { size_t packed, packed_stride, rows, rows_stride, total; };
+GroupArea group_area(const rt_config* c, int places, int packs, int wave_B, int wave_leaf) {
+  GroupArea A;
+  A.packed = align_up((size_t)kGroupJobs * leaf_group_words_bytes(c->d_model, c->d_ff), 256);
+  A.packed_stride = leaf_group_packed_bytes(c->d_model, c->d_ff, places);
+  A.rows = A.packed + align_up(A.packed_stride * packs, 256);
+  A.rows_stride = wave_leaf ? wave_rows_layout(c, wave_B, wave_leaf).total : 0;
+  A.total = A.rows + A.rows_stride * (wave_leaf ? places : 0);
+  return A;
+}
+
+// Bytes of the area that the form of the token loop has to itself: the most that any call of at most B sequences, N positions and n_layers
+// layers asks for, whichever form it takes, so that a workspace reserved for the longest prompt and the fullest batch serves all the others.
+// (What one form asks for by itself does not grow with the shape: beyond kWaveMaxN positions no layers run side by side, from 17
+// sequences on there is no array of g.)
+size_t form_bytes(const rt_config* c, int B, int N, int n_layers) {
+  if (c->dtype != RT_BF16) return 0;
+  if (c->sched != RT_SCHED_TILED || c->recur_block > 1) return 0;
+  const int d = c->d_model, H = c->n_heads, f = c->d_ff, B16 = B < 16 ? B : 16;
+  size_t most = 0;
+  auto need = [&](size_t bytes) { if (bytes > most) most = bytes; };
+  LeafMmaLaunch ml;
+  if (leaf_mma_shape(1, d, H, f, c->leaf, kB200Sms, kB200SmemPerCta, &ml)) need((size_t)(ml.leaf < N ? ml.leaf : N) * 16 * f * 2);      // g of the tensor-core leaf kernel
+  if (N < 2) return most;
+  for (int places = 2; places <= kGroupJobs; ++places) {
+    if (!leaf_group_shape(1, d, H, f, places, kB200SmemPerCta)) continue;
+    if (B > 16 * (places - 1)) need(group_area(c, places, 1, 0, 0).total);
+    if (n_layers >= places) need(group_area(c, places, places, B16, c->leaf ? c->leaf : N <= 128 ? 16 : 32).total);
+  }
+  return most;
 }
 
 WsLayout ws_layout(const rt_config* c, int B, int N, int n_layers) {
@@ -135,23 +169,16 @@ WsLayout ws_layout(const rt_config* c, int B, int N, int n_layers) {
   L.ex_z = take((size_t)B * d * 4);
   L.ex_k = take((size_t)B * d * 4);
   L.ex_part = take((size_t)B * H * kMaxChunks * 68 * 4);
-  // exchange area of the decode kernel (a decode step is a call with N = 1, of any workspace at least that large)
-  L.dec_words_bytes = c->dtype == RT_BF16 && B <= kSmallBatchMax ? decode_words_bytes(n_layers, B, (int)d, (int)H, (int)f) : 0;
-  L.dec_words = take(L.dec_words_bytes);
   // exchange buffers of the tensor-core leaf kernel: c, h, z as flag-carrying words (16 sequence slots each),
-  // raw k|v as flag-carrying fp32 words; g as packed bf16 in fragment order (16 sequence slots), an array per position of a leaf (gx)
+  // raw k|v as flag-carrying fp32 words; g as packed bf16 in fragment order (16 sequence slots), an array per position of a leaf, in `form`
   L.ll_bytes = ((size_t)16 * 3 * (d / 2) + (size_t)B * 2 * d) * 8;
   L.ll = take(L.ll_bytes);
-  // group kernel: one exchange area per group of SMs, the packed weights of a layer (of every layer, when the layers of a
-  // stack run side by side) and, for a stack, a leaf's rows of n, q, k~, v~ and the state per group
-  const Wave wv = stack_wave(c, B, N, n_layers);
-  const Schedule sch = effective_schedule(c, B);
-  L.gx = take(sch.path == kPathMma || sch.path == kPathMmaSplit ? (size_t)(sch.leaf < N ? sch.leaf : N) * 16 * f * 2 : 0);     // g of the tensor-core leaf kernel
-  const bool grp = N > 1 && (wv.places || sch.path == kPathGroups);
-  L.grp = take(grp ? (size_t)kGroupJobs * leaf_group_words_bytes((int)d, (int)f) : 0);
-  L.packed = take(grp ? (wv.places ? (size_t)n_layers : 1) * leaf_group_packed_bytes((int)d, (int)f, wv.places ? wv.places : ceil_div(B, sch.sub)) : 0);
-  L.wave_stride = wv.places ? wave_rows_layout(c, B, wv.leaf).total : 0;
-  L.wave = take(L.wave_stride * wv.places);
+  L.form = take(form_bytes(c, B, N, n_layers));
+  // a decode step uses none of the above but the status block: its exchange area begins right behind that
+  L.dec_words = L.q;
+  const size_t dec = c->dtype == RT_BF16 ? decode_words_bytes(n_layers, B, (int)d, (int)H, (int)f) : 0;
+  if (o < L.dec_words + dec) o = L.dec_words + align_up(dec, 256);
+  L.dec_words_bytes = o - L.dec_words;
   L.hid0 = take(tok * d * e);
   L.hid1 = take(tok * d * e);
   // recurrence over blocks: the position-wise chain of one block (rows = block length x B)
@@ -217,7 +244,7 @@ struct CallCtx { cudaStream_t s; unsigned bar_base = 0; unsigned seq_base = 0; u
 bool zero_groups(const rt_config* c, unsigned char* ws, const WsLayout& L, CallCtx& ctx) {
   if (ctx.groups_zeroed) return true;
   ctx.groups_zeroed = true;
-  return cudaMemsetAsync(ws + L.grp, 0, (size_t)kGroupJobs * leaf_group_words_bytes(c->d_model, c->d_ff), ctx.s) == cudaSuccess;
+  return cudaMemsetAsync(ws + L.form, 0, (size_t)kGroupJobs * leaf_group_words_bytes(c->d_model, c->d_ff), ctx.s) == cudaSuccess;
 }
 GroupCommon group_common(const rt_config* c, int B, unsigned char* ws, const WsLayout& L) {
   GroupCommon g;
@@ -482,7 +509,7 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   {
     unsigned long long* w = (unsigned long long*)(ws + L.ll);
     const size_t bd2 = (size_t)16 * (c->d_model / 2);
-    mb.ll_c = w; mb.ll_h = w + bd2; mb.ll_z = w + 2 * bd2; mb.ll_g = (unsigned long long*)(ws + L.gx);
+    mb.ll_c = w; mb.ll_h = w + bd2; mb.ll_z = w + 2 * bd2; mb.ll_g = (unsigned long long*)(ws + L.form);
     mb.ll_kv = w + 3 * bd2;
   }
   auto leaf_mma = [&](int t0, int t1) -> bool {
@@ -493,7 +520,7 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
       lp.x = (const unsigned char*)x + (size_t)b0 * x_bs * e;
       lp.z = (unsigned char*)z + (size_t)b0 * z_bs * e;
       lp.t0 = t0; lp.t1 = t1; lp.attn_begin = t0; lp.seq_base = ctx.seq_base;
-      if (cudaMemsetAsync(ws + L.gx, 0xff, (size_t)(t1 - t0) * 16 * c->d_ff * 2, s) != cudaSuccess) return false;
+      if (cudaMemsetAsync(ws + L.form, 0xff, (size_t)(t1 - t0) * 16 * c->d_ff * 2, s) != cudaSuccess) return false;
       if (leaf_mma_launch(lp, ml, mb, s) != cudaSuccess) return false;
       ctx.seq_base += (unsigned)(t1 - t0);
     }
@@ -517,9 +544,10 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   };
   const bool groups = !small && plan.path == kPathGroups && pos0 == 0 && n_rows > 1;      // (one position: no workspace for it, see ws_layout)
   const int places = groups ? ceil_div(B, plan.sub) : 0;
+  unsigned char* const packed = groups ? ws + L.form + group_area(c, places, 1, 0, 0).packed : nullptr;
   if (groups) {
     if (!zero_groups(c, ws, L, ctx)) return RT_ERR_CUDA;
-    const GroupPackLayer pl = {w->w_o, w->w_up, w->w_down, w->w_k, w->w_v, ws + L.packed};
+    const GroupPackLayer pl = {w->w_o, w->w_up, w->w_down, w->w_k, w->w_v, packed};
     ProfScope ps(s, kProfPrepass);
     if (leaf_group_pack(&pl, 1, c->d_model, c->d_ff, places, s) != cudaSuccess) return RT_ERR_CUDA;
   }
@@ -531,13 +559,13 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
     for (int i = 0; i < places; ++i) {
       GroupJob& j = jobs[i];
       const int b0 = i * plan.sub;
-      j.packed = ws + L.packed; j.g_mlp = lp.g_mlp; j.g_kv = lp.g_kv; j.g_k = lp.g_k; j.alibi = w->alibi_slopes;
+      j.packed = packed; j.g_mlp = lp.g_mlp; j.g_kv = lp.g_kv; j.g_k = lp.g_k; j.alibi = w->alibi_slopes;
       j.q = lp.q; j.st_o = lp.st_o; j.st_m = lp.st_m; j.st_l = lp.st_l; j.row_off = 0;
       j.x = (const unsigned char*)x + (size_t)b0 * x_bs * e; j.x_bs = x_bs; j.x_ts = x_ts;
       j.z = (unsigned char*)z + (size_t)b0 * z_bs * e; j.z_bs = z_bs; j.z_ts = z_ts;
       j.k_cache = k_cache; j.v_cache = v_cache; j.t0 = t0; j.t1 = t1; j.key0 = t0;
       j.B = B - b0 < plan.sub ? B - b0 : plan.sub; j.b0 = b0;
-      j.words = ws + L.grp + (size_t)i * leaf_group_words_bytes(c->d_model, c->d_ff); j.steps = ctx.group_steps[i];
+      j.words = ws + L.form + (size_t)i * leaf_group_words_bytes(c->d_model, c->d_ff); j.steps = ctx.group_steps[i];
       ctx.group_steps[i] += (unsigned)(t1 - t0);
     }
     return leaf_group_launch(group_common(c, B, ws, L), jobs, places, places, s) == cudaSuccess;
@@ -562,35 +590,39 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
                          void* const* v_caches, int N_max, unsigned char* ws, const WsLayout& L, const Wave& wv, CallCtx& ctx) {
   cudaStream_t s = ctx.s;
   const int places = wv.places, n_leaves = ceil_div(N, wv.leaf);
-  const size_t e = esize_of(c->dtype), d = c->d_model, packed = leaf_group_packed_bytes(c->d_model, c->d_ff, places);
+  const size_t e = esize_of(c->dtype), d = c->d_model;
   const WaveRows W = wave_rows_layout(c, B, wv.leaf);
+  const GroupArea A = group_area(c, places, places, B, wv.leaf);
   if (!zero_groups(c, ws, L, ctx)) return RT_ERR_CUDA;
-  std::vector<GroupPackLayer> pl(n_layers);
-  std::vector<int> start(n_layers);                            // wave in which a layer begins
-  for (int l = 0; l < n_layers; ++l) {
-    const rt_layer_weights& w = layers[l];
-    pl[l] = {w.w_o, w.w_up, w.w_down, w.w_k, w.w_v, ws + L.packed + (size_t)l * packed};
-    start[l] = l == 0 ? 0 : start[l - 1] + 1;
-    if (l >= places && start[l] < start[l - places] + n_leaves) start[l] = start[l - places] + n_leaves;
-  }
-  {
+  // A layer takes the place of the one `places` before it when that has finished its last leaf; its weights are packed into the place then.
+  const int turn = n_leaves > places ? n_leaves : places;
+  auto start = [&](int l) { return l / places * turn + l % places; };                       // wave in which a layer begins
+  auto packed = [&](int place) { return ws + L.form + A.packed + (size_t)place * A.packed_stride; };
+  auto pack = [&](int l0, int n) {
+    GroupPackLayer pl[kGroupJobs];
+    for (int i = 0; i < n; ++i) {
+      const rt_layer_weights& w = layers[l0 + i];
+      pl[i] = {w.w_o, w.w_up, w.w_down, w.w_k, w.w_v, packed((l0 + i) % places)};
+    }
     ProfScope ps(s, kProfPrepass);
-    if (leaf_group_pack(pl.data(), n_layers, c->d_model, c->d_ff, places, s) != cudaSuccess) return RT_ERR_CUDA;
-  }
+    return leaf_group_pack(pl, n, c->d_model, c->d_ff, places, s) == cudaSuccess;
+  };
+  if (!pack(0, places)) return RT_ERR_CUDA;
   const GroupCommon gc = group_common(c, B, ws, L);
   const long long bs = (long long)N * d;
-  for (int wave = 0, waves = start[n_layers - 1] + n_leaves; wave < waves; ++wave) {
+  for (int wave = 0, waves = start(n_layers - 1) + n_leaves; wave < waves; ++wave) {
     GroupJob jobs[kGroupJobs];
     memset(jobs, 0, sizeof(jobs));
     int nj = 0, np = 0;
     PrepassParams pre[kGroupJobs];
     int layer_of[kGroupJobs];
     for (int l = 0; l < n_layers; ++l) {
-      const int k = wave - start[l];
+      const int k = wave - start(l);
       if (k < 0 || k >= n_leaves) continue;
+      if (k == 0 && l >= places && !pack(l, 1)) return RT_ERR_CUDA;
       const rt_layer_weights& w = layers[l];
       const int place = l % places, t0 = k * wv.leaf, t1 = t0 + wv.leaf < N ? t0 + wv.leaf : N;
-      unsigned char* rows = ws + L.wave + L.wave_stride * place;
+      unsigned char* rows = ws + L.form + A.rows + A.rows_stride * place;
       const void* x = hid[l & 1];
       PrepassParams& pp = pre[np];
       memset(&pp, 0, sizeof(pp));
@@ -609,7 +641,7 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
       const int l = layer_of[i];
       const PrepassParams& pp = pre[i];
       const rt_layer_weights& w = layers[l];
-      const int k = wave - start[l], place = l % places, t0 = k * wv.leaf, t1 = t0 + wv.leaf < N ? t0 + wv.leaf : N;
+      const int k = wave - start(l), place = l % places, t0 = k * wv.leaf, t1 = t0 + wv.leaf < N ? t0 + wv.leaf : N;
       const void* x = hid[l & 1];
       GroupJob& j = jobs[nj++];
       j.key0 = 0;
@@ -625,12 +657,12 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
         ProfScope ps(s, kProfTile);
         if (tile_tc_launch(tp, tp.rows_q, tp.rows_kv, tp.sync, s) != cudaSuccess) return RT_ERR_CUDA;
       }
-      j.packed = pl[l].out; j.g_mlp = w.g_mlp; j.g_kv = w.g_kv ? w.g_kv : w.g_attn; j.g_k = w.g_k; j.alibi = w.alibi_slopes;
+      j.packed = packed(place); j.g_mlp = w.g_mlp; j.g_kv = w.g_kv ? w.g_kv : w.g_attn; j.g_k = w.g_k; j.alibi = w.alibi_slopes;
       j.q = pp.q; j.st_o = pp.st_o; j.st_m = pp.st_m; j.st_l = pp.st_l; j.row_off = t0;
       j.x = x; j.x_bs = bs; j.x_ts = (long long)d;
       j.z = l == n_layers - 1 && out ? out : hid[(l + 1) & 1]; j.z_bs = bs; j.z_ts = (long long)d;
       j.k_cache = k_caches[l]; j.v_cache = v_caches[l]; j.t0 = t0; j.t1 = t1; j.B = B; j.b0 = 0;
-      j.words = ws + L.grp + (size_t)place * leaf_group_words_bytes(c->d_model, c->d_ff); j.steps = ctx.group_steps[place];
+      j.words = ws + L.form + (size_t)place * leaf_group_words_bytes(c->d_model, c->d_ff); j.steps = ctx.group_steps[place];
       ctx.group_steps[place] += (unsigned)(t1 - t0);
     }
     ProfScope ps(s, kProfLeaf);

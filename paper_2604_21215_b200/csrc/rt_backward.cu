@@ -1364,7 +1364,7 @@ BwdLayout bwd_layout(const rt_config* c, int B, int N) {
   L.wctr = wide && tc ? take(wide_counter_bytes(B) / 4) : o;
   if (wide && tc && N < 8) L.gprod = take((size_t)8 * B * d);    // parts of split products
   size_t sa_elems = rows_k * (d > f ? d : f), sb_elems = sa_elems;
-  const size_t op_rows = bwd_wide_terms(c, B) == 3 ? kWideTermRows * 3 : B;
+  const size_t op_rows = B < 3 * kWideTermRows ? 3 * kWideTermRows : B;       // (three terms of up to 32 sequences; no less for the batches above that have one)
   if (wide && sb_elems < (2 * d + f) * op_rows + 64) sb_elems = (2 * d + f) * op_rows + 64;     // the operands of one position side by side
   if (wide && sa_elems < d * op_rows) sa_elems = d * op_rows;
   L.sa = take(sa_elems / 2 + 64); L.sb = take(sb_elems / 2 + 64); L.wt = take(d * d / 2 + 64);

@@ -759,13 +759,17 @@ int seg_bound(int quads, int grid) { return ceil_div(grid, quads) + 2; }
 
 int decode_slice(int B) { return ceil_div(B, ceil_div(B, 16)); }
 
-// The largest area that one of the batch's slices asks for.  That need not be the fullest slice: a smaller one has fewer groups of four pairs,
-// hence more partial states for each pair (d = 128, H = 2: 17 sequences are slices of 9 and 8, and the 8 need 10 KB a layer more).
+// Room for every slice of up to min(B, 16) sequences.  What a slice needs does not grow with it: fewer sequences have fewer groups of four
+// pairs, hence more partial states for each pair (d = 128, H = 2: eight sequences need 10 KB a layer more than nine).
 size_t decode_words_bytes(int n_layers, int B, int d, int H, int dff) {
   if (B < 1 || d % 64 || dff % 32) return 0;
-  const int n = n_layers < kDecMaxLayers ? n_layers : kDecMaxLayers, sub = decode_slice(B), last = B - (ceil_div(B, sub) - 1) * sub;
-  auto slice = [&](int b) { return (size_t)(n + 1) * dec_words(b, d, H, dff, seg_bound(ceil_div(b * H, 4), kB200Sms)).bytes; };
-  return slice(sub) > slice(last) ? slice(sub) : slice(last);
+  const int n = n_layers < kDecMaxLayers ? n_layers : kDecMaxLayers;
+  size_t most = 0;
+  for (int b = 1; b <= B && b <= 16; ++b) {
+    const size_t bytes = dec_words(b, d, H, dff, seg_bound(ceil_div(b * H, 4), kB200Sms)).bytes;
+    if (bytes > most) most = bytes;
+  }
+  return (size_t)(n + 1) * most;
 }
 
 cudaError_t decode_launch(const DecodeParams& p0, cudaStream_t s) {

@@ -195,7 +195,7 @@ struct DecodeParams {
 };
 // Sequences per launch: a batch above 16 runs as slices of equal size (the sequences are independent), the last one with what is left.
 int decode_slice(int B);
-// Bytes of exchange area for the slices of a batch of B, one after the other (0: the kernel does not take the shape).
+// Bytes of exchange area for the slices of a batch of at most B, one after the other (0: the kernel does not take the shape).
 size_t decode_words_bytes(int n_layers, int B, int d, int H, int dff);
 cudaError_t decode_launch(const DecodeParams& p, cudaStream_t s);
 

@@ -128,15 +128,35 @@ def test_unknown_flags_are_invalid_configurations():
 
 
 def test_decode_workspace_covers_every_slice_of_the_batch():
-    # A bf16 decode step above 16 sequences runs as slices one after the other in one exchange area, whose size per layer the
-    # workspace shows (nothing else of a one-position workspace depends on the number of layers).  A smaller last slice can need
-    # more of it than the fuller ones: each pair's attention is then split over more CTAs.
-    def per_layer(B, d, dff):
-        ws = [rt.rt_workspace_bytes(rt.make_config(d, d // 64, dff, dtype="bf16"), B, 1, n) for n in (2, 3)]
-        return ws[1] - ws[0]
+    # A bf16 decode step above 16 sequences runs as slices one after the other in one exchange area.  A smaller last slice can need
+    # more of it than the fuller ones: each pair's attention is then split over more CTAs.  So a batch asks for no less than any of its
+    # slices would alone, at any depth (16 layers share a launch: the exchange area is most of that workspace).
     for H in range(1, 17):
-        for B in range(17, 65):
-            slices = -(-B // 16)
-            sub = -(-B // slices)
-            need = max(per_layer(b, 64 * H, 256 * H) for b in (sub, B - (-(-B // sub) - 1) * sub))
-            assert per_layer(B, 64 * H, 256 * H) >= need > 0, (B, H)
+        cfg = rt.make_config(64 * H, H, 256 * H, dtype="bf16")
+        for L in (1, 8, 16):
+            alone = [rt.rt_workspace_bytes(cfg, b, 1, L) for b in range(1, 17)]
+            for B in range(17, 65):
+                assert rt.rt_workspace_bytes(cfg, B, 1, L) >= max(alone), (H, B, L)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_workspace_grows_with_the_shape(dtype):
+    # a workspace reserved for the longest prompt, the fullest batch and the deepest stack serves every smaller call
+    Bs = [1, 2, 5, 8, 9, 15, 16, 17, 23, 32, 33, 48, 49, 64, 65, 200]
+    Ns = [1, 2, 16, 17, 64, 128, 129, 1000, 1024, 1025, 4096]
+    Ls = [1, 2, 3, 4, 8, 24]
+    for d, dff, kw in ((64, 256, {}), (128, 512, {"leaf": 16}), (384, 1536, {}), (768, 3072, {"leaf": 128}), (1024, 4096, {}),
+                       (1024, 4096, {"sched": "naive"}), (1024, 8192, {}), (2048, 8192, {})):
+        cfg = rt.make_config(d, d // 64, dff, dtype=dtype, **kw)
+        ws = {(B, N, L): rt.rt_workspace_bytes(cfg, B, N, L) for B in Bs for N in Ns for L in Ls}
+        for (B, N, L), have in ws.items():
+            for axis, values in enumerate((Bs, Ns, Ls)):
+                at = [B, N, L]
+                i = values.index(at[axis])
+                if i:
+                    at[axis] = values[i - 1]
+                    assert ws[tuple(at)] <= have, (d, dff, kw, tuple(at), (B, N, L))
+        for size in (rt.rt_recompute_workspace_bytes, rt.rt_backward_workspace_bytes):
+            ws = [[size(cfg, B, N) for N in Ns] for B in Bs]
+            assert all(a <= b for row in ws for a, b in zip(row, row[1:])), (size, d, dff, kw)
+            assert all(a <= b for r0, r1 in zip(ws, ws[1:]) for a, b in zip(r0, r1)), (size, d, dff, kw)

@@ -60,3 +60,24 @@ def test_layers_side_by_side_match_oracle(L, d, H, dff, B, N, leaf, gains, alibi
     for l, (k, v) in enumerate(st.caches_numpy(N)):
         check_tensor(f"wave L={L} layer {l}", "k", k, caches_ref[l][0], 2e-2)
         check_tensor(f"wave L={L} layer {l}", "v", v, caches_ref[l][1], 2e-2)
+
+
+@pytest.mark.parametrize("L,B,N", [(6, 2, 77), (2, 16, 130)])
+def test_a_workspace_for_long_prompts_serves_short_ones(L, B, N):
+    import torch
+    from paper_2604_21215_b200 import inputs, rt
+    d, H, dff, V = 512, 8, 1024, 91
+    data = inputs.make_inputs(inputs.Workload("wave", L, B, N, d, H, dff, "bf16", vocab=V, residual_scale=1 / np.sqrt(L)), seed=N)
+    stacks = []
+    for longest in (N, 1500):
+        st = rt.Stack(L, d, H, dff, V, dtype="bf16", residual_scale=1 / np.sqrt(L))
+        st.set_weights(data["layers"], data["emb"])
+        st.reserve(B, longest)
+        ids = torch.as_tensor(data["ids"], dtype=torch.int32, device=st.device).contiguous()
+        hid = torch.empty((B, N, d), dtype=torch.bfloat16, device=st.device)
+        st.prefill_device(ids, hid, None)
+        torch.cuda.synchronize()
+        assert st.status() == rt.RT_OK
+        stacks.append((hid, [k[:N] for k in st.k_caches]))
+    assert torch.equal(stacks[0][0], stacks[1][0])
+    assert all(torch.equal(a, b) for a, b in zip(stacks[0][1], stacks[1][1]))
