@@ -709,8 +709,8 @@ rt_status run_decode(const rt_config* c, int n_layers, const rt_layer_weights* l
   return RT_OK;
 }
 
-// bf16 shapes whose widths fit the decode kernel's 64-byte blocks; everything else takes the generic leaf kernel.
-bool decode_fast(const rt_config* c) { return c->dtype == RT_BF16 && c->d_model % 64 == 0 && c->d_ff % 32 == 0; }
+// bf16 shapes that the decode kernel takes; everything else takes the generic leaf kernel.
+bool decode_fast(const rt_config* c, int B) { return c->dtype == RT_BF16 && decode_shape(B, c->d_model, c->n_heads, c->d_ff); }
 
 rt_status common_checks(const rt_config* c, int B, int N, int n_layers, void* ws, size_t ws_bytes, bool wide_ok = false) {
   if (!config_ok(c) || B <= 0 || N <= 0 || n_layers <= 0 || !ws || !aligned16(ws)) return RT_ERR_INVALID_ARG;
@@ -887,7 +887,7 @@ rt_status rt_layer_decode_step(const rt_config* cfg, const rt_layer_weights* w, 
   const WsLayout L = ws_layout(cfg, B, 1, 1);
   if (cudaMemsetAsync(ws + L.sync, 0, sizeof(SyncArea), s) != cudaSuccess) return RT_ERR_CUDA;
   const long long d = cfg->d_model;
-  if (decode_fast(cfg)) {
+  if (decode_fast(cfg, B)) {
     void* hid[2] = {ws + L.hid0, ws + L.hid1};
     return run_decode(cfg, 1, w, x, d, nullptr, nullptr, 0, B, pos, z, d, &k_cache, &v_cache, ws, L, hid, nullptr, 0, s);
   }
@@ -969,7 +969,7 @@ rt_status rt_decode_step(const rt_config* cfg, int32_t n_layers, const rt_layer_
   rt_config c = *cfg;
   c.sched = RT_SCHED_NAIVE;
   void* bufs[2] = {ws + L.hid0, ws + L.hid1};
-  if (decode_fast(cfg)) {
+  if (decode_fast(cfg, B)) {
     // the last launch's output goes to the buffer that the last but one does not use
     void* z = bufs[(ceil_div(n_layers, kDecMaxLayers) - 1) & 1];
     st = run_decode(cfg, n_layers, layers, nullptr, 0, emb, ids, vocab, B, pos, z, d, k_caches, v_caches, ws, L, bufs, emb,

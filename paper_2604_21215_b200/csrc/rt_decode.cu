@@ -759,10 +759,17 @@ int seg_bound(int quads, int grid) { return ceil_div(grid, quads) + 2; }
 
 int decode_slice(int B) { return ceil_div(B, ceil_div(B, 16)); }
 
+// Widths in whole 64-byte blocks whose reduction buffers leave room in shared memory (five d-wide matrices at once: d up to about 12000 with
+// d_ff = 4 d; d_ff up to about 65000), and no more groups of four pairs than warps (pure arithmetic).
+bool decode_shape(int B, int d, int H, int dff) {
+  return d % 64 == 0 && dff % 32 == 0 && dec_layout(d, dff, kB200Sms, kB200SmemPerCta).total <= kB200SmemPerCta &&
+         (long long)(B < 16 ? B : 16) * H <= 4LL * kB200Sms * kDecWarps;
+}
+
 // Room for every slice of up to min(B, 16) sequences.  What a slice needs does not grow with it: fewer sequences have fewer groups of four
 // pairs, hence more partial states for each pair (d = 128, H = 2: eight sequences need 10 KB a layer more than nine).
 size_t decode_words_bytes(int n_layers, int B, int d, int H, int dff) {
-  if (B < 1 || d % 64 || dff % 32) return 0;
+  if (B < 1 || !decode_shape(1, d, H, dff)) return 0;
   const int n = n_layers < kDecMaxLayers ? n_layers : kDecMaxLayers;
   size_t most = 0;
   for (int b = 1; b <= B && b <= 16; ++b) {

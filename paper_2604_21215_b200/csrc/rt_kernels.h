@@ -193,6 +193,7 @@ struct DecodeParams {
   DecLayer layer[kDecMaxLayers];
   int quads, chunks, chunk_len, warps_per_cta, pf_keys;   // attention split, set by the launcher
 };
+bool decode_shape(int B, int d, int H, int dff);   // whether the kernel takes the slices of a batch of B
 // Sequences per launch: a batch above 16 runs as slices of equal size (the sequences are independent), the last one with what is left.
 int decode_slice(int B);
 // Bytes of exchange area for the slices of a batch of at most B, one after the other (0: the kernel does not take the shape).

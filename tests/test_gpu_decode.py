@@ -23,7 +23,8 @@ def _case(d, H, dff, B, N, seed, gains):
 @pytest.mark.parametrize("d,H,dff,B,pos,gains", [
     (128, 2, 256, 1, 0, False), (128, 2, 512, 3, 1, True), (192, 3, 224, 1, 7, False), (192, 3, 768, 5, 8, True),
     (256, 4, 1024, 8, 9, False), (320, 5, 1280, 9, 33, True), (768, 12, 3072, 16, 70, False), (1024, 16, 4096, 16, 40, True),
-    (256, 4, 1024, 17, 100, False), (128, 2, 512, 48, 19, True), (1408, 22, 5632, 2, 12, False), (64, 1, 128, 1, 300, False)])
+    (256, 4, 1024, 17, 100, False), (128, 2, 512, 48, 19, True), (1408, 22, 5632, 2, 12, False), (64, 1, 128, 1, 300, False),
+    (64, 1, 66560, 2, 5, False)])                               # (an MLP whose partial sums do not fit the decode kernel)
 def test_decode_step_matches_oracle(d, H, dff, B, pos, gains):
     import torch
     from oracle import RTConfig, RTWeights, layer_seq
