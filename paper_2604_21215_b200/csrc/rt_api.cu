@@ -671,18 +671,27 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
   return RT_OK;
 }
 
-// One decode step through all layers on the decode kernel (bf16): slices of at most 16 sequences, launches of at most
+// Whether the vectors between the phases of a decode step stay fp32: wherever the generic leaf kernel would answer otherwise, which holds
+// them so (batches above 16, a first position, layers off the tensor-core leaf kernel).  The error of the appended k, v rows against 64 bits is
+// 3.5e-3 that way and 4.1e-3 with bf16 vectors (d = 1024, 8 layers, 512 positions), for d = 2048 2.0e-3 and 2.9e-3.
+bool decode_full(const rt_config* c, int B, int pos) {
+  LeafMmaLaunch ml;
+  return B > 16 || pos == 0 || !leaf_mma_shape(B, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml);
+}
+
+// One decode step through all layers on the decode kernel (bf16): slices of at most 16 (fp32 vectors: 8) sequences, launches of at most
 // kDecMaxLayers layers.  Input rows x (row stride x_bs) or embedding rows emb[ids]; output rows z.  `hid` holds [B, d] rows between launches.
 rt_status run_decode(const rt_config* c, int n_layers, const rt_layer_weights* layers, const void* x, long long x_bs, const void* emb,
                      const int32_t* ids, int vocab, int B, int pos, void* z, long long z_bs, void* const* k_caches, void* const* v_caches,
                      unsigned char* ws, const WsLayout& L, void* const* hid, const void* next_bytes, size_t next_size, cudaStream_t s) {
-  const int sub = decode_slice(B), d = c->d_model;
+  const bool full = decode_full(c, B, pos);
+  const int sub = decode_slice(B, full), d = c->d_model;
   ProfScope ps(s, kProfLeaf);
   for (int b0 = 0; b0 < B; b0 += sub) {
     DecodeParams p;
     memset(&p, 0, sizeof(p));
     p.B = B - b0 < sub ? B - b0 : sub; p.Bs = B; p.b0 = b0;
-    p.d = d; p.H = c->n_heads; p.dff = c->d_ff; p.pos = pos;
+    p.d = d; p.H = c->n_heads; p.dff = c->d_ff; p.pos = pos; p.full = full ? 1 : 0;
     p.norm_flags = c->norm_flags; p.eps = c->rms_eps; p.scale_log2 = c->softmax_scale * kLog2e; p.alpha = c->residual_scale;
     p.words = ws + L.dec_words; p.words_size = L.dec_words_bytes; p.sync = (SyncArea*)(ws + L.sync);
     for (int l0 = 0; l0 < n_layers; l0 += kDecMaxLayers) {

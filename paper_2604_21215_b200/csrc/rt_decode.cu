@@ -12,6 +12,8 @@
 //   * phases hand their vectors over through L2 words that are their own flags: the exchange area is filled with
 //     0xFFFFFFFF (a NaN pattern no conversion produces) before the launch, every word is written once, and a consumer
 //     polls the words themselves.  No barrier across CTAs, no second round trip.
+// The vectors c, h, g, z travel as bf16, up to 16 sequences a launch, or (FULL) as fp32, up to eight: a value is then multiplied as three
+// bf16 terms whose sum it is (24 bits), the first two in the rows that the other eight sequences would take, the third in a second MMA.
 // Phases of layer l (K split over warps, partial sums through shared memory; sequences are the MMA's rows):
 //   1. x = z^{l-1}: q, k~, v~ of layer l and the raw persistent k, v of layer l-1 (raw fp32 words)
 //   2. attention over the cache: warp = (four heads, chunk of positions), Algorithm 2 per group of eight positions;
@@ -142,11 +144,19 @@ __device__ __noinline__ bool give_up(SyncArea* s, volatile int* s_abort, unsigne
   return true;
 }
 
-// Byte offset of element k of slot b in a vector of the exchange area.
-__device__ __forceinline__ size_t vec_off(int b, int k) { return ((size_t)((k >> 5) * 16 + b) << 6) + (size_t)(k & 31) * 2; }
+// Byte offset of element k of slot b in a vector of the exchange area (16 slots of bf16 or eight of fp32).
+template <bool FULL> __device__ __forceinline__ size_t vec_off(int b, int k) {
+  return FULL ? ((size_t)((k >> 5) * 8 + b) << 7) + (size_t)(k & 31) * 4 : ((size_t)((k >> 5) * 16 + b) << 6) + (size_t)(k & 31) * 2;
+}
+// Elements k, k + 1 (k even) into a vector.
+template <bool FULL> __device__ __forceinline__ void st_pair(unsigned char* vec, int b, int k, float x0, float x1) {
+  if (FULL) st_words2(vec + vec_off<true>(b, k), x0, x1);
+  else st_word(vec + vec_off<false>(b, k), pack_bf(x0, x1));
+}
 
-// Polls n <= KP blocks of 32 k of a vector (slots g and g + 8) until every word is there; all loads of a round are in flight before any is looked at.
-template <int MB, int KP>
+// Polls n <= KP blocks of 32 k of a vector (eight consecutive k of slots g and g + 8, or two groups of four of slot g) until every word is
+// there; all loads of a round are in flight before any is looked at.  STRIDE: bytes between the two pieces.
+template <int MB, int KP, int STRIDE>
 __device__ __forceinline__ void poll_vec(const unsigned char* base, int n, bool on0, bool on1, uint4 (&a)[KP][MB], SyncArea* sync, volatile int* s_abort) {
   unsigned need[MB];
 #pragma unroll
@@ -162,7 +172,7 @@ __device__ __forceinline__ void poll_vec(const unsigned char* base, int n, bool 
 #pragma unroll
     for (int i = 0; i < KP; ++i)
 #pragma unroll
-      for (int r = 0; r < MB; ++r) w[i][r] = ld_words_if(base + (size_t)i * 1024 + r * 512, (need[r] >> i) & 1u);
+      for (int r = 0; r < MB; ++r) w[i][r] = ld_words_if(base + (size_t)i * 1024 + r * STRIDE, (need[r] >> i) & 1u);
     unsigned left = 0;
 #pragma unroll
     for (int r = 0; r < MB; ++r) {
@@ -217,6 +227,27 @@ __device__ __forceinline__ void tile_products(const uint4 (&a)[KP][MB], int n, i
     *dst = v;
   }
 }
+// The same with three terms per value, of up to eight sequences.
+template <int KP, class RowFn>
+__device__ __forceinline__ void tile_products3(const uint4 (&a)[KP][3], int n, int tiles, float4* red, int red_stride, bool add, RowFn row) {
+#pragma unroll 1
+  for (int t = 0; t < tiles; ++t) {
+    const unsigned char* w = row(t);
+    float ce[4] = {0.f, 0.f, 0.f, 0.f}, co[4] = {0.f, 0.f, 0.f, 0.f}, le[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < KP; ++i) {
+      const uint4 bw = *reinterpret_cast<const uint4*>(w + (i < n ? i : 0) * 64);      // (blocks beyond n multiply zeros)
+      mma16816(ce, a[i][0].x, a[i][1].x, a[i][0].y, a[i][1].y, bw.x, bw.y);
+      mma16816(co, a[i][0].z, a[i][1].z, a[i][0].w, a[i][1].w, bw.z, bw.w);
+      mma16816(le, a[i][2].x, 0u, a[i][2].y, 0u, bw.x, bw.y);
+      mma16816(le, a[i][2].z, 0u, a[i][2].w, 0u, bw.z, bw.w);
+    }
+    float4 v = make_float4((ce[0] + co[0]) + ((ce[2] + co[2]) + le[0]), (ce[1] + co[1]) + ((ce[3] + co[3]) + le[1]), 0.f, 0.f);
+    float4* dst = red + (size_t)t * red_stride;
+    if (add) { const float4 o = *dst; v.x += o.x; v.y += o.y; }
+    *dst = v;
+  }
+}
 __device__ __forceinline__ float4 sum_parts(const float4* red, int nw) {
   float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 8
@@ -232,7 +263,30 @@ __device__ __forceinline__ uint4 scale8(const uint4& v, const uint4& g) {
   return make_uint4(scale2(v.x, g.x), scale2(v.y, g.y), scale2(v.z, g.z), scale2(v.w, g.w));
 }
 
-template <int MB, bool GAINS>
+// Eight fp32 values (times eight bf16 gains) as three bf16 terms; a value beyond bf16's range keeps its infinity or NaN in the first.
+__device__ __forceinline__ void split_pair(float x0, float x1, unsigned& hi, unsigned& mid, unsigned& lo) {
+  constexpr float kMax = 3.38e38f;
+  hi = pack_bf(x0, x1);
+  x0 = fabsf(x0) <= kMax ? x0 - lo_f(hi) : 0.f; x1 = fabsf(x1) <= kMax ? x1 - hi_f(hi) : 0.f;
+  mid = pack_bf(x0, x1);
+  lo = pack_bf(x0 - lo_f(mid), x1 - hi_f(mid));
+}
+__device__ __forceinline__ void split8(const uint4& v0, const uint4& v1, const uint4& g, bool scaled, uint4 (&t)[3]) {
+  float x[8] = {__uint_as_float(v0.x), __uint_as_float(v0.y), __uint_as_float(v0.z), __uint_as_float(v0.w),
+                __uint_as_float(v1.x), __uint_as_float(v1.y), __uint_as_float(v1.z), __uint_as_float(v1.w)};
+  if (scaled) {
+    x[0] *= lo_f(g.x); x[1] *= hi_f(g.x); x[2] *= lo_f(g.y); x[3] *= hi_f(g.y);
+    x[4] *= lo_f(g.z); x[5] *= hi_f(g.z); x[6] *= lo_f(g.w); x[7] *= hi_f(g.w);
+  }
+  split_pair(x[0], x[1], t[0].x, t[1].x, t[2].x); split_pair(x[2], x[3], t[0].y, t[1].y, t[2].y);
+  split_pair(x[4], x[5], t[0].z, t[1].z, t[2].z); split_pair(x[6], x[7], t[0].w, t[1].w, t[2].w);
+}
+__device__ __forceinline__ float ssq4(const uint4& w) {
+  const float a = __uint_as_float(w.x), b = __uint_as_float(w.y), c = __uint_as_float(w.z), d = __uint_as_float(w.w);
+  return (a * a + b * b) + (c * c + d * d);
+}
+
+template <int MB, bool GAINS, bool FULL>
 __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __grid_constant__ DecodeParams p, const DecLayout L, const DecWords W) {
   extern __shared__ __align__(128) unsigned char smem[];
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem);
@@ -257,6 +311,10 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
   const bool has0 = g < B, has1 = MB == 2 && g + 8 < B;
   const int pairs = B * H;
   SyncArea* const sync = p.sync;
+  static_assert(!FULL || MB == 1, "three terms take the rows of sequences 8 to 15");
+  constexpr int KP = FULL ? 2 : 4, NP = FULL ? 2 : MB;         // blocks of 32 k in flight (FULL: two, or the terms would not fit the registers); 16-byte pieces per block and thread
+  constexpr int kPiece = FULL ? 16 : 512;                      // bytes between the pieces
+  const int vec_at = FULL ? g * 128 + c * 32 : g * 64 + c * 16;
 
   if (tid == 0) {
     *s_abort = 0;
@@ -327,14 +385,13 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
     // =================== 1. projections of x = z^{l-1} (all five matrices in one pass) ===================
     if (warp < kMvWarps) {
       const int nkp = d >> 5, per = (nkp + kMvWarps - 1) / kMvWarps, kp0 = warp * per, kp1 = min(kp0 + per, nkp);
-      constexpr int KP = 4;
-      float sq0 = 0.f, sq1 = 0.f;
+      float sq0 = 0.f, sq1 = 0.f;                              // (FULL: of x, which is z in the storage type, and of z)
       const int m_lo = last ? 3 : 0, m_hi = l == 0 ? 3 : 5;
       if (kp0 >= kp1)
         for (int t = m_lo * nt_d; t < m_hi * nt_d; ++t) red[(t * kMvWarps + warp) * 32 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
       for (int k0 = kp0; k0 < kp1; k0 += KP) {
         const int n = min(KP, kp1 - k0);
-        uint4 a[KP][MB];
+        uint4 a[KP][MB], zf[FULL ? KP : 1][2], zt[FULL ? KP : 1][3];
         if (l == 0) {
 #pragma unroll
           for (int i = 0; i < KP; ++i)
@@ -349,8 +406,16 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
                 a[i][r] = *reinterpret_cast<const uint4*>(row + (k0 + i) * 32 + 8 * c);
               }
             }
+        } else if constexpr (FULL) {
+          poll_vec<2, KP, kPiece>(xw - W.bytes + W.z + (size_t)k0 * 1024 + vec_at, n, has0, has0, zf, sync, s_abort);
+#pragma unroll
+          for (int i = 0; i < KP; ++i) {
+            split8(zf[i][0], zf[i][1], zf[i][0], false, zt[i]);
+            a[i][0] = zt[i][0];
+            sq1 += ssq4(zf[i][0]) + ssq4(zf[i][1]);
+          }
         } else {
-          poll_vec<MB, KP>(xw - W.bytes + W.z + (size_t)k0 * 1024 + g * 64 + c * 16, n, has0, has1, a, sync, s_abort);
+          poll_vec<MB, KP, kPiece>(xw - W.bytes + W.z + (size_t)k0 * 1024 + vec_at, n, has0, has1, a, sync, s_abort);
         }
 #pragma unroll
         for (int i = 0; i < KP; ++i) { sq0 += ssq8(a[i][0]); if (MB == 2) sq1 += ssq8(a[i][MB - 1]); }
@@ -372,7 +437,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
             for (int r = 0; r < MB; ++r) ag[i][r] = scaled ? scale8(a[i][r], gv) : a[i][r];
           }
           const int m0 = set == 0 ? 0 : 3, nm = set == 0 ? 3 : 2;
-          tile_products<MB, KP>(ag, n, nm * nt_d, red + ((size_t)m0 * nt_d * kMvWarps + warp) * 32 + lane, kMvWarps * 32, k0 > kp0, [&](int t) {
+          auto weight_row = [&](int t) {
             const int m = m0 + t / nt_d, r0 = (t % nt_d) * 8, r = r0 + (g < nd - r0 ? g : nd - r0 - 1);
             const unsigned char* base; size_t rs;
             const int lw = m < 3 ? l : l - 1;
@@ -381,7 +446,20 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
             else if (m == 1 || m == 3) slice(L.has_d, kv_off, L.stride_d, p.layer[lw].w_k, d_lo, d, base, rs);
             else slice(L.has_d, kv_off + wd_bytes, L.stride_d, p.layer[lw].w_v, d_lo, d, base, rs);
             return base + (size_t)r * rs + (size_t)k0 * 64 + c * 16;
-          });
+          };
+          float4* dst = red + ((size_t)m0 * nt_d * kMvWarps + warp) * 32 + lane;
+          if constexpr (FULL) {
+            if (set == 1) {                                    // the pair comes from z in fp32
+              if (scaled) {
+#pragma unroll
+                for (int i = 0; i < KP; ++i)
+                  split8(zf[i][0], zf[i][1], *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(gain) + (k0 + (i < n ? i : 0)) * 32 + 8 * c), true, zt[i]);
+              }
+              tile_products3<KP>(zt, n, nm * nt_d, dst, kMvWarps * 32, k0 > kp0, weight_row);
+              continue;
+            }
+          }
+          tile_products<MB, KP>(ag, n, nm * nt_d, dst, kMvWarps * 32, k0 > kp0, weight_row);
         }
       }
       sq0 += __shfl_xor_sync(0xffffffffu, sq0, 1); sq0 += __shfl_xor_sync(0xffffffffu, sq0, 2);
@@ -396,7 +474,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
           float s0 = 0.f, s1 = 0.f;
 #pragma unroll
           for (int w = 0; w < kMvWarps; ++w) { s0 += ssq_red[w * 16 + g]; s1 += ssq_red[w * 16 + 8 + g]; }
-          rs0 = rsqrtf(s0 * inv_d + p.eps); rs1 = rsqrtf(s1 * inv_d + p.eps);
+          rs0 = rsqrtf((FULL && m >= 3 ? s1 : s0) * inv_d + p.eps); rs1 = rsqrtf(s1 * inv_d + p.eps);
         }
         if (rl < nd) {
           unsigned char* dst = xw + W.raw + ((size_t)m * B * d + d_lo + rl) * 4;
@@ -562,7 +640,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
             a0 = fmaf(f, ow.x, a0); a1 = fmaf(f, ow.y, a1); den = fmaf(f, src[kHeadDim + 1], den);
           }
           const float inv = 1.0f / den;
-          st_word(xw + W.c + vec_off(b, h * kHeadDim + 2 * lane), pack_bf(a0 * inv, a1 * inv));
+          st_pair<FULL>(xw + W.c, b, h * kHeadDim + 2 * lane, a0 * inv, a1 * inv);
         }
         if (cta + (k + 2) * G < pairs) asm volatile("bar.sync %0, 256;" ::"r"(2 + half) : "memory");
       }
@@ -595,7 +673,6 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
       }
     } else {
       const int nkp = d >> 5, per = (nkp + kMvWarps - 1) / kMvWarps, kp0 = warp * per, kp1 = min(kp0 + per, nkp);
-      constexpr int KP = 4;
 #pragma unroll 1
       for (int ph = 4; ph <= 5; ++ph) {
         // =================== 4. h = x + alpha W_o c     5. g = GELU(W_up RMS(h)) ===================
@@ -608,9 +685,18 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
           for (int t = 0; t < tiles; ++t) red[(t * kMvWarps + warp) * 32 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int k0 = kp0; k0 < kp1; k0 += KP) {
           const int n = min(KP, kp1 - k0);
-          uint4 a[KP][MB];
-          poll_vec<MB, KP>(xw + (ph == 4 ? W.c : W.h) + (size_t)k0 * 1024 + g * 64 + c * 16, n, has0, has1, a, sync, s_abort);
-          if (ph == 5) {
+          uint4 a[KP][NP], at[FULL ? KP : 1][3];
+          poll_vec<NP, KP, kPiece>(xw + (ph == 4 ? W.c : W.h) + (size_t)k0 * 1024 + vec_at, n, has0, FULL ? has0 : has1, a, sync, s_abort);
+          if constexpr (FULL) {
+            const bool scaled = GAINS && ph == 5 && pre && ly.g_mlp;
+#pragma unroll
+            for (int i = 0; i < KP; ++i) {
+              uint4 gv = make_uint4(0u, 0u, 0u, 0u);
+              if (scaled) gv = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(ly.g_mlp) + (k0 + (i < n ? i : 0)) * 32 + 8 * c);
+              split8(a[i][0], a[i][1], gv, scaled, at[i]);
+              sq0 += ssq4(a[i][0]) + ssq4(a[i][1]);
+            }
+          } else if (ph == 5) {
 #pragma unroll
             for (int i = 0; i < KP; ++i) { sq0 += ssq8(a[i][0]); if (MB == 2) sq1 += ssq8(a[i][MB - 1]); }
             if (GAINS && pre && ly.g_mlp) {
@@ -626,10 +712,12 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
             if (ph == 4) { if (L.has_d) mbar_wait(bar_q, 1, s_abort, sync); }
             else if (L.has_up) mbar_wait(bar_up, l & 1, s_abort, sync);
           }
-          tile_products<MB, KP>(a, n, tiles, red + warp * 32 + lane, kMvWarps * 32, k0 > kp0, [&](int t) {
+          auto weight_row = [&](int t) {
             const int r0 = t * 8, r = r0 + (g < rows - r0 ? g : rows - r0 - 1);
             return base + (size_t)r * rs + (size_t)k0 * 64 + c * 16;
-          });
+          };
+          if constexpr (FULL) tile_products3<KP>(at, n, tiles, red + warp * 32 + lane, kMvWarps * 32, k0 > kp0, weight_row);
+          else tile_products<MB, KP>(a, n, tiles, red + warp * 32 + lane, kMvWarps * 32, k0 > kp0, weight_row);
         }
         if (ph == 5) {
           sq0 += __shfl_xor_sync(0xffffffffu, sq0, 1); sq0 += __shfl_xor_sync(0xffffffffu, sq0, 2);
@@ -656,7 +744,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
               }
               const float h0 = lo_f(xv) + p.alpha * (r ? y.z : y.x), h1 = hi_f(xv) + p.alpha * (r ? y.w : y.y);
               *reinterpret_cast<float2*>(hown + b * L.max_nd + rl) = make_float2(h0, h1);
-              st_word(xw + W.h + vec_off(b, d_lo + rl), pack_bf(h0, h1));
+              st_pair<FULL>(xw + W.h, b, d_lo + rl, h0, h1);
             }
           } else {
             float rs0 = 1.f, rs1 = 1.f;
@@ -666,8 +754,8 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
               for (int w = 0; w < kMvWarps; ++w) { s0 += ssq_red[w * 16 + g]; s1 += ssq_red[w * 16 + 8 + g]; }
               rs0 = rsqrtf(s0 * inv_d + p.eps); rs1 = rsqrtf(s1 * inv_d + p.eps);
             }
-            if (has0) st_word(xw + W.g + vec_off(g, f_lo + rl), pack_bf(gelu_erf(y.x * rs0), gelu_erf(y.y * rs0)));
-            if (has1) st_word(xw + W.g + vec_off(g + 8, f_lo + rl), pack_bf(gelu_erf(y.z * rs1), gelu_erf(y.w * rs1)));
+            if (has0) st_pair<FULL>(xw + W.g, g, f_lo + rl, gelu_erf(y.x * rs0), gelu_erf(y.y * rs0));
+            if (has1) st_pair<FULL>(xw + W.g, g + 8, f_lo + rl, gelu_erf(y.z * rs1), gelu_erf(y.w * rs1));
           }
         }
         bar_named<1, kMvWarps * 32>();                         // red may be written again; the slice's place is free
@@ -678,20 +766,24 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
     {
       // =================== 6. z = h + alpha W_down g, all sixteen warps ===================
       const int nkp = dff >> 5, per = (nkp + kDecWarps - 1) / kDecWarps, kp0 = warp * per, kp1 = min(kp0 + per, nkp);
-      constexpr int KP = 4;
       const unsigned char* base; size_t rs;
       slice(L.has_dn, L.off_dn, L.stride_f, ly.w_down, d_lo, dff, base, rs);
       if (kp0 >= kp1)
         for (int t = 0; t < nt_d; ++t) red[(t * kDecWarps + warp) * 32 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
       for (int k0 = kp0; k0 < kp1; k0 += KP) {
         const int n = min(KP, kp1 - k0);
-        uint4 a[KP][MB];
-        poll_vec<MB, KP>(xw + W.g + (size_t)k0 * 1024 + g * 64 + c * 16, n, has0, has1, a, sync, s_abort);
+        uint4 a[KP][NP], at[FULL ? KP : 1][3];
+        poll_vec<NP, KP, kPiece>(xw + W.g + (size_t)k0 * 1024 + vec_at, n, has0, FULL ? has0 : has1, a, sync, s_abort);
         if (k0 == kp0 && L.has_dn) mbar_wait(bar_dn, l & 1, s_abort, sync);
-        tile_products<MB, KP>(a, n, nt_d, red + warp * 32 + lane, kDecWarps * 32, k0 > kp0, [&](int t) {
+        auto weight_row = [&](int t) {
           const int r0 = t * 8, r = r0 + (g < nd - r0 ? g : nd - r0 - 1);
           return base + (size_t)r * rs + (size_t)k0 * 64 + c * 16;
-        });
+        };
+        if constexpr (FULL) {
+#pragma unroll
+          for (int i = 0; i < KP; ++i) split8(a[i][0], a[i][1], a[i][0], false, at[i]);
+          tile_products3<KP>(at, n, nt_d, red + warp * 32 + lane, kDecWarps * 32, k0 > kp0, weight_row);
+        } else tile_products<MB, KP>(a, n, nt_d, red + warp * 32 + lane, kDecWarps * 32, k0 > kp0, weight_row);
       }
       __syncthreads();
       if (warp == kDecWarps - 1 && l + 1 < n_layers) fetch_dn(l + 1);
@@ -705,8 +797,9 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_stack_kernel(const __gr
             const int b = g + 8 * r;
             if (b >= B) continue;
             const float2 h = *reinterpret_cast<const float2*>(hown + b * L.max_nd + rl);
-            const unsigned zw = pack_bf(h.x + p.alpha * (r ? y.z : y.x), h.y + p.alpha * (r ? y.w : y.y));
-            st_word(xw + W.z + vec_off(b, d_lo + rl), zw);
+            const float z0 = h.x + p.alpha * (r ? y.z : y.x), z1 = h.y + p.alpha * (r ? y.w : y.y);
+            const unsigned zw = pack_bf(z0, z1);
+            st_pair<FULL>(xw + W.z, b, d_lo + rl, z0, z1);
             *reinterpret_cast<unsigned*>(zown + b * L.max_nd + rl) = zw;
             if (l == n_layers - 1)
               *reinterpret_cast<unsigned*>(reinterpret_cast<__nv_bfloat16*>(p.z_out) + (size_t)b * p.z_bs + d_lo + rl) = zw;
@@ -757,7 +850,7 @@ int seg_bound(int quads, int grid) { return ceil_div(grid, quads) + 2; }
 
 }  // namespace
 
-int decode_slice(int B) { return ceil_div(B, ceil_div(B, 16)); }
+int decode_slice(int B, bool full) { return ceil_div(B, ceil_div(B, full ? 8 : 16)); }
 
 // Widths in whole 64-byte blocks whose reduction buffers leave room in shared memory (five d-wide matrices at once: d up to about 12000 with
 // d_ff = 4 d; d_ff up to about 65000), and no more groups of four pairs than warps (pure arithmetic).
@@ -810,8 +903,10 @@ cudaError_t decode_launch(const DecodeParams& p0, cudaStream_t s) {
   bool gains = false;
   for (int l = 0; l < p.n_layers; ++l)
     gains = gains || p.layer[l].g_attn || p.layer[l].g_mlp || p.layer[l].g_kv || p.layer[l].g_q || p.layer[l].g_k;
-  const void* fn = p.B > 8 ? (gains ? (const void*)&decode_stack_kernel<2, true> : (const void*)&decode_stack_kernel<2, false>)
-                           : (gains ? (const void*)&decode_stack_kernel<1, true> : (const void*)&decode_stack_kernel<1, false>);
+  if (p.B > (p.full ? 8 : 16)) return cudaErrorInvalidConfiguration;
+  const void* fn = p.full ? (gains ? (const void*)&decode_stack_kernel<1, true, true> : (const void*)&decode_stack_kernel<1, false, true>)
+                   : p.B > 8 ? (gains ? (const void*)&decode_stack_kernel<2, true, false> : (const void*)&decode_stack_kernel<2, false, false>)
+                             : (gains ? (const void*)&decode_stack_kernel<1, true, false> : (const void*)&decode_stack_kernel<1, false, false>);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(p.words, 0xff, (size_t)(p.n_layers + 1) * W.bytes, s);

@@ -180,6 +180,7 @@ struct DecLayer {
 };
 struct DecodeParams {
   int n_layers, B, d, H, dff;                      // B: sequences of this launch
+  int full;                                        // 1: the vectors between the phases stay fp32 (at most eight sequences)
   int pos;                                         // positions in the caches
   int Bs, b0;                                      // sequences per cache row, first of this launch
   int norm_flags;
@@ -194,8 +195,8 @@ struct DecodeParams {
   int quads, chunks, chunk_len, warps_per_cta, pf_keys;   // attention split, set by the launcher
 };
 bool decode_shape(int B, int d, int H, int dff);   // whether the kernel takes the slices of a batch of B
-// Sequences per launch: a batch above 16 runs as slices of equal size (the sequences are independent), the last one with what is left.
-int decode_slice(int B);
+// Sequences per launch: a batch above 16 (full: above eight) runs as slices of equal size (the sequences are independent), the last one with what is left.
+int decode_slice(int B, bool full);
 // Bytes of exchange area for the slices of a batch of at most B, one after the other (0: the kernel does not take the shape).
 size_t decode_words_bytes(int n_layers, int B, int d, int H, int dff);
 cudaError_t decode_launch(const DecodeParams& p, cudaStream_t s);

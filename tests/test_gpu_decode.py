@@ -89,3 +89,27 @@ def test_decode_slices_stay_inside_the_workspace(d, H, B, L):
     assert bool((ws[need:] == 0x5a).all())
     got = logits.double().cpu().numpy()
     assert np.abs(got - ref).max() <= 2 * TOL * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("d,H,dff,B,pos,leaf,gains", [
+    (512, 8, 2048, 17, 40, 0, True), (256, 4, 1024, 48, 9, 0, False), (512, 8, 2048, 12, 0, 0, True), (512, 8, 2048, 5, 70, 128, False),
+    (1408, 22, 5632, 3, 30, 0, True), (192, 3, 224, 33, 3, 0, True)])
+def test_decode_keeps_fp32_between_the_phases(d, H, dff, B, pos, leaf, gains):
+    # Batches above 16, a first position, layers off the tensor-core leaf kernel.  2-norms: the rounding of the result to bf16 is 1.7e-3 of
+    # it, the rounded q, k~, v~ bring that to 1.9e-3, at a first position, where v~ is not averaged, to 2.4e-3.  With c, h, g, z rounded on
+    # the way k and v come to 2.6e-3 .. 3.0e-3, at a first position to 3.5e-3.
+    import torch
+    from oracle import RTConfig, RTWeights, layer_seq
+    from paper_2604_21215_b200 import rt
+    x, lw = _case(d, H, dff, B, pos + 1, 7 * pos + B, gains)
+    ref = layer_seq(RTConfig(d, H, 64, dff), RTWeights(**lw), x)
+    layer = rt.Layer(d, H, dff, dtype="bf16", leaf=leaf)
+    layer.set_weights(lw)
+    layer.reserve(B, 1, pos + 1)
+    for cache, r in ((layer.k_cache, ref[1]), (layer.v_cache, ref[2])):
+        cache[:pos] = torch.from_numpy(np.ascontiguousarray(r[:, :pos].transpose(1, 0, 2))).to(cache)
+    z = layer.decode(x[:, pos], pos)
+    rows = [c[pos].to(torch.float64).cpu().numpy() for c in (layer.k_cache, layer.v_cache)]
+    for name, got, want in (("z", z, ref[0][:, pos]), ("k", rows[0], ref[1][:, pos]), ("v", rows[1], ref[2][:, pos])):
+        err = np.linalg.norm(got - want) / np.linalg.norm(want)
+        assert err <= (2.25e-3 if pos else 2.6e-3), (name, err)
