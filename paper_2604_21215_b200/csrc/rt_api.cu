@@ -55,6 +55,7 @@ enum ChainPath { kPathGeneric = 0, kPathMma = 1, kPathWide = 2, kPathBlocks = 3,
 struct Schedule { ChainPath path; int leaf; int sub; };      // sub: sequences per slice (kPathMmaSplit, kPathGroups)
 constexpr int kWideLeafDefault = 16;    // leaf of the dense-product token steps: the in-leaf attention re-reads the leaf's pairs for every position,
                                         // so short leaves win (p512: 16 -> 41.6 ms, 32 -> 42.3, 64 -> 45.9 per layer)
+constexpr int kWideFrom = 24;            // smallest bf16 batch that runs as dense products rather than through the generic kernel
 constexpr int kMmaSplitMax = 48;         // largest batch that runs as slices of at most 16 sequences through the tensor-core leaf kernel
 constexpr int kGroupsMax = 64;           // largest batch that runs as slices of at most 16 sequences side by side on groups of SMs
 Schedule effective_schedule(const rt_config* c, int B) {
@@ -62,9 +63,12 @@ Schedule effective_schedule(const rt_config* c, int B) {
   if (c->sched == RT_SCHED_TILED) {
     LeafMmaLaunch ml;
     if (c->dtype == RT_BF16 && B > 16 && B <= kGroupsMax) {
-      // slices side by side, a group of SMs each (rt_leaf_group.cu)
+      // slices side by side, a group of SMs each (rt_leaf_group.cu), unless the layer would otherwise take the generic kernel: that one holds
+      // the vectors between the phases in fp32, the others round them to bf16 (d = 512, B = 20, leaves of 128: error of k against 64 bits
+      // 1.9e-3 and 3.0e-3)
       const int n_sub = ceil_div(B, 16), sub = ceil_div(B, n_sub);
-      if (leaf_group_shape(sub, c->d_model, c->n_heads, c->d_ff, n_sub, kB200SmemPerCta))
+      if (leaf_group_shape(sub, c->d_model, c->n_heads, c->d_ff, n_sub, kB200SmemPerCta) &&
+          (B >= kWideFrom || leaf_mma_shape(sub, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml)))
         return {kPathGroups, c->leaf ? c->leaf : kAutoLeaf, sub};
     }
     if (c->dtype == RT_BF16 && B > 16 && B <= kMmaSplitMax) {
@@ -78,7 +82,7 @@ Schedule effective_schedule(const rt_config* c, int B) {
     // bf16 batches beyond that (or whose slices the tensor-core leaf kernel does not take) run as dense products from
     // 24 sequences on, where they overtake the generic kernel (measured at d = 1024: 53 us per token step at B = 32
     // against 99 us); fp32 keeps the generic kernel up to its limit
-    if (B > kSmallBatchMax || (c->dtype == RT_BF16 && B >= 24)) return {kPathWide, c->leaf ? c->leaf : kWideLeafDefault, 0};
+    if (B > kSmallBatchMax || (c->dtype == RT_BF16 && B >= kWideFrom)) return {kPathWide, c->leaf ? c->leaf : kWideLeafDefault, 0};
     if (c->dtype == RT_BF16 && leaf_mma_shape(B, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml))
       return {kPathMma, ml.leaf, B};
   }
@@ -96,6 +100,8 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
   if (n_layers < 2 || N < 2 || c->dtype != RT_BF16 || c->sched != RT_SCHED_TILED || c->recur_block > 1) return none;
   const int places = n_layers < kGroupJobs ? n_layers : kGroupJobs;
   if (!leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, places, kB200SmemPerCta)) return none;
+  LeafMmaLaunch ml;                                            // (a stack of layers for the generic kernel keeps its fp32 vectors)
+  if (!leaf_mma_shape(B, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml)) return none;
   // A leaf meets all earlier pairs at once when its queries exist (they depend on the layer below, so Algorithm 1's tiles cannot
   // run ahead): each leaf reads the layer's whole cache so far, which a launch hides only while that is short.  Longer
   // sequences go layer by layer, as the same layers called one by one do (and give the same bits).

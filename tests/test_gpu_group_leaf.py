@@ -81,3 +81,45 @@ def test_a_workspace_for_long_prompts_serves_short_ones(L, B, N):
         stacks.append((hid, [k[:N] for k in st.k_caches]))
     assert torch.equal(stacks[0][0], stacks[1][0])
     assert all(torch.equal(a, b) for a, b in zip(stacks[0][1], stacks[1][1]))
+
+
+def _leaf128(L, B, N):
+    from paper_2604_21215_b200 import inputs
+    d, H, dff, V = 512, 8, 1024, 91
+    data = inputs.make_inputs(inputs.Workload("wave", L, B, N, d, H, dff, "bf16", vocab=V, residual_scale=1 / np.sqrt(L)), seed=N)
+    return d, H, dff, V, data
+
+
+def test_a_stack_of_generic_layers_keeps_their_arithmetic():
+    # leaves of 128 positions do not fit the tensor-core leaf kernel: the layers take the generic kernel, whose vectors stay fp32, also in a stack
+    import torch
+    from paper_2604_21215_b200 import rt
+    L, B, N = 3, 3, 150
+    d, H, dff, V, data = _leaf128(L, B, N)
+    kw = dict(dtype="bf16", leaf=128, residual_scale=1 / np.sqrt(L))
+    st = rt.Stack(L, d, H, dff, V, **kw)
+    st.set_weights(data["layers"], data["emb"])
+    hid, _ = st.prefill(data["ids"])
+    x = st.emb[torch.as_tensor(data["ids"], dtype=torch.long, device=st.device)].double().cpu().numpy()
+    for l in range(L):
+        layer = rt.Layer(d, H, dff, **kw)
+        layer.set_weights(data["layers"][l])
+        x, k, v = layer.prefill(x)
+        got = st.caches_numpy(N)[l]
+        assert np.array_equal(got[0], k) and np.array_equal(got[1], v)
+    assert np.array_equal(hid, x)
+
+
+def test_a_batch_on_the_generic_kernel_keeps_its_arithmetic():
+    # the same layer with 20 sequences: as five batches of four, which are too few for the group kernel
+    from paper_2604_21215_b200 import rt
+    B, N = 20, 140
+    d, H, dff, V, data = _leaf128(1, B, N)
+    x = np.random.default_rng(3).standard_normal((B, N, d))
+    outs = []
+    for lo, hi in ((0, B), (0, 4), (4, 8), (8, 12), (12, 16), (16, 20)):
+        layer = rt.Layer(d, H, dff, dtype="bf16", leaf=128)
+        layer.set_weights(data["layers"][0])
+        outs.append(layer.prefill(x[lo:hi]))
+    for i in range(3):
+        assert np.array_equal(outs[0][i], np.concatenate([o[i] for o in outs[1:]]))
