@@ -590,6 +590,16 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   return RT_OK;
 }
 
+// Whether any two caches share rows.  Layers one after the other may (a program that wants the logits only can give every layer the same
+// pair); side by side they write their rows at the same time.
+bool caches_overlap(const rt_config* c, int n_layers, int B, int N, void* const* k_caches, void* const* v_caches) {
+  const size_t bytes = (size_t)N * B * c->d_model * esize_of(c->dtype);
+  for (int i = 0; i < 2 * n_layers; ++i)
+    for (int j = 0; j < i; ++j)
+      if (overlaps(i < n_layers ? k_caches[i] : v_caches[i - n_layers], bytes, j < n_layers ? k_caches[j] : v_caches[j - n_layers], bytes)) return true;
+  return false;
+}
+
 // All layers of a stack, several at a time (stack_wave): x^0 in hid[0], layer l reads hid[l & 1] and writes hid[(l + 1) & 1] (the
 // last one `out`, if given); a row is overwritten only after the layer that reads it has finished it.
 rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weights* layers, void* const* hid, void* out, int B, int N, void* const* k_caches,
@@ -939,7 +949,8 @@ rt_status rt_stack_prefill(const rt_config* cfg, int32_t n_layers, const rt_laye
     if (embed_launch(cfg->dtype, emb, ids, B, N, (int)d, vocab, bufs[0], s) != cudaSuccess) return RT_ERR_CUDA;
   }
   const void* cur = bufs[0];
-  const Wave wv = stack_wave(cfg, B, N, n_layers);
+  Wave wv = stack_wave(cfg, B, N, n_layers);
+  if (wv.places && caches_overlap(cfg, n_layers, B, N, k_caches, v_caches)) wv.places = 0;
   if (wv.places) {
     st = run_stack_wave(cfg, n_layers, layers, bufs, hidden, B, N, k_caches, v_caches, N_max, ws, L, wv, ctx);
     if (st != RT_OK) return st;

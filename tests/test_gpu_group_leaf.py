@@ -123,3 +123,26 @@ def test_a_batch_on_the_generic_kernel_keeps_its_arithmetic():
         outs.append(layer.prefill(x[lo:hi]))
     for i in range(3):
         assert np.array_equal(outs[0][i], np.concatenate([o[i] for o in outs[1:]]))
+
+
+def test_layers_may_share_one_pair_of_caches():
+    # a program that wants hidden states and logits only gives every layer the same caches
+    import ctypes as C
+    from oracle import RTConfig, RTWeights, stack_prefill
+    from paper_2604_21215_b200 import inputs, rt
+    L, d, H, dff, B, N, V = 5, 512, 8, 1024, 2, 100, 91
+    wl = inputs.Workload("wave", L, B, N, d, H, dff, "bf16", vocab=V, residual_scale=1 / np.sqrt(L))
+    data = inputs.make_inputs(wl, seed=6)
+    hid_ref, logits_ref, caches_ref = stack_prefill(RTConfig(d, H, 64, dff, residual_scale=wl.residual_scale), [RTWeights(**w) for w in data["layers"]],
+                                                    data["emb"], None, data["ids"])
+    st = rt.Stack(L, d, H, dff, V, dtype="bf16", residual_scale=wl.residual_scale)
+    st.set_weights(data["layers"], data["emb"])
+    st.reserve(B, N)
+    st._kp = (C.c_void_p * L)(*[st.k_caches[0].data_ptr()] * L)
+    st._vp = (C.c_void_p * L)(*[st.v_caches[0].data_ptr()] * L)
+    hid, logits = st.prefill(data["ids"])
+    check_tensor("shared caches", "hidden", hid, hid_ref, 2e-2)
+    assert np.abs(logits - logits_ref).max() <= 2e-2 * np.abs(logits_ref).max()
+    k, v = st.caches_numpy(N)[0]                                # the last layer's pairs
+    check_tensor("shared caches", "k", k, caches_ref[L - 1][0], 2e-2)
+    check_tensor("shared caches", "v", v, caches_ref[L - 1][1], 2e-2)
