@@ -1596,13 +1596,23 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   BwdLeafParams bl;
   memset(&bl, 0, sizeof(bl));
   if (fast) {
+    // the leaf kernel fetches four entries of a gain at once; the other kernels take gains at any address, so one that is off goes through a
+    // copy in the workspace (the partial column sums, not used before the end)
+    __nv_bfloat16* spare = reinterpret_cast<__nv_bfloat16*>(ws + L.part);
+    auto aligned_gain = [&](const T* g) -> const void* {
+      if (!g || ((uintptr_t)g & 7) == 0) return g;
+      if (cudaMemcpyAsync(spare, g, (size_t)d * sizeof(T), cudaMemcpyDeviceToDevice, s) != cudaSuccess) return nullptr;
+      spare += d;
+      return spare - d;
+    };
     // the exchanged arrays double as their own flags
     for (size_t at : {L.dkraw, L.dvf, L.dr, L.du, L.dc}) RT_TRY(cudaMemsetAsync(ws + at, 0xff, rows * d * sizeof(float), s));
     RT_TRY(cudaMemsetAsync(ws + L.dpre, 0xff, rows * f * sizeof(float), s));
     bl.Bs = B; bl.d = d; bl.H = H; bl.dff = f; bl.z_norm = z_norm ? 1 : 0; bl.pre = pre ? 1 : 0; bl.qk = qk ? 1 : 0;
     bl.eps = eps; bl.alpha = alpha; bl.scale = c->softmax_scale; bl.scale_log2 = ab.scale_log2;
     bl.wkT = WkT; bl.wvT = WvT; bl.wdnT = WdnT; bl.wupT = WupT; bl.woT = WoT;
-    bl.g_k = g_k; bl.g_kv = g_kv; bl.g_mlp = g_mlp; bl.alibi = w->alibi_slopes;
+    bl.g_k = g_k; bl.g_kv = aligned_gain(g_kv); bl.g_mlp = aligned_gain(g_mlp); bl.alibi = w->alibi_slopes;
+    if ((g_kv && !bl.g_kv) || (g_mlp && !bl.g_mlp)) return RT_ERR_CUDA;
     bl.z = z; bl.z_bs = xbs; bl.z_ts = xts; bl.dz = dz; bl.dz_bs = xbs; bl.dz_ts = xts;
     bl.q = ab.q; bl.k = ab.k; bl.v = ab.v; bl.kt = ab.kt; bl.vt = ab.vt; bl.c = ab.c; bl.lse = ab.lse; bl.kraw = F(L.kraw); bl.h = F(L.h); bl.act = F(L.act);
     bl.dK = F(L.dK); bl.dV = F(L.dV); bl.dvf = F(L.dvf); bl.dkraw = F(L.dkraw); bl.dr = F(L.dr); bl.Gz = F(L.Gz); bl.dpre = F(L.dpre);

@@ -72,3 +72,30 @@ def test_loop_of_up_to_32_sequences(d, H, dff, B, N, flags, gains, alibi, alpha)
     (128, 2, 256, 1030, 18, 3, ("g_k", "g_kv"), False, 1.0)])                # too many groups: the launches of every position
 def test_dense_products_over_wide_batches(d, H, dff, B, N, flags, gains, alibi, alpha):
     _check(d, H, dff, B, N, flags, gains, alibi, alpha)
+
+
+def test_gains_at_any_address():
+    # the backward pass has never asked for aligned gains: views into one packed array give the bits of separate arrays
+    import torch
+    from paper_2604_21215_b200 import inputs, rt
+    d, H, dff, B, N = 256, 4, 1024, 3, 70
+    wl = inputs.Workload("gains", 1, B, N, d, H, dff, "bf16")
+    data = inputs.make_inputs(wl, seed=8)
+    lw = data["layers"][0]
+    rng = np.random.default_rng(2)
+    for g in G_NAMES:
+        lw[g] = inputs.round_to(1.0 + 0.2 * rng.standard_normal(d), "bf16")
+    layer = rt.Layer(d, H, dff, dtype="bf16")
+    layer.set_weights(lw)
+    z, _, _ = layer.prefill(data["x"])
+    dz = rng.standard_normal(z.shape)
+    want = layer.backward(data["x"], z, dz)
+    packed = torch.empty(1 + 5 * (d + 1), dtype=torch.bfloat16, device=layer.device)
+    for i, g in enumerate(G_NAMES):
+        view = packed[1 + i * (d + 1):][:d]                     # the first four 2, 4, 6 and 0 bytes off a multiple of eight
+        view.copy_(torch.as_tensor(lw[g]))
+        setattr(layer.w, g, view.data_ptr())
+    got = layer.backward(data["x"], z, dz)
+    assert np.array_equal(got[0], want[0])
+    for n in want[1]:
+        assert np.array_equal(got[1][n], want[1][n]), n
