@@ -17,6 +17,7 @@
 #include "rt_bwd.cuh"
 #include "rt_common.cuh"
 #include "rt_kernels.h"
+#include "rt_tc.cuh"
 
 namespace rt {
 namespace {
@@ -1541,7 +1542,7 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   if (smem_max > 200 * 1024) return RT_ERR_UNSUPPORTED;
   const void* step_fn = reinterpret_cast<const void*>(&rowmat_kernel<T, 4>);
   const void* loop_fn = reinterpret_cast<const void*>(&bwd_loop_kernel<T, 4>);
-  RT_TRY(cudaFuncSetAttribute(step_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
+  RT_TRY(ensure_dynamic_smem(step_fn, (int)smem_max));
   auto rowmat = [&](int mode, int i, int K, int Ncols, const void* W1, const void* W2, const void* gain, int norm_on, float al, int cols,
                     int nsplit, int n_in) {
     rp.mode = mode; rp.i = i; rp.K = K; rp.Ncols = Ncols; rp.W1 = W1; rp.W2 = W2; rp.gain = gain;
@@ -1549,7 +1550,7 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
     const dim3 grid(rowmat_tasks(rp, rb)), block(kRmThreads);
     return launch_chained(rowmat_kernel<T, 4>, grid, block, smem_max, s, true, rp);
   };
-  RT_TRY(cudaFuncSetAttribute(loop_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
+  RT_TRY(ensure_dynamic_smem(loop_fn, (int)smem_max));
   RT_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bwd_loop_kernel<T, 4>, kRmThreads, smem_max));
   // RT_FLAG_BACKWARD_STEP_LAUNCHES in the configuration forces the one-launch-per-step form (what a device without
   // cooperative launch gets; the tests run both forms)
@@ -1562,7 +1563,7 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   bool resident = false;
   if (use_coop && one_task && smem_max + slice_bytes <= 220 * 1024) {
     int per_sm_res = 0;
-    RT_TRY(cudaFuncSetAttribute(loop_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem_max + slice_bytes)));
+    RT_TRY(ensure_dynamic_smem(loop_fn, (int)(smem_max + slice_bytes)));
     RT_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_res, bwd_loop_kernel<T, 4>, kRmThreads, smem_max + slice_bytes));
     if (per_sm_res >= 1) { resident = true; loop_smem = smem_max + slice_bytes; }
   }

@@ -907,7 +907,7 @@ cudaError_t decode_launch(const DecodeParams& p0, cudaStream_t s) {
   const void* fn = p.full ? (gains ? (const void*)&decode_stack_kernel<1, true, true> : (const void*)&decode_stack_kernel<1, false, true>)
                    : p.B > 8 ? (gains ? (const void*)&decode_stack_kernel<2, true, false> : (const void*)&decode_stack_kernel<2, false, false>)
                              : (gains ? (const void*)&decode_stack_kernel<1, true, false> : (const void*)&decode_stack_kernel<1, false, false>);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+  cudaError_t e = ensure_dynamic_smem(fn, (int)L.total);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(p.words, 0xff, (size_t)(p.n_layers + 1) * W.bytes, s);
   if (e != cudaSuccess) return e;

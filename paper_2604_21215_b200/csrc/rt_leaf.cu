@@ -16,6 +16,7 @@
 // chunk) and reduce with warp shuffles, so every activation element is loaded exactly once
 // per CTA and never staged.
 #include "rt_kernels.h"
+#include "rt_tc.cuh"
 
 namespace rt {
 
@@ -464,7 +465,7 @@ cudaError_t leaf_launch(int dtype, const LeafParams& p_in, const LeafLaunch& l, 
   const int NB = pick_nb(p.B);
   LeafSmemLayout L = leaf_smem_layout(p.B, p.d, p.dff, l.grid, NB, esize);
   const void* fn = dtype == RT_BF16 ? leaf_fn<__nv_bfloat16>(NB) : leaf_fn<float>(NB);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
+  cudaError_t e = ensure_dynamic_smem(fn, (int)l.smem);
   if (e != cudaSuccess) return e;
   void* args[] = {(void*)&p, (void*)&L};
   return cudaLaunchCooperativeKernel(fn, dim3(l.grid), dim3(l.block), args, l.smem, s);

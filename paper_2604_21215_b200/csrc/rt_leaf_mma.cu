@@ -706,7 +706,7 @@ cudaError_t leaf_mma_launch(const LeafParams& p, const LeafMmaLaunch& l, const L
     return l.q_smem ? pick2(mb, std::true_type{}) : pick2(mb, std::false_type{});
   };
   const void* fn = p.B > 8 ? pick(std::integral_constant<int, 2>{}) : pick(std::integral_constant<int, 1>{});
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
+  cudaError_t e = ensure_dynamic_smem(fn, (int)l.smem);
   if (e != cudaSuccess) return e;
   LeafParams pp = p;
   LeafMmaBuffers b = buf;

@@ -426,7 +426,7 @@ bool leaf_small_shape(int dtype, int B, int d, int H, int dff, int leaf, size_t 
 cudaError_t leaf_small_launch(int dtype, const LeafParams& p, const LeafSmallLaunch& l, cudaStream_t s) {
   const SmallLayout L = small_layout(dtype == RT_BF16 ? 2 : 4, l.nb, p.d, p.dff);
   auto go = [&](auto kernel) -> cudaError_t {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), (int)L.total);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;

@@ -2,6 +2,7 @@
 // logits = E . RMS_{g_final}(x^L) at one position per sequence.  The paper treats both as those
 // of an ordinary Transformer (Sec. 6, "The setup") and leaves them out of its latency numbers.
 #include "rt_kernels.h"
+#include "rt_tc.cuh"
 
 namespace rt {
 
@@ -159,7 +160,7 @@ cudaError_t head_launch(int dtype, const void* emb, const void* g_final, const v
   cudaError_t e;
   if (dtype == RT_BF16 && B <= 16 && d % 16 == 0 && (size_t)2 * 16 * (d + 16) * 2 <= 200 * 1024) {
     const size_t sm2 = (size_t)2 * 16 * (d + 16) * 2;
-    e = cudaFuncSetAttribute(head_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+    e = ensure_dynamic_smem(reinterpret_cast<const void*>(&head_mma_kernel), (int)sm2);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -169,13 +170,13 @@ cudaError_t head_launch(int dtype, const void* emb, const void* g_final, const v
                           (const __nv_bfloat16*)hidden, h_bs, B, d, vocab, norm_flags, eps, logits);
   }
   if (dtype == RT_BF16) {
-    e = cudaFuncSetAttribute(head_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = ensure_dynamic_smem(reinterpret_cast<const void*>(&head_kernel<__nv_bfloat16>), (int)smem);
     if (e != cudaSuccess) return e;
     head_kernel<__nv_bfloat16><<<blocks, 256, smem, s>>>((const __nv_bfloat16*)emb, (const __nv_bfloat16*)g_final,
                                                          (const __nv_bfloat16*)hidden, h_bs, B, d, vocab, norm_flags,
                                                          eps, logits);
   } else {
-    e = cudaFuncSetAttribute(head_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = ensure_dynamic_smem(reinterpret_cast<const void*>(&head_kernel<float>), (int)smem);
     if (e != cudaSuccess) return e;
     head_kernel<float><<<blocks, 256, smem, s>>>((const float*)emb, (const float*)g_final, (const float*)hidden, h_bs,
                                                  B, d, vocab, norm_flags, eps, logits);

@@ -180,19 +180,25 @@ inline bool tensor_map_rows_bf16(CUtensorMap* out, const void* base, long long r
   return true;
 }
 
-// cudaFuncSetAttribute(max dynamic shared memory) once per (kernel, device) instead of before every launch.
+// Lets a kernel take `bytes` of dynamic shared memory, once per (thread, kernel, device) instead of before every launch.  The limit belongs to the
+// kernel and not to the thread that sets it, so it always becomes all that the device has beside the kernel's static arrays: a limit fitted to one
+// launch would take the shared memory from a wider launch of the same kernel by another thread.
 inline cudaError_t ensure_dynamic_smem(const void* fn, int bytes) {
   struct Entry { const void* fn; int dev, bytes; };
-  constexpr int kEntries = 32;
+  constexpr int kEntries = 64;
   thread_local Entry tab[kEntries];
   thread_local int used = 0;
-  int dev = 0;
+  int dev = 0, most = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   for (int i = 0; i < used; ++i)
-    if (tab[i].fn == fn && tab[i].dev == dev && tab[i].bytes >= bytes) return cudaSuccess;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess && used < kEntries) { tab[used].fn = fn; tab[used].dev = dev; tab[used].bytes = bytes; ++used; }
+    if (tab[i].fn == fn && tab[i].dev == dev) return bytes <= tab[i].bytes ? cudaSuccess : cudaErrorInvalidValue;
+  cudaFuncAttributes attr;
+  if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess || (e = cudaFuncGetAttributes(&attr, fn)) != cudaSuccess) return e;
+  most -= (int)attr.sharedSizeBytes;
+  if (bytes > most) return cudaErrorInvalidValue;
+  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess && used < kEntries) { tab[used].fn = fn; tab[used].dev = dev; tab[used].bytes = most; ++used; }
   return e;
 }
 

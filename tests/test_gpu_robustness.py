@@ -501,3 +501,29 @@ def test_decode_over_a_long_cache_matches_oracle(alibi):
     v = layer.v_cache.permute(1, 0, 2).to(torch.float64).cpu().numpy()
     check_tensor("long-cache decode", "k", k, ref[1], TOL["bf16"])
     check_tensor("long-cache decode", "v", v, ref[2], TOL["bf16"])
+
+
+def test_threads_with_layers_of_different_widths():
+    # The limit of a kernel's dynamic shared memory is the kernel's, not the thread's: a narrow layer in one thread must not take it from
+    # a wide one in another (group kernel; decode kernel).
+    import concurrent.futures
+    import torch
+    from paper_2604_21215_b200 import rt
+
+    def make(d, B, **kw):
+        layer = rt.Layer(d, d // 64, 4 * d, dtype="bf16", **kw)
+        gen = torch.Generator(device="cuda:0").manual_seed(d)
+        shapes = {"w_up": (4 * d, d), "w_down": (d, 4 * d)}
+        layer.set_weights({n: torch.randn(shapes.get(n, (d, d)), generator=gen, device="cuda:0") / d ** 0.5 for n in ("w_q", "w_k", "w_v", "w_o", "w_up", "w_down")})
+        return layer, torch.randn((B, 20, d), generator=gen, device="cuda:0")
+
+    (wide, xw), (narrow, xn) = make(768, 32), make(256, 32, leaf=128)
+    with concurrent.futures.ThreadPoolExecutor(1) as a, concurrent.futures.ThreadPoolExecutor(1) as b:
+        first = a.submit(wide.prefill, xw).result()
+        step = a.submit(wide.decode, xw[:, 0], 19).result()
+        for _ in range(2):
+            b.submit(narrow.prefill, xn).result()
+            b.submit(narrow.decode, xn[:, 0], 19).result()
+            again = a.submit(wide.prefill, xw).result()
+            assert all(np.array_equal(x, y) for x, y in zip(first, again))
+            assert np.array_equal(a.submit(wide.decode, xw[:, 0], 19).result(), step)
