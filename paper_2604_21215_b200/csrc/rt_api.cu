@@ -58,11 +58,12 @@ constexpr int kWideLeafDefault = 16;    // leaf of the dense-product token steps
 constexpr int kWideFrom = 24;            // smallest bf16 batch that runs as dense products rather than through the generic kernel
 constexpr int kMmaSplitMax = 48;         // largest batch that runs as slices of at most 16 sequences through the tensor-core leaf kernel
 constexpr int kGroupsMax = 64;           // largest batch that runs as slices of at most 16 sequences side by side on groups of SMs
-Schedule effective_schedule(const rt_config* c, int B) {
+Schedule effective_schedule(const rt_config* c, int B, int N) {
   if (c->recur_block > 1) return {kPathBlocks, c->recur_block, 0};
   if (c->sched == RT_SCHED_TILED) {
     LeafMmaLaunch ml;
-    if (c->dtype == RT_BF16 && B > 16 && B <= kGroupsMax) {
+    // (a single position does not pay for packing the weights: d = 1024, B = 32 takes 65 us without, 120 us through the generic kernel)
+    if (c->dtype == RT_BF16 && B > 16 && B <= kGroupsMax && N > 1) {
       // slices side by side, a group of SMs each (rt_leaf_group.cu), unless the layer would otherwise take the generic kernel: that one holds
       // the vectors between the phases in fp32, the others round them to bf16 (d = 512, B = 20, leaves of 128: error of k against 64 bits
       // 1.9e-3 and 3.0e-3)
@@ -375,7 +376,7 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
     return RT_OK;
   }
 
-  const Schedule plan = effective_schedule(c, B);
+  const Schedule plan = effective_schedule(c, B, n_rows);
   const bool wide = plan.path == kPathWide && pos0 == 0;
   if (wide) {
     // Wide batches (the regime of the paper's own experiments, Sec. 6: B in the hundreds): a token step is a chain
@@ -548,7 +549,7 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
     ProfScope ps(s, kProfLeaf);
     return leaf_small_launch(c->dtype, lp, sl, s) == cudaSuccess;
   };
-  const bool groups = !small && plan.path == kPathGroups && pos0 == 0 && n_rows > 1;      // (one position: no workspace for it, see ws_layout)
+  const bool groups = !small && plan.path == kPathGroups && pos0 == 0;
   const int places = groups ? ceil_div(B, plan.sub) : 0;
   unsigned char* const packed = groups ? ws + L.form + group_area(c, places, 1, 0, 0).packed : nullptr;
   if (groups) {
@@ -1132,7 +1133,7 @@ rt_status rt_plan_counters(const rt_config* cfg, int32_t B, int32_t N, int32_t n
     fl_leaf += 4 * d * b * (n * (n - 1) / 2);
   } else {
     // the schedule that runs: leaf (or block) granularity of the chain form this shape takes
-    const Schedule plan = effective_schedule(cfg, B);
+    const Schedule plan = effective_schedule(cfg, B, N);
     const Wave wv = stack_wave(cfg, B, N, n_layers);             // layers side by side: every leaf meets all earlier pairs at once
     const uint64_t Lf = wv.places ? wv.leaf : plan.leaf;
     for (uint64_t s0 = 0; s0 < n; s0 += Lf) {

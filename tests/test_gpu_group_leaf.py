@@ -146,3 +146,22 @@ def test_layers_may_share_one_pair_of_caches():
     k, v = st.caches_numpy(N)[0]                                # the last layer's pairs
     check_tensor("shared caches", "k", k, caches_ref[L - 1][0], 2e-2)
     check_tensor("shared caches", "v", v, caches_ref[L - 1][1], 2e-2)
+
+
+@pytest.mark.parametrize("B", [20, 48, 64])
+def test_one_position_takes_the_tensor_core_kernels(B):
+    # a prefill of one position has no use for packed weights: slices of the leaf kernel or dense products, not the generic kernel, which
+    # would read the chain weights once for all sequences
+    from oracle import RTConfig, RTWeights, layer_seq
+    from paper_2604_21215_b200 import inputs, rt
+    d, H, dff = 512, 8, 2048
+    data = inputs.make_inputs(inputs.Workload("one", 1, B, 1, d, H, dff, "bf16"), seed=B)
+    lw = data["layers"][0]
+    ref = layer_seq(RTConfig(d, H, 64, dff), RTWeights(**lw), data["x"])
+    layer = rt.Layer(d, H, dff, dtype="bf16")
+    layer.set_weights(lw)
+    for name, a, b in zip(("z", "k", "v"), layer.prefill(data["x"]), ref):
+        check_tensor(f"one position B={B}", name, a, b, 2e-2)
+    chain_w, pre_w = (3 * d * d + 2 * d * dff) * 2, 3 * d * d * 2
+    per_token = (rt.rt_plan_counters(layer.cfg, 16, 1)["model_bytes_read"] - chain_w - pre_w) // 16
+    assert rt.rt_plan_counters(layer.cfg, B, 1)["model_bytes_read"] - B * per_token - pre_w == chain_w * (1 if B > 48 else -(-B // 16))
