@@ -61,7 +61,7 @@ constexpr size_t kB200SmemPerCta = 232448;
 cudaError_t leaf_mma_launch(const LeafParams& p, const LeafMmaLaunch& l, const LeafMmaBuffers& buf, cudaStream_t s);
 
 // Leaf kernel for layers that fit one cluster's shared memory (rt_leaf_small.cu).
-struct LeafSmallLaunch { int nb, leaf; size_t smem; };
+struct LeafSmallLaunch { int nb, leaf; size_t smem; float step_us; };      // step_us: estimate of the time per position
 bool leaf_small_shape(int dtype, int B, int d, int H, int dff, int leaf, size_t max_smem, LeafSmallLaunch* out);
 cudaError_t leaf_small_launch(int dtype, const LeafParams& p, const LeafSmallLaunch& l, cudaStream_t s);
 

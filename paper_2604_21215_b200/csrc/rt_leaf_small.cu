@@ -406,7 +406,13 @@ constexpr int kClusters = 7;
 
 // Whether the shape runs on this kernel with leaves of `leaf` positions (pure arithmetic), and how many sequences a cluster
 // carries: one to three, whatever makes rounds of clusters x time per round least (a step with 2 or 3 sequences measured about 1.35 and
-// 1.7 times one with a single sequence at d = 128 .. 256).
+// 1.7 times one with a single sequence at d = 128 .. 256; that one 3.1, 3.3, 4.0, 4.5, 5.8 and 6.3 us at d = 64, 128, ... 384 in bf16).
+//
+// The values between the phases stay fp32 here, so fp32 layers always stay (the generic kernel takes three times as long or more), and bf16
+// layers up to the time that the same batch takes with its values in bf16 as slices of 16 sequences one after the other through the tensor-core leaf
+// kernel, 11.3 us each, or, above 48, as dense products, 38 us.  Per 256 positions at d = 384: 15 sequences take 4.3 ms here (two rounds) and 2.9
+// there, 32 6.8 and 6.0, 64 11.4 and 9.8, but 24 4.6 and 5.9; up to d = 320 every batch is within the bound.  (The group kernel, also on
+// bf16 values, is the fastest from about two rounds on: 3.8 ms against 5.9 for d = 256, B = 48; it takes what is beyond the bound.)
 bool leaf_small_shape(int dtype, int B, int d, int H, int dff, int leaf, size_t max_smem, LeafSmallLaunch* out) {
   if (d % 64 || dff % 64 || d > 512 || leaf > kSmLeafMax) return false;
   int nb = 0;
@@ -419,8 +425,9 @@ bool leaf_small_shape(int dtype, int B, int d, int H, int dff, int leaf, size_t 
   const size_t es = dtype == RT_BF16 ? 2 : 4;
   const SmallLayout L = small_layout(es, nb, d, dff);
   if (L.total > max_smem) return false;
-  out->nb = nb; out->leaf = leaf; out->smem = L.total;
-  return true;
+  const float weights_kb = (float)(L.total - L.off_wo) * (1.0f / 1024.0f);
+  out->nb = nb; out->leaf = leaf; out->smem = L.total; out->step_us = best * (3.0f + weights_kb * (1.0f / 60.0f));
+  return dtype != RT_BF16 || out->step_us <= (B > 48 ? 38.0f : 11.3f * ceil_div(B, 16));
 }
 
 cudaError_t leaf_small_launch(int dtype, const LeafParams& p, const LeafSmallLaunch& l, cudaStream_t s) {

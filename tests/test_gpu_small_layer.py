@@ -29,3 +29,18 @@ def test_small_layer_matches_oracle(dtype, d, H, dff, B, N, leaf, alibi):
     got = layer.prefill(data["x"])
     for name, a, b in zip(("z", "k", "v"), got, ref):
         check_tensor(f"small {dtype} d={d} B={B} N={N}", name, a, b, TOL[dtype])
+
+
+@pytest.mark.parametrize("B,N", [(14, 70), (15, 70), (28, 40), (32, 40), (64, 20)])
+def test_batches_around_the_bound_of_the_cluster_kernel(B, N):
+    # d = 384: one and two rounds of clusters, and the batches that the tensor-core leaf kernel and the group kernel take instead
+    from oracle import RTConfig, RTWeights, layer_seq
+    from paper_2604_21215_b200 import inputs, rt
+    d, H, dff = 384, 6, 1536
+    data = inputs.make_inputs(inputs.Workload("bound", 1, B, N, d, H, dff, "bf16"), seed=B)
+    lw = data["layers"][0]
+    ref = layer_seq(RTConfig(d, H, 64, dff), RTWeights(**lw), data["x"])
+    layer = rt.Layer(d, H, dff, dtype="bf16")
+    layer.set_weights(lw)
+    for name, a, b in zip(("z", "k", "v"), layer.prefill(data["x"]), ref):
+        check_tensor(f"bound B={B}", name, a, b, TOL["bf16"])
