@@ -113,8 +113,9 @@ __global__ void transpose_bf16_kernel(const TI* __restrict__ in, long long R, in
 }
 
 // The same for fp32 arrays whose width and padded row count are multiples of 64: 16-byte loads and stores on both sides (the kernel above moves
-// 2.1 TB/s, 35 us for 12288 x 1024: its stores are 64 bytes per warp).  grid (C / 64, ld / 64), 256 threads.
-__global__ void __launch_bounds__(256) transpose_f32_kernel(const float* __restrict__ in, long long R, int C, __nv_bfloat16* __restrict__ out, long long ld) {
+// 2.1 TB/s, 35 us for 12288 x 1024: its stores are 64 bytes per warp).  grid (C / 64, ld / 64), 256 threads.  With `rest` two more terms per
+// entry go there, [2][C, ld]: the three bf16 values of an entry are its fp32 value.
+__global__ void __launch_bounds__(256) transpose_f32_kernel(const float* __restrict__ in, long long R, int C, __nv_bfloat16* __restrict__ out, __nv_bfloat16* __restrict__ rest, long long ld) {
   __shared__ float tile[64][65];
   const long long r0 = (long long)blockIdx.y * 64;
   const int c0 = blockIdx.x * 64, tid = threadIdx.x;
@@ -128,13 +129,16 @@ __global__ void __launch_bounds__(256) transpose_f32_kernel(const float* __restr
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     const int c = (tid >> 3) + 32 * k, r = 8 * (tid & 7);
-    unsigned w[4];
+    const long long at = (long long)(c0 + c) * ld + r0 + r;
+    F8 x;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const __nv_bfloat162 v = __floats2bfloat162_rn(tile[r + 2 * e][c], tile[r + 2 * e + 1][c]);
-      w[e] = *reinterpret_cast<const unsigned*>(&v);
+    for (int e = 0; e < 8; ++e) x.v[e] = tile[r + e][c];
+    store_operand8(out + at, x, 1, 0);
+    if (rest) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) x.v[e] = isfinite(x.v[e]) ? x.v[e] - __bfloat162float(__float2bfloat16_rn(x.v[e])) : 0.f;
+      store_operand8(rest + at, x, 2, (long long)C * ld);
     }
-    *reinterpret_cast<uint4*>(out + (long long)(c0 + c) * ld + r0 + r) = make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
@@ -1320,6 +1324,10 @@ struct BwdLayout {
 };
 constexpr int kColParts = 128;
 constexpr int kWideLeaf = 16;
+// Weight gradients whose row count is no multiple of 64 are fp32 products of fp32 operands: on CUDA cores below this many rows, on three bf16
+// terms per operand (six products of the tensor cores, to 2^-24) from it on.  Whole backward pass: 100 rows of d = 768 1.95 ms and 2.47, 1000 rows 16.9 and
+// 16.9, 6000 rows 34.9 and 31.8; d = 512 and 1024 cross between 900 and 1200 rows, d = 128 at 1300.
+constexpr int kGemmRows = 1000;
 constexpr int kWideBatchFrom = 32;      // above this many sequences a step of the reverse loop runs as dense products over the batch
 
 // Up to 32 sequences the reverse loop keeps its operands to fp32 (three bf16 terms): up to 8 as mat-vecs of one launch per leaf
@@ -1343,10 +1351,12 @@ BwdLayout bwd_layout(const rt_config* c, int B, int N) {
   size_t o = 0;
   auto take = [&](size_t floats) { size_t at = o; o += align_up(floats * 4, 256); return at; };
   L.sync = take(sizeof(SyncArea) / 4);
-  L.n = take(rows * d); L.qraw = take(rows * d); L.ktraw = take(rows * d); L.vt = take(rows * d);
+  // (qraw, ktraw and act take the further terms of the weight gradients' operands in the end, whose rows are padded to whole blocks of 64)
+  const size_t rows_k = align_up(rows, 64);
+  L.n = take(rows * d); L.qraw = take(rows_k * d); L.ktraw = take(rows_k * d); L.vt = take(rows * d);
   L.q = take(rows * d); L.kt = take(rows * d); L.r = take(rows * d); L.kraw = take(rows * d);
   L.k = take(rows * d); L.v = take(rows * d); L.c = take(rows * d); L.h = take(rows * d); L.u = take(rows * d);
-  L.act = take(rows * f); L.gl = take(rows * f); L.lse = take(rows * H); L.D = take(rows * H);
+  L.act = take(rows_k * f); L.gl = take(rows * f); L.lse = take(rows * H); L.D = take(rows * H);
   L.zero_begin = o;
   L.dK = take(rows * d); L.dV = take(rows * d);
   L.zero_end = o;
@@ -1361,7 +1371,6 @@ BwdLayout bwd_layout(const rt_config* c, int B, int N) {
   L.qkv16 = take(3 * rows * d / 2 + 64);                       // bf16 copies of q, k, v for the tile kernels
   L.wt5 = take((3 * d * d + 2 * d * f) / 2 + 64); L.dzp = wide && !tc ? take(rows * d) : o;
   // bf16 operands of the tensor-core products (bf16 storage): two [rows, max(d, d_ff)] arrays and one [d, d]
-  const size_t rows_k = align_up(rows, 64);
   L.wctr = wide && tc ? take(wide_counter_bytes(B) / 4) : o;
   if (wide && tc && N < 8) L.gprod = take((size_t)8 * B * d);    // parts of split products
   size_t sa_elems = rows_k * (d > f ? d : f), sb_elems = sa_elems;
@@ -1428,8 +1437,8 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   auto to_bf16 = [&](const float* in, __nv_bfloat16* out, long long n) {
     to_bf16_kernel<<<elems_grid((n + 3) / 4), tpb, 0, s>>>(in, out, n);
   };
-  auto transpose_f = [&](const float* in, long long R, int C, __nv_bfloat16* out) {
-    transpose_f32_kernel<<<dim3(C / 64, (unsigned)(rows_k / 64)), 256, 0, s>>>(in, R, C, out, rows_k);      // (tensor cores: widths of 128)
+  auto transpose_f = [&](const float* in, long long R, int C, __nv_bfloat16* out, __nv_bfloat16* rest) {
+    transpose_f32_kernel<<<dim3(C / 64, (unsigned)(rows_k / 64)), 256, 0, s>>>(in, R, C, out, rest, rows_k);      // (tensor cores: widths of 128)
   };
   const float* sa_holds = nullptr;                               // which array SA currently holds as a plain bf16 copy
   // out[rows, n_out] = A[rows, k] W[n_out, k]^T  (a product of the forward pass)
@@ -1813,11 +1822,24 @@ rt_status backward_impl(const rt_config* c, const rt_layer_weights* w, const T* 
   }
   // parameter matrices: dW[o, i] = sum_rows dY[row, o] X[row, i]
   const float* sb_holds = nullptr;                               // which array SB currently holds transposed
+  const bool full = rows % 64 != 0;
   auto wgrad = [&](float* out, const float* dY, int n_out, const float* X, int n_in, float al, bool acc) -> cudaError_t {
-    if (!tc) return gemm<float, float>(n_out, n_in, (int)rows, dY, 1, n_out, X, n_in, 1, out, n_in, al, acc, s);
-    transpose_f(dY, rows, n_out, SA); sa_holds = nullptr;
-    if (sb_holds != X) { transpose_f(X, rows, n_in, SB); sb_holds = X; }
-    return tc_product(n_out, n_in, (int)rows_k, SA, SB, out, al, acc, true);     // d x d results are 64 tiles at d = 1024: in parts over the rows
+    if (!tc || (full && rows < kGemmRows)) return gemm<float, float>(n_out, n_in, (int)rows, dY, 1, n_out, X, n_in, 1, out, n_in, al, acc, s);
+    // terms beyond the first: of the wider operand in act, of the others in qraw (dY) and ktraw (X), which nobody reads any more
+    auto rest = [&](int n, size_t at) { return full ? reinterpret_cast<__nv_bfloat16*>(ws + (n == f && f != d ? L.act : at)) : nullptr; };
+    __nv_bfloat16 *ra = rest(n_out, L.qraw), *rb = rest(n_in, L.ktraw);
+    transpose_f(dY, rows, n_out, SA, ra); sa_holds = nullptr;
+    if (sb_holds != X) { transpose_f(X, rows, n_in, SB, rb); sb_holds = X; }
+    // d x d results are 64 tiles at d = 1024: in parts over the rows
+    if (!full) return tc_product(n_out, n_in, (int)rows_k, SA, SB, out, al, acc, true);
+    const __nv_bfloat16 *A[3] = {SA, ra, ra + rows_k * n_out}, *Bt[3] = {SB, rb, rb + rows_k * n_in};
+    for (int sum = 2; sum >= 0; --sum)                           // the smallest products first; what is left out is 2^-24 of the whole
+      for (int i = 0; i <= sum; ++i) {
+        const cudaError_t e = tc_product(n_out, n_in, (int)rows_k, A[i], Bt[sum - i], out, al, acc, true);
+        if (e != cudaSuccess) return e;
+        acc = true;
+      }
+    return cudaSuccess;
   };
   if (gr->w_k) RT_TRY(wgrad(gr->w_k, F(L.dkraw), d, F(L.r), d, 1.f, false));
   if (gr->w_v) RT_TRY(wgrad(gr->w_v, F(L.dvf), d, F(L.r), d, 1.f, false));

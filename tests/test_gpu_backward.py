@@ -157,3 +157,25 @@ def test_backward_argument_errors():
     blocked = rt.make_config(128, 2, 256, dtype="f32", recur_block=4)
     assert call(xd.data_ptr(), need, blocked) == rt.RT_ERR_UNSUPPORTED
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("B", [3, 63, 999, 1010, 1023])
+def test_weight_gradients_of_ragged_row_counts_keep_fp32_operands(B):
+    # One position: dz is the gradient of z itself, so dW_down = sum_b dz_b (x) g_b has its columns in the span of the dz_b, and dW_v = sum_b dv~_b (x)
+    # RMS(x_b) its rows in the span of the x_b, for the few sequences whose dz is not zero.  Operands rounded to bf16 leave those spans by 2^-9; fp32
+    # operands, or three bf16 terms of them, by the rounding of the sums only (2^-24 an operation, here at most about 20 of them in a row).
+    from paper_2604_21215_b200 import inputs, rt
+    d, H, dff, live = 128, 2, 512, 3
+    data = inputs.make_inputs(inputs.Workload("ragged", 1, B, 1, d, H, dff, "bf16"), seed=B)
+    layer = rt.Layer(d, H, dff, dtype="bf16")
+    layer.set_weights(data["layers"][0])
+    z, _, _ = layer.prefill(data["x"])
+    dz = np.zeros_like(z)
+    at = np.linspace(0, B - 1, live).astype(int)
+    dz[at] = np.random.default_rng(B).standard_normal((live, 1, d)).astype(np.float32)
+    _, g = layer.backward(data["x"], z, dz)
+    def off_span(m, basis):                                     # share of the rows of m that is not in the span of the rows of basis
+        q, _ = np.linalg.qr(basis.T)
+        return np.linalg.norm(m - (m @ q) @ q.T) / np.linalg.norm(m)
+    assert off_span(g["w_down"].T, dz[at, 0]) <= 2.0 ** -19
+    assert off_span(g["w_v"], np.asarray(data["x"])[at, 0]) <= 2.0 ** -19
