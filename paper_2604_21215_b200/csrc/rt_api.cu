@@ -109,7 +109,19 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
   if (N > kWaveMaxN || (size_t)N * B * c->d_model * 4 > kWaveCacheMax) return none;
   // Short leaves fill the pipeline of layers sooner, long ones have fewer launches.
   const int leaf = c->leaf ? c->leaf : N <= 128 ? 16 : 32;
-  return {places, leaf};
+  // Side by side a position costs a layer more (fewer SMs, weights from L2), so enough layers have to be at work at the same time: on average
+  // n_layers * N / (waves * leaf) of them.  Break even was measured at 1.3 to 2.3, growing with the weights that the groups stream (places x MB
+  // per layer) and above four sequences: 8 layers of d = 1024, B = 1, take 1.69 times as long as one after the other for 16 positions (one layer at a
+  // time), 1.05 for 32, 0.84 for 48, 0.72 for 77; B = 16 1.98, 1.20, 0.95 and for 64 0.83; 2 layers 1.33, 1.09, 1.03 and for 128 0.97.  Layers
+  // that fit a cluster (rt_leaf_small.cu) are faster alone than the tensor-core leaf kernel, taken as 8.3 us a position, above eight sequences 10.5; it
+  // takes as many more.  Over 2 to 8 layers, d = 128 to 1024, 1 to 16 sequences and 16 to 400 positions the side taken is at most about a tenth slower than the other.
+  const int n_leaves = ceil_div(N, leaf), turn = n_leaves > places ? n_leaves : places;
+  const float waves = (float)((n_layers - 1) / places * turn + (n_layers - 1) % places + n_leaves), at_work = (float)n_layers * (float)N / (waves * (float)leaf);
+  const float layer_mb = (3.0f * c->d_model + 2.0f * c->d_ff) * c->d_model * 2e-6f, mma_us = B > 8 ? 10.5f : 8.3f;
+  LeafSmallLaunch sl;
+  const bool small = leaf_small_shape(c->dtype, B, c->d_model, c->n_heads, c->d_ff, ml.leaf, kB200SmemPerCta, &sl);
+  const float even = (1.26f + 0.008f * places * layer_mb + (B > 4 ? 0.15f : 0.0f)) * (small && sl.step_us < mma_us ? mma_us / sl.step_us : 1.0f);
+  return at_work > even ? Wave{places, leaf} : none;
 }
 struct WaveRows { size_t n, q, kt, vt, st_o, st_m, st_l, total; };
 WaveRows wave_rows_layout(const rt_config* c, int B, int leaf) {

@@ -160,3 +160,19 @@ def test_workspace_grows_with_the_shape(dtype):
             ws = [[size(cfg, B, N) for N in Ns] for B in Bs]
             assert all(a <= b for row in ws for a, b in zip(row, row[1:])), (size, d, dff, kw)
             assert all(a <= b for r0, r1 in zip(ws, ws[1:]) for a, b in zip(r0, r1)), (size, d, dff, kw)
+
+
+def test_layers_run_side_by_side_where_enough_of_them_are_at_work():
+    # Side by side every leaf meets all earlier pairs at once, one after the other Algorithm 1's tiles do: the counters tell which.  A prompt
+    # of one leaf has one layer at work at a time; deep stacks of longer prompts have all places busy; two layers never more than two.
+    def side_by_side(d, B, N, L):
+        cfg = rt.make_config(d, d // 64, 4 * d, dtype="bf16")
+        return rt.rt_plan_counters(cfg, B, N, L)["kv_bytes_read"] != L * rt.rt_plan_counters(cfg, B, N, 1)["kv_bytes_read"]
+    for d in (128, 256, 384, 512, 768, 1024):
+        for B in (1, 4, 8, 9, 16):
+            assert not any(side_by_side(d, B, 16, L) for L in (2, 4, 8)), (d, B)
+    for d in (512, 768, 1024):
+        for B in (1, 4, 16):
+            assert side_by_side(d, B, 77, 8) and side_by_side(d, B, 128, 4) and side_by_side(d, B, 1024, 8), (d, B)
+            assert not side_by_side(d, B, 24, 8) and not side_by_side(d, B, 32, 2), (d, B)
+    assert not side_by_side(128, 1, 64, 8) and side_by_side(384, 4, 64, 8) and side_by_side(256, 16, 200, 8)

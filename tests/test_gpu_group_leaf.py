@@ -39,7 +39,8 @@ def test_slices_match_oracle(d, H, dff, B, N, leaf, gains, alibi):
 
 @pytest.mark.parametrize("L,d,H,dff,B,N,leaf,gains,alibi", [
     (2, 512, 8, 2048, 1, 2, 0, False, False), (5, 512, 8, 1024, 3, 77, 0, True, True), (9, 448, 7, 896, 1, 17, 0, False, False),
-    (3, 768, 12, 3072, 9, 300, 0, True, True), (6, 512, 8, 512, 2, 230, 16, False, True), (4, 640, 10, 1280, 16, 130, 64, True, False)])
+    (3, 768, 12, 3072, 9, 300, 0, True, True), (6, 512, 8, 512, 2, 230, 16, False, True), (4, 640, 10, 1280, 16, 130, 64, True, False),
+    (9, 448, 7, 896, 1, 130, 0, True, False), (4, 640, 10, 1280, 16, 200, 64, False, True)])
 def test_layers_side_by_side_match_oracle(L, d, H, dff, B, N, leaf, gains, alibi):
     from oracle import RTConfig, RTWeights, stack_prefill
     from paper_2604_21215_b200 import inputs, rt
