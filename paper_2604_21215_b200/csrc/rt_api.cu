@@ -18,7 +18,7 @@ constexpr int kSmallBatchMax = 64;      // above this the per-token chain runs a
 constexpr int kAutoLeaf = 64;
 
 struct WsLayout {
-  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, ll, ll_bytes, form, dec_words, dec_words_bytes, hid0, hid1,
+  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, ll, ll_bytes, form, g_arrays, dec_words, dec_words_bytes, hid0, hid1,
       blk_h, blk_u, blk_c, blk_g, total;
 };
 
@@ -148,6 +148,14 @@ GroupArea group_area(const rt_config* c, int places, int packs, int wave_B, int 
   return A;
 }
 
+// Positions that the tensor-core leaf kernel has an array of g for: a leaf, or all layers of a prompt shorter than that (one fill serves
+// them: 8 layers of one position, d = 1024, 305 -> 291 us).
+int g_positions(const rt_config* c, int N, int n_layers) {
+  LeafMmaLaunch ml;
+  if (!leaf_mma_shape(1, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml)) return 0;
+  return (long long)N * n_layers < ml.leaf ? N * n_layers : ml.leaf;
+}
+
 // Bytes of the area that the form of the token loop has to itself: the most that any call of at most B sequences, N positions and n_layers
 // layers asks for, whichever form it takes, so that a workspace reserved for the longest prompt and the fullest batch serves all the others.
 // (What one form asks for by itself does not grow with the shape: beyond kWaveMaxN positions no layers run side by side, from 17
@@ -158,8 +166,7 @@ size_t form_bytes(const rt_config* c, int B, int N, int n_layers) {
   const int d = c->d_model, H = c->n_heads, f = c->d_ff, B16 = B < 16 ? B : 16;
   size_t most = 0;
   auto need = [&](size_t bytes) { if (bytes > most) most = bytes; };
-  LeafMmaLaunch ml;
-  if (leaf_mma_shape(1, d, H, f, c->leaf, kB200Sms, kB200SmemPerCta, &ml)) need((size_t)(ml.leaf < N ? ml.leaf : N) * 16 * f * 2);      // g of the tensor-core leaf kernel
+  need((size_t)g_positions(c, N, n_layers) * 16 * f * 2);
   if (N < 2) return most;
   for (int places = 2; places <= kGroupJobs; ++places) {
     if (!leaf_group_shape(1, d, H, f, places, kB200SmemPerCta)) continue;
@@ -192,6 +199,7 @@ WsLayout ws_layout(const rt_config* c, int B, int N, int n_layers) {
   // raw k|v as flag-carrying fp32 words; g as packed bf16 in fragment order (16 sequence slots), an array per position of a leaf, in `form`
   L.ll_bytes = ((size_t)16 * 3 * (d / 2) + (size_t)B * 2 * d) * 8;
   L.ll = take(L.ll_bytes);
+  L.g_arrays = c->dtype == RT_BF16 ? g_positions(c, N, n_layers) : 0;
   L.form = take(form_bytes(c, B, N, n_layers));
   // a decode step uses none of the above but the status block: its exchange area begins right behind that
   L.dec_words = L.q;
@@ -257,7 +265,7 @@ struct ProfScope {
 };
 
 // State of one API call: the stream and the barrier arrivals enqueued so far.
-struct CallCtx { cudaStream_t s; unsigned bar_base = 0; unsigned seq_base = 0; unsigned group_steps[kGroupJobs] = {0, 0, 0, 0}; bool groups_zeroed = false; };
+struct CallCtx { cudaStream_t s; unsigned bar_base = 0; unsigned seq_base = 0; unsigned group_steps[kGroupJobs] = {0, 0, 0, 0}; bool groups_zeroed = false; int g_left = 0; };      // g_left: arrays of g still filled
 
 // The exchange areas of the group kernel start from zero, once per API call.
 bool zero_groups(const rt_config* c, unsigned char* ws, const WsLayout& L, CallCtx& ctx) {
@@ -528,7 +536,7 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   {
     unsigned long long* w = (unsigned long long*)(ws + L.ll);
     const size_t bd2 = (size_t)16 * (c->d_model / 2);
-    mb.ll_c = w; mb.ll_h = w + bd2; mb.ll_z = w + 2 * bd2; mb.ll_g = (unsigned long long*)(ws + L.form);
+    mb.ll_c = w; mb.ll_h = w + bd2; mb.ll_z = w + 2 * bd2;
     mb.ll_kv = w + 3 * bd2;
   }
   auto leaf_mma = [&](int t0, int t1) -> bool {
@@ -539,7 +547,14 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
       lp.x = (const unsigned char*)x + (size_t)b0 * x_bs * e;
       lp.z = (unsigned char*)z + (size_t)b0 * z_bs * e;
       lp.t0 = t0; lp.t1 = t1; lp.attn_begin = t0; lp.seq_base = ctx.seq_base;
-      if (cudaMemsetAsync(ws + L.form, 0xff, (size_t)(t1 - t0) * 16 * c->d_ff * 2, s) != cudaSuccess) return false;
+      // fresh arrays of g for the positions of this launch; filled all at once when they run out
+      const size_t g_bytes = (size_t)16 * c->d_ff * 2;
+      if (ctx.g_left < t1 - t0) {
+        if (cudaMemsetAsync(ws + L.form, 0xff, L.g_arrays * g_bytes, s) != cudaSuccess) return false;
+        ctx.g_left = (int)L.g_arrays;
+      }
+      mb.ll_g = (unsigned long long*)(ws + L.form + (L.g_arrays - (size_t)ctx.g_left) * g_bytes);
+      ctx.g_left -= t1 - t0;
       if (leaf_mma_launch(lp, ml, mb, s) != cudaSuccess) return false;
       ctx.seq_base += (unsigned)(t1 - t0);
     }
