@@ -2,6 +2,7 @@
 // row-wise steps over at most 128 sequences.  Warp 0 fetches operands and watches the group's counters, warp 1 issues the products, eight warps
 // do the row work.
 #pragma once
+#include "rt_gelu.h"
 #include "rt_kernels.h"
 #include "rt_tc.cuh"
 
@@ -41,15 +42,12 @@ __device__ __forceinline__ float sum8(float v) {           // over the eight lan
   v += __shfl_xor_sync(0xffffffffu, v, 4);
   return v;
 }
-// x Phi(x) with erfc by Abramowitz and Stegun 7.1.26.  Largest error 2.1e-7 (0.5 x (1 + erff) in fp32: 6.8e-7), and no cancellation for
-// negative x; a third of the instructions, which a step that applies it to 128 x 128 accumulators per CTA notices (4 us before).
-__device__ __forceinline__ float gelu_wide(float x) {
-  float t;                                                 // 1 / (1 + 0.3275911 |x| / sqrt(2))
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.3275911f * 0.70710678f, fabsf(x), 1.0f)));
-  const float poly = t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 0.5f * 1.061405429f, -0.5f * 1.453152027f), 0.5f * 1.421413741f), -0.5f * 0.284496736f), 0.5f * 0.254829592f);
-  const float q = poly * ex2(x * x * (-0.5f * kLog2e));    // Phi(-|x|)
-  return x * (x < 0.f ? q : 1.0f - q);
+__device__ __forceinline__ float erfc_step(float x) {      // t of rt_gelu.h
+  float t;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(kErfcSlope, fabsf(x), 1.0f)));
+  return t;
 }
+__device__ __forceinline__ float gelu_wide(float x) { return gelu_of(x, erfc_step(x), ex2(x * x * (-0.5f * kLog2e))); }
 
 static __device__ __noinline__ bool wide_wait(uint32_t bar, uint32_t parity, volatile int* s_abort, SyncArea* sync) { return warp_mbar_wait(bar, parity, s_abort, sync); }
 

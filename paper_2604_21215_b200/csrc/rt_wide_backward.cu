@@ -20,14 +20,7 @@ enum { B_KV = 0, B_RZ = 1, B_DOWN = 2, B_UP = 3, B_RH = 4, B_OUT = 5, B_ATTN = 6
 // The products in order (indices of WideBwdParams::st): W_k | W_v, W_down, W_up, W_o (all transposed).
 struct WideBwdMaps { CUtensorMap a[4], w[4]; };
 
-// Phi(a) + a phi(a), Phi as in gelu_wide
-__device__ __forceinline__ float gelu_grad_wide(float x) {
-  float t;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.3275911f * 0.70710678f, fabsf(x), 1.0f)));
-  const float poly = t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 0.5f * 1.061405429f, -0.5f * 1.453152027f), 0.5f * 1.421413741f), -0.5f * 0.284496736f), 0.5f * 0.254829592f);
-  const float e = ex2(x * x * (-0.5f * kLog2e)), q = poly * e;
-  return (x < 0.f ? q : 1.0f - q) + x * 0.3989422804014327f * e;
-}
+__device__ __forceinline__ float gelu_grad_wide(float x) { return gelu_grad_of(x, erfc_step(x), ex2(x * x * (-0.5f * kLog2e))); }
 __device__ __forceinline__ F8 ldcg8(const float* p) {
   const float4 a = __ldcg(reinterpret_cast<const float4*>(p)), b = __ldcg(reinterpret_cast<const float4*>(p + 4));
   return F8{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
