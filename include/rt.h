@@ -111,8 +111,11 @@ size_t rt_workspace_bytes(const rt_config *cfg, int32_t B, int32_t N, int32_t n_
  * Batch sizes (tiled schedule): B <= 16 in bf16 takes the persistent tensor-core leaf kernel (small layers of either
  * type a kernel inside thread-block clusters); 17 <= B <= 64 in bf16 runs as slices of at most 16 sequences side by side
  * on groups of SMs (the sequences are independent), sharing the pre-pass and the cross tiles; larger batches run each
- * token step as dense products over the batch (the regime of the paper's own experiments, Sec. 6).  fp32 up to B = 64,
- * the naive schedule and decode up to B = 64 take a generic kernel.
+ * token step as dense products over the batch (the regime of the paper's own experiments, Sec. 6).  fp32 up to B = 64 (larger
+ * layers), the naive schedule and bf16 layers that fit none of these take a generic kernel.  Decode in bf16 takes one launch for
+ * all layers (up to 16): a batch of at most 16 sequences at once, its vectors between the products rounded to bf16 like the
+ * prefill's; above 16, at position 0 and for layers off the leaf kernel in slices of at most 8 with fp32 vectors.  fp32 and
+ * widths that this kernel does not take decode through the generic one.
  * The naive schedule and the decode entry points return RT_ERR_UNSUPPORTED for B > 64. */
 rt_status rt_layer_prefill(const rt_config *cfg, const rt_layer_weights *w,
                            const void *x, int32_t B, int32_t N,
@@ -240,8 +243,8 @@ rt_status rt_layer_recompute(const rt_config *cfg, const rt_layer_weights *w, co
  * pairs, dx and every parameter gradient as products over all B*N rows at once.
  * With bf16 storage the reverse loop runs on the tensor cores: up to 32 sequences with operands kept to 2^-24 (three
  * bf16 terms), above (Sec. 6's regime, dense products over the batch) with operands rounded to bf16; the products over
- * all rows round their operands to bf16 too.  Accumulation is fp32 throughout; the attention terms and everything with
- * fp32 storage are fp32 on CUDA cores.  recur_block > 1 returns RT_ERR_UNSUPPORTED.
+ * all rows round their operands to bf16 too, but for weight gradients where B*N is no multiple of 64, whose operands stay
+ * fp32.  Accumulation is fp32 throughout; the attention terms and everything with fp32 storage are fp32 on CUDA cores.  recur_block > 1 returns RT_ERR_UNSUPPORTED.
  * The workspace needs rt_backward_workspace_bytes (about 40 fp32 arrays of B*N*d plus 4 of B*N*d_ff: 1.1 GB at B=4, N=2048, d=768; 48 GB at B=N=512, d=1024). */
 typedef struct {
   float *w_q, *w_k, *w_v, *w_o, *w_up, *w_down;   /* shapes of rt_layer_weights */

@@ -53,8 +53,9 @@ int leaf_size(const rt_config* c) { return c->leaf ? c->leaf : kAutoLeaf; }
 // a B200).
 enum ChainPath { kPathGeneric = 0, kPathMma = 1, kPathWide = 2, kPathBlocks = 3, kPathMmaSplit = 4, kPathGroups = 5 };
 struct Schedule { ChainPath path; int leaf; int sub; };      // sub: sequences per slice (kPathMmaSplit, kPathGroups)
-constexpr int kWideLeafDefault = 16;    // leaf of the dense-product token steps: the in-leaf attention re-reads the leaf's pairs for every position,
-                                        // so short leaves win (p512: 16 -> 41.6 ms, 32 -> 42.3, 64 -> 45.9 per layer)
+constexpr int kWideLeafDefault = 16;    // leaf of the dense-product token steps.  As launches per position, whose in-leaf attention re-reads the leaf's pairs
+                                        // for every position, short leaves win (p512: 16 -> 41.6 ms, 32 -> 42.3, 64 -> 45.9 per layer); in one launch per leaf
+                                        // 32 or 64 would be 1.5 to 6 % faster, but the modelled schedule of wide batches is that of 16
 constexpr int kWideFrom = 24;            // smallest bf16 batch that runs as dense products rather than through the generic kernel
 constexpr int kMmaSplitMax = 48;         // largest batch that runs as slices of at most 16 sequences through the tensor-core leaf kernel
 constexpr int kGroupsMax = 64;           // largest batch that runs as slices of at most 16 sequences side by side on groups of SMs
@@ -73,9 +74,9 @@ Schedule effective_schedule(const rt_config* c, int B, int N) {
         return {kPathGroups, c->leaf ? c->leaf : kAutoLeaf, sub};
     }
     if (c->dtype == RT_BF16 && B > 16 && B <= kMmaSplitMax) {
-      // Sequences are independent (Sec. 2.2 states the layer per sequence) and a token step of the tensor-core leaf
-      // kernel costs 10 - 14 us whatever its batch, against 53 us for the dense-product step at B = 32: up to 48
-      // sequences run as 2 or 3 slices of at most 16 through that kernel, leaf by leaf, and share the cross tiles.
+      // What the group kernel does not take (a single position, layers that fit no group): sequences are independent (Sec. 2.2 states
+      // the layer per sequence) and a token step of the tensor-core leaf kernel costs 9 - 14 us whatever its batch, against 53 us for the
+      // dense-product step at B = 32: up to 48 sequences run as 2 or 3 slices of at most 16 through that kernel, leaf by leaf, and share the cross tiles.
       const int n_sub = (B + 15) / 16, sub = (B + n_sub - 1) / n_sub;
       if (leaf_mma_shape(sub, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml))
         return {kPathMmaSplit, ml.leaf, sub};
@@ -104,8 +105,9 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
   LeafMmaLaunch ml;                                            // (a stack of layers for the generic kernel keeps its fp32 vectors)
   if (!leaf_mma_shape(B, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml)) return none;
   // A leaf meets all earlier pairs at once when its queries exist (they depend on the layer below, so Algorithm 1's tiles cannot
-  // run ahead): each leaf reads the layer's whole cache so far, which a launch hides only while that is short.  Longer
-  // sequences go layer by layer, as the same layers called one by one do (and give the same bits).
+  // run ahead): each leaf reads the layer's whole cache so far.  Longer sequences go layer by layer and give the bits of the same layers called one by
+  // one, which the group kernel, whose sums have another order, does not; that is the whole reason.  Side by side would be faster at every length
+  // measured: 8 layers of d = 1024, ms, one by one -> side by side: B = 1 1024 positions 74 -> 45, 2048 150 -> 85, 4096 299 -> 173; B = 16 110 -> 74, 220 -> 147, 447 -> 295.
   if (N > kWaveMaxN || (size_t)N * B * c->d_model * 4 > kWaveCacheMax) return none;
   // Short leaves fill the pipeline of layers sooner, long ones have fewer launches.
   const int leaf = c->leaf ? c->leaf : N <= 128 ? 16 : 32;

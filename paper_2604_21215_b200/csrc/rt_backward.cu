@@ -8,8 +8,10 @@
 //      (the same tiles, visited in reverse order, each as one launch over all its keys),
 //   3. computes everything else -- dq, the temporary pairs, dx and all parameter gradients -- as large products over
 //      all rows at once.
-// The reverse loop and the attention terms are fp32 on CUDA cores; the products over all rows of stages 1 and 3 run on
-// the tensor cores (bf16 copies of the operands, fp32 accumulation) when the storage type is bf16.
+// With bf16 storage the reverse loop runs on the tensor cores, up to 32 sequences on operands of three bf16 terms (2^-24; rt_backward_loop.cu,
+// rt_wide_backward.cu), above on operands rounded to bf16 (rt_wide_backward.cu), and so do the products over all rows of stages 1 and 3, on bf16
+// copies of their operands (weight gradients of ragged row counts: on fp32 operands, see kGemmRows); sums are fp32.  The attention terms
+// and everything with fp32 storage are fp32 on CUDA cores, here.
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>

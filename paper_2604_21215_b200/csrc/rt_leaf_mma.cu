@@ -98,10 +98,9 @@ __device__ __forceinline__ uint4 ld_relaxed_v4_if(const void* p, unsigned on) {
                : "+l"(w0), "+l"(w1) : "l"(p), "r"(on) : "memory");
   return make_uint4((unsigned)w0, (unsigned)(w0 >> 32), (unsigned)w1, (unsigned)(w1 >> 32));
 }
-// 8 bytes through L2 under a predicate (zeros when `on` is zero).  An asm statement, so that a run
-// of these stays a run of loads: written as plain loads the compiler placed each one's first use
-// right behind it and the round trips added up.
-// Words that are their own flags: all ones = not written yet (no pair of bf16 results is: NaN results are 0x7fff).
+// Words that are their own flags: all ones = not written yet (no pair of bf16 results is: NaN results are 0x7fff).  The load
+// fetches 8 bytes again if one of their words is missing; an asm statement, so that a run of these stays a run of loads (written
+// as plain loads the compiler placed each one's first use right behind it and the round trips added up).
 constexpr unsigned kNotYet = 0xffffffffu;
 __device__ __forceinline__ bool missing(const uint2& w) { return (w.x == kNotYet) | (w.y == kNotYet); }
 __device__ __forceinline__ void ld_relaxed_v2_missing(const void* p, uint2& w) {

@@ -1,7 +1,7 @@
 // Leaf recurrence for layers whose weights fit the shared memory of ONE cluster (fp32 up to d = 256, bf16 up to d = 384 with
 // d_ff = 4 d): the sequential part of Algorithm 1 for the positions [t0, t1) of one leaf.
 //
-// The sequences are independent (Sec. 2.2 states the layer per sequence), so a cluster of 16 CTAs takes one or two of them
+// The sequences are independent (Sec. 2.2 states the layer per sequence), so a cluster of 16 CTAs takes one to three of them
 // and clusters never talk to each other.  Inside a cluster a token step is the usual chain of five small all-to-all
 // exchanges, but through distributed shared memory: every vector has a copy in each CTA, the warp that finishes rows of it
 // sends them to all 16 copies with st.async, and the stores count themselves into the receiver's mbarrier.  No flags, no
