@@ -333,9 +333,9 @@ def run_cuda(args):
         leaf_ms = prof["leaf"]["ms"] / n_leaf
         alg_bytes = (chain_w + act) * tok_steps_per_launch
         achieved = alg_bytes / (leaf_ms * 1e-3) / 1e9 if leaf_ms > 0 else 0.0
-        roofline = {"kernel": "leaf_mma_kernel" if (wl.dtype == "bf16" and args.sched == "tiled") else "leaf_kernel", "bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"],
+        roofline = {"kernel": ("leaf_mma_kernel" if B <= 16 else "leaf_group_kernel") if (wl.dtype == "bf16" and args.sched == "tiled") else "leaf_kernel", "bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"],
                     "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"], "peak_source": peaks["source"],
-                    "traffic": leaf_traffic_table().get(wl.name),
+                    "traffic": leaf_traffic_table().get(wl.name) if B <= 16 and not args.batch else None,
                     "algorithmic_bytes_per_launch": alg_bytes, "avg_launch_ms": leaf_ms,
                     "us_per_token_step": 1e3 * leaf_ms / max(tok_steps_per_launch, 1),
                     "note": "weights stay in shared memory for a whole launch, so the kernel is bound by the "
@@ -344,18 +344,18 @@ def run_cuda(args):
                             "traffic is the DRAM bytes ncu counted for one launch"}
         if wl.B > 64:
             # wide batches: the token step is a chain of dense products over the B rows (tcgen05), one position at
-            # a time; the leaf class of the profile holds them together with the small in-leaf attention kernels
+            # a time, a leaf of them in one launch; the leaf class of the profile holds them with the in-leaf attention
             tf_peak = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))).get("bf16_tflops_sustained", 1403.5)) \
                 if os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")) else 1400.0
             flops = 2.0 * B * (5 * d * d + 2 * d * f) * wl.N * wl.n_layers * args.steps      # W_o, W_up, W_down, W_k, W_v per step
             ms_all = prof["leaf"]["ms"]
             achieved = flops / (ms_all * 1e-3) / 1e12 if ms_all > 0 else 0.0
-            roofline = {"kernel": "dense_tc_kernel (wide-batch token steps, with their small kernels)", "bound": "tensor",
+            roofline = {"kernel": "wide_forward_kernel" if wl.dtype == "bf16" and B <= 1024 else "dense products of a token step, with their small kernels", "bound": "tensor",
                         "achieved": achieved, "peak": tf_peak, "unit": "TFLOP/s", "frac": achieved / tf_peak,
                         "peak_source": "measured (sustained)", "traffic": None,
                         "us_per_token_step": 1e3 * ms_all / max(wl.N * wl.n_layers * args.steps, 1),
-                        "note": "M = B rows per product: each token step is seven short dependent launches, so launch latency "
-                                "and the L2 stream of the weights, not the tensor pipe, set the time"}
+                        "note": "M = B rows per product: a token step is six dependent steps between barriers, each fetching its weights "
+                                "from L2 again, and that stream and the barriers, not the tensor pipe, set the time"}
         if args.recur_block > 1:
             # recurrence over blocks: every block is a parallel sweep of dense products and attention tiles
             tf_peak = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))).get("bf16_tflops_sustained", 1403.5)) \
@@ -394,7 +394,7 @@ def run_cuda(args):
                 "n_gpus": world, "steps": args.steps, "warmup": max(args.warmup, 3),
                 "ms_per_step": total_ms / args.steps, "higher_is_better": True, "scaling": "weak",
                 "vs_baseline": None, "dtype": "bf16/f32-accumulate" if wl.dtype == "bf16" else "f32",
-                "data": "synthetic", "config": config_dict(wl, args.sched, {"alibi": bool(args.alibi), "recur_block": int(args.recur_block), "leaf": int(model.cfg.leaf) or (32 if wl.B > 64 else 64),
+                "data": "synthetic", "config": config_dict(wl, args.sched, {"alibi": bool(args.alibi), "recur_block": int(args.recur_block), "leaf": int(model.cfg.leaf) or (16 if wl.B > 64 else 64),
                                                                             "parallelism": f"replicas x{world}"}),
                 "clocks": clocks,
                 "e2e": {"value": replicas.aggregate_tokens_per_s(tokens, args.steps, world, e2e_total), "unit": UNIT,
@@ -700,8 +700,8 @@ def run_backward_bench(args):
                       "backward_tokens_per_s": tok / (bwd_ms * 1e-3), "backward_over_forward": bwd_ms / fwd_ms,
                       "us_per_position_reverse_loop": prof["leaf"]["ms"] * 1e3 / wl.N,
                       "gflop": 3.0 * flops_fwd / 1e9, "tflops": 3.0 * flops_fwd / (bwd_ms * 1e-3) / 1e12,
-                      "arithmetic": "reverse loop and attention terms fp32 on CUDA cores; products over all rows on the tensor cores "
-                                    "for bf16 storage",
+                      "arithmetic": "bf16 storage: reverse loop and products over all rows on the tensor cores (operands of the loop in three bf16 "
+                                    "terms up to 32 sequences, rounded above); attention terms, and all of fp32 storage, fp32 on CUDA cores",
                       "ms_by_phase": {"sweep_of_intermediates": prof["prepass"]["ms"], "reverse_loop_steps": prof["leaf"]["ms"],
                                       "reverse_loop_tiles": prof["tile"]["ms"], "products_over_all_rows": prof["other"]["ms"]},
                       "workspace_gb": ws.numel() / 1e9}))
