@@ -166,3 +166,28 @@ def test_one_position_takes_the_tensor_core_kernels(B):
     chain_w, pre_w = (3 * d * d + 2 * d * dff) * 2, 3 * d * d * 2
     per_token = (rt.rt_plan_counters(layer.cfg, 16, 1)["model_bytes_read"] - chain_w - pre_w) // 16
     assert rt.rt_plan_counters(layer.cfg, B, 1)["model_bytes_read"] - B * per_token - pre_w == chain_w * (1 if B > 48 else -(-B // 16))
+
+
+# One after the other, the layers of a short prompt share arrays of g that are filled together: a launch takes fresh ones, and the last ones do
+# not always suffice for the next layer (64 arrays; 30 + 30 positions and 4 left, 21 x 3 and 1 left; 64 + 6 with a leaf of its own in between).
+@pytest.mark.parametrize("L,B,N", [(24, 1, 3), (3, 9, 30), (2, 4, 70), (5, 20, 1)])
+def test_layers_one_after_the_other_give_the_bits_of_single_layers(L, B, N):
+    import torch
+    from paper_2604_21215_b200 import inputs, rt
+    d, H, dff, V = 640, 10, 1280, 91
+    data = inputs.make_inputs(inputs.Workload("chain", L, B, N, d, H, dff, "bf16", vocab=V, residual_scale=1 / np.sqrt(L)), seed=N)
+    kw = dict(dtype="bf16", leaf=64 if N == 70 else 0, residual_scale=1 / np.sqrt(L))
+    st = rt.Stack(L, d, H, dff, V, **kw)
+    st.set_weights(data["layers"], data["emb"])
+    hid, _ = st.prefill(data["ids"])
+    ids = torch.as_tensor(np.asarray(data["ids"]), dtype=torch.int64, device="cuda")
+    x = st.emb[ids].contiguous()
+    for lw in data["layers"]:
+        layer = rt.Layer(d, H, dff, **kw)
+        layer.set_weights(lw)
+        layer.reserve(B, N)
+        z = torch.empty_like(x)
+        layer.prefill_device(x, z)
+        torch.cuda.synchronize()
+        x = z
+    assert (x.float().cpu().numpy() == hid).all()
