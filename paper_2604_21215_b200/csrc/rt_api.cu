@@ -91,37 +91,69 @@ Schedule effective_schedule(const rt_config* c, int B, int N) {
   return {kPathGeneric, leaf_size(c), 0};
 }
 
-// The layers of a stack side by side (rt_leaf_group.cu): layer l works on a leaf that layer l-1 finished one launch
-// earlier, up to `places` layers in a launch, a group of SMs each.  places = 0: one layer after the other.
+// The layers of a stack side by side (rt_leaf_group.cu): layer l works on a leaf that layer l-1 finished in an earlier
+// launch, up to `places` layers in a launch, a group of SMs each.  places = 0: one layer after the other.
 struct Wave { int places, leaf; };
-constexpr size_t kWaveCacheMax = (size_t)512 << 20;
-constexpr int kWaveMaxN = 1024;
-constexpr int kWaveFoldMax = 192;        // leaves that begin earlier absorb all earlier pairs inside the leaf kernel
+constexpr int kWaveBand = 16;            // layers whose packed weights the workspace holds at a time
+// longest leaf of layers side by side (what the workspace holds rows for)
+int wave_leaf_max(const rt_config* c, int N) { return c->leaf ? c->leaf : N <= 128 ? 16 : N <= 1024 ? 32 : 64; }
+constexpr int kWaveBlock = 64;           // earlier pairs come by whole blocks of this many from the tile kernel, the rest of them inside the leaf kernel
+// Which leaves of which layers of a stack run together: a leaf is ready when the layer below has finished it and its own layer the one before.  Of
+// the ready ones those with the most leaves still to come after them in a row (of their layer and the layers above) go first, of equal ones the
+// deepest layer: 8 layers of 5 leaves in 4 places take 13 launches, 12 being the least possible, of 64 leaves in 6 places 91 (86).
+struct WaveOrder {
+  int n_layers, n_leaves, done[kWaveBand];
+  WaveOrder(int layers, int leaves) : n_layers(layers), n_leaves(leaves), done{} {}
+  // The next launch: up to `places` (layer, leaf) pairs; 0 when all leaves are done.
+  int next(int places, int* layer, int* leaf) {
+    int n = 0;
+    for (int sum = 0; sum <= n_layers + n_leaves && n < places; ++sum)       // layer + leaf: the smaller, the more is to come
+      for (int l = n_layers - 1; l >= 0 && n < places; --l)
+        if (done[l] < n_leaves && l + done[l] == sum && (l == 0 || done[l - 1] > done[l])) { layer[n] = l; leaf[n++] = done[l]; }
+    for (int i = 0; i < n; ++i) ++done[layer[i]];
+    return n;
+  }
+};
 Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
   const Wave none = {0, 0};
   if (n_layers < 2 || N < 2 || c->dtype != RT_BF16 || c->sched != RT_SCHED_TILED || c->recur_block > 1) return none;
-  const int places = n_layers < kGroupJobs ? n_layers : kGroupJobs;
-  if (!leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, places, kB200SmemPerCta)) return none;
   LeafMmaLaunch ml;                                            // (a stack of layers for the generic kernel keeps its fp32 vectors)
   if (!leaf_mma_shape(B, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml)) return none;
   // A leaf meets all earlier pairs at once when its queries exist (they depend on the layer below, so Algorithm 1's tiles cannot
-  // run ahead): each leaf reads the layer's whole cache so far.  Longer sequences go layer by layer and give the bits of the same layers called one by
-  // one, which the group kernel, whose sums have another order, does not; that is the whole reason.  Side by side would be faster at every length
-  // measured: 8 layers of d = 1024, ms, one by one -> side by side: B = 1 1024 positions 74 -> 45, 2048 150 -> 85, 4096 299 -> 173; B = 16 110 -> 74, 220 -> 147, 447 -> 295.
-  if (N > kWaveMaxN || (size_t)N * B * c->d_model * 4 > kWaveCacheMax) return none;
-  // Short leaves fill the pipeline of layers sooner, long ones have fewer launches.
-  const int leaf = c->leaf ? c->leaf : N <= 128 ? 16 : 32;
+  // run ahead): each leaf reads the layer's whole cache so far, in the parts in which those tiles would have brought it.  The group kernel's sums have the order
+  // of the leaf kernel, so a stack gives the bits of the same layers called one by one, where those take leaves of kWaveBlock positions and widths for which
+  // both deal out the contractions alike; elsewhere long sequences go layer by layer for the sake of these bits.
+  if (N > 1024 && (ml.leaf != kWaveBlock || !leaf_group_same_sums(c->d_model, c->d_ff))) return none;
+  // How many layers at a time, and by which leaves: the least of launches x (positions x time of a position + what a launch costs besides: pre-passes, tiles, the
+  // first weights, us measured as below).  More places fill and drain the pipeline of layers in fewer launches, but a group of fewer SMs streams and multiplies
+  // more weights per SM; short leaves fill it sooner, long ones have fewer launches.  8 layers, ms for 4 / 6 / 8 places with leaves of 16, then of 32: d = 1024,
+  // B = 16, N = 512 31.4 32.7 35.1, 30.0 32.5 35.6; d = 768 25.3 21.6 23.8, 24.3 21.1 24.2; d = 512 20.5 16.3 15.5, 19.5 16.6 16.0; d = 1024, B = 1 22.9 22.7 21.3, 21.8 23.6 22.9.
+  const float layer_mb = (3.0f * c->d_model + 2.0f * c->d_ff) * c->d_model * 2e-6f;
+  const int band = n_layers < kWaveBand ? n_layers : kWaveBand;
+  int places = 0, leaf = 0, launches = 0;
+  float least = 0.0f;
+  for (int pl = 2; pl <= kGroupJobs && pl <= n_layers; ++pl) {
+    if (!leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, pl, kB200SmemPerCta)) continue;
+    const float step = leaf_group_step_us(B, c->d_model, c->d_ff, pl);
+    for (int lf = c->leaf ? c->leaf : 16; lf <= wave_leaf_max(c, N); lf *= 2) {
+      WaveOrder order(band, ceil_div(N, lf));
+      int n = 0, layer_of[kGroupJobs], leaf_of[kGroupJobs];
+      while (order.next(pl, layer_of, leaf_of) > 0) ++n;
+      const float us = (float)n * ((float)lf * step + (B > 8 ? 20.0f + 1.35f * layer_mb * (float)pl : 33.0f + 0.35f * layer_mb * (float)pl));
+      if (!places || us < least) { places = pl; leaf = lf; launches = n; least = us; }
+    }
+  }
+  if (!places) return none;
   // Side by side a position costs a layer more (fewer SMs, weights from L2), so enough layers have to be at work at the same time: on average
   // n_layers * N / (waves * leaf) of them.  Break even was measured at 1.3 to 2.3, growing with the weights that the groups stream (places x MB
   // per layer) and above four sequences: 8 layers of d = 1024, B = 1, take 1.69 times as long as one after the other for 16 positions (one layer at a
   // time), 1.05 for 32, 0.84 for 48, 0.72 for 77; B = 16 1.98, 1.20, 0.95 and for 64 0.83; 2 layers 1.33, 1.09, 1.03 and for 128 0.97.  Layers
   // that fit a cluster (rt_leaf_small.cu) are faster alone than the tensor-core leaf kernel, taken as 8.3 us a position, above eight sequences 10.5; it
   // takes as many more.  Over 2 to 8 layers, d = 128 to 1024, 1 to 16 sequences and 16 to 400 positions the side taken is at most about a tenth slower than the other.
-  const int n_leaves = ceil_div(N, leaf), turn = n_leaves > places ? n_leaves : places;
-  const float waves = (float)((n_layers - 1) / places * turn + (n_layers - 1) % places + n_leaves), at_work = (float)n_layers * (float)N / (waves * (float)leaf);
-  const float layer_mb = (3.0f * c->d_model + 2.0f * c->d_ff) * c->d_model * 2e-6f, mma_us = B > 8 ? 10.5f : 8.3f;
+  const float at_work = (float)band * (float)N / ((float)launches * (float)leaf), mma_us = B > 8 ? 10.5f : 8.3f;
   LeafSmallLaunch sl;
   const bool small = leaf_small_shape(c->dtype, B, c->d_model, c->n_heads, c->d_ff, ml.leaf, kB200SmemPerCta, &sl);
+  if (small && N > 1024) return none;                          // (the bits of that kernel)
   const float even = (1.26f + 0.008f * places * layer_mb + (B > 4 ? 0.15f : 0.0f)) * (small && sl.step_us < mma_us ? mma_us / sl.step_us : 1.0f);
   return at_work > even ? Wave{places, leaf} : none;
 }
@@ -160,8 +192,7 @@ int g_positions(const rt_config* c, int N, int n_layers) {
 
 // Bytes of the area that the form of the token loop has to itself: the most that any call of at most B sequences, N positions and n_layers
 // layers asks for, whichever form it takes, so that a workspace reserved for the longest prompt and the fullest batch serves all the others.
-// (What one form asks for by itself does not grow with the shape: beyond kWaveMaxN positions no layers run side by side, from 17
-// sequences on there is no array of g.)
+// (What one form asks for by itself does not grow with the shape: from 17 sequences on there is no array of g.)
 size_t form_bytes(const rt_config* c, int B, int N, int n_layers) {
   if (c->dtype != RT_BF16) return 0;
   if (c->sched != RT_SCHED_TILED || c->recur_block > 1) return 0;
@@ -173,7 +204,7 @@ size_t form_bytes(const rt_config* c, int B, int N, int n_layers) {
   for (int places = 2; places <= kGroupJobs; ++places) {
     if (!leaf_group_shape(1, d, H, f, places, kB200SmemPerCta)) continue;
     if (B > 16 * (places - 1)) need(group_area(c, places, 1, 0, 0).total);
-    if (n_layers >= places) need(group_area(c, places, places, B16, c->leaf ? c->leaf : N <= 128 ? 16 : 32).total);
+    if (n_layers >= places) need(group_area(c, places, n_layers < kWaveBand ? n_layers : kWaveBand, B16, wave_leaf_max(c, N)).total);
   }
   return most;
 }
@@ -267,13 +298,13 @@ struct ProfScope {
 };
 
 // State of one API call: the stream and the barrier arrivals enqueued so far.
-struct CallCtx { cudaStream_t s; unsigned bar_base = 0; unsigned seq_base = 0; unsigned group_steps[kGroupJobs] = {0, 0, 0, 0}; bool groups_zeroed = false; int g_left = 0; };      // g_left: arrays of g still filled
+struct CallCtx { cudaStream_t s; unsigned bar_base = 0; unsigned seq_base = 0; unsigned group_steps[kGroupJobs] = {}; bool groups_cleared = false; int g_left = 0; };      // g_left: arrays of g still filled
 
-// The exchange areas of the group kernel start from zero, once per API call.
-bool zero_groups(const rt_config* c, unsigned char* ws, const WsLayout& L, CallCtx& ctx) {
-  if (ctx.groups_zeroed) return true;
-  ctx.groups_zeroed = true;
-  return cudaMemsetAsync(ws + L.form, 0, (size_t)kGroupJobs * leaf_group_words_bytes(c->d_model, c->d_ff), ctx.s) == cudaSuccess;
+// The exchange areas of the group kernel start from ones (no word written), once per API call.
+bool clear_groups(const rt_config* c, unsigned char* ws, const WsLayout& L, CallCtx& ctx) {
+  if (ctx.groups_cleared) return true;
+  ctx.groups_cleared = true;
+  return cudaMemsetAsync(ws + L.form, 0xFF, (size_t)kGroupJobs * leaf_group_words_bytes(c->d_model, c->d_ff), ctx.s) == cudaSuccess;
 }
 GroupCommon group_common(const rt_config* c, int B, unsigned char* ws, const WsLayout& L) {
   GroupCommon g;
@@ -582,7 +613,7 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   const int places = groups ? ceil_div(B, plan.sub) : 0;
   unsigned char* const packed = groups ? ws + L.form + group_area(c, places, 1, 0, 0).packed : nullptr;
   if (groups) {
-    if (!zero_groups(c, ws, L, ctx)) return RT_ERR_CUDA;
+    if (!clear_groups(c, ws, L, ctx)) return RT_ERR_CUDA;
     const GroupPackLayer pl = {w->w_o, w->w_up, w->w_down, w->w_k, w->w_v, packed};
     ProfScope ps(s, kProfPrepass);
     if (leaf_group_pack(&pl, 1, c->d_model, c->d_ff, places, s) != cudaSuccess) return RT_ERR_CUDA;
@@ -635,84 +666,92 @@ bool caches_overlap(const rt_config* c, int n_layers, int B, int N, void* const*
 rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weights* layers, void* const* hid, void* out, int B, int N, void* const* k_caches,
                          void* const* v_caches, int N_max, unsigned char* ws, const WsLayout& L, const Wave& wv, CallCtx& ctx) {
   cudaStream_t s = ctx.s;
-  const int places = wv.places, n_leaves = ceil_div(N, wv.leaf);
+  const int places = wv.places, n_leaves = ceil_div(N, wv.leaf), band_max = n_layers < kWaveBand ? n_layers : kWaveBand;
   const size_t e = esize_of(c->dtype), d = c->d_model;
   const WaveRows W = wave_rows_layout(c, B, wv.leaf);
-  const GroupArea A = group_area(c, places, places, B, wv.leaf);
-  if (!zero_groups(c, ws, L, ctx)) return RT_ERR_CUDA;
-  // A layer takes the place of the one `places` before it when that has finished its last leaf; its weights are packed into the place then.
-  const int turn = n_leaves > places ? n_leaves : places;
-  auto start = [&](int l) { return l / places * turn + l % places; };                       // wave in which a layer begins
-  auto packed = [&](int place) { return ws + L.form + A.packed + (size_t)place * A.packed_stride; };
-  auto pack = [&](int l0, int n) {
-    GroupPackLayer pl[kGroupJobs];
-    for (int i = 0; i < n; ++i) {
-      const rt_layer_weights& w = layers[l0 + i];
-      pl[i] = {w.w_o, w.w_up, w.w_down, w.w_k, w.w_v, packed((l0 + i) % places)};
-    }
-    ProfScope ps(s, kProfPrepass);
-    return leaf_group_pack(pl, n, c->d_model, c->d_ff, places, s) == cudaSuccess;
-  };
-  if (!pack(0, places)) return RT_ERR_CUDA;
+  const GroupArea A = group_area(c, places, band_max, B, wv.leaf);
+  if (!clear_groups(c, ws, L, ctx)) return RT_ERR_CUDA;
+  auto packed = [&](int l) { return ws + L.form + A.packed + (size_t)l * A.packed_stride; };
   const GroupCommon gc = group_common(c, B, ws, L);
   const long long bs = (long long)N * d;
-  for (int wave = 0, waves = start(n_layers - 1) + n_leaves; wave < waves; ++wave) {
-    GroupJob jobs[kGroupJobs];
-    memset(jobs, 0, sizeof(jobs));
-    int nj = 0, np = 0;
-    PrepassParams pre[kGroupJobs];
-    int layer_of[kGroupJobs];
-    for (int l = 0; l < n_layers; ++l) {
-      const int k = wave - start(l);
-      if (k < 0 || k >= n_leaves) continue;
-      if (k == 0 && l >= places && !pack(l, 1)) return RT_ERR_CUDA;
-      const rt_layer_weights& w = layers[l];
-      const int place = l % places, t0 = k * wv.leaf, t1 = t0 + wv.leaf < N ? t0 + wv.leaf : N;
-      unsigned char* rows = ws + L.form + A.rows + A.rows_stride * place;
-      const void* x = hid[l & 1];
-      PrepassParams& pp = pre[np];
-      memset(&pp, 0, sizeof(pp));
-      layer_of[np++] = l;
-      pp.B = B; pp.N = t1 - t0; pp.d = c->d_model; pp.H = c->n_heads; pp.norm_flags = c->norm_flags; pp.eps = c->rms_eps; pp.scale_log2 = gc.scale_log2;
-      pp.x = (const unsigned char*)x + (size_t)t0 * d * e; pp.x_bs = bs; pp.x_ts = (long long)d;
-      pp.w_q = w.w_q; pp.w_k = w.w_k; pp.w_v = w.w_v; pp.g_attn = w.g_attn; pp.g_q = w.g_q; pp.g_k = w.g_k;
-      pp.n = rows + W.n; pp.q = rows + W.q; pp.kt = rows + W.kt; pp.vt = rows + W.vt;
-      pp.st_o = (float*)(rows + W.st_o); pp.st_m = (float*)(rows + W.st_m); pp.st_l = (float*)(rows + W.st_l); pp.sync = gc.sync;
-    }
+  for (int l0 = 0; l0 < n_layers; l0 += kWaveBand) {
+    const int band = n_layers - l0 < kWaveBand ? n_layers - l0 : kWaveBand;
     {
       ProfScope ps(s, kProfPrepass);
-      if (prepass_batch_launch(c->dtype, pre, np, s) != cudaSuccess) return RT_ERR_CUDA;
-    }
-    for (int i = 0; i < np; ++i) {
-      const int l = layer_of[i];
-      const PrepassParams& pp = pre[i];
-      const rt_layer_weights& w = layers[l];
-      const int k = wave - start(l), place = l % places, t0 = k * wv.leaf, t1 = t0 + wv.leaf < N ? t0 + wv.leaf : N;
-      const void* x = hid[l & 1];
-      GroupJob& j = jobs[nj++];
-      j.key0 = 0;
-      if (t0 >= kWaveFoldMax) {
-        // the leaf's queries against the whole blocks of 64 earlier pairs; the kernel's attention warps absorb the rest
-        TileParams tp;
-        memset(&tp, 0, sizeof(tp));
-        tp.B = B; tp.d = c->d_model; tp.H = c->n_heads; tp.scale_log2 = gc.scale_log2; tp.alibi = w.alibi_slopes;
-        tp.q = pp.q; tp.k_cache = k_caches[l]; tp.v_cache = v_caches[l]; tp.st_o = pp.st_o; tp.st_m = pp.st_m; tp.st_l = pp.st_l;
-        tp.rows_q = t1 - t0; tp.rows_kv = N_max; tp.sync = gc.sync; tp.q_pos0 = t0;
-        tp.q0 = 0; tp.q1 = t1 - t0; tp.k0 = 0; tp.k1 = t0 & ~63;
-        j.key0 = tp.k1;
-        ProfScope ps(s, kProfTile);
-        if (tile_tc_launch(tp, tp.rows_q, tp.rows_kv, tp.sync, s) != cudaSuccess) return RT_ERR_CUDA;
+      for (int i = 0; i < band; i += kGroupPackLayers) {
+        GroupPackLayer pl[kGroupPackLayers];
+        const int here = band - i < kGroupPackLayers ? band - i : kGroupPackLayers;
+        for (int k = 0; k < here; ++k) {
+          const rt_layer_weights& w = layers[l0 + i + k];
+          pl[k] = {w.w_o, w.w_up, w.w_down, w.w_k, w.w_v, packed(i + k)};
+        }
+        if (leaf_group_pack(pl, here, c->d_model, c->d_ff, places, s) != cudaSuccess) return RT_ERR_CUDA;
       }
-      j.packed = packed(place); j.g_mlp = w.g_mlp; j.g_kv = w.g_kv ? w.g_kv : w.g_attn; j.g_k = w.g_k; j.alibi = w.alibi_slopes;
-      j.q = pp.q; j.st_o = pp.st_o; j.st_m = pp.st_m; j.st_l = pp.st_l; j.row_off = t0;
-      j.x = x; j.x_bs = bs; j.x_ts = (long long)d;
-      j.z = l == n_layers - 1 && out ? out : hid[(l + 1) & 1]; j.z_bs = bs; j.z_ts = (long long)d;
-      j.k_cache = k_caches[l]; j.v_cache = v_caches[l]; j.t0 = t0; j.t1 = t1; j.B = B; j.b0 = 0;
-      j.words = ws + L.form + (size_t)place * leaf_group_words_bytes(c->d_model, c->d_ff); j.steps = ctx.group_steps[place];
-      ctx.group_steps[place] += (unsigned)(t1 - t0);
     }
-    ProfScope ps(s, kProfLeaf);
-    if (leaf_group_launch(gc, jobs, nj, places, s) != cudaSuccess) return RT_ERR_CUDA;
+    WaveOrder order(band, n_leaves);
+    int of[kGroupJobs], leaf_of[kGroupJobs];
+    for (int nj; (nj = order.next(places, of, leaf_of)) > 0;) {
+      GroupJob jobs[kGroupJobs];
+      PrepassParams pre[kGroupJobs];
+      memset(jobs, 0, sizeof(jobs));
+      memset(pre, 0, sizeof(pre));
+      for (int i = 0; i < nj; ++i) {
+        const int l = l0 + of[i], t0 = leaf_of[i] * wv.leaf, t1 = t0 + wv.leaf < N ? t0 + wv.leaf : N;
+        const rt_layer_weights& w = layers[l];
+        unsigned char* rows = ws + L.form + A.rows + A.rows_stride * i;
+        PrepassParams& pp = pre[i];
+        pp.B = B; pp.N = t1 - t0; pp.d = c->d_model; pp.H = c->n_heads; pp.norm_flags = c->norm_flags; pp.eps = c->rms_eps; pp.scale_log2 = gc.scale_log2;
+        pp.x = (const unsigned char*)hid[l & 1] + (size_t)t0 * d * e; pp.x_bs = bs; pp.x_ts = (long long)d;
+        pp.w_q = w.w_q; pp.w_k = w.w_k; pp.w_v = w.w_v; pp.g_attn = w.g_attn; pp.g_q = w.g_q; pp.g_k = w.g_k;
+        pp.n = rows + W.n; pp.q = rows + W.q; pp.kt = rows + W.kt; pp.vt = rows + W.vt;
+        pp.st_o = (float*)(rows + W.st_o); pp.st_m = (float*)(rows + W.st_m); pp.st_l = (float*)(rows + W.st_l); pp.sync = gc.sync;
+        GroupJob& j = jobs[i];
+        j.packed = packed(of[i]); j.g_mlp = w.g_mlp; j.g_kv = w.g_kv ? w.g_kv : w.g_attn; j.g_k = w.g_k; j.alibi = w.alibi_slopes;
+        j.q = pp.q; j.st_o = pp.st_o; j.st_m = pp.st_m; j.st_l = pp.st_l; j.row_off = t0;
+        j.x = hid[l & 1]; j.x_bs = bs; j.x_ts = (long long)d;
+        j.z = l == n_layers - 1 && out ? out : hid[(l + 1) & 1]; j.z_bs = bs; j.z_ts = (long long)d;
+        j.k_cache = k_caches[l]; j.v_cache = v_caches[l]; j.t0 = t0; j.t1 = t1; j.B = B; j.b0 = 0;
+        j.key0 = t0 / kWaveBlock * kWaveBlock;
+        j.words = ws + L.form + (size_t)i * leaf_group_words_bytes(c->d_model, c->d_ff); j.steps = ctx.group_steps[i];
+        ctx.group_steps[i] += (unsigned)(t1 - t0);
+      }
+      {
+        ProfScope ps(s, kProfPrepass);
+        if (prepass_batch_launch(c->dtype, pre, nj, s) != cudaSuccess) return RT_ERR_CUDA;
+      }
+      // The leaf's queries against the whole blocks of kWaveBlock earlier pairs, in the parts in which Algorithm 1's tiles would have brought them
+      // (the powers of two that the number of blocks consists of, largest first): the same states to the bit.  The kernel absorbs the rest.
+      for (int part = 0, more = 1; more; ++part) {
+        more = 0;
+        for (int sloped = 0; sloped < 2; ++sloped) {
+          TileParams tiles[kGroupJobs];
+          int nt = 0;
+          for (int i = 0; i < nj; ++i) {
+            int blocks = jobs[i].key0 / kWaveBlock, k0 = 0, size = 0;
+            for (int skip = 0; blocks && skip <= part; ++skip) {
+              k0 += size;
+              size = 1;
+              while (size * 2 <= blocks) size *= 2;
+              blocks -= size;
+              if (skip == part) {
+                more |= blocks > 0;
+                if ((jobs[i].alibi != nullptr) != (sloped != 0)) break;
+                TileParams& tp = tiles[nt++];
+                memset(&tp, 0, sizeof(tp));
+                tp.B = B; tp.d = c->d_model; tp.H = c->n_heads; tp.scale_log2 = gc.scale_log2; tp.alibi = jobs[i].alibi;
+                tp.q = pre[i].q; tp.k_cache = jobs[i].k_cache; tp.v_cache = jobs[i].v_cache; tp.st_o = pre[i].st_o; tp.st_m = pre[i].st_m; tp.st_l = pre[i].st_l;
+                tp.rows_q = pre[i].N; tp.rows_kv = N_max; tp.sync = gc.sync; tp.q_pos0 = jobs[i].t0;
+                tp.q0 = 0; tp.q1 = pre[i].N; tp.k0 = k0 * kWaveBlock; tp.k1 = (k0 + size) * kWaveBlock;
+              }
+            }
+          }
+          ProfScope ps(s, kProfTile);
+          if (tile_tc_batch_launch(tiles, nt, gc.sync, s) != cudaSuccess) return RT_ERR_CUDA;
+        }
+      }
+      ProfScope ps(s, kProfLeaf);
+      if (leaf_group_launch(gc, jobs, nj, places, s) != cudaSuccess) return RT_ERR_CUDA;
+    }
   }
   return RT_OK;
 }

@@ -66,7 +66,7 @@ bool leaf_small_shape(int dtype, int B, int d, int H, int dff, int leaf, size_t 
 cudaError_t leaf_small_launch(int dtype, const LeafParams& p, const LeafSmallLaunch& l, cudaStream_t s);
 
 // Leaf kernel for several independent (layer, slice) jobs side by side, a group of SMs each (bf16; rt_leaf_group.cu).
-constexpr int kGroupJobs = 4;
+constexpr int kGroupJobs = 8;
 struct GroupJob {
   const void* packed;                            // W_o, W_up, W_down, W_k, W_v in the order of use (leaf_group_pack)
   const void *g_mlp, *g_kv, *g_k;                // storage type or NULL
@@ -80,7 +80,7 @@ struct GroupJob {
   int t0, t1;                                    // positions
   int key0;                                      // first position whose pair is not in the states yet (key0 <= t0)
   int B, b0;                                     // sequences of the slice, first column in q / state / caches
-  unsigned char* words;                          // exchange area of the job's place, zeroed once per API call
+  unsigned char* words;                          // exchange area of the job's place, filled with ones once per API call
   unsigned steps;                                // token steps enqueued on that place before this launch in the same call
 };
 struct GroupCommon {
@@ -93,6 +93,8 @@ constexpr int kGroupPackLayers = 8;
 struct GroupPackLayer { const void *w_o, *w_up, *w_down, *w_k, *w_v; void* out; };
 struct GroupPackArgs { int d, dff, g; GroupPackLayer layer[kGroupPackLayers]; };
 bool leaf_group_shape(int B, int d, int H, int dff, int places, size_t max_smem);   // B: sequences of one job; groups of 148 / places SMs
+bool leaf_group_same_sums(int d, int dff);
+float leaf_group_step_us(int B, int d, int dff, int places);                         // estimate of the time per position
 size_t leaf_group_words_bytes(int d, int dff);   // exchange area of one place
 size_t leaf_group_packed_bytes(int d, int dff, int places);
 cudaError_t leaf_group_pack(const GroupPackLayer* layers, int n, int d, int dff, int places, cudaStream_t s);
@@ -135,7 +137,7 @@ struct PrepassParams {
 };
 cudaError_t prepass_launch(int dtype, const PrepassParams& p, cudaStream_t s);
 // The pre-passes of up to kPrepassBatch layers' rows together (same B, d and flags): three launches for all of them.
-constexpr int kPrepassBatch = 4;
+constexpr int kPrepassBatch = 8;
 struct PrepassBatch { PrepassParams p[kPrepassBatch]; };
 cudaError_t prepass_batch_launch(int dtype, const PrepassParams* p, int n, cudaStream_t s);
 // tensor-core projection (bf16, d a multiple of 128)
@@ -166,6 +168,8 @@ struct TileParams {
 cudaError_t tile_launch(int dtype, const TileParams& p, cudaStream_t s);
 // tensor-core version (bf16, key count a multiple of 64)
 cudaError_t tile_tc_launch(const TileParams& p, int rows_q, int rows_kv, SyncArea* sync, cudaStream_t s);
+// one tile of each of n layers (n <= kGroupJobs, key counts multiples of 64, the same B, d, H; slopes in all or none)
+cudaError_t tile_tc_batch_launch(const TileParams* p, int n, SyncArea* sync, cudaStream_t s);
 cudaError_t tile_simt_launch(int dtype, const TileParams& p, cudaStream_t s);
 // one query row (position q0) per (sequence, head) against the pairs [k0, k1): the in-leaf step of wide batches
 cudaError_t row_attn_launch(int dtype, const TileParams& p, cudaStream_t s);

@@ -165,7 +165,7 @@ __device__ __forceinline__ void frag_ssq_gain(unsigned (&a)[4], const __nv_bfloa
 #pragma unroll
   for (int r = 0; r < MB; ++r) {
     const float v0 = bf_lo(a[r]), v1 = bf_hi(a[r]), v2 = bf_lo(a[2 + r]), v3 = bf_hi(a[2 + r]);
-    const float s = v0 * v0 + v1 * v1 + v2 * v2 + v3 * v3;
+    const float s = fmaf(v3, v3, fmaf(v2, v2, fmaf(v1, v1, v0 * v0)));
     if (r == 0) sq0 += s; else sq1 += s;
     if (gp) { a[r] = pack_bf2(v0 * gn[0], v1 * gn[1]); a[2 + r] = pack_bf2(v2 * gn[2], v3 * gn[3]); }
   }
@@ -244,7 +244,7 @@ __device__ void attention_role(const LeafParams& p, const LeafMmaLayout& L, unsi
     if (timing) { const unsigned long long now = globaltimer_ns(); a_wait += now - t_mark; t_mark = now; }
     // Eq. (1): qkRMS over the head, then the storage rounding the cache applies
     const float k0 = __uint_as_float(kw.x), k1 = __uint_as_float(kw.z);
-    const float ss = warp_sum(k0 * k0 + k1 * k1);
+    const float ss = warp_sum(fmaf(k1, k1, k0 * k0));
     const float rs = qkn ? rsqrtf(ss * (1.0f / kHeadDim) + p.eps) : 1.0f;
     const unsigned kq = pack_bf2(k0 * rs * gk0, k1 * rs * gk1);
     const unsigned vq = pack_bf2(__uint_as_float(vw.x), __uint_as_float(vw.z));
@@ -257,13 +257,13 @@ __device__ void attention_role(const LeafParams& p, const LeafMmaLayout& L, unsi
       // critical path: finish query j+1 and publish c_{j+1}
       const int i = j + 1;
       const unsigned qw = QSMEM ? *reinterpret_cast<const unsigned*>(qs + i * kQStride + 2 * lane) : q_next;
-      const float s = warp_sum(bf_lo(qw) * kf0 + bf_hi(qw) * kf1) * p.scale_log2 - slope_l2;      // distance (j+1) - j = 1
+      const float s = fmaf(warp_sum(fmaf(bf_hi(qw), kf1, bf_lo(qw) * kf0)), p.scale_log2, -slope_l2);      // distance (j+1) - j = 1
       const float m_old = ms[i], l_old = ls[i];
       const float m_new = fmaxf(m_old, s);
       const float corr = exp2f(m_old - m_new), pj = exp2f(s - m_new);
-      const float il = 1.0f / (l_old * corr + pj);
-      const float o0 = os[i * kOStride + 2 * lane] * corr + pj * vf0;
-      const float o1 = os[i * kOStride + 2 * lane + 1] * corr + pj * vf1;
+      const float il = 1.0f / fmaf(l_old, corr, pj);
+      const float o0 = fmaf(os[i * kOStride + 2 * lane], corr, pj * vf0);
+      const float o1 = fmaf(os[i * kOStride + 2 * lane + 1], corr, pj * vf1);
       st_relaxed_u64(c_word, pack_bf2(o0 * il, o1 * il), seq + 1u);
     }
     // off the critical path: fold (k_j, v_j) into the later queries of the leaf, one query per lane
@@ -271,34 +271,39 @@ __device__ void attention_role(const LeafParams& p, const LeafMmaLayout& L, unsi
     vbuf[2 * lane] = vf0; vbuf[2 * lane + 1] = vf1;
     __syncwarp();
     for (int i = j + 2 + lane; i < n; i += 32) {
-      float s = 0.f;
+      // the product with the query in the order of warp_sum (term L = dimensions 2 L, 2 L + 1; neighbours at distance 16, 8, 4, 2, 1), as everywhere
+      float part[8];
       if (QSMEM) {
         const __nv_bfloat16* qi = qs + i * kQStride;
-#pragma unroll 8
-        for (int e = 0; e < kHeadDim; e += 2) {
-          const unsigned qw = *reinterpret_cast<const unsigned*>(qi + e);
-          s += bf_lo(qw) * kbuf[e] + bf_hi(qw) * kbuf[e + 1];
-        }
+        auto term = [&](int t) {
+          const unsigned qw = *reinterpret_cast<const unsigned*>(qi + 2 * t);
+          return fmaf(bf_hi(qw), kbuf[2 * t + 1], bf_lo(qw) * kbuf[2 * t]);
+        };
+#pragma unroll
+        for (int t = 0; t < 8; ++t) part[t] = (term(t) + term(t + 16)) + (term(t + 8) + term(t + 24));
       } else {
         const uint4* qg = reinterpret_cast<const uint4*>(q + ((size_t)(p.t0 - p.row_off + i) * Bs + bc) * d + h * kHeadDim);
         uint4 qv[8];
 #pragma unroll
         for (int v = 0; v < 8; ++v) qv[v] = qg[v];
+        auto term = [&](int t) {
+          const uint4& w = qv[t >> 2];
+          const unsigned qw = (t & 3) == 0 ? w.x : (t & 3) == 1 ? w.y : (t & 3) == 2 ? w.z : w.w;
+          return fmaf(bf_hi(qw), kbuf[2 * t + 1], bf_lo(qw) * kbuf[2 * t]);
+        };
 #pragma unroll
-        for (int v = 0; v < 8; ++v) {
-          s += bf_lo(qv[v].x) * kbuf[8 * v] + bf_hi(qv[v].x) * kbuf[8 * v + 1] + bf_lo(qv[v].y) * kbuf[8 * v + 2] + bf_hi(qv[v].y) * kbuf[8 * v + 3] +
-               bf_lo(qv[v].z) * kbuf[8 * v + 4] + bf_hi(qv[v].z) * kbuf[8 * v + 5] + bf_lo(qv[v].w) * kbuf[8 * v + 6] + bf_hi(qv[v].w) * kbuf[8 * v + 7];
-        }
+        for (int t = 0; t < 8; ++t) part[t] = (term(t) + term(t + 16)) + (term(t + 8) + term(t + 24));
       }
-      s = s * p.scale_log2 - slope_l2 * (float)(i - j);
+      float s = ((part[0] + part[4]) + (part[2] + part[6])) + ((part[1] + part[5]) + (part[3] + part[7]));
+      s = fmaf(s, p.scale_log2, -(slope_l2 * (float)(i - j)));
       const float m_old = ms[i];
       const float m_new = fmaxf(m_old, s);
       const float corr = exp2f(m_old - m_new), pj = exp2f(s - m_new);
       ms[i] = m_new;
-      ls[i] = ls[i] * corr + pj;
+      ls[i] = fmaf(ls[i], corr, pj);
       float* oi = os + i * kOStride;
 #pragma unroll 8
-      for (int e = 0; e < kHeadDim; ++e) oi[e] = oi[e] * corr + pj * vbuf[e];
+      for (int e = 0; e < kHeadDim; ++e) oi[e] = fmaf(oi[e], corr, pj * vbuf[e]);
     }
     __syncwarp();
   }

@@ -104,9 +104,7 @@ enum { BAR_KV_FULL = 0, BAR_KV_EMPTY = 2, BAR_Q_FULL = 4, BAR_S_READY = 5, BAR_P
 // ALIBI / CAUSAL are compile-time so that the plain kernel carries none of their registers or instructions
 // (four CTAs per SM leave its softmax threads 88 registers, and it loses up to a fifth of its rate to a few spills).
 template <bool ALIBI, bool CAUSAL>
-__global__ void __launch_bounds__(TcCfg::threads, TcCfg::ctas_per_sm)
-tile_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-               const __grid_constant__ CUtensorMap map_v, const TileParams p, SyncArea* sync) {
+__device__ __forceinline__ void tile_tc(const CUtensorMap& map_q, const CUtensorMap& map_k, const CUtensorMap& map_v, const TileParams& p, SyncArea* sync) {
   using C = TcCfg;
   constexpr int kStages = C::stages;
   constexpr int kMmaWarp = 4, kTmaWarp = 5;
@@ -117,6 +115,7 @@ tile_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   const int b = blockIdx.y / p.H, h = blockIdx.y % p.H;
   // copy blockIdx.z of the tile (one level of Algorithm 1 in one launch); the few values derived from it are
   // recomputed where they are used rather than kept in registers across the roles
+  // (tiles of several layers in one launch: blockIdx.z is the layer, batch_stride 0)
   auto shift = [&]() { return (int)blockIdx.z * p.batch_stride; };
   auto q_end = [&]() { const int q1 = p.q1 + shift(); return (p.q_limit > 0 && q1 > p.q_limit) ? p.q_limit : q1; };
   // (whole causal prefix in one launch: the CTAs with the most key blocks come first)
@@ -360,6 +359,20 @@ tile_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   }
 }
 
+template <bool ALIBI, bool CAUSAL>
+__global__ void __launch_bounds__(TcCfg::threads, TcCfg::ctas_per_sm)
+tile_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+               const __grid_constant__ CUtensorMap map_v, const __grid_constant__ TileParams p, SyncArea* sync) {
+  tile_tc<ALIBI, CAUSAL>(map_q, map_k, map_v, p, sync);
+}
+// One tile of each of several layers (the layers of a stack side by side).
+struct TileBatch { CUtensorMap map[kGroupJobs][3]; TileParams p[kGroupJobs]; };
+template <bool ALIBI>
+__global__ void __launch_bounds__(TcCfg::threads, TcCfg::ctas_per_sm) tile_tc_batch_kernel(const __grid_constant__ TileBatch t, SyncArea* sync) {
+  const int i = blockIdx.z;
+  tile_tc<ALIBI, false>(t.map[i][0], t.map[i][1], t.map[i][2], t.p[i], sync);
+}
+
 // ------------------------------------------------------------------------------------ host
 
 static bool make_map_uncached(CUtensorMap* map, const void* base, int rows, int B, int H, int box_rows) {
@@ -414,6 +427,29 @@ cudaError_t tile_tc_launch(const TileParams& p, int rows_q, int rows_kv, SyncAre
   if (alibi) return go(tile_tc_kernel<true, false>);
   if (causal) return go(tile_tc_kernel<false, true>);
   return go(tile_tc_kernel<false, false>);
+}
+
+// Tiles of n <= kGroupJobs layers (the same B, d, H; slopes in all or none), as many queries each as the first at most.
+cudaError_t tile_tc_batch_launch(const TileParams* p, int n, SyncArea* sync, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  TileBatch t;
+  int nq = 0;
+  for (int i = 0; i < kGroupJobs; ++i) {
+    const TileParams& x = p[i < n ? i : 0];
+    if (!make_map(&t.map[i][0], x.q, x.rows_q, x.B, x.H, kBM) || !make_map(&t.map[i][1], x.k_cache, x.rows_kv, x.B, x.H, kBK) ||
+        !make_map(&t.map[i][2], x.v_cache, x.rows_kv, x.B, x.H, kBK))
+      return cudaErrorInvalidValue;
+    t.p[i] = x;
+    if (x.q1 - x.q0 > nq) nq = x.q1 - x.q0;
+  }
+  const size_t smem = TcCfg::total + 1024;
+  auto go = [&](auto kernel) -> cudaError_t {
+    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), (int)smem);
+    if (e != cudaSuccess) return e;
+    kernel<<<dim3(ceil_div(nq, kBM), p[0].B * p[0].H, n), TcCfg::threads, smem, s>>>(t, sync);
+    return cudaGetLastError();
+  };
+  return p[0].alibi ? go(tile_tc_batch_kernel<true>) : go(tile_tc_batch_kernel<false>);
 }
 
 }  // namespace rt

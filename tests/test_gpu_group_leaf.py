@@ -191,3 +191,39 @@ def test_layers_one_after_the_other_give_the_bits_of_single_layers(L, B, N):
         torch.cuda.synchronize()
         x = z
     assert (x.float().cpu().numpy() == hid).all()
+
+
+# Layers side by side take every sum in the order of the leaf kernel and their earlier pairs in the parts of Algorithm 1's tiles: a long stack is its layers
+# one by one, to the bit.  Lengths that end inside a leaf, slopes in some layers only, six and eight places.
+@pytest.mark.parametrize("L,d,H,B,N,gains", [(8, 512, 8, 2, 1100, True), (6, 768, 12, 9, 1050, False), (2, 1024, 16, 1, 1089, True), (17, 512, 8, 1, 1030, False)])
+def test_long_stacks_give_the_bits_of_single_layers(L, d, H, B, N, gains):
+    import torch
+    from paper_2604_21215_b200 import inputs, rt
+    V = 91
+    data = inputs.make_inputs(inputs.Workload("long", L, B, N, d, H, 4 * d, "bf16", vocab=V, residual_scale=1 / np.sqrt(L)), seed=N)
+    if gains:
+        for i, lw in enumerate(data["layers"]):
+            _gains(lw, d, i)
+    layers = [dict(lw, alibi_slopes=[2.0 ** (-8.0 * (h + 1) / H) for h in range(H)] if gains and i % 3 == 1 else None) for i, lw in enumerate(data["layers"])]
+    kw = dict(dtype="bf16", residual_scale=1 / np.sqrt(L))
+    cfg = rt.make_config(d, H, 4 * d, **kw)
+    assert rt.rt_plan_counters(cfg, B, N, L)["kv_bytes_read"] != L * rt.rt_plan_counters(cfg, B, N, 1)["kv_bytes_read"]      # side by side
+    st = rt.Stack(L, d, H, 4 * d, V, **kw)
+    st.set_weights(layers, data["emb"])
+    st.reserve(B, N)
+    ids = torch.as_tensor(np.asarray(data["ids"]), dtype=torch.int32, device=st.device).contiguous()
+    hid = torch.empty((B, N, d), dtype=torch.bfloat16, device=st.device)
+    st.prefill_device(ids, hid, None)
+    torch.cuda.synchronize()
+    assert st.status() == rt.RT_OK
+    x = st.emb[ids.long()].contiguous()
+    for i, lw in enumerate(layers):
+        layer = rt.Layer(d, H, 4 * d, **kw)
+        layer.set_weights(lw)
+        layer.reserve(B, N)
+        z = torch.empty_like(x)
+        layer.prefill_device(x, z)
+        torch.cuda.synchronize()
+        assert torch.equal(layer.k_cache, st.k_caches[i]) and torch.equal(layer.v_cache, st.v_caches[i]), i
+        x = z
+    assert torch.equal(x, hid)
