@@ -121,9 +121,9 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
   if (!leaf_mma_shape(B, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml)) return none;
   // A leaf meets all earlier pairs at once when its queries exist (they depend on the layer below, so Algorithm 1's tiles cannot
   // run ahead): each leaf reads the layer's whole cache so far, in the parts in which those tiles would have brought it.  The group kernel's sums have the order
-  // of the leaf kernel, so a stack gives the bits of the same layers called one by one, where those take leaves of kWaveBlock positions and widths for which
-  // both deal out the contractions alike; elsewhere long sequences go layer by layer for the sake of these bits.
-  if (N > 1024 && (ml.leaf != kWaveBlock || !leaf_group_same_sums(c->d_model, c->d_ff))) return none;
+  // of the leaf kernel, so a stack gives the bits of the same layers called one by one, where those take leaves of kWaveBlock positions;
+  // elsewhere long sequences go layer by layer for the sake of these bits.
+  if (N > 1024 && ml.leaf != kWaveBlock) return none;
   // How many layers at a time, and by which leaves: the least of launches x (positions x time of a position + what a launch costs besides: pre-passes, tiles, the
   // first weights, us measured as below).  More places fill and drain the pipeline of layers in fewer launches, but a group of fewer SMs streams and multiplies
   // more weights per SM; short leaves fill it sooner, long ones have fewer launches.  8 layers, ms for 4 / 6 / 8 places with leaves of 16, then of 32: d = 1024,
@@ -199,7 +199,7 @@ size_t form_bytes(const rt_config* c, int B, int N, int n_layers) {
   const int d = c->d_model, H = c->n_heads, f = c->d_ff, B16 = B < 16 ? B : 16;
   size_t most = 0;
   auto need = [&](size_t bytes) { if (bytes > most) most = bytes; };
-  need((size_t)g_positions(c, N, n_layers) * 16 * f * 2);
+  need((size_t)g_positions(c, N, n_layers) * leaf_mma_set_bytes(d, f));
   if (N < 2) return most;
   for (int places = 2; places <= kGroupJobs; ++places) {
     if (!leaf_group_shape(1, d, H, f, places, kB200SmemPerCta)) continue;
@@ -230,7 +230,7 @@ WsLayout ws_layout(const rt_config* c, int B, int N, int n_layers) {
   L.ex_part = take((size_t)B * H * kMaxChunks * 68 * 4);
   // exchange buffers of the tensor-core leaf kernel: c, h, z as flag-carrying words (16 sequence slots each),
   // raw k|v as flag-carrying fp32 words; g as packed bf16 in fragment order (16 sequence slots), an array per position of a leaf, in `form`
-  L.ll_bytes = ((size_t)16 * 3 * (d / 2) + (size_t)B * 2 * d) * 8;
+  L.ll_bytes = (size_t)B * 2 * d * 8;
   L.ll = take(L.ll_bytes);
   L.g_arrays = c->dtype == RT_BF16 ? g_positions(c, N, n_layers) : 0;
   L.form = take(form_bytes(c, B, N, n_layers));
@@ -566,12 +566,7 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   const bool use_mma = !small && c->dtype == RT_BF16 && c->sched == RT_SCHED_TILED && pos0 == 0 &&
                        leaf_mma_plan(b_sub, c->d_model, c->n_heads, c->d_ff, c->leaf, &ml);
   LeafMmaBuffers mb;
-  {
-    unsigned long long* w = (unsigned long long*)(ws + L.ll);
-    const size_t bd2 = (size_t)16 * (c->d_model / 2);
-    mb.ll_c = w; mb.ll_h = w + bd2; mb.ll_z = w + 2 * bd2;
-    mb.ll_kv = w + 3 * bd2;
-  }
+  mb.vectors = nullptr; mb.ll_kv = (unsigned long long*)(ws + L.ll);
   auto leaf_mma = [&](int t0, int t1) -> bool {
     ProfScope ps(s, kProfLeaf);
     const size_t e = esize_of(c->dtype);
@@ -581,12 +576,12 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
       lp.z = (unsigned char*)z + (size_t)b0 * z_bs * e;
       lp.t0 = t0; lp.t1 = t1; lp.attn_begin = t0; lp.seq_base = ctx.seq_base;
       // fresh arrays of g for the positions of this launch; filled all at once when they run out
-      const size_t g_bytes = (size_t)16 * c->d_ff * 2;
+      const size_t g_bytes = leaf_mma_set_bytes(c->d_model, c->d_ff);
       if (ctx.g_left < t1 - t0) {
         if (cudaMemsetAsync(ws + L.form, 0xff, L.g_arrays * g_bytes, s) != cudaSuccess) return false;
         ctx.g_left = (int)L.g_arrays;
       }
-      mb.ll_g = (unsigned long long*)(ws + L.form + (L.g_arrays - (size_t)ctx.g_left) * g_bytes);
+      mb.vectors = ws + L.form + (L.g_arrays - (size_t)ctx.g_left) * g_bytes;
       ctx.g_left -= t1 - t0;
       if (leaf_mma_launch(lp, ml, mb, s) != cudaSuccess) return false;
       ctx.seq_base += (unsigned)(t1 - t0);

@@ -52,7 +52,9 @@ cudaError_t wait_expiry_selftest_launch(SyncArea* sync, cudaStream_t s);
 
 // bf16 / tiled-schedule leaf kernel (tensor-core mat-vecs, flag-carrying exchange words).
 struct LeafMmaLaunch { int grid, block; size_t smem; int leaf; int q_smem; };
-struct LeafMmaBuffers { unsigned long long *ll_c, *ll_h, *ll_g, *ll_z, *ll_kv; };   // [16,d/2] words x3, packed bf16 [positions of the leaf][16][dff] filled with ones before the launch, [B,2d] words
+// vectors: c, h, z, g of every position of the launch, packed bf16 [positions][16 (3 d + dff)], filled with ones before; raw k|v as words beside their step number [B,2d]
+struct LeafMmaBuffers { unsigned char* vectors; unsigned long long* ll_kv; };
+inline size_t leaf_mma_set_bytes(int d, int dff) { return (size_t)32 * (3 * (size_t)d + (size_t)((dff + 31) & ~31)); }
 bool leaf_mma_plan(int B, int d, int H, int dff, int want_leaf, LeafMmaLaunch* out);
 // the same decision for a device with `sms` multiprocessors and `max_smem` bytes of shared memory per CTA (no CUDA call)
 bool leaf_mma_shape(int B, int d, int H, int dff, int want_leaf, int sms, size_t max_smem, LeafMmaLaunch* out);
@@ -93,7 +95,6 @@ constexpr int kGroupPackLayers = 8;
 struct GroupPackLayer { const void *w_o, *w_up, *w_down, *w_k, *w_v; void* out; };
 struct GroupPackArgs { int d, dff, g; GroupPackLayer layer[kGroupPackLayers]; };
 bool leaf_group_shape(int B, int d, int H, int dff, int places, size_t max_smem);   // B: sequences of one job; groups of 148 / places SMs
-bool leaf_group_same_sums(int d, int dff);
 float leaf_group_step_us(int B, int d, int dff, int places);                         // estimate of the time per position
 size_t leaf_group_words_bytes(int d, int dff);   // exchange area of one place
 size_t leaf_group_packed_bytes(int d, int dff, int places);

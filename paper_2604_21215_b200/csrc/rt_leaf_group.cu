@@ -102,7 +102,8 @@ __device__ __forceinline__ uint4 ld_two_words(const void* p) {
   return make_uint4((unsigned)a, (unsigned)(a >> 32), (unsigned)b, (unsigned)(b >> 32));
 }
 constexpr unsigned kUnset = 0xffffffffu;
-__device__ __forceinline__ bool unset(const uint4& w) { return (w.x == kUnset) | (w.y == kUnset) | (w.z == kUnset) | (w.w == kUnset); }
+__device__ __forceinline__ unsigned top(const uint4& w) { return max(max(max(w.x, w.y), w.z), w.w); }
+__device__ __forceinline__ bool unset(const uint4& w) { return top(w) == kUnset; }
 // Fetches 16 bytes again while one of their words has not been written.
 __device__ __forceinline__ void ld_unset(const void* p, uint4& w) {
   asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %5, 0;\n @q ld.relaxed.gpu.global.v4.u32 {%0,%1,%2,%3}, [%4];\n}"
@@ -524,12 +525,12 @@ __global__ void __launch_bounds__(kGThreads, 1) leaf_group_kernel(const __grid_c
           unsigned spins = 0;
           unsigned long long t0 = 0;
           while (true) {                                       // (the first round of loads is under way)
-            bool more = false;
+            unsigned most = 0u;
 #pragma unroll
             for (int i = 0; i < kKP; ++i)
 #pragma unroll
-              for (int r = 0; r < MB; ++r) more |= unset(an[i][r]);
-            if (__all_sync(0xffffffffu, !more)) break;
+              for (int r = 0; r < MB; ++r) most = max(most, top(an[i][r]));
+            if (__all_sync(0xffffffffu, most != kUnset)) break;
             if ((++spins & 63u) == 0u && __any_sync(0xffffffffu, group_give_up(sync, s_abort, &t0))) break;
             load(an, base);
           }
@@ -667,12 +668,6 @@ __global__ void __launch_bounds__(kGThreads, 1) leaf_group_kernel(const __grid_c
 
 // SMs of a group; every CTA owns rows of W_down (what the words are set back by: whoever publishes z has read all that came before).
 static int group_size(int d, int places) { const int g = kB200Sms / places; return g < d / 2 ? g : d / 2; }
-
-// Whether a warp's share of the contractions is the one that it has in the tensor-core leaf kernel (which deals out 16 k at a time, this one 32).
-bool leaf_group_same_sums(int d, int dff) {
-  const GroupShape s = group_shape(d, dff, 1);
-  return ceil_div(d / 16, kGMma) == 2 * s.bd && ceil_div(dff / 16, kGMma) == 2 * s.bf;
-}
 
 // Microseconds per position, estimated: the exchanges, and the rounds of four tiles that a warp goes through.  Measured, 4 / 6 / 8 places: d = 1024,
 // B = 16 24.2, -, 40.3 (11 and 22 rounds); d = 768 19.7, 20.1, 27.5 (9, 10, 17); d = 512 15.7, -, 18.5 (6, 9); d = 1024, B = 1 17.6, -, 28.2; d = 512, B = 4 12.7, -, 14.7.

@@ -4,11 +4,10 @@
 // Same decomposition as the generic leaf kernel (one persistent CTA per SM, each CTA owning a
 // fixed slice of the output rows of W_o, W_up, W_down, W_k, W_v in shared memory), but built
 // for latency, because a token step is a chain of five all-to-all exchanges of small vectors:
-//   * exchange words carry their own validity flag.  Every published 64-bit word holds a
-//     payload (two bf16, or one fp32) and the 32-bit sequence number of the token step.
-//     A consumer polls the payload words themselves: one L2 round trip per exchange, no
-//     separate fence + counter + reload.  Flags are unique per step of an API call and the
-//     buffers are zeroed at the start of the call.
+//   * exchange words carry their own validity flag.  Every position of the leaf has its own arrays of c, h, g and z,
+//     packed bf16, filled with ones before the launch, which no pair of results is; raw k|v travel as 64-bit words of an
+//     fp32 and the 32-bit sequence number of the token step (zeroed at the start of the call).  A consumer polls the
+//     payload words themselves: one L2 round trip per exchange, no separate fence + counter + reload.
 //   * the mat-vec products run on the tensor cores as m16n8k16 MMAs with the B sequences as
 //     the M dimension (rows >= B are zero) and 8 weight rows as the N dimension, K split over
 //     the 8 MMA warps of the CTA and reduced through shared memory.  The fragments of the
@@ -60,7 +59,7 @@ LeafMmaLayout leaf_mma_layout(int d, int dff, int grid, int lf, int slots, int q
   L.lf = lf;
   L.q_smem = q_smem;
   size_t o = 64;                                             // abort flag
-  L.off_red = o;   o += sizeof(float4) * kMmaWarps * kNT * 32;
+  L.off_red = o;   o += sizeof(float2) * 2 * kMmaWarps * kNT * 32;
   L.off_ssq = o;   o += sizeof(float) * kMmaWarps * 16;
   L.off_hown = o;  o += align_up(sizeof(float) * 16 * (size_t)L.max_nd, 16);
   L.attn_bytes = align_up((q_smem ? (size_t)lf * kQStride * 2 : 0) + (size_t)lf * kOStride * 4 + (size_t)lf * 8 + 2 * kHeadDim * 4, 16);
@@ -90,28 +89,18 @@ __device__ __forceinline__ uint4 ld_relaxed_v4(const void* p) {
   asm volatile("ld.relaxed.gpu.global.v2.u64 {%0,%1}, [%2];" : "=l"(w0), "=l"(w1) : "l"(p) : "memory");
   return make_uint4((unsigned)w0, (unsigned)(w0 >> 32), (unsigned)w1, (unsigned)(w1 >> 32));
 }
-// The same load under a predicate (no branch): when `on` is zero nothing is read and the result is
-// two zero words (flag 0 never matches a step number).
-__device__ __forceinline__ uint4 ld_relaxed_v4_if(const void* p, unsigned on) {
-  unsigned long long w0 = 0ull, w1 = 0ull;
-  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %3, 0;\n @q ld.relaxed.gpu.global.v2.u64 {%0,%1}, [%2];\n}"
-               : "+l"(w0), "+l"(w1) : "l"(p), "r"(on) : "memory");
-  return make_uint4((unsigned)w0, (unsigned)(w0 >> 32), (unsigned)w1, (unsigned)(w1 >> 32));
-}
 // Words that are their own flags: all ones = not written yet (no pair of bf16 results is: NaN results are 0x7fff).  The load
-// fetches 8 bytes again if one of their words is missing; an asm statement, so that a run of these stays a run of loads (written
+// fetches 16 bytes again if one of their words is missing; an asm statement, so that a run of these stays a run of loads (written
 // as plain loads the compiler placed each one's first use right behind it and the round trips added up).
 constexpr unsigned kNotYet = 0xffffffffu;
-__device__ __forceinline__ bool missing(const uint2& w) { return (w.x == kNotYet) | (w.y == kNotYet); }
-__device__ __forceinline__ void ld_relaxed_v2_missing(const void* p, uint2& w) {
-  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %3, 0;\n @q ld.relaxed.gpu.global.v2.u32 {%0,%1}, [%2];\n}"
-               : "+r"(w.x), "+r"(w.y) : "l"(p), "r"(missing(w) ? 1u : 0u) : "memory");
+// (through the largest of the words: three-input maxima instead of a chain of compares, which many words in a row made hundreds of cycles long)
+__device__ __forceinline__ unsigned top(const uint4& w) { return max(max(max(w.x, w.y), w.z), w.w); }
+__device__ __forceinline__ bool missing(const uint4& w) { return top(w) == kNotYet; }
+__device__ __forceinline__ void ld_relaxed_v4_missing(const void* p, uint4& w) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %5, 0;\n @q ld.relaxed.gpu.global.v4.u32 {%0,%1,%2,%3}, [%4];\n}"
+               : "+r"(w.x), "+r"(w.y), "+r"(w.z), "+r"(w.w) : "l"(p), "r"(missing(w) ? 1u : 0u) : "memory");
 }
 __device__ __forceinline__ void st_relaxed_u32(void* p, unsigned v) { asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory"); }
-__device__ __forceinline__ void st_relaxed_u64(void* p, unsigned lo, unsigned hi) {
-  const unsigned long long w = ((unsigned long long)hi << 32) | lo;
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
-}
 __device__ __forceinline__ void st_relaxed_v4(void* p, unsigned a, unsigned b, unsigned c, unsigned d) {
   const unsigned long long w0 = ((unsigned long long)b << 32) | a, w1 = ((unsigned long long)d << 32) | c;
   asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1,%2};" ::"l"(p), "l"(w0), "l"(w1) : "memory");
@@ -145,12 +134,11 @@ __device__ __forceinline__ bool wait_expired(SyncArea* s, unsigned long long& t_
 }
 
 // What one mat-vec phase works on.  Tiles are groups of 8 weight rows in shared memory.
-// Exchange words of a [B, K] bf16 vector are stored in the order the MMA fragments are read:
-// [k-step of 16][16 sequence slots][4 groups of 4 k][2 words of 2 k], so that one warp-wide
-// 16-byte load (8 sequences x 4 groups) covers 512 contiguous bytes.  Index of the word that
-// holds elements k, k+1 (k even) of sequence b:
-__device__ __forceinline__ size_t ll_word(int b, int k) {
-  return ((size_t)((k >> 4) * 16 + b) * 4 + ((k & 15) >> 2)) * 2 + ((k & 3) >> 1);
+// The vectors c, h, z of a position are packed bf16 in the order the MMA fragments are read: [block of 32 k][16 sequence slots][32 k], a thread's
+// sixteen bytes being its four k of the block's first 16 and its four of the second, so that one warp-wide load (8 sequences x 4 groups)
+// covers 512 contiguous bytes and two k-steps.  Byte offset of elements k, k + 1 (k even) of sequence b:
+__device__ __forceinline__ unsigned vec_off(int b, int k) {
+  return ((unsigned)((k >> 5) * 16 + b) << 6) + (unsigned)(((k & 15) >> 2) * 8 + ((k >> 4) & 1) * 4 + (k & 3)) * 2u;
 }
 
 // Sum of squares (of the raw values) and optional gain for one k-step of fragments; gp points
@@ -175,7 +163,7 @@ __device__ __forceinline__ void frag_ssq_gain(unsigned (&a)[4], const __nv_bfloa
 // QSMEM (compile-time, like the other switches: see the kernel): the leaf's queries are copied to shared memory.
 template <bool TIMERS, bool QSMEM>
 __device__ void attention_role(const LeafParams& p, const LeafMmaLayout& L, unsigned char* smem_slot, int pair,
-                               const unsigned long long* ll_kv, unsigned long long* ll_c) {
+                               const unsigned long long* ll_kv, unsigned char* vectors, size_t set) {
   const int lane = threadIdx.x & 31;
   const int B = p.B, d = p.d, H = p.H;
   const int b = pair / H, h = pair % H;
@@ -211,11 +199,11 @@ __device__ void attention_role(const LeafParams& p, const LeafMmaLayout& L, unsi
   __syncwarp();
   const float gk0 = qkn ? gain_at(g_k, h * kHeadDim + 2 * lane) : 1.0f;
   const float gk1 = qkn ? gain_at(g_k, h * kHeadDim + 2 * lane + 1) : 1.0f;
-  unsigned long long* c_word = ll_c + ll_word(b, h * kHeadDim + 2 * lane);
+  unsigned char* const c_word = vectors + vec_off(b, h * kHeadDim + 2 * lane);      // + `set` per position
   // c of the first position: nothing of this leaf to fold in
   {
     const float il = 1.0f / ls[0];
-    st_relaxed_u64(c_word, pack_bf2(os[2 * lane] * il, os[2 * lane + 1] * il), p.seq_base + 1u);
+    st_relaxed_u32(c_word, pack_bf2(os[2 * lane] * il, os[2 * lane + 1] * il));
   }
   const unsigned long long* k_words = ll_kv + (size_t)b * (2 * d) + h * kHeadDim + 2 * lane;
   const unsigned long long* v_words = k_words + d;
@@ -264,7 +252,7 @@ __device__ void attention_role(const LeafParams& p, const LeafMmaLayout& L, unsi
       const float il = 1.0f / fmaf(l_old, corr, pj);
       const float o0 = fmaf(os[i * kOStride + 2 * lane], corr, pj * vf0);
       const float o1 = fmaf(os[i * kOStride + 2 * lane + 1], corr, pj * vf1);
-      st_relaxed_u64(c_word, pack_bf2(o0 * il, o1 * il), seq + 1u);
+      st_relaxed_u32(c_word + (size_t)i * set, pack_bf2(o0 * il, o1 * il));
     }
     // off the critical path: fold (k_j, v_j) into the later queries of the leaf, one query per lane
     kbuf[2 * lane] = kf0; kbuf[2 * lane + 1] = kf1;
@@ -314,12 +302,10 @@ __device__ void attention_role(const LeafParams& p, const LeafMmaLayout& L, unsi
 // instruction and live register that is compiled in costs time even when its branch is not taken.
 template <int MB, bool TIMERS, bool GAINS, bool QSMEM>
 __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const LeafParams p, const LeafMmaLayout L,
-                                                                      unsigned long long* ll_c, unsigned long long* ll_h,
-                                                                      unsigned long long* ll_g, unsigned long long* ll_z,
-                                                                      unsigned long long* ll_kv) {
+                                                                      unsigned char* vectors, unsigned long long* ll_kv) {
   extern __shared__ __align__(128) unsigned char smem[];
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem);
-  float4* red = reinterpret_cast<float4*>(smem + L.off_red);
+  float2* red = reinterpret_cast<float2*>(smem + L.off_red);        // [eight sequences][warp][tile][lane]: rows 2 c, 2 c + 1 of a tile
   float* ssq_red = reinterpret_cast<float*>(smem + L.off_ssq);
   float* hown = reinterpret_cast<float*>(smem + L.off_hown);
   __nv_bfloat16* s_wo = reinterpret_cast<__nv_bfloat16*>(smem + L.off_wo);
@@ -332,6 +318,8 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
   const int G = gridDim.x, cta = blockIdx.x;
   const int B = p.B, d = p.d, H = p.H, dff = p.dff;
   if (*reinterpret_cast<volatile unsigned*>(&p.sync->abort_flag)) return;
+  const unsigned vec = 32u * (unsigned)d;                     // bytes of c, h or z of a position; its g follows them
+  const size_t set = 3 * (size_t)vec + 32 * (size_t)((dff + 31) & ~31);
   // rows are dealt out in pairs so that a published word (two consecutive rows) has one owner
   const int d_lo = 2 * (int)((long long)(d / 2) * cta / G), d_hi = 2 * (int)((long long)(d / 2) * (cta + 1) / G);
   const int f_lo = 2 * (int)((long long)(dff / 2) * cta / G), f_hi = 2 * (int)((long long)(dff / 2) * (cta + 1) / G);
@@ -365,7 +353,7 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsAttn));
     const int slot = warp - kMmaWarps;
     const int pair = cta + slot * G;
-    if (slot < kAttnSlots && pair < B * H) attention_role<TIMERS, QSMEM>(p, L, smem + L.off_attn + (size_t)slot * L.attn_bytes, pair, ll_kv, ll_c);
+    if (slot < kAttnSlots && pair < B * H) attention_role<TIMERS, QSMEM>(p, L, smem + L.off_attn + (size_t)slot * L.attn_bytes, pair, ll_kv, vectors, set);
     return;
   }
 
@@ -381,11 +369,13 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
   const bool kv_norm = pre && !(p.norm_flags & RT_NORM_SKIP_Z);
   const __nv_bfloat16* x = reinterpret_cast<const __nv_bfloat16*>(p.x);
   __nv_bfloat16* z = reinterpret_cast<__nv_bfloat16*>(p.z);
-  // g as packed bf16 in the order the fragments are read: [k-step of 16][16 sequence slots][16 k], so the
-  // 8 sequences x 32 bytes one warp-wide load touches are 256 contiguous bytes (2 lines instead of 8).  Every position of the leaf has its
-  // own array, filled with the pattern of kNotYet before the launch, so a word is its own flag and nobody waits for a barrier: the release,
-  // the count and the first load behind it were 0.7 us of a token step (9.8 -> 9.1 us at B = 4, d = 768, 13.9 -> 13.2 at B = 16, d = 1024).
-  auto g_index = [](int b, int k) -> size_t { return ((size_t)((k >> 4) * 16 + b) << 4) + (size_t)(k & 15); };
+  // Every position of the leaf has its own arrays of c, h, z and g, filled with the pattern of kNotYet before the launch, so a word is its own flag and nobody
+  // waits for a barrier: for g the release, the count and the first load behind it were 0.7 us of a token step (9.8 -> 9.1 us at B = 4, d = 768, 13.9 -> 13.2
+  // at B = 16, d = 1024); for c, h and z, which had a step number beside every word, half the bytes and a quarter of the loads (9.1 -> 8.5, 13.4 -> 11.6).
+  constexpr int kPlane = kMmaWarps * kNT * 32;
+  // what this thread finishes of a pass: tile u_f, sequence b_f
+  const int u_f = warp % kNT, half_f = warp / kNT, b_f = g + 8 * half_f;
+  const bool has_f = half_f < MB && b_f < B;
   const float inv_d = 1.0f / (float)d;
   const int nt_d = (nd + 7) / 8, nt_f = (nf + 7) / 8;
   const bool has0 = g < B, has1 = (MB == 2) && (g + 8 < B);
@@ -400,7 +390,7 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
 
   for (int t = p.t0; t < p.t1; ++t) {
     const unsigned seq = p.seq_base + (unsigned)(t - p.t0) + 1u;
-    __nv_bfloat16* g_pk = reinterpret_cast<__nv_bfloat16*>(ll_g) + (size_t)(t - p.t0) * 16 * dff;
+    unsigned char* const v_c = vectors + (size_t)(t - p.t0) * set;
 #pragma unroll 1
     for (int ph = 0; ph < 4; ++ph) {                              // 0: W_o   1: W_up   2: W_down   3: W_k | W_v
       // ---- what this phase multiplies ----
@@ -409,7 +399,6 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
       const int nrows = (ph == 1) ? nf : nd;                       // rows per matrix of this phase
       const int nt_one = (ph == 1) ? nt_f : nt_d;
       const int nt_all = (ph == 3) ? 2 * nt_d : nt_one;
-      const unsigned long long* act_ll = (ph == 0) ? ll_c : ((ph == 1) ? ll_h : ll_z);
       const __nv_bfloat16* gain = nullptr;
       bool want_ssq = false;
       if (ph == 1 && pre) { if (GAINS) gain = reinterpret_cast<const __nv_bfloat16*>(p.g_mlp); want_ssq = true; }
@@ -417,23 +406,21 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
       const __nv_bfloat16* gp = (GAINS && gain) ? gain + 4 * c : nullptr;
       unsigned long long wait_ns = 0;
       const int n_ks = K / 16;
-      const int ks_per_warp = (n_ks + kMmaWarps - 1) / kMmaWarps;
+      const int ks_per_warp = 2 * ((n_ks + 2 * kMmaWarps - 1) / (2 * kMmaWarps));      // (whole blocks of 32 k, as in rt_leaf_group.cu)
       const int ks0 = warp * ks_per_warp;
       const int ks1 = ks0 + ks_per_warp < n_ks ? ks0 + ks_per_warp : n_ks;
 
       const int tile_step = (ph == 2) ? 1 : kNT;                   // W_down: one tile per pass (see below)
       for (int t0n = 0; t0n < nt_all; t0n += tile_step) {
         const int n_tiles = nt_all - t0n < tile_step ? nt_all - t0n : tile_step;
-        // rows this thread finishes after the reduction (warp w finishes tile t0n + w)
-        const int ti_e = t0n + warp;
+        // rows this thread finishes after the reduction
+        const int ti_e = t0n + u_f;
         const bool second_e = (ph == 3) && ti_e >= nt_d;
         const int rl = (second_e ? ti_e - nt_d : ti_e) * 8 + 2 * c;
-        const bool mine = warp < n_tiles && rl < nrows;
-        unsigned xw0 = 0, xw1 = 0;
-        if (ph == 0 && mine) {                                     // x_t for the residual, fetched before the wait
-          if (has0) xw0 = *reinterpret_cast<const unsigned*>(x + (size_t)g * p.x_bs + (size_t)(t - p.row_off) * p.x_ts + d_lo + rl);
-          if (has1) xw1 = *reinterpret_cast<const unsigned*>(x + (size_t)(g + 8) * p.x_bs + (size_t)(t - p.row_off) * p.x_ts + d_lo + rl);
-        }
+        const bool mine = has_f && u_f < n_tiles && rl < nrows;
+        unsigned xw = 0;
+        if (ph == 0 && mine)                                       // x_t for the residual, fetched before the wait
+          xw = *reinterpret_cast<const unsigned*>(x + (size_t)b_f * p.x_bs + (size_t)(t - p.row_off) * p.x_ts + d_lo + rl);
 
         // The loops below are written without branches around the loads and the products (indices
         // are clamped, missing sequences and k-steps contribute zeros): a branch per product costs
@@ -453,35 +440,36 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
           // this thread's 8 bytes of weight row g (clamped to the rows that exist) of the tile, at k = 4c
           const int valid = nrows - t0n * 8 < 8 ? nrows - t0n * 8 : 8;
           const unsigned char* wd0 = reinterpret_cast<const unsigned char*>(s_wdn + (size_t)(t0n * 8 + (g < valid ? g : valid - 1)) * stride + 4 * c);
-          const __nv_bfloat16* b0p = g_pk + g_index(g0, 4 * c);          // + 256 elements per k-step
-          const __nv_bfloat16* b1p = g_pk + g_index(g1, 4 * c);
+          const unsigned char* const b0p = v_c + 3 * (size_t)vec + g0 * 64 + 16 * c;      // + 1024 bytes per block of two k-steps
+          const unsigned char* const b1p = b0p + (g1 - g0) * 64;
           for (int kc0 = ks0; kc0 < ks1; kc0 += KD) {
             unsigned ad[KD][4];
             const int n_here = ks1 - kc0;
-            uint2 w0[KD], w1[MB == 2 ? KD : 1];
+            uint4 w0[KD / 2], w1[MB == 2 ? KD / 2 : 1];
 #pragma unroll
-            for (int i = 0; i < KD; ++i) {
-              w0[i].x = w0[i].y = i < n_here ? keep0 : 0u;             // all ones: to be fetched
-              if (MB == 2) w1[i].x = w1[i].y = i < n_here ? keep1 : 0u;
+            for (int i = 0; i < KD / 2; ++i) {
+              const unsigned on0 = 2 * i < n_here ? keep0 : 0u, on1 = 2 * i < n_here ? keep1 : 0u;      // all ones: to be fetched
+              w0[i] = make_uint4(on0, on0, on0, on0);
+              if (MB == 2) w1[i] = make_uint4(on1, on1, on1, on1);
             }
             unsigned spins = 0;
             unsigned long long t_start = 0;
             const unsigned long long t_poll = timing ? globaltimer_ns() : 0ull;
             while (alive) {
 #pragma unroll
-              for (int i = 0; i < KD; ++i) ld_relaxed_v2_missing(b0p + (size_t)(kc0 + (i < n_here ? i : 0)) * 256, w0[i]);
+              for (int i = 0; i < KD / 2; ++i) ld_relaxed_v4_missing(b0p + (size_t)((kc0 >> 1) + i) * 1024, w0[i]);
               if (MB == 2) {
 #pragma unroll
-                for (int i = 0; i < KD; ++i) ld_relaxed_v2_missing(b1p + (size_t)(kc0 + (i < n_here ? i : 0)) * 256, w1[i]);
+                for (int i = 0; i < KD / 2; ++i) ld_relaxed_v4_missing(b1p + (size_t)((kc0 >> 1) + i) * 1024, w1[i]);
               }
-              bool more = false;
+              unsigned most[2] = {0u, 0u};
 #pragma unroll
-              for (int i = 0; i < KD; ++i) more |= missing(w0[i]);
+              for (int i = 0; i < KD / 2; ++i) most[i & 1] = max(most[i & 1], top(w0[i]));
               if (MB == 2) {
 #pragma unroll
-                for (int i = 0; i < KD; ++i) more |= missing(w1[i]);
+                for (int i = 0; i < KD / 2; ++i) most[i & 1] = max(most[i & 1], top(w1[i]));
               }
-              if (__all_sync(0xffffffffu, !more)) break;
+              if (__all_sync(0xffffffffu, max(most[0], most[1]) != kNotYet)) break;
               if ((++spins & 63u) == 0u) {
                 int bad = 0;
                 if (lane == 0) bad = wait_expired(p.sync, t_start) ? 1 : 0;
@@ -490,9 +478,10 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
             }
             if (timing) wait_ns += globaltimer_ns() - t_poll;
 #pragma unroll
-            for (int i = 0; i < KD; ++i) {
-              ad[i][0] = w0[i].x; ad[i][2] = w0[i].y;
-              if (MB == 2) { ad[i][1] = w1[i].x; ad[i][3] = w1[i].y; } else { ad[i][1] = 0u; ad[i][3] = 0u; }
+            for (int i = 0; i < KD / 2; ++i) {
+              ad[2 * i][0] = w0[i].x; ad[2 * i][2] = w0[i].y; ad[2 * i + 1][0] = w0[i].z; ad[2 * i + 1][2] = w0[i].w;
+              if (MB == 2) { ad[2 * i][1] = w1[i].x; ad[2 * i][3] = w1[i].y; ad[2 * i + 1][1] = w1[i].z; ad[2 * i + 1][3] = w1[i].w; }
+              else { ad[2 * i][1] = ad[2 * i][3] = ad[2 * i + 1][1] = ad[2 * i + 1][3] = 0u; }
             }
             const unsigned char* wd = wd0 + (size_t)kc0 * 32;
 #pragma unroll
@@ -501,55 +490,44 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
               mma_bf16(acc[i & 1], ad[i], bw.x, bw.y);
             }
           }
-          red[(warp * kNT) * 32 + lane] = make_float4(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1], acc[0][2] + acc[1][2], acc[0][3] + acc[1][3]);
+          red[(warp * kNT) * 32 + lane] = make_float2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
+          if (MB == 2) red[kPlane + (warp * kNT) * 32 + lane] = make_float2(acc[0][2] + acc[1][2], acc[0][3] + acc[1][3]);
         } else {
         if (ks0 >= ks1) {                                          // a warp without k-steps (narrow layers) contributes zeros
-          for (int nt = 0; nt < n_tiles; ++nt) red[(warp * kNT + nt) * 32 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int nt = 0; nt < n_tiles * MB; ++nt) red[(nt / n_tiles) * kPlane + (warp * kNT + nt % n_tiles) * 32 + lane] = make_float2(0.f, 0.f);
         }
         for (int kc0 = ks0; kc0 < ks1; kc0 += KC) {
           unsigned a[KC][4];
-#pragma unroll
-          for (int i = 0; i < KC; ++i) { a[i][0] = a[i][1] = a[i][2] = a[i][3] = 0u; }
-          const int n_here = ks1 - kc0;                             // k-steps of this round (the rest stay zero)
+          const int n_here = ks1 - kc0;                             // k-steps of this round (the rest stay zero); whole blocks of two
           {
-            // flag-carrying words: a k-step is 8 words per sequence, this thread takes the 2 adjacent ones at 4c
-            const unsigned long long* base0 = act_ll + ll_word(g0, 4 * c) + (size_t)kc0 * 128;   // + 128 words per k-step
-            const unsigned long long* base1 = act_ll + ll_word(g1, 4 * c) + (size_t)kc0 * 128;
-            unsigned need0 = 0, need1 = 0;
+            const unsigned char* base = v_c + (ph == 0 ? 0u : ph == 1 ? vec : 2 * vec) + (size_t)(kc0 >> 1) * 1024 + 16 * c;
+            const unsigned char *const base0 = base + g0 * 64, *const base1 = base + g1 * 64;
+            uint4 w0[KC / 2], w1[MB == 2 ? KC / 2 : 1];
 #pragma unroll
-            for (int i = 0; i < KC; ++i) {
-              if (i < n_here) { need0 |= (1u << i) & keep0; need1 |= (1u << i) & keep1; }
+            for (int i = 0; i < KC / 2; ++i) {
+              const unsigned on0 = 2 * i < n_here ? keep0 : 0u, on1 = 2 * i < n_here ? keep1 : 0u;      // all ones: to be fetched
+              w0[i] = make_uint4(on0, on0, on0, on0);
+              if (MB == 2) w1[i] = make_uint4(on1, on1, on1, on1);
             }
             unsigned spins = 0;
             unsigned long long t_start = 0;
             const unsigned long long t_poll = timing ? globaltimer_ns() : 0ull;
             while (alive) {
-              // every outstanding word of the round is loaded (under a predicate, not a branch) before
-              // any flag is looked at, so the loads overlap
-              uint4 w0[KC], w1[MB == 2 ? KC : 1];
+              // every outstanding word of the round is loaded (under a predicate, not a branch) before any is looked at, so the loads overlap
 #pragma unroll
-              for (int i = 0; i < KC; ++i) w0[i] = ld_relaxed_v4_if(base0 + (size_t)(i < n_here ? i : 0) * 128, (need0 >> i) & 1u);
+              for (int i = 0; i < KC / 2; ++i) ld_relaxed_v4_missing(base0 + i * 1024, w0[i]);
               if (MB == 2) {
 #pragma unroll
-                for (int i = 0; i < KC; ++i) w1[i] = ld_relaxed_v4_if(base1 + (size_t)(i < n_here ? i : 0) * 128, (need1 >> i) & 1u);
+                for (int i = 0; i < KC / 2; ++i) ld_relaxed_v4_missing(base1 + i * 1024, w1[i]);
               }
+              unsigned most[2] = {0u, 0u};
 #pragma unroll
-              for (int i = 0; i < KC; ++i) {
-                const bool okw = (w0[i].y == seq) & (w0[i].w == seq) & ((need0 >> i) & 1u);
-                a[i][0] = okw ? w0[i].x : a[i][0];
-                a[i][2] = okw ? w0[i].z : a[i][2];
-                need0 &= okw ? ~(1u << i) : 0xffffffffu;
-              }
+              for (int i = 0; i < KC / 2; ++i) most[i & 1] = max(most[i & 1], top(w0[i]));
               if (MB == 2) {
 #pragma unroll
-                for (int i = 0; i < KC; ++i) {
-                  const bool okw = (w1[i].y == seq) & (w1[i].w == seq) & ((need1 >> i) & 1u);
-                  a[i][1] = okw ? w1[i].x : a[i][1];
-                  a[i][3] = okw ? w1[i].z : a[i][3];
-                  need1 &= okw ? ~(1u << i) : 0xffffffffu;
-                }
+                for (int i = 0; i < KC / 2; ++i) most[i & 1] = max(most[i & 1], top(w1[i]));
               }
-              if (__all_sync(0xffffffffu, (need0 | need1) == 0u)) break;
+              if (__all_sync(0xffffffffu, max(most[0], most[1]) != kNotYet)) break;
               if ((++spins & 63u) == 0u) {
                 int bad = 0;
                 if (lane == 0) bad = wait_expired(p.sync, t_start) ? 1 : 0;
@@ -557,6 +535,12 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
               }
             }
             if (timing) wait_ns += globaltimer_ns() - t_poll;
+#pragma unroll
+            for (int i = 0; i < KC / 2; ++i) {
+              a[2 * i][0] = w0[i].x; a[2 * i][2] = w0[i].y; a[2 * i + 1][0] = w0[i].z; a[2 * i + 1][2] = w0[i].w;
+              if (MB == 2) { a[2 * i][1] = w1[i].x; a[2 * i][3] = w1[i].y; a[2 * i + 1][1] = w1[i].z; a[2 * i + 1][3] = w1[i].w; }
+              else { a[2 * i][1] = a[2 * i][3] = a[2 * i + 1][1] = a[2 * i + 1][3] = 0u; }
+            }
           }
           const __nv_bfloat16* gc = (GAINS && gp) ? gp + (size_t)kc0 * 16 : nullptr;
           if (want_ssq) {
@@ -581,9 +565,13 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
               const uint2 bw = *reinterpret_cast<const uint2*>(w + (i < n_here ? i : 0) * 32);
               if (i & 1) mma_bf16(co, a[i], bw.x, bw.y); else mma_bf16(ce, a[i], bw.x, bw.y);
             }
-            float4 v = make_float4(ce[0] + co[0], ce[1] + co[1], ce[2] + co[2], ce[3] + co[3]);
-            if (kc0 > ks0) { const float4 o = red[(warp * kNT + nt) * 32 + lane]; v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w; }
-            red[(warp * kNT + nt) * 32 + lane] = v;
+#pragma unroll
+            for (int r = 0; r < MB; ++r) {
+              float2& at = red[r * kPlane + (warp * kNT + nt) * 32 + lane];
+              float2 v = make_float2(ce[2 * r] + co[2 * r], ce[2 * r + 1] + co[2 * r + 1]);
+              if (kc0 > ks0) { v.x += at.x; v.y += at.y; }
+              at = v;
+            }
           }
         }
         }
@@ -595,62 +583,39 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
         }
         mma_warps_sync();
         if (*s_abort) return;
-        float y0 = 0.f, y1 = 0.f, y2 = 0.f, y3 = 0.f, ssq_lo = 0.f, ssq_hi = 0.f;
-        if (warp < n_tiles) {
+        float y0 = 0.f, y1 = 0.f, ssq = 0.f;
+        if (half_f < MB && u_f < n_tiles) {
 #pragma unroll
           for (int w = 0; w < kMmaWarps; ++w) {
-            const float4 v = red[(w * kNT + warp) * 32 + lane];
-            y0 += v.x; y1 += v.y; y2 += v.z; y3 += v.w;
+            const float2 v = red[half_f * kPlane + (w * kNT + u_f) * 32 + lane];
+            y0 += v.x; y1 += v.y;
           }
           if (want_ssq) {
 #pragma unroll
-            for (int w = 0; w < kMmaWarps; ++w) { ssq_lo += ssq_red[w * 16 + g]; ssq_hi += ssq_red[w * 16 + 8 + g]; }
+            for (int w = 0; w < kMmaWarps; ++w) ssq += ssq_red[w * 16 + b_f];
           }
         }
         mma_warps_sync();       // red / ssq_red may be overwritten from here on
-        // ---- epilogue: y0, y1 = rows rl, rl+1 for sequence g; y2, y3 = the same rows for sequence g+8 ----
+        // ---- epilogue: y0, y1 = rows rl, rl+1 for sequence b_f ----
         if (mine) {
-          if (ph == 0) {                                            // h = x_t + alpha W_o c_t
-            if (has0) {
-              const float h0 = bf_lo(xw0) + p.alpha * y0, h1 = bf_hi(xw0) + p.alpha * y1;
-              hown[g * L.max_nd + rl] = h0; hown[g * L.max_nd + rl + 1] = h1;
-              st_relaxed_u64(ll_h + ll_word(g, d_lo + rl), pack_bf2(h0, h1), seq);
+          if (ph == 3) {                                            // raw k_t, v_t from RMS(z_t): Eqs. (1)-(2) before qkRMS
+            const float rs = kv_norm ? rsqrtf(ssq * inv_d + p.eps) : 1.0f;
+            st_relaxed_v4(ll_kv + (size_t)b_f * (2 * d) + (second_e ? d : 0) + d_lo + rl, __float_as_uint(y0 * rs), seq, __float_as_uint(y1 * rs), seq);
+          } else {
+            unsigned word;
+            if (ph == 1) {                                          // g = GELU(W_up RMS(h))
+              const float rs = pre ? rsqrtf(ssq * inv_d + p.eps) : 1.0f;
+              word = pack_bf2(gelu_erf_f(y0 * rs), gelu_erf_f(y1 * rs));
+              if ((dff & 16) && f_lo + rl + 2 == dff)               // the half block that d_ff ends with: zeros
+                for (int k = 0; k < 16; k += 2) st_relaxed_u32(v_c + 3 * vec + vec_off(b_f, dff + k), 0u);
+            } else {                                                // h = x_t + alpha W_o c_t, then z_t = h + alpha W_down g   (layer output)
+              float2& h = *reinterpret_cast<float2*>(hown + b_f * L.max_nd + rl);
+              const float2 v = make_float2((ph == 0 ? bf_lo(xw) : h.x) + p.alpha * y0, (ph == 0 ? bf_hi(xw) : h.y) + p.alpha * y1);
+              word = pack_bf2(v.x, v.y);
+              if (ph == 0) h = v;
+              else *reinterpret_cast<unsigned*>(z + (size_t)b_f * p.z_bs + (size_t)(t - p.row_off) * p.z_ts + d_lo + rl) = word;
             }
-            if (has1) {
-              const float h0 = bf_lo(xw1) + p.alpha * y2, h1 = bf_hi(xw1) + p.alpha * y3;
-              hown[(g + 8) * L.max_nd + rl] = h0; hown[(g + 8) * L.max_nd + rl + 1] = h1;
-              st_relaxed_u64(ll_h + ll_word(g + 8, d_lo + rl), pack_bf2(h0, h1), seq);
-            }
-          } else if (ph == 1) {                                     // g = GELU(W_up RMS(h)), packed bf16
-            if (has0) {
-              const float rs = pre ? rsqrtf(ssq_lo * inv_d + p.eps) : 1.0f;
-              st_relaxed_u32(g_pk + g_index(g, f_lo + rl), pack_bf2(gelu_erf_f(y0 * rs), gelu_erf_f(y1 * rs)));
-            }
-            if (has1) {
-              const float rs = pre ? rsqrtf(ssq_hi * inv_d + p.eps) : 1.0f;
-              st_relaxed_u32(g_pk + g_index(g + 8, f_lo + rl), pack_bf2(gelu_erf_f(y2 * rs), gelu_erf_f(y3 * rs)));
-            }
-          } else if (ph == 2) {                                     // z_t = h + alpha W_down g   (layer output)
-            if (has0) {
-              const unsigned zw = pack_bf2(hown[g * L.max_nd + rl] + p.alpha * y0, hown[g * L.max_nd + rl + 1] + p.alpha * y1);
-              *reinterpret_cast<unsigned*>(z + (size_t)g * p.z_bs + (size_t)(t - p.row_off) * p.z_ts + d_lo + rl) = zw;
-              st_relaxed_u64(ll_z + ll_word(g, d_lo + rl), zw, seq);
-            }
-            if (has1) {
-              const unsigned zw = pack_bf2(hown[(g + 8) * L.max_nd + rl] + p.alpha * y2, hown[(g + 8) * L.max_nd + rl + 1] + p.alpha * y3);
-              *reinterpret_cast<unsigned*>(z + (size_t)(g + 8) * p.z_bs + (size_t)(t - p.row_off) * p.z_ts + d_lo + rl) = zw;
-              st_relaxed_u64(ll_z + ll_word(g + 8, d_lo + rl), zw, seq);
-            }
-          } else {                                                  // raw k_t, v_t from RMS(z_t): Eqs. (1)-(2) before qkRMS
-            const size_t col = (size_t)(second_e ? d : 0) + d_lo + rl;
-            if (has0) {
-              const float rs = kv_norm ? rsqrtf(ssq_lo * inv_d + p.eps) : 1.0f;
-              st_relaxed_v4(ll_kv + (size_t)g * (2 * d) + col, __float_as_uint(y0 * rs), seq, __float_as_uint(y1 * rs), seq);
-            }
-            if (has1) {
-              const float rs = kv_norm ? rsqrtf(ssq_hi * inv_d + p.eps) : 1.0f;
-              st_relaxed_v4(ll_kv + (size_t)(g + 8) * (2 * d) + col, __float_as_uint(y2 * rs), seq, __float_as_uint(y3 * rs), seq);
-            }
+            st_relaxed_u32(v_c + (ph == 0 ? vec : ph == 1 ? 3 * vec : 2 * vec) + vec_off(b_f, (ph == 1 ? f_lo : d_lo) + rl), word);
           }
         }
       }
@@ -714,7 +679,7 @@ cudaError_t leaf_mma_launch(const LeafParams& p, const LeafMmaLaunch& l, const L
   if (e != cudaSuccess) return e;
   LeafParams pp = p;
   LeafMmaBuffers b = buf;
-  void* args[] = {(void*)&pp, (void*)&L, (void*)&b.ll_c, (void*)&b.ll_h, (void*)&b.ll_g, (void*)&b.ll_z, (void*)&b.ll_kv};
+  void* args[] = {(void*)&pp, (void*)&L, (void*)&b.vectors, (void*)&b.ll_kv};
   return cudaLaunchCooperativeKernel(fn, dim3(l.grid), dim3(l.block), args, l.smem, s);
 }
 
