@@ -333,15 +333,22 @@ def run_cuda(args):
         leaf_ms = prof["leaf"]["ms"] / n_leaf
         alg_bytes = (chain_w + act) * tok_steps_per_launch
         achieved = alg_bytes / (leaf_ms * 1e-3) / 1e9 if leaf_ms > 0 else 0.0
-        roofline = {"kernel": ("leaf_mma_kernel" if B <= 16 else "leaf_group_kernel") if (wl.dtype == "bf16" and args.sched == "tiled") else "leaf_kernel", "bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"],
+        # the layers of a stack side by side take the group kernel (its leaves meet all earlier pairs at once, which the counters show)
+        one = rt.rt_plan_counters(model.cfg, wl.B, wl.N, 1, 0)["kv_bytes_read"]
+        side_by_side = wl.n_layers > 1 and counters["kv_bytes_read"] != wl.n_layers * one
+        roofline = {"kernel": ("leaf_mma_kernel" if B <= 16 and not side_by_side else "leaf_group_kernel") if (wl.dtype == "bf16" and args.sched == "tiled") else "leaf_kernel", "bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"],
                     "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"], "peak_source": peaks["source"],
-                    "traffic": leaf_traffic_table().get(wl.name) if B <= 16 and not args.batch else None,
+                    "traffic": leaf_traffic_table().get(wl.name) if B <= 16 and not args.batch and not side_by_side else None,
                     "algorithmic_bytes_per_launch": alg_bytes, "avg_launch_ms": leaf_ms,
                     "us_per_token_step": 1e3 * leaf_ms / max(tok_steps_per_launch, 1),
                     "note": "weights stay in shared memory for a whole launch, so the kernel is bound by the "
                             "latency of its five all-to-all exchanges per token step (L2 round trips), not by HBM; "
                             "the fraction is the effective weight+activation stream against the HBM copy peak and "
                             "traffic is the DRAM bytes ncu counted for one launch"}
+        if side_by_side:
+            roofline["note"] = ("several layers per launch, a group of SMs each, weights streamed from L2: bound by the exchanges of a "
+                                "token step, its products and instruction issue; us_per_token_step is the launch time over all (layer, position) "
+                                "pairs in it; the fraction is the effective weight+activation stream against the HBM copy peak")
         if wl.B > 64:
             # wide batches: the token step is a chain of dense products over the B rows (tcgen05), one position at
             # a time, a leaf of them in one launch; the leaf class of the profile holds them with the in-leaf attention

@@ -740,6 +740,7 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
               }
             }
           }
+          if (!nt) continue;
           ProfScope ps(s, kProfTile);
           if (tile_tc_batch_launch(tiles, nt, gc.sync, s) != cudaSuccess) return RT_ERR_CUDA;
         }

@@ -430,9 +430,8 @@ __global__ void __launch_bounds__(kLeafMmaThreads, 1) leaf_mma_kernel(const Leaf
         const int g0 = has0 ? g : 0, g1 = has1 ? g + 8 : 0;        // rows read by lanes without a sequence (masked below)
         const unsigned keep0 = has0 ? 0xffffffffu : 0u, keep1 = has1 ? 0xffffffffu : 0u;
         if (ph == 2) {
-          // W_down reads g as packed bf16 words that are their own flags, and ALL of this warp's
-          // k-steps are in flight before the first product (at d_ff = 4096: 32 k-steps, 64 loads when B > 8).  One tile per
-          // pass keeps this at 32 products; the two accumulators halve the dependent chain.
+          // W_down: ALL of this warp's k-steps of g are in flight before the first product (at d_ff = 4096: 32 k-steps, 16 loads, 32 when
+          // B > 8).  One tile per pass keeps this at 32 products; the two accumulators halve the dependent chain.
           constexpr int KD = 32;
           float acc[2][4];
 #pragma unroll
