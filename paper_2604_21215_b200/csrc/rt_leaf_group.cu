@@ -21,7 +21,8 @@
 //
 // What bounds a step (37 SMs a group, d = 1024, B = 16: 45 thousand cycles, clock stamps): a fifth each products (an m16n8k16 takes a scheduler 16 cycles) and waiting for
 // words, the rest instructions that run once or a few times per phase: row sums and epilogues 5, partial sums 4, weights not there yet 5, set-up of the phases
-// 7 thousand.  Code size counts: dividing by H in the attention warps and a second copy of their loop (12 KB) cost 5 to 15 %.  Measured against the form before
+// 7 thousand.  Stalls at B = 40, d = 768 (ncu, warps per issue slot): words polled 3.2, fixed latencies 1.9, fences 0.5, instruction fetch 0.4, tensor pipe 0.2.
+// Dividing by H in the attention warps and a second copy of their loop (12 KB of code) cost 5 to 15 %.  Measured against the form before
 // (counter barrier for g, words with their own step number, windows of 16 queries, four places): 8 layers of d = 1024, B = 16, N = 2048 220 (one by one) -> 114 ms;
 // B = 1, N = 77 4.77 -> 4.41; 8 layers of d = 768, B = 16, N = 512 31.9 -> 20.4; one layer, B = 40, d = 768, N = 333 7.0 -> 5.5, B = 64, d = 1024 9.65 -> 7.0.
 // Tried: warps of their own for the row sums (640 threads, 152 registers: slower, 36 against 31 ms for B = 16, N = 512); polling one word before the rest and
