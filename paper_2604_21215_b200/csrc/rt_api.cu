@@ -98,6 +98,11 @@ constexpr int kWaveBand = 16;            // layers whose packed weights the work
 // longest leaf of layers side by side (what the workspace holds rows for)
 int wave_leaf_max(const rt_config* c, int N) { return c->leaf ? c->leaf : N <= 128 ? 16 : N <= 1024 ? 32 : 64; }
 constexpr int kWaveBlock = 64;           // earlier pairs come by whole blocks of this many from the tile kernel, the rest of them inside the leaf kernel
+// First position whose pair a leaf beginning at t0 meets inside the leaf kernel, in fp32; the tile kernel, which rounds its probabilities to bf16, brings
+// those before.  Stacks of up to kWaveFoldN positions keep leaves that begin before kWaveFoldMax out of the tile kernel altogether; longer ones
+// give the bits of the same layers one by one, whose tiles begin with the second block.
+constexpr int kWaveFoldN = 1024, kWaveFoldMax = 192;
+int wave_first_key(int N, int t0) { return N <= kWaveFoldN && t0 < kWaveFoldMax ? 0 : t0 / kWaveBlock * kWaveBlock; }
 // Which leaves of which layers of a stack run together: a leaf is ready when the layer below has finished it and its own layer the one before.  Of
 // the ready ones those with the most leaves still to come after them in a row (of their layer and the layers above) go first, of equal ones the
 // deepest layer: 8 layers of 5 leaves in 4 places take 13 launches, 12 being the least possible, of 64 leaves in 6 places 91 (86).
@@ -706,7 +711,7 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
         j.x = hid[l & 1]; j.x_bs = bs; j.x_ts = (long long)d;
         j.z = l == n_layers - 1 && out ? out : hid[(l + 1) & 1]; j.z_bs = bs; j.z_ts = (long long)d;
         j.k_cache = k_caches[l]; j.v_cache = v_caches[l]; j.t0 = t0; j.t1 = t1; j.B = B; j.b0 = 0;
-        j.key0 = t0 / kWaveBlock * kWaveBlock;
+        j.key0 = wave_first_key(N, t0);
         j.words = ws + L.form + (size_t)i * leaf_group_words_bytes(c->d_model, c->d_ff); j.steps = ctx.group_steps[i];
         ctx.group_steps[i] += (unsigned)(t1 - t0);
       }

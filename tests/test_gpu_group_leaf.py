@@ -227,3 +227,28 @@ def test_long_stacks_give_the_bits_of_single_layers(L, d, H, B, N, gains):
         assert torch.equal(layer.k_cache, st.k_caches[i]) and torch.equal(layer.v_cache, st.v_caches[i]), i
         x = z
     assert torch.equal(x, hid)
+
+
+# Up to 1024 positions, leaves that begin before position 192 meet all earlier pairs in the leaf kernel, whose probabilities are fp32: no tile is launched
+# (the tile kernel rounds them to bf16).  The leaf that begins at 192 or later takes one for each power of two of its 64-blocks, at most.
+@pytest.mark.parametrize("L,d,H,B,N,tiles", [(8, 512, 8, 1, 77, False), (8, 1024, 16, 1, 190, False), (4, 768, 12, 9, 192, False), (8, 512, 8, 2, 230, True)])
+def test_probabilities_of_the_first_leaves_stay_fp32(L, d, H, B, N, tiles):
+    import torch
+    from paper_2604_21215_b200 import inputs, rt
+    V = 91
+    data = inputs.make_inputs(inputs.Workload("first", L, B, N, d, H, 4 * d, "bf16", vocab=V, residual_scale=1 / np.sqrt(L)), seed=N)
+    st = rt.Stack(L, d, H, 4 * d, V, dtype="bf16", residual_scale=1 / np.sqrt(L))
+    assert rt.rt_plan_counters(st.cfg, B, N, L)["kv_bytes_read"] != L * rt.rt_plan_counters(st.cfg, B, N, 1)["kv_bytes_read"]      # side by side
+    st.set_weights(data["layers"], data["emb"])
+    st.reserve(B, N)
+    ids = torch.as_tensor(data["ids"], dtype=torch.int32, device=st.device).contiguous()
+    rt.rt_profile_read()
+    rt.rt_profile_enable(True)
+    try:
+        st.prefill_device(ids, None, None)
+        torch.cuda.synchronize()
+        launches = rt.rt_profile_read()["tile"]["launches"]
+    finally:
+        rt.rt_profile_enable(False)
+    assert st.status() == rt.RT_OK
+    assert (launches > 0) == tiles, launches
