@@ -150,17 +150,24 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
   }
   if (!places) return none;
   // Side by side a position costs a layer more (fewer SMs, weights from L2), so enough layers have to be at work at the same time: on average
-  // n_layers * N / (waves * leaf) of them.  Break even was measured at 1.3 to 2.3, growing with the weights that the groups stream (places x MB
+  // n_layers * N / (launches * leaf) of them.  Break even was measured at 1.3 to 2.3, growing with the weights that the groups stream (places x MB
   // per layer) and above four sequences: 8 layers of d = 1024, B = 1, take 1.69 times as long as one after the other for 16 positions (one layer at a
-  // time), 1.05 for 32, 0.84 for 48, 0.72 for 77; B = 16 1.98, 1.20, 0.95 and for 64 0.83; 2 layers 1.33, 1.09, 1.03 and for 128 0.97.  Layers
-  // that fit a cluster (rt_leaf_small.cu) are faster alone than the tensor-core leaf kernel, taken as 8.3 us a position, above eight sequences 10.5; it
-  // takes as many more.  Over 2 to 8 layers, d = 128 to 1024, 1 to 16 sequences and 16 to 400 positions the side taken is at most about a tenth slower than the other.
-  const float at_work = (float)band * (float)N / ((float)launches * (float)leaf), mma_us = B > 8 ? 10.5f : 8.3f;
+  // time), 1.05 for 32, 0.84 for 48, 0.72 for 77; B = 16 1.98, 1.20, 0.95 and for 64 0.83; 2 layers 1.33, 1.09, 1.03 and for 128 0.97.
+  auto even = [&](int pl) { return 1.26f + 0.008f * (float)pl * layer_mb + (B > 4 ? 0.15f : 0.0f); };
   LeafSmallLaunch sl;
-  const bool small = leaf_small_shape(c->dtype, B, c->d_model, c->n_heads, c->d_ff, ml.leaf, kB200SmemPerCta, &sl);
-  if (small && N > 1024) return none;                          // (the bits of that kernel)
-  const float even = (1.26f + 0.008f * places * layer_mb + (B > 4 ? 0.15f : 0.0f)) * (small && sl.step_us < mma_us ? mma_us / sl.step_us : 1.0f);
-  return at_work > even ? Wave{places, leaf} : none;
+  if (leaf_small_shape(c->dtype, B, c->d_model, c->n_heads, c->d_ff, ml.leaf, kB200SmemPerCta, &sl)) {
+    // Layers that fit a cluster (rt_leaf_small.cu) hold the values between the phases in fp32 there, in bf16 here (8 layers of d = 128, B = 1, N = 200: error
+    // of the last k against 64 bits 4.95e-3 and 5.2e-3; 2 layers of d = 384 2.97e-3 and 3.3e-3).  So more than four places are no reason to take them
+    // off it: they go side by side only where four, each layer in the place of the one four before it, pay against that kernel, which is faster than the
+    // tensor-core leaf kernel (taken as 8.3 us a position, above eight sequences 10.5): as many more layers have to be at work.
+    if (N > kWaveFoldN) return none;                           // (the bits of that kernel)
+    const int four = n_layers < 4 ? n_layers : 4, lf = c->leaf ? c->leaf : N <= 128 ? 16 : 32, n = ceil_div(N, lf), turn = n > four ? n : four;
+    const float mma_us = B > 8 ? 10.5f : 8.3f, faster = sl.step_us < mma_us ? mma_us / sl.step_us : 1.0f;
+    const float at_work = (float)n_layers * (float)N / (float)(((n_layers - 1) / four * turn + (n_layers - 1) % four + n) * lf);
+    return leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, four, kB200SmemPerCta) && at_work > even(four) * faster ? Wave{places, leaf} : none;
+  }
+  const float at_work = (float)band * (float)N / ((float)launches * (float)leaf);
+  return at_work > even(places) ? Wave{places, leaf} : none;
 }
 struct WaveRows { size_t n, q, kt, vt, st_o, st_m, st_l, total; };
 WaveRows wave_rows_layout(const rt_config* c, int B, int leaf) {

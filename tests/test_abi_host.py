@@ -176,3 +176,6 @@ def test_layers_run_side_by_side_where_enough_of_them_are_at_work():
             assert side_by_side(d, B, 77, 8) and side_by_side(d, B, 128, 4) and side_by_side(d, B, 1024, 8), (d, B)
             assert not side_by_side(d, B, 24, 8) and not side_by_side(d, B, 32, 2), (d, B)
     assert not side_by_side(128, 1, 64, 8) and side_by_side(384, 4, 64, 8) and side_by_side(256, 16, 200, 8)
+    # layers of the cluster kernel, which holds their values between the phases in fp32, are not taken off it because more than four fit side by side
+    for d, B, N, L in ((64, 4, 400, 4), (128, 1, 77, 8), (128, 1, 200, 8), (128, 8, 256, 3), (256, 1, 256, 3), (256, 8, 48, 4), (384, 1, 200, 2), (192, 1, 200, 4)):
+        assert not side_by_side(d, B, N, L), (d, B, N, L)

@@ -193,6 +193,27 @@ def test_layers_one_after_the_other_give_the_bits_of_single_layers(L, B, N):
     assert (x.float().cpu().numpy() == hid).all()
 
 
+# ... and so do layers that fit the cluster kernel, whose values between the phases are fp32, wherever four of them side by side do not pay
+@pytest.mark.parametrize("L,d,B,N", [(8, 128, 1, 77), (8, 128, 1, 200), (4, 256, 8, 48), (2, 384, 1, 200)])
+def test_stacks_of_small_layers_give_the_bits_of_single_layers(L, d, B, N):
+    import torch
+    from paper_2604_21215_b200 import inputs, rt
+    V = 91
+    data = inputs.make_inputs(inputs.Workload("small", L, B, N, d, d // 64, 4 * d, "bf16", vocab=V, residual_scale=1 / np.sqrt(L)), seed=N)
+    kw = dict(dtype="bf16", residual_scale=1 / np.sqrt(L))
+    st = rt.Stack(L, d, d // 64, 4 * d, V, **kw)
+    st.set_weights(data["layers"], data["emb"])
+    hid, _ = st.prefill(data["ids"])
+    x = st.emb[torch.as_tensor(np.asarray(data["ids"]), dtype=torch.int64, device="cuda")].double().cpu().numpy()
+    for i, lw in enumerate(data["layers"]):
+        layer = rt.Layer(d, d // 64, 4 * d, **kw)
+        layer.set_weights(lw)
+        x, k, v = layer.prefill(x)
+        got = st.caches_numpy(N)[i]
+        assert np.array_equal(got[0], k) and np.array_equal(got[1], v), i
+    assert np.array_equal(hid, x)
+
+
 # Layers side by side take every sum in the order of the leaf kernel and their earlier pairs in the parts of Algorithm 1's tiles: a long stack is its layers
 # one by one, to the bit.  Lengths that end inside a leaf, slopes in some layers only, six and eight places.
 @pytest.mark.parametrize("L,d,H,B,N,gains", [(8, 512, 8, 2, 1100, True), (6, 768, 12, 9, 1050, False), (2, 1024, 16, 1, 1089, True), (17, 512, 8, 1, 1030, False)])
