@@ -98,11 +98,11 @@ constexpr int kWaveBand = 16;            // layers whose packed weights the work
 // longest leaf of layers side by side (what the workspace holds rows for)
 int wave_leaf_max(const rt_config* c, int N) { return c->leaf ? c->leaf : N <= 128 ? 16 : N <= 1024 ? 32 : 64; }
 constexpr int kWaveBlock = 64;           // earlier pairs come by whole blocks of this many from the tile kernel, the rest of them inside the leaf kernel
-// First position whose pair a leaf beginning at t0 meets inside the leaf kernel, in fp32; the tile kernel, which rounds its probabilities to bf16, brings
-// those before.  Stacks of up to kWaveFoldN positions keep leaves that begin before kWaveFoldMax out of the tile kernel altogether; longer ones
-// give the bits of the same layers one by one, whose tiles begin with the second block.
-constexpr int kWaveFoldN = 1024, kWaveFoldMax = 192;
-int wave_first_key(int N, int t0) { return N <= kWaveFoldN && t0 < kWaveFoldMax ? 0 : t0 / kWaveBlock * kWaveBlock; }
+// The whole blocks of 64 pairs before a leaf that begins at t0 come from the fp32 tile kernel, not from the tensor-core one, which rounds its
+// probabilities to bf16: in stacks of up to kWaveExactN positions, for leaves that begin before kWaveExactMax.  Longer stacks give the bits of the
+// same layers one by one, whose tiles begin with the second block.
+constexpr int kWaveExactN = 1024, kWaveExactMax = 192;
+bool wave_exact_tile(int N, int t0) { return N <= kWaveExactN && t0 < kWaveExactMax; }
 // Which leaves of which layers of a stack run together: a leaf is ready when the layer below has finished it and its own layer the one before.  Of
 // the ready ones those with the most leaves still to come after them in a row (of their layer and the layers above) go first, of equal ones the
 // deepest layer: 8 layers of 5 leaves in 4 places take 13 launches, 12 being the least possible, of 64 leaves in 6 places 91 (86).
@@ -160,7 +160,7 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
     // of the last k against 64 bits 4.95e-3 and 5.2e-3; 2 layers of d = 384 2.97e-3 and 3.3e-3).  So more than four places are no reason to take them
     // off it: they go side by side only where four, each layer in the place of the one four before it, pay against that kernel, which is faster than the
     // tensor-core leaf kernel (taken as 8.3 us a position, above eight sequences 10.5): as many more layers have to be at work.
-    if (N > kWaveFoldN) return none;                           // (the bits of that kernel)
+    if (N > kWaveExactN) return none;                           // (the bits of that kernel)
     const int four = n_layers < 4 ? n_layers : 4, lf = c->leaf ? c->leaf : N <= 128 ? 16 : 32, n = ceil_div(N, lf), turn = n > four ? n : four;
     const float mma_us = B > 8 ? 10.5f : 8.3f, faster = sl.step_us < mma_us ? mma_us / sl.step_us : 1.0f;
     const float at_work = (float)n_layers * (float)N / (float)(((n_layers - 1) / four * turn + (n_layers - 1) % four + n) * lf);
@@ -718,7 +718,7 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
         j.x = hid[l & 1]; j.x_bs = bs; j.x_ts = (long long)d;
         j.z = l == n_layers - 1 && out ? out : hid[(l + 1) & 1]; j.z_bs = bs; j.z_ts = (long long)d;
         j.k_cache = k_caches[l]; j.v_cache = v_caches[l]; j.t0 = t0; j.t1 = t1; j.B = B; j.b0 = 0;
-        j.key0 = wave_first_key(N, t0);
+        j.key0 = t0 / kWaveBlock * kWaveBlock;
         j.words = ws + L.form + (size_t)i * leaf_group_words_bytes(c->d_model, c->d_ff); j.steps = ctx.group_steps[i];
         ctx.group_steps[i] += (unsigned)(t1 - t0);
       }
@@ -726,15 +726,34 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
         ProfScope ps(s, kProfPrepass);
         if (prepass_batch_launch(c->dtype, pre, nj, s) != cudaSuccess) return RT_ERR_CUDA;
       }
-      // The leaf's queries against the whole blocks of kWaveBlock earlier pairs, in the parts in which Algorithm 1's tiles would have brought them
-      // (the powers of two that the number of blocks consists of, largest first): the same states to the bit.  The kernel absorbs the rest.
+      // The leaf's queries against the whole blocks of kWaveBlock earlier pairs; the kernel absorbs the rest.
+      TileParams tiles[kGroupJobs];
+      auto tile_of = [&](int i, int k0, int k1) {
+        TileParams tp;
+        memset(&tp, 0, sizeof(tp));
+        tp.B = B; tp.d = c->d_model; tp.H = c->n_heads; tp.scale_log2 = gc.scale_log2; tp.alibi = jobs[i].alibi;
+        tp.q = pre[i].q; tp.k_cache = jobs[i].k_cache; tp.v_cache = jobs[i].v_cache; tp.st_o = pre[i].st_o; tp.st_m = pre[i].st_m; tp.st_l = pre[i].st_l;
+        tp.rows_q = pre[i].N; tp.rows_kv = N_max; tp.sync = gc.sync; tp.q_pos0 = jobs[i].t0;
+        tp.q0 = 0; tp.q1 = pre[i].N; tp.k0 = k0; tp.k1 = k1;
+        return tp;
+      };
+      {
+        int nt = 0;
+        for (int i = 0; i < nj; ++i)
+          if (jobs[i].key0 && wave_exact_tile(N, jobs[i].t0)) tiles[nt++] = tile_of(i, 0, jobs[i].key0);
+        if (nt) {
+          ProfScope ps(s, kProfTile);
+          if (tile_simt_batch_launch(tiles, nt, s) != cudaSuccess) return RT_ERR_CUDA;
+        }
+      }
+      // On tensor cores they come in the parts in which Algorithm 1's tiles would have brought them (the powers of two that the number of blocks
+      // consists of, largest first): the same states to the bit.
       for (int part = 0, more = 1; more; ++part) {
         more = 0;
         for (int sloped = 0; sloped < 2; ++sloped) {
-          TileParams tiles[kGroupJobs];
           int nt = 0;
           for (int i = 0; i < nj; ++i) {
-            int blocks = jobs[i].key0 / kWaveBlock, k0 = 0, size = 0;
+            int blocks = wave_exact_tile(N, jobs[i].t0) ? 0 : jobs[i].key0 / kWaveBlock, k0 = 0, size = 0;
             for (int skip = 0; blocks && skip <= part; ++skip) {
               k0 += size;
               size = 1;
@@ -743,12 +762,7 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
               if (skip == part) {
                 more |= blocks > 0;
                 if ((jobs[i].alibi != nullptr) != (sloped != 0)) break;
-                TileParams& tp = tiles[nt++];
-                memset(&tp, 0, sizeof(tp));
-                tp.B = B; tp.d = c->d_model; tp.H = c->n_heads; tp.scale_log2 = gc.scale_log2; tp.alibi = jobs[i].alibi;
-                tp.q = pre[i].q; tp.k_cache = jobs[i].k_cache; tp.v_cache = jobs[i].v_cache; tp.st_o = pre[i].st_o; tp.st_m = pre[i].st_m; tp.st_l = pre[i].st_l;
-                tp.rows_q = pre[i].N; tp.rows_kv = N_max; tp.sync = gc.sync; tp.q_pos0 = jobs[i].t0;
-                tp.q0 = 0; tp.q1 = pre[i].N; tp.k0 = k0 * kWaveBlock; tp.k1 = (k0 + size) * kWaveBlock;
+                tiles[nt++] = tile_of(i, k0 * kWaveBlock, (k0 + size) * kWaveBlock);
               }
             }
           }

@@ -162,7 +162,7 @@ struct TileParams {
                                                  // launch over [q0,q1) x [k0,k1) covers every query's whole causal prefix; heavy tiles first
   int chained;                                   // row_attn only: launch as a programmatic dependent launch
   void* c_out;                                   // row_attn only: also write the attention value o/l of the row, [B, d] storage type
-  int q_pos0;                                    // position of query row 0 (ALiBi distances; tensor-core kernel without a mask only)
+  int q_pos0;                                    // position of query row 0 (ALiBi distances; kernels without a mask only)
   int rows_q, rows_kv;                           // rows held by the query buffer / the caches (tensor-map bounds)
   SyncArea* sync;
 };
@@ -172,6 +172,8 @@ cudaError_t tile_tc_launch(const TileParams& p, int rows_q, int rows_kv, SyncAre
 // one tile of each of n layers (n <= kGroupJobs, key counts multiples of 64, the same B, d, H; slopes in all or none)
 cudaError_t tile_tc_batch_launch(const TileParams* p, int n, SyncArea* sync, cudaStream_t s);
 cudaError_t tile_simt_launch(int dtype, const TileParams& p, cudaStream_t s);
+// bf16 tiles of n layers (1 <= n <= kGroupJobs, the same B, d, H), probabilities in fp32
+cudaError_t tile_simt_batch_launch(const TileParams* p, int n, cudaStream_t s);
 // one query row (position q0) per (sequence, head) against the pairs [k0, k1): the in-leaf step of wide batches
 cudaError_t row_attn_launch(int dtype, const TileParams& p, cudaStream_t s);
 

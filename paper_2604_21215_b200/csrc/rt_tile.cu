@@ -11,7 +11,7 @@ constexpr int kTQ = 16;    // query rows per CTA
 constexpr int kTK = 32;    // keys per shared-memory chunk
 
 template <typename T>
-__global__ void __launch_bounds__(128) tile_simt_kernel(const TileParams p) {
+__device__ __forceinline__ void tile_simt(const TileParams& p) {
   __shared__ float Qs[kTQ][kHeadDim];
   __shared__ float Ks[kTK][kHeadDim + 1];
   __shared__ float Vs[kTK][kHeadDim];
@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(128) tile_simt_kernel(const TileParams p) {
       float s = 0.f;
 #pragma unroll 16
       for (int e = 0; e < kHeadDim; ++e) s += Qs[qr][e] * Ks[lane][e];
-      const float s2 = valid ? s * p.scale_log2 - slope_l2 * (float)(qb + qr - (kb + lane)) : -INFINITY;
+      const float s2 = valid ? s * p.scale_log2 - slope_l2 * (float)(p.q_pos0 + qb + qr - (kb + lane)) : -INFINITY;
       const float m_new = fmaxf(m[i], warp_max(s2));
       const float pj = valid ? exp2f(s2 - m_new) : 0.f;
       const float corr = exp2f(m[i] - m_new);
@@ -91,6 +91,24 @@ __global__ void __launch_bounds__(128) tile_simt_kernel(const TileParams p) {
       p.st_o[sidx * p.d + h * kHeadDim + lane + 32] = ob[i];
     }
   }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(128) tile_simt_kernel(const TileParams p) { tile_simt<T>(p); }
+
+// One tile of each of several layers (the layers of a stack side by side); blockIdx.z is the layer, batch_stride 0.
+struct TileSimtBatch { TileParams p[kGroupJobs]; };
+__global__ void __launch_bounds__(128) tile_simt_batch_kernel(const __grid_constant__ TileSimtBatch t) { tile_simt<__nv_bfloat16>(t.p[blockIdx.z]); }
+
+cudaError_t tile_simt_batch_launch(const TileParams* p, int n, cudaStream_t s) {
+  TileSimtBatch t;
+  int nq = 0;
+  for (int i = 0; i < kGroupJobs; ++i) {
+    t.p[i] = p[i < n ? i : 0];
+    if (t.p[i].q1 - t.p[i].q0 > nq) nq = t.p[i].q1 - t.p[i].q0;
+  }
+  tile_simt_batch_kernel<<<dim3(ceil_div(nq, kTQ), p[0].B * p[0].H, n), 128, 0, s>>>(t);
+  return cudaGetLastError();
 }
 
 cudaError_t tile_simt_launch(int dtype, const TileParams& p, cudaStream_t s) {
