@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "rt_kernels.h"
+#include "rt_wave.h"
 
 using namespace rt;
 
@@ -94,7 +95,6 @@ Schedule effective_schedule(const rt_config* c, int B, int N) {
 // The layers of a stack side by side (rt_leaf_group.cu): layer l works on a leaf that layer l-1 finished in an earlier
 // launch, up to `places` layers in a launch, a group of SMs each.  places = 0: one layer after the other.
 struct Wave { int places, leaf; };
-constexpr int kWaveBand = 16;            // layers whose packed weights the workspace holds at a time
 // longest leaf of layers side by side (what the workspace holds rows for)
 int wave_leaf_max(const rt_config* c, int N) { return c->leaf ? c->leaf : N <= 128 ? 16 : N <= 1024 ? 32 : 64; }
 constexpr int kWaveBlock = 64;           // earlier pairs come by whole blocks of this many from the tile kernel, the rest of them inside the leaf kernel
@@ -103,22 +103,6 @@ constexpr int kWaveBlock = 64;           // earlier pairs come by whole blocks o
 // same layers one by one, whose tiles begin with the second block.
 constexpr int kWaveExactN = 1024, kWaveExactMax = 192;
 bool wave_exact_tile(int N, int t0) { return N <= kWaveExactN && t0 < kWaveExactMax; }
-// Which leaves of which layers of a stack run together: a leaf is ready when the layer below has finished it and its own layer the one before.  Of
-// the ready ones those with the most leaves still to come after them in a row (of their layer and the layers above) go first, of equal ones the
-// deepest layer: 8 layers of 5 leaves in 4 places take 13 launches, 12 being the least possible, of 64 leaves in 6 places 91 (86).
-struct WaveOrder {
-  int n_layers, n_leaves, done[kWaveBand];
-  WaveOrder(int layers, int leaves) : n_layers(layers), n_leaves(leaves), done{} {}
-  // The next launch: up to `places` (layer, leaf) pairs; 0 when all leaves are done.
-  int next(int places, int* layer, int* leaf) {
-    int n = 0;
-    for (int sum = 0; sum <= n_layers + n_leaves && n < places; ++sum)       // layer + leaf: the smaller, the more is to come
-      for (int l = n_layers - 1; l >= 0 && n < places; --l)
-        if (done[l] < n_leaves && l + done[l] == sum && (l == 0 || done[l - 1] > done[l])) { layer[n] = l; leaf[n++] = done[l]; }
-    for (int i = 0; i < n; ++i) ++done[layer[i]];
-    return n;
-  }
-};
 Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
   const Wave none = {0, 0};
   if (n_layers < 2 || N < 2 || c->dtype != RT_BF16 || c->sched != RT_SCHED_TILED || c->recur_block > 1) return none;
@@ -135,15 +119,14 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
   // B = 16, N = 512 31.4 32.7 35.1, 30.0 32.5 35.6; d = 768 25.3 21.6 23.8, 24.3 21.1 24.2; d = 512 20.5 16.3 15.5, 19.5 16.6 16.0; d = 1024, B = 1 22.9 22.7 21.3, 21.8 23.6 22.9.
   const float layer_mb = (3.0f * c->d_model + 2.0f * c->d_ff) * c->d_model * 2e-6f;
   const int band = n_layers < kWaveBand ? n_layers : kWaveBand;
-  int places = 0, leaf = 0, launches = 0;
+  int places = 0, leaf = 0;
+  long long launches = 0;
   float least = 0.0f;
   for (int pl = 2; pl <= kGroupJobs && pl <= n_layers; ++pl) {
     if (!leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, pl, kB200SmemPerCta)) continue;
     const float step = leaf_group_step_us(B, c->d_model, c->d_ff, pl);
     for (int lf = c->leaf ? c->leaf : 16; lf <= wave_leaf_max(c, N); lf *= 2) {
-      WaveOrder order(band, ceil_div(N, lf));
-      int n = 0, layer_of[kGroupJobs], leaf_of[kGroupJobs];
-      while (order.next(pl, layer_of, leaf_of) > 0) ++n;
+      const long long n = wave_launches(band, ceil_div(N, lf), pl);
       const float us = (float)n * ((float)lf * step + (B > 8 ? 20.0f + 1.35f * layer_mb * (float)pl : 33.0f + 0.35f * layer_mb * (float)pl));
       if (!places || us < least) { places = pl; leaf = lf; launches = n; least = us; }
     }
