@@ -103,6 +103,30 @@ constexpr int kWaveBlock = 64;           // earlier pairs come by whole blocks o
 // same layers one by one, whose tiles begin with the second block.
 constexpr int kWaveExactN = 1024, kWaveExactMax = 192;
 bool wave_exact_tile(int N, int t0) { return N <= kWaveExactN && t0 < kWaveExactMax; }
+// Estimates (us) of a stack's token loops, side by side and one after the other.  Fitted to 16 widths from d = 64 to 1024, 1 to 16 sequences, 2 to 8 places and leaves of
+// 16, 32 and 64 (256 positions; 5 % off on average from d = 320 on) and checked on long stacks, ms measured / estimated, side by side and one after the other: 8 layers of d = 1024,
+// B = 1, N = 2048 82.6 / 75, 139 / 145, 16384 743 / 651, 1116 / 1161, 65536 3651 / 3519, 4480 / 4704; B = 16, N = 2048 111 / 101, 190 / 192, 16384 1146 / 1040, 1601 / 1606, 65536
+// 7596 / 7570, 7472 / 7391; d = 512, B = 16, N = 32768 1149 / 1175, 2785 / 2853; 2 layers of d = 1024, B = 16, N = 16384 372 / 402, 401 / 402, 32768 861 / 947, 845 / 843.
+// Tiles are what grows with the length: a leaf reads its layer's whole cache so far, so side by side they cost (N / 64)^2 / 2 blocks of 64 pairs x 64 queries a layer and (sequence,
+// head), 1.15 us each behind one another or 4.2 ns where they fill the chip; the same pairs cost 1.2 ns in Algorithm 1's larger tiles.  So one after the other, whose
+// cache traffic is N log N, is the faster form again from some length on: some 65 thousand positions for 8 layers of d = 1024, B = 16, some 20 thousand for 2.
+// Widths that are no multiple of 128 take the fp32 pre-pass, whose time per launch of leaves is 0.05 d us a layer and more.
+bool tensor_prepass(const rt_config* c) { return c->d_model % 128 == 0; }
+float wave_us(const rt_config* c, int B, int N, int n_layers, int places, int leaf) {
+  const float d = (float)c->d_model, tiles = (float)(places * B * c->n_heads), blocks = (float)N / (float)kWaveBlock;
+  long long launches = 0;
+  for (int l0 = 0; l0 < n_layers; l0 += kWaveBand) launches += wave_launches(n_layers - l0 < kWaveBand ? n_layers - l0 : kWaveBand, ceil_div(N, leaf), places);
+  float us = (float)leaf * leaf_group_step_us(B, c->d_model, c->d_ff, places) + 21.0f + 3.5e-4f * (float)(places * B) * d;
+  if (!tensor_prepass(c)) us += (float)places * d * (0.048f + 4.2e-7f * (float)B * d);
+  // of the whole blocks that come before a leaf, on average half: a launch for each power of two that their number consists of
+  if (blocks > 1.0f) us += (1.0f - 1.0f / blocks) * ((0.5f * log2f(blocks) + 0.9f) * (9.0f + 0.01f * tiles) + 0.5f * blocks * fmaxf(1.15f, 4.2e-3f * tiles));
+  return (float)launches * us;
+}
+float alone_us(const rt_config* c, int B, int N, int n_layers) {
+  const float d = (float)c->d_model, blocks = (float)N / (float)kWaveBlock;
+  const float step = 7.4f + 1.3e-3f * d + 8.6e-5f * (float)B * d + (B > 8 ? 1.5f : 0.0f) + (tensor_prepass(c) ? 0.0f : 2.0e-7f * (float)B * d * d);
+  return (float)n_layers * ((float)N * step + 0.6e-3f * (float)(B * c->n_heads) * blocks * blocks);
+}
 Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
   const Wave none = {0, 0};
   if (n_layers < 2 || N < 2 || c->dtype != RT_BF16 || c->sched != RT_SCHED_TILED || c->recur_block > 1) return none;
@@ -112,45 +136,42 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
   // run ahead): each leaf reads the layer's whole cache so far, in the parts in which those tiles would have brought it.  The group kernel's sums have the order
   // of the leaf kernel, so a stack gives the bits of the same layers called one by one, where those take leaves of kWaveBlock positions;
   // elsewhere long sequences go layer by layer for the sake of these bits.
-  if (N > 1024 && ml.leaf != kWaveBlock) return none;
-  // How many layers at a time, and by which leaves: the least of launches x (positions x time of a position + what a launch costs besides: pre-passes, tiles, the
-  // first weights, us measured as below).  More places fill and drain the pipeline of layers in fewer launches, but a group of fewer SMs streams and multiplies
-  // more weights per SM; short leaves fill it sooner, long ones have fewer launches.  8 layers, ms for 4 / 6 / 8 places with leaves of 16, then of 32: d = 1024,
-  // B = 16, N = 512 31.4 32.7 35.1, 30.0 32.5 35.6; d = 768 25.3 21.6 23.8, 24.3 21.1 24.2; d = 512 20.5 16.3 15.5, 19.5 16.6 16.0; d = 1024, B = 1 22.9 22.7 21.3, 21.8 23.6 22.9.
-  const float layer_mb = (3.0f * c->d_model + 2.0f * c->d_ff) * c->d_model * 2e-6f;
-  const int band = n_layers < kWaveBand ? n_layers : kWaveBand;
+  if (N > kWaveExactN && ml.leaf != kWaveBlock) return none;
+  // How many layers at a time, and by which leaves: the least time estimated.  More places fill and drain the pipeline of layers in fewer launches, but a
+  // group of fewer SMs streams and multiplies more weights per SM; short leaves fill it sooner, long ones have fewer launches.
   int places = 0, leaf = 0;
-  long long launches = 0;
   float least = 0.0f;
   for (int pl = 2; pl <= kGroupJobs && pl <= n_layers; ++pl) {
     if (!leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, pl, kB200SmemPerCta)) continue;
-    const float step = leaf_group_step_us(B, c->d_model, c->d_ff, pl);
     for (int lf = c->leaf ? c->leaf : 16; lf <= wave_leaf_max(c, N); lf *= 2) {
-      const long long n = wave_launches(band, ceil_div(N, lf), pl);
-      const float us = (float)n * ((float)lf * step + (B > 8 ? 20.0f + 1.35f * layer_mb * (float)pl : 33.0f + 0.35f * layer_mb * (float)pl));
-      if (!places || us < least) { places = pl; leaf = lf; launches = n; least = us; }
+      const float us = wave_us(c, B, N, n_layers, pl, lf);
+      if (!places || us < least) { places = pl; leaf = lf; least = us; }
     }
   }
   if (!places) return none;
-  // Side by side a position costs a layer more (fewer SMs, weights from L2), so enough layers have to be at work at the same time: on average
-  // n_layers * N / (launches * leaf) of them.  Break even was measured at 1.3 to 2.3, growing with the weights that the groups stream (places x MB
-  // per layer) and above four sequences: 8 layers of d = 1024, B = 1, take 1.69 times as long as one after the other for 16 positions (one layer at a
-  // time), 1.05 for 32, 0.84 for 48, 0.72 for 77; B = 16 1.98, 1.20, 0.95 and for 64 0.83; 2 layers 1.33, 1.09, 1.03 and for 128 0.97.
-  auto even = [&](int pl) { return 1.26f + 0.008f * (float)pl * layer_mb + (B > 4 ? 0.15f : 0.0f); };
+  // Four layers side by side, each in the place of the one four before it, pay where enough of them are at work at the same time: on average n_layers * N /
+  // (launches * leaf) of them, 1.3 to 2.3, more the more weights the groups stream (places x MB per layer) and above four sequences.
+  const float layer_mb = (3.0f * c->d_model + 2.0f * c->d_ff) * c->d_model * 2e-6f, mma_us = B > 8 ? 10.5f : 8.3f;
+  auto four_pay = [&](float step_us) {                         // step_us: the time per position that the layers take alone, at most mma_us
+    const int four = n_layers < 4 ? n_layers : 4, lf = c->leaf ? c->leaf : N <= 128 ? 16 : 32, n = ceil_div(N, lf), turn = n > four ? n : four;
+    const float at_work = (float)n_layers * (float)N / (float)(((n_layers - 1) / four * turn + (n_layers - 1) % four + n) * lf);
+    const float even = (1.26f + 0.008f * (float)four * layer_mb + (B > 4 ? 0.15f : 0.0f)) * (step_us < mma_us ? mma_us / step_us : 1.0f);
+    return leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, four, kB200SmemPerCta) && at_work > even;
+  };
   LeafSmallLaunch sl;
   if (leaf_small_shape(c->dtype, B, c->d_model, c->n_heads, c->d_ff, ml.leaf, kB200SmemPerCta, &sl)) {
     // Layers that fit a cluster (rt_leaf_small.cu) hold the values between the phases in fp32 there, in bf16 here (8 layers of d = 128, B = 1, N = 200: error
     // of the last k against 64 bits 4.95e-3 and 5.2e-3; 2 layers of d = 384 2.97e-3 and 3.3e-3).  So more than four places are no reason to take them
-    // off it: they go side by side only where four, each layer in the place of the one four before it, pay against that kernel, which is faster than the
-    // tensor-core leaf kernel (taken as 8.3 us a position, above eight sequences 10.5): as many more layers have to be at work.
+    // off it: they go side by side only where four pay against that kernel, which is faster than the tensor-core leaf kernel (taken as mma_us a position).
     if (N > kWaveExactN) return none;                           // (the bits of that kernel)
-    const int four = n_layers < 4 ? n_layers : 4, lf = c->leaf ? c->leaf : N <= 128 ? 16 : 32, n = ceil_div(N, lf), turn = n > four ? n : four;
-    const float mma_us = B > 8 ? 10.5f : 8.3f, faster = sl.step_us < mma_us ? mma_us / sl.step_us : 1.0f;
-    const float at_work = (float)n_layers * (float)N / (float)(((n_layers - 1) / four * turn + (n_layers - 1) % four + n) * lf);
-    return leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, four, kB200SmemPerCta) && at_work > even(four) * faster ? Wave{places, leaf} : none;
+    return four_pay(sl.step_us) ? Wave{places, leaf} : none;
   }
-  const float at_work = (float)band * (float)N / ((float)launches * (float)leaf);
-  return at_work > even(places) ? Wave{places, leaf} : none;
+  // All others go side by side where that is estimated to be faster, and between 65 and 1024 positions also wherever four layers pay: there the pairs of the
+  // leaves that begin before position 192 keep fp32 probabilities, which layers one after the other round to bf16 from position 64 on.  Over 2 to 8 layers of
+  // d = 448, 512, 768, 960 and 1024, 1 to 16 sequences and 32 to 1024 positions (1100 stacks, both ways timed) the estimate's choice is on average 0.4 % and at most
+  // 16 % slower than the other; with one break-even for all widths stacks of d = 960 went side by side at up to 1.45 times the time (2 layers, N = 129: 2.30 and 3.34
+  // ms; d = 448, N = 100: 1.65 and 1.95) and 4 layers of d = 1024, B = 16, N = 64 did not at 1.19 times (2.99 and 2.52).
+  return 0.95f * least < alone_us(c, B, N, n_layers) || (N > kWaveBlock && N <= kWaveExactN && four_pay(mma_us)) ? Wave{places, leaf} : none;
 }
 struct WaveRows { size_t n, q, kt, vt, st_o, st_m, st_l, total; };
 WaveRows wave_rows_layout(const rt_config* c, int B, int leaf) {

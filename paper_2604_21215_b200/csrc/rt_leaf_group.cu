@@ -670,13 +670,14 @@ __global__ void __launch_bounds__(kGThreads, 1) leaf_group_kernel(const __grid_c
 // SMs of a group; every CTA owns rows of W_down (what the words are set back by: whoever publishes z has read all that came before).
 static int group_size(int d, int places) { const int g = kB200Sms / places; return g < d / 2 ? g : d / 2; }
 
-// Microseconds per position, estimated: the exchanges, and the rounds of four tiles that a warp goes through.  Measured, 4 / 6 / 8 places: d = 1024,
-// B = 16 24.2, -, 40.3 (11 and 22 rounds); d = 768 19.7, 20.1, 27.5 (9, 10, 17); d = 512 15.7, -, 18.5 (6, 9); d = 1024, B = 1 17.6, -, 28.2; d = 512, B = 4 12.7, -, 14.7.
+// Microseconds per position, estimated: the exchanges, and the rounds of four tiles that a warp goes through.  Measured / estimated for 2, 4, 6, 8 places (d = 768 six, d = 1024
+// four at most, see leaf_group_shape): B = 1 d = 512 11.9 / 12.4, 12.0 / 12.6, 13.5 / 13.1, 14.3 / 13.3; d = 768 14.1 / 13.6, 15.0 / 14.4, 14.8 / 14.7; d = 1024 14.5 / 14.9, 16.5 / 16.4;
+// B = 16 d = 512 14.4 / 14.4, 14.1 / 14.8, 15.3 / 15.5, 16.6 / 15.9; d = 768 16.7 / 16.5, 17.4 / 17.6, 18.1 / 18.2; d = 1024 17.8 / 18.6, 19.8 / 20.8.
 float leaf_group_step_us(int B, int d, int dff, int places) {
   const GroupShape s = group_shape(d, dff, group_size(d, places));
   auto rounds = [](int tiles) { return (tiles + kQuad - 1) / kQuad; };
-  const int n = 1 + s.nq + rounds(s.nt_f) + rounds(2 * s.nt_d);
-  return B > 8 ? 9.5f + 1.4e-3f * (float)(n * d) : 8.0f + 1.0e-3f * (float)(n * d);
+  const float n = (float)((1 + s.nq + rounds(s.nt_f) + rounds(2 * s.nt_d)) * d), b = 0.2f * (float)B;
+  return B > 8 ? 9.3f + b + 7.4e-4f * n : 11.0f + b + 4.6e-4f * n;
 }
 
 size_t leaf_group_words_bytes(int d, int dff) { return align_up((size_t)kTurns * (3 * 32 * d + 32 * dff) + (size_t)16 * 2 * d * 8, 256); }

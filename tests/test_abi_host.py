@@ -179,3 +179,10 @@ def test_layers_run_side_by_side_where_enough_of_them_are_at_work():
     # layers of the cluster kernel, which holds their values between the phases in fp32, are not taken off it because more than four fit side by side
     for d, B, N, L in ((64, 4, 400, 4), (128, 1, 77, 8), (128, 1, 200, 8), (128, 8, 256, 3), (256, 1, 256, 3), (256, 8, 48, 4), (384, 1, 200, 2), (192, 1, 200, 4)):
         assert not side_by_side(d, B, N, L), (d, B, N, L)
+    # the others where it was measured to be faster: widths that are no multiple of 128 pay for a pre-pass per launch, wide layers of nine and more sequences gain most;
+    # a leaf reads its layer's whole cache so far, so the longest prompts go one after the other (crossing measured between 16 and 32 thousand positions for two
+    # layers, 33 and 65 thousand for eight, d = 1024, B = 16)
+    for d, B, N, L in ((448, 1, 64, 2), (448, 4, 48, 3), (960, 4, 64, 2), (960, 1, 200, 2), (960, 4, 129, 3), (768, 1, 48, 2), (1024, 16, 32768, 2), (1024, 16, 131072, 8), (1024, 1, 400000, 8)):
+        assert not side_by_side(d, B, N, L), (d, B, N, L)
+    for d, B, N, L in ((1024, 16, 64, 4), (1024, 9, 129, 4), (512, 1, 77, 8), (448, 9, 200, 4), (1024, 16, 16384, 2), (1024, 16, 32768, 8), (512, 16, 32768, 8), (1024, 1, 65536, 8)):
+        assert side_by_side(d, B, N, L), (d, B, N, L)
