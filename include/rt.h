@@ -45,7 +45,7 @@ typedef enum {
   RT_OK = 0,
   RT_ERR_INVALID_ARG = 1,   /* null pointer, non-positive size, misaligned pointer, inconsistent shape */
   RT_ERR_UNSUPPORTED = 2,   /* valid request this build has no kernel for (e.g. head_dim != 64) */
-  RT_ERR_WORKSPACE = 3,     /* workspace_bytes < rt_workspace_bytes(...) */
+  RT_ERR_WORKSPACE = 3,     /* workspace_bytes < rt_workspace_bytes(...), see there */
   RT_ERR_CUDA = 4,          /* a CUDA runtime call failed (launch, attribute query) */
   RT_ERR_TIMEOUT = 5        /* a bounded device-side wait expired; outputs are invalid */
 } rt_status;
@@ -103,7 +103,10 @@ typedef struct {            /* device pointers; read-only */
 /* Bytes of workspace a call with these shapes needs (N = positions per call: the prefill
  * length, or 1 for decode).  n_layers >= 1.  Returns 0 for an invalid configuration.  Never
  * smaller for a larger B, N or n_layers (the same holds for the two sizes below): a workspace for
- * the fullest batch, the longest prompt and the deepest stack serves every smaller call. */
+ * the fullest batch, the longest prompt and the deepest stack serves every smaller call.
+ * rt_stack_prefill also takes less, down to the size for one layer: the rest holds weights of layers that
+ * run side by side, in packed form (of up to 16 layers; 23 MB each at d_model = 1024), and with less of
+ * it fewer of them do, down to none. */
 size_t rt_workspace_bytes(const rt_config *cfg, int32_t B, int32_t N, int32_t n_layers);
 
 /* One RT layer over x[B,N,d] (Sec. 2.2; Algorithm 1).  Writes z[B,N,d] and rows [0,N) of

@@ -19,7 +19,7 @@ constexpr int kSmallBatchMax = 64;      // above this the per-token chain runs a
 constexpr int kAutoLeaf = 64;
 
 struct WsLayout {
-  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, ll, ll_bytes, form, g_arrays, dec_words, dec_words_bytes, hid0, hid1,
+  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, ll, ll_bytes, form, form_bytes, g_arrays, dec_words, dec_words_bytes, hid0, hid1,
       blk_h, blk_u, blk_c, blk_g, total;
 };
 
@@ -94,7 +94,7 @@ Schedule effective_schedule(const rt_config* c, int B, int N) {
 
 // The layers of a stack side by side (rt_leaf_group.cu): layer l works on a leaf that layer l-1 finished in an earlier
 // launch, up to `places` layers in a launch, a group of SMs each.  places = 0: one layer after the other.
-struct Wave { int places, leaf; };
+struct Wave { int places, leaf, packs; };      // packs: layers whose packed weights are held at a time; deeper stacks run band after band
 // longest leaf of layers side by side (what the workspace holds rows for)
 int wave_leaf_max(const rt_config* c, int N) { return c->leaf ? c->leaf : N <= 128 ? 16 : N <= 1024 ? 32 : 64; }
 constexpr int kWaveBlock = 64;           // earlier pairs come by whole blocks of this many from the tile kernel, the rest of them inside the leaf kernel
@@ -111,11 +111,13 @@ bool wave_exact_tile(int N, int t0) { return N <= kWaveExactN && t0 < kWaveExact
 // head), 1.15 us each behind one another or 4.2 ns where they fill the chip; the same pairs cost 1.2 ns in Algorithm 1's larger tiles.  So one after the other, whose
 // cache traffic is N log N, is the faster form again from some length on: some 65 thousand positions for 8 layers of d = 1024, B = 16, some 20 thousand for 2.
 // Widths that are no multiple of 128 take the fp32 pre-pass, whose time per launch of leaves is 0.05 d us a layer and more.
+int band_begin(int n_layers, int bands, int b) { return (int)((long long)n_layers * b / bands); }      // (bands of about the same depth)
 bool tensor_prepass(const rt_config* c) { return c->d_model % 128 == 0; }
-float wave_us(const rt_config* c, int B, int N, int n_layers, int places, int leaf) {
+float wave_us(const rt_config* c, int B, int N, int n_layers, const Wave& w) {
+  const int places = w.places, leaf = w.leaf, bands = ceil_div(n_layers, w.packs);
   const float d = (float)c->d_model, tiles = (float)(places * B * c->n_heads), blocks = (float)N / (float)kWaveBlock;
   long long launches = 0;
-  for (int l0 = 0; l0 < n_layers; l0 += kWaveBand) launches += wave_launches(n_layers - l0 < kWaveBand ? n_layers - l0 : kWaveBand, ceil_div(N, leaf), places);
+  for (int b = 0; b < bands; ++b) launches += wave_launches(band_begin(n_layers, bands, b + 1) - band_begin(n_layers, bands, b), ceil_div(N, leaf), places);
   float us = (float)leaf * leaf_group_step_us(B, c->d_model, c->d_ff, places) + 21.0f + 3.5e-4f * (float)(places * B) * d;
   if (!tensor_prepass(c)) us += (float)places * d * (0.048f + 4.2e-7f * (float)B * d);
   // of the whole blocks that come before a leaf, on average half: a launch for each power of two that their number consists of
@@ -126,52 +128,6 @@ float alone_us(const rt_config* c, int B, int N, int n_layers) {
   const float d = (float)c->d_model, blocks = (float)N / (float)kWaveBlock;
   const float step = 7.4f + 1.3e-3f * d + 8.6e-5f * (float)B * d + (B > 8 ? 1.5f : 0.0f) + (tensor_prepass(c) ? 0.0f : 2.0e-7f * (float)B * d * d);
   return (float)n_layers * ((float)N * step + 0.6e-3f * (float)(B * c->n_heads) * blocks * blocks);
-}
-Wave stack_wave(const rt_config* c, int B, int N, int n_layers) {
-  const Wave none = {0, 0};
-  if (n_layers < 2 || N < 2 || c->dtype != RT_BF16 || c->sched != RT_SCHED_TILED || c->recur_block > 1) return none;
-  LeafMmaLaunch ml;                                            // (a stack of layers for the generic kernel keeps its fp32 vectors)
-  if (!leaf_mma_shape(B, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml)) return none;
-  // A leaf meets all earlier pairs at once when its queries exist (they depend on the layer below, so Algorithm 1's tiles cannot
-  // run ahead): each leaf reads the layer's whole cache so far, in the parts in which those tiles would have brought it.  The group kernel's sums have the order
-  // of the leaf kernel, so a stack gives the bits of the same layers called one by one, where those take leaves of kWaveBlock positions;
-  // elsewhere long sequences go layer by layer for the sake of these bits.
-  if (N > kWaveExactN && ml.leaf != kWaveBlock) return none;
-  // How many layers at a time, and by which leaves: the least time estimated.  More places fill and drain the pipeline of layers in fewer launches, but a
-  // group of fewer SMs streams and multiplies more weights per SM; short leaves fill it sooner, long ones have fewer launches.
-  int places = 0, leaf = 0;
-  float least = 0.0f;
-  for (int pl = 2; pl <= kGroupJobs && pl <= n_layers; ++pl) {
-    if (!leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, pl, kB200SmemPerCta)) continue;
-    for (int lf = c->leaf ? c->leaf : 16; lf <= wave_leaf_max(c, N); lf *= 2) {
-      const float us = wave_us(c, B, N, n_layers, pl, lf);
-      if (!places || us < least) { places = pl; leaf = lf; least = us; }
-    }
-  }
-  if (!places) return none;
-  // Four layers side by side, each in the place of the one four before it, pay where enough of them are at work at the same time: on average n_layers * N /
-  // (launches * leaf) of them, 1.3 to 2.3, more the more weights the groups stream (places x MB per layer) and above four sequences.
-  const float layer_mb = (3.0f * c->d_model + 2.0f * c->d_ff) * c->d_model * 2e-6f, mma_us = B > 8 ? 10.5f : 8.3f;
-  auto four_pay = [&](float step_us) {                         // step_us: the time per position that the layers take alone, at most mma_us
-    const int four = n_layers < 4 ? n_layers : 4, lf = c->leaf ? c->leaf : N <= 128 ? 16 : 32, n = ceil_div(N, lf), turn = n > four ? n : four;
-    const float at_work = (float)n_layers * (float)N / (float)(((n_layers - 1) / four * turn + (n_layers - 1) % four + n) * lf);
-    const float even = (1.26f + 0.008f * (float)four * layer_mb + (B > 4 ? 0.15f : 0.0f)) * (step_us < mma_us ? mma_us / step_us : 1.0f);
-    return leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, four, kB200SmemPerCta) && at_work > even;
-  };
-  LeafSmallLaunch sl;
-  if (leaf_small_shape(c->dtype, B, c->d_model, c->n_heads, c->d_ff, ml.leaf, kB200SmemPerCta, &sl)) {
-    // Layers that fit a cluster (rt_leaf_small.cu) hold the values between the phases in fp32 there, in bf16 here (8 layers of d = 128, B = 1, N = 200: error
-    // of the last k against 64 bits 4.95e-3 and 5.2e-3; 2 layers of d = 384 2.97e-3 and 3.3e-3).  So more than four places are no reason to take them
-    // off it: they go side by side only where four pay against that kernel, which is faster than the tensor-core leaf kernel (taken as mma_us a position).
-    if (N > kWaveExactN) return none;                           // (the bits of that kernel)
-    return four_pay(sl.step_us) ? Wave{places, leaf} : none;
-  }
-  // All others go side by side where that is estimated to be faster, and between 65 and 1024 positions also wherever four layers pay: there the pairs of the
-  // leaves that begin before position 192 keep fp32 probabilities, which layers one after the other round to bf16 from position 64 on.  Over 2 to 8 layers of
-  // d = 448, 512, 768, 960 and 1024, 1 to 16 sequences and 32 to 1024 positions (1100 stacks, both ways timed) the estimate's choice is on average 0.4 % and at most
-  // 16 % slower than the other; with one break-even for all widths stacks of d = 960 went side by side at up to 1.45 times the time (2 layers, N = 129: 2.30 and 3.34
-  // ms; d = 448, N = 100: 1.65 and 1.95) and 4 layers of d = 1024, B = 16, N = 64 did not at 1.19 times (2.99 and 2.52).
-  return 0.95f * least < alone_us(c, B, N, n_layers) || (N > kWaveBlock && N <= kWaveExactN && four_pay(mma_us)) ? Wave{places, leaf} : none;
 }
 struct WaveRows { size_t n, q, kt, vt, st_o, st_m, st_l, total; };
 WaveRows wave_rows_layout(const rt_config* c, int B, int leaf) {
@@ -190,7 +146,7 @@ WaveRows wave_rows_layout(const rt_config* c, int B, int leaf) {
 struct GroupArea { size_t packed, packed_stride, rows, rows_stride, total; };
 GroupArea group_area(const rt_config* c, int places, int packs, int wave_B, int wave_leaf) {
   GroupArea A;
-  A.packed = align_up((size_t)kGroupJobs * leaf_group_words_bytes(c->d_model, c->d_ff), 256);
+  A.packed = align_up((size_t)places * leaf_group_words_bytes(c->d_model, c->d_ff), 256);
   A.packed_stride = leaf_group_packed_bytes(c->d_model, c->d_ff, places);
   A.rows = A.packed + align_up(A.packed_stride * packs, 256);
   A.rows_stride = wave_leaf ? wave_rows_layout(c, wave_B, wave_leaf).total : 0;
@@ -198,6 +154,56 @@ GroupArea group_area(const rt_config* c, int places, int packs, int wave_B, int 
   return A;
 }
 
+// `form`: bytes of the area that the groups work in.
+Wave stack_wave(const rt_config* c, int B, int N, int n_layers, size_t form) {
+  const Wave none = {0, 0, 0};
+  if (n_layers < 2 || N < 2 || c->dtype != RT_BF16 || c->sched != RT_SCHED_TILED || c->recur_block > 1) return none;
+  LeafMmaLaunch ml;                                            // (a stack of layers for the generic kernel keeps its fp32 vectors)
+  if (!leaf_mma_shape(B, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml)) return none;
+  // A leaf meets all earlier pairs at once when its queries exist (they depend on the layer below, so Algorithm 1's tiles cannot
+  // run ahead): each leaf reads the layer's whole cache so far, in the parts in which those tiles would have brought it.  The group kernel's sums have the order
+  // of the leaf kernel, so a stack gives the bits of the same layers called one by one, where those take leaves of kWaveBlock positions;
+  // elsewhere long sequences go layer by layer for the sake of these bits.
+  if (N > kWaveExactN && ml.leaf != kWaveBlock) return none;
+  // How many layers at a time, and by which leaves: the least time estimated.  More places fill and drain the pipeline of layers in fewer launches, but a
+  // group of fewer SMs streams and multiplies more weights per SM; short leaves fill it sooner, long ones have fewer launches.
+  Wave best = none;
+  float least = 0.0f;
+  for (int pl = 2; pl <= kGroupJobs && pl <= n_layers; ++pl) {
+    if (!leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, pl, kB200SmemPerCta)) continue;
+    for (int lf = c->leaf ? c->leaf : 16; lf <= wave_leaf_max(c, N); lf *= 2) {
+      Wave w = {pl, lf, n_layers < kWaveBand ? n_layers : kWaveBand};
+      while (w.packs > 1 && group_area(c, pl, w.packs, B, lf).total > form) --w.packs;
+      if (w.packs < 2) continue;
+      const float us = wave_us(c, B, N, n_layers, w);
+      if (!best.places || us < least) { best = w; least = us; }
+    }
+  }
+  if (!best.places) return none;
+  // Four layers side by side, each in the place of the one four before it, pay where enough of them are at work at the same time: on average n_layers * N /
+  // (launches * leaf) of them, 1.3 to 2.3, more the more weights the groups stream (places x MB per layer) and above four sequences.
+  const float layer_mb = (3.0f * c->d_model + 2.0f * c->d_ff) * c->d_model * 2e-6f, mma_us = B > 8 ? 10.5f : 8.3f;
+  auto four_pay = [&](float step_us) {                         // step_us: the time per position that the layers take alone, at most mma_us
+    const int four = n_layers < 4 ? n_layers : 4, lf = c->leaf ? c->leaf : N <= 128 ? 16 : 32, n = ceil_div(N, lf), turn = n > four ? n : four;
+    const float at_work = (float)n_layers * (float)N / (float)(((n_layers - 1) / four * turn + (n_layers - 1) % four + n) * lf);
+    const float even = (1.26f + 0.008f * (float)four * layer_mb + (B > 4 ? 0.15f : 0.0f)) * (step_us < mma_us ? mma_us / step_us : 1.0f);
+    return leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, four, kB200SmemPerCta) && at_work > even;
+  };
+  LeafSmallLaunch sl;
+  if (leaf_small_shape(c->dtype, B, c->d_model, c->n_heads, c->d_ff, ml.leaf, kB200SmemPerCta, &sl)) {
+    // Layers that fit a cluster (rt_leaf_small.cu) hold the values between the phases in fp32 there, in bf16 here (8 layers of d = 128, B = 1, N = 200: error
+    // of the last k against 64 bits 4.95e-3 and 5.2e-3; 2 layers of d = 384 2.97e-3 and 3.3e-3).  So more than four places are no reason to take them
+    // off it: they go side by side only where four pay against that kernel, which is faster than the tensor-core leaf kernel (taken as mma_us a position).
+    if (N > kWaveExactN) return none;                           // (the bits of that kernel)
+    return four_pay(sl.step_us) ? best : none;
+  }
+  // All others go side by side where that is estimated to be faster, and between 65 and 1024 positions also wherever four layers pay: there the pairs of the
+  // leaves that begin before position 192 keep fp32 probabilities, which layers one after the other round to bf16 from position 64 on.  Over 2 to 8 layers of
+  // d = 448, 512, 768, 960 and 1024, 1 to 16 sequences and 32 to 1024 positions (1100 stacks, both ways timed) the estimate's choice is on average 0.4 % and at most
+  // 16 % slower than the other; with one break-even for all widths stacks of d = 960 went side by side at up to 1.45 times the time (2 layers, N = 129: 2.30 and 3.34
+  // ms; d = 448, N = 100: 1.65 and 1.95) and 4 layers of d = 1024, B = 16, N = 64 did not at 1.19 times (2.99 and 2.52).
+  return 0.95f * least < alone_us(c, B, N, n_layers) || (N > kWaveBlock && N <= kWaveExactN && four_pay(mma_us)) ? best : none;
+}
 // Positions that the tensor-core leaf kernel has an array of g for: a leaf, or all layers of a prompt shorter than that (one fill serves
 // them: 8 layers of one position, d = 1024, 305 -> 291 us).
 int g_positions(const rt_config* c, int N, int n_layers) {
@@ -225,7 +231,8 @@ size_t form_bytes(const rt_config* c, int B, int N, int n_layers) {
   return most;
 }
 
-WsLayout ws_layout(const rt_config* c, int B, int N, int n_layers) {
+// more_form: bytes that the area of the token loop's form gets beyond what it needs.
+WsLayout ws_layout(const rt_config* c, int B, int N, int n_layers, size_t more_form = 0) {
   WsLayout L;
   const size_t e = esize_of(c->dtype), d = c->d_model, H = c->n_heads, f = c->d_ff;
   const size_t tok = (size_t)B * N;
@@ -249,7 +256,8 @@ WsLayout ws_layout(const rt_config* c, int B, int N, int n_layers) {
   L.ll_bytes = (size_t)B * 2 * d * 8;
   L.ll = take(L.ll_bytes);
   L.g_arrays = c->dtype == RT_BF16 ? g_positions(c, N, n_layers) : 0;
-  L.form = take(form_bytes(c, B, N, n_layers));
+  L.form_bytes = form_bytes(c, B, N, n_layers) + more_form;
+  L.form = take(L.form_bytes);
   // a decode step uses none of the above but the status block: its exchange area begins right behind that
   L.dec_words = L.q;
   const size_t dec = c->dtype == RT_BF16 ? decode_words_bytes(n_layers, B, (int)d, (int)H, (int)f) : 0;
@@ -317,10 +325,10 @@ struct ProfScope {
 struct CallCtx { cudaStream_t s; unsigned bar_base = 0; unsigned seq_base = 0; unsigned group_steps[kGroupJobs] = {}; bool groups_cleared = false; int g_left = 0; };      // g_left: arrays of g still filled
 
 // The exchange areas of the group kernel start from ones (no word written), once per API call.
-bool clear_groups(const rt_config* c, unsigned char* ws, const WsLayout& L, CallCtx& ctx) {
+bool clear_groups(const rt_config* c, int places, unsigned char* ws, const WsLayout& L, CallCtx& ctx) {
   if (ctx.groups_cleared) return true;
   ctx.groups_cleared = true;
-  return cudaMemsetAsync(ws + L.form, 0xFF, (size_t)kGroupJobs * leaf_group_words_bytes(c->d_model, c->d_ff), ctx.s) == cudaSuccess;
+  return cudaMemsetAsync(ws + L.form, 0xFF, (size_t)places * leaf_group_words_bytes(c->d_model, c->d_ff), ctx.s) == cudaSuccess;
 }
 GroupCommon group_common(const rt_config* c, int B, unsigned char* ws, const WsLayout& L) {
   GroupCommon g;
@@ -624,7 +632,7 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
   const int places = groups ? ceil_div(B, plan.sub) : 0;
   unsigned char* const packed = groups ? ws + L.form + group_area(c, places, 1, 0, 0).packed : nullptr;
   if (groups) {
-    if (!clear_groups(c, ws, L, ctx)) return RT_ERR_CUDA;
+    if (!clear_groups(c, places, ws, L, ctx)) return RT_ERR_CUDA;
     const GroupPackLayer pl = {w->w_o, w->w_up, w->w_down, w->w_k, w->w_v, packed};
     ProfScope ps(s, kProfPrepass);
     if (leaf_group_pack(&pl, 1, c->d_model, c->d_ff, places, s) != cudaSuccess) return RT_ERR_CUDA;
@@ -677,16 +685,16 @@ bool caches_overlap(const rt_config* c, int n_layers, int B, int N, void* const*
 rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weights* layers, void* const* hid, void* out, int B, int N, void* const* k_caches,
                          void* const* v_caches, int N_max, unsigned char* ws, const WsLayout& L, const Wave& wv, CallCtx& ctx) {
   cudaStream_t s = ctx.s;
-  const int places = wv.places, n_leaves = ceil_div(N, wv.leaf), band_max = n_layers < kWaveBand ? n_layers : kWaveBand;
+  const int places = wv.places, n_leaves = ceil_div(N, wv.leaf), bands = ceil_div(n_layers, wv.packs);
   const size_t e = esize_of(c->dtype), d = c->d_model;
   const WaveRows W = wave_rows_layout(c, B, wv.leaf);
-  const GroupArea A = group_area(c, places, band_max, B, wv.leaf);
-  if (!clear_groups(c, ws, L, ctx)) return RT_ERR_CUDA;
+  const GroupArea A = group_area(c, places, wv.packs, B, wv.leaf);
+  if (!clear_groups(c, places, ws, L, ctx)) return RT_ERR_CUDA;
   auto packed = [&](int l) { return ws + L.form + A.packed + (size_t)l * A.packed_stride; };
   const GroupCommon gc = group_common(c, B, ws, L);
   const long long bs = (long long)N * d;
-  for (int l0 = 0; l0 < n_layers; l0 += kWaveBand) {
-    const int band = n_layers - l0 < kWaveBand ? n_layers - l0 : kWaveBand;
+  for (int b = 0; b < bands; ++b) {
+    const int l0 = band_begin(n_layers, bands, b), band = band_begin(n_layers, bands, b + 1) - l0;
     {
       ProfScope ps(s, kProfPrepass);
       for (int i = 0; i < band; i += kGroupPackLayers) {
@@ -832,7 +840,7 @@ rt_status run_decode(const rt_config* c, int n_layers, const rt_layer_weights* l
 // bf16 shapes that the decode kernel takes; everything else takes the generic leaf kernel.
 bool decode_fast(const rt_config* c, int B) { return c->dtype == RT_BF16 && decode_shape(B, c->d_model, c->n_heads, c->d_ff); }
 
-rt_status common_checks(const rt_config* c, int B, int N, int n_layers, void* ws, size_t ws_bytes, bool wide_ok = false) {
+rt_status common_checks(const rt_config* c, int B, int N, int n_layers, void* ws, size_t ws_bytes, bool wide_ok = false) {      // n_layers: that the workspace has to suffice for
   if (!config_ok(c) || B <= 0 || N <= 0 || n_layers <= 0 || !ws || !aligned16(ws)) return RT_ERR_INVALID_ARG;
   const rt_status st = config_supported(c, B, wide_ok);
   if (st != RT_OK) return st;
@@ -1022,7 +1030,8 @@ rt_status rt_stack_prefill(const rt_config* cfg, int32_t n_layers, const rt_laye
                            const void* g_final, int32_t vocab, const int32_t* ids, int32_t B, int32_t N, void* hidden,
                            float* logits_last, void* const* k_caches, void* const* v_caches, int32_t N_max,
                            void* workspace, size_t workspace_bytes, void* cuda_stream) {
-  rt_status st = common_checks(cfg, B, N, n_layers, workspace, workspace_bytes, true);
+  if (n_layers <= 0) return RT_ERR_INVALID_ARG;
+  rt_status st = common_checks(cfg, B, N, 1, workspace, workspace_bytes, true);
   if (st != RT_OK) return st;
   if (!layers || !emb || !ids || !k_caches || !v_caches || vocab <= 0 || N_max < N) return RT_ERR_INVALID_ARG;
   if (!aligned16(emb) || (hidden && !aligned16(hidden)) || (g_final && !aligned16(g_final))) return RT_ERR_INVALID_ARG;
@@ -1033,7 +1042,9 @@ rt_status rt_stack_prefill(const rt_config* cfg, int32_t n_layers, const rt_laye
   if ((size_t)B * cfg->d_model * 4 > 200 * 1024) return RT_ERR_UNSUPPORTED;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   unsigned char* ws = (unsigned char*)workspace;
-  const WsLayout L = ws_layout(cfg, B, N, n_layers);
+  WsLayout L = ws_layout(cfg, B, N, n_layers);
+  if (workspace_bytes < L.total)                               // what there is beyond a single layer's goes to layers side by side
+    L = ws_layout(cfg, B, N, 1, (workspace_bytes - ws_layout(cfg, B, N, 1).total) & ~(size_t)255);
   if (cudaMemsetAsync(ws + L.sync, 0, sizeof(SyncArea), s) != cudaSuccess) return RT_ERR_CUDA;
   if (cudaMemsetAsync(ws + L.ll, 0, L.ll_bytes, s) != cudaSuccess) return RT_ERR_CUDA;
   const long long d = cfg->d_model;
@@ -1044,7 +1055,7 @@ rt_status rt_stack_prefill(const rt_config* cfg, int32_t n_layers, const rt_laye
     if (embed_launch(cfg->dtype, emb, ids, B, N, (int)d, vocab, bufs[0], s) != cudaSuccess) return RT_ERR_CUDA;
   }
   const void* cur = bufs[0];
-  Wave wv = stack_wave(cfg, B, N, n_layers);
+  Wave wv = stack_wave(cfg, B, N, n_layers, L.form_bytes);
   if (wv.places && caches_overlap(cfg, n_layers, B, N, k_caches, v_caches)) wv.places = 0;
   if (wv.places) {
     st = run_stack_wave(cfg, n_layers, layers, bufs, hidden, B, N, k_caches, v_caches, N_max, ws, L, wv, ctx);
@@ -1228,7 +1239,7 @@ rt_status rt_plan_counters(const rt_config* cfg, int32_t B, int32_t N, int32_t n
   } else {
     // the schedule that runs: leaf (or block) granularity of the chain form this shape takes
     const Schedule plan = effective_schedule(cfg, B, N);
-    const Wave wv = stack_wave(cfg, B, N, n_layers);             // layers side by side: every leaf meets all earlier pairs at once
+    const Wave wv = stack_wave(cfg, B, N, n_layers, SIZE_MAX);             // layers side by side: every leaf meets all earlier pairs at once
     const uint64_t Lf = wv.places ? wv.leaf : plan.leaf;
     for (uint64_t s0 = 0; s0 < n; s0 += Lf) {
       const uint64_t e0 = s0 + Lf < n ? s0 + Lf : n, len = e0 - s0;

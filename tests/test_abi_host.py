@@ -186,3 +186,17 @@ def test_layers_run_side_by_side_where_enough_of_them_are_at_work():
         assert not side_by_side(d, B, N, L), (d, B, N, L)
     for d, B, N, L in ((1024, 16, 64, 4), (1024, 9, 129, 4), (512, 1, 77, 8), (448, 9, 200, 4), (1024, 16, 16384, 2), (1024, 16, 32768, 8), (512, 16, 32768, 8), (1024, 1, 65536, 8)):
         assert side_by_side(d, B, N, L), (d, B, N, L)
+
+
+def test_a_stack_prefill_is_refused_only_below_the_workspace_of_one_layer():
+    # what it has beyond that holds weights of layers side by side: the first figure is a size that once sufficed.  (Refused later on, for the missing layers.)
+    buf = (C.c_char * 4096)()
+    addr = (C.addressof(buf) + 255) & ~255
+    for d, B, N, L, given in ((1024, 1, 77, 8, 106650880), (768, 4, 512, 8, 90797312), (1024, 16, 2048, 8, None), (128, 2, 300, 4, None), (512, 40, 100, 3, None)):
+        cfg = rt.make_config(d, d // 64, 4 * d, dtype="bf16")
+        least = rt.rt_workspace_bytes(cfg, B, N, 1)
+        def call(size):
+            return rt.rt_stack_prefill(cfg, L, None, addr, None, 10, addr, B, N, None, None, None, None, N, addr, size, None)
+        assert least <= rt.rt_workspace_bytes(cfg, B, N, L)
+        assert call(least - 1) == rt.RT_ERR_WORKSPACE and call(least) == rt.RT_ERR_INVALID_ARG
+        assert given is None or call(given) == rt.RT_ERR_INVALID_ARG

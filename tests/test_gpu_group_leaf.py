@@ -84,6 +84,41 @@ def test_a_workspace_for_long_prompts_serves_short_ones(L, B, N):
     assert all(torch.equal(a, b) for a, b in zip(stacks[0][1], stacks[1][1]))
 
 
+# With less workspace than all layers side by side would use, fewer of them are (two at a time, in bands), or none; nothing is written behind what was given.  Beyond 1024
+# positions every form gives the same bits.
+@pytest.mark.parametrize("L,d,H,B,N", [(6, 512, 8, 2, 1090), (5, 768, 12, 9, 100), (3, 1024, 16, 20, 40)])
+def test_a_stack_runs_in_less_workspace(L, d, H, B, N):
+    import torch
+    from paper_2604_21215_b200 import inputs, rt
+    V, dff = 91, 4 * d
+    data = inputs.make_inputs(inputs.Workload("less", L, B, N, d, H, dff, "bf16", vocab=V, residual_scale=1 / np.sqrt(L)), seed=N)
+    st = rt.Stack(L, d, H, dff, V, dtype="bf16", residual_scale=1 / np.sqrt(L))
+    st.set_weights(data["layers"], data["emb"])
+    want, _ = st.prefill(data["ids"])
+    caches = st.caches_numpy(N)
+    if N < 1024 and B <= 16:                                    # the forms differ in rounding: each against the oracle
+        from oracle import RTConfig, RTWeights, stack_prefill
+        ref = stack_prefill(RTConfig(d, H, 64, dff, residual_scale=1 / np.sqrt(L)), [RTWeights(**lw) for lw in data["layers"]], data["emb"], None, data["ids"])[0]
+    least, full = rt.rt_workspace_bytes(st.cfg, B, N, 1), rt.rt_workspace_bytes(st.cfg, B, N, L)
+    ids = torch.as_tensor(data["ids"], dtype=torch.int32, device=st.device).contiguous()
+    layer_bytes = 11 * d * d * 2
+    for size in (least, least + 3 * layer_bytes, (least + full) // 2 + 100, full - 1):
+        if size > full:
+            continue
+        ws = torch.full((size + 65536,), 0x5A, dtype=torch.uint8, device=st.device)
+        st.ws = ws[:size]
+        hid = torch.empty((B, N, d), dtype=torch.bfloat16, device=st.device)
+        st.prefill_device(ids, hid, None)
+        torch.cuda.synchronize()
+        assert st.status() == rt.RT_OK and bool((ws[size:] == 0x5A).all())
+        got = hid.to(torch.float64).cpu().numpy()
+        if N > 1024 or B > 16:
+            assert np.array_equal(got, want)
+            assert all(np.array_equal(a, b) for p, q in zip(st.caches_numpy(N), caches) for a, b in zip(p, q))
+        else:
+            check_tensor(f"workspace of {size}", "hidden", got, ref, 2e-2)
+
+
 def _leaf128(L, B, N):
     from paper_2604_21215_b200 import inputs
     d, H, dff, V = 512, 8, 1024, 91
