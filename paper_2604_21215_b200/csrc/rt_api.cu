@@ -94,15 +94,15 @@ Schedule effective_schedule(const rt_config* c, int B, int N) {
 
 // The layers of a stack side by side (rt_leaf_group.cu): layer l works on a leaf that layer l-1 finished in an earlier
 // launch, up to `places` layers in a launch, a group of SMs each.  places = 0: one layer after the other.
-struct Wave { int places, leaf, packs; };      // packs: layers whose packed weights are held at a time; deeper stacks run band after band
+struct Wave { int places, leaf, packs, exact; };      // packs: layers whose packed weights are held at a time; deeper stacks run band after band.  exact: see wave_exact_tile
 // longest leaf of layers side by side (what the workspace holds rows for)
 int wave_leaf_max(const rt_config* c, int N) { return c->leaf ? c->leaf : N <= 128 ? 16 : N <= 1024 ? 32 : 64; }
 constexpr int kWaveBlock = 64;           // earlier pairs come by whole blocks of this many from the tile kernel, the rest of them inside the leaf kernel
-// The whole blocks of 64 pairs before a leaf that begins at t0 come from the fp32 tile kernel, not from the tensor-core one, which rounds its
-// probabilities to bf16: in stacks of up to kWaveExactN positions, for leaves that begin before kWaveExactMax.  Longer stacks give the bits of the
-// same layers one by one, whose tiles begin with the second block.
+// Stacks of up to kWaveExactN positions whose layers run, or by the four-place line of stack_wave could run, side by side: the whole blocks of 64 pairs before a
+// leaf that begins at t0 < kWaveExactMax come from a tile kernel with fp32 probabilities, not from the tensor-core one, which rounds them to bf16.  All other
+// stacks give the bits of the same layers one by one, whose tiles begin with the second block.
 constexpr int kWaveExactN = 1024, kWaveExactMax = 192;
-bool wave_exact_tile(int N, int t0) { return N <= kWaveExactN && t0 < kWaveExactMax; }
+bool wave_exact_tile(bool exact, int t0) { return exact && t0 < kWaveExactMax; }
 // Estimates (us) of a stack's token loops, side by side and one after the other.  Fitted to 16 widths from d = 64 to 1024, 1 to 16 sequences, 2 to 8 places and leaves of
 // 16, 32 and 64 (256 positions; 5 % off on average from d = 320 on) and checked on long stacks, ms measured / estimated, side by side and one after the other: 8 layers of d = 1024,
 // B = 1, N = 2048 82.6 / 75, 139 / 145, 16384 743 / 651, 1116 / 1161, 65536 3651 / 3519, 4480 / 4704; B = 16, N = 2048 111 / 101, 190 / 192, 16384 1146 / 1040, 1601 / 1606, 65536
@@ -156,7 +156,7 @@ GroupArea group_area(const rt_config* c, int places, int packs, int wave_B, int 
 
 // `form`: bytes of the area that the groups work in.
 Wave stack_wave(const rt_config* c, int B, int N, int n_layers, size_t form) {
-  const Wave none = {0, 0, 0};
+  const Wave none = {0, 0, 0, 0};
   if (n_layers < 2 || N < 2 || c->dtype != RT_BF16 || c->sched != RT_SCHED_TILED || c->recur_block > 1) return none;
   LeafMmaLaunch ml;                                            // (a stack of layers for the generic kernel keeps its fp32 vectors)
   if (!leaf_mma_shape(B, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml)) return none;
@@ -172,7 +172,7 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers, size_t form) {
   for (int pl = 2; pl <= kGroupJobs && pl <= n_layers; ++pl) {
     if (!leaf_group_shape(B, c->d_model, c->n_heads, c->d_ff, pl, kB200SmemPerCta)) continue;
     for (int lf = c->leaf ? c->leaf : 16; lf <= wave_leaf_max(c, N); lf *= 2) {
-      Wave w = {pl, lf, n_layers < kWaveBand ? n_layers : kWaveBand};
+      Wave w = {pl, lf, n_layers < kWaveBand ? n_layers : kWaveBand, N <= kWaveExactN};
       while (w.packs > 1 && group_area(c, pl, w.packs, B, lf).total > form) --w.packs;
       if (w.packs < 2) continue;
       const float us = wave_us(c, B, N, n_layers, w);
@@ -197,12 +197,14 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers, size_t form) {
     if (N > kWaveExactN) return none;                           // (the bits of that kernel)
     return four_pay(sl.step_us) ? best : none;
   }
-  // All others go side by side where that is estimated to be faster, and between 65 and 1024 positions also wherever four layers pay: there the pairs of the
-  // leaves that begin before position 192 keep fp32 probabilities, which layers one after the other round to bf16 from position 64 on.  Over 2 to 8 layers of
-  // d = 448, 512, 768, 960 and 1024, 1 to 16 sequences and 32 to 1024 positions (1100 stacks, both ways timed) the estimate's choice is on average 0.4 % and at most
-  // 16 % slower than the other; with one break-even for all widths stacks of d = 960 went side by side at up to 1.45 times the time (2 layers, N = 129: 2.30 and 3.34
-  // ms; d = 448, N = 100: 1.65 and 1.95) and 4 layers of d = 1024, B = 16, N = 64 did not at 1.19 times (2.99 and 2.52).
-  return 0.95f * least < alone_us(c, B, N, n_layers) || (N > kWaveBlock && N <= kWaveExactN && four_pay(mma_us)) ? best : none;
+  // All others go side by side where that is estimated to be faster.  Over 2 to 8 layers of d = 448, 512, 768, 960 and 1024, 1 to 16 sequences and 32 to 1024
+  // positions (1100 stacks, both ways timed) the choice is on average 0.4 % and at most 16 % slower than the other; with one break-even for all widths
+  // stacks of d = 960 went side by side at up to 1.45 times the time (2 layers, N = 129: 2.30 and 3.34 ms; d = 448, N = 100: 1.65 and 1.95) and 4
+  // layers of d = 1024, B = 16, N = 64 did not at 1.19 times (2.99 and 2.52).  The line for four places tells which stacks keep fp32 probabilities one after the other.
+  if (0.95f * least < alone_us(c, B, N, n_layers)) return best;
+  Wave alone = none;
+  alone.exact = N > kWaveBlock && N <= kWaveExactN && four_pay(mma_us);
+  return alone;
 }
 // Positions that the tensor-core leaf kernel has an array of g for: a leaf, or all layers of a prompt shorter than that (one fill serves
 // them: 8 layers of one position, d = 1024, 305 -> 291 us).
@@ -322,7 +324,7 @@ struct ProfScope {
 };
 
 // State of one API call: the stream and the barrier arrivals enqueued so far.
-struct CallCtx { cudaStream_t s; unsigned bar_base = 0; unsigned seq_base = 0; unsigned group_steps[kGroupJobs] = {}; bool groups_cleared = false; int g_left = 0; };      // g_left: arrays of g still filled
+struct CallCtx { cudaStream_t s; unsigned bar_base = 0; unsigned seq_base = 0; unsigned group_steps[kGroupJobs] = {}; bool groups_cleared = false; int g_left = 0; bool exact = false; };      // g_left: sets of vectors still filled; exact: first tiles with fp32 probabilities
 
 // The exchange areas of the group kernel start from ones (no word written), once per API call.
 bool clear_groups(const rt_config* c, int places, unsigned char* ws, const WsLayout& L, CallCtx& ctx) {
@@ -664,7 +666,7 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
       const int P = e0 & -e0;                              // largest power of two dividing the block end
       tp.q0 = e0; tp.q1 = e0 + P < N ? e0 + P : N; tp.k0 = e0 - P; tp.k1 = e0;
       ProfScope ps(s, kProfTile);
-      if (tile_launch(c->dtype, tp, s) != cudaSuccess) return RT_ERR_CUDA;
+      if ((wave_exact_tile(ctx.exact, e0) && P % kWaveBlock == 0 ? tile_rows_batch_launch(&tp, 1, s) : tile_launch(c->dtype, tp, s)) != cudaSuccess) return RT_ERR_CUDA;
     }
   }
   return RT_OK;
@@ -752,10 +754,10 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
       {
         int nt = 0;
         for (int i = 0; i < nj; ++i)
-          if (jobs[i].key0 && wave_exact_tile(N, jobs[i].t0)) tiles[nt++] = tile_of(i, 0, jobs[i].key0);
+          if (jobs[i].key0 && wave_exact_tile(wv.exact, jobs[i].t0)) tiles[nt++] = tile_of(i, 0, jobs[i].key0);
         if (nt) {
           ProfScope ps(s, kProfTile);
-          if (tile_simt_batch_launch(tiles, nt, s) != cudaSuccess) return RT_ERR_CUDA;
+          if (tile_rows_batch_launch(tiles, nt, s) != cudaSuccess) return RT_ERR_CUDA;
         }
       }
       // On tensor cores they come in the parts in which Algorithm 1's tiles would have brought them (the powers of two that the number of blocks
@@ -765,7 +767,7 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
         for (int sloped = 0; sloped < 2; ++sloped) {
           int nt = 0;
           for (int i = 0; i < nj; ++i) {
-            int blocks = wave_exact_tile(N, jobs[i].t0) ? 0 : jobs[i].key0 / kWaveBlock, k0 = 0, size = 0;
+            int blocks = wave_exact_tile(wv.exact, jobs[i].t0) ? 0 : jobs[i].key0 / kWaveBlock, k0 = 0, size = 0;
             for (int skip = 0; blocks && skip <= part; ++skip) {
               k0 += size;
               size = 1;
@@ -1057,6 +1059,7 @@ rt_status rt_stack_prefill(const rt_config* cfg, int32_t n_layers, const rt_laye
   const void* cur = bufs[0];
   Wave wv = stack_wave(cfg, B, N, n_layers, L.form_bytes);
   if (wv.places && caches_overlap(cfg, n_layers, B, N, k_caches, v_caches)) wv.places = 0;
+  ctx.exact = wv.exact != 0;
   if (wv.places) {
     st = run_stack_wave(cfg, n_layers, layers, bufs, hidden, B, N, k_caches, v_caches, N_max, ws, L, wv, ctx);
     if (st != RT_OK) return st;

@@ -172,8 +172,8 @@ cudaError_t tile_tc_launch(const TileParams& p, int rows_q, int rows_kv, SyncAre
 // one tile of each of n layers (n <= kGroupJobs, key counts multiples of 64, the same B, d, H; slopes in all or none)
 cudaError_t tile_tc_batch_launch(const TileParams* p, int n, SyncArea* sync, cudaStream_t s);
 cudaError_t tile_simt_launch(int dtype, const TileParams& p, cudaStream_t s);
-// bf16 tiles of n layers (1 <= n <= kGroupJobs, the same B, d, H), probabilities in fp32
-cudaError_t tile_simt_batch_launch(const TileParams* p, int n, cudaStream_t s);
+// bf16 tiles of n layers (1 <= n <= kGroupJobs, the same B, d, H; pairs by whole blocks of 32), probabilities in fp32
+cudaError_t tile_rows_batch_launch(const TileParams* p, int n, cudaStream_t s);
 // one query row (position q0) per (sequence, head) against the pairs [k0, k1): the in-leaf step of wide batches
 cudaError_t row_attn_launch(int dtype, const TileParams& p, cudaStream_t s);
 

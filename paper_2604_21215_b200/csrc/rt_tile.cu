@@ -11,7 +11,7 @@ constexpr int kTQ = 16;    // query rows per CTA
 constexpr int kTK = 32;    // keys per shared-memory chunk
 
 template <typename T>
-__device__ __forceinline__ void tile_simt(const TileParams& p) {
+__global__ void __launch_bounds__(128) tile_simt_kernel(const TileParams p) {
   __shared__ float Qs[kTQ][kHeadDim];
   __shared__ float Ks[kTK][kHeadDim + 1];
   __shared__ float Vs[kTK][kHeadDim];
@@ -66,7 +66,7 @@ __device__ __forceinline__ void tile_simt(const TileParams& p) {
       float s = 0.f;
 #pragma unroll 16
       for (int e = 0; e < kHeadDim; ++e) s += Qs[qr][e] * Ks[lane][e];
-      const float s2 = valid ? s * p.scale_log2 - slope_l2 * (float)(p.q_pos0 + qb + qr - (kb + lane)) : -INFINITY;
+      const float s2 = valid ? s * p.scale_log2 - slope_l2 * (float)(qb + qr - (kb + lane)) : -INFINITY;
       const float m_new = fmaxf(m[i], warp_max(s2));
       const float pj = valid ? exp2f(s2 - m_new) : 0.f;
       const float corr = exp2f(m[i] - m_new);
@@ -91,24 +91,6 @@ __device__ __forceinline__ void tile_simt(const TileParams& p) {
       p.st_o[sidx * p.d + h * kHeadDim + lane + 32] = ob[i];
     }
   }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(128) tile_simt_kernel(const TileParams p) { tile_simt<T>(p); }
-
-// One tile of each of several layers (the layers of a stack side by side); blockIdx.z is the layer, batch_stride 0.
-struct TileSimtBatch { TileParams p[kGroupJobs]; };
-__global__ void __launch_bounds__(128) tile_simt_batch_kernel(const __grid_constant__ TileSimtBatch t) { tile_simt<__nv_bfloat16>(t.p[blockIdx.z]); }
-
-cudaError_t tile_simt_batch_launch(const TileParams* p, int n, cudaStream_t s) {
-  TileSimtBatch t;
-  int nq = 0;
-  for (int i = 0; i < kGroupJobs; ++i) {
-    t.p[i] = p[i < n ? i : 0];
-    if (t.p[i].q1 - t.p[i].q0 > nq) nq = t.p[i].q1 - t.p[i].q0;
-  }
-  tile_simt_batch_kernel<<<dim3(ceil_div(nq, kTQ), p[0].B * p[0].H, n), 128, 0, s>>>(t);
-  return cudaGetLastError();
 }
 
 cudaError_t tile_simt_launch(int dtype, const TileParams& p, cudaStream_t s) {
@@ -276,6 +258,82 @@ cudaError_t tile_rows_launch(int dtype, const TileParams& p, cudaStream_t s) {
   auto go = [&](auto kern) { return launch_chained(kern, grid, dim3(128), 0, s, p.chained != 0, p); };
   if (dtype == RT_BF16) return nk > 8 ? go(tile_rows_kernel<__nv_bfloat16, 2>) : go(tile_rows_kernel<__nv_bfloat16, 1>);
   return nk > 8 ? go(tile_rows_kernel<float, 2>) : go(tile_rows_kernel<float, 1>);
+}
+
+// ---- tiles of several layers, probabilities in fp32 ------------------------------------------------------
+// The first tiles of the layers of a stack (leaves that begin at position 64 or 128), one of each layer: a warp takes one (sequence, head) and Q queries, 32 pairs at a
+// time as in row_attn_kernel.  What bounds it is a warp's chain where few sequences leave the chip to a few warps each SM (Q = 1), the instructions of the reductions where
+// many do (Q = 4: K and V rows are fetched once for four queries).
+struct TileRowsBatch { TileParams p[kGroupJobs]; };
+template <int Q>
+__global__ void __launch_bounds__(128) tile_rows_batch_kernel(const __grid_constant__ TileRowsBatch t) {
+  const TileParams& p = t.p[blockIdx.z];
+  const int lane = threadIdx.x & 31, u = blockIdx.x * 4 + (threadIdx.x >> 5), qa = p.q0 + (int)blockIdx.y * Q;
+  if (u >= p.B * p.H || qa >= p.q1) return;
+  const int b = u / p.H, h = u - b * p.H;
+  const __nv_bfloat16 *Kc = reinterpret_cast<const __nv_bfloat16*>(p.k_cache), *Vc = reinterpret_cast<const __nv_bfloat16*>(p.v_cache);
+  const size_t col = (size_t)b * p.d + h * kHeadDim + 2 * lane, rstride = (size_t)p.B * p.d;
+  const float slope_l2 = p.alibi ? p.alibi[h] * kLog2e : 0.f;
+  float2 qq[Q], o[Q];
+  float m[Q], l[Q];
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const int r = qa + i < p.q1 ? qa + i : p.q1 - 1;              // (rows beyond the tile repeat its last query and are not stored)
+    const size_t sidx = (size_t)r * p.B + b;
+    qq[i] = ldcg_T2(reinterpret_cast<const __nv_bfloat16*>(p.q) + (size_t)r * rstride + col);
+    o[i] = __ldcg(reinterpret_cast<const float2*>(p.st_o + sidx * p.d + h * kHeadDim + 2 * lane));
+    m[i] = __ldcg(p.st_m + sidx * p.H + h);
+    l[i] = __ldcg(p.st_l + sidx * p.H + h);
+  }
+#pragma unroll 1
+  for (int j = p.k0; j < p.k1; j += 32) {
+    unsigned kw[32], vw[32];                                      // two bf16 each
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+      kw[e] = __ldcg(reinterpret_cast<const unsigned*>(Kc + (size_t)(j + e) * rstride + col));
+      vw[e] = __ldcg(reinterpret_cast<const unsigned*>(Vc + (size_t)(j + e) * rstride + col));
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      float prod[32];
+#pragma unroll
+      for (int e = 0; e < 32; ++e) prod[e] = qq[i].x * __uint_as_float(kw[e] << 16) + qq[i].y * __uint_as_float(kw[e] & 0xffff0000u);
+      warp_transpose_sum32(prod, lane);
+      const float s2 = prod[0] * p.scale_log2 - slope_l2 * (float)(p.q_pos0 + qa + i - (j + lane));
+      const float m_new = fmaxf(m[i], warp_max(s2));
+      const float pj = exp2f(s2 - m_new), corr = exp2f(m[i] - m_new);
+      l[i] = l[i] * corr + warp_sum(pj);
+      o[i].x *= corr; o[i].y *= corr;
+#pragma unroll
+      for (int e = 0; e < 32; ++e) {
+        const float pw = __shfl_sync(0xffffffffu, pj, e);
+        o[i].x += pw * __uint_as_float(vw[e] << 16); o[i].y += pw * __uint_as_float(vw[e] & 0xffff0000u);
+      }
+      m[i] = m_new;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    if (qa + i < p.q1) {
+      const size_t sidx = (size_t)(qa + i) * p.B + b;
+      if (lane == 0) { p.st_m[sidx * p.H + h] = m[i]; p.st_l[sidx * p.H + h] = l[i]; }
+      *reinterpret_cast<float2*>(p.st_o + sidx * p.d + h * kHeadDim + 2 * lane) = o[i];
+    }
+  }
+}
+
+cudaError_t tile_rows_batch_launch(const TileParams* p, int n, cudaStream_t s) {
+  TileRowsBatch t;
+  int nq = 0;
+  for (int i = 0; i < kGroupJobs; ++i) {
+    t.p[i] = p[i < n ? i : 0];
+    if (t.p[i].q1 - t.p[i].q0 > nq) nq = t.p[i].q1 - t.p[i].q0;
+  }
+  const int pairs = p[0].B * p[0].H;
+  auto go = [&](auto kern, int q) { kern<<<dim3(ceil_div(pairs, 4), ceil_div(nq, q), n), 128, 0, s>>>(t); };
+  if ((long long)pairs * nq * n <= 16 * kB200Sms) go(tile_rows_batch_kernel<1>, 1);      // up to four warps a scheduler with one query each
+  else go(tile_rows_batch_kernel<4>, 4);
+  return cudaGetLastError();
 }
 
 cudaError_t tile_launch(int dtype, const TileParams& p, cudaStream_t s) {
