@@ -19,7 +19,7 @@ constexpr int kSmallBatchMax = 64;      // above this the per-token chain runs a
 constexpr int kAutoLeaf = 64;
 
 struct WsLayout {
-  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, ll, ll_bytes, form, form_bytes, g_arrays, dec_words, dec_words_bytes, hid0, hid1,
+  size_t sync, q, kt, vt, n, st_o, st_m, st_l, ex_h, ex_g, ex_z, ex_k, ex_part, ll, ll_bytes, form, form_bytes, sets, dec_words, dec_words_bytes, hid0, hid1,
       blk_h, blk_u, blk_c, blk_g, total;
 };
 
@@ -110,7 +110,7 @@ bool wave_exact_tile(bool exact, int t0) { return exact && t0 < kWaveExactMax; }
 // Tiles are what grows with the length: a leaf reads its layer's whole cache so far, so side by side they cost (N / 64)^2 / 2 blocks of 64 pairs x 64 queries a layer and (sequence,
 // head), 1.15 us each behind one another or 4.2 ns where they fill the chip; the same pairs cost 1.2 ns in Algorithm 1's larger tiles.  So one after the other, whose
 // cache traffic is N log N, is the faster form again from some length on: some 65 thousand positions for 8 layers of d = 1024, B = 16, some 20 thousand for 2.
-// Widths that are no multiple of 128 take the fp32 pre-pass, whose time per launch of leaves is 0.05 d us a layer and more.
+// Widths that are no multiple of 128 take the fp32 pre-pass, whose time per launch of leaves is 0.06 d us a layer and more.
 int band_begin(int n_layers, int bands, int b) { return (int)((long long)n_layers * b / bands); }      // (bands of about the same depth)
 bool tensor_prepass(const rt_config* c) { return c->d_model % 128 == 0; }
 float wave_us(const rt_config* c, int B, int N, int n_layers, const Wave& w) {
@@ -119,7 +119,7 @@ float wave_us(const rt_config* c, int B, int N, int n_layers, const Wave& w) {
   long long launches = 0;
   for (int b = 0; b < bands; ++b) launches += wave_launches(band_begin(n_layers, bands, b + 1) - band_begin(n_layers, bands, b), ceil_div(N, leaf), places);
   float us = (float)leaf * leaf_group_step_us(B, c->d_model, c->d_ff, places) + 21.0f + 3.5e-4f * (float)(places * B) * d;
-  if (!tensor_prepass(c)) us += (float)places * d * (0.048f + 4.2e-7f * (float)B * d);
+  if (!tensor_prepass(c)) us += (float)places * d * (0.06f + 1.2e-6f * (float)B * d);
   // of the whole blocks that come before a leaf, on average half: a launch for each power of two that their number consists of
   if (blocks > 1.0f) us += (1.0f - 1.0f / blocks) * ((0.5f * log2f(blocks) + 0.9f) * (9.0f + 0.01f * tiles) + 0.5f * blocks * fmaxf(1.15f, 4.2e-3f * tiles));
   return (float)launches * us;
@@ -197,8 +197,8 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers, size_t form) {
     if (N > kWaveExactN) return none;                           // (the bits of that kernel)
     return four_pay(sl.step_us) ? best : none;
   }
-  // All others go side by side where that is estimated to be faster.  Over 2 to 8 layers of d = 448, 512, 768, 960 and 1024, 1 to 16 sequences and 32 to 1024
-  // positions (1100 stacks, both ways timed) the choice is on average 0.4 % and at most 16 % slower than the other; with one break-even for all widths
+  // All others go side by side where that is estimated to be faster.  Over 2 to 8 layers of eight widths from d = 448 to 1024, 1, 5 and 16 sequences and 32 to
+  // 700 positions (720 stacks, both ways timed) the choice is on average 0.2 % and at most 8 % slower than the better one; with one break-even for all widths
   // stacks of d = 960 went side by side at up to 1.45 times the time (2 layers, N = 129: 2.30 and 3.34 ms; d = 448, N = 100: 1.65 and 1.95) and 4
   // layers of d = 1024, B = 16, N = 64 did not at 1.19 times (2.99 and 2.52).  The line for four places tells which stacks keep fp32 probabilities one after the other.
   if (0.95f * least < alone_us(c, B, N, n_layers)) return best;
@@ -206,9 +206,9 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers, size_t form) {
   alone.exact = N > kWaveBlock && N <= kWaveExactN && four_pay(mma_us);
   return alone;
 }
-// Positions that the tensor-core leaf kernel has an array of g for: a leaf, or all layers of a prompt shorter than that (one fill serves
+// Positions that the tensor-core leaf kernel has arrays of c, h, z and g for: a leaf, or all layers of a prompt shorter than that (one fill serves
 // them: 8 layers of one position, d = 1024, 305 -> 291 us).
-int g_positions(const rt_config* c, int N, int n_layers) {
+int set_positions(const rt_config* c, int N, int n_layers) {
   LeafMmaLaunch ml;
   if (!leaf_mma_shape(1, c->d_model, c->n_heads, c->d_ff, c->leaf, kB200Sms, kB200SmemPerCta, &ml)) return 0;
   return (long long)N * n_layers < ml.leaf ? N * n_layers : ml.leaf;
@@ -216,14 +216,14 @@ int g_positions(const rt_config* c, int N, int n_layers) {
 
 // Bytes of the area that the form of the token loop has to itself: the most that any call of at most B sequences, N positions and n_layers
 // layers asks for, whichever form it takes, so that a workspace reserved for the longest prompt and the fullest batch serves all the others.
-// (What one form asks for by itself does not grow with the shape: from 17 sequences on there is no array of g.)
+// (What one form asks for by itself does not grow with the shape: from 17 sequences on there are no arrays of the leaf kernel.)
 size_t form_bytes(const rt_config* c, int B, int N, int n_layers) {
   if (c->dtype != RT_BF16) return 0;
   if (c->sched != RT_SCHED_TILED || c->recur_block > 1) return 0;
   const int d = c->d_model, H = c->n_heads, f = c->d_ff, B16 = B < 16 ? B : 16;
   size_t most = 0;
   auto need = [&](size_t bytes) { if (bytes > most) most = bytes; };
-  need((size_t)g_positions(c, N, n_layers) * leaf_mma_set_bytes(d, f));
+  need((size_t)set_positions(c, N, n_layers) * leaf_mma_set_bytes(d, f));
   if (N < 2) return most;
   for (int places = 2; places <= kGroupJobs; ++places) {
     if (!leaf_group_shape(1, d, H, f, places, kB200SmemPerCta)) continue;
@@ -253,11 +253,11 @@ WsLayout ws_layout(const rt_config* c, int B, int N, int n_layers, size_t more_f
   L.ex_z = take((size_t)B * d * 4);
   L.ex_k = take((size_t)B * d * 4);
   L.ex_part = take((size_t)B * H * kMaxChunks * 68 * 4);
-  // exchange buffers of the tensor-core leaf kernel: c, h, z as flag-carrying words (16 sequence slots each),
-  // raw k|v as flag-carrying fp32 words; g as packed bf16 in fragment order (16 sequence slots), an array per position of a leaf, in `form`
+  // exchange buffer of the tensor-core leaf kernel: raw k|v as fp32 words beside their step number (c, h, z and g, packed bf16 in fragment order for 16
+  // sequence slots, have arrays per position of a leaf, in `form`)
   L.ll_bytes = (size_t)B * 2 * d * 8;
   L.ll = take(L.ll_bytes);
-  L.g_arrays = c->dtype == RT_BF16 ? g_positions(c, N, n_layers) : 0;
+  L.sets = c->dtype == RT_BF16 ? set_positions(c, N, n_layers) : 0;
   L.form_bytes = form_bytes(c, B, N, n_layers) + more_form;
   L.form = take(L.form_bytes);
   // a decode step uses none of the above but the status block: its exchange area begins right behind that
@@ -324,7 +324,7 @@ struct ProfScope {
 };
 
 // State of one API call: the stream and the barrier arrivals enqueued so far.
-struct CallCtx { cudaStream_t s; unsigned bar_base = 0; unsigned seq_base = 0; unsigned group_steps[kGroupJobs] = {}; bool groups_cleared = false; int g_left = 0; bool exact = false; };      // g_left: sets of vectors still filled; exact: first tiles with fp32 probabilities
+struct CallCtx { cudaStream_t s; unsigned bar_base = 0; unsigned seq_base = 0; unsigned group_steps[kGroupJobs] = {}; bool groups_cleared = false; int sets_left = 0; bool exact = false; };      // sets_left: arrays of c, h, z, g still filled; exact: first tiles with fp32 probabilities
 
 // The exchange areas of the group kernel start from ones (no word written), once per API call.
 bool clear_groups(const rt_config* c, int places, unsigned char* ws, const WsLayout& L, CallCtx& ctx) {
@@ -601,14 +601,14 @@ rt_status run_layer(const rt_config* c, const rt_layer_weights* w, const void* x
       lp.x = (const unsigned char*)x + (size_t)b0 * x_bs * e;
       lp.z = (unsigned char*)z + (size_t)b0 * z_bs * e;
       lp.t0 = t0; lp.t1 = t1; lp.attn_begin = t0; lp.seq_base = ctx.seq_base;
-      // fresh arrays of g for the positions of this launch; filled all at once when they run out
-      const size_t g_bytes = leaf_mma_set_bytes(c->d_model, c->d_ff);
-      if (ctx.g_left < t1 - t0) {
-        if (cudaMemsetAsync(ws + L.form, 0xff, L.g_arrays * g_bytes, s) != cudaSuccess) return false;
-        ctx.g_left = (int)L.g_arrays;
+      // fresh arrays of c, h, z and g for the positions of this launch; filled all at once when they run out
+      const size_t set_bytes = leaf_mma_set_bytes(c->d_model, c->d_ff);
+      if (ctx.sets_left < t1 - t0) {
+        if (cudaMemsetAsync(ws + L.form, 0xff, L.sets * set_bytes, s) != cudaSuccess) return false;
+        ctx.sets_left = (int)L.sets;
       }
-      mb.vectors = ws + L.form + (L.g_arrays - (size_t)ctx.g_left) * g_bytes;
-      ctx.g_left -= t1 - t0;
+      mb.vectors = ws + L.form + (L.sets - (size_t)ctx.sets_left) * set_bytes;
+      ctx.sets_left -= t1 - t0;
       if (leaf_mma_launch(lp, ml, mb, s) != cudaSuccess) return false;
       ctx.seq_base += (unsigned)(t1 - t0);
     }
