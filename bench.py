@@ -346,9 +346,13 @@ def run_cuda(args):
                             "the fraction is the effective weight+activation stream against the HBM copy peak and "
                             "traffic is the DRAM bytes ncu counted for one launch"}
         if side_by_side:
-            roofline["note"] = ("several layers per launch, a group of SMs each, weights streamed from L2: bound by the exchanges of a "
-                                "token step, its products and instruction issue; us_per_token_step is the launch time over all (layer, position) "
-                                "pairs in it; the fraction is the effective weight+activation stream against the HBM copy peak")
+            # every step of every layer streams its weights from L2: 145 GB/s per SM as bulk copies, 18 TB/s from all of them together
+            # while the layers in a launch fit L2
+            l2_gbs = 18000.0
+            roofline.update(bound="l2", peak=l2_gbs, frac=achieved / l2_gbs, peak_source="measured: packed weights that fit L2, bulk copies into all SMs")
+            roofline["note"] = ("several layers per launch, a group of SMs each, weights streamed from L2 every step: bound by the exchanges of a "
+                                "token step, its products and instruction issue, not by that stream; us_per_token_step is the launch time over all "
+                                "(layer, position) pairs in it; the fraction is the weight+activation stream against what L2 delivers")
         if wl.B > 64:
             # wide batches: the token step is a chain of dense products over the B rows (tcgen05), one position at
             # a time, a leaf of them in one launch; the leaf class of the profile holds them with the in-leaf attention

@@ -1,6 +1,6 @@
 // Leaf recurrence of several independent (layer, slice of sequences) jobs at once, bf16: the SMs are split into groups of
 // equal size, one job each.  Used where jobs exist side by side: the layers of a stack (layer l works on a leaf that layer
-// l-1 finished one launch earlier) and batches of more than 16 sequences (slices of at most 16).
+// l-1 finished in an earlier launch) and batches of more than 16 sequences (slices of at most 16).
 //
 // A token step is a chain of exchanges whose length does not depend on how many SMs take part, so a single job leaves
 // 148 SMs waiting most of the time (rt_leaf_mma.cu).  Several jobs side by side fill the waits.  A group's weights (23 MB at
@@ -686,7 +686,8 @@ size_t leaf_group_packed_bytes(int d, int dff, int places) {
   return align_up((size_t)g * group_shape(d, dff, g).step_bytes, 256);
 }
 
-// Whether jobs of B sequences run on groups of 148 / places SMs (pure arithmetic).
+// Whether jobs of B sequences run on groups of 148 / places SMs (pure arithmetic).  A CTA's rows of d are at most kQuad tiles, so that one pass finishes them: d = 1024
+// takes four places at most, 768 six, 576 and less eight.
 bool leaf_group_shape(int B, int d, int H, int dff, int places, size_t max_smem) {
   if (B < 1 || B > 16 || places < 1 || places > kGroupJobs || d % 64 || d > 1024 || dff % 32 || dff > 8 * d) return false;
   const int g = group_size(d, places);

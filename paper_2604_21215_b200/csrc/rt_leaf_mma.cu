@@ -82,8 +82,8 @@ __device__ __forceinline__ unsigned pack_bf2(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const unsigned*>(&v);
 }
-// Every published word is one 64-bit scalar (payload in the low half, step number in the high
-// half), so a reader never sees a payload without its flag.  Loads fetch two adjacent words.
+// A word of k|v is one 64-bit scalar (payload in the low half, step number in the high half), so a
+// reader never sees a payload without its flag.  Loads fetch two adjacent words.
 __device__ __forceinline__ uint4 ld_relaxed_v4(const void* p) {
   unsigned long long w0, w1;
   asm volatile("ld.relaxed.gpu.global.v2.u64 {%0,%1}, [%2];" : "=l"(w0), "=l"(w1) : "l"(p) : "memory");

@@ -429,7 +429,7 @@ cudaError_t tile_tc_launch(const TileParams& p, int rows_q, int rows_kv, SyncAre
   return go(tile_tc_kernel<false, false>);
 }
 
-// Tiles of n <= kGroupJobs layers (the same B, d, H; slopes in all or none), as many queries each as the first at most.
+// Tiles of n <= kGroupJobs layers (the same B, d, H; slopes in all or none); the grid is that of the most queries, a CTA without any leaves at once.
 cudaError_t tile_tc_batch_launch(const TileParams* p, int n, SyncArea* sync, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   TileBatch t;

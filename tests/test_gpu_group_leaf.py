@@ -203,7 +203,7 @@ def test_one_position_takes_the_tensor_core_kernels(B):
     assert rt.rt_plan_counters(layer.cfg, B, 1)["model_bytes_read"] - B * per_token - pre_w == chain_w * (1 if B > 48 else -(-B // 16))
 
 
-# One after the other, the layers of a short prompt share arrays of g that are filled together: a launch takes fresh ones, and the last ones do
+# One after the other, the layers of a short prompt share arrays of c, h, z and g that are filled together: a launch takes fresh ones, and the last ones do
 # not always suffice for the next layer (64 arrays; 30 + 30 positions and 4 left, 21 x 3 and 1 left; 64 + 6 with a leaf of its own in between).
 @pytest.mark.parametrize("L,B,N", [(24, 1, 3), (3, 9, 30), (2, 4, 70), (5, 20, 1)])
 def test_layers_one_after_the_other_give_the_bits_of_single_layers(L, B, N):
