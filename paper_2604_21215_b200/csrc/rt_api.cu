@@ -742,6 +742,8 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
       }
       // The leaf's queries against the whole blocks of kWaveBlock earlier pairs; the kernel absorbs the rest.
       TileParams tiles[kGroupJobs];
+      // (distances alone, without a scale, are not for the tensor-core tile either)
+      auto fp32_tile = [&](int i) { return wave_exact_tile(wv.exact, jobs[i].t0) || (jobs[i].alibi && gc.scale_log2 == 0.f); };
       auto tile_of = [&](int i, int k0, int k1) {
         TileParams tp;
         memset(&tp, 0, sizeof(tp));
@@ -754,7 +756,7 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
       {
         int nt = 0;
         for (int i = 0; i < nj; ++i)
-          if (jobs[i].key0 && wave_exact_tile(wv.exact, jobs[i].t0)) tiles[nt++] = tile_of(i, 0, jobs[i].key0);
+          if (jobs[i].key0 && fp32_tile(i)) tiles[nt++] = tile_of(i, 0, jobs[i].key0);
         if (nt) {
           ProfScope ps(s, kProfTile);
           if (tile_rows_batch_launch(tiles, nt, s) != cudaSuccess) return RT_ERR_CUDA;
@@ -767,7 +769,7 @@ rt_status run_stack_wave(const rt_config* c, int n_layers, const rt_layer_weight
         for (int sloped = 0; sloped < 2; ++sloped) {
           int nt = 0;
           for (int i = 0; i < nj; ++i) {
-            int blocks = wave_exact_tile(wv.exact, jobs[i].t0) ? 0 : jobs[i].key0 / kWaveBlock, k0 = 0, size = 0;
+            int blocks = fp32_tile(i) ? 0 : jobs[i].key0 / kWaveBlock, k0 = 0, size = 0;
             for (int skip = 0; blocks && skip <= part; ++skip) {
               k0 += size;
               size = 1;

@@ -330,3 +330,27 @@ def test_first_tiles_match_oracle(L, d, H, B, N):
         check_tensor(f"first tiles layer {i}", "k", got[0], k, 2e-2)
         check_tensor(f"first tiles layer {i}", "v", got[1], v, 2e-2)
     check_tensor("first tiles", "hidden", hid, x, 2e-2)
+
+
+# Distances alone (scale 0) set the weights: a layer whose second block meets the first through a tile, the parallel sweep, and layers side by side beyond position 192.
+@pytest.mark.parametrize("L,N", [(1, 150), (8, 290)])
+def test_distances_without_a_scale(L, N):
+    from oracle import RTConfig, RTWeights, layer_seq
+    from paper_2604_21215_b200 import inputs, rt
+    d, H, B, V = 512, 8, 2, 91
+    data = inputs.make_inputs(inputs.Workload("dist", L, B, N, d, H, d, "bf16", vocab=V, residual_scale=1 / np.sqrt(L)), seed=N)
+    slopes = [2.0 ** -(h + 3) for h in range(H)]
+    kw = dict(residual_scale=1 / np.sqrt(L), softmax_scale=0.0)
+    st = rt.Stack(L, d, H, d, V, dtype="bf16", **kw)
+    st.set_weights([dict(lw, alibi_slopes=slopes) for lw in data["layers"]], data["emb"])
+    hid, _ = st.prefill(data["ids"])
+    x = np.asarray(data["emb"], dtype=np.float64)[np.asarray(data["ids"])]
+    for lw in data["layers"]:
+        x0 = x
+        x, k, v = layer_seq(RTConfig(d, H, 64, d, alibi_slopes=slopes, **kw), RTWeights(**lw), x)
+    check_tensor("distances alone", "hidden", hid, x, 2e-2)
+    if L == 1:
+        layer = rt.Layer(d, H, d, dtype="bf16", **kw)
+        layer.set_weights(dict(data["layers"][0], alibi_slopes=slopes))
+        z, _, _ = layer.recompute(x0, x)
+        check_tensor("distances alone", "sweep", z, x, 2e-2)
