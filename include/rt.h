@@ -106,7 +106,7 @@ typedef struct {            /* device pointers; read-only */
  * the fullest batch, the longest prompt and the deepest stack serves every smaller call.
  * rt_stack_prefill also takes less, down to the size for one layer: the rest holds weights of layers that
  * run side by side, in packed form (of up to 16 layers; 23 MB each at d_model = 1024), and with less of
- * it fewer of them do, down to none. */
+ * it fewer of them do, down to none (the same values; up to 1024 positions their rounding may differ). */
 size_t rt_workspace_bytes(const rt_config *cfg, int32_t B, int32_t N, int32_t n_layers);
 
 /* One RT layer over x[B,N,d] (Sec. 2.2; Algorithm 1).  Writes z[B,N,d] and rows [0,N) of
