@@ -179,7 +179,6 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers, size_t form) {
       if (!best.places || us < least) { best = w; least = us; }
     }
   }
-  if (!best.places) return none;
   // Four layers side by side, each in the place of the one four before it, pay where enough of them are at work at the same time: on average n_layers * N /
   // (launches * leaf) of them, 1.3 to 2.3, more the more weights the groups stream (places x MB per layer) and above four sequences.
   const float layer_mb = (3.0f * c->d_model + 2.0f * c->d_ff) * c->d_model * 2e-6f, mma_us = B > 8 ? 10.5f : 8.3f;
@@ -195,16 +194,16 @@ Wave stack_wave(const rt_config* c, int B, int N, int n_layers, size_t form) {
     // of the last k against 64 bits 4.95e-3 and 5.2e-3; 2 layers of d = 384 2.97e-3 and 3.3e-3).  So more than four places are no reason to take them
     // off it: they go side by side only where four pay against that kernel, which is faster than the tensor-core leaf kernel (taken as mma_us a position).
     if (N > kWaveExactN) return none;                           // (the bits of that kernel)
-    return four_pay(sl.step_us) ? best : none;
+    if (!four_pay(sl.step_us)) return none;
+    if (best.places) return best;
+    return {0, 0, 0, N > kWaveBlock};
   }
   // All others go side by side where that is estimated to be faster.  Over 2 to 8 layers of eight widths from d = 448 to 1024, 1, 5 and 16 sequences and 32 to
   // 700 positions (720 stacks, both ways timed) the choice is on average 0.2 % and at most 8 % slower than the better one; with one break-even for all widths
   // stacks of d = 960 went side by side at up to 1.45 times the time (2 layers, N = 129: 2.30 and 3.34 ms; d = 448, N = 100: 1.65 and 1.95) and 4
   // layers of d = 1024, B = 16, N = 64 did not at 1.19 times (2.99 and 2.52).  The line for four places tells which stacks keep fp32 probabilities one after the other.
-  if (0.95f * least < alone_us(c, B, N, n_layers)) return best;
-  Wave alone = none;
-  alone.exact = N > kWaveBlock && N <= kWaveExactN && four_pay(mma_us);
-  return alone;
+  if (best.places && 0.95f * least < alone_us(c, B, N, n_layers)) return best;
+  return {0, 0, 0, N > kWaveBlock && N <= kWaveExactN && four_pay(mma_us)};
 }
 // Positions that the tensor-core leaf kernel has arrays of c, h, z and g for: a leaf, or all layers of a prompt shorter than that (one fill serves
 // them: 8 layers of one position, d = 1024, 305 -> 291 us).
