@@ -261,12 +261,15 @@ cudaError_t tile_rows_launch(int dtype, const TileParams& p, cudaStream_t s) {
 }
 
 // ---- tiles of several layers, probabilities in fp32 ------------------------------------------------------
-// The first tiles of the layers of a stack (leaves that begin at position 64 or 128), one of each layer: a warp takes one (sequence, head) and Q queries, 32 pairs at a
-// time as in row_attn_kernel.  What bounds it is a warp's chain where few sequences leave the chip to a few warps each SM (Q = 1), the instructions of the reductions where
-// many do (Q = 4: K and V rows are fetched once for four queries).
+// The first tiles of the layers of a stack (leaves that begin at position 64 or 128), one of each layer: a warp takes one (sequence, head) and four queries, for which
+// it fetches the K and V rows once, 32 pairs at a time as in row_attn_kernel.  What bounds it is a warp's chain (two or four rounds of 32 pairs, a reduction and 32 weighted rows for
+// each query) where sequences are few, the instructions of the reductions where they are many.  8 layers of d = 1024, us per launch with one query a warp / four: N = 77, B = 1 12.5 / 11.2,
+// B = 16 15.0 / 12.5; N = 190, B = 1 17.7 / 16.8, B = 4 20.5 / 17.3, B = 16 45.5 / 36.8 (a leaf launch takes 280 to 640).  Against the kernel of 16 queries above, whole calls: B = 1, N = 77
+// 4.49 -> 4.36 ms; six and more layers of N = 150 to 200 gain 4 %.
+constexpr int kBatchTileQueries = 4;
 struct TileRowsBatch { TileParams p[kGroupJobs]; };
-template <int Q>
 __global__ void __launch_bounds__(128) tile_rows_batch_kernel(const __grid_constant__ TileRowsBatch t) {
+  constexpr int Q = kBatchTileQueries;
   const TileParams& p = t.p[blockIdx.z];
   const int lane = threadIdx.x & 31, u = blockIdx.x * 4 + (threadIdx.x >> 5), qa = p.q0 + (int)blockIdx.y * Q;
   if (u >= p.B * p.H || qa >= p.q1) return;
@@ -329,10 +332,7 @@ cudaError_t tile_rows_batch_launch(const TileParams* p, int n, cudaStream_t s) {
     t.p[i] = p[i < n ? i : 0];
     if (t.p[i].q1 - t.p[i].q0 > nq) nq = t.p[i].q1 - t.p[i].q0;
   }
-  const int pairs = p[0].B * p[0].H;
-  auto go = [&](auto kern, int q) { kern<<<dim3(ceil_div(pairs, 4), ceil_div(nq, q), n), 128, 0, s>>>(t); };
-  if ((long long)pairs * nq * n <= 16 * kB200Sms) go(tile_rows_batch_kernel<1>, 1);      // up to four warps a scheduler with one query each
-  else go(tile_rows_batch_kernel<4>, 4);
+  tile_rows_batch_kernel<<<dim3(ceil_div(p[0].B * p[0].H, 4), ceil_div(nq, kBatchTileQueries), n), 128, 0, s>>>(t);
   return cudaGetLastError();
 }
 

@@ -323,7 +323,7 @@ def test_probabilities_of_the_first_leaves_are_not_rounded(L, H, side, least):
     assert abs(factor) <= 2e-4, factor
 
 
-# The kernel of those tiles at the edges of its rows: one query and full leaves in the last leaf, few warps (a query each) and many (four each), slopes in some layers.
+# The kernel of those tiles at the edges of its rows: one query, a rest of three and full leaves in the last leaf, few warps and many, slopes in some layers.
 @pytest.mark.parametrize("L,d,H,B,N", [(8, 512, 8, 1, 65), (8, 512, 8, 16, 130), (4, 1024, 16, 9, 191), (2, 448, 7, 5, 187)])
 def test_first_tiles_match_oracle(L, d, H, B, N):
     from oracle import RTConfig, RTWeights, layer_seq
